@@ -431,7 +431,7 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
     // tensor-core path: its kernel also writes the kept-dim rows of the middle from the boxes it loads; the partition
     // kernel is left with the windows and the counters
     bool tc2 = tc && compress_tc2_supported(s);             // CTA pairs where the row tiles pair up
-    bool tc_rows = tc && (tc2 ? compress_tc2_gathers(s) : compress_tc_gathers(s));
+    bool tc_rows = tc && (tc2 || compress_tc_gathers(s));
     if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, !tc, ordered, !tc_rows, true, cs) != cudaSuccess)
         return FA_ERR_CUDA;
     if (tc2 && launch_compress_tc2(s, make_cache(*cache), K, V, sbb, stride_t, stride_h, L, ordered, tc_rows, cs) != cudaSuccess) {
@@ -476,7 +476,7 @@ bool compress_is_pair_form(const fa_layout* layout, int64_t stride_b, int64_t st
     const int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;
     const int64_t sbb = s.B > 1 ? stride_b : 0;
     return L > 0 && L - n_init - n_local >= 1024 && compress_tc_supported(s, layout->kv_dtype, sbb, stride_t, stride_h) &&
-           compress_tc2_supported(s) && compress_tc2_gathers(s);
+           compress_tc2_supported(s);
 }
 }  // namespace
 

@@ -108,7 +108,6 @@ cudaError_t launch_compress(const Dims&, const CacheDev&, int dtype, const void*
 bool compress_tc_gathers(const Dims& s);
 // The same path on CTA pairs (fa_compress_tc2.cu): needs an even number of 128-row tiles.
 bool compress_tc2_supported(const Dims& s);
-bool compress_tc2_gathers(const Dims& s);
 cudaError_t launch_compress_tc2(const Dims&, const CacheDev&, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh,
                                 int L, bool ordered, bool gather, cudaStream_t);
 // Tensor-core reconstruction of the dimension selection (fa_select_tc.cu).

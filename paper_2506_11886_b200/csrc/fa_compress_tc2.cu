@@ -14,6 +14,7 @@
 // signals the stage barriers of both CTAs (multicast of the ARRIVAL, not of a load).
 // Every wait is bounded; tensor memory is freed on every path; both CTAs meet before they leave.
 #include <mutex>
+#include <type_traits>
 
 #include "fa_umma.cuh"
 
@@ -24,9 +25,23 @@ using bf16 = __nv_bfloat16;
 constexpr int kBM = 128;          // coefficient rows per CTA (256 per pair)
 constexpr int kBK = 64;           // tokens per pipeline stage
 constexpr int kGenWarps = 8;       // basis generators (and epilogue): 16 tokens of two rows per thread and stage
-constexpr int kGatherWarps = 4;    // kept-dim rows of the middle, from the B boxes
-constexpr int kGatherItems = 4;    // 16-byte chunks per gather thread and stage, at most
-constexpr int kThreadsTc = 64 + 32 * (kGenWarps + kGatherWarps);
+constexpr int kGatherItems = 4;    // 16-byte chunks per gather thread and round, at most
+// Rounds in which the gather warps take the rows of a stage: a round is 64 / rounds consecutive rows, so that a thread's
+// items of round q lie a constant q * (64 / rounds) * 128 bytes behind those of round 0 (the swizzle repeats every
+// eight rows) and only one round's offsets are held in registers.  The smallest power of two with which the pairs of
+// a team cover the kept dims; eight rounds always do (8 rows x 2 heads x 16 chunks = 256 of 512 items).
+__host__ __device__ inline int gather_rounds(int n_pairs, int hp, int nf, int gw) {
+    int r = 1;
+    while (r < 8 && ((kBK / r + n_pairs - 1) / n_pairs) * hp * (nf >> 3) > kGatherItems * 32 * gw) r *= 2;
+    return r;
+}
+// Warps that write the kept-dim rows of the middle from the B boxes: four where one round of their items covers a stage
+// (more of them only draw power: the 32K contraction runs at the power cap and loses 3 % with six), eight where it
+// does not (one or two pairs per team and many kept dims: every pair writes most rows of its boxes itself; 4 K
+// tokens of the 32-head MHA layout, 48 kept dims: fa_compress 264 us with four, 234 with six, 227 with eight, and 320 with
+// the rows left to the partition kernel, which then reads the whole prefill once more).
+constexpr int kFewGather = 4, kManyGather = 8;
+constexpr int threads_tc(int gw) { return 64 + 32 * (kGenWarps + gw); }
 using namespace umma;
 
 // Work of a launch: the token blocks of all (batch, head group) units, laid end to end: position = unit * blocks + block.
@@ -42,8 +57,9 @@ struct TeamCuts { uint32_t start[kMaxTeams + 1]; };
 
 // D = head dim (64 or 128): N = 2 D accumulator columns per KV head (K dims, then V dims); HP heads share the pair
 // and its generated basis tiles (HP * N <= 512 tensor-memory columns).  grid 2 * teams * (M / 256), clusters of two.
-template <int D, int HP>
-__global__ void __launch_bounds__(kThreadsTc, 1) compress_tc2_kernel(const __grid_constant__ CUtensorMap tmK,
+// kGatherWarps: kFewGather or kManyGather (the latter may take several rounds).
+template <int D, int HP, int kGatherWarps>
+__global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV, Dims s,
                                                                      CacheDev c, int L, const __grid_constant__ TeamCuts cuts,
                                                                      int per, int gather) {
@@ -203,8 +219,9 @@ __global__ void __launch_bounds__(kThreadsTc, 1) compress_tc2_kernel(const __gri
             const int gt = tid - 32 * (2 + kGenWarps);           // 0 .. 32 kGatherWarps - 1
             const int cph = nf_side >> 3;                                      // 16-byte chunks per kept-dim row of this side
             // the pairs of the team load the same boxes and share the tokens: this pair takes rows pair, pair + n_pairs, ...
-            const int n_tok = pair < kBK ? (kBK - pair + n_pairs - 1) / n_pairs : 0;
-            const int n_items = gather ? n_tok * HP * cph : 0;                // <= kGatherItems per thread (checked on the host)
+            const int rounds = kGatherWarps == kManyGather ? gather_rounds(n_pairs, HP, nf_side, kGatherWarps) : 1, rpr = kBK / rounds;
+            const int n_tok = pair < rpr ? (rpr - pair + n_pairs - 1) / n_pairs : 0;
+            const int n_items = gather ? n_tok * HP * cph : 0;                // per round, <= kGatherItems per thread
             const bool p2 = (s.P & (s.P - 1)) == 0;
             const int lgP = 31 - __clz(s.P);
             int it = 0;
@@ -252,34 +269,39 @@ __global__ void __launch_bounds__(kThreadsTc, 1) compress_tc2_kernel(const __gri
                     const int st = it % kStagesTc;
                     if (!mbar_wait(full + st, (it / kStagesTc) & 1, fail, c.status)) { live = false; break; }
                     const unsigned char* bsrc = stage0 + (size_t)st * kStageBytesTc + kABytes;
-                    const int jb = kb * kBK;               // first middle token of the block
-                    uint4 val[kGatherItems];
+                    int jb = kb * kBK;                     // first middle token of the round
+#pragma unroll 1
+                    for (int q = 0; q < rounds; ++q, bsrc += rpr * 128, jb += rpr) {
+                        uint4 val[kGatherItems];
 #pragma unroll
-                    for (int u = 0; u < kGatherItems; ++u) {
-                        uint32_t w[4] = {0u, 0u, 0u, 0u};
-                        if (meta[u] >= 0) {
+                        for (int u = 0; u < kGatherItems; ++u) {
+                            uint32_t w[4] = {0u, 0u, 0u, 0u};
+                            if (meta[u] >= 0) {
 #pragma unroll
-                            for (int i2 = 0; i2 < 4; ++i2) {
-                                const uint32_t lo = *reinterpret_cast<const uint16_t*>(bsrc + (src[u][i2] & 0xffffu));
-                                const uint32_t hi = *reinterpret_cast<const uint16_t*>(bsrc + (src[u][i2] >> 16));
-                                w[i2] = lo | (hi << 16);
+                                for (int i2 = 0; i2 < 4; ++i2) {
+                                    const uint32_t lo = *reinterpret_cast<const uint16_t*>(bsrc + (src[u][i2] & 0xffffu));
+                                    const uint32_t hi = *reinterpret_cast<const uint16_t*>(bsrc + (src[u][i2] >> 16));
+                                    w[i2] = lo | (hi << 16);
+                                }
                             }
+                            val[u] = make_uint4(w[0], w[1], w[2], w[3]);
                         }
-                        val[u] = make_uint4(w[0], w[1], w[2], w[3]);
-                    }
-                    __syncwarp();                          // the values are in registers: the stage goes back before the stores
-                    if (lane == 0) mbar_arrive(empty + st);
+                        if (q + 1 == rounds) {
+                            __syncwarp();                  // the values are in registers: the stage goes back before the stores
+                            if (lane == 0) mbar_arrive(empty + st);
+                        }
 #pragma unroll
-                    for (int u = 0; u < kGatherItems; ++u) {
-                        const int j = jb + (meta[u] & 0xff);
-                        if (meta[u] >= 0 && j < n_mid) {
-                            const int hh = (meta[u] >> 8) & 0xf, lch = meta[u] >> 16;
-                            const int cls = p2 ? (j & (s.P - 1)) : j % s.P, slot = p2 ? (j >> lgP) : j / s.P;
-                            const int nfull = nf_side;
-                            // logical chunk lch of a V^mu row is stored at chunk lch ^ swizzle
-                            const int ch = side ? (lch ^ v_swz(slot, nfull >> 3)) : lch;
-                            bf16* dst = mid_row<bf16>(side ? c.v_mid : c.k_mid, s, g.b, g.h0 + hh, cls, slot, nfull);
-                            reinterpret_cast<uint4*>(dst)[ch] = val[u];
+                        for (int u = 0; u < kGatherItems; ++u) {
+                            const int j = jb + (meta[u] & 0xff);
+                            if (meta[u] >= 0 && j < n_mid) {
+                                const int hh = (meta[u] >> 8) & 0xf, lch = meta[u] >> 16;
+                                const int cls = p2 ? (j & (s.P - 1)) : j % s.P, slot = p2 ? (j >> lgP) : j / s.P;
+                                const int nfull = nf_side;
+                                // logical chunk lch of a V^mu row is stored at chunk lch ^ swizzle
+                                const int ch = side ? (lch ^ v_swz(slot, nfull >> 3)) : lch;
+                                bf16* dst = mid_row<bf16>(side ? c.v_mid : c.k_mid, s, g.b, g.h0 + hh, cls, slot, nfull);
+                                reinterpret_cast<uint4*>(dst)[ch] = val[u];
+                            }
                         }
                     }
                 }
@@ -461,13 +483,13 @@ bool make_map2(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, int HP>
+template <int D, int HP, int GW>
 cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, int n_mid,
                          bool ordered, bool gather, cudaStream_t stream) {
     constexpr size_t stage = (size_t)kBM * kBK * 2 + (size_t)HP * (D / 64) * kBK * 64 * 2;
     constexpr size_t n_stages = (200 * 1024) / stage < 6 ? (200 * 1024) / stage : 6;
     const size_t smem = n_stages * stage + 8 * (3 * n_stages + 3) + 16 + sizeof(int) * HP * D + 64 + 1024;
-    cudaError_t err = ensure_dynamic_smem(compress_tc2_kernel<D, HP>, smem);
+    cudaError_t err = ensure_dynamic_smem(compress_tc2_kernel<D, HP, GW>, smem);
     if (err != cudaSuccess) return err;
     const int n_pairs = s.M / (2 * kBM);
     const int nkb = (n_mid + kBK - 1) / kBK;
@@ -475,7 +497,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
     const long long total = n_units * nkb;                      // positions: the blocks of all units, end to end
     if (total <= 0 || total >= (1ll << 31)) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kThreadsTc);
+    cfg.blockDim = dim3(threads_tc(GW));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -506,7 +528,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
             cfg.gridDim = dim3(2 * sm_count());
             cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, compress_tc2_kernel<D, HP>, &cfg) != cudaSuccess || n < 1) {
+            if (cudaOccupancyMaxActiveClusters(&n, compress_tc2_kernel<D, HP, GW>, &cfg) != cudaSuccess || n < 1) {
                 cudaGetLastError();
                 n = sm_count() / 2 - 2;
             }
@@ -548,23 +570,13 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
         cuts.start[n_teams] = (uint32_t)total;
     }
     cfg.gridDim = dim3(2 * n_teams * n_pairs);
-    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP>, tmK, tmV, s, c, L, cuts, per, gather ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW>, tmK, tmV, s, c, L, cuts, per, gather ? 1 : 0);
 }
 
 }  // namespace
 
 // True if the pair kernel serves this layout: what the single-CTA kernel needs, and an even number of row tiles.
 bool compress_tc2_supported(const Dims& s) { return s.M % (2 * kBM) == 0; }
-
-// True if the pair kernel can also write the kept-dim rows of the middle (its gather warps hold at most
-// kGatherItems chunks per thread and stage); otherwise the partition kernel writes them.
-bool compress_tc2_gathers(const Dims& s) {
-    const int n_pairs = s.M / (2 * kBM);
-    const int hp = s.Hkv % 2 == 0 ? 2 : 1;
-    const int n_tok = (kBK + n_pairs - 1) / n_pairs;
-    const int nf = s.nfk > s.nfv ? s.nfk : s.nfv;
-    return n_tok * hp * (nf >> 3) <= kGatherItems * 32 * kGatherWarps;
-}
 
 // Coefficients (the caller has zeroed them) and, with gather, the kept-dim rows of the middle tokens; the windows
 // and the counters are the caller's (the partition kernel).
@@ -574,12 +586,18 @@ cudaError_t launch_compress_tc2(const Dims& s, const CacheDev& c, const void* K,
     const int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;
     const int n_mid = L - n_init - n_local;
     if (n_mid <= 0) return cudaSuccess;
-    if (gather && !compress_tc2_gathers(s)) return cudaErrorInvalidValue;
     CUtensorMap tmK, tmV;
     if (!make_map2(&tmK, K, s, sb, st, sh, L) || !make_map2(&tmV, V, s, sb, st, sh, L)) return cudaErrorInvalidValue;
     const bool pair = s.Hkv % 2 == 0;                        // two heads share a CTA pair and its basis tiles
-    if (s.d == 128) return pair ? launch_tc2_t<128, 2>(tmK, tmV, s, c, L, n_mid, ordered, gather, stream) : launch_tc2_t<128, 1>(tmK, tmV, s, c, L, n_mid, ordered, gather, stream);
-    return pair ? launch_tc2_t<64, 2>(tmK, tmV, s, c, L, n_mid, ordered, gather, stream) : launch_tc2_t<64, 1>(tmK, tmV, s, c, L, n_mid, ordered, gather, stream);
+    const int nf = s.nfk > s.nfv ? s.nfk : s.nfv;
+    const bool many = gather && gather_rounds(s.M / (2 * kBM), pair ? 2 : 1, nf, kFewGather) > 1;
+    auto go = [&](auto d, auto hp) {
+        return many ? launch_tc2_t<d, hp, kManyGather>(tmK, tmV, s, c, L, n_mid, ordered, gather, stream)
+                    : launch_tc2_t<d, hp, kFewGather>(tmK, tmV, s, c, L, n_mid, ordered, gather, stream);
+    };
+    using std::integral_constant;
+    if (s.d == 128) return pair ? go(integral_constant<int, 128>{}, integral_constant<int, 2>{}) : go(integral_constant<int, 128>{}, integral_constant<int, 1>{});
+    return pair ? go(integral_constant<int, 64>{}, integral_constant<int, 2>{}) : go(integral_constant<int, 64>{}, integral_constant<int, 1>{});
 }
 
 }  // namespace fa
