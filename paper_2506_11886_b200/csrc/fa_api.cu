@@ -91,6 +91,11 @@ cudaError_t ensure_dynamic_smem_impl(const void* kernel, size_t bytes) {
     return cudaSuccess;
 }
 
+// The tensor-core path rounds the basis to bf16 (relative error 2^-9 per term); summed over n middle
+// tokens the coefficient error relative to the largest coefficient falls like 1 / sqrt(n): shorter
+// middles (where the tensor cores would idle anyway) take the fp32 kernel to stay within 1e-3.
+constexpr int kTcMinMid = 1024;
+
 static int ilog2_exact(int v) {
     int l = 0;
     while ((1 << l) < v) ++l;
@@ -411,7 +416,7 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
         // transform path: one store per coefficient, nothing to clear
         int log2S = 0;
         if (!compress_fft_supported(s, &log2S)) return FA_ERR_UNSUPPORTED;
-        if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, false, true, true, false, cs) != cudaSuccess)
+        if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, false, true, kNoTc, false, cs) != cudaSuccess)
             return FA_ERR_CUDA;
         if (L > 0 && launch_compress_fft(s, make_cache(*cache), layout->kv_dtype, K, V, sbb, stride_t, stride_h, L, log2S, cs) != cudaSuccess)
             return FA_ERR_CUDA;
@@ -423,16 +428,13 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
         }
         return FA_OK;
     }
-    // The tensor-core path rounds the basis to bf16 (relative error 2^-9 per term); summed over n middle
-    // tokens the coefficient error relative to the largest coefficient falls like 1 / sqrt(n): short
-    // middles (where the tensor cores would idle anyway) take the fp32 kernel to stay within 1e-3.
     const int n_mid_host = L - n_init - n_local;
-    const bool tc = L > 0 && n_mid_host >= 1024 && compress_tc_supported(s, layout->kv_dtype, sbb, stride_t, stride_h);
+    const bool tc = L > 0 && n_mid_host >= kTcMinMid && compress_tc_supported(s, layout->kv_dtype, sbb, stride_t, stride_h);
     // tensor-core path: its kernel also writes the kept-dim rows of the middle from the boxes it loads; the partition
     // kernel is left with the windows and the counters
     bool tc2 = tc && compress_tc2_supported(s);             // CTA pairs where the row tiles pair up
     bool tc_rows = tc && (tc2 || compress_tc_gathers(s));
-    if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, !tc, ordered, !tc_rows, true, cs) != cudaSuccess)
+    if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, !tc, ordered, tc_rows ? kTcMinMid : kNoTc, true, cs) != cudaSuccess)
         return FA_ERR_CUDA;
     if (tc2 && launch_compress_tc2(s, make_cache(*cache), K, V, sbb, stride_t, stride_h, L, ordered, tc_rows, cs) != cudaSuccess) {
         // the cluster launch was refused (e.g. a partitioned device): the single-CTA kernel does the same work; if it
@@ -441,7 +443,7 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
         tc2 = false;
         if (tc_rows && !compress_tc_gathers(s)) {
             tc_rows = false;
-            if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, false, ordered, true, true, cs) != cudaSuccess)
+            if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, false, ordered, kNoTc, true, cs) != cudaSuccess)
                 return FA_ERR_CUDA;
         }
     }
@@ -475,7 +477,7 @@ bool compress_is_pair_form(const fa_layout* layout, int64_t stride_b, int64_t st
     const int n_init = L < s.l_init ? L : s.l_init;
     const int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;
     const int64_t sbb = s.B > 1 ? stride_b : 0;
-    return L > 0 && L - n_init - n_local >= 1024 && compress_tc_supported(s, layout->kv_dtype, sbb, stride_t, stride_h) &&
+    return L > 0 && L - n_init - n_local >= kTcMinMid && compress_tc_supported(s, layout->kv_dtype, sbb, stride_t, stride_h) &&
            compress_tc2_supported(s);
 }
 }  // namespace
@@ -509,7 +511,7 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
     const bool ordered = (flags & FA_COMPRESS_ORDERED) != 0;
     for (int i = 0; i < n_layers; ++i) {
         const Dims s = make_dims(layouts[i]);
-        if (launch_compress(s, make_cache(caches[i]), layouts[i].kv_dtype, K[i], V[i], stride_b, stride_t, stride_h, L, false, ordered, false,
+        if (launch_compress(s, make_cache(caches[i]), layouts[i].kv_dtype, K[i], V[i], stride_b, stride_t, stride_h, L, false, ordered, kTcMinMid,
                             true, cs, i > 0) != cudaSuccess)
             return FA_ERR_CUDA;
     }
@@ -542,15 +544,29 @@ fa_status fa_compress_ragged(const fa_layout* layout, fa_cache* cache, const voi
     st = check_cache(layout, cache);
     if (st != FA_OK) return st;
     if (!lengths || stride_b < 0) return FA_ERR_INVALID_ARG;
-    // every batch row is a one-row cache of its own: same index sets and status word, its own slices
-    fa_layout one = *layout;
-    one.batch = 1;
-    fa_cache_sizes sz;
-    st = fa_cache_sizes_of(&one, &sz);
-    if (st != FA_OK) return st;
-    const size_t eb = elt_bytes(layout->kv_dtype);
+    const Dims all = make_dims(*layout);
+    int Lmax = 0;
+    bool tc_row = false;
     for (int b = 0; b < layout->batch; ++b) {
         if (lengths[b] < 0) return FA_ERR_INVALID_ARG;
+        if (mid_of(all, lengths[b]) > all.max_mid) return FA_ERR_CAPACITY;
+        Lmax = lengths[b] > Lmax ? lengths[b] : Lmax;
+        tc_row = tc_row || mid_of(all, lengths[b]) >= kTcMinMid;
+    }
+    if (Lmax > 0) {
+        if (!K || !V || !aligned16(K) || !aligned16(V)) return FA_ERR_INVALID_ARG;
+        if (stride_t < layout->head_dim || stride_h < layout->head_dim) return FA_ERR_INVALID_ARG;
+    }
+    if ((stride_b | stride_t | stride_h) & 7) return FA_ERR_INVALID_ARG;
+    // Every batch row is a one-row cache of its own: same index sets and status word, its own slices.  `rows` rows from
+    // row b on as a cache and a layout:
+    fa_layout part = *layout;
+    fa_cache_sizes sz;
+    part.batch = 1;
+    st = fa_cache_sizes_of(&part, &sz);
+    if (st != FA_OK) return st;
+    const size_t eb = elt_bytes(layout->kv_dtype);
+    auto slice = [&](int b) {
         fa_cache row = *cache;
         auto at = [&](void* p, size_t bytes) -> void* { return p ? static_cast<char*>(p) + (size_t)b * bytes : nullptr; };
         row.k_init = at(cache->k_init, sz.k_init);     row.v_init = at(cache->v_init, sz.v_init);
@@ -559,10 +575,51 @@ fa_status fa_compress_ragged(const fa_layout* layout, fa_cache* cache, const voi
         row.coef_k = static_cast<float*>(at(cache->coef_k, sz.coef_k));
         row.coef_v = static_cast<float*>(at(cache->coef_v, sz.coef_v));
         row.state = static_cast<int32_t*>(at(cache->state, sz.state));
-        const char* Kb = static_cast<const char*>(K) + (size_t)b * (size_t)stride_b * eb;
-        const char* Vb = static_cast<const char*>(V) + (size_t)b * (size_t)stride_b * eb;
-        st = fa_compress(&one, &row, lengths[b] ? Kb : (K ? Kb : nullptr), lengths[b] ? Vb : (V ? Vb : nullptr), stride_b, stride_t,
-                         stride_h, lengths[b], ws, ws_bytes, stream);
+        return row;
+    };
+    auto prefill = [&](const void* X, int b) -> const void* {
+        return X ? static_cast<const char*>(X) + (size_t)b * (size_t)stride_b * eb : nullptr;
+    };
+    // One set of launches for up to kMaxRagged rows: the partition kernel over all of them (rows of too short a middle for
+    // the tensor cores get their coefficients from the CUDA-core kernel behind it), then the pair contraction over the
+    // token blocks of the long rows laid end to end.  (A set per row: 201 us for six rows of 3.3 to 12.3 K tokens
+    // of a 24 / 8 head layout, each contraction too small for the chip.)  The boxes of a row's last block may reach up
+    // to 63 tokens past its middle: with a local window of that size they stay inside the row.
+    const int64_t sbt = layout->batch > 1 ? stride_b : 0;
+    const bool tc_ok = compress_tc_supported(all, layout->kv_dtype, sbt, stride_t, stride_h);
+    const bool pairs = tc_ok && compress_tc2_supported(all) && all.l_local >= 63;
+    cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    int b0 = 0;
+    if (Lmax > 0 && (pairs || !tc_row || !tc_ok)) {
+        for (; b0 < layout->batch; b0 += part.batch) {
+            part.batch = layout->batch - b0 < kMaxRagged ? layout->batch - b0 : kMaxRagged;
+            const fa_cache rows = slice(b0);
+            const Dims s = make_dims(part);
+            RowLens lens = {};
+            lens.n = part.batch;
+            int L = 0, shortest = 0;
+            for (int i = 0; i < part.batch; ++i) {
+                lens.len[i] = lengths[b0 + i];
+                L = lens.len[i] > L ? lens.len[i] : L;
+                shortest += mid_of(s, lens.len[i]) < kTcMinMid;
+            }
+            if (L == 0) { L = Lmax; }                     // (the kernels go by the rows' lengths)
+            const void *Kb = prefill(K, b0), *Vb = prefill(V, b0);
+            const bool tc = pairs && shortest < part.batch;
+            if (launch_compress(s, make_cache(rows), layout->kv_dtype, Kb, Vb, stride_b, stride_t, stride_h, L, true, false,
+                                tc ? kTcMinMid : kNoTc, true, cs, false, &lens) != cudaSuccess)
+                return FA_ERR_CUDA;
+            if (tc && launch_compress_tc2(s, make_cache(rows), Kb, Vb, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, false, true, cs, &lens,
+                                          kTcMinMid) != cudaSuccess) {
+                cudaGetLastError();                       // the cluster launch was refused: these rows and the rest one by one
+                break;
+            }
+        }
+    }
+    part.batch = 1;
+    for (int b = b0; b < layout->batch; ++b) {
+        fa_cache row = slice(b);
+        st = fa_compress(&part, &row, prefill(K, b), prefill(V, b), stride_b, stride_t, stride_h, lengths[b], ws, ws_bytes, stream);
         if (st != FA_OK) return st;
     }
     return FA_OK;

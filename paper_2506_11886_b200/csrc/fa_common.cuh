@@ -100,16 +100,31 @@ int sm_count();                          // SMs of the current device, cached pe
 bool cooperative_launch_supported();     // of the current device, cached per device
 fa_status check_layout(const fa_layout* l);
 
+// Prompt lengths of the batch rows of one compress launch: n = 0 says that all rows have the launch's L tokens.
+constexpr int kMaxRagged = 64;
+struct RowLens {
+    int32_t n;
+    int32_t len[kMaxRagged];
+};
+__host__ __device__ inline int row_len(const RowLens& r, int L, int b) { return r.n ? r.len[b] : L; }
+// Middle tokens of a prompt of L tokens.
+__host__ __device__ inline int mid_of(const Dims& s, int L) {
+    const int rest = L - (L < s.l_init ? L : s.l_init);
+    return rest > s.l_local ? rest - s.l_local : 0;
+}
+// Rows with at least tc_min middle tokens are the tensor-core path's (their kept-dim rows too); kNoTc: none are.
+constexpr int kNoTc = 0x7fffffff;
+
 // Kernel launchers (defined next to their kernels).  All return the launch error, if any.
 cudaError_t launch_validate(const Dims&, const CacheDev&, cudaStream_t);
 cudaError_t launch_compress(const Dims&, const CacheDev&, int dtype, const void* K, const void* V, int64_t sb,
-                            int64_t st, int64_t sh, int L, bool with_coef, bool ordered, bool mid_rows, bool zero_coef, cudaStream_t,
-                            bool chained = false);
+                            int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, bool zero_coef, cudaStream_t,
+                            bool chained = false, const RowLens* lens = nullptr);
 bool compress_tc_gathers(const Dims& s);
 // The same path on CTA pairs (fa_compress_tc2.cu): needs an even number of 128-row tiles.
 bool compress_tc2_supported(const Dims& s);
 cudaError_t launch_compress_tc2(const Dims&, const CacheDev&, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh,
-                                int L, bool ordered, bool gather, cudaStream_t);
+                                int L, bool ordered, bool gather, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
 // Tensor-core reconstruction of the dimension selection (fa_select_tc.cu).
 bool reconstruct_tc_supported(const Dims& s, int dtype, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int n_mid);
 size_t reconstruct_tc_scratch_bytes(const Dims& s);

@@ -47,11 +47,24 @@ cudaError_t launch_validate(const Dims& s, const CacheDev& c, cudaStream_t st) {
 // per chunk, then one thread per output chunk either copies it (window rows) or gathers its dims
 // through the index set (kept-dim rows; for V^mu of bf16 caches the chunk it writes is the permuted one).
 constexpr int kRowsPerCta = 64;
+// The i-th chunk that holds window tokens (chunk 0 always counts: it writes the counters), and how many there are.
+__host__ __device__ inline int window_skip(int L, int n_init, int n_local, int* first) {
+    int a = (n_init + kRowsPerCta - 1) / kRowsPerCta;    // first chunk past the initial window
+    const int c = (L - n_local) / kRowsPerCta;           // first chunk with a token of the local window
+    if (a < 1) a = 1;
+    *first = a;
+    return c > a ? c - a : 0;
+}
+__host__ __device__ inline int window_chunk(int i, int L, int n_init, int n_local) {
+    int a;
+    const int skip = window_skip(L, n_init, n_local, &a);
+    return i < a ? i : i + skip;
+}
 
 template <typename KV>
 __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev c, const KV* __restrict__ K,
                                                                    const KV* __restrict__ V, int64_t sb, int64_t st,
-                                                                   int64_t sh, int L, int mid_rows, int skip_a, int skip_c, int zero_coef) {
+                                                                   int64_t sh, int Lmax, const __grid_constant__ RowLens lens, int tc_min, int zero_coef) {
     constexpr int EPC = 16 / (int)sizeof(KV);            // elements per chunk
     extern __shared__ __align__(16) unsigned char gsm[];
     // the contraction kernel behind this one may start at once (programmatic dependent launch): it waits for this
@@ -60,6 +73,7 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
     KV* rows_s = reinterpret_cast<KV*>(gsm);                                         // [64][d]
     int32_t* idf_s = reinterpret_cast<int32_t*>(gsm + (size_t)kRowsPerCta * s.d * sizeof(KV));   // [nfull]
     const int h = blockIdx.y, b = blockIdx.z >> 1, side = blockIdx.z & 1;
+    const int L = row_len(lens, Lmax, b);
     const int n_init = min(L, s.l_init);
     const int n_local = min(L - n_init, s.l_local);
     const int n_mid = L - n_init - n_local;
@@ -82,8 +96,9 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
     void* w_init = side == 0 ? c.k_init : c.v_init;
     void* w_local = side == 0 ? c.k_local : c.v_local;
     void* w_mid = side == 0 ? c.k_mid : c.v_mid;
-    // without the kept-dim rows (the tensor-core kernel writes them) the chunks [skip_a, skip_c) of middle tokens only are not launched
-    const int chunk = (int)blockIdx.x < skip_a ? (int)blockIdx.x : (int)blockIdx.x + (skip_c - skip_a);
+    // without the kept-dim rows (the tensor-core kernel writes them) the chunks of middle tokens only are left out
+    const bool mid_rows = n_mid < tc_min;
+    const int chunk = mid_rows ? (int)blockIdx.x : window_chunk((int)blockIdx.x, L, n_init, n_local);
     const int t0 = chunk * kRowsPerCta, nrow = min(L - t0, kRowsPerCta);
     const int cpr = s.d / EPC;                            // chunks per input row
     for (int i = threadIdx.x; i < nfull; i += blockDim.x) idf_s[i] = idf[i];
@@ -136,7 +151,7 @@ constexpr int kTM = 32, kTJ = 64;
 template <typename KV>
 __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, const KV* __restrict__ K,
                                                             const KV* __restrict__ V, int64_t sb, int64_t st, int64_t sh,
-                                                            int L, int chunks_per_split) {
+                                                            int Lmax, int chunks_per_split, const __grid_constant__ RowLens lens, int tc_min) {
     extern __shared__ float smem[];
     int side = blockIdx.z & 1;
     int bh = blockIdx.z >> 1;
@@ -144,9 +159,9 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
     int nfull = side == 0 ? s.nfk : s.nfv;
     int ncomp = s.d - nfull;
     if (ncomp == 0) return;
-    int n_init = min(L, s.l_init);
-    int n_local = min(L - n_init, s.l_local);
-    int n_mid = L - n_init - n_local;
+    const int L = row_len(lens, Lmax, b);
+    const int n_init = min(L, s.l_init), n_mid = mid_of(s, L);
+    if (n_mid >= tc_min) return;                         // the tensor-core kernel's row
     const KV* X = (side == 0 ? K : V) + (size_t)b * sb + (size_t)h * sh;
     const int32_t* idc = (side == 0 ? c.idx_comp_k : c.idx_comp_v) + (size_t)h * ncomp;
     float* coef = coef_rows(side == 0 ? c.coef_k : c.coef_v, s, b, h, ncomp);
@@ -210,17 +225,18 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
 
 template <typename KV>
 static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb,
-                                     int64_t st, int64_t sh, int L, bool with_coef, bool ordered, bool mid_rows, bool zero_coef, bool chained,
-                                     cudaStream_t stream) {
-    int chunks_rows = (L + kRowsPerCta - 1) / kRowsPerCta;
-    if (chunks_rows < 1) chunks_rows = 1;
-    int skip_a = 0, skip_c = 0;
-    if (!mid_rows) {
-        const int ni = L < s.l_init ? L : s.l_init, nl = (L - ni) < s.l_local ? (L - ni) : s.l_local;
-        skip_a = (ni + kRowsPerCta - 1) / kRowsPerCta;          // first chunk past the initial window
-        skip_c = (L - nl) / kRowsPerCta;                        // first chunk with a token of the local window
-        if (skip_a < 1) skip_a = 1;                             // chunk 0 always runs: it writes the counters
-        if (skip_c < skip_a) skip_c = skip_a;
+                                     int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, bool zero_coef, bool chained,
+                                     const RowLens* lens, cudaStream_t stream) {
+    RowLens rl = {};
+    if (lens) rl = *lens;
+    // chunks and short middles (not the tensor-core kernel's) of the longest row
+    int chunks_rows = 1, n_mid = 0;
+    for (int b = 0; b < (rl.n ? rl.n : 1); ++b) {
+        const int Lb = row_len(rl, L, b), ni = Lb < s.l_init ? Lb : s.l_init, nl = (Lb - ni) < s.l_local ? (Lb - ni) : s.l_local;
+        int chunks = (Lb + kRowsPerCta - 1) / kRowsPerCta, first;
+        if (Lb - ni - nl >= tc_min) chunks -= window_skip(Lb, ni, nl, &first);
+        else if (Lb - ni - nl > n_mid) n_mid = Lb - ni - nl;
+        if (chunks > chunks_rows) chunks_rows = chunks;
     }
     constexpr int EPC = 16 / (int)sizeof(KV);
     if (s.d % EPC || s.nfk % EPC || s.nfv % EPC || sb % EPC || st % EPC || sh % EPC || (reinterpret_cast<uintptr_t>(K) & 15) ||
@@ -232,7 +248,7 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     if (err != cudaSuccess) return err;
     {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(chunks_rows - (skip_c - skip_a), s.Hkv, s.B * 2);
+        cfg.gridDim = dim3(chunks_rows, s.Hkv, s.B * 2);
         cfg.blockDim = dim3(256);
         cfg.dynamicSmemBytes = gsmem;
         cfg.stream = stream;
@@ -242,12 +258,9 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
         cfg.attrs = attr;
         cfg.numAttrs = chained ? 1 : 0;
         err = cudaLaunchKernelEx(&cfg, partition_gather_kernel<KV>, s, c, static_cast<const KV*>(K), static_cast<const KV*>(V), sb, st, sh, L,
-                                 mid_rows ? 1 : 0, skip_a, skip_c, zero_coef ? 1 : 0);
+                                 rl, tc_min, zero_coef ? 1 : 0);
     }
     if (err != cudaSuccess) return err;
-    int n_init = L < s.l_init ? L : s.l_init;
-    int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;
-    int n_mid = L - n_init - n_local;
     int max_comp = s.dck > s.dcv ? s.dck : s.dcv;
     if (n_mid == 0 || max_comp == 0 || !with_coef) return cudaSuccess;
     int row_tiles = (s.M + kTM - 1) / kTM;
@@ -262,18 +275,19 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     err = ensure_dynamic_smem(compress_coef_kernel<KV>, smem);
     if (err != cudaSuccess) return err;
     compress_coef_kernel<KV><<<dim3(row_tiles, n_tsplit, s.B * s.Hkv * 2), 256, smem, stream>>>(
-        s, c, static_cast<const KV*>(K), static_cast<const KV*>(V), sb, st, sh, L, cps);
+        s, c, static_cast<const KV*>(K), static_cast<const KV*>(V), sb, st, sh, L, cps, rl, tc_min);
     return cudaGetLastError();
 }
 
 // with_coef = false runs only the partition / gather kernel (the tensor-core or the transform path computes the
-// coefficients); mid_rows = false leaves the kept-dim rows of the middle out too (windows and counters only);
+// coefficients); rows with at least tc_min middle tokens get no kept-dim rows and no coefficients here (windows and
+// counters only: the tensor-core kernel writes the rest); lens: prompt lengths of the batch rows (at most L), or none;
 // zero_coef clears the coefficients in the same launch (for the contraction kernels, which add to them).
 cudaError_t launch_compress(const Dims& s, const CacheDev& c, int dtype, const void* K, const void* V, int64_t sb,
-                            int64_t st, int64_t sh, int L, bool with_coef, bool ordered, bool mid_rows, bool zero_coef,
-                            cudaStream_t stream, bool chained) {
-    if (dtype == FA_BF16) return launch_compress_t<__nv_bfloat16>(s, c, K, V, sb, st, sh, L, with_coef, ordered, mid_rows, zero_coef, chained, stream);
-    return launch_compress_t<float>(s, c, K, V, sb, st, sh, L, with_coef, ordered, mid_rows, zero_coef, chained, stream);
+                            int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, bool zero_coef,
+                            cudaStream_t stream, bool chained, const RowLens* lens) {
+    if (dtype == FA_BF16) return launch_compress_t<__nv_bfloat16>(s, c, K, V, sb, st, sh, L, with_coef, ordered, tc_min, zero_coef, chained, lens, stream);
+    return launch_compress_t<float>(s, c, K, V, sb, st, sh, L, with_coef, ordered, tc_min, zero_coef, chained, lens, stream);
 }
 
 }  // namespace fa

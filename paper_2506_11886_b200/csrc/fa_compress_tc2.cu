@@ -54,6 +54,12 @@ using namespace umma;
 // then zero plus two terms, and the sum of two floats does not depend on which arrives first).
 constexpr int kMaxTeams = 96;
 struct TeamCuts { uint32_t start[kMaxTeams + 1]; };
+// Rows of different length: the position of every row's first block (a row of fewer than the tensor-core path's
+// tokens has none), and their lengths.  lens.n = 0: all rows are alike.
+struct RowCuts {
+    RowLens lens;
+    uint32_t first[kMaxRagged + 1];
+};
 
 // D = head dim (64 or 128): N = 2 D accumulator columns per KV head (K dims, then V dims); HP heads share the pair
 // and its generated basis tiles (HP * N <= 512 tensor-memory columns).  grid 2 * teams * (M / 256), clusters of two.
@@ -61,8 +67,8 @@ struct TeamCuts { uint32_t start[kMaxTeams + 1]; };
 template <int D, int HP, int kGatherWarps>
 __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV, Dims s,
-                                                                     CacheDev c, int L, const __grid_constant__ TeamCuts cuts,
-                                                                     int per, int gather) {
+                                                                     CacheDev c, int Lall, const __grid_constant__ TeamCuts cuts,
+                                                                     const __grid_constant__ RowCuts rows, int per, int gather) {
     constexpr int N = 2 * D;
     constexpr int kABytes = kBM * kBK * 2;                 // 16 KB basis tile
     constexpr int kBoxBytes = kBK * 64 * 2;                // 8 KB per [64 tokens x 64 dims] box
@@ -95,25 +101,34 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
     const int cluster = (int)blockIdx.x >> 1, team = cluster / n_pairs, pair = cluster - team * n_pairs;
     const int mt = 2 * pair + (int)rank;                   // this CTA's row tile, the same in every segment
     const int n_hg = s.Hkv / HP;
-    const int n_init = min(L, s.l_init);
-    const int n_local = min(L - n_init, s.l_local);
-    const int n_mid = L - n_init - n_local;
-    const int nkb = (n_mid + kBK - 1) / kBK;
+    const int n_init = s.l_init;                           // every row with a middle has its windows full
+    const int n_mid_all = mid_of(s, Lall), nkb_all = (n_mid_all + kBK - 1) / kBK;
     uint32_t pos_begin, pos_end;
     if (per > 0) {                                         // uniform cut: every unit in ceil(blocks / per) pieces of per blocks
-        const int pieces = (nkb + per - 1) / per, unit = team / pieces, piece = team - unit * pieces;
-        pos_begin = (uint32_t)unit * (uint32_t)nkb + (uint32_t)(piece * per);
-        pos_end = (uint32_t)unit * (uint32_t)nkb + (uint32_t)min(nkb, (piece + 1) * per);
+        const int pieces = (nkb_all + per - 1) / per, unit = team / pieces, piece = team - unit * pieces;
+        pos_begin = (uint32_t)unit * (uint32_t)nkb_all + (uint32_t)(piece * per);
+        pos_end = (uint32_t)unit * (uint32_t)nkb_all + (uint32_t)min(nkb_all, (piece + 1) * per);
     } else {
         pos_begin = cuts.start[team];
         pos_end = cuts.start[team + 1];
     }
     // the segment that starts at position pos: its unit (batch b, heads h0 ...) and blocks kb0 .. kb1
-    struct Seg { int b, h0, kb0, kb1; };
+    struct Seg { int b, h0, kb0, kb1, n_mid; };
     auto seg_at = [&](uint32_t pos) {
-        const int unit = (int)(pos / (uint32_t)nkb), kb0 = (int)(pos - (uint32_t)unit * (uint32_t)nkb);
-        const int kb1 = (int)min((uint32_t)nkb, (uint32_t)kb0 + (pos_end - pos));
-        return Seg{unit / n_hg, (unit % n_hg) * HP, kb0, kb1};
+        int b = 0, n_mid = n_mid_all, nkb = nkb_all;
+        const uint32_t end = pos_end;
+        uint32_t off = pos;
+        if (rows.lens.n) {
+            while (pos >= rows.first[b + 1]) ++b;
+            off = pos - rows.first[b];
+            n_mid = mid_of(s, rows.lens.len[b]);
+            nkb = (n_mid + kBK - 1) / kBK;
+        }
+        int unit = (int)(off / (uint32_t)nkb);
+        const int kb0 = (int)(off - (uint32_t)unit * (uint32_t)nkb);
+        const int kb1 = (int)min((uint32_t)nkb, (uint32_t)kb0 + (end - pos));
+        if (!rows.lens.n) { b = unit / n_hg; unit -= b * n_hg; }
+        return Seg{b, unit * HP, kb0, kb1, n_mid};
     };
 
     // The contraction of the next layer (a call over several layers launches them one behind the other, programmatically)
@@ -293,7 +308,7 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
 #pragma unroll
                         for (int u = 0; u < kGatherItems; ++u) {
                             const int j = jb + (meta[u] & 0xff);
-                            if (meta[u] >= 0 && j < n_mid) {
+                            if (meta[u] >= 0 && j < g.n_mid) {
                                 const int hh = (meta[u] >> 8) & 0xf, lch = meta[u] >> 16;
                                 const int cls = p2 ? (j & (s.P - 1)) : j % s.P, slot = p2 ? (j >> lgP) : j / s.P;
                                 const int nfull = nf_side;
@@ -353,7 +368,7 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
                         asm("mov.b64 %0, {%1,%2};" : "=l"(C) : "f"(__cosf(aa)), "f"(__cosf(ab)));
                         asm("mov.b64 %0, {%1,%2};" : "=l"(S) : "f"(__sinf(aa)), "f"(__sinf(ab)));
                     }
-                    const bool whole = row_on && j0 + 16 <= n_mid;      // no masking needed in the common case
+                    const bool whole = row_on && j0 + 16 <= g.n_mid;      // no masking needed in the common case
 #pragma unroll
                     for (int ch = 0; ch < 2; ++ch) {       // 8 tokens = one 16-byte chunk of each row
                         uint32_t wc[4], wsn[4];
@@ -364,7 +379,7 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
                             asm("mov.b64 {%0,%1}, %2;" : "=f"(s0), "=f"(s1) : "l"(S));
                             if (!whole) {
                                 const int j = j0 + ch * 8 + i2 * 2;
-                                const bool v0 = row_on && j < n_mid, v1 = row_on && j + 1 < n_mid;
+                                const bool v0 = row_on && j < g.n_mid, v1 = row_on && j + 1 < g.n_mid;
                                 c0 = v0 ? c0 : 0.f; s0 = v0 ? s0 : 0.f; c1 = v1 ? c1 : 0.f; s1 = v1 ? s1 : 0.f;
                             }
                             const __nv_bfloat162 pc = __floats2bfloat162_rn(c0, c1);
@@ -484,7 +499,7 @@ bool make_map2(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int
 }
 
 template <int D, int HP, int GW>
-cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, int n_mid,
+cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, const RowCuts& rows,
                          bool ordered, bool gather, cudaStream_t stream) {
     constexpr size_t stage = (size_t)kBM * kBK * 2 + (size_t)HP * (D / 64) * kBK * 64 * 2;
     constexpr size_t n_stages = (200 * 1024) / stage < 6 ? (200 * 1024) / stage : 6;
@@ -492,9 +507,9 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
     cudaError_t err = ensure_dynamic_smem(compress_tc2_kernel<D, HP, GW>, smem);
     if (err != cudaSuccess) return err;
     const int n_pairs = s.M / (2 * kBM);
-    const int nkb = (n_mid + kBK - 1) / kBK;
-    const long long n_units = (long long)(s.Hkv / HP) * s.B;
-    const long long total = n_units * nkb;                      // positions: the blocks of all units, end to end
+    const int nkb = (mid_of(s, L) + kBK - 1) / kBK;
+    const long long n_hg = s.Hkv / HP, n_units = n_hg * s.B;
+    const long long total = rows.lens.n ? (long long)rows.first[rows.lens.n] : n_units * nkb;   // positions: the blocks of all units, end to end
     if (total <= 0 || total >= (1ll << 31)) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(threads_tc(GW));
@@ -542,6 +557,13 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
         // Equal cost per team: a segment costs its blocks plus kEpi (epilogue, pipeline refill, in blocks).  The smallest
         // budget with which the walk below covers all positions in n_teams teams, by bisection.
         constexpr long long kEpi = 12, kMinSeg = 8;
+        auto unit_end_of = [&](long long pos) {
+            if (!rows.lens.n) return (pos / nkb + 1) * nkb;
+            int b = 0;
+            while (pos >= (long long)rows.first[b + 1]) ++b;
+            const long long first = rows.first[b], per_unit = ((long long)rows.first[b + 1] - first) / n_hg;
+            return first + ((pos - first) / per_unit + 1) * per_unit;
+        };
         auto walk = [&](long long budget, uint32_t* start) {
             long long pos = 0;
             int t = 0;
@@ -549,7 +571,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
                 if (start) start[t] = (uint32_t)pos;
                 long long left = budget;
                 while (pos < total && left >= kEpi + kMinSeg) {
-                    const long long unit_end = (pos / nkb + 1) * nkb;
+                    const long long unit_end = unit_end_of(pos);
                     long long take = unit_end - pos < left - kEpi ? unit_end - pos : left - kEpi;
                     if (unit_end - pos - take > 0 && unit_end - pos - take < kMinSeg) take = unit_end - pos - kMinSeg;   // no crumbs for the next team
                     if (take <= 0) break;
@@ -570,7 +592,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
         cuts.start[n_teams] = (uint32_t)total;
     }
     cfg.gridDim = dim3(2 * n_teams * n_pairs);
-    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW>, tmK, tmV, s, c, L, cuts, per, gather ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW>, tmK, tmV, s, c, L, cuts, rows, per, gather ? 1 : 0);
 }
 
 }  // namespace
@@ -579,21 +601,34 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
 bool compress_tc2_supported(const Dims& s) { return s.M % (2 * kBM) == 0; }
 
 // Coefficients (the caller has zeroed them) and, with gather, the kept-dim rows of the middle tokens; the windows
-// and the counters are the caller's (the partition kernel).
+// and the counters are the caller's (the partition kernel).  lens: prompt lengths of the batch rows (at most L; rows with
+// fewer than tc_min middle tokens are left out), or none.
 cudaError_t launch_compress_tc2(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb, int64_t st,
-                                int64_t sh, int L, bool ordered, bool gather, cudaStream_t stream) {
-    const int n_init = L < s.l_init ? L : s.l_init;
-    const int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;
-    const int n_mid = L - n_init - n_local;
-    if (n_mid <= 0) return cudaSuccess;
+                                int64_t sh, int L, bool ordered, bool gather, cudaStream_t stream, const RowLens* lens, int tc_min) {
+    RowCuts rows = {};
+    if (lens && lens->n) {
+        if (ordered || lens->n != s.B) return cudaErrorInvalidValue;
+        rows.lens = *lens;
+        const int n_hg = s.Hkv % 2 == 0 ? s.Hkv / 2 : s.Hkv;
+        long long at = 0;
+        for (int b = 0; b < lens->n; ++b) {
+            const int m = mid_of(s, lens->len[b]);
+            at += m >= tc_min ? (long long)n_hg * ((m + kBK - 1) / kBK) : 0;
+            if (at >= (1ll << 31)) return cudaErrorInvalidValue;
+            rows.first[b + 1] = (uint32_t)at;
+        }
+        if (at == 0) return cudaSuccess;
+    } else if (mid_of(s, L) <= 0) {
+        return cudaSuccess;
+    }
     CUtensorMap tmK, tmV;
     if (!make_map2(&tmK, K, s, sb, st, sh, L) || !make_map2(&tmV, V, s, sb, st, sh, L)) return cudaErrorInvalidValue;
     const bool pair = s.Hkv % 2 == 0;                        // two heads share a CTA pair and its basis tiles
     const int nf = s.nfk > s.nfv ? s.nfk : s.nfv;
     const bool many = gather && gather_rounds(s.M / (2 * kBM), pair ? 2 : 1, nf, kFewGather) > 1;
     auto go = [&](auto d, auto hp) {
-        return many ? launch_tc2_t<d, hp, kManyGather>(tmK, tmV, s, c, L, n_mid, ordered, gather, stream)
-                    : launch_tc2_t<d, hp, kFewGather>(tmK, tmV, s, c, L, n_mid, ordered, gather, stream);
+        return many ? launch_tc2_t<d, hp, kManyGather>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
+                    : launch_tc2_t<d, hp, kFewGather>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
     };
     using std::integral_constant;
     if (s.d == 128) return pair ? go(integral_constant<int, 128>{}, integral_constant<int, 2>{}) : go(integral_constant<int, 128>{}, integral_constant<int, 1>{});

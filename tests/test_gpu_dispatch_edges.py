@@ -1,8 +1,9 @@
 """Layouts at the edges of the kernel dispatch: each test names the branch it takes and checks it against the oracle."""
 import pytest
+import torch
 
 from paper_2506_11886_b200 import fa, synth
-from tests.parity_util import make_pair
+from tests.parity_util import layout_of, make_pair
 
 pytestmark = pytest.mark.gpu
 
@@ -18,3 +19,33 @@ def test_pair_compress_writes_many_kept_dims(kw):
                                             L_local=64), **kw, **({"Hq": kw["Hkv"]} if "Hkv" in kw else {})})
     pair, _ = make_pair(shape, seed=31, P=2, max_mid=shape.T, algo=fa.FA_DECODE_DIRECT)
     pair.check_state()
+
+
+@pytest.mark.parametrize("B,M,lengths", [
+    (5, 256, [0, 2600, 1091, 1092, 70]),                 # empty, long, one below / at the tensor path's 1024 middle tokens, no middle
+    (3, 512, [1100, 1155, 1156]),                        # middles of 1032, 1087, 1088 tokens: ragged and whole last blocks
+    (66, 256, [1100 + 7 * (b % 9) for b in range(66)]),  # more rows than one launch takes
+    (2, 128, [2000, 300]),                               # odd number of row tiles: row by row
+])
+def test_ragged_compress_in_one_launch_equals_row_by_row(B, M, lengths):
+    shape = synth.Shape("ragged", B=B, layers=1, Hq=4, Hkv=2, d=64, L=max(lengths), dtype="bf16", n_full_k=16, n_full_v=24,
+                        M=M, T=4096, L_init=4, L_local=64)
+    stream = synth.KVStream(shape, seed=5, device="cuda")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    for b, n in enumerate(lengths):
+        K[b, n:], V[b, n:] = float("nan"), float("nan")   # rows past a prompt's length are not read
+    layout = layout_of(shape, max_mid=shape.T, P=8)
+    one = layout_of(shape.with_(B=1), max_mid=shape.T, P=8)
+    got, ws = fa.Cache(layout, stream.idx_full_k, stream.idx_full_v), fa.new_workspace(layout)
+    got.coef_k.fill_(7.0)
+    fa.fa_compress_ragged(layout, got, K, V, lengths, ws)
+    for b in sorted({0, 1, B // 2, B - 2, B - 1}):
+        ref = fa.Cache(one, stream.idx_full_k, stream.idx_full_v)
+        fa.fa_compress(one, ref, K[b:b + 1, :lengths[b]], V[b:b + 1, :lengths[b]], ws)
+        for n in ("k_init", "v_init", "k_local", "v_local", "k_mid", "v_mid", "state"):
+            assert torch.equal(getattr(got, n)[b], getattr(ref, n)[0]), (b, n)
+        for n in ("coef_k", "coef_v"):
+            g, r = getattr(got, n)[b], getattr(ref, n)[0]
+            # (basis phasors are seeded where a CTA's blocks begin: some bf16 roundings of the basis differ)
+            assert (g - r).abs().max() <= 2e-4 * r.abs().max() + 1e-6, (b, n)
+    assert fa.fa_poll_status(got) == fa.FA_OK
