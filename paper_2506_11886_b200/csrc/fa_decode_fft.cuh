@@ -202,12 +202,6 @@ __device__ __forceinline__ float2 cis_frac(float frac) {
     const float a = 6.283185307179586f * (frac - (frac >= 0.5f ? 1.0f : 0.0f));
     return make_float2(__cosf(a), __sinf(a));
 }
-// Order-independent accumulation of fp32 values: 64-bit fixed point, 30 fractional bits.  The sums here are
-// probabilities (<= 1 each, at most 2^20 of them) times bf16 values, far inside the 33 integer bits.
-constexpr float kFix = 1073741824.0f, kFixInv = 1.0f / 1073741824.0f;     // (scaling by a power of two is exact in fp32)
-__device__ __forceinline__ void fix_add(long long* p, float v) {
-    atomicAdd(reinterpret_cast<unsigned long long*>(p), (unsigned long long)__float2ll_rn(v * kFix));
-}
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -415,7 +409,7 @@ __device__ __forceinline__ WinSegs win_segments(int t0, int t1, int n_init, int 
 }
 
 struct FftSmem {
-    int stages_off, fbuf_off, kb_off, pbt_off, twf_off, rev_off, E_off, ut_off, z_off, o_off, red_off, pend_off, zero_off, total;
+    int stages_off, fbuf_off, kb_off, pbt_off, twf_off, rev_off, E_off, ut_off, z_off, o_off, inv_off, red_off, pend_off, zero_off, total;
     int fb_floats, pbs;
 };
 // True if the kernel packs two residue classes of ONE query head into a complex transform (one query head per KV head:
@@ -431,7 +425,8 @@ __host__ __device__ inline FftSmem fft_smem_layout(int log2S, int k, int GH, int
     L.zero_off = off; off += 16;
     off = 1024;                                           // stages are 1024-byte aligned (swizzled window tiles)
     L.stages_off = off; off += ring_stages(occ, split) * kStageBytes;
-    L.fbuf_off = off; off += 4 * NT * L.fb_floats;
+    // (also the warps' output fragments, [warp][slot][d], while no transform is under way)
+    L.fbuf_off = off; off += 4 * (NT * L.fb_floats > kWarps * GH * d ? NT * L.fb_floats : kWarps * GH * d);
     off = (off + 15) / 16 * 16;
     L.kb_off = off; off += 4 * NT * S * GH;               // kept-dim scores of the batch, natural token order
     off = (off + 15) / 16 * 16;
@@ -444,7 +439,9 @@ __host__ __device__ inline FftSmem fft_smem_layout(int log2S, int k, int GH, int
     L.ut_off = off; off += (8 * k * GH + 15) / 16 * 16;
     L.z_off = off; off += (8 * k * GH + 15) / 16 * 16;
     off = (off + 15) / 16 * 16;
-    L.o_off = off; off += 8 * GH * d;
+    L.o_off = off; off += 4 * GH * d;
+    L.inv_off = off; off += 2 * d;
+    off = (off + 15) / 16 * 16;
     L.red_off = off; off += 4 * ((split ? kSplitWarps : kWarps) * GH + GH + 8);
     off = (off + 15) / 16 * 16;
     L.pend_off = off; off += 8 * d + 4 * kPendRows + 4 * d + 2 * GH * d + 4 * d;   // fused step: compressed dims of the leaving row, basis column of this part's rows, the leaving row; the query rows
@@ -508,9 +505,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     float2* E = reinterpret_cast<float2*>(smem_raw + L.E_off);            // e^{i theta n}
     float* ut = reinterpret_cast<float*>(smem_raw + L.ut_off);            // [k] (A.re, A.im, B.re, B.im) x N: (1/2) u~
     float* z_s = reinterpret_cast<float*>(smem_raw + L.z_off);            // [k] same packing
-    // [GH heads][d]: the warps' output fragments are summed here as 64-bit fixed-point numbers (scale 2^30):
-    // integer additions commute, so the shared-memory atomics give the same bits in whatever order they land
-    long long* o_s = reinterpret_cast<long long*>(smem_raw + L.o_off);
+    float* o_s = reinterpret_cast<float*>(smem_raw + L.o_off);            // [GH slots][d] what the window tokens give
+    int16_t* inv_v = reinterpret_cast<int16_t*>(smem_raw + L.inv_off);    // [d] position of a dim in D^vu, or -1
     float* red_s = reinterpret_cast<float*>(smem_raw + L.red_off);        // [kAllW][GH] + l_s[GH]
     const int fb_floats = L.fb_floats, pbs = L.pbs;
 
@@ -552,7 +548,15 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         #pragma unroll 1
         for (int a = tid; a < S; a += kAll) rev[a] = (uint16_t)dif_pos<LS>(a);
         if (tid < GH + 8) red_s[kAllW * GH + tid] = 0.f;
-
+        {
+            const int32_t* idf_v = c.idx_full_v + (size_t)h * s.nfv;
+            #pragma unroll 1
+            for (int e = tid; e < s.d; e += kAll) {
+                int lo = 0, hi = s.nfv;                   // the index set is ascending
+                while (lo < hi) { const int mid = (lo + hi) >> 1; if (idf_v[mid] < e) lo = mid + 1; else hi = mid; }
+                inv_v[e] = (int16_t)(lo < s.nfv && idf_v[lo] == e ? lo : -1);
+            }
+        }
     }
     // This part's rows of C^K start towards the transform buffers, and its rows of C^V towards L2, as soon as
     // the kernels before this one are done (the previous step's kernel writes coefficient rows).
@@ -958,7 +962,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         // everything above is independent of the prologue kernel; its output u is first needed here
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
-    for (int i = tid; i < GH * s.d; i += kAll) o_s[i] = 0;
+    for (int i = tid; i < GH * s.d; i += kAll) o_s[i] = 0.f;
     // ut[n] = (A.re, A.im, B.re, B.im), A = heads of the real slots, B = heads of the imaginary slots;
     // all loads of an entry are issued together
     #pragma unroll 1
@@ -983,9 +987,9 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     }
     all_sync();
 
-    float m_run[GH], l_acc[GH];                           // per slot
+    float m_run[GH], l_acc[GH], o_scale[GH];              // per slot; o_scale: how far the class batches have rescaled o_s
 #pragma unroll
-    for (int g = 0; g < GH; ++g) { m_run[g] = kNegBig; l_acc[g] = 0.f; }
+    for (int g = 0; g < GH; ++g) { m_run[g] = kNegBig; l_acc[g] = 0.f; o_scale[g] = 1.f; }
     // per-slot maximum over per-thread partial maxima, broadcast to every consumer thread
     auto block_max = [&](float (&mx)[GH]) {
 #pragma unroll
@@ -1206,16 +1210,24 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 }
             all_sync();
         }
-        // the window fragments open o_s; the class batches rescale it as the running maximum moves
-        if (2 * tq < GH) {
-            long long* o_lo = o_s + hperm<GH>(2 * tq) * s.d;
-            long long* o_hi = o_s + hperm<GH>(2 * tq + 1) * s.d;
+        // the warps' fragments side by side, then summed in warp order (the same bits on every run)
+        float* frag = fbuf;                               // [warp][slot][d]
+        if (2 * tq < GH && is_m) {
+            float* f_lo = frag + (wm * GH + 2 * tq) * s.d;
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) {
                 const int e_lo = 16 * mt + gq, e_hi = e_lo + 8;
-                if (e_lo < s.d) { fix_add(o_lo + e_lo, accw[mt][0]); fix_add(o_hi + e_lo, accw[mt][1]); }
-                if (e_hi < s.d) { fix_add(o_lo + e_hi, accw[mt][2]); fix_add(o_hi + e_hi, accw[mt][3]); }
+                if (e_lo < s.d) { f_lo[e_lo] = accw[mt][0]; f_lo[s.d + e_lo] = accw[mt][1]; }
+                if (e_hi < s.d) { f_lo[e_hi] = accw[mt][2]; f_lo[s.d + e_hi] = accw[mt][3]; }
             }
+        }
+        all_sync();
+        #pragma unroll 1
+        for (int i = tid; i < GH * s.d; i += kAll) {
+            float v = 0.f;
+#pragma unroll
+            for (int w = 0; w < kMW; ++w) v += frag[w * GH * s.d + i];
+            o_s[i] = v;
         }
     }
     all_sync();
@@ -1243,18 +1255,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             }
         }
         const uint32_t p_lane = smem_addr(pbt) + (uint32_t)((gq & (GH - 1)) * pbs + 2 * tq) * 2;
-        // natural positions of this lane's output rows (D^vu), fetched long before they are needed
-        int o_idx[4][2];
-        {
-            const int32_t* idf_v = c.idx_full_v + (size_t)h * s.nfv;
-#pragma unroll
-            for (int mt = 0; mt < 4; ++mt) {
-                const int e_lo = 16 * mt + gq, e_hi = e_lo + 8;
-                o_idx[mt][0] = e_lo < s.nfv ? idf_v[e_lo] : -1;
-                o_idx[mt][1] = e_hi < s.nfv ? idf_v[e_hi] : -1;
-            }
-        }
-
         if constexpr (!SPLIT) {
         if (cp) {
             // a class has one row of probabilities, read by its own slot; the other slot reads the row of zeros behind them
@@ -1377,13 +1377,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 #pragma unroll
                 for (int mt = 0; mt < 4; ++mt) { acc[mt][0] *= al; acc[mt][1] *= ah; acc[mt][2] *= al; acc[mt][3] *= ah; }
             }
-            for (int i = tid; i < GH * s.d; i += kAll) {          // what the windows left in o_s (rows are heads)
-                const int g = i / s.d;
-                float a = alpha[0];
 #pragma unroll
-                for (int sl = 1; sl < GH; ++sl) if (hperm<GH>(sl) == g) a = alpha[sl];
-                o_s[i] = __float2ll_rn(__ll2float_rn(o_s[i]) * a);
-            }
+            for (int g = 0; g < GH; ++g) o_scale[g] *= alpha[g];
             all_sync();
 
             if (cb == c0) TL(10);
@@ -1690,13 +1685,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 }
                 store_vals(pt, v);
             }
-            for (int i = tid; i < GH * s.d; i += kConsumers) {          // what the windows left in o_s (rows are heads)
-                const int g = i / s.d;
-                float a = alpha[0];
 #pragma unroll
-                for (int sl = 1; sl < GH; ++sl) if (hperm<GH>(sl) == g) a = alpha[sl];
-                o_s[i] = __float2ll_rn(__ll2float_rn(o_s[i]) * a);
-            }
+            for (int g = 0; g < GH; ++g) o_scale[g] *= alpha[g];
                     if (tid < GH) alpha_s[tid] = alpha[0];
 #pragma unroll
                     for (int g = 1; g < GH; ++g) if (tid == g) alpha_s[g] = alpha[g];
@@ -1770,14 +1760,14 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             all_sync();
         }
         TL(13);
-        // fold the per-warp output fragments into o_s at the natural positions of D^vu
+        // the warps' fragments of the kept dims side by side (the transform buffers are idle)
         if (2 * tq < GH && is_m) {
-            long long* o_lo = o_s + hperm<GH>(2 * tq) * s.d;
-            long long* o_hi = o_s + hperm<GH>(2 * tq + 1) * s.d;
+            float* f_lo = fbuf + (wm * GH + 2 * tq) * s.nfv;
 #pragma unroll
             for (int mt = 0; mt < 4; ++mt) {
-                if (o_idx[mt][0] >= 0) { fix_add(o_lo + o_idx[mt][0], acc[mt][0]); fix_add(o_hi + o_idx[mt][0], acc[mt][1]); }
-                if (o_idx[mt][1] >= 0) { fix_add(o_lo + o_idx[mt][1], acc[mt][2]); fix_add(o_hi + o_idx[mt][1], acc[mt][3]); }
+                const int e_lo = 16 * mt + gq, e_hi = e_lo + 8;
+                if (e_lo < s.nfv) { f_lo[e_lo] = acc[mt][0]; f_lo[s.nfv + e_lo] = acc[mt][1]; }
+                if (e_hi < s.nfv) { f_lo[e_hi] = acc[mt][2]; f_lo[s.nfv + e_hi] = acc[mt][3]; }
             }
         }
     }
@@ -1789,39 +1779,49 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) red_s[warp * GH + g] = v;
     }
-    all_sync();
-    if (tid < GH) {
-        float v = 0.f;
+    if (SPLIT && tid == 0) {
 #pragma unroll
-        for (int w = 0; w < kAllW; ++w) v += red_s[w * GH + tid];
-        red_s[kAllW * GH + tid] = v;
+        for (int g = 0; g < GH; ++g) red_s[kAllW * GH + GH + g] = o_scale[g];      // the tile group has none of its own
     }
     all_sync();
-
-    if (cp) {
-        // class pairs: slot 1 (the odd classes of the batches) into slot 0, as two partial softmax results of one head
-        const float mm = fmaxf(m_run[0], m_run[1]);
-        const float e0 = ex2(m_run[0] - mm), e1 = ex2(m_run[1] - mm);
-        #pragma unroll 1
-        for (int e = tid; e < s.d; e += kAll)
-            o_s[e] = __float2ll_rn(__ll2float_rn(o_s[e]) * e0 + __ll2float_rn(o_s[s.d + e]) * e1);
-        #pragma unroll 1
-        for (int n = tid; n < s.k; n += kAll) {
-            float* e = z_s + n * 2 * GH;                  // (re, im) of slot 0, then of slot 1
-            e[0] = e0 * e[0] + e1 * e[2];
-            e[1] = e0 * e[1] + e1 * e[3];
-        }
-        all_sync();
-        if (tid == 0) red_s[kAllW * GH] = e0 * red_s[kAllW * GH] + e1 * red_s[kAllW * GH + 1];
-        m_run[0] = mm;
-        all_sync();
+    if (SPLIT) {
+#pragma unroll
+        for (int g = 0; g < GH; ++g) o_scale[g] = red_s[kAllW * GH + GH + g];
     }
-
     TL(14);
     // ------------------------------ partial results ------------------------------
-    for (int i = tid; i < GH * s.d; i += kAll) {
-        const int g = i / s.d, e = i - g * s.d;
-        if (g < ng) ws.o[(((size_t)b * s.Hq + g_first + g) * p.n_part + part) * s.d + e] = __ll2float_rn(o_s[i]) * kFixInv;
+    // class pairs: slot 1 (the odd classes of the batches) goes into slot 0, as two partial softmax results of one head
+    float e0 = 1.f, e1 = 0.f;
+    if (cp) {
+        const float mm = fmaxf(m_run[0], m_run[1]);
+        e0 = ex2(m_run[0] - mm);
+        e1 = ex2(m_run[1] - mm);
+        m_run[0] = mm;
+    }
+    // output of slot sl, dim e: the windows' share, rescaled, and the warps' class fragments in warp order
+    auto o_of = [&](int sl, int e) -> float {
+        float sc = o_scale[0];
+#pragma unroll
+        for (int x = 1; x < GH; ++x) if (sl == x) sc = o_scale[x];
+        float v = o_s[sl * s.d + e] * sc;
+        const int iv = inv_v[e];
+        if (iv >= 0) {
+            const float* f = fbuf + sl * s.nfv + iv;
+            float w = 0.f;
+#pragma unroll
+            for (int x = 0; x < kMW; ++x) w += f[x * GH * s.nfv];
+            v += w;
+        }
+        return v;
+    };
+    #pragma unroll 1
+    for (int i = tid; i < (cp ? 1 : GH) * s.d; i += kAll) {
+        const int sl = i / s.d, e = i - sl * s.d, g = hperm<GH>(sl);      // hperm is its own inverse
+        if (g < ng) {
+            float v = o_of(sl, e);
+            if (cp) v = e0 * v + e1 * o_of(1, e);
+            ws.o[(((size_t)b * s.Hq + g_first + g) * p.n_part + part) * s.d + e] = v;
+        }
     }
     #pragma unroll 1
     for (int n = tid; n < s.k; n += kAll) {
@@ -1831,7 +1831,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             const int g = hperm<GH>(sl), ab = sl / N, ln = sl - ab * N;
             if (g < ng)
                 *reinterpret_cast<float2*>(ws.z + (((size_t)b * s.Hq + g_first + g) * p.n_part + part) * s.M + 2 * n) =
-                    make_float2(e[(2 * ab) * N + ln], e[(2 * ab + 1) * N + ln]);
+                    cp ? make_float2(e0 * e[0] + e1 * e[2], e0 * e[1] + e1 * e[3]) : make_float2(e[(2 * ab) * N + ln], e[(2 * ab + 1) * N + ln]);
         }
     }
     if (tid < GH) {
@@ -1841,8 +1841,14 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             float mv = m_run[0];
 #pragma unroll
             for (int sl = 1; sl < GH; ++sl) if (tid == sl) mv = m_run[sl];
+            auto l_of = [&](int sl) {                     // sum of p of a slot: the warps' sums in a fixed order
+                float v = 0.f;
+#pragma unroll
+                for (int w = 0; w < kAllW; ++w) v += red_s[w * GH + sl];
+                return v;
+            };
             ml[0] = mv;
-            ml[1] = red_s[kAllW * GH + tid];
+            ml[1] = cp ? e0 * l_of(0) + e1 * l_of(1) : l_of(tid);
         }
     }
     TL(15);
