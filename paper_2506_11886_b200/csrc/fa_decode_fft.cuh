@@ -82,7 +82,7 @@ constexpr int kStagesOcc2 = 3;             // with two CTAs per SM (small transf
 // (the split build runs a ring of three as well: its tile group drains the ring steadily, and the two stages it gives
 // up are what lets a batch hold two classes of the longest transforms)
 __host__ __device__ constexpr int ring_stages(int occ, int split = 0) { return (occ == 2 || split) ? kStagesOcc2 : kStages; }
-constexpr int kPendRows = 256;            // rows of a part whose basis values are tabulated for the fused step's update
+constexpr int kPendRows = 520;            // rows of a part at most in a fused step (n_coef <= 4096 over eight parts or more)
 constexpr int kWinRowsPerTile = 64;       // rows of one window tile: two [64 rows x 64 dims] TMA boxes, 128-byte swizzle
 constexpr int kWinHalfBytes = kWinRowsPerTile * 128;
 constexpr uint32_t kSpinLimit = 1u << 24;
@@ -106,11 +106,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t b, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// Bounded wait: gives up after kSpinLimit polls, records the failure, never hangs.  The common case
-// (the phase is already complete) is one inlined test; the polling loop is a call, so that the many
-// wait sites do not bloat the kernel (its code is fetched cold: every phase runs once per CTA).
+// Bounded wait: gives up after kSpinLimit polls, records the failure, never hangs.  The common case (the phase is
+// already complete) is one inlined test; the polling loop is a call, so that the many wait sites do not bloat the
+// kernel (inlined everywhere: +3 % on the long-context token step).
 __device__ __noinline__ bool mbar_wait_slow(uint32_t b, uint32_t parity, volatile int* fail, int32_t* status) {
     if (*fail) return false;
+#pragma unroll 1
     for (uint32_t i = 0; i < kSpinLimit; ++i)
         if (mbar_try_wait(b, parity)) return true;
     *fail = 1;
@@ -124,7 +125,7 @@ __device__ __forceinline__ void mbar_wait(uint64_t* b, uint32_t parity, volatile
 __device__ __forceinline__ bool mbar_wait_u(uint32_t b, uint32_t parity, volatile int* fail, int32_t* status) {
     return mbar_try_wait(b, parity) || mbar_wait_slow(b, parity, fail, status);
 }
-// Eq.4 for one (row, column): a call, for the same reason.
+// Eq.4 for one (row, column).
 __device__ __noinline__ float basis_value(int m, int j, int T) {
     float cs, sn;
     basis_cs(m >> 1, j, T, &cs, &sn);
@@ -483,7 +484,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     // Consumer threads: kAll of them; the warps that consume ring tiles (kept-dim and window products) are all of them,
     // or, in the split kernel, the last six, while the first eight (the transform group) run the compressed-dim phases
     // of the class batches beside them.
-    constexpr int kAll = SPLIT ? kSplitConsumers : kConsumers, kAllW = kAll / 32, kAllT = kAll + 32;
+    constexpr int kAll = SPLIT ? kSplitConsumers : kConsumers, kAllW = kAll / 32;
     constexpr int kMW = SPLIT ? kAllW - kWarps : kWarps, kM0 = SPLIT ? kWarps : 0;
     auto all_sync = [] { consumer_sync<kAll, 1>(); };
     extern __shared__ __align__(128) unsigned char smem_unaligned[];
@@ -548,15 +549,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         #pragma unroll 1
         for (int a = tid; a < S; a += kAll) rev[a] = (uint16_t)dif_pos<LS>(a);
         if (tid < GH + 8) red_s[kAllW * GH + tid] = 0.f;
-        {
-            const int32_t* idf_v = c.idx_full_v + (size_t)h * s.nfv;
-            #pragma unroll 1
-            for (int e = tid; e < s.d; e += kAll) {
-                int lo = 0, hi = s.nfv;                   // the index set is ascending
-                while (lo < hi) { const int mid = (lo + hi) >> 1; if (idf_v[mid] < e) lo = mid + 1; else hi = mid; }
-                inv_v[e] = (int16_t)(lo < s.nfv && idf_v[lo] == e ? lo : -1);
-            }
-        }
+        for (int e = tid; e < s.d; e += kAll) inv_v[e] = -1;
     }
     // This part's rows of C^K start towards the transform buffers, and its rows of C^V towards L2, as soon as
     // the kernels before this one are done (the previous step's kernel writes coefficient rows).
@@ -674,10 +667,11 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         *fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // stale shared memory must hold finite numbers: rows past the end of a tile are multiplied by p = 0
-    #pragma unroll 1
-    for (int i = tid; i < (NS * kStageBytes) / 16; i += kAllT) reinterpret_cast<uint4*>(stages)[i] = make_uint4(0, 0, 0, 0);
     if (tid < 4) reinterpret_cast<uint32_t*>(zero16)[tid] = 0;
+    // stale shared memory must hold finite numbers: rows past the end of a tile are multiplied by p = 0 (clearing only
+    // those rows, in the tile loops, measured 1-3 % slower)
+    #pragma unroll 1
+    for (int i = tid; i < (NS * kStageBytes) / 16; i += kAll + 32) reinterpret_cast<uint4*>(stages)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     TL(1);
@@ -704,44 +698,41 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 dst += kStageBytes;
                 if (++st == (uint32_t)NS) { st = 0; phase ^= 1; bar_u = full_u; dst = stages_base; }
             };
-            const size_t cls_k = (size_t)s.S_cap * rowb_k, cls_v = (size_t)s.S_cap * rowb_v;      // bytes from one class to the next
-            const char* base_k = rowb_k ? reinterpret_cast<const char*>(mid_row<bf16>(c.k_mid, s, b, h, c0, 0, s.nfk)) : nullptr;
-            const char* base_v = rowb_v ? reinterpret_cast<const char*>(mid_row<bf16>(c.v_mid, s, b, h, c0, 0, s.nfv)) : nullptr;
-            const uint32_t tile_k = (uint32_t)(ts_k * rowb_k), tile_v = (uint32_t)(ts_v * rowb_v);
-            auto class_tiles = [&](int cb, int nb, int side) -> bool {
-                const uint32_t tile = side == 0 ? tile_k : tile_v;
-                if (tile == 0) return true;
-                const uint32_t rowb = (uint32_t)(side == 0 ? rowb_k : rowb_v);
-                const size_t cstride = side == 0 ? cls_k : cls_v;
-                const char* src_c = (side == 0 ? base_k : base_v) + (size_t)(cb - c0) * cstride;
+            // K tiles of batch 0, windows, then V tiles of batch 0, K and V tiles of batch 1, ...: turn 2 i is the K side of
+            // batch i, turn 2 i + 1 its V side
 #pragma unroll 1
-                for (int cls = cb; cls < cb + nb; ++cls, src_c += cstride) {
+            for (int turn = 0;; ++turn) {
+                const int side = turn & 1, cb = c0 + (turn >> 1) * NB, cend = min(cb + NB, c1);
+                if (cb >= c1 && turn > 0) break;
+                const uint32_t rowb = (uint32_t)(side == 0 ? rowb_k : rowb_v), tile = rowb * (uint32_t)(side == 0 ? ts_k : ts_v);
+                const size_t cstride = (size_t)s.S_cap * rowb;                                     // bytes from one class to the next
+                const char* src_c = rowb ? reinterpret_cast<const char*>(side == 0 ? mid_row<bf16>(c.k_mid, s, b, h, cb, 0, s.nfk)
+                                                                                   : mid_row<bf16>(c.v_mid, s, b, h, cb, 0, s.nfv)) : nullptr;
+#pragma unroll 1
+                for (int cls = cb; cls < cend; ++cls, src_c += cstride) {
                     const char* src = src_c;
 #pragma unroll 1
                     for (int left = n_of_class(cls) * (int)rowb; left > 0; left -= (int)tile, src += tile) {
                         const uint32_t bytes = min((uint32_t)left, tile);
-                        if (!acquire(bytes)) return false;
+                        if (!acquire(bytes)) return;
                         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                                      "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(bar_u)
                                      : "memory");
                         advance();
                     }
                 }
-                return true;
-            };
-            if (c0 < c1 && !class_tiles(c0, min(NB, c1 - c0), 0)) return;
-            // window rows: tiles of 64 rows, one TMA box per 64 dims
+                if (turn > 0) continue;
+                // window rows: tiles of 64 rows, one TMA box per 64 dims
 #pragma unroll 1
-            for (int t0 = w0; t0 < w1; t0 += wchunk) {
-                const WinSegs sg = win_segments(t0, min(w1, t0 + wchunk), n_init, n_local, head, s.l_local);
+                for (int t0 = w0; t0 < w1; t0 += wchunk) {
+                    const WinSegs sg = win_segments(t0, min(w1, t0 + wchunk), n_init, n_local, head, s.l_local);
 #pragma unroll 1
-                for (int side = 0; side < 2; ++side)
+                    for (int i = 0; i < 2 * sg.n; ++i) {
+                        const int sd = i >= sg.n, si = sd ? i - sg.n : i;
+                        const CUtensorMap* tm = sg.buf[si] == 0 ? (sd == 0 ? &tm_ki : &tm_vi) : (sd == 0 ? &tm_kl : &tm_vl);
+                        const int row1 = sg.row[si] + sg.cnt[si];
 #pragma unroll 1
-                    for (int i = 0; i < sg.n; ++i) {
-                        const CUtensorMap* tm = sg.buf[i] == 0 ? (side == 0 ? &tm_ki : &tm_vi) : (side == 0 ? &tm_kl : &tm_vl);
-                        const int row1 = sg.row[i] + sg.cnt[i];
-#pragma unroll 1
-                        for (int r0 = sg.row[i]; r0 < row1; r0 += ts_w) {
+                        for (int r0 = sg.row[si]; r0 < row1; r0 += ts_w) {
                             if (!acquire((uint32_t)(nhalf * kWinHalfBytes))) return;
 #pragma unroll 1
                             for (int hf = 0; hf < nhalf; ++hf)
@@ -752,12 +743,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                             advance();
                         }
                     }
-            }
-#pragma unroll 1
-            for (int cb = c0; cb < c1; cb += NB) {
-                const int nb = min(NB, c1 - cb);
-                if (cb != c0 && !class_tiles(cb, nb, 0)) return;
-                if (!class_tiles(cb, nb, 1)) return;
+                }
             }
         }
         return;
@@ -770,6 +756,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     const int gq = lane >> 2, tq = lane & 3;              // mma fragment coordinates
     const int npk = s.nfk >> 3, nchv = s.nfv >> 3, npw = s.d >> 3;
     const float sl2 = s.scale * kLog2e;
+
+    for (int e = tid; e < s.nfv; e += kAll) inv_v[c.idx_full_v[(size_t)h * s.nfv + e]] = (int16_t)e;
 
     int32_t* bar = ws.bar + 4 * (((size_t)b * s.Hkv + h) * p.n_pass + pass);
     // gathered query of the compressed K dims (one element per thread and round), loaded early
@@ -787,13 +775,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             xp_s[i] = i < s.dck ? __bfloat162float(xrow_s[c.idx_comp_k[(size_t)h * s.dck + i]])
                                 : __bfloat162float(xrow_s[s.d + c.idx_comp_v[(size_t)h * s.dcv + i - s.dck]]);
 #pragma unroll 1
-        for (int r = tid; r < min(m1 - m0, kPendRows); r += kAll) f_s[r] = basis_value(m0 + r, j_pend, s.T);
+        for (int r = tid; r < m1 - m0; r += kAll) f_s[r] = basis_value(m0 + r, j_pend, s.T);
     }
-    // basis value of row r of this part (tabulated for the first kPendRows rows)
-    auto f_row = [&](int r) -> float {
-        return r < kPendRows ? f_s[r] : basis_value(m0 + r, j_pend, s.T);
-    };
-
     // B fragments of q for the kept K dims: column gq is slot gq = head hperm(gq);
     // round rd covers pieces 4 rd + tq of a row, two k-steps each
     const int my_head = hperm<GH>(gq & (GH - 1));
@@ -920,7 +903,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                         const float4* row = reinterpret_cast<const float4*>(fbuf + (r - q0) * s.dck);
                         // fused step: the rank-1 update of Eq.5 that the light append kernel left pending, applied to
                         // each piece of this part's rows as it passes here (exactly once), and written back
-                        const float f = j_pend >= 0 ? f_row(r - m0) : 0.f;
+                        const float f = j_pend >= 0 ? f_s[r - m0] : 0.f;
 #pragma unroll 1
                         for (int v = l8; v < nv; v += 8) {
                             float4 x = row[v];
@@ -1974,7 +1957,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     if (j_pend >= 0) {
                         // fused step: the pending rank-1 update of this piece of a C^V row (every piece passes here
                         // exactly once), used below and written back
-                        const float f = f_row(r0 + r);
+                        const float f = f_s[r0 + r];
                         const float4 y = *reinterpret_cast<const float4*>(xp_s + s.dck + 4 * v);
                         x.x = fmaf(f, y.x, x.x); x.y = fmaf(f, y.y, x.y); x.z = fmaf(f, y.z, x.z); x.w = fmaf(f, y.w, x.w);
                         *reinterpret_cast<float4*>(cvg + (size_t)(r0 + r) * s.dcv + 4 * v) = x;
