@@ -355,20 +355,28 @@ __device__ __forceinline__ void fft_pass(float* fbuf, int fb_floats, int nb, con
     }
 }
 
-// All passes of the transform, ending each with a barrier of the consumer warps.
+// The passes of the transform except the one over the shortest sub-transforms (the last of the score transform, the first
+// of the probability transform), which is done together with the softmax below; each ends with a barrier.
 // (kConsumers threads take part: all consumer warps, or the transform group of the split kernel with its barrier BID)
 template <int GH, int LS, int LL, bool DIT, int BID = 1>
 __device__ __forceinline__ void fft_run(float* fbuf, int fb_floats, int nb, const float* twf, int tid) {
     constexpr int RL = radix_log2(LL);
-    if constexpr (!DIT) {
-        fft_pass<GH, LS, LL, false>(fbuf, fb_floats, nb, twf, tid);
-        consumer_sync<kConsumers, BID>();
-        if constexpr (LL - RL > 0) fft_run<GH, LS, LL - RL, false, BID>(fbuf, fb_floats, nb, twf, tid);
-    } else {
-        if constexpr (LL - RL > 0) fft_run<GH, LS, LL - RL, true, BID>(fbuf, fb_floats, nb, twf, tid);
-        fft_pass<GH, LS, LL, true>(fbuf, fb_floats, nb, twf, tid);
-        consumer_sync<kConsumers, BID>();
+    if constexpr (LL - RL > 0) {
+        if constexpr (!DIT) {
+            fft_pass<GH, LS, LL, false>(fbuf, fb_floats, nb, twf, tid);
+            consumer_sync<kConsumers, BID>();
+            fft_run<GH, LS, LL - RL, false, BID>(fbuf, fb_floats, nb, twf, tid);
+        } else {
+            fft_run<GH, LS, LL - RL, true, BID>(fbuf, fb_floats, nb, twf, tid);
+            fft_pass<GH, LS, LL, true>(fbuf, fb_floats, nb, twf, tid);
+            consumer_sync<kConsumers, BID>();
+        }
     }
+}
+__host__ __device__ constexpr int last_radix_log2(int LS) {
+    int cur = LS, rl = 0;
+    while (cur > 0) { rl = radix_log2(cur); cur -= rl; }
+    return rl;
 }
 
 // Position of output index a after the decimation-in-frequency passes.
@@ -383,6 +391,82 @@ __host__ __device__ constexpr int dif_pos(int a) {
     }
     return pos;
 }
+
+// Softmax of a batch between the two transforms, in registers.  The last pass of the score transform and the first of the
+// probability transform both work on R neighbouring points without twiddles, and the R outputs of the one are the
+// inputs of the other: a thread finishes the scores of its R tokens per transform (token j + r S / R sits at point
+// dif_pos(j) + r), adds the kept-dim scores, takes part in the maximum, and after it turns them into
+// probabilities, keeps their bf16 copies for the V products and runs the first butterfly of the way back.  (As passes of
+// their own through shared memory the three took 9.8 of the 62 K cycles of a 32 K-token step.)
+template <int GH, int LS>
+struct BatchSoftmax {
+    static constexpr int N = GH / 2, RL = last_radix_log2(LS), R = 1 << RL, JL = LS - RL, kRounds = 8 / R;   // a batch has at most 8 kConsumers points
+    PC<N> v[kRounds][R];
+
+    // scores and the thread's maxima per slot; n0 / n1(ci): tokens of slot 0's / slot 1's class of transform ci
+    template <class F0, class F1>
+    __device__ __forceinline__ void scores(float* fbuf, int fb_floats, int nbt, const float* kb, bool have_k, bool have_c, int tid, F0 n0, F1 n1,
+                                           float (&mx)[GH]) {
+#pragma unroll
+        for (int rd = 0; rd < kRounds; ++rd) {
+            const int item = tid + rd * kConsumers, ci = item >> JL, j = item & ((1 << JL) - 1);
+            if (ci < nbt) {
+                const float* base = fbuf + ci * fb_floats;
+                const int p0 = dif_pos<LS>(j) * GH;
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[rd][r] = have_c ? ld_pt<N>(base + pf(p0 + r * GH)) : PC<N>{splat<N>(0.f), splat<N>(0.f)};
+                dft<R, N>(v[rd]);
+                const int na = n0(ci), nb1 = n1(ci);
+                const float* kp = kb + ((ci << LS) + j) * GH;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (have_k) v[rd][r] = v[rd][r] + ld_pt<N>(kp + (r << JL) * GH);
+                    float x[GH];
+                    vals(v[rd][r], x);
+                    const int a = j + (r << JL);
+#pragma unroll
+                    for (int g = 0; g < GH; ++g) if (a < (g == 1 ? nb1 : na)) mx[g] = fmaxf(mx[g], x[g]);
+                }
+            }
+        }
+    }
+    // probabilities from the scores; put(ci, slot, token, p) keeps the copies for the V products
+    template <class F0, class F1, class P>
+    __device__ __forceinline__ void probs(float* fbuf, int fb_floats, int nbt, bool have_c, int tid, F0 n0, F1 n1, const float (&m)[GH], float (&l)[GH], P put) {
+#pragma unroll
+        for (int rd = 0; rd < kRounds; ++rd) {
+            const int item = tid + rd * kConsumers, ci = item >> JL, j = item & ((1 << JL) - 1);
+            if (ci < nbt) {
+                const int na = n0(ci), nb1 = n1(ci);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    float x[GH];
+                    vals(v[rd][r], x);
+                    const int a = j + (r << JL);
+#pragma unroll
+                    for (int g = 0; g < GH; ++g) {
+                        x[g] = a < (g == 1 ? nb1 : na) ? ex2(x[g] - m[g]) : 0.f;
+                        l[g] += x[g];
+                        put(ci, g, a, x[g]);
+                    }
+                    if constexpr (N == 2) v[rd][r] = PC<N>{pk(x[0], x[1]), pk(x[2], x[3])};
+                    else v[rd][r] = PC<N>{PR<1>{x[0]}, PR<1>{x[1]}};
+                }
+                if (have_c) {
+                    dft<R, N>(v[rd]);
+                    float* base = fbuf + ci * fb_floats;
+                    const int p0 = dif_pos<LS>(j) * GH;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) st_pt(base + pf(p0 + r * GH), v[rd][r]);
+                }
+            }
+        }
+    }
+    __device__ __forceinline__ static void vals(const PC<N>& p, float (&x)[GH]) {
+        if constexpr (N == 2) { unpk(p.re, x[0], x[1]); unpk(p.im, x[2], x[3]); }
+        else { x[0] = p.re.v; x[1] = p.im.v; }
+    }
+};
 
 // Physical row ranges of the logical window tokens [t0, t1): init rows, then up to two ring pieces.
 struct WinSegs {
@@ -410,7 +494,7 @@ __device__ __forceinline__ WinSegs win_segments(int t0, int t1, int n_init, int 
 }
 
 struct FftSmem {
-    int stages_off, fbuf_off, kb_off, pbt_off, twf_off, rev_off, E_off, ut_off, z_off, o_off, inv_off, red_off, pend_off, zero_off, total;
+    int stages_off, fbuf_off, kb_off, pbt_off, twf_off, E_off, ut_off, z_off, o_off, inv_off, red_off, pend_off, zero_off, total;
     int fb_floats, pbs;
 };
 // True if the kernel packs two residue classes of ONE query head into a complex transform (one query head per KV head:
@@ -434,7 +518,6 @@ __host__ __device__ inline FftSmem fft_smem_layout(int log2S, int k, int GH, int
     L.pbt_off = off; off += cp ? 2 * (NB + 1) * L.pbs : 2 * NB * GH * L.pbs;   // class pairs: one row per class and one of zeros
     off = (off + 15) / 16 * 16;
     L.twf_off = off; off += 8 * (tw_total(log2S) + 1);
-    L.rev_off = off; off += 2 * S;
     off = (off + 15) / 16 * 16;
     L.E_off = off; off += (8 * k + 15) / 16 * 16;
     L.ut_off = off; off += (8 * k * GH + 15) / 16 * 16;
@@ -502,7 +585,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     float* kb = reinterpret_cast<float*>(smem_raw + L.kb_off);            // [NB][S][GH]
     bf16* pbt = reinterpret_cast<bf16*>(smem_raw + L.pbt_off);           // [NB][GH slots][pbs]
     float* twf = reinterpret_cast<float*>(smem_raw + L.twf_off);          // pass twiddles (float2 each)
-    uint16_t* rev = reinterpret_cast<uint16_t*>(smem_raw + L.rev_off);    // slot -> point after the DIF passes
     float2* E = reinterpret_cast<float2*>(smem_raw + L.E_off);            // e^{i theta n}
     float* ut = reinterpret_cast<float*>(smem_raw + L.ut_off);            // [k] (A.re, A.im, B.re, B.im) x N: (1/2) u~
     float* z_s = reinterpret_cast<float*>(smem_raw + L.z_off);            // [k] same packing
@@ -546,8 +628,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             }
             l -= rl;
         }
-        #pragma unroll 1
-        for (int a = tid; a < S; a += kAll) rev[a] = (uint16_t)dif_pos<LS>(a);
         if (tid < GH + 8) red_s[kAllW * GH + tid] = 0.f;
         for (int e = tid; e < s.d; e += kAll) inv_v[e] = -1;
     }
@@ -1295,41 +1375,20 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 }
                 all_sync();
                 if (cb == c0) TL(8);
-                fft_run<GH, LS, LS, false>(fbuf, fb_floats, nbt, twf, tid);       // score of slot a at point rev[a]
+                fft_run<GH, LS, LS, false>(fbuf, fb_floats, nbt, twf, tid);
                 if (cb == c0) TL(9);
             } else {
-                #pragma unroll 1
-                for (int i = tid; i < nbt * fb_floats; i += kAll) fbuf[i] = 0.f;
-                all_sync();
+                all_sync();                               // the kept-dim scores
             }
 
-            all_sync();
-
-            // online softmax over the batch
+            // online softmax over the batch; class pairs: slot g of a point is the token of class cstep ci + g
+            BatchSoftmax<GH, LS> sm;
+            auto n0 = [&](int ci) { return n_of_class(cb + cstep * ci); };
+            auto n1 = [&](int ci) { return cp ? (2 * ci + 1 < nb ? n_of_class(cb + 2 * ci + 1) : 0) : n_of_class(cb + ci); };
             float mx[GH], alpha[GH];
 #pragma unroll
             for (int g = 0; g < GH; ++g) mx[g] = kNegBig;
-            #pragma unroll 1
-            for (int i = tid; i < (nbt << LS); i += kAll) {
-                const int ci = i >> LS, a = i & (S - 1);
-                // class pairs: slot g of the point is token a of class cstep ci + g
-                const bool ok0 = a < n_of_class(cb + cstep * ci);
-                const bool ok1 = cp ? (2 * ci + 1 < nb && a < n_of_class(cb + 2 * ci + 1)) : ok0;
-                if (ok0 || ok1) {
-                    // score = compressed part (transform output) + kept part
-                    float* pt = fbuf + ci * fb_floats + pf(rev[a] * GH);
-                    float v[GH], kv[GH];
-                    load_vals(pt, v);
-                    if (ts_k) {
-                        load_vals(kb + (size_t)i * GH, kv);
-#pragma unroll
-                        for (int g = 0; g < GH; ++g) v[g] += kv[g];
-                        store_vals(pt, v);
-                    }
-#pragma unroll
-                    for (int g = 0; g < GH; ++g) if (g == 1 ? ok1 : ok0) mx[g] = fmaxf(mx[g], v[g]);
-                }
-            }
+            sm.scores(fbuf, fb_floats, nbt, kb, ts_k != 0, s.dck > 0, tid, n0, n1, mx);
             block_max(mx);
 #pragma unroll
             for (int g = 0; g < GH; ++g) {
@@ -1337,31 +1396,17 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 alpha[g] = ex2(m_run[g] - m_new);
                 m_run[g] = m_new;
                 l_acc[g] *= alpha[g];
+                o_scale[g] *= alpha[g];
             }
-            #pragma unroll 1
-            for (int i = tid; i < (nbt << LS); i += kAll) {
-                const int ci = i >> LS, a = i & (S - 1);
-                float* pt = fbuf + ci * fb_floats + pf(rev[a] * GH);
-                float v[GH];
-                load_vals(pt, v);
-                const bool ok0 = a < n_of_class(cb + cstep * ci);
-                const bool ok1 = cp ? (2 * ci + 1 < nb && a < n_of_class(cb + 2 * ci + 1)) : ok0;
-#pragma unroll
-                for (int g = 0; g < GH; ++g) {
-                    v[g] = (g == 1 ? ok1 : ok0) ? ex2(v[g] - m_run[g]) : 0.f;
-                    l_acc[g] += v[g];
-                    if (!cp) pbt[(ci * GH + g) * pbs + a] = __float2bfloat16_rn(v[g]);
-                    else if (2 * ci + g < nb) pbt[(2 * ci + g) * pbs + a] = __float2bfloat16_rn(v[g]);
-                }
-                store_vals(pt, v);
-            }
+            sm.probs(fbuf, fb_floats, nbt, s.dcv > 0, tid, n0, n1, m_run, l_acc, [&](int ci, int g, int a, float x) {
+                if (!cp) pbt[(ci * GH + g) * pbs + a] = __float2bfloat16_rn(x);
+                else if (2 * ci + g < nb) pbt[(2 * ci + g) * pbs + a] = __float2bfloat16_rn(x);
+            });
             {
                 const float al = alpha[(2 * tq) & (GH - 1)], ah = alpha[(2 * tq + 1) & (GH - 1)];
 #pragma unroll
                 for (int mt = 0; mt < 4; ++mt) { acc[mt][0] *= al; acc[mt][1] *= ah; acc[mt][2] *= al; acc[mt][3] *= ah; }
             }
-#pragma unroll
-            for (int g = 0; g < GH; ++g) o_scale[g] *= alpha[g];
             all_sync();
 
             if (cb == c0) TL(10);
@@ -1606,41 +1651,20 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     }
                 }
                 xf_sync();
-                fft_run<GH, LS, LS, false, 2>(fbuf, fb_floats, nb, twf, tid);        // score of slot a at point rev[a]
-            } else {
-                #pragma unroll 1
-                for (int i = tid; i < nb * fb_floats; i += kConsumers) fbuf[i] = 0.f;
-                xf_sync();
+                fft_run<GH, LS, LS, false, 2>(fbuf, fb_floats, nb, twf, tid);
             }
-
-                    xf_sync();
                     // the kept-dim scores of this batch (batch 0: formed by everybody's earlier barriers)
                     if (bi >= 1) {
                         if (tid == 0) mbar_wait(kb_full, (bi - 1) & 1, fail, c.status);   // one thread polls
                         xf_sync();
                     }
             // online softmax over the batch
+            BatchSoftmax<GH, LS> sm;
+            auto n0 = [&](int ci) { return n_of_class(cb + ci); };
             float mx[GH], alpha[GH];
 #pragma unroll
             for (int g = 0; g < GH; ++g) mx[g] = kNegBig;
-            #pragma unroll 1
-            for (int i = tid; i < (nb << LS); i += kConsumers) {
-                const int ci = i >> LS, a = i & (S - 1);
-                if (a < n_of_class(cb + ci)) {
-                    // score = compressed part (transform output) + kept part
-                    float* pt = fbuf + ci * fb_floats + pf(rev[a] * GH);
-                    float v[GH], kv[GH];
-                    load_vals(pt, v);
-                    if (ts_k) {
-                        load_vals(kbuf + (size_t)i * GH, kv);
-#pragma unroll
-                        for (int g = 0; g < GH; ++g) v[g] += kv[g];
-                        store_vals(pt, v);
-                    }
-#pragma unroll
-                    for (int g = 0; g < GH; ++g) mx[g] = fmaxf(mx[g], v[g]);
-                }
-            }
+            sm.scores(fbuf, fb_floats, nb, kbuf, ts_k != 0, s.dck > 0, tid, n0, n0, mx);
             block_max_t(mx);
 #pragma unroll
             for (int g = 0; g < GH; ++g) {
@@ -1648,28 +1672,14 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 alpha[g] = ex2(m_run[g] - m_new);
                 m_run[g] = m_new;
                 l_acc[g] *= alpha[g];
+                o_scale[g] *= alpha[g];
             }
             if (bi >= 1) {                                // the tile group is done with the previous batch's probabilities
                 if (tid == 0) mbar_wait(p_free, (bi - 1) & 1, fail, c.status);
                 xf_sync();
             }
-            #pragma unroll 1
-            for (int i = tid; i < (nb << LS); i += kConsumers) {
-                const int ci = i >> LS, a = i & (S - 1);
-                float* pt = fbuf + ci * fb_floats + pf(rev[a] * GH);
-                float v[GH];
-                load_vals(pt, v);
-                const bool ok = a < n_of_class(cb + ci);
-#pragma unroll
-                for (int g = 0; g < GH; ++g) {
-                    v[g] = ok ? ex2(v[g] - m_run[g]) : 0.f;
-                    l_acc[g] += v[g];
-                    pbuf[(ci * GH + g) * pbs + a] = __float2bfloat16_rn(v[g]);
-                }
-                store_vals(pt, v);
-            }
-#pragma unroll
-            for (int g = 0; g < GH; ++g) o_scale[g] *= alpha[g];
+            sm.probs(fbuf, fb_floats, nb, s.dcv > 0, tid, n0, n0, m_run, l_acc,
+                     [&](int ci, int g, int a, float x) { pbuf[(ci * GH + g) * pbs + a] = __float2bfloat16_rn(x); });
                     if (tid < GH) alpha_s[tid] = alpha[0];
 #pragma unroll
                     for (int g = 1; g < GH; ++g) if (tid == g) alpha_s[g] = alpha[g];
