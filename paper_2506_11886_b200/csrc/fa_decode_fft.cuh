@@ -203,6 +203,9 @@ __device__ __forceinline__ float2 cis_frac(float frac) {
     const float a = 6.283185307179586f * (frac - (frac >= 0.5f ? 1.0f : 0.0f));
     return make_float2(__cosf(a), __sinf(a));
 }
+// a / n for 0 <= a < 2^21, n > 0: six instructions instead of some twenty (the division's relative error of 2^-22 stays
+// below half a unit of the quotient's last multiple of 1 / n).
+__device__ __forceinline__ int idiv(int a, int n) { return __float2int_rz(__fdividef((float)a + 0.5f, (float)n)); }
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -296,7 +299,8 @@ __device__ __forceinline__ void dft(PC<N> (&v)[R]) {
 // Shared-memory float index of float f of a transform buffer: 16 bytes of padding after every
 // 128 bytes, every 1 KB and every 8 KB.  Points stay 16-byte aligned; the strided point accesses
 // of the passes and the digit-reversed accesses of token-ordered code (consecutive slots sit 64, 8
-// or 1 points apart after a radix-8 decimation) all spread over the banks.
+// or 1 points apart after a radix-8 decimation) all spread over the banks.  Indices without a bit in common add:
+// pf(a + b) = pf(a) + pf(b), which makes the points of a butterfly constants apart.
 __host__ __device__ constexpr int pf(int f) { return f + ((f >> 5) << 2) + ((f >> 8) << 2) + ((f >> 11) << 2); }
 __host__ __device__ constexpr int pf_size(int floats) { return pf(floats) + 8; }
 
@@ -328,10 +332,10 @@ __device__ __forceinline__ void fft_pass(float* fbuf, int fb_floats, int nb, con
         const int ci = item >> PERL, rest = item & ((1 << PERL) - 1);
         const int blk = rest >> STL, j = rest & ((1 << STL) - 1);
         float* base = fbuf + ci * fb_floats;
-        const int e0 = (blk << LL) + j;
+        base += pf(((blk << LL) + j) * GH);               // the points' offsets have no bit in common with it: constants from here
         PC<N> v[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = ld_pt<N>(base + pf((e0 + (r << STL)) * GH));
+        for (int r = 0; r < R; ++r) v[r] = ld_pt<N>(base + pf((r << STL) * GH));
         PR<N> wr[R], wi[R];
         if constexpr (kTw) {
 #pragma unroll
@@ -351,7 +355,7 @@ __device__ __forceinline__ void fft_pass(float* fbuf, int fb_floats, int nb, con
             for (int q = 1; q < R; ++q) v[q] = cmulw(v[q], wr[q], wi[q]);
         }
 #pragma unroll
-        for (int r = 0; r < R; ++r) st_pt(base + pf((e0 + (r << STL)) * GH), v[r]);
+        for (int r = 0; r < R; ++r) st_pt(base + pf((r << STL) * GH), v[r]);
     }
 }
 
@@ -411,10 +415,9 @@ struct BatchSoftmax {
         for (int rd = 0; rd < kRounds; ++rd) {
             const int item = tid + rd * kConsumers, ci = item >> JL, j = item & ((1 << JL) - 1);
             if (ci < nbt) {
-                const float* base = fbuf + ci * fb_floats;
-                const int p0 = dif_pos<LS>(j) * GH;
+                const float* base = fbuf + ci * fb_floats + pf(dif_pos<LS>(j) * GH);
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[rd][r] = have_c ? ld_pt<N>(base + pf(p0 + r * GH)) : PC<N>{splat<N>(0.f), splat<N>(0.f)};
+                for (int r = 0; r < R; ++r) v[rd][r] = have_c ? ld_pt<N>(base + pf(r * GH)) : PC<N>{splat<N>(0.f), splat<N>(0.f)};
                 dft<R, N>(v[rd]);
                 const int na = n0(ci), nb1 = n1(ci);
                 const float* kp = kb + ((ci << LS) + j) * GH;
@@ -454,10 +457,9 @@ struct BatchSoftmax {
                 }
                 if (have_c) {
                     dft<R, N>(v[rd]);
-                    float* base = fbuf + ci * fb_floats;
-                    const int p0 = dif_pos<LS>(j) * GH;
+                    float* base = fbuf + ci * fb_floats + pf(dif_pos<LS>(j) * GH);
 #pragma unroll
-                    for (int r = 0; r < R; ++r) st_pt(base + pf(p0 + r * GH), v[rd][r]);
+                    for (int r = 0; r < R; ++r) st_pt(base + pf(r * GH), v[rd][r]);
                 }
             }
         }
@@ -483,7 +485,8 @@ __device__ __forceinline__ WinSegs win_segments(int t0, int t1, int n_init, int 
     if (a1 > a0) { w.buf[w.n] = 0; w.row[w.n] = a0; w.cnt[w.n] = a1 - a0; w.tok[w.n] = 0; ++w.n; }
     int u0 = max(t0 - n_init, 0), u1 = min(t1 - n_init, n_local);
     if (u1 > u0) {
-        int ps = (head + u0) % l_local;
+        int ps = head + u0;
+        if (ps >= l_local) ps -= l_local;
         int len1 = min(u1 - u0, l_local - ps);
         w.buf[w.n] = 1; w.row[w.n] = ps; w.cnt[w.n] = len1; w.tok[w.n] = n_init + u0 - t0; ++w.n;
         if (u1 - u0 > len1) {
@@ -595,7 +598,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 
     const int part = blockIdx.x;                          // partial-result index: class CTAs, then window CTAs
     const bool is_win = part >= p.n_split;
-    const int h = blockIdx.y / p.n_pass, pass = blockIdx.y % p.n_pass;
+    const int h = idiv(blockIdx.y, p.n_pass), pass = blockIdx.y - h * p.n_pass;
     const int b = blockIdx.z;
     const int g_first = h * s.G + pass * GH;
     const int ng = min(GH, s.G - pass * GH);
@@ -608,13 +611,17 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     const int tid = threadIdx.x;
     const int log2P = 31 - __clz(s.P);
 
+    const float inv_T = __int_as_float((127 << 23) - ((31 - __clz(s.T)) << 23));      // 1 / T, a power of two
+    const float w_paper = __fdiv_rn(1.0f, (float)s.k);
+    // reconstruction weight of row m (recon_weight of fa_common.cuh without its divisions)
+    auto w_row = [&](int m) { return s.norm == FA_NORM_PAPER ? w_paper : m == 0 ? inv_T : m == 1 ? 0.f : 2.f * inv_T; };
     TL(0);
     SPAN(0);
     // ---- one-time set-up, independent of the cache: it may overlap the tail of the previous kernel ----
     if (tid < kAll) {
         #pragma unroll 1
         for (int i = tid; i < s.k; i += kAll) {
-            E[i] = cis_frac((float)i / (float)s.T);
+            E[i] = cis_frac((float)i * inv_T);
         }
         for (int l = LS; l > 0;) {
             const int rl = radix_log2(l), R = 1 << rl, st = 1 << (l - rl);
@@ -622,8 +629,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 const int off = tw_offset(LS, l);
                 #pragma unroll 1
                 for (int i = tid; i < (R - 1) * st; i += kAll) {
-                    const int qm1 = i / st, j = i - qm1 * st;
-                    reinterpret_cast<float2*>(twf)[off + i] = cis_frac((float)(((qm1 + 1) * j) & ((1 << l) - 1)) / (float)(1 << l));
+                    const int qm1 = i >> (l - rl), j = i & (st - 1);
+                    reinterpret_cast<float2*>(twf)[off + i] = cis_frac((float)(((qm1 + 1) * j) & ((1 << l) - 1)) * (1.0f / (float)(1 << l)));
                 }
             }
             l -= rl;
@@ -633,10 +640,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     }
     // This part's rows of C^K start towards the transform buffers, and its rows of C^V towards L2, as soon as
     // the kernels before this one are done (the previous step's kernel writes coefficient rows).
-    const int m0 = part * (s.M >> 2) / p.n_part * 4, m1 = (part + 1) * (s.M >> 2) / p.n_part * 4;
+    const int m0 = 4 * idiv(part * (s.M >> 2), p.n_part), m1 = 4 * idiv((part + 1) * (s.M >> 2), p.n_part);
     // rows of C^K staged at a time: the transform buffers and, behind them, the kept-dim score and probability
     // buffers (one contiguous area, all idle until the first batch)
-    const int uch = s.dck > 0 ? (((L.twf_off - L.fbuf_off) >> 2) / s.dck) & ~3 : 0;
+    const int uch = s.dck > 0 ? idiv((L.twf_off - L.fbuf_off) >> 2, s.dck) & ~3 : 0;
     auto start_coef_rows = [&]() {
         if (tid >= kAll) return;
         if (s.dck > 0) {
@@ -661,12 +668,12 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     auto stage_inputs = [&]() {
         const int per_row = s.d >> 3;
         if (tid < GH * per_row) {
-            const int g = tid / per_row, ch = tid - g * per_row;
+            const int g = idiv(tid, per_row), ch = tid - g * per_row;
             uint4 v = make_uint4(0, 0, 0, 0);
             if (g < ng) v = *reinterpret_cast<const uint4*>(q + ((size_t)b * s.Hq + g_first + g) * s.d + 8 * ch);
             *reinterpret_cast<uint4*>(qs_s + g * s.d + 8 * ch) = v;
         } else if (STEP && tid < (GH + 2) * per_row) {
-            const int side = (tid - GH * per_row) / per_row, ch = tid - (GH + side) * per_row;
+            const int side = tid >= (GH + 1) * per_row, ch = tid - (GH + side) * per_row;
             *reinterpret_cast<uint4*>(nrow_s + side * s.d + 8 * ch) =
                 *reinterpret_cast<const uint4*>((side == 0 ? k_new : v_new) + ((size_t)b * s.Hkv + h) * s.d + 8 * ch);
         }
@@ -699,10 +706,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         } else if (to_init) {
             new_buf = 0; new_row = n_init; new_tok = n_init; ++n_init;
         } else if (!evict) {
-            new_buf = 1; new_row = (head + n_local) % s.l_local; new_tok = n_init + n_local; ++n_local;
+            new_buf = 1; new_row = head + n_local - (head + n_local >= s.l_local ? s.l_local : 0); new_tok = n_init + n_local; ++n_local;
         } else {
             j_pend = n_mid_raw; ++n_mid_raw;
-            if (s.l_local > 0) { new_buf = 1; new_row = head; head = (head + 1) % s.l_local; new_tok = n_init + n_local - 1; }
+            if (s.l_local > 0) { new_buf = 1; new_row = head; head = head + 1 == s.l_local ? 0 : head + 1; new_tok = n_init + n_local - 1; }
         }
     }
     const int n_mid = min(n_mid_raw, s.max_mid);
@@ -710,7 +717,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     // the row that leaves the local window (or the new token itself without a local window), both sides, natural dim order
     if (j_pend >= 0 && tid >= kAll - 2 * (s.d >> 3) && tid < kAll) {
         const int t2 = tid - (kAll - 2 * (s.d >> 3));
-        const int side = t2 / (s.d >> 3), ch = t2 - side * (s.d >> 3);
+        const int side = t2 >= (s.d >> 3), ch = t2 - side * (s.d >> 3);
         if (s.l_local > 0)
             *reinterpret_cast<uint4*>(xrow_s + side * s.d + 8 * ch) =
                 *reinterpret_cast<const uint4*>(win_row<bf16>(side == 0 ? c.k_local : c.v_local, s, b, h, s.l_local, new_row) + 8 * ch);
@@ -729,7 +736,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 
     const int rowb_k = s.nfk * 2, rowb_v = s.nfv * 2;
     const int nhalf = (s.d + 63) >> 6;                                     // 64-dim boxes per window row
-    const int ts_k = rowb_k ? (kStageBytes / rowb_k) & ~15 : 0, ts_v = rowb_v ? (kStageBytes / rowb_v) & ~15 : 0;
+    const int ts_k = rowb_k ? idiv(kStageBytes, rowb_k) & ~15 : 0, ts_v = rowb_v ? idiv(kStageBytes, rowb_v) & ~15 : 0;
     const int ts_w = kWinRowsPerTile;
     // window tokens per softmax chunk: the score and probability buffers of all NB classes when
     // they can be addressed as one, else those of one class
@@ -843,7 +850,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     // gathered query of the compressed K dims (one element per thread and round), loaded early
     float qc_early = 0.f;
     if (p.fused && s.dck > 0 && tid < GH * s.dck) {
-        const int g = tid / s.dck, e = tid - g * s.dck;
+        const int g = idiv(tid, s.dck), e = tid - g * s.dck;
         if (g < ng) qc_early = __bfloat162float(qs_s[g * s.d + c.idx_comp_k[(size_t)h * s.dck + e]]);
     }
     // fused step: the coefficient update the light append kernel left pending (basis column j_pend, or -1);
@@ -958,7 +965,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             float* qc = reinterpret_cast<float*>(o_s);     // [GH][dck] gathered query, fp32 (o_s is not in use yet)
             const int32_t* idc_k = c.idx_comp_k + (size_t)h * s.dck;
             for (int i = tid; i < GH * s.dck; i += kAll) {
-                const int g = i / s.dck, e = i - g * s.dck;
+                const int g = idiv(i, s.dck), e = i - g * s.dck;
                 qc[i] = i < kAll ? qc_early : (g < ng ? __bfloat162float(qs_s[g * s.d + idc_k[e]]) : 0.f);
             }
             const int l8 = tid & 7, rgi = tid >> 3, nv = s.dck >> 2;
@@ -1009,7 +1016,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 #pragma unroll
                     for (int g = 1; g < GH; ++g) if (l8 == g) mine = a[g];
                     if (r < q1 && l8 < ng)
-                        ws.u[((size_t)b * s.Hq + g_first + l8) * s.M + r] = recon_weight(s.norm, r, s.k, s.T) * sl2 * mine;
+                        ws.u[((size_t)b * s.Hq + g_first + l8) * s.M + r] = w_row(r) * sl2 * mine;
                 }
             }
             TL(2);
@@ -1108,7 +1115,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     };
     const PC<N> czero = PC<N>{splat<N>(0.f), splat<N>(0.f)};
     auto seed_tw = [&](int n, int cls) -> float2 {
-        return cis_frac((float)((n * cls) & (s.T - 1)) / (float)s.T);
+        return cis_frac((float)((n * cls) & (s.T - 1)) * inv_T);
     };
 
     // fused step: writes the new token's row (all d dims) over row `prow` of a window tile (128-byte swizzle), by one warp
@@ -1156,7 +1163,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     const unsigned char* tile = wait_tile();
                     const int nrow = new_buf == sg.buf[si] ? new_row - (sg.row[si] + r0) : -1;   // fused step: the new token's row in this tile
                     #pragma unroll 1
-                    for (int grp = (wm + kMW - (it * (kWinRowsPerTile / 16)) % kMW) % kMW; grp * 16 < nt; grp += kMW) {   // tiles rotate over the warps
+                    for (int grp = (int)((unsigned)(wm + kMW) - (unsigned)(it * (kWinRowsPerTile / 16)) % (unsigned)kMW) % (unsigned)kMW; grp * 16 < nt; grp += kMW) {   // tiles rotate over the warps
                         if (STEP && nrow >= grp * 16 && nrow < grp * 16 + 16) patch_win(tile, nrow, knew_bh);
                         const unsigned char* r_lo = tile + (size_t)(grp * 16 + gq) * 128;      // row & 7 == gq for both rows
                         float d4[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1233,7 +1240,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     const unsigned char* tile = wait_tile();
                     const int nrow = new_buf == sg.buf[si] ? new_row - (sg.row[si] + r0) : -1;
                     #pragma unroll 1
-                    for (int grp = (wm + kMW - (it * (kWinRowsPerTile / 16)) % kMW) % kMW; grp * 16 < nt; grp += kMW) {
+                    for (int grp = (int)((unsigned)(wm + kMW) - (unsigned)(it * (kWinRowsPerTile / 16)) % (unsigned)kMW) % (unsigned)kMW; grp * 16 < nt; grp += kMW) {
                         if (STEP && nrow >= grp * 16 && nrow < grp * 16 + 16) patch_win(tile, nrow, vnew_bh);
                         const int a = sg.tok[si] + r0 + grp * 16;
                         // the tile's rows may start at any token of the chunk: gather the four p values one by one
@@ -1250,7 +1257,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                             const int rem = nt - grp * 16, per_row = nhalf * 8;
                             #pragma unroll 1
                             for (int i = lane; i < (16 - rem) * per_row; i += 32) {
-                                const int rr = grp * 16 + rem + i / per_row, cc = i % per_row;
+                                const int rr = grp * 16 + rem + idiv(i, per_row), cc = i - idiv(i, per_row) * per_row;
                                 *reinterpret_cast<uint4*>(const_cast<unsigned char*>(tile) + (cc >> 3) * kWinHalfBytes + rr * 128 + ((cc & 7) << 4)) =
                                     make_uint4(0, 0, 0, 0);
                             }
@@ -1809,7 +1816,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     };
     #pragma unroll 1
     for (int i = tid; i < (cp ? 1 : GH) * s.d; i += kAll) {
-        const int sl = i / s.d, e = i - sl * s.d, g = hperm<GH>(sl);      // hperm is its own inverse
+        const int sl = idiv(i, s.d), e = i - sl * s.d, g = hperm<GH>(sl);      // hperm is its own inverse
         if (g < ng) {
             float v = o_of(sl, e);
             if (cp) v = e0 * v + e1 * o_of(1, e);
@@ -1857,11 +1864,11 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     const int np = p.n_part;
     const int rows = m1 - m0;
     const size_t qh0 = (size_t)b * s.Hq + g_first;
-    const int nv = s.dcv >> 2, nrg = nv ? kAll / nv : 0;
+    const int nv = s.dcv >> 2, nrg = nv ? idiv(kAll, nv) : 0;
     // rows of the slice handled at a time: what the stage ring holds of C^V rows, z slices and weighted z
     constexpr int kRing = NS * kStageBytes / 4;
     const int head_f = (2 * GH * np + GH + 3) & ~3;
-    const int mch = max(4, min((rows + 3) & ~3, ((kRing - head_f - nrg * GH * s.dcv) / (GH + s.dcv + GH * np)) & ~3));
+    const int mch = max(4, min((rows + 3) & ~3, idiv(kRing - head_f - nrg * GH * s.dcv, GH + s.dcv + GH * np) & ~3));
     float* al_s = reinterpret_cast<float*>(stages);        // [GH][np] maxima, then exp2(m - max)
     float* l_s = al_s + GH * np;                           // [GH][np]
     float* linv_s = l_s + GH * np;                         // [GH]
@@ -1894,7 +1901,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             for (int e = tid; e < s.nfv; e += kAll) dv[v_mid_col(astar, e, s.nfv, FA_BF16)] = xrow_s[s.d + c.idx_full_v[(size_t)h * s.nfv + e]];
         }
         if (new_buf >= 0 && new_tok >= w0 && new_tok < w1 && tid < 2 * (s.d >> 3)) {
-            const int side = tid / (s.d >> 3), ch = tid - side * (s.d >> 3);
+            const int side = tid >= (s.d >> 3), ch = tid - side * (s.d >> 3);
             bf16* dst = new_buf == 0 ? win_row<bf16>(side == 0 ? c.k_init : c.v_init, s, b, h, s.l_init, new_row)
                                      : win_row<bf16>(side == 0 ? c.k_local : c.v_local, s, b, h, s.l_local, new_row);
             *reinterpret_cast<uint4*>(dst + 8 * ch) = *reinterpret_cast<const uint4*>((side == 0 ? knew_bh : vnew_bh) + 8 * ch);
@@ -1903,7 +1910,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 #pragma unroll 1
     for (int i = tid; i < GH * np; i += kAll) {
         float2 ml = make_float2(kNegBig, 0.f);
-        if (i / np < ng) ml = __ldcg(reinterpret_cast<const float2*>(ws.ml + (qh0 * np + i) * 2));
+        if (i < ng * np) ml = __ldcg(reinterpret_cast<const float2*>(ws.ml + (qh0 * np + i) * 2));
         al_s[i] = ml.x;
         l_s[i] = ml.y;
     }
@@ -1921,8 +1928,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             const int r4 = cr >> 2;
 #pragma unroll 1
             for (int i = tid; i < GH * np * r4; i += kAll) {
-                const int gs = i / r4, j = i - gs * r4, g = gs / np;
-                if (g < ng) cp_async16(zs_s + gs * mch + 4 * j, ws.z + (qh0 * np + gs) * s.M + m0 + r0 + 4 * j);
+                const int gs = idiv(i, r4), j = i - gs * r4;
+                if (gs < ng * np) cp_async16(zs_s + gs * mch + 4 * j, ws.z + (qh0 * np + gs) * s.M + m0 + r0 + 4 * j);
             }
         }
         cp_async_wait_all();
@@ -1948,19 +1955,19 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         if (s.dcv > 0) {
 #pragma unroll 1
             for (int t = tid; t < GH * cr; t += kAll) {
-                const int g = t / cr, r = t - g * cr;
+                const int g = idiv(t, cr), r = t - g * cr;
                 float v = 0.f;
                 if (g < ng) {
                     const float* z = zs_s + g * np * mch + r;
 #pragma unroll 2
                     for (int sp = 0; sp < np; ++sp) v = fmaf(al_s[g * np + sp], z[sp * mch], v);
-                    v *= recon_weight(s.norm, m0 + r0 + r, s.k, s.T);
+                    v *= w_row(m0 + r0 + r);
                 }
                 zw_s[g * mch + r] = v;
             }
             all_sync();
             if (tid < nrg * nv) {
-                const int v = tid % nv, rgi = tid / nv;
+                const int rgi = idiv(tid, nv), v = tid - rgi * nv;
 #pragma unroll 1
                 for (int r = rgi; r < cr; r += nrg) {
                     float4 x = *reinterpret_cast<const float4*>(cv_s + r * s.dcv + 4 * v);
@@ -1986,14 +1993,14 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     }
     if (s.dcv > 0) {
         if (tid < nrg * nv) {
-            const int v = tid % nv, rgi = tid / nv;
+            const int rgi = idiv(tid, nv), v = tid - rgi * nv;
 #pragma unroll
             for (int g = 0; g < GH; ++g) *reinterpret_cast<float4*>(ps_s + (rgi * GH + g) * s.dcv + 4 * v) = acc4[g];
         }
         all_sync();
 #pragma unroll 1
         for (int t = tid; t < GH * s.dcv; t += kAll) {
-            const int g = t / s.dcv, e = t - g * s.dcv;
+            const int g = idiv(t, s.dcv), e = t - g * s.dcv;
             float v = 0.f;
 #pragma unroll 1
             for (int rgi = 0; rgi < nrg; ++rgi) v += ps_s[(rgi * GH + g) * s.dcv + e];
@@ -2036,7 +2043,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     all_sync();
 #pragma unroll 1
     for (int t = tid; t < ng * s.d; t += kAll) {
-        const int g = t / s.d, e = t - g * s.d;
+        const int g = idiv(t, s.d), e = t - g * s.d;
         const float* o = op_s + g * np * s.d + e;
         float v = 0.f;
 #pragma unroll 2
