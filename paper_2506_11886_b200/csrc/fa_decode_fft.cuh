@@ -153,7 +153,7 @@ __device__ __forceinline__ void part_arrive(int32_t* cnt, int n, int tid) {
         asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
     }
 }
-template <int NT = kConsumers>
+template <int NT = kConsumers, int ID = 1>
 __device__ __forceinline__ void part_wait(const int32_t* cnt, int n, int tid, volatile int* fail, int32_t* status) {
     if (n > 1 && tid == 0 && !*fail) {
         bool ok = false;
@@ -165,7 +165,7 @@ __device__ __forceinline__ void part_wait(const int32_t* cnt, int n, int tid, vo
         }
         if (!ok) { *fail = 1; atomicExch(status, (int)FA_ERR_TIMEOUT); }
     }
-    consumer_sync<NT>();
+    consumer_sync<NT, ID>();
 }
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
@@ -765,8 +765,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 
     // ============================ producer warp =================================
     if (tid >= kAll) {
-        // Same order as the consumers: the K tiles of the first batch of classes, the window rows,
-        // then per batch the V tiles (and, from the second batch on, its K tiles first).
+        // Same order as the consumers: the window rows (they need nothing but q), then per batch of classes its K tiles and
+        // its V tiles.
         // One lane issues every tile of the CTA, and between a freed stage and its next tile stands this lane's chain of
         // instructions: it is what sets the rate of the streams (about 1.1 K cycles per 16 KB tile when addresses, stage
         // numbers and the failure flag were worked out per tile), so a tile costs an addition, one barrier test, the
@@ -785,12 +785,33 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 dst += kStageBytes;
                 if (++st == (uint32_t)NS) { st = 0; phase ^= 1; bar_u = full_u; dst = stages_base; }
             };
-            // K tiles of batch 0, windows, then V tiles of batch 0, K and V tiles of batch 1, ...: turn 2 i is the K side of
-            // batch i, turn 2 i + 1 its V side
+                            // window rows: tiles of 64 rows, one TMA box per 64 dims
+            #pragma unroll 1
+                            for (int t0 = w0; t0 < w1; t0 += wchunk) {
+                                const WinSegs sg = win_segments(t0, min(w1, t0 + wchunk), n_init, n_local, head, s.l_local);
+            #pragma unroll 1
+                                for (int i = 0; i < 2 * sg.n; ++i) {
+                                    const int sd = i >= sg.n, si = sd ? i - sg.n : i;
+                                    const CUtensorMap* tm = sg.buf[si] == 0 ? (sd == 0 ? &tm_ki : &tm_vi) : (sd == 0 ? &tm_kl : &tm_vl);
+                                    const int row1 = sg.row[si] + sg.cnt[si];
+            #pragma unroll 1
+                                    for (int r0 = sg.row[si]; r0 < row1; r0 += ts_w) {
+                                        if (!acquire((uint32_t)(nhalf * kWinHalfBytes))) return;
+            #pragma unroll 1
+                                        for (int hf = 0; hf < nhalf; ++hf)
+                                            asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+                                                             dst + hf * kWinHalfBytes),
+                                                         "l"(reinterpret_cast<uint64_t>(tm)), "r"(hf * 64), "r"(r0), "r"(b * s.Hkv + h), "r"(bar_u)
+                                                         : "memory");
+                                        advance();
+                                    }
+                                }
+                            }
+            // turn 2 i is the K side of batch i, turn 2 i + 1 its V side
 #pragma unroll 1
             for (int turn = 0;; ++turn) {
                 const int side = turn & 1, cb = c0 + (turn >> 1) * NB, cend = min(cb + NB, c1);
-                if (cb >= c1 && turn > 0) break;
+                if (cb >= c1) break;
                 const uint32_t rowb = (uint32_t)(side == 0 ? rowb_k : rowb_v), tile = rowb * (uint32_t)(side == 0 ? ts_k : ts_v);
                 const size_t cstride = (size_t)s.S_cap * rowb;                                     // bytes from one class to the next
                 const char* src_c = rowb ? reinterpret_cast<const char*>(side == 0 ? mid_row<bf16>(c.k_mid, s, b, h, cb, 0, s.nfk)
@@ -806,29 +827,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                                      "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(bar_u)
                                      : "memory");
                         advance();
-                    }
-                }
-                if (turn > 0) continue;
-                // window rows: tiles of 64 rows, one TMA box per 64 dims
-#pragma unroll 1
-                for (int t0 = w0; t0 < w1; t0 += wchunk) {
-                    const WinSegs sg = win_segments(t0, min(w1, t0 + wchunk), n_init, n_local, head, s.l_local);
-#pragma unroll 1
-                    for (int i = 0; i < 2 * sg.n; ++i) {
-                        const int sd = i >= sg.n, si = sd ? i - sg.n : i;
-                        const CUtensorMap* tm = sg.buf[si] == 0 ? (sd == 0 ? &tm_ki : &tm_vi) : (sd == 0 ? &tm_kl : &tm_vl);
-                        const int row1 = sg.row[si] + sg.cnt[si];
-#pragma unroll 1
-                        for (int r0 = sg.row[si]; r0 < row1; r0 += ts_w) {
-                            if (!acquire((uint32_t)(nhalf * kWinHalfBytes))) return;
-#pragma unroll 1
-                            for (int hf = 0; hf < nhalf; ++hf)
-                                asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
-                                                 dst + hf * kWinHalfBytes),
-                                             "l"(reinterpret_cast<uint64_t>(tm)), "r"(hf * 64), "r"(r0), "r"(b * s.Hkv + h), "r"(bar_u)
-                                             : "memory");
-                            advance();
-                        }
                     }
                 }
             }
@@ -956,9 +954,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             }
         }
     };
-    const bool has_classes = !is_win && c0 < c1 && n_of_class(c0) > 0;
-    // Fused kernel: this part's rows of u first, then the kept-dim scores of the first batch (they need
-    // only q) while the other parts finish theirs, then the wait for all of u.
+    // Fused kernel: this part's rows of u first, then the window tokens and the kept-dim scores of the first batch (they
+    // need only q) while the other parts finish theirs, then the wait for all of u.
     if (p.fused) {
         // u_g[m] = scale * log2(e) * w_m * sum_e C^K[m][e] q_g[D^kc[e]] for rows [m0, m1): eight lanes per row
         if (s.dck > 0) {
@@ -1023,38 +1020,40 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             part_arrive<kAll>(bar + 0, p.n_part, tid);
         }
         TL(3);
-        if (has_classes) k_phase(c0, min(NB, c1 - c0), kb);
-        TL(4);
-        if (s.dck > 0 && !is_win) part_wait<kAll>(bar + 0, p.n_part, tid, fail, c.status);
-        TL(5);
     } else {
-        if (has_classes) k_phase(c0, min(NB, c1 - c0), kb);
-        // everything above is independent of the prologue kernel; its output u is first needed here
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.wait;" ::: "memory");    // u and the workspace are the kernels' before this one
     }
     for (int i = tid; i < GH * s.d; i += kAll) o_s[i] = 0.f;
-    // ut[n] = (A.re, A.im, B.re, B.im), A = heads of the real slots, B = heads of the imaginary slots;
-    // all loads of an entry are issued together
     #pragma unroll 1
-    for (int n = tid; n < s.k; n += kAll) {
-        float2 uv[GH];
+    for (int i = tid; i < 2 * GH * s.k; i += kAll) z_s[i] = 0.f;
+    // ut[n] = (A.re, A.im, B.re, B.im), A = heads of the real slots, B = heads of the imaginary slots; all loads of
+    // an entry are issued together.  By the warps that build spectra, once the other parts' rows of u are in.
+    constexpr int kXf = SPLIT ? kConsumers : kAll, kXfBar = SPLIT ? 2 : 1;
+    auto load_u = [&]() {
+        if (s.dck == 0) return;
+        if (p.fused) part_wait<kXf, kXfBar>(bar + 0, p.n_part, tid, fail, c.status);
+        TL(5);
+        const float* ug = ws.u + ((size_t)b * s.Hq + g_first) * s.M;
+        #pragma unroll 1
+        for (int n = tid; n < s.k; n += kXf) {
+            float2 uv[GH];
 #pragma unroll
-        for (int sl = 0; sl < GH; ++sl) {
-            const int g = hperm<GH>(sl);
-            uv[sl] = make_float2(0.f, 0.f);
-            if (g < ng && s.dck > 0 && !is_win) uv[sl] = __ldcg(reinterpret_cast<const float2*>(ws.u + ((size_t)b * s.Hq + g_first + g) * s.M + 2 * n));
+            for (int sl = 0; sl < GH; ++sl) {
+                const int g = hperm<GH>(sl);
+                uv[sl] = make_float2(0.f, 0.f);
+                if (g < ng) uv[sl] = __ldcg(reinterpret_cast<const float2*>(ug + g * s.M + 2 * n));
+            }
+            float* e = ut + n * 2 * GH;
+            if constexpr (GH == 4) {
+                *reinterpret_cast<float4*>(e) = make_float4(0.5f * uv[0].x, 0.5f * uv[1].x, -0.5f * uv[0].y, -0.5f * uv[1].y);
+                *reinterpret_cast<float4*>(e + 4) = make_float4(0.5f * uv[2].x, 0.5f * uv[3].x, -0.5f * uv[2].y, -0.5f * uv[3].y);
+            } else {
+                *reinterpret_cast<float4*>(e) = make_float4(0.5f * uv[0].x, -0.5f * uv[0].y, 0.5f * uv[1].x, -0.5f * uv[1].y);
+            }
         }
-        float* e = ut + n * 2 * GH;
-        float* zz = z_s + n * 2 * GH;
-#pragma unroll
-        for (int sl = 0; sl < GH; ++sl) {
-            const int ab = sl / N, ln = sl - ab * N;
-            e[(2 * ab) * N + ln] = 0.5f * uv[sl].x;
-            e[(2 * ab + 1) * N + ln] = -0.5f * uv[sl].y;
-            zz[(2 * ab) * N + ln] = 0.f;
-            zz[(2 * ab + 1) * N + ln] = 0.f;
-        }
-    }
+        consumer_sync<kXf, kXfBar>();
+        TL(6);
+    };
     all_sync();
 
     float m_run[GH], l_acc[GH], o_scale[GH];              // per slot; o_scale: how far the class batches have rescaled o_s
@@ -1127,7 +1126,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         __syncwarp();
     };
 
-    TL(6);
     // ------------------------------ window tokens -------------------------------
     if (w1 > w0) {
         uint32_t qw[4][2][2];
@@ -1336,7 +1334,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         for (int cb = c0; cb < c1; cb += NB) {
             const int nb = min(NB, c1 - cb);
             if (n_of_class(cb) == 0) break;               // classes are filled in order: nothing further on
-            if (cb != c0) k_phase(cb, nb, kb);
+            k_phase(cb, nb, kb);
+            if (cb == c0) { TL(4); load_u(); }
             // transforms of the batch, and classes from one transform to the next
             const int nbt = cp ? (nb + 1) >> 1 : nb, cstep = cp ? 2 : 1;
 
@@ -1529,7 +1528,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             // read them), p_full (transform group -> tile group: probabilities and the rescale factors of the batch are
             // in), p_free (back: the V products have read them).  The scores of a batch are formed under its spectra and
             // score transform, its V products run under its probability transform and fold (and the next batch's
-            // scores under that batch's spectra).  Batch 0's scores were formed before the window tokens.
+            // scores under that batch's spectra).
             uint64_t* kb_full = reinterpret_cast<uint64_t*>(smem_raw + 160);
             uint64_t* kb_free = kb_full + 1;
             uint64_t* p_full = kb_full + 2;
@@ -1546,10 +1545,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     if (bi >= 1) {
                         if (lane == 0) mbar_wait(kb_free, (bi - 1) & 1, fail, c.status);   // softmax of the previous batch has read the scores
                         __syncwarp();
-                        k_phase(cb, nb, kb);
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(kb_full);
                     }
+                    k_phase(cb, nb, kb);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(kb_full);
                     if (lane == 0) mbar_wait(p_full, bi & 1, fail, c.status);   // one lane polls, the warp follows
                     __syncwarp();
                     {
@@ -1616,6 +1615,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                         mx[g] = r;
                     }
                 };
+                if (n_bat > 0) load_u();
                 #pragma unroll 1
                 for (int bi = 0; bi < n_bat; ++bi) {
                     const int cb = c0 + bi * NB, nb = min(NB, c1 - cb);
@@ -1660,11 +1660,9 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 xf_sync();
                 fft_run<GH, LS, LS, false, 2>(fbuf, fb_floats, nb, twf, tid);
             }
-                    // the kept-dim scores of this batch (batch 0: formed by everybody's earlier barriers)
-                    if (bi >= 1) {
-                        if (tid == 0) mbar_wait(kb_full, (bi - 1) & 1, fail, c.status);   // one thread polls
-                        xf_sync();
-                    }
+                    // the kept-dim scores of this batch
+                    if (tid == 0) mbar_wait(kb_full, bi & 1, fail, c.status);   // one thread polls
+                    xf_sync();
             // online softmax over the batch
             BatchSoftmax<GH, LS> sm;
             auto n0 = [&](int ci) { return n_of_class(cb + ci); };
