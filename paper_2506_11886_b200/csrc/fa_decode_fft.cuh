@@ -168,6 +168,26 @@ __device__ __forceinline__ void part_wait(const int32_t* cnt, int n, int tid, vo
     consumer_sync<NT, ID>();
 }
 
+__device__ __forceinline__ float warp_max_redux(float v) {
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+// Per-slot maximum over the threads of NW warps (barrier BID), broadcast to all of them; red: [NW][GH].
+template <int GH, int NW, int NT, int BID>
+__device__ __forceinline__ void block_max_t(float (&mx)[GH], float* red, int warp, int lane) {
+#pragma unroll
+    for (int g = 0; g < GH; ++g) mx[g] = warp_max_redux(mx[g]);
+    if (lane == 0) {
+        if constexpr (GH == 4) *reinterpret_cast<float4*>(red + 4 * warp) = make_float4(mx[0], mx[1], mx[2], mx[3]);
+        else *reinterpret_cast<float2*>(red + 2 * warp) = make_float2(mx[0], mx[1]);
+    }
+    consumer_sync<NT, BID>();
+    // (every lane takes one warp's maxima, a second reduction gives all lanes the result)
+#pragma unroll
+    for (int g = 0; g < GH; ++g) mx[g] = warp_max_redux(red[(lane % NW) * GH + g]);
+}
+
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                          uint32_t b1) {
     asm volatile(
@@ -190,6 +210,9 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a) {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
     return v;
+}
+__device__ __forceinline__ void sts128(uint32_t a, uint4 v) {
+    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 __device__ __forceinline__ void sts64(uint32_t a, float x, float y) {
     asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(a), "f"(x), "f"(y) : "memory");
@@ -499,6 +522,8 @@ __device__ __forceinline__ WinSegs win_segments(int t0, int t1, int n_init, int 
 struct FftSmem {
     int stages_off, fbuf_off, kb_off, pbt_off, twf_off, E_off, ut_off, z_off, o_off, inv_off, red_off, pend_off, zero_off, total;
     int fb_floats, pbs;
+    // derived sizes that every CTA would otherwise work out: rows of C^K staged at a time, rows of a K / V tile
+    int uch, ts_k, ts_v, wchunk, pbw;
 };
 // True if the kernel packs two residue classes of ONE query head into a complex transform (one query head per KV head:
 // the second slot would otherwise be empty).  Then a batch of NB classes needs half the transform and score buffers.
@@ -514,11 +539,19 @@ __host__ __device__ inline FftSmem fft_smem_layout(int log2S, int k, int GH, int
     off = 1024;                                           // stages are 1024-byte aligned (swizzled window tiles)
     L.stages_off = off; off += ring_stages(occ, split) * kStageBytes;
     // (also the warps' output fragments, [warp][slot][d], while no transform is under way)
-    L.fbuf_off = off; off += 4 * (NT * L.fb_floats > kWarps * GH * d ? NT * L.fb_floats : kWarps * GH * d);
+    int ff = NT * L.fb_floats > kWarps * GH * d ? NT * L.fb_floats : kWarps * GH * d;
+    if (ff < 136 * GH) ff = 136 * GH;
+    L.fbuf_off = off; off += 4 * ff;
     off = (off + 15) / 16 * 16;
     L.kb_off = off; off += 4 * NT * S * GH;               // kept-dim scores of the batch, natural token order
     off = (off + 15) / 16 * 16;
-    L.pbt_off = off; off += cp ? 2 * (NB + 1) * L.pbs : 2 * NB * GH * L.pbs;   // class pairs: one row per class and one of zeros
+    int np = cp ? (NB + 1) * L.pbs : NB * GH * L.pbs;     // class pairs: one row per class and one of zeros
+    if (np < 136 * GH) np = 136 * GH;
+    L.pbt_off = off; off += 2 * np;
+    // window tokens: probabilities of a slot pbw apart (an odd multiple of eight: conflict-free fragment loads); a chunk has
+    // room for its segments' padding to whole groups of 16
+    L.pbw = (((np / GH) - 8) & ~63) + 8;
+    L.wchunk = ((ff / GH < L.pbw ? ff / GH : L.pbw) & ~15) - 48;
     off = (off + 15) / 16 * 16;
     L.twf_off = off; off += 8 * (tw_total(log2S) + 1);
     off = (off + 15) / 16 * 16;
@@ -560,7 +593,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                                                                   const __grid_constant__ CUtensorMap tm_vi,
                                                                   const __grid_constant__ CUtensorMap tm_kl,
                                                                   const __grid_constant__ CUtensorMap tm_vl, Dims s, CacheDev c,
-                                                                  DecodePlan p, const bf16* __restrict__ q, bf16* __restrict__ out,
+                                                                  DecodePlan p, const __grid_constant__ FftSmem L, const bf16* __restrict__ q, bf16* __restrict__ out,
                                                                   char* wsp, const bf16* __restrict__ k_new,
                                                                   const bf16* __restrict__ v_new) {
     constexpr bool step = STEP;
@@ -578,7 +611,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the epilogue may be scheduled behind us at once
     Ws ws = ws_view(wsp, p);
     const int NB = p.nb;
-    const FftSmem L = fft_smem_layout(LS, s.k, GH, NB, s.d, OCC, SPLIT ? 1 : 0, class_pairs(s.G, GH, SPLIT ? 1 : 0));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw);
     uint64_t* empty = full + NS;
     volatile int* fail = reinterpret_cast<volatile int*>(smem_raw + 128);
@@ -643,7 +675,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     const int m0 = 4 * idiv(part * (s.M >> 2), p.n_part), m1 = 4 * idiv((part + 1) * (s.M >> 2), p.n_part);
     // rows of C^K staged at a time: the transform buffers and, behind them, the kept-dim score and probability
     // buffers (one contiguous area, all idle until the first batch)
-    const int uch = s.dck > 0 ? idiv((L.twf_off - L.fbuf_off) >> 2, s.dck) & ~3 : 0;
+    const int uch = L.uch;
     auto start_coef_rows = [&]() {
         if (tid >= kAll) return;
         if (s.dck > 0) {
@@ -736,14 +768,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 
     const int rowb_k = s.nfk * 2, rowb_v = s.nfv * 2;
     const int nhalf = (s.d + 63) >> 6;                                     // 64-dim boxes per window row
-    const int ts_k = rowb_k ? idiv(kStageBytes, rowb_k) & ~15 : 0, ts_v = rowb_v ? idiv(kStageBytes, rowb_v) & ~15 : 0;
-    const int ts_w = kWinRowsPerTile;
-    // window tokens per softmax chunk: the score and probability buffers of all NB classes when
-    // they can be addressed as one, else those of one class
-    const int NT = class_pairs(s.G, GH, SPLIT ? 1 : 0) ? (NB + 1) >> 1 : NB;       // transform buffers of a batch
-    const int wchunk = pf_size(NT * S * GH) <= NT * L.fb_floats ? NT * S : S;
-    // row stride of the window probabilities (class pairs: two rows in the NB + 1 rows of the classes)
-    const int pbw = class_pairs(s.G, GH, SPLIT ? 1 : 0) ? (((NB + 1) * L.pbs) >> 1) & ~7 : NB * L.pbs;
+    const int ts_k = L.ts_k, ts_v = L.ts_v;
 
     if (tid == 0) {
         for (int i = 0; i < NS; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, kMW); }
@@ -787,15 +812,15 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             };
                             // window rows: tiles of 64 rows, one TMA box per 64 dims
             #pragma unroll 1
-                            for (int t0 = w0; t0 < w1; t0 += wchunk) {
-                                const WinSegs sg = win_segments(t0, min(w1, t0 + wchunk), n_init, n_local, head, s.l_local);
+                            for (int t0 = w0; t0 < w1; t0 += L.wchunk) {
+                                const WinSegs sg = win_segments(t0, min(w1, t0 + L.wchunk), n_init, n_local, head, s.l_local);
             #pragma unroll 1
                                 for (int i = 0; i < 2 * sg.n; ++i) {
                                     const int sd = i >= sg.n, si = sd ? i - sg.n : i;
                                     const CUtensorMap* tm = sg.buf[si] == 0 ? (sd == 0 ? &tm_ki : &tm_vi) : (sd == 0 ? &tm_kl : &tm_vl);
                                     const int row1 = sg.row[si] + sg.cnt[si];
             #pragma unroll 1
-                                    for (int r0 = sg.row[si]; r0 < row1; r0 += ts_w) {
+                                    for (int r0 = sg.row[si]; r0 < row1; r0 += kWinRowsPerTile) {
                                         if (!acquire((uint32_t)(nhalf * kWinHalfBytes))) return;
             #pragma unroll 1
                                         for (int hf = 0; hf < nhalf; ++hf)
@@ -1060,23 +1085,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 #pragma unroll
     for (int g = 0; g < GH; ++g) { m_run[g] = kNegBig; l_acc[g] = 0.f; o_scale[g] = 1.f; }
     // per-slot maximum over per-thread partial maxima, broadcast to every consumer thread
-    auto block_max = [&](float (&mx)[GH]) {
-#pragma unroll
-        for (int g = 0; g < GH; ++g) {
-            float v = mx[g];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-            if (lane == 0) red_s[warp * GH + g] = v;
-        }
-        all_sync();
-#pragma unroll
-        for (int g = 0; g < GH; ++g) {
-            float r = red_s[g];
-#pragma unroll
-            for (int w = 1; w < kAllW; ++w) r = fmaxf(r, red_s[w * GH + g]);
-            mx[g] = r;
-        }
-    };
+    auto block_max = [&](float (&mx)[GH]) { block_max_t<GH, kAllW, kAll, 1>(mx, red_s, warp, lane); };
     auto load_vals = [&](const float* pt, float (&v)[GH]) {
         if constexpr (GH == 4) {
             const float4 x = *reinterpret_cast<const float4*>(pt);
@@ -1117,89 +1126,87 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         return cis_frac((float)((n * cls) & (s.T - 1)) * inv_T);
     };
 
-    // fused step: writes the new token's row (all d dims) over row `prow` of a window tile (128-byte swizzle), by one warp
-    auto patch_win = [&](const unsigned char* tile, int prow, const bf16* src) {
-#pragma unroll 1
-        for (int cc = lane; cc < npw; cc += 32)
-            *reinterpret_cast<uint4*>(const_cast<unsigned char*>(tile) + (cc >> 3) * kWinHalfBytes + prow * 128 + (((cc & 7) ^ (prow & 7)) << 4)) =
-                *reinterpret_cast<const uint4*>(src + 8 * cc);
-        __syncwarp();
-    };
-
     // ------------------------------ window tokens -------------------------------
+    // Scores and probabilities of a chunk lie in tile order: every segment of rows starts at a multiple of 16, the rows that
+    // fill up its last group score -inf.
     if (w1 > w0) {
-        uint32_t qw[4][2][2];
+        uint32_t qw[4][4];                                 // piece rd of the row: B fragments of its two k-steps
 #pragma unroll
-        for (int rd = 0; rd < 4; ++rd)
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-                // round rd covers the 16-byte pieces 2 tq + (rd & 1) of half rd >> 1: with the 128-byte
-                // swizzle the eight lanes of a quarter warp (two rows) then hit eight different bank groups
-                const int piece = ((rd >> 1) << 3) + 2 * tq + (rd & 1), e0 = 8 * piece + 4 * ks;
-                const bool on = col_on && piece < npw;
-                qw[rd][ks][0] = on ? pack_bf16(qrow[e0], qrow[e0 + 1]) : 0u;
-                qw[rd][ks][1] = on ? pack_bf16(qrow[e0 + 2], qrow[e0 + 3]) : 0u;
-            }
+        for (int rd = 0; rd < 4; ++rd) {
+            // round rd covers the 16-byte pieces 2 tq + (rd & 1) of half rd >> 1: with the 128-byte
+            // swizzle the eight lanes of a quarter warp (two rows) then hit eight different bank groups
+            const int piece = ((rd >> 1) << 3) + 2 * tq + (rd & 1);
+            uint4 x = make_uint4(0, 0, 0, 0);
+            if (col_on && piece < npw) x = *reinterpret_cast<const uint4*>(qrow + 8 * piece);
+            qw[rd][0] = x.x; qw[rd][1] = x.y; qw[rd][2] = x.z; qw[rd][3] = x.w;
+        }
         float accw[8][4];
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
             for (int i = 0; i < 4; ++i) accw[mt][i] = 0.f;
-        const int nmtw = (s.d + 15) >> 4;
-        float* sb = fbuf;                                 // natural order, no transform
-        bf16* pb = pbt;
-        #pragma unroll 1
-        for (int t0 = w0; t0 < w1; t0 += wchunk) {
-            const int n_tok = min(w1, t0 + wchunk) - t0;
-            const WinSegs sg = win_segments(t0, t0 + n_tok, n_init, n_local, head, s.l_local);
+        const int nmtw = (s.d + 15) >> 4, wchunk = L.wchunk, pbw = L.pbw;
+        const uint32_t sb_u = smem_addr(fbuf), pb_u = smem_addr(pbt);
+        // one pass over the tiles of a chunk's side: body(tile address, position of its first row, group, rows of the tile)
+        auto win_tiles = [&](const WinSegs& sg, const bf16* newrow, auto&& body) {
+            int pos = 0;
             #pragma unroll 1
-            for (int si = 0; si < sg.n; ++si)
+            for (int si = 0; si < sg.n; ++si) {
                 #pragma unroll 1
-                for (int r0 = 0; r0 < sg.cnt[si]; r0 += ts_w) {
-                    const int nt = min(ts_w, sg.cnt[si] - r0);
-                    if (!is_m) continue;
-                    const unsigned char* tile = wait_tile();
-                    const int nrow = new_buf == sg.buf[si] ? new_row - (sg.row[si] + r0) : -1;   // fused step: the new token's row in this tile
+                for (int r0 = 0; r0 < sg.cnt[si]; r0 += kWinRowsPerTile) {
+                    const int nt = min(kWinRowsPerTile, sg.cnt[si] - r0);
+                    const uint32_t tile = wait_tile_u();
+                    // tiles rotate over the warps
                     #pragma unroll 1
-                    for (int grp = (int)((unsigned)(wm + kMW) - (unsigned)(it * (kWinRowsPerTile / 16)) % (unsigned)kMW) % (unsigned)kMW; grp * 16 < nt; grp += kMW) {   // tiles rotate over the warps
-                        if (STEP && nrow >= grp * 16 && nrow < grp * 16 + 16) patch_win(tile, nrow, knew_bh);
-                        const unsigned char* r_lo = tile + (size_t)(grp * 16 + gq) * 128;      // row & 7 == gq for both rows
-                        float d4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                        for (int rd = 0; rd < 4; ++rd) {
-                            const int cj = 2 * tq + (rd & 1), piece = ((rd >> 1) << 3) + cj;
-                            if (((rd >> 1) << 3) < npw) {
-                                uint4 lo = make_uint4(0, 0, 0, 0), hi = make_uint4(0, 0, 0, 0);
-                                if (piece < npw) {
-                                    const unsigned char* src = r_lo + (rd >> 1) * kWinHalfBytes + ((cj ^ gq) << 4);
-                                    lo = *reinterpret_cast<const uint4*>(src);
-                                    hi = *reinterpret_cast<const uint4*>(src + 8 * 128);
-                                }
-                                mma_bf16(d4, lo.x, hi.x, lo.y, hi.y, qw[rd][0][0], qw[rd][0][1]);
-                                mma_bf16(d4, lo.z, hi.z, lo.w, hi.w, qw[rd][1][0], qw[rd][1][1]);
+                    for (int grp = (int)((unsigned)(wm + 4 * kMW) - (unsigned)(it & 3) * (kWinRowsPerTile / 16)) % kMW; grp * 16 < nt; grp += kMW) {
+                        if (STEP) {
+                            // fused step: the new token's row is not in the cache yet
+                            const int prow = new_buf == sg.buf[si] ? new_row - (sg.row[si] + r0) : -1;
+                            if (prow >= grp * 16 && prow < grp * 16 + 16) {
+                                if (lane < npw)
+                                    sts128(tile + (lane >> 3) * kWinHalfBytes + prow * 128 + (((lane & 7) ^ (prow & 7)) << 4),
+                                           *reinterpret_cast<const uint4*>(newrow + 8 * lane));
+                                __syncwarp();
                             }
                         }
-                        if (2 * tq < GH) {
-                            const int i_lo = grp * 16 + gq, i_hi = i_lo + 8;
-                            if (i_lo < nt)
-                                *reinterpret_cast<float2*>(sb + pf((sg.tok[si] + r0 + i_lo) * GH + 2 * tq)) = make_float2(d4[0] * sl2, d4[1] * sl2);
-                            if (i_hi < nt)
-                                *reinterpret_cast<float2*>(sb + pf((sg.tok[si] + r0 + i_hi) * GH + 2 * tq)) = make_float2(d4[2] * sl2, d4[3] * sl2);
-                        }
+                        body(tile + grp * 16 * 128, pos + r0 + grp * 16, nt - grp * 16);
                     }
                     release_tile();
                 }
-            all_sync();
-            float mx[GH], alpha[GH];
-#pragma unroll
-            for (int g = 0; g < GH; ++g) mx[g] = kNegBig;
-            #pragma unroll 1
-            for (int a = tid; a < n_tok; a += kAll) {
-                float v[GH];
-                load_vals(sb + pf(a * GH), v);
-#pragma unroll
-                for (int g = 0; g < GH; ++g) if (!(cp && g == 1)) mx[g] = fmaxf(mx[g], v[g]);
+                pos += (sg.cnt[si] + 15) & ~15;
             }
+            return pos;
+        };
+        #pragma unroll 1
+        for (int t0 = w0; t0 < w1; t0 += wchunk) {
+            const WinSegs sg = win_segments(t0, min(w1, t0 + wchunk), n_init, n_local, head, s.l_local);
+            float mx[GH], alpha[GH], m_lo = kNegBig, m_hi = kNegBig;
+            if (is_m)
+                win_tiles(sg, knew_bh, [&](uint32_t rows, int pos, int rem) {
+                    const uint32_t r_lo = rows + gq * 128;            // row & 7 == gq for both rows
+                    float da[4] = {0.f, 0.f, 0.f, 0.f}, db[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int rd = 0; rd < 4; ++rd) {
+                        if ((rd >> 1) < nhalf) {                      // (dims past head_dim arrive as zeros)
+                            const uint32_t src = r_lo + (rd >> 1) * kWinHalfBytes + (((2 * tq + (rd & 1)) ^ gq) << 4);
+                            const uint4 lo = lds128(src), hi = lds128(src + 8 * 128);
+                            mma_bf16(da, lo.x, hi.x, lo.y, hi.y, qw[rd][0], qw[rd][1]);
+                            mma_bf16(db, lo.z, hi.z, lo.w, hi.w, qw[rd][2], qw[rd][3]);
+                        }
+                    }
+                    if (2 * tq < GH) {
+                        const bool ok_lo = gq < rem, ok_hi = gq + 8 < rem;
+                        const float x0 = ok_lo ? (da[0] + db[0]) * sl2 : 2.f * kNegBig, y0 = ok_lo && !cp ? (da[1] + db[1]) * sl2 : 2.f * kNegBig;
+                        const float x1 = ok_hi ? (da[2] + db[2]) * sl2 : 2.f * kNegBig, y1 = ok_hi && !cp ? (da[3] + db[3]) * sl2 : 2.f * kNegBig;
+                        m_lo = fmaxf(m_lo, fmaxf(x0, x1));
+                        m_hi = fmaxf(m_hi, fmaxf(y0, y1));
+                        const uint32_t dst = sb_u + (uint32_t)((pos + gq) * GH + 2 * tq) * 4;
+                        sts64(dst, x0, y0);
+                        sts64(dst + 8 * GH * 4, x1, y1);
+                    }
+                });
+#pragma unroll
+            for (int g = 0; g < GH; ++g) mx[g] = g == 2 * tq ? m_lo : g == 2 * tq + 1 ? m_hi : kNegBig;
             block_max(mx);
 #pragma unroll
             for (int g = 0; g < GH; ++g) {
@@ -1208,18 +1215,18 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 m_run[g] = m_new;
                 l_acc[g] *= alpha[g];
             }
-            const int n_pad = (n_tok + 15) & ~15;
+            int n_pos = 0;
             #pragma unroll 1
-            for (int a = tid; a < n_pad; a += kAll) {
+            for (int si = 0; si < sg.n; ++si) n_pos += (sg.cnt[si] + 15) & ~15;
+            #pragma unroll 1
+            for (int a = tid; a < n_pos; a += kAll) {
                 float v[GH];
-#pragma unroll
-                for (int g = 0; g < GH; ++g) v[g] = 0.f;
-                if (a < n_tok) load_vals(sb + pf(a * GH), v);
+                load_vals(fbuf + a * GH, v);
 #pragma unroll
                 for (int g = 0; g < GH; ++g) {
-                    v[g] = (a < n_tok && !(cp && g == 1)) ? ex2(v[g] - m_run[g]) : 0.f;
+                    v[g] = ex2(v[g] - m_run[g]);
                     l_acc[g] += v[g];
-                    pb[g * pbw + a] = __float2bfloat16_rn(v[g]);
+                    pbt[g * pbw + a] = __float2bfloat16_rn(v[g]);
                 }
             }
             {
@@ -1228,54 +1235,34 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 for (int mt = 0; mt < 8; ++mt) { accw[mt][0] *= al; accw[mt][1] *= ah; accw[mt][2] *= al; accw[mt][3] *= ah; }
             }
             all_sync();
-            const bf16* prow = pb + (size_t)(gq & (GH - 1)) * pbw;
-            #pragma unroll 1
-            for (int si = 0; si < sg.n; ++si)
-                #pragma unroll 1
-                for (int r0 = 0; r0 < sg.cnt[si]; r0 += ts_w) {
-                    const int nt = min(ts_w, sg.cnt[si] - r0);
-                    if (!is_m) continue;
-                    const unsigned char* tile = wait_tile();
-                    const int nrow = new_buf == sg.buf[si] ? new_row - (sg.row[si] + r0) : -1;
-                    #pragma unroll 1
-                    for (int grp = (int)((unsigned)(wm + kMW) - (unsigned)(it * (kWinRowsPerTile / 16)) % (unsigned)kMW) % (unsigned)kMW; grp * 16 < nt; grp += kMW) {
-                        if (STEP && nrow >= grp * 16 && nrow < grp * 16 + 16) patch_win(tile, nrow, vnew_bh);
-                        const int a = sg.tok[si] + r0 + grp * 16;
-                        // the tile's rows may start at any token of the chunk: gather the four p values one by one
-                        uint32_t b0 = 0, b1 = 0;
-                        if (gq < GH) {
-                            const int rem = nt - grp * 16;
-                            const bf16 zero = __float2bfloat16_rn(0.f);
-                            b0 = pack_bf16(2 * tq < rem ? prow[a + 2 * tq] : zero, 2 * tq + 1 < rem ? prow[a + 2 * tq + 1] : zero);
-                            b1 = pack_bf16(2 * tq + 8 < rem ? prow[a + 2 * tq + 8] : zero, 2 * tq + 9 < rem ? prow[a + 2 * tq + 9] : zero);
-                        }
-                        if (nt - grp * 16 < 16) {
-                            // rows past the end of the segment hold whatever follows it in the cache: zero them,
-                            // p = 0 does not stop a NaN
-                            const int rem = nt - grp * 16, per_row = nhalf * 8;
+            const uint32_t prow_u = pb_u + (uint32_t)((gq & (GH - 1)) * pbw + 2 * tq) * 2;
+            const int mi = lane >> 3, tok = ((mi >> 1) << 3) + (lane & 7);
+            const uint32_t v_lane = tok * 128, v_sw = (uint32_t)((tok & 7) ^ (mi & 1)) << 4;
+            if (is_m)
+                win_tiles(sg, vnew_bh, [&](uint32_t rows, int pos, int rem) {
+                    uint32_t b0 = 0, b1 = 0;
+                    if (gq < GH) {
+                        b0 = lds32(prow_u + pos * 2);
+                        b1 = lds32(prow_u + pos * 2 + 16);
+                    }
+                    if (rem < 16) {
+                        // rows past the end of the segment hold whatever follows it in the cache: zero them,
+                        // p = 0 does not stop a NaN
+                        #pragma unroll 1
+                        for (int i = lane; i < (16 - rem) * 8; i += 32)
                             #pragma unroll 1
-                            for (int i = lane; i < (16 - rem) * per_row; i += 32) {
-                                const int rr = grp * 16 + rem + idiv(i, per_row), cc = i - idiv(i, per_row) * per_row;
-                                *reinterpret_cast<uint4*>(const_cast<unsigned char*>(tile) + (cc >> 3) * kWinHalfBytes + rr * 128 + ((cc & 7) << 4)) =
-                                    make_uint4(0, 0, 0, 0);
-                            }
-                            __syncwarp();
-                        }
-                        const int mi = lane >> 3, tok = ((mi >> 1) << 3) + (lane & 7);
-                        const unsigned char* vrow = tile + (size_t)(grp * 16 + tok) * 128;
+                            for (int hf = 0; hf < nhalf; ++hf) sts128(rows + hf * kWinHalfBytes + (uint32_t)(rem * 8 + i) * 16, make_uint4(0, 0, 0, 0));
+                        __syncwarp();
+                    }
 #pragma unroll
-                        for (int mt = 0; mt < 8; ++mt) {
-                            if (mt < nmtw) {
-                                const int chunk = 2 * mt + (mi & 1);
-                                const unsigned char* src = chunk < npw ? vrow + (chunk >> 3) * kWinHalfBytes + (((chunk & 7) ^ (tok & 7)) << 4) : zero16;
-                                uint32_t af[4];
-                                ldmatrix_x4_trans(af, smem_addr(src));
-                                mma_bf16(accw[mt], af[0], af[1], af[2], af[3], b0, b1);
-                            }
+                    for (int mt = 0; mt < 8; ++mt) {
+                        if (mt < nmtw) {
+                            uint32_t af[4];
+                            ldmatrix_x4_trans(af, rows + v_lane + (mt >> 2) * kWinHalfBytes + (v_sw ^ (uint32_t)((2 * mt & 7) << 4)));
+                            mma_bf16(accw[mt], af[0], af[1], af[2], af[3], b0, b1);
                         }
                     }
-                    release_tile();
-                }
+                });
             all_sync();
         }
         // the warps' fragments side by side, then summed in warp order (the same bits on every run)
@@ -1597,24 +1584,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 }
             } else {
                 // ================= transform group =================
-                // per-slot maximum over the group's threads (as block_max, on the group's barrier)
-                auto block_max_t = [&](float (&mx)[GH]) {
-#pragma unroll
-                    for (int g = 0; g < GH; ++g) {
-                        float v = mx[g];
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-                        if (lane == 0) red_s[warp * GH + g] = v;
-                    }
-                    xf_sync();
-#pragma unroll
-                    for (int g = 0; g < GH; ++g) {
-                        float r = red_s[g];
-#pragma unroll
-                        for (int w = 1; w < kWarps; ++w) r = fmaxf(r, red_s[w * GH + g]);
-                        mx[g] = r;
-                    }
-                };
                 if (n_bat > 0) load_u();
                 #pragma unroll 1
                 for (int bi = 0; bi < n_bat; ++bi) {
@@ -1670,7 +1639,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 #pragma unroll
             for (int g = 0; g < GH; ++g) mx[g] = kNegBig;
             sm.scores(fbuf, fb_floats, nb, kbuf, ts_k != 0, s.dck > 0, tid, n0, n0, mx);
-            block_max_t(mx);
+            block_max_t<GH, kWarps, kConsumers, 2>(mx, red_s, warp, lane);
 #pragma unroll
             for (int g = 0; g < GH; ++g) {
                 const float m_new = fmaxf(m_run[g], mx[g]);
@@ -2074,7 +2043,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
 template <int GH, int LS, int OCC, bool STEP, bool SPLIT = false>
 cudaError_t launch_fft_t(const Dims& s, const CacheDev& c, const DecodePlan& p, const void* q, void* out, char* ws, int step,
                          const void* k_new, const void* v_new, cudaStream_t st) {
-    const FftSmem L = fft_smem_layout(LS, s.k, GH, p.nb, s.d, OCC, SPLIT ? 1 : 0, class_pairs(s.G, GH, SPLIT ? 1 : 0));
+    FftSmem L = fft_smem_layout(LS, s.k, GH, p.nb, s.d, OCC, SPLIT ? 1 : 0, class_pairs(s.G, GH, SPLIT ? 1 : 0));
+    L.uch = s.dck > 0 ? (((L.twf_off - L.fbuf_off) >> 2) / s.dck) & ~3 : 0;
+    L.ts_k = s.nfk ? (kStageBytes / (2 * s.nfk)) & ~15 : 0;
+    L.ts_v = s.nfv ? (kStageBytes / (2 * s.nfv)) & ~15 : 0;
     cudaError_t err = ensure_dynamic_smem(decode_fft_kernel<GH, LS, OCC, STEP, SPLIT>, (size_t)L.total);
     if (err != cudaSuccess) return err;
     // window buffers as tensor maps (cached per buffer)
@@ -2106,7 +2078,7 @@ cudaError_t launch_fft_t(const Dims& s, const CacheDev& c, const DecodePlan& p, 
             cfg.attrs = attr + 1;                                          // not probed yet: stay on the plain cooperative launch
         } else if (known != 0) {
             cfg.numAttrs = 2;
-            cudaError_t err2 = cudaLaunchKernelEx(&cfg, decode_fft_kernel<GH, LS, OCC, STEP, SPLIT>, tki, tvi, tkl, tvl, s, c, p,
+            cudaError_t err2 = cudaLaunchKernelEx(&cfg, decode_fft_kernel<GH, LS, OCC, STEP, SPLIT>, tki, tvi, tkl, tvl, s, c, p, L,
                                                   static_cast<const bf16*>(q), static_cast<bf16*>(out), ws,
                                                   static_cast<const bf16*>(k_new), static_cast<const bf16*>(v_new));
             if (err2 == cudaSuccess) { coop_pdl_state(1); return err2; }
@@ -2119,7 +2091,7 @@ cudaError_t launch_fft_t(const Dims& s, const CacheDev& c, const DecodePlan& p, 
             cfg.attrs = attr + 1;
         }
     }
-    return cudaLaunchKernelEx(&cfg, decode_fft_kernel<GH, LS, OCC, STEP, SPLIT>, tki, tvi, tkl, tvl, s, c, p, static_cast<const bf16*>(q),
+    return cudaLaunchKernelEx(&cfg, decode_fft_kernel<GH, LS, OCC, STEP, SPLIT>, tki, tvi, tkl, tvl, s, c, p, L, static_cast<const bf16*>(q),
                               static_cast<bf16*>(out), ws, static_cast<const bf16*>(k_new), static_cast<const bf16*>(v_new));
 }
 
