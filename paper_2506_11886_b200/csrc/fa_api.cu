@@ -258,13 +258,16 @@ fa_status plan_decode(const fa_layout& l, DecodePlan* p) {
     p->n_slice = s.dcv > 0 ? (s.M + 63) / 64 : 1;
     size_t off = 0;
     p->off_bar = off; off = align_up(off + sizeof(int32_t) * 4 * (size_t)kBarSlots, 256);   // same place and size for every layout
-    p->off_u = off;   off = align_up(off + sizeof(float) * (size_t)s.B * s.Hq * s.M, 256);
-    p->off_ml = off;  off = align_up(off + sizeof(float) * (size_t)s.B * s.Hq * p->n_part * 2, 256);
-    p->off_o = off;   off = align_up(off + sizeof(float) * (size_t)s.B * s.Hq * p->n_part * s.d, 256);
-    p->off_z = off;   off = align_up(off + sizeof(float) * (size_t)s.B * s.Hq * p->n_part * s.M, 256);
-    const int n_oc = p->n_slice > p->n_part ? p->n_slice : p->n_part;
-    p->off_oc = off;  off = align_up(off + sizeof(float) * (size_t)s.B * s.Hq * n_oc * (s.dcv > 0 ? s.dcv : 1), 256);
-    p->off_om = off;  off = align_up(off + sizeof(float) * (size_t)s.B * s.Hq * s.d, 256);
+    // heads as the kernels' passes take them (gh to a pass); a part on its own exchanges nothing
+    const size_t heads = (size_t)s.B * (p->algo == FA_DECODE_FFT && p->fused ? s.Hkv * p->n_pass * p->gh : s.Hq);
+    const size_t parts = p->fused && p->n_part == 1 ? 0 : (size_t)p->n_part, zparts = p->fused ? (parts ? (size_t)p->n_split : 0) : parts;
+    p->off_u = off;   off = align_up(off + sizeof(float) * (p->fused && !parts ? 0 : heads * s.M), 256);
+    p->off_ml = off;  off = align_up(off + sizeof(float) * heads * parts * 2, 256);
+    p->off_o = off;   off = align_up(off + sizeof(float) * heads * parts * s.d, 256);
+    p->off_z = off;   off = align_up(off + sizeof(float) * heads * zparts * s.M, 256);
+    const size_t n_oc = p->fused ? parts : (size_t)(p->n_slice > p->n_part ? p->n_slice : p->n_part);
+    p->off_oc = off;  off = align_up(off + sizeof(float) * heads * n_oc * (s.dcv > 0 ? s.dcv : 1), 256);
+    p->off_om = off;  off = align_up(off + sizeof(float) * heads * s.d, 256);
     p->off_cnt = off; off = align_up(off + sizeof(int32_t) * (size_t)s.B * s.Hkv, 256);
     p->total = off;
     return FA_OK;

@@ -79,12 +79,12 @@ bool decode_fft_fused_fits(const Dims& s, int log2S, int gh, int nb, int n_part,
     const FftSmem L = fft_smem_layout(log2S, s.k, gh, nb, s.d, occ, split, class_pairs(s.G, gh, split));
     // at least eight rows of C^K per staged chunk (class pairs: the chunk may use the score and probability buffers too, as the kernel does)
     if (s.dck > 0 && (class_pairs(s.G, gh, split) ? (long long)((L.twf_off - L.fbuf_off) >> 2) : (long long)nb * L.fb_floats) < 8LL * s.dck) return false;
-    const long long ring = (long long)ring_stages(occ, split) * kStageBytes / 4;
-    const long long nrg = s.dcv ? (split ? kSplitConsumers : kConsumers) / (s.dcv >> 2) : 0;
-    const long long head = ((2LL * gh * n_part + gh + 3) & ~3LL);
-    if (s.dcv > 0 && (ring - head - nrg * gh * s.dcv) / (gh + s.dcv + (long long)gh * n_part) < 8) return false;   // and of C^V
-    const long long step2 = (long long)gh * n_part * (s.d + s.dcv) + s.d;               // the last part's merge of all parts
-    return head + 8LL * gh + step2 <= ring;
+    const int ring = ring_stages(occ, split) * kStageBytes / 4;
+    const int nrg = s.dcv ? (split ? kSplitConsumers : kConsumers) / (s.dcv >> 2) : 0;
+    const int rows = (s.M / 4 + n_part - 1) / n_part * 4 + 4;
+    const MergePlan m = merge_plan(ring, gh, n_part, n_part, s.d, s.dcv, nrg, rows);
+    if (s.dcv > 0 && m.mch < 8) return false;                                                 // rows of C^V at a time
+    return m.head + (long long)gh * n_part * s.dcv + gh * s.d <= ring;                        // the last part's merge of all parts
 }
 
 cudaError_t launch_decode_fft(const Dims& s, const CacheDev& c, int dtype, const DecodePlan& p, const void* q, void* out,

@@ -94,6 +94,9 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count));
 }
+__device__ __forceinline__ void mbar_arrive_u(uint32_t b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
+}
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(b)) : "memory");
 }
@@ -569,6 +572,23 @@ __host__ __device__ inline FftSmem fft_smem_layout(int log2S, int k, int GH, int
     return L;
 }
 
+// Shared memory of the merge in the stage ring (floats): head = the parts' (m, l) and the 1 / l; mch = coefficient rows
+// handled at a time (weighted z, rows of C^V, the parts' z); o_per = a part's slice of the outputs.
+struct MergePlan {
+    int head, mch, o_per;
+};
+__host__ __device__ inline MergePlan merge_plan(int ring, int GH, int np, int nz, int d, int dcv, int nrg, int rows) {
+    MergePlan m;
+    m.head = (2 * GH * np + GH + 3) & ~3;
+    m.o_per = ((GH * d + np - 1) / np + 3) & ~3;
+    const int room = ring - m.head - nrg * GH * dcv - (np > 1 ? np * m.o_per : 0), per_row = GH + dcv + (np > 1 ? GH * nz : 0);
+    m.mch = (room / per_row) & ~3;
+    const int all = (rows + 3) & ~3;
+    if (m.mch > all) m.mch = all;
+    if (m.mch < 4) m.mch = 4;
+    return m;
+}
+
 // Fused step: the kept dims of the middle token that is not in the cache yet, written by one warp over its row of a
 // tile in shared memory.  Out of line: taken once per kernel, and the tile loops keep their registers.
 __device__ __noinline__ void patch_mid_k(uint32_t row_addr, const int32_t* idf, int nfk, const bf16* xrow, int lane) {
@@ -624,7 +644,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     float* ut = reinterpret_cast<float*>(smem_raw + L.ut_off);            // [k] (A.re, A.im, B.re, B.im) x N: (1/2) u~
     float* z_s = reinterpret_cast<float*>(smem_raw + L.z_off);            // [k] same packing
     float* o_s = reinterpret_cast<float*>(smem_raw + L.o_off);            // [GH slots][d] what the window tokens give
-    int16_t* inv_v = reinterpret_cast<int16_t*>(smem_raw + L.inv_off);    // [d] position of a dim in D^vu, or -1
+    int16_t* inv_v = reinterpret_cast<int16_t*>(smem_raw + L.inv_off);    // [d] position of a dim in D^vu, or -1 - position in D^vc
     float* red_s = reinterpret_cast<float*>(smem_raw + L.red_off);        // [kAllW][GH] + l_s[GH]
     const int fb_floats = L.fb_floats, pbs = L.pbs;
 
@@ -668,7 +688,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             l -= rl;
         }
         if (tid < GH + 8) red_s[kAllW * GH + tid] = 0.f;
-        for (int e = tid; e < s.d; e += kAll) inv_v[e] = -1;
     }
     // This part's rows of C^K start towards the transform buffers, and its rows of C^V towards L2, as soon as
     // the kernels before this one are done (the previous step's kernel writes coefficient rows).
@@ -867,7 +886,11 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     const int npk = s.nfk >> 3, nchv = s.nfv >> 3, npw = s.d >> 3;
     const float sl2 = s.scale * kLog2e;
 
-    for (int e = tid; e < s.nfv; e += kAll) inv_v[c.idx_full_v[(size_t)h * s.nfv + e]] = (int16_t)e;
+    // where a dim of V is: e in D^vu as e, in D^vc as -1 - e
+    if (tid < s.d) {
+        if (tid < s.nfv) inv_v[c.idx_full_v[h * s.nfv + tid]] = (int16_t)tid;
+        else inv_v[c.idx_comp_v[h * s.dcv + tid - s.nfv]] = (int16_t)(s.nfv - 1 - tid);
+    }
 
     int32_t* bar = ws.bar + 4 * (((size_t)b * s.Hkv + h) * p.n_pass + pass);
     // gathered query of the compressed K dims (one element per thread and round), loaded early
@@ -905,23 +928,18 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 qk[rd][ks][1] = on ? pack_bf16(qrow[idf_k[e0 + 2]], qrow[idf_k[e0 + 3]]) : 0u;
             }
     }
-    int it = 0;                                           // tile counter, mirrors the producer's
-
-    auto wait_tile = [&]() -> const unsigned char* {
-        const int st = it % NS;
-        mbar_wait(full + st, (it / NS) & 1, fail, c.status);
-        return stages + (size_t)st * kStageBytes;
-    };
-    const uint32_t stages_u = smem_addr(stages), zero_u = smem_addr(zero16);
-    auto wait_tile_u = [&]() -> uint32_t {                // the same, as a shared-memory address
-        const int st = it % NS;
-        mbar_wait(full + st, (it / NS) & 1, fail, c.status);
-        return stages_u + (uint32_t)st * kStageBytes;
+    // the ring as the consumers see it: stage and phase of the next tile, in the producer's order
+    const uint32_t stages_u = smem_addr(stages), zero_u = smem_addr(zero16), full_u = smem_addr(full);
+    uint32_t c_st = 0, c_ph = 0, c_par = 0;               // c_par: parity of the tile
+    auto wait_tile_u = [&]() -> uint32_t {
+        if (!mbar_try_wait(full_u + 8 * c_st, c_ph)) mbar_wait_slow(full_u + 8 * c_st, c_ph, fail, c.status);
+        return stages_u + c_st * kStageBytes;
     };
     auto release_tile = [&]() {
         __syncwarp();
-        if (lane == 0) mbar_arrive(empty + (it % NS));
-        ++it;
+        if (lane == 0) mbar_arrive_u(full_u + 8 * (NS + c_st));
+        c_par ^= 1;
+        if (++c_st == (uint32_t)NS) { c_st = 0; c_ph ^= 1; }
     };
     // kept dims of one batch of classes: kb[class][token][slot] = sl2 * (q_u . K^mu), 16 tokens per mma.
     // It needs nothing but q, so the first batch runs before u is known.
@@ -981,6 +999,11 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     };
     // Fused kernel: this part's rows of u first, then the window tokens and the kept-dim scores of the first batch (they
     // need only q) while the other parts finish theirs, then the wait for all of u.
+    // Exchange areas of this (b, KV head, pass): u, and of every part (m, l) per slot, o, z (window parts have no z),
+    // its slice of o^c; all in slot order.  u and z as ut / z_s hold them.  A part on its own exchanges nothing.
+    constexpr int EF = 2 * GH;                            // floats of an entry of ut / z_s
+    const int np = p.n_part, nz = p.n_split, job = (b * s.Hkv + h) * p.n_pass + pass;
+    float* ug = np > 1 ? ws.u + (size_t)job * (EF * s.k) : ut;
     if (p.fused) {
         // u_g[m] = scale * log2(e) * w_m * sum_e C^K[m][e] q_g[D^kc[e]] for rows [m0, m1): eight lanes per row
         if (s.dck > 0) {
@@ -1037,8 +1060,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     float mine = a[0];
 #pragma unroll
                     for (int g = 1; g < GH; ++g) if (l8 == g) mine = a[g];
-                    if (r < q1 && l8 < ng)
-                        ws.u[((size_t)b * s.Hq + g_first + l8) * s.M + r] = w_row(r) * sl2 * mine;
+                    if (r < q1 && l8 < GH) {
+                        const int sl = hperm<GH>(l8);
+                        ug[(r >> 1) * EF + (2 * (sl / N) + (r & 1)) * N + (sl & (N - 1))] = ((r & 1) ? -0.5f : 0.5f) * w_row(r) * sl2 * mine;
+                    }
                 }
             }
             TL(2);
@@ -1058,22 +1083,17 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         if (s.dck == 0) return;
         if (p.fused) part_wait<kXf, kXfBar>(bar + 0, p.n_part, tid, fail, c.status);
         TL(5);
-        const float* ug = ws.u + ((size_t)b * s.Hq + g_first) * s.M;
-        #pragma unroll 1
-        for (int n = tid; n < s.k; n += kXf) {
-            float2 uv[GH];
-#pragma unroll
-            for (int sl = 0; sl < GH; ++sl) {
-                const int g = hperm<GH>(sl);
-                uv[sl] = make_float2(0.f, 0.f);
-                if (g < ng) uv[sl] = __ldcg(reinterpret_cast<const float2*>(ug + g * s.M + 2 * n));
-            }
-            float* e = ut + n * 2 * GH;
-            if constexpr (GH == 4) {
-                *reinterpret_cast<float4*>(e) = make_float4(0.5f * uv[0].x, 0.5f * uv[1].x, -0.5f * uv[0].y, -0.5f * uv[1].y);
-                *reinterpret_cast<float4*>(e + 4) = make_float4(0.5f * uv[2].x, 0.5f * uv[3].x, -0.5f * uv[2].y, -0.5f * uv[3].y);
-            } else {
-                *reinterpret_cast<float4*>(e) = make_float4(0.5f * uv[0].x, -0.5f * uv[0].y, 0.5f * uv[1].x, -0.5f * uv[1].y);
+        if (p.fused) {
+            if (np > 1)
+                #pragma unroll 1
+                for (int i = 4 * (int)tid; i < EF * s.k; i += 4 * kXf) cp_async16(ut + i, ug + i);
+            cp_async_wait_all();
+        } else {
+            // the prologue kernel's u: [head][M], unscaled
+            #pragma unroll 1
+            for (int i = tid; i < EF * s.k; i += kXf) {
+                const int n = i / EF, j = i & (EF - 1), im = (j / N) & 1, g = hperm<GH>((j / (2 * N)) * N + (j & (N - 1)));
+                ut[i] = g < ng ? (im ? -0.5f : 0.5f) * __ldcg(ws.u + ((size_t)b * s.Hq + g_first + g) * s.M + 2 * n + im) : 0.f;
             }
         }
         consumer_sync<kXf, kXfBar>();
@@ -1158,7 +1178,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     const uint32_t tile = wait_tile_u();
                     // tiles rotate over the warps
                     #pragma unroll 1
-                    for (int grp = (int)((unsigned)(wm + 4 * kMW) - (unsigned)(it & 3) * (kWinRowsPerTile / 16)) % kMW; grp * 16 < nt; grp += kMW) {
+                    for (int grp = (int)((unsigned)wm + c_par * (kWinRowsPerTile / 16)) % kMW; grp * 16 < nt; grp += kMW) {
                         if (STEP) {
                             // fused step: the new token's row is not in the cache yet
                             const int prow = new_buf == sg.buf[si] ? new_row - (sg.row[si] + r0) : -1;
@@ -1781,77 +1801,90 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         }
         return v;
     };
-    #pragma unroll 1
-    for (int i = tid; i < (cp ? 1 : GH) * s.d; i += kAll) {
-        const int sl = idiv(i, s.d), e = i - sl * s.d, g = hperm<GH>(sl);      // hperm is its own inverse
-        if (g < ng) {
-            float v = o_of(sl, e);
-            if (cp) v = e0 * v + e1 * o_of(1, e);
-            ws.o[(((size_t)b * s.Hq + g_first + g) * p.n_part + part) * s.d + e] = v;
+    auto l_of = [&](int sl) {                             // sum of p of a slot: the warps' sums in a fixed order
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < kAllW; ++w) v += red_s[w * GH + sl];
+        return v;
+    };
+    auto m_of = [&](int sl) {
+        float mv = m_run[0];
+#pragma unroll
+        for (int x = 1; x < GH; ++x) if (sl == x) mv = m_run[x];
+        return mv;
+    };
+    auto o_val = [&](int sl, int e) { const float v = o_of(sl, e); return cp ? e0 * v + e1 * o_of(1, e) : v; };
+    if (cp) {
+        #pragma unroll 1
+        for (int n = tid; n < s.k; n += kAll) {
+            float* e = z_s + n * EF;
+            e[0] = e0 * e[0] + e1 * e[2];
+            e[1] = e0 * e[1] + e1 * e[3];
         }
     }
-    #pragma unroll 1
-    for (int n = tid; n < s.k; n += kAll) {
-        const float* e = z_s + n * 2 * GH;
-#pragma unroll
-        for (int sl = 0; sl < GH; ++sl) {
-            const int g = hperm<GH>(sl), ab = sl / N, ln = sl - ab * N;
-            if (g < ng)
-                *reinterpret_cast<float2*>(ws.z + (((size_t)b * s.Hq + g_first + g) * p.n_part + part) * s.M + 2 * n) =
-                    cp ? make_float2(e0 * e[0] + e1 * e[2], e0 * e[1] + e1 * e[3]) : make_float2(e[(2 * ab) * N + ln], e[(2 * ab + 1) * N + ln]);
+    if (!p.fused) {
+        // for the epilogue kernel: per head and part
+        #pragma unroll 1
+        for (int i = tid; i < GH * s.d; i += kAll) {
+            const int sl = idiv(i, s.d), e = i - sl * s.d, g = hperm<GH>(sl);
+            if (g < ng) ws.o[(((size_t)b * s.Hq + g_first + g) * np + part) * s.d + e] = o_val(sl, e);
         }
-    }
-    if (tid < GH) {
-        const int g = hperm<GH>(tid);                     // slot tid holds head g
-        if (g < ng) {
-            float* ml = ws.ml + (((size_t)b * s.Hq + g_first + g) * p.n_part + part) * 2;
-            float mv = m_run[0];
-#pragma unroll
-            for (int sl = 1; sl < GH; ++sl) if (tid == sl) mv = m_run[sl];
-            auto l_of = [&](int sl) {                     // sum of p of a slot: the warps' sums in a fixed order
-                float v = 0.f;
-#pragma unroll
-                for (int w = 0; w < kAllW; ++w) v += red_s[w * GH + sl];
-                return v;
-            };
-            ml[0] = mv;
+        if (cp) all_sync();
+        #pragma unroll 1
+        for (int i = tid; i < EF * s.k; i += kAll) {
+            const int n = i / EF, j = i & (EF - 1), g = hperm<GH>((j / (2 * N)) * N + (j & (N - 1)));
+            if (g < ng) ws.z[(((size_t)b * s.Hq + g_first + g) * np + part) * s.M + 2 * n + ((j / N) & 1)] = z_s[i];
+        }
+        if (tid < GH && hperm<GH>(tid) < ng) {
+            float* ml = ws.ml + (((size_t)b * s.Hq + g_first + hperm<GH>(tid)) * np + part) * 2;
+            ml[0] = m_of(tid);
             ml[1] = cp ? e0 * l_of(0) + e1 * l_of(1) : l_of(tid);
         }
+        return;
+    }
+    float* og = ws.o + (size_t)job * np * (GH * s.d);
+    float* zg = ws.z + (size_t)job * nz * (EF * s.k);
+    float* mlg = ws.ml + (size_t)job * np * EF;
+    if (np > 1) {
+        if (cp) all_sync();
+        #pragma unroll 1
+        for (int i = tid; i < GH * s.d; i += kAll) {
+            const int sl = idiv(i, s.d);
+            og[part * GH * s.d + i] = o_val(sl, i - sl * s.d);
+        }
+        if (!is_win)
+            #pragma unroll 1
+            for (int i = tid; i < EF * s.k / 4; i += kAll)
+                reinterpret_cast<float4*>(zg + part * EF * s.k)[i] = reinterpret_cast<const float4*>(z_s)[i];
+        if (tid < GH) *reinterpret_cast<float2*>(mlg + (part * GH + tid) * 2) = make_float2(m_of(tid), cp ? e0 * l_of(0) + e1 * l_of(1) : l_of(tid));
     }
     TL(15);
-    if (!p.fused) return;
 
     // ------------------------------ merge (fused kernel) ------------------------------
-    // All parts of this (b, KV head, pass) have written their partial results.  Each part then
-    // merges a slice of the coefficient rows: its rows of every part's z against its rows of C^V.
-    // The last part to finish adds the slices and the parts' o in a fixed order, normalises and
-    // writes the output rows.  Everything a step needs from global memory is fetched with one batch
-    // of 16-byte asynchronous copies into the stage ring (every tile has been consumed), so each
-    // step costs one memory round trip.
-    const int np = p.n_part;
+    // All parts of this (b, KV head, pass) have written their partial results.  Each part then merges a slice of the
+    // coefficient rows (its rows of every part's z against its rows of C^V) and a slice of the outputs o.  The last part
+    // to finish adds the slices of o^c in a fixed order, normalises and writes the output rows.  Everything a step
+    // needs from global memory is fetched with one batch of 16-byte asynchronous copies into the stage ring (every
+    // tile has been consumed), so each step costs one memory round trip.  A part on its own works from its own
+    // shared memory.
     const int rows = m1 - m0;
-    const size_t qh0 = (size_t)b * s.Hq + g_first;
     const int nv = s.dcv >> 2, nrg = nv ? idiv(kAll, nv) : 0;
-    // rows of the slice handled at a time: what the stage ring holds of C^V rows, z slices and weighted z
-    constexpr int kRing = NS * kStageBytes / 4;
-    const int head_f = (2 * GH * np + GH + 3) & ~3;
-    const int mch = max(4, min((rows + 3) & ~3, idiv(kRing - head_f - nrg * GH * s.dcv, GH + s.dcv + GH * np) & ~3));
-    float* al_s = reinterpret_cast<float*>(stages);        // [GH][np] maxima, then exp2(m - max)
-    float* l_s = al_s + GH * np;                           // [GH][np]
-    float* linv_s = l_s + GH * np;                         // [GH]
-    float* zw_s = al_s + head_f;                           // [GH][mch]
-    float* big_s = zw_s + GH * mch;                        // step 1: C^V rows, z slices, partial sums; step 2: o and o^c parts
-    float* cv_s = big_s;                                   // [mch][dcv]
-    float* zs_s = cv_s + mch * s.dcv;                      // [GH][np][mch]
-    float* ps_s = zs_s + GH * np * mch;                    // [row groups][GH][dcv]
+    const MergePlan mp = merge_plan(NS * kStageBytes / 4, GH, np, nz, s.d, s.dcv, nrg, rows);
+    float* al_s = reinterpret_cast<float*>(stages);        // [np][GH] maxima, then exp2(m - max)
+    float* linv_s = al_s + EF * np;                        // [GH] (al_s holds (m, l) pairs)
+    float* zw_s = al_s + mp.head;                          // [mch / 2][EF] weighted z
+    float* cv_s = zw_s + GH * mp.mch;                      // [mch][dcv]
+    float* zs_s = cv_s + mp.mch * s.dcv;                   // [nz][mch / 2][EF]
+    float* op_s = zs_s + (np > 1 ? GH * nz * mp.mch : 0);  // [np][o_per]
+    float* ps_s = op_s + (np > 1 ? np * mp.o_per : 0);     // [row groups][GH][dcv]
     volatile int* last_s = fail + 1;
     float* cvg = s.dcv > 0 ? coef_rows(c.coef_v, s, b, h, s.dcv) + (size_t)m0 * s.dcv : nullptr;
     auto stage_cv = [&](int r0, int cr) {
 #pragma unroll 1
-        for (int i = tid; i < cr * nv; i += kAll) cp_async16(cv_s + 4 * i, cvg + (size_t)r0 * s.dcv + 4 * i);
+        for (int i = tid; i < cr * nv; i += kAll) cp_async16(cv_s + 4 * i, cvg + r0 * s.dcv + 4 * i);
     };
 
-    if (s.dcv > 0) stage_cv(0, min(rows, mch));            // under the barrier
+    if (s.dcv > 0) stage_cv(0, min(rows, mp.mch));         // under the barrier
     part_arrive<kAll>(bar + 1, np, tid);
     TL(16);
     part_wait<kAll>(bar + 1, np, tid, fail, c.status);
@@ -1874,67 +1907,86 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             *reinterpret_cast<uint4*>(dst + 8 * ch) = *reinterpret_cast<const uint4*>((side == 0 ? knew_bh : vnew_bh) + 8 * ch);
         }
     }
+    const int o0 = part * mp.o_per, o_n = max(0, min(mp.o_per, GH * s.d - o0));      // this part's slice of o
+    float* omg = ws.om + (size_t)job * (GH * s.d);
+    float* ocg = ws.oc + (size_t)job * np * (GH * s.dcv);
+    if (np > 1) {
 #pragma unroll 1
-    for (int i = tid; i < GH * np; i += kAll) {
-        float2 ml = make_float2(kNegBig, 0.f);
-        if (i < ng * np) ml = __ldcg(reinterpret_cast<const float2*>(ws.ml + (qh0 * np + i) * 2));
-        al_s[i] = ml.x;
-        l_s[i] = ml.y;
+        for (int i = tid; i < GH * np / 2; i += kAll) cp_async16(al_s + 4 * i, mlg + 4 * i);
+#pragma unroll 1
+        for (int i = tid; i < np * (o_n >> 2); i += kAll) {
+            const int sp = idiv(i, o_n >> 2), j = i - sp * (o_n >> 2);
+            cp_async16(op_s + sp * mp.o_per + 4 * j, og + sp * GH * s.d + o0 + 4 * j);
+        }
     }
     float4 acc4[GH];
 #pragma unroll
     for (int g = 0; g < GH; ++g) acc4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-    for (int r0 = 0; r0 < rows || r0 == 0; r0 += mch) {
-        const int cr = max(0, min(rows - r0, mch));
-        if (s.dcv > 0) {
-            if (r0 > 0) {
-                all_sync();                           // the previous chunk has been consumed
-                stage_cv(r0, cr);
-            }
-            const int r4 = cr >> 2;
+    for (int r0 = 0; r0 < rows || r0 == 0; r0 += mp.mch) {
+        const int cr = max(0, min(rows - r0, mp.mch)), ze = GH * cr;      // floats of a part's z in this chunk
+        if (r0 > 0) {
+            all_sync();                                   // the previous chunk has been consumed
+            stage_cv(r0, cr);
+        }
+        if (np > 1 && s.dcv > 0) {
 #pragma unroll 1
-            for (int i = tid; i < GH * np * r4; i += kAll) {
-                const int gs = idiv(i, r4), j = i - gs * r4;
-                if (gs < ng * np) cp_async16(zs_s + gs * mch + 4 * j, ws.z + (qh0 * np + gs) * s.M + m0 + r0 + 4 * j);
+            for (int i = tid; i < nz * (ze >> 2); i += kAll) {
+                const int sp = idiv(i, ze >> 2), j = i - sp * (ze >> 2);
+                cp_async16(zs_s + sp * GH * mp.mch + 4 * j, zg + sp * EF * s.k + (m0 + r0) * GH + 4 * j);
             }
         }
         cp_async_wait_all();
         all_sync();
         if (r0 == 0) {
-            if (warp < GH) {                               // one warp per head, lanes over the parts
-                float mx = kNegBig;
-#pragma unroll 1
-                for (int sp = lane; sp < np; sp += 32) mx = fmaxf(mx, al_s[warp * np + sp]);
-                mx = warp_max(mx);
-                float Lsum = 0.f;
-#pragma unroll 1
-                for (int sp = lane; sp < np; sp += 32) {
-                    const float a = ex2(al_s[warp * np + sp] - mx);
-                    al_s[warp * np + sp] = a;
-                    Lsum = fmaf(a, l_s[warp * np + sp], Lsum);
+            if (np == 1) {
+                if (tid < GH) {
+                    const float l = cp ? e0 * l_of(0) + e1 * l_of(1) : l_of(tid);
+                    linv_s[tid] = l > 0.f ? __fdividef(1.0f, l) : 0.f;
                 }
-                Lsum = warp_sum(Lsum);
-                if (lane == 0) linv_s[warp] = Lsum > 0.f ? __fdividef(1.0f, Lsum) : 0.f;
+            } else {
+                if (warp < GH) {                           // one warp per slot, lanes over the parts
+                    float mx = kNegBig;
+#pragma unroll 1
+                    for (int sp = lane; sp < np; sp += 32) mx = fmaxf(mx, al_s[(sp * GH + warp) * 2]);
+                    mx = warp_max_redux(mx);
+                    float Lsum = 0.f;
+#pragma unroll 1
+                    for (int sp = lane; sp < np; sp += 32) {
+                        const float2 ml = *reinterpret_cast<const float2*>(al_s + (sp * GH + warp) * 2);
+                        const float a = ex2(ml.x - mx);
+                        al_s[(sp * GH + warp) * 2] = a;
+                        Lsum = fmaf(a, ml.y, Lsum);
+                    }
+                    Lsum = warp_sum(Lsum);
+                    if (lane == 0) linv_s[warp] = Lsum > 0.f ? __fdividef(1.0f, Lsum) : 0.f;
+                }
+                all_sync();
+                if (tid < o_n) {
+                    const int sl = idiv(o0 + tid, s.d);
+                    float v = 0.f;
+#pragma unroll 2
+                    for (int sp = 0; sp < np; ++sp) v = fmaf(al_s[(sp * GH + sl) * 2], op_s[sp * mp.o_per + tid], v);
+                    omg[o0 + tid] = v;
+                }
             }
         }
-        all_sync();
         if (s.dcv > 0) {
 #pragma unroll 1
-            for (int t = tid; t < GH * cr; t += kAll) {
-                const int g = idiv(t, cr), r = t - g * cr;
+            for (int t = tid; t < ze; t += kAll) {
+                const int j = t & (EF - 1), sl = (j / (2 * N)) * N + (j & (N - 1)), im = (j / N) & 1;
                 float v = 0.f;
-                if (g < ng) {
-                    const float* z = zs_s + g * np * mch + r;
+                if (np == 1) {
+                    v = z_s[(m0 + r0) * GH + t];
+                } else {
 #pragma unroll 2
-                    for (int sp = 0; sp < np; ++sp) v = fmaf(al_s[g * np + sp], z[sp * mch], v);
-                    v *= w_row(m0 + r0 + r);
+                    for (int sp = 0; sp < nz; ++sp) v = fmaf(al_s[(sp * GH + sl) * 2], zs_s[sp * GH * mp.mch + t], v);
                 }
-                zw_s[g * mch + r] = v;
+                zw_s[t] = v * w_row(m0 + r0 + 2 * (t / EF) + im);
             }
             all_sync();
-            if (tid < nrg * nv) {
-                const int rgi = idiv(tid, nv), v = tid - rgi * nv;
+            const int rgi = idiv(tid, nv), v = tid - rgi * nv;
+            if (rgi < nrg) {
 #pragma unroll 1
                 for (int r = rgi; r < cr; r += nrg) {
                     float4 x = *reinterpret_cast<const float4*>(cv_s + r * s.dcv + 4 * v);
@@ -1944,11 +1996,12 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                         const float f = f_s[r0 + r];
                         const float4 y = *reinterpret_cast<const float4*>(xp_s + s.dck + 4 * v);
                         x.x = fmaf(f, y.x, x.x); x.y = fmaf(f, y.y, x.y); x.z = fmaf(f, y.z, x.z); x.w = fmaf(f, y.w, x.w);
-                        *reinterpret_cast<float4*>(cvg + (size_t)(r0 + r) * s.dcv + 4 * v) = x;
+                        *reinterpret_cast<float4*>(cvg + (r0 + r) * s.dcv + 4 * v) = x;
                     }
+                    const float* zr = zw_s + (r >> 1) * EF + (r & 1) * N;
 #pragma unroll
                     for (int g = 0; g < GH; ++g) {
-                        const float w = zw_s[g * mch + r];
+                        const float w = zr[(g / N) * 2 * N + (g & (N - 1))];
                         acc4[g].x = fmaf(w, x.x, acc4[g].x);
                         acc4[g].y = fmaf(w, x.y, acc4[g].y);
                         acc4[g].z = fmaf(w, x.z, acc4[g].z);
@@ -1958,72 +2011,55 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             }
         }
     }
+    // o^c of a slot's slice: the row groups in order; to the last part, or (a part on its own) to shared memory
+    float* oc_dst = np > 1 ? ocg + part * GH * s.dcv : zw_s;
     if (s.dcv > 0) {
-        if (tid < nrg * nv) {
-            const int rgi = idiv(tid, nv), v = tid - rgi * nv;
+        const int rgi = idiv(tid, nv), v = tid - rgi * nv;
+        if (rgi < nrg) {
 #pragma unroll
             for (int g = 0; g < GH; ++g) *reinterpret_cast<float4*>(ps_s + (rgi * GH + g) * s.dcv + 4 * v) = acc4[g];
         }
         all_sync();
 #pragma unroll 1
         for (int t = tid; t < GH * s.dcv; t += kAll) {
-            const int g = idiv(t, s.dcv), e = t - g * s.dcv;
-            float v = 0.f;
-#pragma unroll 1
-            for (int rgi = 0; rgi < nrg; ++rgi) v += ps_s[(rgi * GH + g) * s.dcv + e];
-            if (g < ng) ws.oc[((qh0 + g) * np + part) * s.dcv + e] = v;
+            float v2 = 0.f;
+#pragma unroll 2
+            for (int x = 0; x < nrg; ++x) v2 += ps_s[x * GH * s.dcv + t];
+            oc_dst[t] = v2;
         }
     }
     TL(18);
     // ticket: the last part to get here finishes the rows
     all_sync();
-    if (tid == 0) {
-        int old = 0;
-        if (np > 1) {
+    if (np > 1) {
+        if (tid == 0) {
+            int old = 0;
             __threadfence();
             asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(bar + 2) : "memory");
+            *last_s = old == np - 1;
         }
-        *last_s = old == np - 1;
-    }
-    all_sync();
-    TL(19);
-    if (!*last_s) { SPAN(2); return; }
-    float* op_s = zw_s;                                    // [GH][np][d] (the slice buffers are free again)
-    float* ocp_s = op_s + GH * np * s.d;                   // [GH][np][dcv]
-    int* inv_s = reinterpret_cast<int*>(ocp_s + GH * np * s.dcv);   // [d] dim -> slot in D^vc, or -1
-    {
-        const int nd4 = s.d >> 2;
+        all_sync();
+        TL(19);
+        if (!*last_s) { SPAN(2); return; }
 #pragma unroll 1
-        for (int i = tid; i < ng * np * nd4; i += kAll) cp_async16(op_s + 4 * i, ws.o + qh0 * np * s.d + 4 * i);
-#pragma unroll 1
-        for (int i = tid; i < ng * np * nv; i += kAll) cp_async16(ocp_s + 4 * i, ws.oc + qh0 * np * s.dcv + 4 * i);
+        for (int i = tid; i < np * GH * nv; i += kAll) cp_async16(zw_s + 4 * i, ocg + 4 * i);       // [np][GH][dcv]
+        cp_async_wait_all();
+        all_sync();
     }
 #pragma unroll 1
-    for (int e = tid; e < s.d; e += kAll) inv_s[e] = -1;
-    all_sync();
-    if (s.dcv > 0) {
-        const int32_t* idc_v = c.idx_comp_v + (size_t)h * s.dcv;
-#pragma unroll 1
-        for (int e = tid; e < s.dcv; e += kAll) inv_s[idc_v[e]] = e;
-    }
-    cp_async_wait_all();
-    all_sync();
-#pragma unroll 1
-    for (int t = tid; t < ng * s.d; t += kAll) {
-        const int g = idiv(t, s.d), e = t - g * s.d;
-        const float* o = op_s + g * np * s.d + e;
-        float v = 0.f;
-#pragma unroll 2
-        for (int sp = 0; sp < np; ++sp) v = fmaf(al_s[g * np + sp], o[sp * s.d], v);
-        const int slot = inv_s[e];
-        if (slot >= 0) {
-            const float* oc = ocp_s + g * np * s.dcv + slot;
+    for (int t = tid; t < GH * s.d; t += kAll) {
+        const int sl = idiv(t, s.d), e = t - sl * s.d, g = hperm<GH>(sl);
+        if (g >= ng) continue;
+        float v = np > 1 ? __ldcg(omg + t) : o_val(sl, e);
+        const int iv = inv_v[e];
+        if (iv < 0) {
+            const float* oc = zw_s + sl * s.dcv + (-1 - iv);
             float w = 0.f;
 #pragma unroll 2
-            for (int x = 0; x < np; ++x) w += oc[x * s.dcv];
+            for (int x = 0; x < np; ++x) w += oc[x * GH * s.dcv];
             v += w;
         }
-        out[(qh0 + g) * s.d + e] = __float2bfloat16_rn(v * linv_s[g]);
+        out[((size_t)b * s.Hq + g_first + g) * s.d + e] = __float2bfloat16_rn(v * linv_s[sl]);
     }
     TL(20);
     SPAN(3);
