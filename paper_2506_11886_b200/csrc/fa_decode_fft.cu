@@ -79,7 +79,7 @@ bool decode_fft_fused_fits(const Dims& s, int log2S, int gh, int nb, int n_part,
     const FftSmem L = fft_smem_layout(log2S, s.k, gh, nb, s.d, occ, split, class_pairs(s.G, gh, split));
     // at least eight rows of C^K per staged chunk (class pairs: the chunk may use the score and probability buffers too, as the kernel does)
     if (s.dck > 0 && (class_pairs(s.G, gh, split) ? (long long)((L.twf_off - L.fbuf_off) >> 2) : (long long)nb * L.fb_floats) < 8LL * s.dck) return false;
-    const int ring = ring_stages(occ, split) * kStageBytes / 4;
+    const int ring = (L.twf_off - L.stages_off) >> 2;
     const int nrg = s.dcv ? (split ? kSplitConsumers : kConsumers) / (s.dcv >> 2) : 0;
     const int rows = (s.M / 4 + n_part - 1) / n_part * 4 + 4;
     const MergePlan m = merge_plan(ring, gh, n_part, n_part, s.d, s.dcv, nrg, rows);

@@ -572,7 +572,7 @@ __host__ __device__ inline FftSmem fft_smem_layout(int log2S, int k, int GH, int
     return L;
 }
 
-// Shared memory of the merge in the stage ring (floats): head = the parts' (m, l) and the 1 / l; mch = coefficient rows
+// Shared memory of the merge in the stage ring and the buffers behind it (floats): head = the parts' (m, l) and the 1 / l; mch = coefficient rows
 // handled at a time (weighted z, rows of C^V, the parts' z); o_per = a part's slice of the outputs.
 struct MergePlan {
     int head, mch, o_per;
@@ -581,11 +581,11 @@ __host__ __device__ inline MergePlan merge_plan(int ring, int GH, int np, int nz
     MergePlan m;
     m.head = (2 * GH * np + GH + 3) & ~3;
     m.o_per = ((GH * d + np - 1) / np + 3) & ~3;
-    const int room = ring - m.head - nrg * GH * dcv - (np > 1 ? np * m.o_per : 0), per_row = GH + dcv + (np > 1 ? GH * nz : 0);
+    const int room = ring - m.head - (np > 1 ? np * m.o_per : 0), per_row = GH + dcv + (np > 1 ? GH * nz : 0);
     m.mch = (room / per_row) & ~3;
     const int all = (rows + 3) & ~3;
     if (m.mch > all) m.mch = all;
-    if (m.mch < 4) m.mch = 4;
+    if (m.mch < 4 || nrg * GH * dcv + GH * dcv > ring - m.head) m.mch = 4;      // (not enough room: the plan is refused)
     return m;
 }
 
@@ -619,6 +619,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     constexpr bool step = STEP;
     constexpr int N = GH / 2;
     constexpr int S = 1 << LS;
+    constexpr bool kSplitPairs = S / 2 < kConsumers;      // fewer pairs of bins than threads
     constexpr int NS = ring_stages(OCC, SPLIT ? 1 : 0);
     // Consumer threads: kAll of them; the warps that consume ring tiles (kept-dim and window products) are all of them,
     // or, in the split kernel, the last six, while the first eight (the transform group) run the compressed-dim phases
@@ -1349,9 +1350,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             // packed Hermitian spectra of the nb classes: X_m = V^A_m + i V^B_m per complex lane,
             // V_m = v_m + conj(v_{S-m}), v_n = (1/2) u~_n e^{i theta n c}.  Pair 0 is bins (0, S/2).
             if (s.dck > 0) {
-                // neighbouring lanes share a pair of bins and take half of the classes each (a batch of one
-                // class: one lane per pair, half as many rounds)
-                const bool split2 = nbt > 1;
+                // short transforms: neighbouring lanes share a pair of bins and take half of the classes each
+                const bool split2 = kSplitPairs && nbt > 1;
                 const int hcls = split2 ? (nbt + 1) >> 1 : nbt;
                 #pragma unroll 1
                 for (int item = tid; item < (split2 ? S : S / 2); item += kAll) {
@@ -1468,7 +1468,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 if constexpr (N == 2) { alA = pk(alpha[0], alpha[1]); alB = pk(alpha[2], alpha[3]); }
                 else { alA = PR<1>{alpha[0]}; alB = PR<1>{alpha[1]}; }
                 const PR<N> half = splat<N>(0.5f);
-                const bool split2 = nbt > 1;               // as for the spectra: one lane per pair when the batch is one transform
+                const bool split2 = kSplitPairs && nbt > 1;       // as for the spectra
                 const int hcls = split2 ? (nbt + 1) >> 1 : nbt;
                 #pragma unroll 1
                 for (int item = tid; item < (split2 ? S : S / 2); item += kAll) {       // split: whole warps (S is a multiple of 32)
@@ -1613,9 +1613,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             // packed Hermitian spectra of the nb classes: X_m = V^A_m + i V^B_m per complex lane,
             // V_m = v_m + conj(v_{S-m}), v_n = (1/2) u~_n e^{i theta n c}.  Pair 0 is bins (0, S/2).
             if (s.dck > 0) {
-                // neighbouring lanes share a pair of bins and take half of the classes each (a batch of one
-                // class: one lane per pair, half as many rounds)
-                const bool split2 = nb > 1;
+                // short transforms: neighbouring lanes share a pair of bins and take half of the classes each
+                const bool split2 = kSplitPairs && nb > 1;
                 const int hcls = split2 ? (nb + 1) >> 1 : nb;
                 #pragma unroll 1
                 for (int item = tid; item < (split2 ? S : S / 2); item += kConsumers) {
@@ -1686,7 +1685,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 if constexpr (N == 2) { alA = pk(alpha[0], alpha[1]); alB = pk(alpha[2], alpha[3]); }
                 else { alA = PR<1>{alpha[0]}; alB = PR<1>{alpha[1]}; }
                 const PR<N> half = splat<N>(0.5f);
-                const bool split2 = nb > 1;                // as for the spectra: one lane per pair when the batch is one class
+                const bool split2 = kSplitPairs && nb > 1;        // as for the spectra
                 const int hcls = split2 ? (nb + 1) >> 1 : nb;
                 #pragma unroll 1
                 for (int item = tid; item < (split2 ? S : S / 2); item += kConsumers) {       // split: whole warps (S is a multiple of 32)
@@ -1813,7 +1812,14 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         for (int x = 1; x < GH; ++x) if (sl == x) mv = m_run[x];
         return mv;
     };
-    auto o_val = [&](int sl, int e) { const float v = o_of(sl, e); return cp ? e0 * v + e1 * o_of(1, e) : v; };
+    // (in place; class pairs: slot 0 alone is left)
+    #pragma unroll 1
+    for (int i = tid; i < (cp ? 1 : GH) * s.d; i += kAll) {
+        const int sl = idiv(i, s.d), e = i - sl * s.d;
+        float v = o_of(sl, e);
+        if (cp) v = e0 * v + e1 * o_of(1, e);
+        o_s[i] = v;
+    }
     if (cp) {
         #pragma unroll 1
         for (int n = tid; n < s.k; n += kAll) {
@@ -1827,7 +1833,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         #pragma unroll 1
         for (int i = tid; i < GH * s.d; i += kAll) {
             const int sl = idiv(i, s.d), e = i - sl * s.d, g = hperm<GH>(sl);
-            if (g < ng) ws.o[(((size_t)b * s.Hq + g_first + g) * np + part) * s.d + e] = o_val(sl, e);
+            if (g < ng) ws.o[(((size_t)b * s.Hq + g_first + g) * np + part) * s.d + e] = o_s[i];
         }
         if (cp) all_sync();
         #pragma unroll 1
@@ -1848,10 +1854,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     if (np > 1) {
         if (cp) all_sync();
         #pragma unroll 1
-        for (int i = tid; i < GH * s.d; i += kAll) {
-            const int sl = idiv(i, s.d);
-            og[part * GH * s.d + i] = o_val(sl, i - sl * s.d);
-        }
+        for (int i = tid; i < GH * s.d; i += kAll) og[part * GH * s.d + i] = o_s[i];      // (each thread the values it wrote)
         if (!is_win)
             #pragma unroll 1
             for (int i = tid; i < EF * s.k / 4; i += kAll)
@@ -1864,19 +1867,20 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     // All parts of this (b, KV head, pass) have written their partial results.  Each part then merges a slice of the
     // coefficient rows (its rows of every part's z against its rows of C^V) and a slice of the outputs o.  The last part
     // to finish adds the slices of o^c in a fixed order, normalises and writes the output rows.  Everything a step
-    // needs from global memory is fetched with one batch of 16-byte asynchronous copies into the stage ring (every
-    // tile has been consumed), so each step costs one memory round trip.  A part on its own works from its own
+    // needs from global memory is fetched with one batch of 16-byte asynchronous copies into the stage ring and the
+    // transform buffers (all idle), so each step costs one memory round trip.  A part on its own works from its own
     // shared memory.
     const int rows = m1 - m0;
     const int nv = s.dcv >> 2, nrg = nv ? idiv(kAll, nv) : 0;
-    const MergePlan mp = merge_plan(NS * kStageBytes / 4, GH, np, nz, s.d, s.dcv, nrg, rows);
+    const MergePlan mp = merge_plan((L.twf_off - L.stages_off) >> 2, GH, np, nz, s.d, s.dcv, nrg, rows);
     float* al_s = reinterpret_cast<float*>(stages);        // [np][GH] maxima, then exp2(m - max)
     float* linv_s = al_s + EF * np;                        // [GH] (al_s holds (m, l) pairs)
     float* zw_s = al_s + mp.head;                          // [mch / 2][EF] weighted z
     float* cv_s = zw_s + GH * mp.mch;                      // [mch][dcv]
     float* zs_s = cv_s + mp.mch * s.dcv;                   // [nz][mch / 2][EF]
     float* op_s = zs_s + (np > 1 ? GH * nz * mp.mch : 0);  // [np][o_per]
-    float* ps_s = op_s + (np > 1 ? np * mp.o_per : 0);     // [row groups][GH][dcv]
+    float* ps_s = zw_s;                                    // [row groups][GH][dcv], when the rows are done
+    float* oc_s = ps_s + nrg * GH * s.dcv;                 // a part on its own: its o^c
     volatile int* last_s = fail + 1;
     float* cvg = s.dcv > 0 ? coef_rows(c.coef_v, s, b, h, s.dcv) + (size_t)m0 * s.dcv : nullptr;
     auto stage_cv = [&](int r0, int cr) {
@@ -1884,6 +1888,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         for (int i = tid; i < cr * nv; i += kAll) cp_async16(cv_s + 4 * i, cvg + r0 * s.dcv + 4 * i);
     };
 
+    all_sync();                                            // the fragments in the transform buffers have been read
     if (s.dcv > 0) stage_cv(0, min(rows, mp.mch));         // under the barrier
     part_arrive<kAll>(bar + 1, np, tid);
     TL(16);
@@ -2012,8 +2017,9 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         }
     }
     // o^c of a slot's slice: the row groups in order; to the last part, or (a part on its own) to shared memory
-    float* oc_dst = np > 1 ? ocg + part * GH * s.dcv : zw_s;
+    float* oc_dst = np > 1 ? ocg + part * GH * s.dcv : oc_s;
     if (s.dcv > 0) {
+        all_sync();                                       // the chunk has been consumed
         const int rgi = idiv(tid, nv), v = tid - rgi * nv;
         if (rgi < nrg) {
 #pragma unroll
@@ -2050,10 +2056,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     for (int t = tid; t < GH * s.d; t += kAll) {
         const int sl = idiv(t, s.d), e = t - sl * s.d, g = hperm<GH>(sl);
         if (g >= ng) continue;
-        float v = np > 1 ? __ldcg(omg + t) : o_val(sl, e);
+        float v = np > 1 ? __ldcg(omg + t) : o_s[t];
         const int iv = inv_v[e];
         if (iv < 0) {
-            const float* oc = zw_s + sl * s.dcv + (-1 - iv);
+            const float* oc = (np > 1 ? zw_s : oc_s) + sl * s.dcv + (-1 - iv);
             float w = 0.f;
 #pragma unroll 2
             for (int x = 0; x < np; ++x) w += oc[x * GH * s.dcv];
