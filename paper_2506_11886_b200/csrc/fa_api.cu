@@ -161,10 +161,11 @@ fa_status plan_decode(const fa_layout& l, DecodePlan* p) {
         p->n_wsplit = 0;
         p->occ = 1;
         p->split = 0;
-        // Short transforms leave room for two CTAs on an SM (a shorter ring, a register cap): one CTA's
-        // dependent phases hide behind the other's, and a head gets twice the CTAs (or, with more heads
-        // than SMs, the waves are twice as wide).  Tried first; one CTA per SM otherwise.
-        for (int occ = log2S <= 8 ? 2 : 1; occ >= 1 && !p->fused && l.decode_algo != FA_DECODE_FFT_SPLIT; --occ) {
+        // Short transforms leave room for two CTAs on an SM (a shorter ring, a register cap under which the instances with
+        // four heads spill).  That pays with more heads than SMs, whose waves are then twice as wide; with fewer, twice
+        // as many parts to a head cost more in exchanges than they save (2 K-token chat at batch 1 / 8: 30.0 / 58.7 us a
+        // step with two, 25.9 / 55.0 with one; MHA 4 K at batch 4: 81.8 / 71.4).
+        for (int occ = log2S <= 8 && jobs > kNumSms ? 2 : 1; occ >= 1 && !p->fused && l.decode_algo != FA_DECODE_FFT_SPLIT; --occ) {
             const size_t smem_limit = occ == 2 ? 113 * 1024 : 227 * 1024;
             const int slots = kNumSms * occ;
             const int per_job = jobs < slots ? slots / jobs : 1;
@@ -677,7 +678,17 @@ fa_status fa_decode_attention(const fa_layout* layout, const fa_cache* cache, co
 
 }  // extern "C"
 
-constexpr int kStepFusedMinParts = 8;
+// Whether the step of this plan is one launch.  With the push inside, the coefficients cross the bus once for reading and
+// the append kernel's launch falls away; against that stands that a part updates its rows one after the other, where
+// the append kernel spreads them over the whole device.  Measured at 256 rows to a part (32 K tokens, batch 4, and MHA
+// at batch 4): 1.8 and 3.6 us faster in one launch; at 512 rows (32 K, batch 8) 5.6 us slower.  The split build's tile
+// group takes no part in the update: eight parts or more there.
+static bool step_in_one_launch(const fa_layout& l, const DecodePlan& p) {
+    if (!p.fused || p.n_pass != 1) return false;
+    if (p.n_part >= 8) return true;
+    const int rows = (l.n_coef / 4 + p.n_part - 1) / p.n_part * 4;
+    return !p.split && rows <= 260 && (p.n_part >= 2 || l.batch * l.n_kv_heads <= sm_count());
+}
 
 // fa_decode_step.  Where the decode call is the fused kernel with one pass and many parts per head, the push
 // rides on that launch; otherwise the two calls are made one after the other.
@@ -699,7 +710,7 @@ static fa_status decode_step_impl(const fa_layout* layout, fa_cache* cache, cons
     // stand-alone append kernel, which spreads the coefficient update over the whole device, is faster
     // (measured: batch 8 MHA 22 us against 35 us inside the decode kernel, batch 4 at 128K 22 against 64).
     // Whether the device can hold all parts at once is asked before anything is enqueued: nothing to undo.
-    if (p.fused && p.n_pass == 1 && p.n_part >= kStepFusedMinParts && cooperative_launch_supported() && decode_fft_launchable(s, p)) {
+    if (step_in_one_launch(*layout, p) && cooperative_launch_supported() && decode_fft_launchable(s, p)) {
         const cudaError_t err = launch_decode_fft(s, make_cache(*cache), layout->kv_dtype, p, q, out, static_cast<char*>(ws), k_new, v_new,
                                                   static_cast<cudaStream_t>(stream));
         if (err == cudaSuccess) return FA_OK;
@@ -818,7 +829,7 @@ int fa_launch_count(const fa_layout* layout, int what) {
         case 3: {           // fa_decode_step: the fused decode kernel alone, or fa_append + fa_decode_attention
             DecodePlan p;
             if (plan_decode(*layout, &p) != FA_OK) return 0;
-            return (p.fused && p.n_pass == 1 && p.n_part >= kStepFusedMinParts) ? 1 : 1 + (p.fused ? 1 : 3);
+            return step_in_one_launch(*layout, p) ? 1 : 1 + (p.fused ? 1 : 3);
         }
         case 4: {           // plan query: the split build of the fused decode kernel
             DecodePlan p;
