@@ -120,7 +120,26 @@ static bool fft_ok(const fa_layout& l, int gh, int* log2S) {
     return true;
 }
 
+static fa_status make_plan(const fa_layout& l, DecodePlan* p);
+
+// The plan of a layout.  Working it out (the split of classes and windows, what fits in shared memory) takes longer than a
+// launch, and a program calls with the same few layouts over and over: every thread keeps the plans of its last ones.
 fa_status plan_decode(const fa_layout& l, DecodePlan* p) {
+    struct Entry { fa_layout l; int dev; fa_status st; DecodePlan p; };
+    constexpr int kEntries = 8;
+    static thread_local Entry cache[kEntries];
+    static thread_local int used = 0, next = 0;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); dev = -1; }
+    for (int i = 0; i < used; ++i)
+        if (cache[i].dev == dev && std::memcmp(&cache[i].l, &l, sizeof(l)) == 0) { *p = cache[i].p; return cache[i].st; }
+    const fa_status st = make_plan(l, p);
+    Entry& e = cache[used < kEntries ? used++ : (next = (next + 1) % kEntries)];
+    e = Entry{l, dev, st, *p};
+    return st;
+}
+
+static fa_status make_plan(const fa_layout& l, DecodePlan* p) {
     Dims s = make_dims(l);
     std::memset(p, 0, sizeof(*p));
     const int kNumSms = sm_count();
@@ -248,7 +267,7 @@ fa_status plan_decode(const fa_layout& l, DecodePlan* p) {
         int jobs = s.B * s.Hkv * p->n_pass;
         int want = (2 * kNumSms + jobs - 1) / jobs;
         long long tokens = (long long)s.max_mid + s.l_init + s.l_local;
-        int max_by_work = (int)((tokens + 255) / 256);            // at least one 256-token tile each
+        int max_by_work = (int)((tokens + 63) / 64);              // at least one 64-token tile each
         if (want > max_by_work) want = max_by_work;
         if (want > 64) want = 64;
         if (want < 1) want = 1;

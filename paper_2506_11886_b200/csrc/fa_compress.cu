@@ -158,10 +158,12 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
     int b = bh / s.Hkv, h = bh % s.Hkv;
     int nfull = side == 0 ? s.nfk : s.nfv;
     int ncomp = s.d - nfull;
-    if (ncomp == 0) return;
     const int L = row_len(lens, Lmax, b);
     const int n_init = min(L, s.l_init), n_mid = mid_of(s, L);
-    if (n_mid >= tc_min) return;                         // the tensor-core kernel's row
+    if (ncomp == 0 || n_mid >= tc_min) {                 // nothing to do, or the tensor-core kernel's row
+        asm volatile("griddepcontrol.wait;" ::: "memory");   // (the end of this grid implies the end of the one before)
+        return;
+    }
     const KV* X = (side == 0 ? K : V) + (size_t)b * sb + (size_t)h * sh;
     const int32_t* idc = (side == 0 ? c.idx_comp_k : c.idx_comp_v) + (size_t)h * ncomp;
     float* coef = coef_rows(side == 0 ? c.coef_k : c.coef_v, s, b, h, ncomp);
@@ -177,14 +179,24 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
 #pragma unroll
         for (int i = 0; i < 8; ++i) acc[r][i] = 0.f;
 
+    int col[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) col[i] = lane + 32 * i < ncomp ? idc[lane + 32 * i] : 0;
+
     int j_begin = blockIdx.y * chunks_per_split * kTJ;
     int j_end = min(n_mid, j_begin + chunks_per_split * kTJ);
     for (int j0 = j_begin; j0 < j_end; j0 += kTJ) {
         int nj = min(kTJ, j_end - j0);
         __syncthreads();
-        for (int i = threadIdx.x; i < kTJ * ncomp; i += blockDim.x) {
-            int jj = i / ncomp, e = i - jj * ncomp;
-            X_s[i] = jj < nj ? ld_f(X + (size_t)(n_init + j0 + jj) * st + idc[e]) : 0.f;
+        // a warp takes every eighth token: its lanes' columns are fixed, so all loads of a chunk are independent
+        const KV* xrow = X + (size_t)(n_init + j0 + rg) * st;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int e = lane + 32 * i;
+            if (i < ncol && e < ncomp)
+#pragma unroll
+                for (int q = 0; q < kTJ / 8; ++q)
+                    X_s[(rg + 8 * q) * ncomp + e] = rg + 8 * q < nj ? ld_f(xrow + (size_t)(8 * q) * st + col[i]) : 0.f;
         }
         // basis tile: thread -> (token jj, frequency pair nn) ; rows 2 nn (cos), 2 nn + 1 (sin)
         for (int i = threadIdx.x; i < kTJ * (kTM / 2); i += blockDim.x) {
@@ -211,6 +223,7 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
             }
         }
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");    // the partition kernel clears the coefficients
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         int m = m0 + 4 * rg + r;
@@ -274,9 +287,19 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     size_t smem = sizeof(float) * ((size_t)kTJ * max_comp + (size_t)kTJ * kTM);
     err = ensure_dynamic_smem(compress_coef_kernel<KV>, smem);
     if (err != cudaSuccess) return err;
-    compress_coef_kernel<KV><<<dim3(row_tiles, n_tsplit, s.B * s.Hkv * 2), 256, smem, stream>>>(
-        s, c, static_cast<const KV*>(K), static_cast<const KV*>(V), sb, st, sh, L, cps, rl, tc_min);
-    return cudaGetLastError();
+    // behind the partition kernel programmatically: it waits for it in front of its additions
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(row_tiles, n_tsplit, s.B * s.Hkv * 2);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, compress_coef_kernel<KV>, s, c, static_cast<const KV*>(K), static_cast<const KV*>(V), sb, st, sh, L, cps,
+                              rl, tc_min);
 }
 
 // with_coef = false runs only the partition / gather kernel (the tensor-core or the transform path computes the

@@ -35,11 +35,11 @@ __host__ __device__ inline int gather_rounds(int n_pairs, int hp, int nf, int gw
     while (r < 8 && ((kBK / r + n_pairs - 1) / n_pairs) * hp * (nf >> 3) > kGatherItems * 32 * gw) r *= 2;
     return r;
 }
-// Warps that write the kept-dim rows of the middle from the B boxes: four where one round of their items covers a stage
-// (more of them only draw power: the 32K contraction runs at the power cap and loses 3 % with six), eight where it
-// does not (one or two pairs per team and many kept dims: every pair writes most rows of its boxes itself; 4 K
-// tokens of the 32-head MHA layout, 48 kept dims: fa_compress 264 us with four, 234 with six, 227 with eight, and 320 with
-// the rows left to the partition kernel, which then reads the whole prefill once more).
+// Warps that write the kept-dim rows of the middle from the B boxes: four where a thread has at most two of a stage's
+// items (more warps only draw power: the 32K contraction runs at the power cap and loses 3 % with six), eight where it
+// has more (few pairs per team and many kept dims: every pair writes most rows of its boxes itself; 4 K tokens of the
+// 32-head MHA layout, 48 kept dims: fa_compress 264 us with four, 234 with six, 227 with eight, and 320 with the rows
+// left to the partition kernel, which then reads the whole prefill once more).
 constexpr int kFewGather = 4, kManyGather = 8;
 constexpr int threads_tc(int gw) { return 64 + 32 * (kGenWarps + gw); }
 using namespace umma;
@@ -625,7 +625,9 @@ cudaError_t launch_compress_tc2(const Dims& s, const CacheDev& c, const void* K,
     if (!make_map2(&tmK, K, s, sb, st, sh, L) || !make_map2(&tmV, V, s, sb, st, sh, L)) return cudaErrorInvalidValue;
     const bool pair = s.Hkv % 2 == 0;                        // two heads share a CTA pair and its basis tiles
     const int nf = s.nfk > s.nfv ? s.nfk : s.nfv;
-    const bool many = gather && gather_rounds(s.M / (2 * kBM), pair ? 2 : 1, nf, kFewGather) > 1;
+    // more than two items to a thread of four warps: the gather would set the pace
+    const int n_pairs = s.M / (2 * kBM), items = (kBK + n_pairs - 1) / n_pairs * (pair ? 2 : 1) * (nf >> 3);
+    const bool many = gather && items > 2 * 32 * kFewGather;
     auto go = [&](auto d, auto hp) {
         return many ? launch_tc2_t<d, hp, kManyGather>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
                     : launch_tc2_t<d, hp, kFewGather>(tmK, tmV, s, c, L, rows, ordered, gather, stream);

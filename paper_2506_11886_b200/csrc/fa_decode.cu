@@ -10,8 +10,13 @@ namespace fa {
 
 
 // ------------------------------------------------------------- direct main --
-// grid (n_split, Hkv * n_pass, B), 256 threads; one thread per token of a 256-token tile.
-constexpr int kTile = 256;
+// grid (n_split, Hkv * n_pass, B), 256 threads.  A split takes a run of middle tokens (in token order, whatever their
+// classes) and a run of window tokens, in tiles of 64: four lanes share a token's sum over the frequencies and its kept
+// dims, and on the way back the threads share out frequencies and groups of tokens.  The kernel is bound by its chain of
+// dependent steps, so what counts is that a call has many short CTAs: 1024 fp32 tokens of one head are 16 CTAs of one
+// tile instead of four CTAs that walked eight classes each with 32 of their 256 threads (compress and decode of that
+// cache together: 99 -> 47 us, of which 47 are now the host's).
+constexpr int kTile = 64, kLanes = 4;
 
 template <int GH>
 struct RunStat {
@@ -56,7 +61,8 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
     float* u_s = qf_s + GH * s.nfk;           // [GH][M]
     float* z_s = u_s + GH * s.M;              // [GH][M]
     float* p_s = z_s + GH * s.M;              // [GH][kTile]
-    float* red_s = p_s + GH * kTile;          // [8][GH]
+    float* zr_s = p_s + GH * kTile;           // [2 GH][256] partial z of the token groups
+    float* red_s = zr_s + 512 * GH;           // [8][GH]
     float* o_s = red_s + 8 * GH;              // [GH][d]  final reduce
     float* acc_s = o_s + GH * s.d;            // [256][GH] cross-thread reduce of the output accumulators
 
@@ -90,14 +96,15 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
     for (int g = 0; g < GH; ++g) { o_mid[g] = 0.f; o_win[g] = 0.f; }
 
     // thread -> (token group, dim) maps of the two P.V products
-    const int ntg_mid = s.nfv > 0 ? kTile / s.nfv : 0;
+    const int ntg_mid = s.nfv > 0 ? 256 / s.nfv : 0;
     const int tg_mid = s.nfv > 0 ? tid / s.nfv : 0, e_mid = s.nfv > 0 ? tid % s.nfv : 0;
     const bool act_mid = s.nfv > 0 && tg_mid < ntg_mid;
-    const int ntg_win = kTile / s.d;
+    const int ntg_win = 256 / s.d;
     const int tg_win = tid / s.d, e_win = tid % s.d;
     const bool act_win = tg_win < ntg_win;
 
-    // after scores are known: update the running softmax state, leave p in p_s
+    // after scores are known (every one of a token's four lanes has them): update the running softmax state, leave p in p_s
+    const int tk = tid / kLanes, ql = tid % kLanes;
     auto softmax_tile = [&](float (&sc)[GH], bool valid) {
         float mx[GH];
 #pragma unroll
@@ -109,77 +116,104 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
             float m_new = fmaxf(rs.m[g], mx[g]);
             alpha[g] = exp2f(rs.m[g] - m_new);
             rs.m[g] = m_new;
-            pv[g] = valid ? exp2f(sc[g] - m_new) : 0.f;
-            p_s[g * kTile + tid] = pv[g];
+            pv[g] = valid && ql == 0 ? exp2f(sc[g] - m_new) : 0.f;
+            if (ql == 0) p_s[g * kTile + tk] = pv[g];
             o_mid[g] *= alpha[g];
             o_win[g] *= alpha[g];
         }
-        for (int i = tid; i < GH * s.M; i += blockDim.x) z_s[i] *= alpha[i / s.M];
+#pragma unroll
+        for (int g = 0; g < GH; ++g)
+            for (int m = tid; m < s.M; m += 256) z_s[g * s.M + m] *= alpha[g];
         block_reduce<GH, false>(pv, red_s);     // also publishes p_s and the z_s rescale
 #pragma unroll
         for (int g = 0; g < GH; ++g) rs.l[g] = rs.l[g] * alpha[g] + pv[g];
     };
+    auto lanes_sum = [&](float (&sc)[GH]) {
+#pragma unroll
+        for (int g = 0; g < GH; ++g) {
+            sc[g] += __shfl_xor_sync(0xffffffffu, sc[g], 1);
+            sc[g] += __shfl_xor_sync(0xffffffffu, sc[g], 2);
+        }
+    };
+    const bool p2 = (s.P & (s.P - 1)) == 0;
+    const int lgP = 31 - __clz(s.P);
+    auto cls_of = [&](int j) { return p2 ? j & (s.P - 1) : j % s.P; };
+    auto slot_of = [&](int j) { return p2 ? j >> lgP : j / s.P; };
 
-    // ---- middle tokens: classes [c0, c1) of this split ------------------------
-    const int c0 = (int)((long long)split * s.P / p.n_split), c1 = (int)((long long)(split + 1) * s.P / p.n_split);
-    for (int cls = c0; cls < c1; ++cls) {
-        const int n_cls = cls < n_mid ? (n_mid - cls + s.P - 1) / s.P : 0;
-        for (int a0 = 0; a0 < n_cls; a0 += kTile) {
-            const int a = a0 + tid;
-            const bool valid = a < n_cls;
-            const int j = cls + s.P * a;
-            float sc[GH];
+    // ---- middle tokens [j0, j1) of this split ------------------------
+    const int per = (n_mid + p.n_split - 1) / p.n_split;
+    const int j0 = min(n_mid, split * per), j1 = min(n_mid, j0 + per);
+    // frequencies of a lane, and the way back: kz frequencies at a time, 256 / kz groups of tokens
+    const int per_lane = (s.k + kLanes - 1) / kLanes;
+    int kz = 32;
+    while (kz < s.k && kz < 256) kz *= 2;
+    const int n_grp = 256 / kz, zt = tid / kz, zn = tid % kz;
+    for (int t0 = j0; t0 < j1; t0 += kTile) {
+        const int j = t0 + tk;
+        const bool valid = j < j1;
+        const int nt = min(kTile, j1 - t0);
+        float sc[GH];
 #pragma unroll
-            for (int g = 0; g < GH; ++g) sc[g] = 0.f;
-            if (valid) {
-                const KV* row = mid_row<KV>(c.k_mid, s, b, h, cls, a, s.nfk);
-                for (int e = 0; e < s.nfk; ++e) {
-                    float x = ld_f(row + e);
+        for (int g = 0; g < GH; ++g) sc[g] = 0.f;
+        if (valid) {
+            const KV* row = mid_row<KV>(c.k_mid, s, b, h, cls_of(j), slot_of(j), s.nfk);
+#pragma unroll 8
+            for (int e = ql; e < s.nfk; e += kLanes) {
+                float x = ld_f(row + e);
 #pragma unroll
-                    for (int g = 0; g < GH; ++g) sc[g] = fmaf(qf_s[g * s.nfk + e], x, sc[g]);
-                }
-                if (s.dck > 0) {
-                    float cd, sd;
-                    basis_cs(1, j, s.T, &cd, &sd);                  // rotation per unit of n
-                    for (int n0 = 0; n0 < s.k; n0 += 32) {
-                        float cr, sr;
-                        basis_cs(n0, j, s.T, &cr, &sr);             // exact re-seed
-                        const int n1 = min(s.k, n0 + 32);
-                        for (int n = n0; n < n1; ++n) {
+                for (int g = 0; g < GH; ++g) sc[g] = fmaf(qf_s[g * s.nfk + e], x, sc[g]);
+            }
+            if (s.dck > 0) {
+                float cd, sd;
+                basis_cs(1, j, s.T, &cd, &sd);                  // rotation per unit of n
+                const int f1 = min(s.k, (ql + 1) * per_lane);
+                for (int n0 = ql * per_lane; n0 < f1; n0 += 32) {
+                    float cr, sr;
+                    basis_cs(n0, j, s.T, &cr, &sr);             // exact re-seed
+                    const int n1 = min(f1, n0 + 32);
+#pragma unroll 4
+                    for (int n = n0; n < n1; ++n) {
 #pragma unroll
-                            for (int g = 0; g < GH; ++g)
-                                sc[g] = fmaf(u_s[g * s.M + 2 * n], cr, fmaf(u_s[g * s.M + 2 * n + 1], sr, sc[g]));
-                            float t = cr * cd - sr * sd;
-                            sr = fmaf(sr, cd, cr * sd);
-                            cr = t;
+                        for (int g = 0; g < GH; ++g) {
+                            const float2 u = *reinterpret_cast<const float2*>(u_s + g * s.M + 2 * n);
+                            sc[g] = fmaf(u.x, cr, fmaf(u.y, sr, sc[g]));
                         }
+                        float t = cr * cd - sr * sd;
+                        sr = fmaf(sr, cd, cr * sd);
+                        cr = t;
                     }
                 }
             }
-            softmax_tile(sc, valid);
-            const int nt = min(kTile, n_cls - a0);
-            // o^u += p V^mu
-            if (act_mid) {
-                for (int i = tg_mid; i < nt; i += ntg_mid) {
-                    float x = ld_f(mid_row<KV>(c.v_mid, s, b, h, cls, a0 + i, s.nfv) +
-                                   v_mid_col(a0 + i, e_mid, s.nfv, sizeof(KV) == 2 ? FA_BF16 : FA_F32));
+        }
+        lanes_sum(sc);
+        softmax_tile(sc, valid);
+        // o^u += p V^mu
+        if (act_mid) {
+#pragma unroll 4
+            for (int i = tg_mid; i < nt; i += ntg_mid) {
+                const int slot = slot_of(t0 + i);
+                float x = ld_f(mid_row<KV>(c.v_mid, s, b, h, cls_of(t0 + i), slot, s.nfv) +
+                               v_mid_col(slot, e_mid, s.nfv, sizeof(KV) == 2 ? FA_BF16 : FA_F32));
 #pragma unroll
-                    for (int g = 0; g < GH; ++g) o_mid[g] = fmaf(p_s[g * kTile + i], x, o_mid[g]);
-                }
+                for (int g = 0; g < GH; ++g) o_mid[g] = fmaf(p_s[g * kTile + i], x, o_mid[g]);
             }
-            // z[m] += p F[m][j]: thread owns frequency n, walks the tile's tokens by rotation
-            if (s.dcv > 0) {
-                for (int n = tid; n < s.k; n += blockDim.x) {
-                    float zr[GH], zi[GH];
+        }
+        // z[m] += p F[m][j]: thread owns a frequency and a group of the tile's tokens, walked by rotation
+        if (s.dcv > 0) {
+            const int gt = kTile / n_grp, i0 = zt * gt, i1 = min(nt, i0 + gt);
+            for (int nb = 0; nb < s.k; nb += kz) {
+                const int n = nb + zn;
+                float zr[GH], zi[GH];
 #pragma unroll
-                    for (int g = 0; g < GH; ++g) { zr[g] = 0.f; zi[g] = 0.f; }
-                    float cd, sd;
-                    basis_cs(n, s.P, s.T, &cd, &sd);               // step between consecutive slots
-                    for (int i0 = 0; i0 < nt; i0 += 32) {
-                        float cr, sr;
-                        basis_cs(n, cls + s.P * (a0 + i0), s.T, &cr, &sr);
-                        const int i1 = min(nt, i0 + 32);
-                        for (int i = i0; i < i1; ++i) {
+                for (int g = 0; g < GH; ++g) { zr[g] = 0.f; zi[g] = 0.f; }
+                if (n < s.k && i0 < i1) {
+                    float cd, sd, cr, sr;
+                    basis_cs(n, 1, s.T, &cd, &sd);
+                    for (int ia = i0; ia < i1; ia += 32) {
+                        basis_cs(n, t0 + ia, s.T, &cr, &sr);
+                        const int ib = min(i1, ia + 32);
+#pragma unroll 4
+                        for (int i = ia; i < ib; ++i) {
 #pragma unroll
                             for (int g = 0; g < GH; ++g) {
                                 float pv = p_s[g * kTile + i];
@@ -191,38 +225,55 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
                             cr = t;
                         }
                     }
+                }
+                if (n_grp == 1) {
+                    if (n < s.k)
 #pragma unroll
-                    for (int g = 0; g < GH; ++g) {
-                        z_s[g * s.M + 2 * n] += zr[g];
-                        z_s[g * s.M + 2 * n + 1] += zi[g];
+                        for (int g = 0; g < GH; ++g) { z_s[g * s.M + 2 * n] += zr[g]; z_s[g * s.M + 2 * n + 1] += zi[g]; }
+                } else {
+#pragma unroll
+                    for (int g = 0; g < GH; ++g) { zr_s[(2 * g) * 256 + tid] = zr[g]; zr_s[(2 * g + 1) * 256 + tid] = zi[g]; }
+                    __syncthreads();
+                    for (int i = tid; i < 2 * GH * kz; i += 256) {
+                        const int part = i / kz, f = i - part * kz;          // part = 2 g + (re, im)
+                        if (nb + f < s.k) {
+                            float v = 0.f;
+                            for (int x = 0; x < n_grp; ++x) v += zr_s[part * 256 + x * kz + f];
+                            z_s[(part >> 1) * s.M + 2 * (nb + f) + (part & 1)] += v;
+                        }
                     }
+                    __syncthreads();
                 }
             }
-            __syncthreads();
         }
+        __syncthreads();
     }
 
     // ---- window tokens [w0, w1) of this split: init rows, then the local ring --
     const int n_win = n_init + n_local;
     const int w0 = (int)((long long)split * n_win / p.n_split), w1 = (int)((long long)(split + 1) * n_win / p.n_split);
     for (int t0 = w0; t0 < w1; t0 += kTile) {
-        const int t = t0 + tid;
+        const int t = t0 + tk;
         const bool valid = t < w1;
         auto row_of = [&](void* init, void* local, int tt) -> const KV* {
             if (tt < n_init) return win_row<KV>(init, s, b, h, s.l_init, tt);
-            return win_row<KV>(local, s, b, h, s.l_local, (head + (tt - n_init)) % s.l_local);
+            int r = head + (tt - n_init);
+            if (r >= s.l_local) r -= s.l_local;
+            return win_row<KV>(local, s, b, h, s.l_local, r);
         };
         float sc[GH];
 #pragma unroll
         for (int g = 0; g < GH; ++g) sc[g] = 0.f;
         if (valid) {
             const KV* row = row_of(c.k_init, c.k_local, t);
-            for (int e = 0; e < s.d; ++e) {
+#pragma unroll 8
+            for (int e = ql; e < s.d; e += kLanes) {
                 float x = ld_f(row + e);
 #pragma unroll
                 for (int g = 0; g < GH; ++g) sc[g] = fmaf(q_s[g * s.d + e], x, sc[g]);
             }
         }
+        lanes_sum(sc);
         softmax_tile(sc, valid);
         const int nt = min(kTile, w1 - t0);
         if (act_win) {
@@ -274,7 +325,7 @@ template <typename KV, int GH>
 static cudaError_t launch_direct_t(const Dims& s, const CacheDev& c, const DecodePlan& p, const void* q, char* ws,
                                    cudaStream_t st) {
     size_t smem = sizeof(float) * ((size_t)GH * s.d * 2 + (size_t)GH * s.nfk + 2 * (size_t)GH * s.M + (size_t)GH * kTile +
-                                   8 * GH + (size_t)256 * GH);
+                                   8 * GH + (size_t)(256 + 512) * GH);
     cudaError_t err = ensure_dynamic_smem(decode_direct_kernel<KV, GH>, smem);
     if (err != cudaSuccess) return err;
     decode_direct_kernel<KV, GH><<<dim3(p.n_split, s.Hkv * p.n_pass, s.B), 256, smem, st>>>(s, c, p, static_cast<const KV*>(q), ws);

@@ -104,13 +104,22 @@ def _check(status: int, what: str) -> None:
         raise FaError(status, what)
 
 
-def _stream(stream) -> C.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+# A call of a small cache is over on the device before Python has marshalled the next one, so the argument path is kept
+# short: plain integers for pointers (the argtypes convert them), the C view of a layout built once per layout, the raw
+# stream handle without a Stream object (40 -> 25 us of host time for a compress and a decode call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
-def _ptr(t) -> C.c_void_p:
-    return C.c_void_p(0 if t is None or t.numel() == 0 else t.data_ptr())
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
+
+
+def _ptr(t) -> int:
+    return 0 if t is None or t.numel() == 0 else t.data_ptr()
 
 
 @dataclass
@@ -133,6 +142,20 @@ class Layout:
     decode_algo: int = FA_DECODE_AUTO
     softmax_scale: float = 1.0
 
+    def __setattr__(self, name, value):
+        self.__dict__.pop("_cref", None)                  # the C view follows the fields
+        self.__dict__[name] = value
+
+    def __getstate__(self):
+        return {k: v for k, v in self.__dict__.items() if k != "_cref"}      # copies make their own view
+
+    def ref(self):
+        """By-reference argument of the C view, built once and again after a field changes."""
+        r = self.__dict__.get("_cref")
+        if r is None:
+            r = self.__dict__["_cref"] = C.byref(self.c())
+        return r
+
     def c(self) -> fa_layout:
         return fa_layout(self.batch, self.n_q_heads, self.n_kv_heads, self.head_dim, self.n_full_k, self.n_full_v,
                          self.n_coef, self.period, self.l_init, self.l_local, self.max_mid, self.mid_classes,
@@ -149,13 +172,13 @@ class Layout:
 
 def fa_cache_sizes_of(layout: Layout) -> dict:
     out = fa_cache_sizes()
-    _check(lib().fa_cache_sizes_of(C.byref(layout.c()), C.byref(out)), "fa_cache_sizes_of")
+    _check(lib().fa_cache_sizes_of(layout.ref(), C.byref(out)), "fa_cache_sizes_of")
     return {n: int(getattr(out, n)) for n in _CACHE_FIELDS}
 
 
 def fa_workspace_bytes(layout: Layout) -> int:
     out = C.c_size_t(0)
-    _check(lib().fa_workspace_bytes(C.byref(layout.c()), C.byref(out)), "fa_workspace_bytes")
+    _check(lib().fa_workspace_bytes(layout.ref(), C.byref(out)), "fa_workspace_bytes")
     return int(out.value)
 
 
@@ -198,10 +221,14 @@ class Cache:
         for n in _CACHE_FIELDS:
             t = getattr(self, n)
             assert t.numel() * t.element_size() == sizes[n], (n, t.shape, sizes[n])
-        self._c = fa_cache(*[_ptr(getattr(self, n)).value for n in _CACHE_FIELDS])
+        self._c = fa_cache(*[_ptr(getattr(self, n)) for n in _CACHE_FIELDS])
+        self._cref = C.byref(self._c)
 
     def c(self) -> fa_cache:
         return self._c
+
+    def ref(self):
+        return self._cref
 
     def bytes(self) -> int:
         return sum(getattr(self, n).numel() * getattr(self, n).element_size() for n in _CACHE_FIELDS)
@@ -218,11 +245,11 @@ def fa_workspace_init(ws: torch.Tensor, stream=None) -> None:
 
 
 def fa_cache_reset(layout: Layout, cache: Cache, stream=None) -> None:
-    _check(lib().fa_cache_reset(C.byref(layout.c()), C.byref(cache.c()), _stream(stream)), "fa_cache_reset")
+    _check(lib().fa_cache_reset(layout.ref(), cache.ref(), _stream(stream)), "fa_cache_reset")
 
 
 def fa_validate(layout: Layout, cache: Cache, stream=None) -> None:
-    _check(lib().fa_validate(C.byref(layout.c()), C.byref(cache.c()), _stream(stream)), "fa_validate")
+    _check(lib().fa_validate(layout.ref(), cache.ref(), _stream(stream)), "fa_validate")
 
 
 def fa_compress(layout: Layout, cache: Cache, K: torch.Tensor, V: torch.Tensor, ws: torch.Tensor, stream=None, flags: int = 0) -> None:
@@ -235,10 +262,10 @@ def fa_compress(layout: Layout, cache: Cache, K: torch.Tensor, V: torch.Tensor, 
     if K.shape[0] == 1:
         sb = 0
     if flags:
-        _check(lib().fa_compress_ex(C.byref(layout.c()), C.byref(cache.c()), _ptr(K), _ptr(V), sb, st, sh, L, int(flags),
+        _check(lib().fa_compress_ex(layout.ref(), cache.ref(), _ptr(K), _ptr(V), sb, st, sh, L, int(flags),
                                     _ptr(ws), ws.numel(), _stream(stream)), "fa_compress_ex")
         return
-    _check(lib().fa_compress(C.byref(layout.c()), C.byref(cache.c()), _ptr(K), _ptr(V), sb, st, sh, L,
+    _check(lib().fa_compress(layout.ref(), cache.ref(), _ptr(K), _ptr(V), sb, st, sh, L,
                              _ptr(ws), ws.numel(), _stream(stream)), "fa_compress")
 
 
@@ -270,26 +297,26 @@ def fa_compress_ragged(layout: Layout, cache: Cache, K: torch.Tensor, V: torch.T
     assert K.is_cuda and V.is_cuda and K.dtype == layout.torch_dtype and K.shape == V.shape and K.stride() == V.stride()
     assert K.stride(3) == 1 and len(lengths) == layout.batch and max(lengths) <= K.shape[1]
     arr = (C.c_int32 * layout.batch)(*[int(x) for x in lengths])
-    _check(lib().fa_compress_ragged(C.byref(layout.c()), C.byref(cache.c()), _ptr(K), _ptr(V), K.stride(0), K.stride(1),
+    _check(lib().fa_compress_ragged(layout.ref(), cache.ref(), _ptr(K), _ptr(V), K.stride(0), K.stride(1),
                                     K.stride(2), arr, _ptr(ws), ws.numel(), _stream(stream)), "fa_compress_ragged")
 
 
 def fa_append(layout: Layout, cache: Cache, k_new: torch.Tensor, v_new: torch.Tensor, stream=None) -> None:
     """k_new, v_new: contiguous [B][H_kv][d]."""
     assert k_new.is_contiguous() and v_new.is_contiguous() and k_new.dtype == layout.torch_dtype and k_new.is_cuda
-    _check(lib().fa_append(C.byref(layout.c()), C.byref(cache.c()), _ptr(k_new), _ptr(v_new), _stream(stream)), "fa_append")
+    _check(lib().fa_append(layout.ref(), cache.ref(), _ptr(k_new), _ptr(v_new), _stream(stream)), "fa_append")
 
 
 def fa_decode_attention(layout: Layout, cache: Cache, q: torch.Tensor, out: torch.Tensor, ws: torch.Tensor, stream=None) -> None:
     """q, out: contiguous [B][H_q][d]."""
     assert q.is_contiguous() and out.is_contiguous() and q.dtype == layout.torch_dtype and out.dtype == q.dtype
     assert q.is_cuda and out.is_cuda
-    _check(lib().fa_decode_attention(C.byref(layout.c()), C.byref(cache.c()), _ptr(q), _ptr(out), _ptr(ws), ws.numel(),
+    _check(lib().fa_decode_attention(layout.ref(), cache.ref(), _ptr(q), _ptr(out), _ptr(ws), ws.numel(),
                                      _stream(stream)), "fa_decode_attention")
 
 
 def fa_step_staging_bytes(layout: Layout) -> int:
-    return int(lib().fa_step_staging_bytes(C.byref(layout.c())))
+    return int(lib().fa_step_staging_bytes(layout.ref()))
 
 
 def fa_select_dims(layout: Layout, K: torch.Tensor, V: torch.Tensor, stream=None):
@@ -299,13 +326,13 @@ def fa_select_dims(layout: Layout, K: torch.Tensor, V: torch.Tensor, stream=None
     B, L, H, d = K.shape
     assert K.stride(3) == 1
     out = C.c_size_t(0)
-    _check(lib().fa_select_workspace_bytes(C.byref(layout.c()), C.byref(out)), "fa_select_workspace_bytes")
+    _check(lib().fa_select_workspace_bytes(layout.ref(), C.byref(out)), "fa_select_workspace_bytes")
     ws = torch.zeros(max(256, out.value), dtype=torch.uint8, device=K.device)
     dev = K.device
     idx = [torch.zeros((H, n), dtype=torch.int32, device=dev) for n in
            (layout.n_full_k, d - layout.n_full_k, layout.n_full_v, d - layout.n_full_v)]
     mse = torch.zeros((B, H, 2, d), dtype=torch.float32, device=dev)
-    _check(lib().fa_select_dims(C.byref(layout.c()), _ptr(K), _ptr(V), K.stride(0), K.stride(1), K.stride(2), L,
+    _check(lib().fa_select_dims(layout.ref(), _ptr(K), _ptr(V), K.stride(0), K.stride(1), K.stride(2), L,
                                 *[_ptr(t) if t.numel() else None for t in idx], _ptr(mse), _ptr(ws), ws.numel(),
                                 _stream(stream)), "fa_select_dims")
     return (*idx, mse)
@@ -316,7 +343,7 @@ def fa_decode_step(layout: Layout, cache: Cache, q: torch.Tensor, k_new: torch.T
     """fa_append(k_new, v_new) then fa_decode_attention(q) as one step (device tensors)."""
     for t in (q, k_new, v_new, out):
         assert t.is_cuda and t.is_contiguous() and t.dtype == layout.torch_dtype
-    _check(lib().fa_decode_step(C.byref(layout.c()), C.byref(cache.c()), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out),
+    _check(lib().fa_decode_step(layout.ref(), cache.ref(), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out),
                                 _ptr(ws), ws.numel(), _stream(stream)), "fa_decode_step")
 
 
@@ -351,17 +378,17 @@ def fa_decode_step_host(layout: Layout, cache: Cache, q_host: torch.Tensor, k_ne
     for t in (q_host, out_host, k_new_host, v_new_host):
         assert t is None or (not t.is_cuda and t.is_contiguous() and t.dtype == layout.torch_dtype)
     assert staging.is_cuda and staging.numel() * staging.element_size() >= fa_step_staging_bytes(layout)
-    _check(lib().fa_decode_step_host(C.byref(layout.c()), C.byref(cache.c()), _ptr(q_host), _ptr(k_new_host),
+    _check(lib().fa_decode_step_host(layout.ref(), cache.ref(), _ptr(q_host), _ptr(k_new_host),
                                      _ptr(v_new_host), _ptr(out_host), _ptr(staging), _ptr(ws), ws.numel(),
                                      _stream(stream)), "fa_decode_step_host")
 
 
 def fa_poll_status(cache: Cache, stream=None) -> int:
-    return int(lib().fa_poll_status(C.byref(cache.c()), _stream(stream)))
+    return int(lib().fa_poll_status(cache.ref(), _stream(stream)))
 
 
 def fa_launch_count(layout: Layout, what: int) -> int:
-    return int(lib().fa_launch_count(C.byref(layout.c()), int(what)))
+    return int(lib().fa_launch_count(layout.ref(), int(what)))
 
 
 def fa_version() -> int:
@@ -385,4 +412,4 @@ def fa_decode_attention_static(layout: Layout, cache: Cache, q: torch.Tensor, ou
     f = lib().fa_decode_attention_static
     f.restype = C.c_int
     f.argtypes = [C.POINTER(fa_layout), C.POINTER(fa_cache), C.c_void_p, C.c_void_p, C.c_void_p]
-    _check(f(C.byref(layout.c()), C.byref(cache.c()), _ptr(q), _ptr(out), _stream(stream)), "fa_decode_attention_static")
+    _check(f(layout.ref(), cache.ref(), _ptr(q), _ptr(out), _stream(stream)), "fa_decode_attention_static")

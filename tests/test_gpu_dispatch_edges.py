@@ -49,3 +49,19 @@ def test_ragged_compress_in_one_launch_equals_row_by_row(B, M, lengths):
             # (basis phasors are seeded where a CTA's blocks begin: some bf16 roundings of the basis differ)
             assert (g - r).abs().max() <= 2e-4 * r.abs().max() + 1e-6, (b, n)
     assert fa.fa_poll_status(got) == fa.FA_OK
+
+
+@pytest.mark.parametrize("kw,P", [
+    (dict(L=63, T=64, M=8), 1),                          # one tile, one frequency group, token-major
+    (dict(L=200, T=400, M=66), 3),                       # odd class count and period, a frequency more than a warp
+    (dict(L=700, T=1024, M=1024, L_init=3, L_local=70), 4),   # more frequencies than threads
+    (dict(L=600, T=1024, M=100, n_full_k=0, n_full_v=128, Hq=3), 2),   # three heads in four slots; no kept K, no compressed V dims
+])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_direct_decode_tiles_of_tokens(kw, P, dtype):
+    shape = synth.Shape("direct", **{**dict(B=2, layers=1, Hq=2, Hkv=1, d=128, dtype=dtype, n_full_k=32, n_full_v=24, L_init=0,
+                                            L_local=0, decode_steps=0), **kw})
+    pair, _ = make_pair(shape, seed=9, P=P, algo=fa.FA_DECODE_DIRECT, freq="offgrid", max_mid=min(shape.T, shape.L))
+    pair.check_state()
+    pair.check_decode(synth.queries(shape, seed=9))
+    pair.check_decode(synth.queries(shape, seed=9, step=1, peak=6.0))
