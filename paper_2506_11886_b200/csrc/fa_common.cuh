@@ -177,6 +177,13 @@ __device__ __forceinline__ float recon_weight(int norm, int m, int k, int T) {
 
 // Eq.4: cos and sin of 2 pi n j / T, with n * j reduced modulo T in integers first.
 __device__ __forceinline__ void basis_cs(int n, int j, int T, float* c, float* s) {
+    if ((T & (T - 1)) == 0) {
+        // a power-of-two period: the product modulo 2^32 is enough, and 2 / T is exact (the 64-bit remainder below took most
+        // of the fp32 contraction's time)
+        const unsigned r = ((unsigned)n * (unsigned)j) & (unsigned)(T - 1);
+        sincospif((float)r * __int_as_float((128 - (31 - __clz(T))) << 23), s, c);
+        return;
+    }
     long long r = ((long long)n * (long long)j) % (long long)T;
     sincospif(2.0f * (float)r / (float)T, s, c);
 }

@@ -243,12 +243,15 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     RowLens rl = {};
     if (lens) rl = *lens;
     // chunks and short middles (not the tensor-core kernel's) of the longest row
-    int chunks_rows = 1, n_mid = 0;
+    int chunks_rows = 1, n_mid = 0, n_short = 0;
     for (int b = 0; b < (rl.n ? rl.n : 1); ++b) {
         const int Lb = row_len(rl, L, b), ni = Lb < s.l_init ? Lb : s.l_init, nl = (Lb - ni) < s.l_local ? (Lb - ni) : s.l_local;
         int chunks = (Lb + kRowsPerCta - 1) / kRowsPerCta, first;
         if (Lb - ni - nl >= tc_min) chunks -= window_skip(Lb, ni, nl, &first);
-        else if (Lb - ni - nl > n_mid) n_mid = Lb - ni - nl;
+        else {
+            ++n_short;
+            if (Lb - ni - nl > n_mid) n_mid = Lb - ni - nl;
+        }
         if (chunks > chunks_rows) chunks_rows = chunks;
     }
     constexpr int EPC = 16 / (int)sizeof(KV);
@@ -278,7 +281,7 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     if (n_mid == 0 || max_comp == 0 || !with_coef) return cudaSuccess;
     int row_tiles = (s.M + kTM - 1) / kTM;
     int chunks = (n_mid + kTJ - 1) / kTJ;
-    int ctas_fixed = row_tiles * s.B * s.Hkv * 2;
+    int ctas_fixed = row_tiles * (rl.n ? n_short : s.B) * s.Hkv * 2;
     int n_tsplit = (4 * sm_count() + ctas_fixed - 1) / ctas_fixed;
     if (n_tsplit > chunks) n_tsplit = chunks;
     if (n_tsplit < 1 || ordered) n_tsplit = 1;               // one split: every coefficient is added to zero exactly once

@@ -22,9 +22,15 @@ constexpr int kMseRows = 32;        // coefficient rows staged per round (16 fre
 
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-__global__ void iota_rows_kernel(int32_t* p, int rows, int d) {
+// What the scratch cache needs before the compression, in one launch: every dim in D^kc and D^vc, the status word, the
+// barrier counters of the workspace and the error sums cleared.
+__global__ void select_init_kernel(int32_t* idx_k, int32_t* idx_v, int H, int d, int32_t* status, int32_t* counters, int n_counters,
+                                   float* sq, int n_sq) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < rows * d) p[i] = i % d;
+    if (i < H * d) { idx_k[i] = i % d; idx_v[i] = i % d; }
+    if (i < 4) status[i] = 0;
+    if (i < n_counters) counters[i] = 0;
+    if (i < n_sq) sq[i] = 0.f;
 }
 
 // grid (ceil(n_mid / 64), Hkv * 2, B), 256 threads = 64 tokens x 4 groups of d/4 dims.
@@ -87,7 +93,7 @@ __global__ void __launch_bounds__(256) mse_kernel(Dims s, const float* __restric
 
 // grid (Hkv, 2), d threads (<= 256).  Normalises the sums to mean squared errors, averages them over
 // the batch rows and ranks the dims: the d - n_full with the smallest (error, index) are compressed.
-__global__ void select_kernel(Dims s, float* __restrict__ sq, int n_mid, int32_t* idx_full_k, int32_t* idx_comp_k,
+__global__ void select_kernel(Dims s, const float* __restrict__ sq, float* __restrict__ mse, int n_mid, int32_t* idx_full_k, int32_t* idx_comp_k,
                               int32_t* idx_full_v, int32_t* idx_comp_v) {
     __shared__ float m_s[256];
     __shared__ int comp_s[256];
@@ -96,9 +102,9 @@ __global__ void select_kernel(Dims s, float* __restrict__ sq, int n_mid, int32_t
     float mean = 0.f;
     if (e < d) {
         for (int b = 0; b < s.B; ++b) {
-            float* p = sq + (((size_t)b * s.Hkv + h) * 2 + side) * d + e;
-            const float v = n_mid > 0 ? *p / (float)n_mid : 0.f;
-            *p = v;
+            const size_t at = (((size_t)b * s.Hkv + h) * 2 + side) * d + e;
+            const float v = n_mid > 0 ? sq[at] / (float)n_mid : 0.f;
+            if (mse) mse[at] = v;
             mean += v;
         }
         mean /= (float)s.B;
@@ -111,14 +117,11 @@ __global__ void select_kernel(Dims s, float* __restrict__ sq, int n_mid, int32_t
         comp_s[e] = rank < d - n_full;
     }
     __syncthreads();
-    if (e == 0) {
-        int32_t* full = (side == 0 ? idx_full_k : idx_full_v) + (size_t)h * n_full;
-        int32_t* comp = (side == 0 ? idx_comp_k : idx_comp_v) + (size_t)h * (d - n_full);
-        int a = 0, c = 0;
-        for (int i = 0; i < d; ++i) {
-            if (comp_s[i]) comp[c++] = i;
-            else full[a++] = i;
-        }
+    if (e < d) {
+        int below = 0;                                    // compressed dims in front of this one
+        for (int i = 0; i < e; ++i) below += comp_s[i];
+        if (comp_s[e]) (side == 0 ? idx_comp_k : idx_comp_v)[(size_t)h * (d - n_full) + below] = e;
+        else (side == 0 ? idx_full_k : idx_full_v)[(size_t)h * n_full + e - below] = e;
     }
 }
 
@@ -216,19 +219,17 @@ fa_status fa_select_dims(const fa_layout* layout, const void* K, const void* V, 
     if (ws_bytes < sc.total) return FA_ERR_WORKSPACE;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const Dims s = make_dims(*layout);
-    const int n_ids = s.Hkv * s.d;
-    iota_rows_kernel<<<(n_ids + 255) / 256, 256, 0, cs>>>(const_cast<int32_t*>(sc.cache.idx_comp_k), s.Hkv, s.d);
-    iota_rows_kernel<<<(n_ids + 255) / 256, 256, 0, cs>>>(const_cast<int32_t*>(sc.cache.idx_comp_v), s.Hkv, s.d);
+    const int n_sq = s.B * s.Hkv * 2 * s.d, n_counters = (int)(sc.ws_compress_bytes < 4096 ? sc.ws_compress_bytes : 4096) / 4;
+    const int n_threads = n_sq > n_counters ? n_sq : n_counters;      // (n_sq >= the index sets' entries)
+    select_init_kernel<<<(n_threads + 255) / 256, 256, 0, cs>>>(const_cast<int32_t*>(sc.cache.idx_comp_k), const_cast<int32_t*>(sc.cache.idx_comp_v),
+                                                               s.Hkv, s.d, sc.cache.status, reinterpret_cast<int32_t*>(sc.ws_compress), n_counters,
+                                                               sc.sq, n_sq);
     if (cudaGetLastError() != cudaSuccess) return FA_ERR_CUDA;
-    if (cudaMemsetAsync(sc.cache.status, 0, 16, cs) != cudaSuccess) return FA_ERR_CUDA;
-    if (cudaMemsetAsync(sc.ws_compress, 0, sc.ws_compress_bytes < 4096 ? sc.ws_compress_bytes : 4096, cs) != cudaSuccess) return FA_ERR_CUDA;
     st = fa_compress(&sc.layout, &sc.cache, K, V, stride_b, stride_t, stride_h, L, sc.ws_compress, sc.ws_compress_bytes, stream);
     if (st != FA_OK) return st;
     const int n_init = L < s.l_init ? L : s.l_init;
     const int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;
     const int n_mid = L - n_init - n_local;
-    const size_t sq_bytes = sizeof(float) * (size_t)s.B * s.Hkv * 2 * s.d;
-    if (cudaMemsetAsync(sc.sq, 0, sq_bytes, cs) != cudaSuccess) return FA_ERR_CUDA;
     if (n_mid > 0 && reconstruct_tc_supported(s, layout->kv_dtype, K, V, stride_b, stride_t, stride_h, n_mid)) {
         if (launch_reconstruct_tc(s, sc.cache.coef_k, sc.cache.coef_v, K, V, stride_b, stride_t, stride_h, n_init, n_mid, sc.sq,
                                   sc.cache.status, sc.wc16, cs) != cudaSuccess)
@@ -239,9 +240,8 @@ fa_status fa_select_dims(const fa_layout* layout, const void* K, const void* V, 
                               : launch_mse<float>(s, sc.cache, K, V, stride_b, stride_t, stride_h, n_init, n_mid, sc.sq, cs);
         if (err != cudaSuccess) return FA_ERR_CUDA;
     }
-    select_kernel<<<dim3(s.Hkv, 2), 256, 0, cs>>>(s, sc.sq, n_mid, idx_full_k, idx_comp_k, idx_full_v, idx_comp_v);
+    select_kernel<<<dim3(s.Hkv, 2), 256, 0, cs>>>(s, sc.sq, mse, n_mid, idx_full_k, idx_comp_k, idx_full_v, idx_comp_v);
     if (cudaGetLastError() != cudaSuccess) return FA_ERR_CUDA;
-    if (mse && cudaMemcpyAsync(mse, sc.sq, sq_bytes, cudaMemcpyDeviceToDevice, cs) != cudaSuccess) return FA_ERR_CUDA;
     return FA_OK;
 }
 

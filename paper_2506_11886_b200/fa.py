@@ -327,11 +327,11 @@ def fa_select_dims(layout: Layout, K: torch.Tensor, V: torch.Tensor, stream=None
     assert K.stride(3) == 1
     out = C.c_size_t(0)
     _check(lib().fa_select_workspace_bytes(layout.ref(), C.byref(out)), "fa_select_workspace_bytes")
-    ws = torch.zeros(max(256, out.value), dtype=torch.uint8, device=K.device)
+    ws = torch.empty(max(256, out.value), dtype=torch.uint8, device=K.device)     # (the call clears what it has to)
     dev = K.device
-    idx = [torch.zeros((H, n), dtype=torch.int32, device=dev) for n in
+    idx = [torch.empty((H, n), dtype=torch.int32, device=dev) for n in
            (layout.n_full_k, d - layout.n_full_k, layout.n_full_v, d - layout.n_full_v)]
-    mse = torch.zeros((B, H, 2, d), dtype=torch.float32, device=dev)
+    mse = torch.empty((B, H, 2, d), dtype=torch.float32, device=dev)
     _check(lib().fa_select_dims(layout.ref(), _ptr(K), _ptr(V), K.stride(0), K.stride(1), K.stride(2), L,
                                 *[_ptr(t) if t.numel() else None for t in idx], _ptr(mse), _ptr(ws), ws.numel(),
                                 _stream(stream)), "fa_select_dims")
