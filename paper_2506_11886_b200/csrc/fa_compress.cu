@@ -141,14 +141,16 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
 }
 
 // ---- Eq.3-4: C[m][e] += sum_j F[m][j] X[n_init + j][D^c[e]] ------------------
-// grid (row tiles of 32 coefficient rows, token splits, B * Hkv * 2 sides).
+// grid (row tiles of 32 or 64 coefficient rows, token splits, B * Hkv * 2 sides).
 // Per 64-token chunk the CTA stages the gathered columns and a 64 x 32 basis
 // tile in shared memory; thread (rg, lane) accumulates rows 4 rg..4 rg + 3 of
 // the tile for columns lane, lane + 32, ...  Partial sums of the token splits
 // are added to the zeroed coefficients with atomics.
-constexpr int kTM = 32, kTJ = 64;
+// R rows per thread: eight where that leaves CTAs enough (half the shared-memory reads per product), else four.
+constexpr int kTJ = 64;
 
-template <typename KV>
+// NC: columns per lane (32 NC >= the compressed dims of either side; the products of lanes without a column are not issued).
+template <typename KV, int NC, int R>
 __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, const KV* __restrict__ K,
                                                             const KV* __restrict__ V, int64_t sb, int64_t st, int64_t sh,
                                                             int Lmax, int chunks_per_split, const __grid_constant__ RowLens lens, int tc_min) {
@@ -168,20 +170,20 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
     const int32_t* idc = (side == 0 ? c.idx_comp_k : c.idx_comp_v) + (size_t)h * ncomp;
     float* coef = coef_rows(side == 0 ? c.coef_k : c.coef_v, s, b, h, ncomp);
 
-    float* X_s = smem;                       // [kTJ][ncomp]
-    float* F_s = smem + kTJ * ncomp;         // [kTJ][kTM]
+    constexpr int kTM = 8 * R, kXs = 32 * NC;
+    float* X_s = smem;                       // [kTJ][kXs], zeros past the compressed dims
+    float* F_s = smem + kTJ * kXs;           // [kTJ][kTM]
     int m0 = blockIdx.x * kTM;
     int rg = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int ncol = (ncomp + 31) / 32;            // <= 8
-    float acc[4][8];
+    float acc[R][NC];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[r][i] = 0.f;
+        for (int i = 0; i < NC; ++i) acc[r][i] = 0.f;
 
-    int col[8];
+    int col[NC];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) col[i] = lane + 32 * i < ncomp ? idc[lane + 32 * i] : 0;
+    for (int i = 0; i < NC; ++i) col[i] = lane + 32 * i < ncomp ? idc[lane + 32 * i] : 0;
 
     int j_begin = blockIdx.y * chunks_per_split * kTJ;
     int j_end = min(n_mid, j_begin + chunks_per_split * kTJ);
@@ -191,12 +193,11 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
         // a warp takes every eighth token: its lanes' columns are fixed, so all loads of a chunk are independent
         const KV* xrow = X + (size_t)(n_init + j0 + rg) * st;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < NC; ++i) {
             const int e = lane + 32 * i;
-            if (i < ncol && e < ncomp)
 #pragma unroll
                 for (int q = 0; q < kTJ / 8; ++q)
-                    X_s[(rg + 8 * q) * ncomp + e] = rg + 8 * q < nj ? ld_f(xrow + (size_t)(8 * q) * st + col[i]) : 0.f;
+                    X_s[(rg + 8 * q) * kXs + e] = e < ncomp && rg + 8 * q < nj ? ld_f(xrow + (size_t)(8 * q) * st + col[i]) : 0.f;
         }
         // basis tile: thread -> (token jj, frequency pair nn) ; rows 2 nn (cos), 2 nn + 1 (sin)
         for (int i = threadIdx.x; i < kTJ * (kTM / 2); i += blockDim.x) {
@@ -208,30 +209,31 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
             F_s[jj * kTM + 2 * nn + 1] = sn;
         }
         __syncthreads();
+#pragma unroll 4
         for (int jj = 0; jj < nj; ++jj) {
-            float4 f = *reinterpret_cast<const float4*>(F_s + jj * kTM + 4 * rg);
+            float f[R];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (i < ncol) {
-                    int e = lane + 32 * i;
-                    float x = e < ncomp ? X_s[jj * ncomp + e] : 0.f;
-                    acc[0][i] = fmaf(f.x, x, acc[0][i]);
-                    acc[1][i] = fmaf(f.y, x, acc[1][i]);
-                    acc[2][i] = fmaf(f.z, x, acc[2][i]);
-                    acc[3][i] = fmaf(f.w, x, acc[3][i]);
-                }
+            for (int r = 0; r < R; r += 4) {
+                const float4 f4 = *reinterpret_cast<const float4*>(F_s + jj * kTM + R * rg + r);
+                f[r] = f4.x; f[r + 1] = f4.y; f[r + 2] = f4.z; f[r + 3] = f4.w;
+            }
+#pragma unroll
+            for (int i = 0; i < NC; ++i) {
+                const float x = X_s[jj * kXs + lane + 32 * i];
+#pragma unroll
+                for (int r = 0; r < R; ++r) acc[r][i] = fmaf(f[r], x, acc[r][i]);
             }
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");    // the partition kernel clears the coefficients
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        int m = m0 + 4 * rg + r;
+    for (int r = 0; r < R; ++r) {
+        int m = m0 + R * rg + r;
         if (m >= s.M) continue;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < NC; ++i) {
             int e = lane + 32 * i;
-            if (i < ncol && e < ncomp) atomicAdd(coef + (size_t)m * ncomp + e, acc[r][i]);
+            if (e < ncomp) atomicAdd(coef + (size_t)m * ncomp + e, acc[r][i]);
         }
     }
 }
@@ -279,17 +281,18 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     if (err != cudaSuccess) return err;
     int max_comp = s.dck > s.dcv ? s.dck : s.dcv;
     if (n_mid == 0 || max_comp == 0 || !with_coef) return cudaSuccess;
-    int row_tiles = (s.M + kTM - 1) / kTM;
+    const int live_rows = rl.n ? n_short : s.B;
+    const int rpt = (long long)((s.M + 63) / 64) * live_rows * s.Hkv * 2 >= 2 * sm_count() ? 8 : 4;
+    const int row_tiles = (s.M + 8 * rpt - 1) / (8 * rpt);
     int chunks = (n_mid + kTJ - 1) / kTJ;
-    int ctas_fixed = row_tiles * (rl.n ? n_short : s.B) * s.Hkv * 2;
+    int ctas_fixed = row_tiles * live_rows * s.Hkv * 2;
     int n_tsplit = (4 * sm_count() + ctas_fixed - 1) / ctas_fixed;
     if (n_tsplit > chunks) n_tsplit = chunks;
     if (n_tsplit < 1 || ordered) n_tsplit = 1;               // one split: every coefficient is added to zero exactly once
     int cps = (chunks + n_tsplit - 1) / n_tsplit;
     n_tsplit = (chunks + cps - 1) / cps;
-    size_t smem = sizeof(float) * ((size_t)kTJ * max_comp + (size_t)kTJ * kTM);
-    err = ensure_dynamic_smem(compress_coef_kernel<KV>, smem);
-    if (err != cudaSuccess) return err;
+    const int nc = max_comp <= 128 ? (max_comp + 31) / 32 : 8;
+    const size_t smem = sizeof(float) * kTJ * (size_t)(32 * nc + 8 * rpt);
     // behind the partition kernel programmatically: it waits for it in front of its additions
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(row_tiles, n_tsplit, s.B * s.Hkv * 2);
@@ -301,8 +304,18 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, compress_coef_kernel<KV>, s, c, static_cast<const KV*>(K), static_cast<const KV*>(V), sb, st, sh, L, cps,
-                              rl, tc_min);
+    auto go = [&](auto kernel) {
+        const cudaError_t e = ensure_dynamic_smem(kernel, smem);
+        if (e != cudaSuccess) return e;
+        return cudaLaunchKernelEx(&cfg, kernel, s, c, static_cast<const KV*>(K), static_cast<const KV*>(V), sb, st, sh, L, cps, rl, tc_min);
+    };
+    switch (nc) {
+        case 1: return rpt == 8 ? go(compress_coef_kernel<KV, 1, 8>) : go(compress_coef_kernel<KV, 1, 4>);
+        case 2: return rpt == 8 ? go(compress_coef_kernel<KV, 2, 8>) : go(compress_coef_kernel<KV, 2, 4>);
+        case 3: return rpt == 8 ? go(compress_coef_kernel<KV, 3, 8>) : go(compress_coef_kernel<KV, 3, 4>);
+        case 4: return rpt == 8 ? go(compress_coef_kernel<KV, 4, 8>) : go(compress_coef_kernel<KV, 4, 4>);
+        default: return rpt == 8 ? go(compress_coef_kernel<KV, 8, 8>) : go(compress_coef_kernel<KV, 8, 4>);
+    }
 }
 
 // with_coef = false runs only the partition / gather kernel (the tensor-core or the transform path computes the

@@ -64,12 +64,14 @@ struct RowCuts {
 // D = head dim (64 or 128): N = 2 D accumulator columns per KV head (K dims, then V dims); HP heads share the pair
 // and its generated basis tiles (HP * N <= 512 tensor-memory columns).  grid 2 * teams * (M / 256), clusters of two.
 // kGatherWarps: kFewGather or kManyGather (the latter may take several rounds).
-template <int D, int HP, int kGatherWarps>
+// RAG: rows of different length.
+template <int D, int HP, int kGatherWarps, bool RAG>
 __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV, Dims s,
                                                                      CacheDev c, int Lall, const __grid_constant__ TeamCuts cuts,
                                                                      const __grid_constant__ RowCuts rows, int per, int gather) {
     constexpr int N = 2 * D;
+    constexpr int kItems = kGatherWarps == kManyGather ? kGatherItems : 2;
     constexpr int kABytes = kBM * kBK * 2;                 // 16 KB basis tile
     constexpr int kBoxBytes = kBK * 64 * 2;                // 8 KB per [64 tokens x 64 dims] box
     constexpr int kBHalf1 = (D / 64) * kBoxBytes;           // this CTA's boxes of one head: all D dims of ONE side
@@ -118,7 +120,7 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
         int b = 0, n_mid = n_mid_all, nkb = nkb_all;
         const uint32_t end = pos_end;
         uint32_t off = pos;
-        if (rows.lens.n) {
+        if (RAG) {
             while (pos >= rows.first[b + 1]) ++b;
             off = pos - rows.first[b];
             n_mid = mid_of(s, rows.lens.len[b]);
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
         int unit = (int)(off / (uint32_t)nkb);
         const int kb0 = (int)(off - (uint32_t)unit * (uint32_t)nkb);
         const int kb1 = (int)min((uint32_t)nkb, (uint32_t)kb0 + (end - pos));
-        if (!rows.lens.n) { b = unit / n_hg; unit -= b * n_hg; }
+        if (!RAG) { b = unit / n_hg; unit -= b * n_hg; }
         return Seg{b, unit * HP, kb0, kb1, n_mid};
     };
 
@@ -256,10 +258,10 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
                 // An item = one 16-byte chunk (8 kept dims) of one kept-dim row.  A thread keeps the same items in every
                 // block: token row r of the boxes, head, side and LOGICAL chunk, so the eight source offsets inside a stage
                 // are constants (two 16-bit offsets per register); only the destination row moves with the token.
-                uint32_t src[kGatherItems][4];
-                int meta[kGatherItems];                    // r | hh << 8 | lch << 16, or -1
+                uint32_t src[kItems][4];
+                int meta[kItems];                    // r | hh << 8 | lch << 16, or -1
 #pragma unroll
-                for (int u = 0; u < kGatherItems; ++u) {
+                for (int u = 0; u < kItems; ++u) {
                     const int idx = gt + u * 32 * kGatherWarps;
                     meta[u] = -1;
 #pragma unroll
@@ -287,9 +289,9 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
                     int jb = kb * kBK;                     // first middle token of the round
 #pragma unroll 1
                     for (int q = 0; q < rounds; ++q, bsrc += rpr * 128, jb += rpr) {
-                        uint4 val[kGatherItems];
+                        uint4 val[kItems];
 #pragma unroll
-                        for (int u = 0; u < kGatherItems; ++u) {
+                        for (int u = 0; u < kItems; ++u) {
                             uint32_t w[4] = {0u, 0u, 0u, 0u};
                             if (meta[u] >= 0) {
 #pragma unroll
@@ -306,9 +308,9 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
                             if (lane == 0) mbar_arrive(empty + st);
                         }
 #pragma unroll
-                        for (int u = 0; u < kGatherItems; ++u) {
+                        for (int u = 0; u < kItems; ++u) {
                             const int j = jb + (meta[u] & 0xff);
-                            if (meta[u] >= 0 && j < g.n_mid) {
+                            if (meta[u] >= 0 && j < (RAG ? g.n_mid : n_mid_all)) {
                                 const int hh = (meta[u] >> 8) & 0xf, lch = meta[u] >> 16;
                                 const int cls = p2 ? (j & (s.P - 1)) : j % s.P, slot = p2 ? (j >> lgP) : j / s.P;
                                 const int nfull = nf_side;
@@ -368,7 +370,8 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
                         asm("mov.b64 %0, {%1,%2};" : "=l"(C) : "f"(__cosf(aa)), "f"(__cosf(ab)));
                         asm("mov.b64 %0, {%1,%2};" : "=l"(S) : "f"(__sinf(aa)), "f"(__sinf(ab)));
                     }
-                    const bool whole = row_on && j0 + 16 <= g.n_mid;      // no masking needed in the common case
+                    const int n_mid = RAG ? g.n_mid : n_mid_all;
+                    const bool whole = row_on && j0 + 16 <= n_mid;      // no masking needed in the common case
 #pragma unroll
                     for (int ch = 0; ch < 2; ++ch) {       // 8 tokens = one 16-byte chunk of each row
                         uint32_t wc[4], wsn[4];
@@ -379,7 +382,7 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
                             asm("mov.b64 {%0,%1}, %2;" : "=f"(s0), "=f"(s1) : "l"(S));
                             if (!whole) {
                                 const int j = j0 + ch * 8 + i2 * 2;
-                                const bool v0 = row_on && j < g.n_mid, v1 = row_on && j + 1 < g.n_mid;
+                                const bool v0 = row_on && j < n_mid, v1 = row_on && j + 1 < n_mid;
                                 c0 = v0 ? c0 : 0.f; s0 = v0 ? s0 : 0.f; c1 = v1 ? c1 : 0.f; s1 = v1 ? s1 : 0.f;
                             }
                             const __nv_bfloat162 pc = __floats2bfloat162_rn(c0, c1);
@@ -498,13 +501,13 @@ bool make_map2(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, int HP, int GW>
+template <int D, int HP, int GW, bool RAG>
 cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, const RowCuts& rows,
                          bool ordered, bool gather, cudaStream_t stream) {
     constexpr size_t stage = (size_t)kBM * kBK * 2 + (size_t)HP * (D / 64) * kBK * 64 * 2;
     constexpr size_t n_stages = (200 * 1024) / stage < 6 ? (200 * 1024) / stage : 6;
     const size_t smem = n_stages * stage + 8 * (3 * n_stages + 3) + 16 + sizeof(int) * HP * D + 64 + 1024;
-    cudaError_t err = ensure_dynamic_smem(compress_tc2_kernel<D, HP, GW>, smem);
+    cudaError_t err = ensure_dynamic_smem(compress_tc2_kernel<D, HP, GW, RAG>, smem);
     if (err != cudaSuccess) return err;
     const int n_pairs = s.M / (2 * kBM);
     const int nkb = (mid_of(s, L) + kBK - 1) / kBK;
@@ -543,7 +546,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
             cfg.gridDim = dim3(2 * sm_count());
             cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, compress_tc2_kernel<D, HP, GW>, &cfg) != cudaSuccess || n < 1) {
+            if (cudaOccupancyMaxActiveClusters(&n, compress_tc2_kernel<D, HP, GW, RAG>, &cfg) != cudaSuccess || n < 1) {
                 cudaGetLastError();
                 n = sm_count() / 2 - 2;
             }
@@ -592,7 +595,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
         cuts.start[n_teams] = (uint32_t)total;
     }
     cfg.gridDim = dim3(2 * n_teams * n_pairs);
-    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW>, tmK, tmV, s, c, L, cuts, rows, per, gather ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW, RAG>, tmK, tmV, s, c, L, cuts, rows, per, gather ? 1 : 0);
 }
 
 }  // namespace
@@ -629,8 +632,11 @@ cudaError_t launch_compress_tc2(const Dims& s, const CacheDev& c, const void* K,
     const int n_pairs = s.M / (2 * kBM), items = (kBK + n_pairs - 1) / n_pairs * (pair ? 2 : 1) * (nf >> 3);
     const bool many = gather && items > 2 * 32 * kFewGather;
     auto go = [&](auto d, auto hp) {
-        return many ? launch_tc2_t<d, hp, kManyGather>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
-                    : launch_tc2_t<d, hp, kFewGather>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
+        if (rows.lens.n)
+            return many ? launch_tc2_t<d, hp, kManyGather, true>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
+                        : launch_tc2_t<d, hp, kFewGather, true>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
+        return many ? launch_tc2_t<d, hp, kManyGather, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
+                    : launch_tc2_t<d, hp, kFewGather, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
     };
     using std::integral_constant;
     if (s.d == 128) return pair ? go(integral_constant<int, 128>{}, integral_constant<int, 2>{}) : go(integral_constant<int, 128>{}, integral_constant<int, 1>{});
