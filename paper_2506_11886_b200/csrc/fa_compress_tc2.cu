@@ -8,7 +8,7 @@
 //
 // Roles per CTA: warp 0 (one lane) TMA producer of its half of the boxes; warp 1 allocates tensor memory (one warp of
 // each CTA, collectively) and, in the even CTA only, issues the MMAs of the pair; warps 2-9 generate the basis tile and
-// run the epilogue; warps 10-13 write the kept-dim rows of the middle (the even CTA K^mu, the odd CTA V^mu).
+// run the epilogue; the warps from 10 on write the kept-dim rows of the middle (the even CTA K^mu, the odd CTA V^mu).
 // Barriers across the pair: a lane of the odd CTA waits for that CTA's basis tile and boxes of a stage and forwards
 // their completion to the even CTA (mapa + remote arrive); the even CTA's tcgen05.commit
 // signals the stage barriers of both CTAs (multicast of the ARRIVAL, not of a load).
@@ -25,22 +25,21 @@ using bf16 = __nv_bfloat16;
 constexpr int kBM = 128;          // coefficient rows per CTA (256 per pair)
 constexpr int kBK = 64;           // tokens per pipeline stage
 constexpr int kGenWarps = 8;       // basis generators (and epilogue): 16 tokens of two rows per thread and stage
-constexpr int kGatherItems = 4;    // 16-byte chunks per gather thread and round, at most
 // Rounds in which the gather warps take the rows of a stage: a round is 64 / rounds consecutive rows, so that a thread's
 // items of round q lie a constant q * (64 / rounds) * 128 bytes behind those of round 0 (the swizzle repeats every
 // eight rows) and only one round's offsets are held in registers.  The smallest power of two with which the pairs of
-// a team cover the kept dims; eight rounds always do (8 rows x 2 heads x 16 chunks = 256 of 512 items).
-__host__ __device__ inline int gather_rounds(int n_pairs, int hp, int nf, int gw) {
+// a team cover the kept dims; eight rounds always do (8 rows x 2 heads x 16 chunks = 256 of 1024 items).
+__host__ __device__ inline int gather_rounds(int n_pairs, int hp, int nf, int per_round) {
     int r = 1;
-    while (r < 8 && ((kBK / r + n_pairs - 1) / n_pairs) * hp * (nf >> 3) > kGatherItems * 32 * gw) r *= 2;
+    while (r < 8 && ((kBK / r + n_pairs - 1) / n_pairs) * hp * (nf >> 3) > per_round) r *= 2;
     return r;
 }
-// Warps that write the kept-dim rows of the middle from the B boxes: four where a thread has at most two of a stage's
-// items (more warps only draw power: the 32K contraction runs at the power cap and loses 3 % with six), eight where it
-// has more (few pairs per team and many kept dims: every pair writes most rows of its boxes itself; 4 K tokens of the
-// 32-head MHA layout, 48 kept dims: fa_compress 264 us with four, 234 with six, 227 with eight, and 320 with the rows
-// left to the partition kernel, which then reads the whole prefill once more).
-constexpr int kFewGather = 4, kManyGather = 8;
+// Warps GW that write the kept-dim rows of the middle from the B boxes, and 16-byte chunks GI per thread and round: as few
+// as hold a stage's items, because the contraction runs at the power cap and idle items and waiting warps cost it clock
+// (32 K tokens: 779 us for six layers with six warps of four items, 751 with four of four, 689 with four of two); eight
+// warps of four where there are more (few pairs per team and many kept dims: every pair writes most rows of its boxes
+// itself; 4 K tokens of the 32-head MHA layout, 48 kept dims: fa_compress 264 us with four warps, 227 with eight, and 320
+// with the rows left to the partition kernel, which then reads the whole prefill once more).
 constexpr int threads_tc(int gw) { return 64 + 32 * (kGenWarps + gw); }
 using namespace umma;
 
@@ -63,15 +62,13 @@ struct RowCuts {
 
 // D = head dim (64 or 128): N = 2 D accumulator columns per KV head (K dims, then V dims); HP heads share the pair
 // and its generated basis tiles (HP * N <= 512 tensor-memory columns).  grid 2 * teams * (M / 256), clusters of two.
-// kGatherWarps: kFewGather or kManyGather (the latter may take several rounds).
 // RAG: rows of different length.
-template <int D, int HP, int kGatherWarps, bool RAG>
+template <int D, int HP, int kGatherWarps, int kItems, bool RAG>
 __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV, Dims s,
                                                                      CacheDev c, int Lall, const __grid_constant__ TeamCuts cuts,
                                                                      const __grid_constant__ RowCuts rows, int per, int gather) {
     constexpr int N = 2 * D;
-    constexpr int kItems = kGatherWarps == kManyGather ? kGatherItems : 2;
     constexpr int kABytes = kBM * kBK * 2;                 // 16 KB basis tile
     constexpr int kBoxBytes = kBK * 64 * 2;                // 8 KB per [64 tokens x 64 dims] box
     constexpr int kBHalf1 = (D / 64) * kBoxBytes;           // this CTA's boxes of one head: all D dims of ONE side
@@ -236,9 +233,9 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
             const int gt = tid - 32 * (2 + kGenWarps);           // 0 .. 32 kGatherWarps - 1
             const int cph = nf_side >> 3;                                      // 16-byte chunks per kept-dim row of this side
             // the pairs of the team load the same boxes and share the tokens: this pair takes rows pair, pair + n_pairs, ...
-            const int rounds = kGatherWarps == kManyGather ? gather_rounds(n_pairs, HP, nf_side, kGatherWarps) : 1, rpr = kBK / rounds;
+            const int rounds = kItems == 4 ? gather_rounds(n_pairs, HP, nf_side, kItems * 32 * kGatherWarps) : 1, rpr = kBK / rounds;
             const int n_tok = pair < rpr ? (rpr - pair + n_pairs - 1) / n_pairs : 0;
-            const int n_items = gather ? n_tok * HP * cph : 0;                // per round, <= kGatherItems per thread
+            const int n_items = gather ? n_tok * HP * cph : 0;                // per round, <= kItems per thread
             const bool p2 = (s.P & (s.P - 1)) == 0;
             const int lgP = 31 - __clz(s.P);
             int it = 0;
@@ -247,7 +244,7 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
             // at the barrier below)
             for (uint32_t pos = pos_begin; pos < pos_end;) {
                 const Seg g = seg_at(pos);
-                // the kept dims of this side of the segment's heads (the four gather warps, on their own barrier)
+                // the kept dims of this side of the segment's heads (the gather warps, on their own barrier)
                 asm volatile("bar.sync 3, %0;" ::"n"(32 * kGatherWarps) : "memory");
                 if (gather)
                     for (int i = gt; i < HP * nf_side; i += 32 * kGatherWarps) {
@@ -501,13 +498,13 @@ bool make_map2(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, int HP, int GW, bool RAG>
+template <int D, int HP, int GW, int GI, bool RAG>
 cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, const RowCuts& rows,
                          bool ordered, bool gather, cudaStream_t stream) {
     constexpr size_t stage = (size_t)kBM * kBK * 2 + (size_t)HP * (D / 64) * kBK * 64 * 2;
     constexpr size_t n_stages = (200 * 1024) / stage < 6 ? (200 * 1024) / stage : 6;
     const size_t smem = n_stages * stage + 8 * (3 * n_stages + 3) + 16 + sizeof(int) * HP * D + 64 + 1024;
-    cudaError_t err = ensure_dynamic_smem(compress_tc2_kernel<D, HP, GW, RAG>, smem);
+    cudaError_t err = ensure_dynamic_smem(compress_tc2_kernel<D, HP, GW, GI, RAG>, smem);
     if (err != cudaSuccess) return err;
     const int n_pairs = s.M / (2 * kBM);
     const int nkb = (mid_of(s, L) + kBK - 1) / kBK;
@@ -546,7 +543,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
             cfg.gridDim = dim3(2 * sm_count());
             cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, compress_tc2_kernel<D, HP, GW, RAG>, &cfg) != cudaSuccess || n < 1) {
+            if (cudaOccupancyMaxActiveClusters(&n, compress_tc2_kernel<D, HP, GW, GI, RAG>, &cfg) != cudaSuccess || n < 1) {
                 cudaGetLastError();
                 n = sm_count() / 2 - 2;
             }
@@ -595,7 +592,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
         cuts.start[n_teams] = (uint32_t)total;
     }
     cfg.gridDim = dim3(2 * n_teams * n_pairs);
-    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW, RAG>, tmK, tmV, s, c, L, cuts, rows, per, gather ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW, GI, RAG>, tmK, tmV, s, c, L, cuts, rows, per, gather ? 1 : 0);
 }
 
 }  // namespace
@@ -628,15 +625,15 @@ cudaError_t launch_compress_tc2(const Dims& s, const CacheDev& c, const void* K,
     if (!make_map2(&tmK, K, s, sb, st, sh, L) || !make_map2(&tmV, V, s, sb, st, sh, L)) return cudaErrorInvalidValue;
     const bool pair = s.Hkv % 2 == 0;                        // two heads share a CTA pair and its basis tiles
     const int nf = s.nfk > s.nfv ? s.nfk : s.nfv;
-    // more than two items to a thread of four warps: the gather would set the pace
-    const int n_pairs = s.M / (2 * kBM), items = (kBK + n_pairs - 1) / n_pairs * (pair ? 2 : 1) * (nf >> 3);
-    const bool many = gather && items > 2 * 32 * kFewGather;
+    const int n_pairs = s.M / (2 * kBM), items = gather ? (kBK + n_pairs - 1) / n_pairs * (pair ? 2 : 1) * (nf >> 3) : 0;
     auto go = [&](auto d, auto hp) {
         if (rows.lens.n)
-            return many ? launch_tc2_t<d, hp, kManyGather, true>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
-                        : launch_tc2_t<d, hp, kFewGather, true>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
-        return many ? launch_tc2_t<d, hp, kManyGather, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
-                    : launch_tc2_t<d, hp, kFewGather, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
+            return items <= 256 ? launch_tc2_t<d, hp, 4, 2, true>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
+                                : launch_tc2_t<d, hp, 8, 4, true>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
+        if (items <= 64) return launch_tc2_t<d, hp, 2, 1, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
+        if (items <= 128) return launch_tc2_t<d, hp, 4, 1, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
+        if (items <= 256) return launch_tc2_t<d, hp, 4, 2, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
+        return launch_tc2_t<d, hp, 8, 4, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
     };
     using std::integral_constant;
     if (s.d == 128) return pair ? go(integral_constant<int, 128>{}, integral_constant<int, 2>{}) : go(integral_constant<int, 128>{}, integral_constant<int, 1>{});
