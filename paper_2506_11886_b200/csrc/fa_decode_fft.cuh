@@ -962,36 +962,55 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             for (int a0 = 0; a0 < n_c; a0 += ts_k) {
                 const int nt = min(ts_k, n_c - a0);
                 const uint32_t tile = wait_tile_u();
+                if (STEP && cb + ci == cstar && astar >= a0 && astar < a0 + nt && wm == ((astar - a0) >> 4) % kMW) {
+                    // fused step: middle token j_pend is not in the cache yet; its kept dims from the row that leaves the window
+                    patch_mid_k(tile + (uint32_t)((astar - a0) * rowb_k), c.idx_full_k + (size_t)h * s.nfk, s.nfk, xrow_s, lane);
+                }
+                // Two groups of the warp at a time, whose loads and products are independent, where registers allow (layer
+                // step at 32 K tokens 35.6 -> 34.0 us, ragged batch 74.7 -> 73.4); one in the two-per-SM and split instances,
+                // which lose 1-2 % to it.
+                constexpr int U = OCC == 1 && !SPLIT ? 2 : 1;
 #pragma unroll 1
-                for (int grp = wm; grp * 16 < nt; grp += kMW) {
+                for (int grp = wm; grp * 16 < nt; grp += U * kMW) {
+                    const bool two = U == 2 && (grp + kMW) * 16 < nt;
                     const uint32_t gbase = tile + (uint32_t)(grp * 16) * rowb_k;
-                    if (STEP && cb + ci == cstar && astar >= a0 + grp * 16 && astar < a0 + grp * 16 + 16) {
-                        // fused step: middle token j_pend is not in the cache yet; its kept dims from the row that leaves the window
-                        patch_mid_k(tile + (uint32_t)((astar - a0) * rowb_k), c.idx_full_k + (size_t)h * s.nfk, s.nfk, xrow_s, lane);
-                    }
-                    float d4[4] = {0.f, 0.f, 0.f, 0.f};
+                    float d4[U][4];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) d4[u][0] = d4[u][1] = d4[u][2] = d4[u][3] = 0.f;
 #pragma unroll
                     for (int rd = 0; rd < 2; ++rd) {
                         if (4 * rd < npk) {
-                            uint4 lo = make_uint4(0, 0, 0, 0), hi = make_uint4(0, 0, 0, 0);
-                            if (k_on[rd]) {
-                                lo = lds128(gbase + k_off[rd]);
-                                hi = lds128(gbase + k_off[rd] + 8 * rowb_k);
+                            uint4 lo[U], hi[U];
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                lo[u] = hi[u] = make_uint4(0, 0, 0, 0);
+                                if (k_on[rd] && (u == 0 || two)) {
+                                    const uint32_t src = gbase + k_off[rd] + (uint32_t)(u * kMW * 16) * rowb_k;
+                                    lo[u] = lds128(src);
+                                    hi[u] = lds128(src + 8 * rowb_k);
+                                }
                             }
-                            mma_bf16(d4, lo.x, hi.x, lo.y, hi.y, qk[rd][0][0], qk[rd][0][1]);
-                            mma_bf16(d4, lo.z, hi.z, lo.w, hi.w, qk[rd][1][0], qk[rd][1][1]);
+#pragma unroll
+                            for (int u = 0; u < U; ++u) mma_bf16(d4[u], lo[u].x, hi[u].x, lo[u].y, hi[u].y, qk[rd][0][0], qk[rd][0][1]);
+#pragma unroll
+                            for (int u = 0; u < U; ++u) mma_bf16(d4[u], lo[u].z, hi[u].z, lo[u].w, hi[u].w, qk[rd][1][0], qk[rd][1][1]);
                         }
                     }
-                    if (cp) {
-                        if (tq == 0) {                      // the head's column, to the slot of this class in its pair
-                            float* dst = kbuf + (((ci >> 1) * S + a0 + grp * 16 + gq) * GH + (ci & 1));
-                            dst[0] = d4[0] * sl2;
-                            dst[8 * GH] = d4[2] * sl2;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        if (u == 1 && !two) break;
+                        const int row = a0 + (grp + u * kMW) * 16;
+                        if (cp) {
+                            if (tq == 0) {                  // the head's column, to the slot of this class in its pair
+                                float* dst = kbuf + (((ci >> 1) * S + row + gq) * GH + (ci & 1));
+                                dst[0] = d4[u][0] * sl2;
+                                dst[8 * GH] = d4[u][2] * sl2;
+                            }
+                        } else if (2 * tq < GH) {
+                            const uint32_t dst = smem_addr(kbuf) + kb_lane_off + (uint32_t)((ci * S + row) * GH) * 4;
+                            sts64(dst, d4[u][0] * sl2, d4[u][1] * sl2);
+                            sts64(dst + 8 * GH * 4, d4[u][2] * sl2, d4[u][3] * sl2);
                         }
-                    } else if (2 * tq < GH) {
-                        const uint32_t dst = smem_addr(kbuf) + kb_lane_off + (uint32_t)((ci * S + a0 + grp * 16) * GH) * 4;
-                        sts64(dst, d4[0] * sl2, d4[1] * sl2);
-                        sts64(dst + 8 * GH * 4, d4[2] * sl2, d4[3] * sl2);
                     }
                 }
                 release_tile();
@@ -1434,12 +1453,11 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     for (int a0 = 0; a0 < n_c; a0 += ts_v) {
                         const int nt = min(ts_v, n_c - a0);
                         const uint32_t tile = wait_tile_u();
+                        if (STEP && cb + ci == cstar && astar >= a0 && astar < a0 + nt && wm == ((astar - a0) >> 4) % kMW)
+                            patch_mid_v(tile + (uint32_t)((astar - a0) * rowb_v), c.idx_full_v + (size_t)h * s.nfv, s.nfv, xrow_s + s.d, astar, lane);
                         #pragma unroll 1
                         for (int grp = wm; grp * 16 < nt; grp += kMW) {
                             const uint32_t gbase = tile + (uint32_t)(grp * 16) * rowb_v;
-                            if (STEP && cb + ci == cstar && astar >= a0 + grp * 16 && astar < a0 + grp * 16 + 16) {
-                                patch_mid_v(tile + (uint32_t)((astar - a0) * rowb_v), c.idx_full_v + (size_t)h * s.nfv, s.nfv, xrow_s + s.d, astar, lane);
-                            }
                             uint32_t b0 = 0, b1 = 0;
                             if (gq < GH) {
                                 b0 = lds32(prow + (uint32_t)(a0 + grp * 16) * 2);
