@@ -189,7 +189,7 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
 /* fa_compress for a batch whose rows have different prompt lengths: row b is compressed from its
  * first lengths[b] tokens (HOST array of B entries, each 0 <= lengths[b] and within the capacity rule
  * of fa_compress; K / V rows beyond a row's length are not read).  Every row becomes what a one-row
- * fa_compress would make of it; fa_append, fa_decode_attention and fa_decode_step then work on the
+ * fa_compress would make of it (coefficients within the same tolerance), in one set of launches for up to 64 rows; fa_append, fa_decode_attention and fa_decode_step then work on the
  * ragged batch as on any other (the token counters are per batch row). */
 fa_status fa_compress_ragged(const fa_layout* layout, fa_cache* cache, const void* K, const void* V,
                              int64_t stride_b, int64_t stride_t, int64_t stride_h, const int32_t* lengths,
@@ -212,14 +212,14 @@ fa_status fa_decode_attention(const fa_layout* layout, const fa_cache* cache, co
 
 /* One decode step with device inputs (Eq.5 then Eq.6): the result and the cache afterwards are those
  * of fa_append(k_new, v_new) followed by fa_decode_attention(q).  Where the decode call is a single
- * fused kernel (see fa_decode_algo), the KV head's query heads fit one pass and a head is spread over
- * at least eight CTAs, the whole step is that ONE launch: every CTA applies the push to its own view of
+ * fused kernel (see fa_decode_algo), the KV head's query heads fit one pass and a CTA has few coefficient
+ * rows to update (at most 260, or a head has at least eight CTAs), the whole step is that ONE launch: every CTA applies the push to its own view of
  * the token counters, the CTA that meets a moved row in a tile (the new token's window row, the kept
  * dims of the row that leaves the local window) patches the tile in shared memory, f_j x^T is added
  * to each coefficient row as the kernel streams it (C^K before forming u, C^V before the output
  * product) and written back, so the coefficients cross the memory bus once per step instead of twice,
  * and the moved rows and the counters are written to the cache once every CTA that reads the old
- * ones is past them.  Otherwise the two calls are made one after the other (with few CTAs per head
+ * ones is past them.  Otherwise the two calls are made one after the other (with many rows per CTA
  * the stand-alone append kernel, which spreads the coefficient update over the whole device, is the
  * faster way).  Same arguments, workspace rule and errors as those two calls (a full middle sets
  * FA_ERR_CAPACITY in cache->status and the step decodes the unchanged cache). */

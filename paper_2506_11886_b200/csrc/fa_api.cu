@@ -709,8 +709,7 @@ static bool step_in_one_launch(const fa_layout& l, const DecodePlan& p) {
     return !p.split && rows <= 260 && (p.n_part >= 2 || l.batch * l.n_kv_heads <= sm_count());
 }
 
-// fa_decode_step.  Where the decode call is the fused kernel with one pass and many parts per head, the push
-// rides on that launch; otherwise the two calls are made one after the other.
+// fa_decode_step.  Where step_in_one_launch says so the push rides on the decode launch; otherwise the two calls are made one after the other.
 static fa_status decode_step_impl(const fa_layout* layout, fa_cache* cache, const void* q, const void* k_new, const void* v_new,
                                   void* out, void* ws, size_t ws_bytes, void* stream) {
     fa_status st = check_layout(layout);
@@ -725,9 +724,7 @@ static fa_status decode_step_impl(const fa_layout* layout, fa_cache* cache, cons
     if (!ws || !aligned16(ws) || ws_bytes < p.total) return FA_ERR_WORKSPACE;
     Dims s = make_dims(*layout);
     // The push rides on the decode launch where a head has many parts (each then updates a small slice of the
-    // coefficient rows as it streams them for u and for the output product).  With few parts per head the
-    // stand-alone append kernel, which spreads the coefficient update over the whole device, is faster
-    // (measured: batch 8 MHA 22 us against 35 us inside the decode kernel, batch 4 at 128K 22 against 64).
+    // coefficient rows as it streams them for u and for the output product).
     // Whether the device can hold all parts at once is asked before anything is enqueued: nothing to undo.
     if (step_in_one_launch(*layout, p) && cooperative_launch_supported() && decode_fft_launchable(s, p)) {
         const cudaError_t err = launch_decode_fft(s, make_cache(*cache), layout->kv_dtype, p, q, out, static_cast<char*>(ws), k_new, v_new,

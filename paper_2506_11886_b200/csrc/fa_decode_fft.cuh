@@ -34,6 +34,13 @@
 // fa_decode_step the fused kernel also adds the pending rank-1 update of Eq.5 to the coefficient
 // rows it stages and writes them back.
 //
+// What bounds it: at batch 1 a chain of some twenty dependent phases, nearly every instruction of which runs once per CTA and
+// is fetched cold, so code size is time (a call of the 32 K-token configuration went from 45.7 to 34.0 us a step with
+// the instance's code, 151 to 124 KB, and the phases that fell away); with several batches per CTA the instruction count of
+// the compressed-dim phases.  Hence: small divisions by idiv, buffer offsets and derived sizes from the host, padded
+// addresses as constants from a first one, one site for every loop that can have one.  HBM is at 20 to 45 % of its
+// measured rate throughout.
+//
 // "Slot" below is the position of a head inside a point / an mma column: slot s holds head
 // hperm(s) = {0, 2, 1, 3}[s] (GH = 4) so that the packed real parts are slots 0, 1 and the
 // packed imaginary parts slots 2, 3.
