@@ -272,10 +272,10 @@ template <int N> __device__ __forceinline__ PC<N> cconj_add(PC<N> a, PC<N> b) { 
 template <int N> __device__ __forceinline__ PC<N> cmulw(PC<N> a, PR<N> wr, PR<N> wi) {
     return PC<N>{(a.re * wr) - (a.im * wi), pfma(a.re, wi, a.im * wr)};
 }
-// a + (the same value of the neighbouring lane)
-__device__ __forceinline__ PR<2> pair_sum(PR<2> a) { PR<2> o; o.v = __shfl_xor_sync(0xffffffffu, a.v, 1); return a + o; }
-__device__ __forceinline__ PR<1> pair_sum(PR<1> a) { return PR<1>{a.v + __shfl_xor_sync(0xffffffffu, a.v, 1)}; }
-template <int N> __device__ __forceinline__ PC<N> pair_sum(PC<N> a) { return PC<N>{pair_sum(a.re), pair_sum(a.im)}; }
+// a + (the same value of the lane at distance d, a power of two)
+__device__ __forceinline__ PR<2> lane_sum(PR<2> a, int d) { PR<2> o; o.v = __shfl_xor_sync(0xffffffffu, a.v, d); return a + o; }
+__device__ __forceinline__ PR<1> lane_sum(PR<1> a, int d) { return PR<1>{a.v + __shfl_xor_sync(0xffffffffu, a.v, d)}; }
+template <int N> __device__ __forceinline__ PC<N> lane_sum(PC<N> a, int d) { return PC<N>{lane_sum(a.re, d), lane_sum(a.im, d)}; }
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -626,7 +626,9 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     constexpr bool step = STEP;
     constexpr int N = GH / 2;
     constexpr int S = 1 << LS;
-    constexpr bool kSplitPairs = S / 2 < kConsumers;      // fewer pairs of bins than threads
+    // Short transforms have fewer pairs of bins than threads: up to 2^kLgPair neighbouring lanes share a pair and take a
+    // share of the batch's classes each.
+    constexpr int kLgPair = LS >= 9 ? 0 : 9 - LS > 4 ? 4 : 9 - LS;
     constexpr int NS = ring_stages(OCC, SPLIT ? 1 : 0);
     // Consumer threads: kAll of them; the warps that consume ring tiles (kept-dim and window products) are all of them,
     // or, in the split kernel, the last six, while the first eight (the transform group) run the compressed-dim phases
@@ -1372,16 +1374,15 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             if (cb == c0) { TL(4); load_u(); }
             // transforms of the batch, and classes from one transform to the next
             const int nbt = cp ? (nb + 1) >> 1 : nb, cstep = cp ? 2 : 1;
+            const int lg_pair = kLgPair == 0 ? 0 : min(kLgPair, 32 - __clz(nbt - 1));     // lanes per pair of bins: no more than classes
 
             // packed Hermitian spectra of the nb classes: X_m = V^A_m + i V^B_m per complex lane,
             // V_m = v_m + conj(v_{S-m}), v_n = (1/2) u~_n e^{i theta n c}.  Pair 0 is bins (0, S/2).
             if (s.dck > 0) {
-                // short transforms: neighbouring lanes share a pair of bins and take half of the classes each
-                const bool split2 = kSplitPairs && nbt > 1;
-                const int hcls = split2 ? (nbt + 1) >> 1 : nbt;
+                const int hcls = (nbt + (1 << lg_pair) - 1) >> lg_pair;
                 #pragma unroll 1
-                for (int item = tid; item < (split2 ? S : S / 2); item += kAll) {
-                    const int pr = split2 ? item >> 1 : item, ci0 = split2 ? (item & 1) * hcls : 0, ci1 = min(nbt, ci0 + hcls);
+                for (int item = tid; item < (S / 2) << lg_pair; item += kAll) {
+                    const int pr = item >> lg_pair, ci0 = (item - (pr << lg_pair)) * hcls, ci1 = min(nbt, ci0 + hcls);
                     const int m = pr, mc = pr == 0 ? S / 2 : S - pr;
                     PC<N> Am = czero, Bm = czero, Ac = czero, Bc = czero;
                     float2 em = make_float2(1.f, 0.f), ec = make_float2(1.f, 0.f);
@@ -1493,11 +1494,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 if constexpr (N == 2) { alA = pk(alpha[0], alpha[1]); alB = pk(alpha[2], alpha[3]); }
                 else { alA = PR<1>{alpha[0]}; alB = PR<1>{alpha[1]}; }
                 const PR<N> half = splat<N>(0.5f);
-                const bool split2 = kSplitPairs && nbt > 1;       // as for the spectra
-                const int hcls = split2 ? (nbt + 1) >> 1 : nbt;
+                const int hcls = (nbt + (1 << lg_pair) - 1) >> lg_pair;
                 #pragma unroll 1
-                for (int item = tid; item < (split2 ? S : S / 2); item += kAll) {       // split: whole warps (S is a multiple of 32)
-                    const int pr = split2 ? item >> 1 : item, ci0 = split2 ? (item & 1) * hcls : 0;
+                for (int item = tid; item < (S / 2) << lg_pair; item += kAll) {       // shared pairs: whole warps (S is a multiple of 32)
+                    const int pr = item >> lg_pair, ci0 = (item - (pr << lg_pair)) * hcls;
                     const int m = pr, mc = pr == 0 ? S / 2 : S - pr;
                     const int ci1 = (m >= s.k && mc >= s.k) ? ci0 : min(nbt, ci0 + hcls);
                     float2 em = make_float2(1.f, 0.f), ec = make_float2(1.f, 0.f);
@@ -1534,9 +1534,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                         twm = cmulf(twm, em);
                         twc = cmulf(twc, ec);
                     }
-                    if (split2) {
-                        zAm = pair_sum(zAm); zBm = pair_sum(zBm); zAc = pair_sum(zAc); zBc = pair_sum(zBc);
-                        if (item & 1) continue;
+                    if constexpr (kLgPair > 0) {
+                        #pragma unroll 1
+                        for (int d = 1; d < 1 << lg_pair; d <<= 1) { zAm = lane_sum(zAm, d); zBm = lane_sum(zBm, d); zAc = lane_sum(zAc, d); zBc = lane_sum(zBc, d); }
+                        if (item != pr << lg_pair) continue;
                     }
                     if (m < s.k) {
                         PC<N> A, B;
@@ -1638,12 +1639,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             // packed Hermitian spectra of the nb classes: X_m = V^A_m + i V^B_m per complex lane,
             // V_m = v_m + conj(v_{S-m}), v_n = (1/2) u~_n e^{i theta n c}.  Pair 0 is bins (0, S/2).
             if (s.dck > 0) {
-                // short transforms: neighbouring lanes share a pair of bins and take half of the classes each
-                const bool split2 = kSplitPairs && nb > 1;
-                const int hcls = split2 ? (nb + 1) >> 1 : nb;
                 #pragma unroll 1
-                for (int item = tid; item < (split2 ? S : S / 2); item += kConsumers) {
-                    const int pr = split2 ? item >> 1 : item, ci0 = split2 ? (item & 1) * hcls : 0, ci1 = min(nb, ci0 + hcls);
+                for (int item = tid; item < S / 2; item += kConsumers) {
+                    constexpr int ci0 = 0;
+                    const int pr = item, ci1 = nb;
                     const int m = pr, mc = pr == 0 ? S / 2 : S - pr;
                     PC<N> Am = czero, Bm = czero, Ac = czero, Bc = czero;
                     float2 em = make_float2(1.f, 0.f), ec = make_float2(1.f, 0.f);
@@ -1710,13 +1709,12 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 if constexpr (N == 2) { alA = pk(alpha[0], alpha[1]); alB = pk(alpha[2], alpha[3]); }
                 else { alA = PR<1>{alpha[0]}; alB = PR<1>{alpha[1]}; }
                 const PR<N> half = splat<N>(0.5f);
-                const bool split2 = kSplitPairs && nb > 1;        // as for the spectra
-                const int hcls = split2 ? (nb + 1) >> 1 : nb;
                 #pragma unroll 1
-                for (int item = tid; item < (split2 ? S : S / 2); item += kConsumers) {       // split: whole warps (S is a multiple of 32)
-                    const int pr = split2 ? item >> 1 : item, ci0 = split2 ? (item & 1) * hcls : 0;
+                for (int item = tid; item < S / 2; item += kConsumers) {
+                    constexpr int ci0 = 0;
+                    const int pr = item;
                     const int m = pr, mc = pr == 0 ? S / 2 : S - pr;
-                    const int ci1 = (m >= s.k && mc >= s.k) ? ci0 : min(nb, ci0 + hcls);
+                    const int ci1 = (m >= s.k && mc >= s.k) ? 0 : nb;
                     float2 em = make_float2(1.f, 0.f), ec = make_float2(1.f, 0.f);
                     if (m < s.k) em = E[m];
                     if (mc < s.k) ec = E[mc];
@@ -1746,10 +1744,6 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                         }
                         twm = cmulf(twm, em);
                         twc = cmulf(twc, ec);
-                    }
-                    if (split2) {
-                        zAm = pair_sum(zAm); zBm = pair_sum(zBm); zAc = pair_sum(zAc); zBc = pair_sum(zBc);
-                        if (item & 1) continue;
                     }
                     if (m < s.k) {
                         PC<N> A, B;

@@ -65,3 +65,21 @@ def test_direct_decode_tiles_of_tokens(kw, P, dtype):
     pair.check_state()
     pair.check_decode(synth.queries(shape, seed=9))
     pair.check_decode(synth.queries(shape, seed=9, step=1, peak=6.0))
+
+
+@pytest.mark.parametrize("Hq,Hkv,B,S,k", [
+    (4, 1, 40, 32, 32),      # sixteen lanes to a pair of bins, every class of a head in one batch
+    (4, 1, 40, 64, 20),      # fewer frequencies than bins
+    (2, 1, 70, 32, 16),      # two heads to a point
+    (1, 1, 130, 32, 32),     # one query head: two classes to a transform
+    (3, 1, 3, 128, 128),     # an odd number of classes, three heads in four slots
+])
+def test_decode_short_transforms_many_classes_in_a_batch(Hq, Hkv, B, S, k):
+    shape = synth.Shape("short", B=B, layers=1, Hq=Hq, Hkv=Hkv, d=64, L=S * 32 - 5, dtype="bf16", n_full_k=16, n_full_v=24, M=2 * k,
+                        T=S * 32, L_init=3, L_local=20, decode_steps=2)
+    pair, stream = make_pair(shape, seed=12, P=32, algo=fa.FA_DECODE_FFT, max_mid=shape.T, freq="offgrid")
+    pair.check_decode(synth.queries(shape, seed=12))
+    K, V = stream.tokens(shape.L, shape.L + 2)
+    for t in range(2):
+        pair.check_step(synth.queries(shape, seed=12, step=t + 1, peak=3.0), K[:, t], V[:, t])
+    pair.check_state()
