@@ -125,8 +125,9 @@ typedef struct fa_cache_sizes {
 /* Host only.  Checks the layout and fills *out.  INVALID_ARG / UNSUPPORTED on a bad layout. */
 fa_status fa_cache_sizes_of(const fa_layout* layout, fa_cache_sizes* out);
 
-/* Host only.  Bytes of workspace fa_decode_attention and fa_compress need for this layout
- * (the larger of the two).  The workspace is scratch whose contents need not survive
+/* Host only.  Bytes of workspace fa_decode_attention needs and, behind them, fa_compress makes use of for this layout
+ * (the latter's share is at most 192 MiB, or what one batch row takes).  Calls of one kind that may overlap on the GPU
+ * need workspaces of their own.  The workspace is scratch whose contents need not survive
  * between calls, with one rule: its first 4 KiB hold barrier counters that must be zero
  * when a call starts.  Zero-fill a new workspace once (cudaMemset); every call that ends
  * without FA_ERR_TIMEOUT leaves the counters at zero again.  After FA_ERR_TIMEOUT
@@ -150,7 +151,10 @@ fa_status fa_validate(const fa_layout* layout, const fa_cache* cache, void* stre
  * layout->kv_dtype.  Overwrites the whole cache: windows, K^mu / V^mu, coefficients
  * (basis column j = t - n_init for middle token t) and state.  n_init = min(L, l_init),
  * n_local = min(L - n_init, l_local), the rest is the middle.  FA_ERR_CAPACITY (host side)
- * if the middle exceeds max_mid.  ws / ws_bytes: workspace as sized by fa_workspace_bytes. */
+ * if the middle exceeds max_mid.  ws / ws_bytes: workspace as sized by fa_workspace_bytes.  bf16 caches with n_coef a multiple
+ * of 256 and period / n_coef >= 16 are compressed by way of block moments, which are kept there between two kernels (groups
+ * of batch rows take turns where the workspace does not hold all); with a smaller workspace, or none, the coefficients
+ * are contracted over the tokens directly, slower and with the basis rounded to bf16. */
 fa_status fa_compress(const fa_layout* layout, fa_cache* cache, const void* K, const void* V,
                       int64_t stride_b, int64_t stride_t, int64_t stride_h, int32_t L,
                       void* ws, size_t ws_bytes, void* stream);
@@ -283,7 +287,7 @@ fa_status fa_select_dims(const fa_layout* layout, const void* K, const void* V, 
  * fa_static_workspace_limit() bytes (8 MiB) built into the library; each GPU that loads the
  * library holds it until the process exits.  No call made here allocates or frees.
  *   - q, out, cache: exactly as for fa_decode_attention; the result is the same.
- *   - Layouts whose fa_workspace_bytes exceeds the limit are refused with FA_ERR_WORKSPACE
+ *   - Layouts whose decode call needs more scratch than the limit are refused with FA_ERR_WORKSPACE
  *     before anything runs; use fa_decode_attention with your own workspace for those.
  *   - The first call on each device looks the array's device address up (with that device
  *     current); make that first call before any stream capture.

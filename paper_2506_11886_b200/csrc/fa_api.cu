@@ -330,6 +330,62 @@ static fa_status check_cache(const fa_layout* l, const fa_cache* c) {
     return FA_OK;
 }
 
+fa_status decode_scratch_bytes(const fa_layout* layout, size_t* out) {
+    fa_status st = check_layout(layout);
+    if (st != FA_OK) return st;
+    if (!out) return FA_ERR_INVALID_ARG;
+    DecodePlan p;
+    st = plan_decode(*layout, &p);
+    if (st != FA_OK) return st;
+    *out = p.total;
+    if (p.fused) {                       // room for the three-kernel form too, should a cooperative launch not fit
+        fa_layout split = *layout;
+        split.decode_algo = FA_DECODE_FFT_SPLIT;
+        DecodePlan p2;
+        if (plan_decode(split, &p2) == FA_OK && p2.total > *out) *out = p2.total;
+    }
+    return FA_OK;
+}
+
+// Scratch of the compression by block moments: behind that of the decode call (a decode step may run on another stream while a
+// prompt is compressed), in two halves (neighbouring launches alternate between them), each for as many batch rows as
+// kMomScratch holds (at least one).
+constexpr size_t kMomScratch = size_t(192) << 20;
+static size_t compress_scratch_bytes(const fa_layout& l) {
+    const Dims s = make_dims(l);
+    if (l.kv_dtype != FA_BF16 || !compress_tc_supported(s, l.kv_dtype, 0, 8, 8) || !compress_mom_supported(s)) return 0;
+    const size_t row = compress_mom_row_bytes(s, s.max_mid);
+    if (row == 0) return 0;
+    size_t rows = kMomScratch / row;
+    if (rows < 1) rows = 1;
+    if (rows > 2 * (size_t)s.B) rows = 2 * (size_t)s.B;
+    return rows * row;
+}
+// Where the moments of a call go and how many bytes there are (0: the direct contraction).
+struct MomentRoom { char* at; size_t bytes; };
+static MomentRoom moment_room(const fa_layout& l, void* ws, size_t ws_bytes) {
+    size_t decode = 0;
+    if (!ws || !aligned16(ws) || !compress_mom_supported(make_dims(l)) || decode_scratch_bytes(&l, &decode) != FA_OK) return {nullptr, 0};
+    decode = align_up(decode, 256);
+    return ws_bytes > decode ? MomentRoom{static_cast<char*>(ws) + decode, ws_bytes - decode} : MomentRoom{nullptr, 0};
+}
+// The two kernels of the block-moment path over all batch rows: all at once, or in groups that take half of the room in turn
+// (one row at least fits).
+static cudaError_t compress_by_moments(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int L,
+                                       MomentRoom room, cudaStream_t stream, const RowLens* lens = nullptr, int tc_min = 1) {
+    int n_mid = lens ? 0 : mid_of(s, L);
+    for (int b = 0; lens && b < s.B; ++b) n_mid = mid_of(s, lens->len[b]) > n_mid ? mid_of(s, lens->len[b]) : n_mid;
+    const size_t row = compress_mom_row_bytes(s, n_mid), fit = room.bytes / row;
+    const int group = fit >= (size_t)s.B ? s.B : fit >= 2 ? (int)(fit / 2) : 1;
+    for (int b0 = 0, i = 0; b0 < s.B; b0 += group, ++i) {
+        const int nb = s.B - b0 < group ? s.B - b0 : group;
+        char* Y = room.at + (fit >= 2 && (i & 1) ? (size_t)group * row : 0);
+        const cudaError_t err = launch_compress_mom(s, c, K, V, sb, st, sh, L, b0, nb, Y, fit < 2 && i > 0, stream, lens, tc_min);
+        if (err != cudaSuccess) return err;
+    }
+    return cudaSuccess;
+}
+
 }  // namespace fa
 
 using namespace fa;
@@ -359,19 +415,9 @@ fa_status fa_cache_sizes_of(const fa_layout* layout, fa_cache_sizes* out) {
 }
 
 fa_status fa_workspace_bytes(const fa_layout* layout, size_t* out) {
-    fa_status st = check_layout(layout);
+    fa_status st = decode_scratch_bytes(layout, out);
     if (st != FA_OK) return st;
-    if (!out) return FA_ERR_INVALID_ARG;
-    DecodePlan p;
-    st = plan_decode(*layout, &p);
-    if (st != FA_OK) return st;
-    *out = p.total;
-    if (p.fused) {                       // room for the three-kernel form too, should a cooperative launch not fit
-        fa_layout split = *layout;
-        split.decode_algo = FA_DECODE_FFT_SPLIT;
-        DecodePlan p2;
-        if (plan_decode(split, &p2) == FA_OK && p2.total > *out) *out = p2.total;
-    }
+    *out = align_up(*out, 256) + compress_scratch_bytes(*layout);
     return FA_OK;
 }
 
@@ -419,7 +465,6 @@ fa_status fa_validate(const fa_layout* layout, const fa_cache* cache, void* stre
 
 fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K, const void* V, int64_t stride_b,
                          int64_t stride_t, int64_t stride_h, int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream) {
-    (void)ws; (void)ws_bytes;
     fa_status st = check_layout(layout);
     if (st != FA_OK) return st;
     st = check_cache(layout, cache);
@@ -453,6 +498,14 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
     }
     const int n_mid_host = L - n_init - n_local;
     const bool tc = L > 0 && n_mid_host >= kTcMinMid && compress_tc_supported(s, layout->kv_dtype, sbb, stride_t, stride_h);
+    // block moments where the workspace has room for them; the order-fixed mode keeps the direct contraction
+    const MomentRoom room = tc && !ordered ? moment_room(*layout, ws, ws_bytes) : MomentRoom{nullptr, 0};
+    if (room.at && room.bytes >= compress_mom_row_bytes(s, n_mid_host)) {
+        if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, false, false, kTcMinMid, true, cs) != cudaSuccess)
+            return FA_ERR_CUDA;
+        if (compress_by_moments(s, make_cache(*cache), K, V, sbb, stride_t, stride_h, L, room, cs) == cudaSuccess) return FA_OK;
+        cudaGetLastError();                                 // the cluster launch was refused: everything below once more
+    }
     // tensor-core path: its kernel also writes the kept-dim rows of the middle from the boxes it loads; the partition
     // kernel is left with the windows and the counters
     bool tc2 = tc && compress_tc2_supported(s);             // CTA pairs where the row tiles pair up
@@ -532,6 +585,22 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
     // leave, and wait for layer i (hence for everything before it) only in front of their reductions.
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const bool ordered = (flags & FA_COMPRESS_ORDERED) != 0;
+    // Block moments where every layer's fit the workspace: two halves where it has them, so that a layer's moments are formed
+    // while the layer's before are still read.
+    size_t half = 0;
+    bool moments = !ordered;
+    MomentRoom room = {nullptr, ~size_t(0)};
+    for (int i = 0; i < n_layers && moments; ++i) {
+        const Dims s = make_dims(layouts[i]);
+        const MomentRoom r = moment_room(layouts[i], ws, ws_bytes);
+        moments = r.at != nullptr;
+        if (!moments) break;
+        if (r.bytes < room.bytes) room = r;                // (the layer with the largest decode scratch leaves the least)
+        const size_t need = (size_t)s.B * compress_mom_row_bytes(s, mid_of(s, L));
+        half = need > half ? need : half;
+    }
+    moments = moments && room.bytes >= half;
+    const bool two = moments && room.bytes >= 2 * half;
     for (int i = 0; i < n_layers; ++i) {
         const Dims s = make_dims(layouts[i]);
         if (launch_compress(s, make_cache(caches[i]), layouts[i].kv_dtype, K[i], V[i], stride_b, stride_t, stride_h, L, false, ordered, kTcMinMid,
@@ -541,7 +610,9 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
     for (int i = 0; i < n_layers; ++i) {
         const Dims s = make_dims(layouts[i]);
         const int64_t sbb = s.B > 1 ? stride_b : 0;
-        if (launch_compress_tc2(s, make_cache(caches[i]), K[i], V[i], sbb, stride_t, stride_h, L, ordered, true, cs) != cudaSuccess) {
+        char* Y = moments ? room.at + (two && (i & 1) ? half : 0) : nullptr;
+        if ((moments ? launch_compress_mom(s, make_cache(caches[i]), K[i], V[i], sbb, stride_t, stride_h, L, 0, s.B, Y, !two && i > 0, cs)
+                     : launch_compress_tc2(s, make_cache(caches[i]), K[i], V[i], sbb, stride_t, stride_h, L, ordered, true, cs)) != cudaSuccess) {
             // the cluster launch was refused: finish this and the remaining layers one by one (each call redoes its layer in full)
             cudaGetLastError();
             for (int j = i; j < n_layers; ++j) {
@@ -632,6 +703,16 @@ fa_status fa_compress_ragged(const fa_layout* layout, fa_cache* cache, const voi
             if (launch_compress(s, make_cache(rows), layout->kv_dtype, Kb, Vb, stride_b, stride_t, stride_h, L, true, false,
                                 tc ? kTcMinMid : kNoTc, true, cs, false, &lens) != cudaSuccess)
                 return FA_ERR_CUDA;
+            int n_mid = 0;
+            for (int i = 0; i < part.batch; ++i) n_mid = mid_of(s, lens.len[i]) > n_mid ? mid_of(s, lens.len[i]) : n_mid;
+            const MomentRoom room = tc ? moment_room(*layout, ws, ws_bytes) : MomentRoom{nullptr, 0};
+            if (room.at && room.bytes >= compress_mom_row_bytes(s, n_mid)) {
+                if (compress_by_moments(s, make_cache(rows), Kb, Vb, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, room, cs, &lens,
+                                        kTcMinMid) == cudaSuccess)
+                    continue;
+                cudaGetLastError();                       // the cluster launch was refused: these rows and the rest one by one
+                break;
+            }
             if (tc && launch_compress_tc2(s, make_cache(rows), Kb, Vb, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, false, true, cs, &lens,
                                           kTcMinMid) != cudaSuccess) {
                 cudaGetLastError();                       // the cluster launch was refused: these rows and the rest one by one

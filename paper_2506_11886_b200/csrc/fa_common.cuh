@@ -96,6 +96,7 @@ __host__ __device__ inline int v_mid_col(int a, int e, int nfv, int dtype) {
 }
 
 fa_status plan_decode(const fa_layout& l, DecodePlan* plan);
+fa_status decode_scratch_bytes(const fa_layout* layout, size_t* out);      // what fa_decode_attention needs of a workspace
 int sm_count();                          // SMs of the current device, cached per device
 bool cooperative_launch_supported();     // of the current device, cached per device
 fa_status check_layout(const fa_layout* l);
@@ -125,6 +126,11 @@ bool compress_tc_gathers(const Dims& s);
 bool compress_tc2_supported(const Dims& s);
 cudaError_t launch_compress_tc2(const Dims&, const CacheDev&, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh,
                                 int L, bool ordered, bool gather, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
+// The contraction by block moments (fa_compress_mom.cu): batch rows b0 .. b0 + nb, moments in Y.
+bool compress_mom_supported(const Dims& s);
+size_t compress_mom_row_bytes(const Dims& s, int n_mid);
+cudaError_t launch_compress_mom(const Dims&, const CacheDev&, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int L, int b0,
+                                int nb, void* Y, bool wait_first, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
 // Tensor-core reconstruction of the dimension selection (fa_select_tc.cu).
 bool reconstruct_tc_supported(const Dims& s, int dtype, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int n_mid);
 size_t reconstruct_tc_scratch_bytes(const Dims& s);

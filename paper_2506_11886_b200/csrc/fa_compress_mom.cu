@@ -1,0 +1,865 @@
+// fa_compress, block-moment path (Eq.3-4; bf16 caches, sm_100a): the projection on the basis in two contractions, the
+// second of them over an axis that is R / 32 times shorter than the token axis.
+//
+// Within a block of R tokens the basis functions of Eq.4 are band-limited: with t in [-1, 1] across the block and
+// phi_n = theta n R / 2 (theta = 2 pi / T) the plane-wave expansion in Legendre polynomials,
+//   e^{i phi t} = sum_r (2 r + 1) i^r j_r(phi) P_r(t)          (j_r: spherical Bessel functions),
+// falls off faster than exponentially beyond r = phi.  R is at most 6 T / k, so phi <= 6 pi, and 32 terms leave at most
+// 4e-5 at the very edge of band and block (1e-6 of the sums' norm).  Hence
+//   C_n = sum_j x_j e^{i theta n j} = sum_blocks e^{i theta n center} sum_{r < 32} (2 r + 1) i^r j_r(phi_n) Y_{block, r}
+//   Y_{block, r} = sum_{t in block} P_r(t) x_t                   (the block's moments).
+//   1. moments_kernel: one pass over the prefill.  Boxes of 64 tokens come in by TMA; the tensor cores multiply them with
+//      P (as bf16 hi + lo: exact to 2^-17; x is bf16 already), the gather warps write the kept-dim rows of the middle from
+//      the same boxes, the epilogue warps write the moments of the compressed dims, again as bf16 hi + lo.
+//   2. moment_project_kernel: C += G Y on CTA pairs (tcgen05.mma.cta_group::2), G generated from exact integer phases
+//      and 32 Bessel factors per frequency; three products hi hi, lo hi, hi lo.
+// Both factors carry 2^-17, where the contraction over tokens rounds its basis to bf16 (2^-9).
+//
+// What bounds it: the first kernel HBM (per box of 64 tokens of one side 740 to 840 cycles against the 700 that 16 KB take at an SM's
+// share of the measured rate; its write of the moments is 10 % of the traffic at k / T = 1 / 64 and 20 % at 1 / 32), the
+// second the tensor cores (1200 cycles a block and pair against 1152 for its products) plus 8 K cycles of reductions per segment.
+// Direct contraction against this path: six layers of 32 K tokens, 1024 rows: 701 -> 374 us; 128 K tokens, batch 4, 2048 rows:
+// 3207 -> 778 us; six ragged rows of 3 to 12 K tokens, 512 rows: 123 -> 85 us; 4 K tokens of 256 heads, 256 rows (T / k = 32, blocks of
+// 192 tokens): 231 -> 221 us.  Relative error of the coefficients 4e-6 against 2.4e-4.
+#include <mutex>
+#include <type_traits>
+
+#include "fa_umma.cuh"
+
+namespace fa {
+namespace {
+
+using bf16 = __nv_bfloat16;
+using namespace umma;
+
+constexpr int kMF = 32;              // moments per block
+constexpr int kChunk = 64;           // tokens per box and pipeline stage
+constexpr int kChunkBytes = 128 * kChunk * 2;      // [64 tokens x 64 dims] twice
+constexpr int kHChunk = 2 * kMF * kChunk * 2;      // P of 64 tokens, hi and lo rows
+constexpr int kAcc = 8;              // accumulators (64 columns each) in tensor memory
+constexpr int kEpiWarps = 4, kGathWarps = 8;
+constexpr int kThreadsMom = 32 * (2 + kEpiWarps + kGathWarps);
+constexpr int kMaxBlockTokens = 768;
+
+__device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x - __uint_as_float(hi << 16), y - __uint_as_float(hi & 0xffff0000u));
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+    uint16_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// Blocks of a launch: batch rows b0 .. b0 + nb of the call; row b owns blocks first[b] .. first[b + 1] of the launch
+// (lens.n = 0: nblk each, and first is not used).  R tokens to a block.
+struct MomRows {
+    int R, nblk, b0, nb, total;
+    RowLens lens;
+    uint32_t first[kMaxRagged + 1];
+};
+
+// Item = (block, KV head[, side]): D = 128: one side's 128 dims, D = 64: K dims and V dims side by side.  A persistent CTA
+// takes items blockIdx.x, blockIdx.x + gridDim.x, ...: CTAs that run together read the same tokens' heads.
+template <int D, bool RAG>
+__global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                                                                 Dims s, CacheDev c, int Lall, const __grid_constant__ MomRows rows, bf16* __restrict__ Y,
+                                                                 int n_stages, int n_items, int wait_first) {
+    constexpr int kSides = D == 128 ? 2 : 1;               // items per (block, head)
+    // A: 64-dim rows of a token, MN-major; B: P, K-major; M = 128 dims, N = 64 (hi and lo rows of P)
+    constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(2 * kMF >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    extern __shared__ unsigned char smem_unaligned[];
+    unsigned char* smem = smem_unaligned + ((1024u - (smem_u32(smem_unaligned) & 1023u)) & 1023u);
+    unsigned char* stage0 = smem;
+    const int n_chunk = rows.R / kChunk;
+    unsigned char* Hs = stage0 + (size_t)n_stages * kChunkBytes;
+    unsigned char* y_s = Hs + (size_t)n_chunk * kHChunk;   // [128 columns][128 bytes] moments of an item on their way out
+    uint64_t* full = reinterpret_cast<uint64_t*>(y_s + 128 * 4 * kMF);
+    uint64_t* empty = full + n_stages;
+    uint64_t* acc_full = empty + n_stages;
+    uint64_t* acc_empty = acc_full + kAcc;
+    uint64_t* masked = acc_empty + kAcc;                   // per stage: rows past the end of a batch row's last box are zero
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(masked + n_stages);
+    volatile int* fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    uint8_t* inv_s = reinterpret_cast<uint8_t*>(tmem_slot + 2);      // [Hkv][2][D] position of a dim among the compressed ones, 255: kept
+    uint8_t* idf_s = inv_s + s.Hkv * 2 * D;                          // [Hkv][nfk + nfv] the kept dims
+    const int nf = s.nfk + s.nfv;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (tid == 0) {
+        for (int i = 0; i < n_stages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1 + kGathWarps); mbar_init(masked + i, kGathWarps); }
+        for (int i = 0; i < kAcc; ++i) { mbar_init(acc_full + i, 1); mbar_init(acc_empty + i, kEpiWarps); }
+        *fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp > 0) {                                        // (the producer's boxes set off meanwhile)
+        constexpr int kW = kThreadsMom / 32 - 1;
+        const int u = tid - 32, wu = warp - 1;
+        // where a dim is: a warp takes whole rows (head, side)
+        for (int r = wu; r < 2 * s.Hkv; r += kW) {
+            const int h = r >> 1, sd = r & 1, nfr = sd ? s.nfv : s.nfk, ncr = D - nfr;
+            const int32_t* idf = (sd ? c.idx_full_v : c.idx_full_k) + h * nfr;
+            const int32_t* idc = (sd ? c.idx_comp_v : c.idx_comp_k) + h * ncr;
+            uint8_t* inv = inv_s + r * D;
+#pragma unroll
+            for (int e0 = 0; e0 < D; e0 += 32) {
+                const int e = e0 + lane;
+                const int d = e < nfr ? idf[e] : idc[e - nfr];
+                if (e < nfr) idf_s[h * nf + (sd ? s.nfk : 0) + e] = (uint8_t)d;
+                inv[d] = e < nfr ? 255 : (uint8_t)(e - nfr);
+            }
+        }
+        // the polynomials, by their recurrence, one token per thread
+        for (int t = u; t < rows.R; t += 32 * kW) {
+            const float x = (float)(2 * t + 1 - rows.R) / (float)rows.R;
+            unsigned char* hq = Hs + (t >> 6) * kHChunk;
+            const int tok = t & 63;
+            float p0 = 1.f, p1 = x;
+#pragma unroll
+            for (int r = 0; r < kMF; ++r) {
+                const bf16 hi = __float2bfloat16_rn(p0), lo = __float2bfloat16_rn(p0 - __bfloat162float(hi));
+                unsigned char* at = hq + (r >> 3) * 1024 + (r & 7) * 128 + (((tok >> 3) ^ (r & 7)) << 4) + (tok & 7) * 2;
+                *reinterpret_cast<bf16*>(at) = hi;
+                *reinterpret_cast<bf16*>(at + (kMF >> 3) * 1024) = lo;
+                const float p2 = ((float)(2 * r + 3) * x * p1 - (float)(r + 1) * p0) * (1.0f / (float)(r + 2));
+                p0 = p1;
+                p1 = p2;
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P is read by the tensor cores
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kW) : "memory");
+    }
+    const uint32_t tmem_base = *tmem_slot;
+
+    // A role's place in the CTA's items: the next item is gridDim.x further on, taken by additions with carries.
+    const int n_mid_all = mid_of(s, Lall);
+    struct Walk { int i, side, h, gblk, b, blk, nblk, n_mid, n_ch; };
+    const int d_side = kSides == 2 ? (int)gridDim.x & 1 : 0, d_t = kSides == 2 ? (int)gridDim.x >> 1 : (int)gridDim.x;
+    const int d_blk = d_t / s.Hkv, d_h = d_t - d_blk * s.Hkv;
+    auto settle = [&](Walk& w) {                           // block number -> batch row and block of the row
+        if (w.i >= n_items) return;
+        while (w.blk >= w.nblk) {
+            w.blk -= w.nblk;
+            ++w.b;
+            if (RAG) w.nblk = (int)(rows.first[w.b + 1] - rows.first[w.b]);
+        }
+        if (RAG) w.n_mid = mid_of(s, rows.lens.len[w.b]);
+        w.n_ch = min(n_chunk, (w.n_mid - w.blk * rows.R + kChunk - 1) / kChunk);
+    };
+    auto walk_begin = [&]() {
+        Walk w;
+        w.i = blockIdx.x;
+        const int t = kSides == 2 ? w.i >> 1 : w.i;
+        w.side = kSides == 2 ? w.i & 1 : 0;
+        w.gblk = t / s.Hkv;
+        w.h = t - w.gblk * s.Hkv;
+        w.blk = w.gblk;
+        w.b = RAG ? 0 : rows.b0;
+        w.nblk = RAG ? (int)rows.first[1] : rows.nblk;
+        w.n_mid = n_mid_all;
+        w.n_ch = 0;
+        settle(w);
+        return w;
+    };
+    auto walk_next = [&](Walk& w) {
+        w.i += gridDim.x;
+        w.side += d_side;
+        int c1 = 0;
+        if (w.side >= 2) { w.side -= 2; c1 = 1; }
+        w.h += d_h + c1;
+        int c2 = 0;
+        if (w.h >= s.Hkv) { w.h -= s.Hkv; c2 = 1; }
+        w.gblk += d_blk + c2;
+        w.blk += d_blk + c2;
+        settle(w);
+    };
+
+    if (warp == 0) {
+        // ---------------- TMA producer ----------------
+        if (lane == 0) {
+            int st = 0, issued = 0;
+            uint32_t par = 1;
+            bool live = true;
+            for (Walk it = walk_begin(); live && it.i < n_items; walk_next(it)) {
+                int tok = s.l_init + it.blk * rows.R;
+                for (int q = 0; q < it.n_ch; ++q, tok += kChunk) {
+                    if (!mbar_wait(empty + st, par, fail, c.status)) { live = false; break; }
+                    unsigned char* dst = stage0 + (size_t)st * kChunkBytes;
+                    mbar_expect_tx(full + st, (uint32_t)kChunkBytes);
+                    if (kSides == 2) {
+                        const CUtensorMap* tm = it.side ? &tmV : &tmK;
+                        tma_load_4d(dst, tm, 0, it.h, tok, it.b, full + st);
+                        tma_load_4d(dst + kChunkBytes / 2, tm, 64, it.h, tok, it.b, full + st);
+                    } else {
+                        tma_load_4d(dst, &tmK, 0, it.h, tok, it.b, full + st);
+                        tma_load_4d(dst + kChunkBytes / 2, &tmV, 0, it.h, tok, it.b, full + st);
+                    }
+                    ++issued;
+                    if (++st == n_stages) { st = 0; par ^= 1; }
+                }
+            }
+            if (!live)                                     // a wait ran out: the boxes still under way land before the CTA ends
+                for (int q = issued - n_stages < 0 ? 0 : issued - n_stages; q < issued; ++q)
+                    for (uint32_t n = 0; n < (1u << 20) && !mbar_try_wait(full + q % n_stages, (uint32_t)(q / n_stages) & 1u); ++n) { }
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: moments[dim][hi rows | lo rows] of a block ----------------
+        if (lane == 0) {
+            int st = 0, a = 0;
+            uint32_t par = 0, mpar = 0;
+            bool live = true;
+            // descriptors with the addresses of stage 0 and box 0 of P (in units of 16 bytes; the sums stay below the field's end)
+            const uint64_t xdesc0 = umma_desc(smem_u32(stage0), (kChunkBytes / 2) >> 4, 1024 >> 4), hdesc0 = umma_desc(smem_u32(Hs), 1, 1024 >> 4);
+            for (Walk it = walk_begin(); live && it.i < n_items; walk_next(it), ++a) {
+                const int ab = a % kAcc;
+                if (a >= kAcc && !mbar_wait(acc_empty + ab, ((a / kAcc) - 1) & 1, fail, c.status)) break;
+                const uint32_t acc = tmem_base + ab * (2 * kMF);
+                uint64_t hdesc = hdesc0;
+                int left = it.n_mid - it.blk * rows.R;
+                for (int q = 0; q < it.n_ch; ++q, left -= kChunk, hdesc += kHChunk >> 4) {
+                    if (!mbar_wait(full + st, par, fail, c.status)) { live = false; break; }
+                    if (left < kChunk) {
+                        if (!mbar_wait(masked + st, (mpar >> st) & 1u, fail, c.status)) { live = false; break; }
+                        mpar ^= 1u << st;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint64_t xdesc = xdesc0 + (uint64_t)(st * (kChunkBytes >> 4));
+#pragma unroll
+                    for (int ks = 0; ks < kChunk / 16; ++ks)
+                        umma_bf16(acc, xdesc + ks * (2048 >> 4), hdesc + ks * 2, kIdesc, (q > 0 || ks > 0) ? 1u : 0u);
+                    umma_commit(empty + st);
+                    if (++st == n_stages) { st = 0; par ^= 1; }
+                }
+                if (live) umma_commit(acc_full + ab);
+            }
+        }
+    } else if (warp < 2 + kEpiWarps) {
+        // ---------------- epilogue: moments of the compressed dims, bf16 hi then lo, 128 bytes per (block, column) ----------------
+        if (wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");   // Y may still be read by the kernel before this one
+        const int lg = warp & 3, e = lg * 32 + lane;       // tensor-memory lane: the dim, or (D = 64) K's dims then V's
+        const int ncol = s.dck + s.dcv;
+        int a = 0;
+        for (Walk it = walk_begin(); it.i < n_items; walk_next(it), ++a) {
+            const int ab = a % kAcc;
+            if (!mbar_wait(acc_full + ab, (a / kAcc) & 1, fail, c.status)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            float y[kMF], y2[kMF];
+            tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(ab * 2 * kMF), y);
+            tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(ab * 2 * kMF + kMF), y2);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty + ab);
+            const int side = kSides == 2 ? it.side : e >> 6, dim = kSides == 2 ? e : e & 63;
+            const int pos = inv_s[(it.h * 2 + side) * D + dim];
+            // The columns of the item are one contiguous run of rows of Y: they are put together in shared memory and leave with one
+            // bulk copy (stored by the lanes, every 16 bytes went to a line of its own).  The 16-byte pieces of a row are
+            // permuted as the 128-byte swizzle of the products' operand wants them, so the second kernel copies rows as they are.
+            if (warp == 2 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the copy before has read the buffer
+            asm volatile("bar.sync 2, %0;" ::"n"(32 * kEpiWarps) : "memory");
+            if (pos != 255) {
+                const int col = (kSides == 1 && side ? s.dck : 0) + pos;
+                unsigned char* dst = y_s + col * (4 * kMF);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    uint32_t hi[4], lo[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) split_bf16(y[8 * r + 2 * u] + y2[8 * r + 2 * u], y[8 * r + 2 * u + 1] + y2[8 * r + 2 * u + 1], hi[u], lo[u]);
+                    *reinterpret_cast<uint4*>(dst + ((r ^ (col & 7)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                    *reinterpret_cast<uint4*>(dst + (((4 + r) ^ (col & 7)) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("bar.sync 2, %0;" ::"n"(32 * kEpiWarps) : "memory");
+            if (warp == 2 && lane == 0) {
+                const int c0 = kSides == 2 && it.side ? s.dck : 0, nc = kSides == 1 ? ncol : it.side ? s.dcv : s.dck;
+                char* dst = reinterpret_cast<char*>(Y) + (((size_t)it.gblk * s.Hkv + it.h) * ncol + c0) * (size_t)(4 * kMF);
+                if (nc > 0)
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(dst)), "r"(smem_u32(y_s)),
+                                 "r"(nc * (4 * kMF))
+                                 : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+        }
+        if (warp == 2 && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        asm volatile("griddepcontrol.wait;" ::: "memory"); // the end of this grid implies the end of the one before
+    } else {
+        // ---------------- kept dims of the middle tokens: boxes -> K^mu, V^mu ----------------
+        // A warp takes eight consecutive rows of a box, a lane eight kept dims (16 bytes of a kept-dim row) of one row.  The swizzle
+        // puts the same dim of eight consecutive rows into eight different bank groups, so a fetch of 8 rows x 4 dims
+        // meets about two dims to a bank.  Four lanes to a row where a row has at most 32 kept dims (all rows in one round), else
+        // 8 or 16 (2 or 4 rounds); in round k the rows differ in the bits above the lanes', which moves a source by an xor.
+        const int w = warp - 2 - kEpiWarps;
+        const bool p2 = (s.P & (s.P - 1)) == 0;
+        const int lgP = 31 - __clz(s.P);
+        // chunk swizzle of V^mu rows as a shift and a mask of the slot (v_swz)
+        const int nchv = s.nfv >> 3, vsh = nchv == 4 ? 1 : nchv == 8 ? 0 : 2, vmask = nchv == 4 ? 3 : nchv == 8 ? 7 : (nchv == 2 || nchv == 6) ? 1 : 0;
+        int st = 0;
+        uint32_t par = 0;
+        bool live = true;
+        for (Walk it = walk_begin(); live && it.i < n_items; walk_next(it)) {
+            // 16-byte chunks of this item's kept-dim rows: one side's, or K's then V's
+            const int nk8 = (kSides == 2 && it.side) ? 0 : s.nfk >> 3, np = kSides == 2 ? (it.side ? s.nfv : s.nfk) >> 3 : nf >> 3;
+            const size_t bh = ((size_t)it.b * s.Hkv + it.h) * (size_t)s.P * (size_t)s.S_cap;
+            auto gather = [&](auto lg_lp) {
+                constexpr int LG = decltype(lg_lp)::value, RP = 32 >> LG, NI = 8 / RP;      // lanes to a row: 2^LG; rows at a time, rounds
+                const int sub = lane >> LG, p = lane & ((1 << LG) - 1);
+                const bool on = p < np, v = p >= nk8;
+                uint32_t o[4];                             // source offsets of the eight dims, two to a register
+                const int rowb = 2 * (v ? s.nfv : s.nfk);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) o[u] = 0;
+                if (on) {
+                    const uint8_t* id = idf_s + it.h * nf + (v ? s.nfk : 0) + 8 * (v ? p - nk8 : p);
+                    const int bx = kSides == 1 && v ? kChunkBytes / 2 : 0;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int d = id[u];
+                        const uint32_t off = (uint32_t)(bx + (d >> 6) * (kChunkBytes / 2) + ((((d & 63) >> 3) ^ sub) << 4) + (d & 7) * 2);
+                        o[u >> 1] |= off << (16 * (u & 1));
+                    }
+                }
+                const uint32_t col = (uint32_t)(16 * (v ? p - nk8 : p));
+                const int mask = v ? vmask : 0;
+                char* dst0 = reinterpret_cast<char*>(v ? c.v_mid : c.k_mid) + bh * (size_t)rowb;
+                int j0 = it.blk * rows.R + 8 * w + sub, left = it.n_mid - it.blk * rows.R;
+                for (int q = 0; q < it.n_ch; ++q, j0 += kChunk, left -= kChunk) {
+                    if (!mbar_wait(full + st, par, fail, c.status)) { live = false; break; }
+                    const uint32_t box = smem_u32(stage0) + (uint32_t)(st * kChunkBytes + w * 1024), src = box + (uint32_t)(sub * 128);
+                    uint4 val[NI];
+#pragma unroll
+                    for (int k = 0; k < NI; ++k) {
+                        uint32_t x[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const uint32_t oo = o[u] ^ (uint32_t)(((k * RP) << 4) * 0x10001);
+                            x[u] = 0;
+                            if (on) x[u] = __byte_perm(lds_u16(src + (uint32_t)(k * RP * 128) + (oo & 0xffffu)), lds_u16(src + (uint32_t)(k * RP * 128) + (oo >> 16)), 0x5410);
+                        }
+                        val[k] = make_uint4(x[0], x[1], x[2], x[3]);
+                    }
+                    if (left < kChunk) {
+                        // rows past the middle would count as tokens: zero them in front of the products
+                        __syncwarp();
+                        const uint32_t z = box + (uint32_t)((lane >> 4) * 128 + ((lane >> 3) & 1) * (kChunkBytes / 2) + (lane & 7) * 16);
+                        for (int k = 0; k < 8; k += 2)
+                            if (8 * w + k + (lane >> 4) >= left)
+                                asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(z + (uint32_t)k * 128u), "r"(0) : "memory");
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(masked + st);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(empty + st);    // the values are in registers: the stage goes back before the stores
+                    if (++st == n_stages) { st = 0; par ^= 1; }
+#pragma unroll
+                    for (int k = 0; k < NI; ++k) {
+                        if (on && 8 * w + sub + k * RP < left) {
+                            const int j = j0 + k * RP;
+                            const int cls = p2 ? (j & (s.P - 1)) : j % s.P, slot = p2 ? (j >> lgP) : j / s.P;
+                            // logical chunk of a V^mu row is stored at chunk ^ swizzle
+                            const uint32_t at = col ^ (uint32_t)(((slot >> vsh) & mask) << 4);
+                            *reinterpret_cast<uint4*>(dst0 + (size_t)(uint32_t)(cls * s.S_cap + slot) * (uint32_t)rowb + at) = val[k];
+                        }
+                    }
+                }
+            };
+            using std::integral_constant;
+            if (np <= 4) gather(integral_constant<int, 2>{});
+            else if (np <= 8) gather(integral_constant<int, 3>{});
+            else gather(integral_constant<int, 4>{});
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+    }
+}
+
+// ---- second contraction ------------------------------------------------------------------------------------------
+constexpr int kBMp = 128;             // coefficient rows per CTA (256 per pair)
+constexpr int kGenWarpsP = 8;
+constexpr int kThreadsP = 64 + 32 * kGenWarpsP;
+constexpr int kABytesP = kBMp * 128;  // rows of 32 hi and 32 lo values
+constexpr int kStagesP = 4;
+
+// Positions: the blocks of all (batch row, head group) units of the launch, laid end to end; a team of M / 256 pairs takes
+// positions start[t] .. start[t + 1] (cut on the host so that every team has the same cost, as in fa_compress_tc2.cu).
+constexpr int kMaxTeamsP = 96;
+struct MomCuts { uint32_t start[kMaxTeamsP + 1]; };
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+                 "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+
+// HP heads share a pair and its basis tiles.  npad: accumulator columns per head (the compressed dims of both sides, up to a
+// multiple of 32); each CTA of a pair brings half of them.
+template <int HP, bool RAG>
+__global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16* __restrict__ Y, Dims s, CacheDev c,
+                                                                      const __grid_constant__ MomRows rows, const __grid_constant__ MomCuts cuts, int npad) {
+    constexpr int kBHalf1 = 128 * 128;                     // room for this CTA's columns of one head: at most 128 rows of 128 bytes
+    constexpr int kStage = kABytesP + HP * kBHalf1;
+    const int nh = npad >> 1;
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(npad >> 3) << 17) | ((uint32_t)((2 * kBMp) >> 4) << 24);
+    extern __shared__ unsigned char smem_unaligned[];
+    unsigned char* smem = smem_unaligned + ((1024u - (smem_u32(smem_unaligned) & 1023u)) & 1023u);
+    unsigned char* stage0 = smem;
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStagesP * kStage);
+    uint64_t* peer = full + kStagesP;                      // even CTA: the odd CTA's stage is complete
+    uint64_t* empty = peer + kStagesP;
+    uint64_t* acc_ready = empty + kStagesP;
+    uint64_t* epi_done = acc_ready + 1;                    // the epilogue has left the stage ring (its scratch)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(epi_done + 1);
+    volatile int* fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t rank = cluster_ctarank();
+    const int n_pairs = s.M / (2 * kBMp);
+    const int cluster = (int)blockIdx.x >> 1, team = cluster / n_pairs, pair = cluster - team * n_pairs;
+    const int mt = 2 * pair + (int)rank;
+    const int n_hg = s.Hkv / HP, ncol = s.dck + s.dcv;
+    const uint32_t pos_begin = cuts.start[team], pos_end = cuts.start[team + 1];
+    struct Seg { int b, h0, kb0, kb1; uint32_t g0; };      // batch row of the cache, heads, blocks, first block of the row in the launch
+    auto seg_at = [&](uint32_t pos) {
+        int b, nblk = rows.nblk;
+        uint32_t g0, off;
+        if (RAG) {
+            b = 0;
+            while (pos >= rows.first[b + 1] * (uint32_t)n_hg) ++b;
+            g0 = rows.first[b];
+            nblk = (int)(rows.first[b + 1] - g0);
+            off = pos - g0 * (uint32_t)n_hg;
+        } else {
+            b = (int)(pos / (uint32_t)(n_hg * nblk));
+            off = pos - (uint32_t)(b * n_hg * nblk);
+            g0 = (uint32_t)(b * nblk);
+            b += rows.b0;
+        }
+        const int hg = (int)(off / (uint32_t)nblk), kb0 = (int)off - hg * nblk;
+        return Seg{b, hg * HP, kb0, (int)min((uint32_t)nblk, (uint32_t)kb0 + (pos_end - pos)), g0};
+    };
+
+    if (tid == 0) {
+        for (int i = 0; i < kStagesP; ++i) {
+            mbar_init(full + i, kGenWarpsP + 1);
+            mbar_init(peer + i, 1);
+            mbar_init(empty + i, 1);
+        }
+        mbar_init(acc_ready, 1);
+        mbar_init(epi_done, kGenWarpsP);
+        *fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(HP * 256) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync_all();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (pos_end > pos_begin) {
+        if (warp == 0) {
+            // ---------------- TMA producer: this CTA's half of the columns ----------------
+            if (lane == 0) {
+                asm volatile("griddepcontrol.wait;" ::: "memory");       // the moments
+                // (only now: a kernel that this lets start may count the kernel before this one as finished)
+                asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+                int it = 0, seg = 0;
+                bool live = true;
+                // (the rows past the last column are whatever the stage held: their accumulator columns are not read)
+                const uint32_t bytes = (uint32_t)min(nh, max(0, ncol - (int)rank * nh)) * (4 * kMF);
+                for (uint32_t pos = pos_begin; live && pos < pos_end; ++seg) {
+                    const Seg g = seg_at(pos);
+                    if (seg > 0 && !mbar_wait(epi_done, (seg - 1) & 1, fail, c.status)) { live = false; break; }
+                    for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
+                        const int st = it % kStagesP;
+                        if (it >= kStagesP && !mbar_wait(empty + st, ((it / kStagesP) - 1) & 1, fail, c.status)) { live = false; break; }
+                        unsigned char* bdst = stage0 + (size_t)st * kStage + kABytesP;
+                        mbar_expect_tx(full + st, HP * bytes);
+                        const char* src = reinterpret_cast<const char*>(Y) +
+                                          ((((size_t)g.g0 + kb) * s.Hkv + g.h0) * ncol + (size_t)rank * nh) * (size_t)(4 * kMF);
+                        if (bytes) {
+#pragma unroll
+                            for (int hh = 0; hh < HP; ++hh) bulk_load(bdst + hh * kBHalf1, src + (size_t)hh * ncol * (4 * kMF), bytes, full + st);
+                        }
+                    }
+                    pos += (uint32_t)(g.kb1 - g.kb0);
+                }
+                if (!live)                                 // a wait ran out: this CTA's boxes under way land, or the bound is reached, before it ends
+                    for (int q = it - kStagesP < 0 ? 0 : it - kStagesP; q < it; ++q)
+                        for (uint32_t n = 0; n < (1u << 16) && !mbar_try_wait(full + q % kStagesP, (uint32_t)(q / kStagesP) & 1u); ++n) { }
+            }
+        } else if (warp == 1) {
+            // ---------------- MMA issuer: the even CTA, for the pair ----------------
+            if (lane == 0 && rank == 0) {
+                int it = 0;
+                bool live = true;
+                for (uint32_t pos = pos_begin; live && pos < pos_end;) {
+                    const Seg g = seg_at(pos);
+                    for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
+                        const int st = it % kStagesP;
+                        const uint32_t par = (it / kStagesP) & 1;
+                        if (!mbar_wait(full + st, par, fail, c.status) || !mbar_wait(peer + st, par, fail, c.status)) { live = false; break; }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t a_addr = smem_u32(stage0 + (size_t)st * kStage), b_addr = a_addr + kABytesP;
+                        // rows of 128 bytes, 32 hi and 32 lo values: hi hi, lo hi, hi lo, sixteen values at a time
+#pragma unroll
+                        for (int pr = 0; pr < 3; ++pr)
+#pragma unroll
+                            for (int ks = 0; ks < 2; ++ks) {
+                                const uint64_t adesc = umma_desc(a_addr + (pr == 1 ? 64 : 0) + ks * 32, 1, 1024 >> 4);
+#pragma unroll
+                                for (int hh = 0; hh < HP; ++hh)
+                                    umma_bf16_pair(tmem_base + hh * 256, adesc, umma_desc(b_addr + hh * kBHalf1 + (pr == 2 ? 64 : 0) + ks * 32, 1, 1024 >> 4),
+                                                   idesc, (kb > g.kb0 || pr > 0 || ks > 0) ? 1u : 0u);
+                            }
+                        umma_commit_pair(empty + st);
+                    }
+                    if (live) umma_commit_pair(acc_ready);
+                    pos += (uint32_t)(g.kb1 - g.kb0);
+                }
+            } else if (lane == 0) {
+                const int n_it = (int)(pos_end - pos_begin);
+                for (int it = 0; it < n_it; ++it) {
+                    const int st = it % kStagesP;
+                    const uint32_t par = (it / kStagesP) & 1;
+                    if (!mbar_wait(full + st, par, fail, c.status)) break;
+                    mbar_arrive_cluster(peer + st, 0);
+                }
+            }
+        } else {
+            // ---------------- generators: rows 2 n (Re) and 2 n + 1 (Im) of e^{i theta n center} (2 r + 1) i^r j_r(phi_n) ----------------
+            const int t = tid - 64;
+            const int fi = t >> 2, tq = t & 3;             // frequency of the tile, quarter of the 32 moments
+            const unsigned n = (unsigned)(mt * (kBMp / 2) + fi);
+            float gb[8];                                   // (2 r + 1) j_r(phi_n) for r = 8 tq .. 8 tq + 7
+            {
+                // j_r by the recurrence downward from r = 10 + 2.4 phi (55 at most: far enough past phi that what is left out is
+                // below 1e-9, near enough that the values stay in range), scaled by the closed form of j_0 or j_1, whichever is larger
+                float keep[8], sn, cs, jn = 0.f, jc = 0.f, j0 = 1.f, j1 = 0.f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) keep[i] = 0.f;
+                const double invd = n ? (double)s.T / (3.14159265358979324 * (double)(n * (unsigned)rows.R)) : 0.0;      // 1 / phi: fp32's rounding of it adds up
+                const float x = (float)(n * (unsigned)rows.R) / (float)s.T, inv = (float)invd;
+                const int top = min(55, 10 + (int)(7.54f * x));
+#pragma unroll 1
+                for (int r8 = 48; r8 >= 0 && n; r8 -= 8) {
+#pragma unroll
+                    for (int i = 7; i >= 0; --i) {         // jc = j_r, jn = j_{r + 1}
+                        const int r = r8 + i;
+                        if (r == top) jc = 1e-20f;
+                        if (r8 == 8 * tq) keep[i] = (float)(2 * r + 1) * jc;
+                        if (i == 1) j1 = jc;
+                        if (i == 0) j0 = jc;
+                        const float jp = fmaf((float)((double)(2 * r + 1) * invd), jc, -jn);
+                        jn = jc;
+                        jc = jp;
+                    }
+                }
+                sincospif(x, &sn, &cs);
+                const float t0 = sn * inv, t1 = (t0 - cs) * inv, sc = fabsf(t0) > fabsf(t1) ? t0 / j0 : t1 / j1;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) gb[i] = n ? keep[i] * sc : (i == 0 && tq == 0 ? 1.f : 0.f);
+            }
+            const int r0 = 2 * fi, r1 = 2 * fi + 1;
+            const uint32_t off0 = (uint32_t)((r0 >> 3) * 1024 + (r0 & 7) * 128), off1 = (uint32_t)((r1 >> 3) * 1024 + (r1 & 7) * 128);
+            const unsigned T2 = 2u * (unsigned)s.T;
+            const float inv_T = 1.0f / (float)s.T;
+            int it = 0, seg = 0;
+            bool live = true;
+            for (uint32_t pos = pos_begin; live && pos < pos_end; ++seg) {
+                const Seg g = seg_at(pos);
+                for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
+                    const int st = it % kStagesP;
+                    // phase of the block's middle: pi n (2 kb R + R - 1) / T, exact in integers
+                    const unsigned ph = (n * (unsigned)(2 * kb * rows.R + rows.R - 1)) % T2;
+                    const float f = (float)ph * inv_T;     // in half turns, [0, 2)
+                    const float an = 3.14159265358979f * (f - (f >= 1.0f ? 2.0f : 0.0f));
+                    const float C = __cosf(an), S = __sinf(an);
+                    if (it >= kStagesP && !mbar_wait(empty + st, ((it / kStagesP) - 1) & 1, fail, c.status)) { live = false; break; }
+                    unsigned char* a_dst = stage0 + (size_t)st * kStage;
+                    uint32_t h0[4], l0[4], h1[4], l1[4];
+#pragma unroll
+                    for (int i2 = 0; i2 < 4; ++i2) {       // moments 2 i2 (i^r = +-1), 2 i2 + 1 (i^r = +-i)
+                        const float sg = (i2 & 1) ? -1.f : 1.f;
+                        const float ga = sg * gb[2 * i2], go = sg * gb[2 * i2 + 1];
+                        split_bf16(ga * C, -go * S, h0[i2], l0[i2]);
+                        split_bf16(ga * S, go * C, h1[i2], l1[i2]);
+                    }
+                    *reinterpret_cast<uint4*>(a_dst + off0 + ((tq ^ (r0 & 7)) << 4)) = make_uint4(h0[0], h0[1], h0[2], h0[3]);
+                    *reinterpret_cast<uint4*>(a_dst + off0 + (((4 + tq) ^ (r0 & 7)) << 4)) = make_uint4(l0[0], l0[1], l0[2], l0[3]);
+                    *reinterpret_cast<uint4*>(a_dst + off1 + ((tq ^ (r1 & 7)) << 4)) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
+                    *reinterpret_cast<uint4*>(a_dst + off1 + (((4 + tq) ^ (r1 & 7)) << 4)) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(full + st);
+                }
+                if (!live) break;
+                // ---------------- epilogue of the segment: accumulators are added to the coefficient rows ----------------
+                const bool ok = mbar_wait(acc_ready, seg & 1, fail, c.status);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                asm volatile("griddepcontrol.wait;" ::: "memory");      // (the coefficients are cleared by a kernel before this one)
+                if (!ok) break;
+                {
+                    const int lane_grp = warp & 3, part = (warp - 2) >> 2;
+                    const int m_base = mt * kBMp + lane_grp * 32;
+                    // 32 rows x 32 columns at a time through the idle ring: then eight lanes hold a row's 128 bytes
+                    float* tile = reinterpret_cast<float*>(stage0) + (warp - 2) * (32 * 36);
+                    const int npc = (ncol + 31) >> 5;      // pieces of 32 columns per head
+#pragma unroll 1
+                    for (int pc = part; pc < HP * npc; pc += 2) {
+                        const int hh = pc / npc, c0 = (pc - hh * npc) * 32;
+                        float v[32];
+                        tmem_ld32(tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(hh * 256 + c0), v);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + lane * 36 + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                        __syncwarp();
+                        const int q = lane & 7, rr0 = lane >> 3, col = c0 + 4 * q;
+                        if (col < ncol) {
+                            const bool is_k = col < s.dck;
+                            const int nc = is_k ? s.dck : s.dcv;
+                            float* dst = coef_rows(is_k ? c.coef_k : c.coef_v, s, g.b, g.h0 + hh, nc) + (size_t)(m_base + rr0) * nc + (is_k ? col : col - s.dck);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const float4 x = *reinterpret_cast<const float4*>(tile + (rr0 + 4 * i) * 36 + 4 * q);
+                                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + (size_t)(4 * i) * nc), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w)
+                                             : "memory");
+                            }
+                        }
+                        __syncwarp();
+                    }
+                }
+                pos += (uint32_t)(g.kb1 - g.kb0);
+                if (pos < pos_end) {
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(epi_done);
+                    if (!mbar_wait(epi_done, seg & 1, fail, c.status)) break;
+                }
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync_all();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(HP * 256) : "memory");
+    }
+}
+
+// 4-D view (dim, head, token, batch) of a prefilled K or V with element strides (1, sh, st, sb); box = 64 dims x 64 tokens.
+bool prefill_map(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int64_t st, int64_t sh, int L) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    cuuint64_t dims[4] = {(cuuint64_t)s.d, (cuuint64_t)s.Hkv, (cuuint64_t)L, (cuuint64_t)s.B};
+    cuuint64_t strides[3] = {(cuuint64_t)sh * 2, (cuuint64_t)st * 2, (cuuint64_t)(s.B > 1 ? sb : st * (int64_t)L) * 2};
+    cuuint32_t box[4] = {64, 1, (cuuint32_t)kChunk, 1};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+int npad_of(const Dims& s) { return (s.dck + s.dcv + 31) / 32 * 32; }
+
+// The longest block of a layout: a whole number of boxes, k R <= 6 T.
+int block_tokens(const Dims& s) {
+    const long long r = 6LL * s.T / s.k / kChunk * kChunk;
+    return (int)(r > kMaxBlockTokens ? kMaxBlockTokens : r);
+}
+
+size_t mom_smem_fixed(const Dims& s) {      // everything but the stages, the slack of the alignment among it
+    return (size_t)block_tokens(s) / kChunk * kHChunk + 128 * 4 * kMF + 8 * (3 * 16 + 2 * kAcc) + 16 + (size_t)s.Hkv * (2 * s.d + s.nfk + s.nfv) + 64 + 1024;
+}
+int mom_stages(const Dims& s) {
+    const long long left = 227 * 1024 - (long long)mom_smem_fixed(s);
+    const int n = (int)(left / kChunkBytes);
+    return n > 16 ? 16 : n;
+}
+
+template <int D, bool RAG>
+cudaError_t launch_moments(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, const MomRows& rows, void* Y,
+                           bool wait_first, cudaStream_t stream) {
+    const int n_stages = mom_stages(s);
+    const size_t smem = mom_smem_fixed(s) + (size_t)n_stages * kChunkBytes;
+    cudaError_t err = ensure_dynamic_smem(moments_kernel<D, RAG>, smem);
+    if (err != cudaSuccess) return err;
+    const long long items = (long long)rows.total * s.Hkv * (D == 128 ? 2 : 1);
+    if (items <= 0 || items >= (1ll << 31)) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(items < sm_count() ? items : sm_count()));
+    cfg.blockDim = dim3(kThreadsMom);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, moments_kernel<D, RAG>, tmK, tmV, s, c, L, rows, static_cast<bf16*>(Y), n_stages, (int)items, wait_first ? 1 : 0);
+}
+
+template <int HP, bool RAG>
+cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev& c, const MomRows& rows, cudaStream_t stream) {
+    const size_t smem = (size_t)kStagesP * (kABytesP + HP * 128 * 128) + 8 * (3 * kStagesP + 2) + 16 + 1024;
+    cudaError_t err = ensure_dynamic_smem(moment_project_kernel<HP, RAG>, smem);
+    if (err != cudaSuccess) return err;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kThreadsP);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const int n_pairs = s.M / (2 * kBMp), n_hg = s.Hkv / HP;
+    const long long total = (long long)rows.total * n_hg;
+    if (total <= 0 || total >= (1ll << 31)) return cudaErrorInvalidValue;
+    int n_teams;
+    {
+        // pairs resident at once (cached per device): the teams fill them, no second wave
+        static int resident[16] = {};
+        static std::mutex mu;
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 16) return cudaErrorInvalidValue;
+        std::lock_guard<std::mutex> lock(mu);
+        if (resident[dev] == 0) {
+            cfg.gridDim = dim3(2 * sm_count());
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, moment_project_kernel<HP, RAG>, &cfg) != cudaSuccess || n < 1) {
+                cudaGetLastError();
+                n = sm_count() / 2 - 2;
+            }
+            cfg.numAttrs = 2;
+            resident[dev] = n;
+        }
+        n_teams = resident[dev] / n_pairs;
+    }
+    if (n_teams < 1) n_teams = 1;
+    if (n_teams > kMaxTeamsP) n_teams = kMaxTeamsP;
+    if (n_teams > total) n_teams = (int)total;
+    // Equal cost per team: a segment costs its blocks plus kEpi (epilogue and refill, in blocks); the smallest budget with
+    // which the walk covers all positions in n_teams teams, by bisection.
+    MomCuts cuts = {};
+    constexpr long long kEpi = 6, kMinSeg = 2;
+    auto unit_end_of = [&](long long pos) {
+        long long first = 0, nblk = rows.nblk;
+        if (RAG) {
+            int b = 0;
+            while (pos >= (long long)rows.first[b + 1] * n_hg) ++b;
+            first = (long long)rows.first[b] * n_hg;
+            nblk = (long long)rows.first[b + 1] - rows.first[b];
+        }
+        return first + ((pos - first) / nblk + 1) * nblk;
+    };
+    auto walk = [&](long long budget, uint32_t* start) {
+        long long pos = 0;
+        int t = 0;
+        for (; t < n_teams && pos < total; ++t) {
+            if (start) start[t] = (uint32_t)pos;
+            long long left = budget;
+            while (pos < total && left >= kEpi + kMinSeg) {
+                const long long unit_end = unit_end_of(pos);
+                long long take = unit_end - pos < left - kEpi ? unit_end - pos : left - kEpi;
+                if (unit_end - pos - take > 0 && unit_end - pos - take < kMinSeg) take = unit_end - pos - kMinSeg;
+                if (take <= 0) break;
+                pos += take;
+                left -= take + kEpi;
+            }
+        }
+        if (start)
+            for (int u = t; u <= n_teams; ++u) start[u] = (uint32_t)(u == n_teams ? total : pos);
+        return pos >= total;
+    };
+    long long lo = kEpi + kMinSeg, hi = total + kEpi * (total + 1) + kMinSeg;
+    while (lo < hi) {
+        const long long mid = (lo + hi) / 2;
+        if (walk(mid, nullptr)) hi = mid; else lo = mid + 1;
+    }
+    while (!walk(lo, cuts.start)) ++lo;
+    cuts.start[n_teams] = (uint32_t)total;
+    cfg.gridDim = dim3(2 * n_teams * n_pairs);
+    return cudaLaunchKernelEx(&cfg, moment_project_kernel<HP, RAG>, static_cast<const bf16*>(Y), s, c, rows, cuts, npad_of(s));
+}
+
+}  // namespace
+
+// True if the two-step contraction serves this layout: what the pair kernel of the direct contraction needs, tables that
+// fit beside the ring, and blocks of at least three boxes (T / k >= 32: the axis is then six times shorter, which three products
+// and the round trip of the moments still leave 5 % ahead of the direct contraction; half of that would lose).
+bool compress_mom_supported(const Dims& s) {
+    if (s.M % (2 * kBMp) != 0 || s.d > 128 || s.dck + s.dcv == 0) return false;
+    if (block_tokens(s) < 3 * kChunk) return false;
+    if (mom_stages(s) < 5) return false;
+    // phases n (2 j + R - 1) stay in 32 bits
+    return (unsigned long long)(s.M / 2) * (2ull * (unsigned long long)s.T + 2ull * kMaxBlockTokens) < (1ull << 32);
+}
+
+// Bytes of moments that a batch row of n_mid middle tokens needs (of a layout that is supported).
+size_t compress_mom_row_bytes(const Dims& s, int n_mid) {
+    const int R = block_tokens(s);
+    return (size_t)((n_mid + R - 1) / R) * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
+}
+
+// Coefficients (the caller has zeroed them) and the kept-dim rows of the middle tokens of batch rows b0 .. b0 + nb; the windows
+// and the counters are the caller's (the partition kernel).  lens: prompt lengths of all batch rows (at most L; rows
+// with fewer than tc_min middle tokens are left out), or none.  Y: room for these rows' moments, 128-byte aligned;
+// wait_first: a kernel of this stream that may still run reads Y.
+cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int L, int b0,
+                                int nb, void* Y, bool wait_first, cudaStream_t stream, const RowLens* lens, int tc_min) {
+    MomRows rows = {};
+    rows.R = block_tokens(s);
+    rows.b0 = b0;
+    rows.nb = nb;
+    if (lens && lens->n) {
+        if (lens->n != s.B) return cudaErrorInvalidValue;
+        rows.lens = *lens;
+        long long at = 0;
+        for (int b = 0; b < s.B; ++b) {
+            const int m = mid_of(s, lens->len[b]);
+            if (b >= b0 && b < b0 + nb && m >= tc_min) at += (m + rows.R - 1) / rows.R;
+            if (at >= (1ll << 24)) return cudaErrorInvalidValue;
+            rows.first[b + 1] = (uint32_t)at;
+        }
+        rows.total = (int)at;
+    } else {
+        rows.nblk = (mid_of(s, L) + rows.R - 1) / rows.R;
+        if ((long long)rows.nblk * nb >= (1ll << 24)) return cudaErrorInvalidValue;
+        rows.total = rows.nblk * nb;
+    }
+    if (rows.total == 0) return cudaSuccess;
+    CUtensorMap tmK, tmV;
+    if (!prefill_map(&tmK, K, s, sb, st, sh, L) || !prefill_map(&tmV, V, s, sb, st, sh, L))
+        return cudaErrorInvalidValue;
+    const bool rag = rows.lens.n != 0;
+    cudaError_t err;
+    if (s.d == 128) err = rag ? launch_moments<128, true>(tmK, tmV, s, c, L, rows, Y, wait_first, stream) : launch_moments<128, false>(tmK, tmV, s, c, L, rows, Y, wait_first, stream);
+    else err = rag ? launch_moments<64, true>(tmK, tmV, s, c, L, rows, Y, wait_first, stream) : launch_moments<64, false>(tmK, tmV, s, c, L, rows, Y, wait_first, stream);
+    if (err != cudaSuccess) return err;
+    if (s.Hkv % 2 == 0) return rag ? launch_project<2, true>(Y, s, c, rows, stream) : launch_project<2, false>(Y, s, c, rows, stream);
+    return rag ? launch_project<1, true>(Y, s, c, rows, stream) : launch_project<1, false>(Y, s, c, rows, stream);
+}
+
+}  // namespace fa

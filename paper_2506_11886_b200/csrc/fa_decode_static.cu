@@ -52,7 +52,7 @@ size_t fa_static_workspace_limit(void) { return fa::kStaticWsBytes; }
 fa_status fa_decode_attention_static(const fa_layout* layout, const fa_cache* cache, const void* q, void* out,
                                      void* stream) {
     size_t need = 0;
-    fa_status st = fa_workspace_bytes(layout, &need);      // also validates the layout; host only
+    fa_status st = fa::decode_scratch_bytes(layout, &need);      // also validates the layout; host only
     if (st != FA_OK) return st;
     if (need > fa::kStaticWsBytes) return FA_ERR_WORKSPACE; // this layout needs more scratch than the fixed array has
     char* ws = nullptr;

@@ -1,0 +1,159 @@
+"""Compression by block moments (fa_compress_mom.cu): where it can go wrong (ends of blocks and boxes, odd head counts, kept
+dims on one side only, rows of different length, little scratch), against the oracle and against the direct contraction.
+
+Bounds.  Both factors of the two products are held as two bf16 numbers: 2^-17 relative each, and the dropped lo x lo term and the
+truncated expansion (1.5e-5 at the edge of the band, 6e-7 rms) are below that; relative to the largest coefficient of a
+head 3e-5 covers four times their sum.  The direct contraction rounds its basis to bf16: 2^-9 a term, averaged over at
+least 1024 tokens, within the 1e-3 that the parity suite allows it."""
+import pytest
+import torch
+
+from paper_2506_11886_b200 import fa, synth
+from tests.parity_util import layout_of, make_pair
+
+pytestmark = pytest.mark.gpu
+
+EXACT_KEYS = ("k_init", "v_init", "k_local", "v_local", "k_mid", "v_mid", "state")
+MOMENT_REL = 3e-5
+
+
+def _shape(**kw):
+    return synth.Shape("moments", **{**dict(B=1, layers=1, Hq=2, Hkv=2, d=128, L=1500, dtype="bf16", n_full_k=32, n_full_v=32, M=256,
+                                            T=4096, L_init=4, L_local=64), **kw})
+
+
+@pytest.mark.parametrize("kw", [
+    dict(L=1024 + 68),                                    # shortest middle of this path; blocks of 192 tokens, the last of 64
+    dict(L=1025 + 68), dict(L=1151 + 68), dict(L=1152 + 68), dict(L=1153 + 68),      # one token into, up to, and past a whole block
+    dict(L=4096 + 68, B=2),                               # period full
+    dict(L=3001, Hkv=3, Hq=3),                            # odd number of heads: one to a pair of CTAs
+    dict(L=3001, n_full_k=0, n_full_v=128),               # nothing kept of K, no coefficients of V
+    dict(L=3001, n_full_k=120, n_full_v=8),               # eight columns of K, four rounds of the gather on one side
+    dict(L=2500, d=64, n_full_k=64, n_full_v=24, Hkv=4, Hq=4),      # K and V in one item
+    dict(L=2500, d=64, n_full_k=8, n_full_v=56),
+    dict(L=5000, M=512, T=16384, L_local=300),            # blocks of 384 tokens, a window that starts inside a box
+    dict(L=3333, M=256, T=65536, L_init=0, L_local=1),    # T / k = 512: the longest blocks, 768 tokens
+    dict(L=3000, M=256, T=5000),                          # period not a power of two
+])
+def test_block_moments_against_oracle(kw):
+    shape = _shape(**kw)
+    P = 1 if shape.T == 5000 else 8
+    pair, _ = make_pair(shape, seed=71, P=P, max_mid=min(shape.T, shape.L), algo=fa.FA_DECODE_DIRECT, freq="offgrid")
+    worst = pair.check_state()
+    assert worst <= MOMENT_REL
+
+
+def _cache(layout, stream):
+    """A cache full of old values: what a call has to write is overwritten, slots past the middle stay."""
+    c = fa.Cache(layout, stream.idx_full_k, stream.idx_full_v)
+    for n in ("coef_k", "coef_v", "k_mid", "v_mid"):
+        getattr(c, n).fill_(3.0)
+    return c
+
+
+def _compress(layout, stream, K, V, ws, lengths=None):
+    c = _cache(layout, stream)
+    if lengths is None:
+        fa.fa_compress(layout, c, K, V, ws)
+    else:
+        fa.fa_compress_ragged(layout, c, K, V, lengths, ws)
+    torch.cuda.synchronize()
+    assert fa.fa_poll_status(c) == fa.FA_OK
+    return c
+
+
+def _same(a, b, rel):
+    for n in EXACT_KEYS:
+        assert torch.equal(getattr(a, n), getattr(b, n)), n
+    for n in ("coef_k", "coef_v"):
+        x, y = getattr(a, n), getattr(b, n)
+        den = y.abs().amax(dim=(-1, -2), keepdim=True)
+        assert ((x - y).abs() <= rel * den).all(), n
+
+
+def _row_bytes(layout, n_mid):
+    R = min(6 * layout.period // (layout.n_coef // 2) // 64 * 64, 768)
+    return -(-n_mid // R) * layout.n_kv_heads * (2 * layout.head_dim - layout.n_full_k - layout.n_full_v) * 128
+
+
+def _workspace(layout, n_mid, rows, short=0):
+    """A workspace with room for the moments of `rows` rows of n_mid middle tokens, less `short` bytes."""
+    decode = fa.fa_workspace_bytes(layout) - 2 * layout.batch * _row_bytes(layout, layout.max_mid)
+    return torch.zeros(decode + rows * _row_bytes(layout, n_mid) - short, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("ragged", [False, True])
+@pytest.mark.parametrize("strided", [False, True])
+def test_groups_of_rows_and_the_direct_contraction_agree(ragged, strided):
+    """A workspace with room for all rows, two, one, or none (the direct contraction): the same cache each time, from
+    contiguous and from strided prefill tensors, rows of equal and of different length."""
+    shape = _shape(B=5, L=2900, n_full_k=24, n_full_v=48)
+    layout = layout_of(shape, max_mid=shape.T, P=16)
+    stream = synth.KVStream(shape, seed=9, device="cuda", freq="offgrid")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    if strided:                                           # [B][H][L][2 d], the second half not used
+        wide = [torch.full((shape.B, shape.Hkv, shape.L, 256), float("nan"), dtype=X.dtype, device="cuda") for X in (K, V)]
+        for w, X in zip(wide, (K, V)):
+            w[..., :128] = X.transpose(1, 2)
+        K, V = (w[..., :128].transpose(1, 2) for w in wide)
+    lengths = [2900, 700, 1092, 1500, 2899] if ragged else None
+    full = _compress(layout, stream, K, V, fa.new_workspace(layout), lengths)
+    direct = _compress(layout, stream, K, V, _workspace(layout, shape.L - 68, 1, short=1), lengths)
+    _same(direct, full, 1e-3)
+    for rows in (1, 2, 3, 5):
+        ws = _workspace(layout, shape.L - 68, rows)
+        _same(_compress(layout, stream, K, V, ws, lengths), full, 2e-6)      # the same products, added in another order
+        assert not ws[:4096].any()                        # the barrier counters of the decode call are left alone
+
+
+@pytest.mark.parametrize("halves", [1, 2])
+def test_layers_in_one_call_and_replayed_from_a_graph(halves):
+    """Layers with scratch for one or two layers at a time, with inputs that change between the replays of a graph."""
+    shape = _shape(B=1, L=3000, Hkv=4, Hq=4)
+    layout = layout_of(shape, max_mid=shape.T, P=16)
+    n = 4
+    streams = [synth.KVStream(shape, seed=20 + i, device="cuda", freq="offgrid") for i in range(n)]
+    toks = [[s.tokens(t, t + shape.L, work_dtype=torch.float32) for s in streams] for t in (0, 1000)]
+    K, V = ([torch.empty_like(p[0]) for p in toks[0]] for _ in range(2))
+    caches = [_cache(layout, s) for s in streams]
+    ws = _workspace(layout, shape.L - 68, halves)
+
+    def fill(which):
+        for i in range(n):
+            K[i].copy_(toks[which][i][0]); V[i].copy_(toks[which][i][1])
+
+    fill(0)
+    fa.fa_compress_layers([layout] * n, caches, K, V, ws)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        fa.fa_compress_layers([layout] * n, caches, K, V, ws)
+    for which in (1, 0, 1):
+        fill(which)
+        g.replay()
+        torch.cuda.synchronize()
+        for i in range(n):
+            one = _compress(layout, streams[i], *toks[which][i], fa.new_workspace(layout))
+            _same(caches[i], one, 2e-6)
+    del g
+    assert all(fa.fa_poll_status(c) == fa.FA_OK for c in caches)
+
+
+def test_not_finite_dims_stay_alone():
+    """A NaN or an infinity in one dim of one token spoils that dim's coefficients only."""
+    shape = _shape(L=2500)
+    layout = layout_of(shape, max_mid=shape.T, P=16)
+    stream = synth.KVStream(shape, seed=4, device="cuda", freq="offgrid")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    want = _compress(layout, stream, K, V, fa.new_workspace(layout))
+    bad = int(want.idx_comp_k[1, 5])
+    kept = int(want.idx_full_k[0, 3])
+    K[0, 777, 1, bad] = float("inf")
+    K[0, 900, 0, kept] = float("nan")
+    got = _compress(layout, stream, K, V, fa.new_workspace(layout))
+    rest = torch.ones_like(got.coef_k, dtype=torch.bool)
+    rest[0, 1, :, 5] = False
+    assert torch.isfinite(got.coef_k[rest]).all() and torch.isfinite(got.coef_v).all()
+    assert not torch.isfinite(got.coef_k[0, 1, :, 5]).all()
+    den = want.coef_k.abs().max()
+    assert ((got.coef_k - want.coef_k).abs()[rest] <= 2e-6 * den).all()
