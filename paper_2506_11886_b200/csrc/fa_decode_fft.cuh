@@ -968,6 +968,24 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         k_on[rd] = 4 * rd + tq < npk;
     }
     const uint32_t kb_lane_off = (uint32_t)(gq * GH + 2 * tq) * 4;
+    // Class tiles: groups of 16 tokens go to the warps in turn, on from where the tile before ended (a tile ends with its class:
+    // started at warp 0 each time, six groups to a class left two of eight warps without work, 16 groups six warps
+    // with three rounds for four of them; MHA at batch 8 992 -> 947 us for eight steps, 128 K tokens 989 -> 968, a 2 K-token chat
+    // 365 -> 362).  Not in the unsplit instances of long classes, whose tiles are whole rounds of eight warps nearly
+    // always (32 K tokens: 545 -> 550).  g_of: this warp's first group of the next tile.
+    constexpr bool kRotate = SPLIT || LS <= 8;
+    int g_of = wm;
+    auto tile_done = [&](int nt) {
+        if constexpr (kRotate) {
+            g_of -= (nt + 15) >> 4;
+            if constexpr (kMW == 8) g_of &= 7;
+            else while (g_of < 0) g_of += kMW;
+        }
+    };
+    auto owns = [&](int grp) {                            // of the tile at hand
+        if constexpr (kRotate) return (grp + kMW - g_of) % kMW == 0;
+        else return wm == grp % kMW;
+    };
     auto k_phase = [&](int cb, int nb, float* kbuf) {
         if (!ts_k || !is_m) return;
 #pragma unroll 1
@@ -977,7 +995,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             for (int a0 = 0; a0 < n_c; a0 += ts_k) {
                 const int nt = min(ts_k, n_c - a0);
                 const uint32_t tile = wait_tile_u();
-                if (STEP && cb + ci == cstar && astar >= a0 && astar < a0 + nt && wm == ((astar - a0) >> 4) % kMW) {
+                if (STEP && cb + ci == cstar && astar >= a0 && astar < a0 + nt && owns((astar - a0) >> 4)) {
                     // fused step: middle token j_pend is not in the cache yet; its kept dims from the row that leaves the window
                     patch_mid_k(tile + (uint32_t)((astar - a0) * rowb_k), c.idx_full_k + (size_t)h * s.nfk, s.nfk, xrow_s, lane);
                 }
@@ -986,7 +1004,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 // which lose 1-2 % to it.
                 constexpr int U = OCC == 1 && !SPLIT ? 2 : 1;
 #pragma unroll 1
-                for (int grp = wm; grp * 16 < nt; grp += U * kMW) {
+                for (int grp = g_of; grp * 16 < nt; grp += U * kMW) {
                     const bool two = U == 2 && (grp + kMW) * 16 < nt;
                     const uint32_t gbase = tile + (uint32_t)(grp * 16) * rowb_k;
                     float d4[U][4];
@@ -1029,6 +1047,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     }
                 }
                 release_tile();
+                tile_done(nt);
             }
         }
     };
@@ -1467,10 +1486,10 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     for (int a0 = 0; a0 < n_c; a0 += ts_v) {
                         const int nt = min(ts_v, n_c - a0);
                         const uint32_t tile = wait_tile_u();
-                        if (STEP && cb + ci == cstar && astar >= a0 && astar < a0 + nt && wm == ((astar - a0) >> 4) % kMW)
+                        if (STEP && cb + ci == cstar && astar >= a0 && astar < a0 + nt && owns((astar - a0) >> 4))
                             patch_mid_v(tile + (uint32_t)((astar - a0) * rowb_v), c.idx_full_v + (size_t)h * s.nfv, s.nfv, xrow_s + s.d, astar, lane);
                         #pragma unroll 1
-                        for (int grp = wm; grp * 16 < nt; grp += kMW) {
+                        for (int grp = g_of; grp * 16 < nt; grp += kMW) {
                             const uint32_t gbase = tile + (uint32_t)(grp * 16) * rowb_v;
                             uint32_t b0 = 0, b1 = 0;
                             if (gq < GH) {
@@ -1487,6 +1506,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                             }
                         }
                         release_tile();
+                        tile_done(nt);
                     }
                 }
             }
@@ -1615,7 +1635,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                         const int nt = min(ts_v, n_c - a0);
                         const uint32_t tile = wait_tile_u();
                         #pragma unroll 1
-                        for (int grp = wm; grp * 16 < nt; grp += kMW) {
+                        for (int grp = g_of; grp * 16 < nt; grp += kMW) {
                             const uint32_t gbase = tile + (uint32_t)(grp * 16) * rowb_v;
                             if (STEP && cb + ci == cstar && astar >= a0 + grp * 16 && astar < a0 + grp * 16 + 16) {
                                 patch_mid_v(tile + (uint32_t)((astar - a0) * rowb_v), c.idx_full_v + (size_t)h * s.nfv, s.nfv, xrow_s + s.d, astar, lane);
@@ -1635,6 +1655,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                             }
                         }
                         release_tile();
+                        tile_done(nt);
                     }
                 }
             }
