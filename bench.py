@@ -190,6 +190,12 @@ def profile_counter(file_key: str, section: str, label: str):
     return float(m.group(1)) if m else None
 
 
+def step_launches(fa, layout):
+    """Kernels of one fa_decode_step."""
+    chain = fa.fa_launch_count(layout, 7)
+    return chain + (layout.n_q_heads > 4 * layout.n_kv_heads) if chain else fa.fa_launch_count(layout, 3)
+
+
 def make_layout(fa, shape):
     return fa.Layout(batch=shape.B, n_q_heads=shape.Hq, n_kv_heads=shape.Hkv, head_dim=shape.d, n_full_k=shape.n_full_k,
                      n_full_v=shape.n_full_v, n_coef=shape.M, period=shape.T, l_init=shape.L_init, l_local=shape.L_local,
@@ -298,7 +304,7 @@ def bench_layers(torch, fa, synth, timer, dev, cfg_id, n_layers, tok_steps, warm
            "decode_gbs": dec_gbs, "frac": dec_gbs / peak,
            "step_gbs": (by["decode"] + by["append"]) * n_layers / (tok["median"] * 1e-6) / 1e9,
            "tokens_per_s": shape.B * 1e6 / tok["median"],
-           "launches_per_token_step": n_layers * fa.fa_launch_count(layout, 3),
+           "launches_per_token_step": n_layers * step_launches(fa, layout),
            "compress_ms_per_layer": min(comp), "compress_tflops": comp_flop / (min(comp) * 1e-3) / 1e12}
     del caches, args
     torch.cuda.empty_cache()
@@ -497,8 +503,8 @@ def run_ours(args):
     eb = 2 if shape.dtype == "bf16" else 4
     q_bytes = shape.B * shape.Hq * shape.d * eb
     kv_bytes = shape.B * shape.Hkv * shape.d * eb
-    launches = K_steps * fa.fa_launch_count(layout, 3)
-    n_dec = fa.fa_launch_count(layout, 2)
+    launches = K_steps * step_launches(fa, layout)
+    n_dec = fa.fa_launch_count(layout, 7) or fa.fa_launch_count(layout, 2)
     # figures of the committed ncu captures (profiles/): DRAM bytes of one decode launch, tensor-pipe share of the compress kernel
     traffic = None
     if args.config == 1:

@@ -69,7 +69,11 @@ typedef enum { FA_NORM_ORTHO = 0, FA_NORM_PAPER = 1 } fa_norm;
  * once, one CTA per (batch, KV head) in waves past that; else as three kernels.
  * FFT_SPLIT always takes the three-kernel form.  AUTO also takes it when there
  * are more (batch, KV head) pairs than SMs and the last wave of the one-kernel
- * form would be nearly empty. */
+ * form would be nearly empty.  For bf16 caches with many (batch, KV head) pairs
+ * and classes (see fa_launch_count, 7) AUTO evaluates the classes by 16 Legendre
+ * channels instead of one transform per class (left out: below 1e-9 relative), as a
+ * chain of three kernels, when ws_bytes has the room that fa_workspace_bytes asks
+ * for; with less it is FFT. */
 typedef enum { FA_DECODE_AUTO = 0, FA_DECODE_DIRECT = 1, FA_DECODE_FFT = 2, FA_DECODE_FFT_SPLIT = 3 } fa_decode_algo;
 
 /* Immutable description of one layer's cache. */
@@ -223,7 +227,8 @@ fa_status fa_decode_attention(const fa_layout* layout, const fa_cache* cache, co
  * to each coefficient row as the kernel streams it (C^K before forming u, C^V before the output
  * product) and written back, so the coefficients cross the memory bus once per step instead of twice,
  * and the moved rows and the counters are written to the cache once every CTA that reads the old
- * ones is past them.  Otherwise the two calls are made one after the other (with many rows per CTA
+ * ones is past them.  In the channel form the push rides on the first and the last of its three kernels
+ * (up to four query heads to a KV head).  Otherwise the two calls are made one after the other (with many rows per CTA
  * the stand-alone append kernel, which spreads the coefficient update over the whole device, is the
  * faster way).  Same arguments, workspace rule and errors as those two calls (a full middle sets
  * FA_ERR_CAPACITY in cache->status and the step decodes the unchanged cache). */
@@ -306,7 +311,9 @@ fa_status fa_poll_status(const fa_cache* cache, void* stream);
  * 2 decode, 3 decode step); for launch accounting by callers.  what >= 4 asks about the decode plan instead:
  * 4: 1 if fa_decode_attention runs the split build of the fused kernel for this layout, else 0;
  * 5: residue classes per batch of the transform kernel (0 for the direct kernel);
- * 6: CTAs per (batch, KV head, pass of query heads).  Unknown values of what return 0. */
+ * 6: CTAs per (batch, KV head, pass of query heads); 7: kernels of a decode call in the channel form, 0 where AUTO does not
+ * take it (2 to 6 answer for the transform or direct kernel, which then is the one for a smaller workspace; a step in the channel
+ * form is the same kernels, plus the append kernel with more than four query heads to a KV head).  Unknown values of what return 0. */
 int fa_launch_count(const fa_layout* layout, int what);
 
 const char* fa_status_string(fa_status s);

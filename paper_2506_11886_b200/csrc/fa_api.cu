@@ -120,12 +120,27 @@ static bool fft_ok(const fa_layout& l, int gh, int* log2S) {
     return true;
 }
 
-static fa_status make_plan(const fa_layout& l, DecodePlan* p);
+static fa_status make_plan(const fa_layout& l, CallPlan* p);
+
+// Whether the channel form is ahead of the transform kernel: it makes 16 transforms per (batch row, KV head) where the other makes
+// one per residue class, but as a chain of three kernels whose first and last cost 10 to 35 us whatever the batch.  So it goes by
+// the class transforms that there are, heads * classes.  A step, transform kernel -> channel form in us (GQA 4 and 3, MHA, kept
+// dims 24 to 48 a side, 131 layouts each way):
+//   from 8192 class transforms (all periods): 64 heads of 128 classes, 4K tokens 66.5 -> 43.7, 12K 99 -> 72, 64K 314 -> 228;
+//     256 heads of 32 classes, 1K 64.5 -> 47.5, 4K 117.7 -> 100; 128 heads of 64 classes, 4K 70.9 -> 67.7, ragged 70 -> 73.5
+//   from 4096 where rows are long: 64 heads of 64 classes, 12K 101.5 -> 83, 32K 189 -> 169; 32 heads of 128, 128K 243 -> 228 to 298 -> 201;
+//     but at 4K tokens 52 -> 57
+//   below: 32 heads of 64 classes, 32K 90 -> 97, 12K 53 -> 64; 64 heads of 32 classes, 4K 50 -> 51, 32K 197 -> 207; 16 heads of
+//     128 classes, 128K 122 -> 159; one row of 8 heads, 32K 38 -> 52
+static bool channels_pay(const Dims& s) {
+    const long long heads = (long long)s.B * s.Hkv, transforms = heads * s.P;
+    return heads >= 32 && (transforms >= 8192 || (transforms >= 4096 && s.T >= 16384));
+}
 
 // The plan of a layout.  Working it out (the split of classes and windows, what fits in shared memory) takes longer than a
 // launch, and a program calls with the same few layouts over and over: every thread keeps the plans of its last ones.
-fa_status plan_decode(const fa_layout& l, DecodePlan* p) {
-    struct Entry { fa_layout l; int dev; fa_status st; DecodePlan p; };
+fa_status plan_decode(const fa_layout& l, CallPlan* p) {
+    struct Entry { fa_layout l; int dev; fa_status st; CallPlan p; };
     constexpr int kEntries = 8;
     static thread_local Entry cache[kEntries];
     static thread_local int used = 0, next = 0;
@@ -139,7 +154,7 @@ fa_status plan_decode(const fa_layout& l, DecodePlan* p) {
     return st;
 }
 
-static fa_status make_plan(const fa_layout& l, DecodePlan* p) {
+static fa_status make_plan(const fa_layout& l, CallPlan* p) {
     Dims s = make_dims(l);
     std::memset(p, 0, sizeof(*p));
     const int kNumSms = sm_count();
@@ -290,6 +305,12 @@ static fa_status make_plan(const fa_layout& l, DecodePlan* p) {
     p->off_om = off;  off = align_up(off + sizeof(float) * heads * s.d, 256);
     p->off_cnt = off; off = align_up(off + sizeof(int32_t) * (size_t)s.B * s.Hkv, 256);
     p->total = off;
+    if (p->algo == FA_DECODE_FFT && l.decode_algo == FA_DECODE_AUTO && channels_pay(s) &&
+        plan_channels(s, log2S, kNumSms, &p->chan)) {
+        // the channel form has its areas behind the barrier counters
+        p->chan.total = place_channels(s, log2S, align_up(sizeof(int32_t) * 4 * (size_t)kBarSlots, 256), &p->chan);
+        p->chan.on = 1;
+    }
     return FA_OK;
 }
 
@@ -334,17 +355,23 @@ fa_status decode_scratch_bytes(const fa_layout* layout, size_t* out) {
     fa_status st = check_layout(layout);
     if (st != FA_OK) return st;
     if (!out) return FA_ERR_INVALID_ARG;
-    DecodePlan p;
+    CallPlan p;
     st = plan_decode(*layout, &p);
     if (st != FA_OK) return st;
     *out = p.total;
     if (p.fused) {                       // room for the three-kernel form too, should a cooperative launch not fit
         fa_layout split = *layout;
         split.decode_algo = FA_DECODE_FFT_SPLIT;
-        DecodePlan p2;
+        CallPlan p2;
         if (plan_decode(split, &p2) == FA_OK && p2.total > *out) *out = p2.total;
     }
     return FA_OK;
+}
+// The same with room for the channel form.
+static size_t decode_room_bytes(const fa_layout& l, size_t least) {
+    CallPlan p;
+    if (plan_decode(l, &p) == FA_OK && p.chan.on && p.chan.total > least) least = p.chan.total;
+    return align_up(least, 256);
 }
 
 // Scratch of the compression by block moments: behind that of the decode call (a decode step may run on another stream while a
@@ -366,7 +393,7 @@ struct MomentRoom { char* at; size_t bytes; };
 static MomentRoom moment_room(const fa_layout& l, void* ws, size_t ws_bytes) {
     size_t decode = 0;
     if (!ws || !aligned16(ws) || !compress_mom_supported(make_dims(l)) || decode_scratch_bytes(&l, &decode) != FA_OK) return {nullptr, 0};
-    decode = align_up(decode, 256);
+    decode = decode_room_bytes(l, decode);
     return ws_bytes > decode ? MomentRoom{static_cast<char*>(ws) + decode, ws_bytes - decode} : MomentRoom{nullptr, 0};
 }
 // The two kernels of the block-moment path over all batch rows: all at once, or in groups that take half of the room in turn
@@ -417,7 +444,7 @@ fa_status fa_cache_sizes_of(const fa_layout* layout, fa_cache_sizes* out) {
 fa_status fa_workspace_bytes(const fa_layout* layout, size_t* out) {
     fa_status st = decode_scratch_bytes(layout, out);
     if (st != FA_OK) return st;
-    *out = align_up(*out, 256) + compress_scratch_bytes(*layout);
+    *out = decode_room_bytes(*layout, *out) + compress_scratch_bytes(*layout);
     return FA_OK;
 }
 
@@ -748,7 +775,7 @@ fa_status fa_decode_attention(const fa_layout* layout, const fa_cache* cache, co
     st = check_cache(layout, cache);
     if (st != FA_OK) return st;
     if (!q || !out || !aligned16(q) || !aligned16(out)) return FA_ERR_INVALID_ARG;
-    DecodePlan p;
+    CallPlan p;
     st = plan_decode(*layout, &p);
     if (st != FA_OK) return st;
     if (!ws || !aligned16(ws) || ws_bytes < p.total) return FA_ERR_WORKSPACE;
@@ -756,6 +783,12 @@ fa_status fa_decode_attention(const fa_layout* layout, const fa_cache* cache, co
     CacheDev c = make_cache(*cache);
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     char* w = static_cast<char*>(ws);
+    if (p.chan.on && ws_bytes >= p.chan.total) {
+        bool begun = false;
+        if (launch_decode_channels(s, c, p.chan, p.fft_log2, q, out, nullptr, nullptr, w, cs, &begun) == cudaSuccess) return FA_OK;
+        if (begun) return FA_ERR_CUDA;
+        cudaGetLastError();                                  // refused before anything ran: the transform kernel
+    }
     if (p.fused) {
         const cudaError_t err = launch_decode_fft(s, c, layout->kv_dtype, p, q, out, w, nullptr, nullptr, cs);
         if (err == cudaSuccess) return FA_OK;
@@ -800,7 +833,7 @@ static fa_status decode_step_impl(const fa_layout* layout, fa_cache* cache, cons
     if (st != FA_OK) return st;
     if (!q || !out || !aligned16(q) || !aligned16(out)) return FA_ERR_INVALID_ARG;
     if (!k_new || !v_new || !aligned16(k_new) || !aligned16(v_new)) return FA_ERR_INVALID_ARG;
-    DecodePlan p;
+    CallPlan p;
     st = plan_decode(*layout, &p);
     if (st != FA_OK) return st;
     if (!ws || !aligned16(ws) || ws_bytes < p.total) return FA_ERR_WORKSPACE;
@@ -808,7 +841,15 @@ static fa_status decode_step_impl(const fa_layout* layout, fa_cache* cache, cons
     // The push rides on the decode launch where a head has many parts (each then updates a small slice of the
     // coefficient rows as it streams them for u and for the output product).
     // Whether the device can hold all parts at once is asked before anything is enqueued: nothing to undo.
-    if (step_in_one_launch(*layout, p) && cooperative_launch_supported() && decode_fft_launchable(s, p)) {
+    const bool channels = p.chan.on && ws_bytes >= p.chan.total;
+    if (channels && p.chan.n_pass == 1) {
+        bool begun = false;
+        if (launch_decode_channels(s, make_cache(*cache), p.chan, p.fft_log2, q, out, k_new, v_new, static_cast<char*>(ws), static_cast<cudaStream_t>(stream), &begun) == cudaSuccess)
+            return FA_OK;
+        if (begun) return FA_ERR_CUDA;
+        cudaGetLastError();                                  // refused before anything ran
+    }
+    if (!(channels && p.chan.n_pass > 1) && step_in_one_launch(*layout, p) && cooperative_launch_supported() && decode_fft_launchable(s, p)) {
         const cudaError_t err = launch_decode_fft(s, make_cache(*cache), layout->kv_dtype, p, q, out, static_cast<char*>(ws), k_new, v_new,
                                                   static_cast<cudaStream_t>(stream));
         if (err == cudaSuccess) return FA_OK;
@@ -839,7 +880,7 @@ fa_status fa_decode_step_layers(int32_t n_layers, const fa_layout* layouts, fa_c
         if (st != FA_OK) return st;
         const void* ptrs[] = {q[i], k_new[i], v_new[i], out[i]};
         for (const void* p : ptrs) if (!p || !aligned16(p)) return FA_ERR_INVALID_ARG;
-        DecodePlan p;
+        CallPlan p;
         st = plan_decode(layouts[i], &p);
         if (st != FA_OK) return st;
         if (!ws || !aligned16(ws) || ws_bytes < p.total) return FA_ERR_WORKSPACE;
@@ -920,29 +961,34 @@ int fa_launch_count(const fa_layout* layout, int what) {
         case 0: return 2;   // partition/gather + coefficient kernel (memsets not counted)
         case 1: return 1;
         case 2: {           // one fused kernel, or prologue + main + epilogue
-            DecodePlan p;
+            CallPlan p;
             if (plan_decode(*layout, &p) != FA_OK) return 0;
             return p.fused ? 1 : 3;
         }
         case 3: {           // fa_decode_step: the fused decode kernel alone, or fa_append + fa_decode_attention
-            DecodePlan p;
+            CallPlan p;
             if (plan_decode(*layout, &p) != FA_OK) return 0;
             return step_in_one_launch(*layout, p) ? 1 : 1 + (p.fused ? 1 : 3);
         }
         case 4: {           // plan query: the split build of the fused decode kernel
-            DecodePlan p;
+            CallPlan p;
             if (plan_decode(*layout, &p) != FA_OK) return 0;
             return (p.fused && p.split) ? 1 : 0;
         }
         case 5: {           // plan query: residue classes per batch of the transform kernel (0: the direct kernel)
-            DecodePlan p;
+            CallPlan p;
             if (plan_decode(*layout, &p) != FA_OK) return 0;
             return p.algo == FA_DECODE_FFT ? p.nb : 0;
         }
         case 6: {           // plan query: CTAs per (batch, KV head, pass) of the decode kernel
-            DecodePlan p;
+            CallPlan p;
             if (plan_decode(*layout, &p) != FA_OK) return 0;
             return p.n_part;
+        }
+        case 7: {           // plan query: kernels of a decode call in the channel form (0: not taken)
+            CallPlan p;
+            if (plan_decode(*layout, &p) != FA_OK) return 0;
+            return p.chan.on ? 3 : 0;
         }
         default: return 0;
     }

@@ -56,6 +56,22 @@ inline CacheDev make_cache(const fa_cache& c) {
     return o;
 }
 
+// Plan of the channel form of the decode call (fa_decode_chan.cu).
+struct ChanPlan {
+    int on;                  // 1: AUTO takes it where the workspace has room
+    int n_pass;              // passes over a KV head's query heads
+    int nh, hp;              // heads of a pass (at most 4), and heads that a token's columns have room for (2 or 4)
+    int slots;               // S = T / P
+    int ns_c, ns_w;          // stages of a warp's ring: class parts, window parts
+    int stage_c;             // bytes of a class part's stage (K or V rows)
+    int ring, smem;          // bytes of a warp's ring, of the main kernel's shared memory
+    int k_sh, k_mask, v_sh, v_mask;      // swizzle of the K / V rows in a stage: chunk ^ ((row >> sh) & mask)
+    int n_cx, n_wpart;       // CTAs per (KV head, pass): class parts of all batch rows, window parts of one
+    int nq, nz;              // channel pairs per CTA of the kernels in front and behind, and CTAs of their clusters
+    int st_in, st_out;       // stages of their streams of coefficient rows
+    size_t off_z, off_w, off_mw, off_ml, off_o, off_g, off_x, off_j, off_p, total;
+};
+
 // Plan of one fa_decode_attention call; a pure function of the layout so that
 // fa_workspace_bytes and the launch agree.
 struct DecodePlan {
@@ -74,6 +90,10 @@ struct DecodePlan {
     int split;         // 1: the split build of the fused kernel (a tile group of warps beside the transform group)
     // workspace offsets in bytes
     size_t off_bar, off_u, off_ml, off_o, off_z, off_oc, off_om, off_cnt, total;
+};
+// The same with the plan of the channel form, whose kernels take only that (and the others not: a launch copies its parameters).
+struct CallPlan : DecodePlan {
+    ChanPlan chan;
 };
 
 // V^mu of bf16 caches is stored with its 16-byte chunks (8 dims) permuted inside each row:
@@ -95,7 +115,7 @@ __host__ __device__ inline int v_mid_col(int a, int e, int nfv, int dtype) {
     return ((((e >> 3) ^ v_swz(a, nfv >> 3)) << 3) | (e & 7));
 }
 
-fa_status plan_decode(const fa_layout& l, DecodePlan* plan);
+fa_status plan_decode(const fa_layout& l, CallPlan* plan);
 fa_status decode_scratch_bytes(const fa_layout* layout, size_t* out);      // what fa_decode_attention needs of a workspace
 int sm_count();                          // SMs of the current device, cached per device
 bool cooperative_launch_supported();     // of the current device, cached per device
@@ -151,6 +171,11 @@ cudaError_t launch_decode_direct(const Dims&, const CacheDev&, int dtype, const 
 // k_new / v_new non-null: a fused step (the push of Eq.5 rides on the decode launch; fused plans with one pass only).
 cudaError_t launch_decode_fft(const Dims&, const CacheDev&, int dtype, const DecodePlan&, const void* q, void* out, char* ws,
                               const void* k_new, const void* v_new, cudaStream_t);
+// The channel form (fa_decode_chan.cu): its plan, its areas of the workspace, its launches (k_new / v_new: behind a push).
+bool plan_channels(const Dims&, int log2S, int sms, ChanPlan*);
+size_t place_channels(const Dims&, int log2S, size_t off, ChanPlan*);
+cudaError_t launch_decode_channels(const Dims&, const CacheDev&, const ChanPlan&, int log2S, const void* q, void* out, const void* k_new, const void* v_new, char* ws,
+                                   cudaStream_t, bool* begun);
 size_t decode_fft_smem_bytes(const Dims&, int log2S, int gh, int nb, int occ = 1, int split = 0);
 bool decode_fft_fused_fits(const Dims&, int log2S, int gh, int nb, int n_part, int occ = 1, int split = 0);
 bool decode_fft_launchable(const Dims&, const DecodePlan&);

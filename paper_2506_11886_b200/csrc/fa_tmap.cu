@@ -17,29 +17,29 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-bool window_map(CUtensorMap* tm, const void* base, int rows, int d, int n_bh) {
+bool window_map(CUtensorMap* tm, const void* base, int rows, int d, int n_bh, int box_rows) {
     std::memset(tm, 0, sizeof(*tm));
     if (rows <= 0 || !base) return false;
     // A direct-mapped table: a model has four window buffers per layer, all of them used once per token, so a list of the
     // last few maps would encode every one anew.
-    struct Entry { const void* base; int rows, d, n_bh; CUtensorMap tm; };
+    struct Entry { const void* base; int rows, d, n_bh, box; CUtensorMap tm; };
     constexpr int kEntries = 1024;
     static Entry cache[kEntries];
     static std::mutex mu;
-    const uint64_t key = (reinterpret_cast<uint64_t>(base) >> 4) * 0x9E3779B97F4A7C15ull;
+    const uint64_t key = ((reinterpret_cast<uint64_t>(base) >> 4) + (uint64_t)box_rows) * 0x9E3779B97F4A7C15ull;
     Entry& e = cache[key >> 54];
     std::lock_guard<std::mutex> lock(mu);
-    if (e.base == base && e.rows == rows && e.d == d && e.n_bh == n_bh) { *tm = e.tm; return true; }
+    if (e.base == base && e.rows == rows && e.d == d && e.n_bh == n_bh && e.box == box_rows) { *tm = e.tm; return true; }
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)rows, (cuuint64_t)n_bh};
     cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)rows * d * 2};
-    cuuint32_t box[3] = {64, 64, 1};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     if (fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
-    e = Entry{base, rows, d, n_bh, *tm};
+    e = Entry{base, rows, d, n_bh, box_rows, *tm};
     return true;
 }
 
