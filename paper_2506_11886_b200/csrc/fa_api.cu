@@ -375,8 +375,7 @@ static size_t decode_room_bytes(const fa_layout& l, size_t least) {
 }
 
 // Scratch of the compression by block moments: behind that of the decode call (a decode step may run on another stream while a
-// prompt is compressed), in two halves (neighbouring launches alternate between them), each for as many batch rows as
-// kMomScratch holds (at least one).
+// prompt is compressed), for the moments of up to kMomLayers layers, as many batch rows as kMomScratch holds (at least one).
 constexpr size_t kMomScratch = size_t(192) << 20;
 static size_t compress_scratch_bytes(const fa_layout& l) {
     const Dims s = make_dims(l);
@@ -385,7 +384,7 @@ static size_t compress_scratch_bytes(const fa_layout& l) {
     if (row == 0) return 0;
     size_t rows = kMomScratch / row;
     if (rows < 1) rows = 1;
-    if (rows > 2 * (size_t)s.B) rows = 2 * (size_t)s.B;
+    if (rows > (size_t)kMomLayers * s.B) rows = (size_t)kMomLayers * s.B;
     return rows * row;
 }
 // Where the moments of a call go and how many bytes there are (0: the direct contraction).
@@ -612,34 +611,53 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
     // leave, and wait for layer i (hence for everything before it) only in front of their reductions.
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const bool ordered = (flags & FA_COMPRESS_ORDERED) != 0;
-    // Block moments where every layer's fit the workspace: two halves where it has them, so that a layer's moments are formed
-    // while the layer's before are still read.
-    size_t half = 0;
+    // Block moments where every layer's fit the workspace, those of several layers of one shape side by side for one projection.
+    size_t most = 0;
     bool moments = !ordered;
     MomentRoom room = {nullptr, ~size_t(0)};
+    auto moment_bytes = [&](int i) { const Dims s = make_dims(layouts[i]); return (size_t)s.B * compress_mom_row_bytes(s, mid_of(s, L)); };
     for (int i = 0; i < n_layers && moments; ++i) {
-        const Dims s = make_dims(layouts[i]);
         const MomentRoom r = moment_room(layouts[i], ws, ws_bytes);
         moments = r.at != nullptr;
         if (!moments) break;
         if (r.bytes < room.bytes) room = r;                // (the layer with the largest decode scratch leaves the least)
-        const size_t need = (size_t)s.B * compress_mom_row_bytes(s, mid_of(s, L));
-        half = need > half ? need : half;
+        const size_t need = moment_bytes(i);
+        most = need > most ? need : most;
     }
-    moments = moments && room.bytes >= half;
-    const bool two = moments && room.bytes >= 2 * half;
+    moments = moments && room.bytes >= most;
     for (int i = 0; i < n_layers; ++i) {
         const Dims s = make_dims(layouts[i]);
         if (launch_compress(s, make_cache(caches[i]), layouts[i].kv_dtype, K[i], V[i], stride_b, stride_t, stride_h, L, false, ordered, kTcMinMid,
                             true, cs, i > 0) != cudaSuccess)
             return FA_ERR_CUDA;
     }
-    for (int i = 0; i < n_layers; ++i) {
+    // Groups of layers take the two halves of the room in turn where they fit them, so that a group's moments are formed while
+    // the projection in front still reads its own; else each waits for the one before.
+    const size_t half = room.bytes / 2 / 256 * 256;
+    bool behind_whole = false, odd = false;
+    for (int i = 0, n = 1; i < n_layers; i += n) {
         const Dims s = make_dims(layouts[i]);
         const int64_t sbb = s.B > 1 ? stride_b : 0;
-        char* Y = moments ? room.at + (two && (i & 1) ? half : 0) : nullptr;
-        if ((moments ? launch_compress_mom(s, make_cache(caches[i]), K[i], V[i], sbb, stride_t, stride_h, L, 0, s.B, Y, !two && i > 0, cs)
-                     : launch_compress_tc2(s, make_cache(caches[i]), K[i], V[i], sbb, stride_t, stride_h, L, ordered, true, cs)) != cudaSuccess) {
+        cudaError_t err;
+        n = 1;
+        if (moments) {
+            const size_t need = moment_bytes(i);
+            const size_t fit = need ? room.bytes / need : 1;
+            int alike = 1;                                 // layers of this one's shape from here on
+            while (i + alike < n_layers && std::memcmp(&layouts[i + alike], &layouts[i], sizeof(fa_layout)) == 0) ++alike;
+            const int most_n = fit < (size_t)kMomLayers ? (int)fit : kMomLayers, parts = (alike + most_n - 1) / most_n;
+            n = (alike + parts - 1) / parts;
+            CacheDev c[kMomLayers];
+            for (int j = 0; j < n; ++j) c[j] = make_cache(caches[i + j]);
+            const bool whole = n * need > half;
+            err = launch_compress_mom_layers(s, c, K + i, V + i, n, sbb, stride_t, stride_h, L, room.at + (!whole && odd ? half : 0),
+                                             i > 0 && (whole || behind_whole), cs);
+            behind_whole = whole;
+            odd = !odd;
+        } else {
+            err = launch_compress_tc2(s, make_cache(caches[i]), K[i], V[i], sbb, stride_t, stride_h, L, ordered, true, cs);
+        }
+        if (err != cudaSuccess) {
             // the cluster launch was refused: finish this and the remaining layers one by one (each call redoes its layer in full)
             cudaGetLastError();
             for (int j = i; j < n_layers; ++j) {

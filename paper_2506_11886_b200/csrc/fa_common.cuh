@@ -151,6 +151,9 @@ bool compress_mom_supported(const Dims& s);
 size_t compress_mom_row_bytes(const Dims& s, int n_mid);
 cudaError_t launch_compress_mom(const Dims&, const CacheDev&, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int L, int b0,
                                 int nb, void* Y, bool wait_first, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
+constexpr int kMomLayers = 8;        // layers of a launch_compress_mom_layers call
+cudaError_t launch_compress_mom_layers(const Dims&, const CacheDev*, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
+                                       int64_t sh, int L, void* Y, bool wait_first, cudaStream_t);
 // Tensor-core reconstruction of the dimension selection (fa_select_tc.cu).
 bool reconstruct_tc_supported(const Dims& s, int dtype, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int n_mid);
 size_t reconstruct_tc_scratch_bytes(const Dims& s);

@@ -398,6 +398,8 @@ constexpr int kStagesP = 4;
 // positions start[t] .. start[t + 1] (cut on the host so that every team has the same cost, as in fa_compress_tc2.cu).
 constexpr int kMaxTeamsP = 96;
 struct MomCuts { uint32_t start[kMaxTeamsP + 1]; };
+// Coefficients of the layers of a launch: its batch row b is row b % B of layer b / B.
+struct MomLayers { int n; float *k[kMomLayers], *v[kMomLayers]; int32_t* status[kMomLayers]; };
 
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
@@ -408,7 +410,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 // HP heads share a pair and its basis tiles.  npad: accumulator columns per head (the compressed dims of both sides, up to a
 // multiple of 32); each CTA of a pair brings half of them.
 template <int HP, bool RAG>
-__global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16* __restrict__ Y, Dims s, CacheDev c,
+__global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16* __restrict__ Y, Dims s, const __grid_constant__ MomLayers layers,
                                                                       const __grid_constant__ MomRows rows, const __grid_constant__ MomCuts cuts, int npad) {
     constexpr int kBHalf1 = 128 * 128;                     // room for this CTA's columns of one head: at most 128 rows of 128 bytes
     constexpr int kStage = kABytesP + HP * kBHalf1;
@@ -432,7 +434,8 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
     const int mt = 2 * pair + (int)rank;
     const int n_hg = s.Hkv / HP, ncol = s.dck + s.dcv;
     const uint32_t pos_begin = cuts.start[team], pos_end = cuts.start[team + 1];
-    struct Seg { int b, h0, kb0, kb1; uint32_t g0; };      // batch row of the cache, heads, blocks, first block of the row in the launch
+    int32_t* status = layers.status[0];
+    struct Seg { int b, h0, kb0, kb1; uint32_t g0; };      // batch row, heads, blocks, first block of the row in the launch
     auto seg_at = [&](uint32_t pos) {
         int b, nblk = rows.nblk;
         uint32_t g0, off;
@@ -486,10 +489,10 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                 const uint32_t bytes = (uint32_t)min(nh, max(0, ncol - (int)rank * nh)) * (4 * kMF);
                 for (uint32_t pos = pos_begin; live && pos < pos_end; ++seg) {
                     const Seg g = seg_at(pos);
-                    if (seg > 0 && !mbar_wait(epi_done, (seg - 1) & 1, fail, c.status)) { live = false; break; }
+                    if (seg > 0 && !mbar_wait(epi_done, (seg - 1) & 1, fail, status)) { live = false; break; }
                     for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
                         const int st = it % kStagesP;
-                        if (it >= kStagesP && !mbar_wait(empty + st, ((it / kStagesP) - 1) & 1, fail, c.status)) { live = false; break; }
+                        if (it >= kStagesP && !mbar_wait(empty + st, ((it / kStagesP) - 1) & 1, fail, status)) { live = false; break; }
                         unsigned char* bdst = stage0 + (size_t)st * kStage + kABytesP;
                         mbar_expect_tx(full + st, HP * bytes);
                         const char* src = reinterpret_cast<const char*>(Y) +
@@ -515,7 +518,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                     for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
                         const int st = it % kStagesP;
                         const uint32_t par = (it / kStagesP) & 1;
-                        if (!mbar_wait(full + st, par, fail, c.status) || !mbar_wait(peer + st, par, fail, c.status)) { live = false; break; }
+                        if (!mbar_wait(full + st, par, fail, status) || !mbar_wait(peer + st, par, fail, status)) { live = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint32_t a_addr = smem_u32(stage0 + (size_t)st * kStage), b_addr = a_addr + kABytesP;
                         // rows of 128 bytes, 32 hi and 32 lo values: hi hi, lo hi, hi lo, sixteen values at a time
@@ -539,7 +542,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                 for (int it = 0; it < n_it; ++it) {
                     const int st = it % kStagesP;
                     const uint32_t par = (it / kStagesP) & 1;
-                    if (!mbar_wait(full + st, par, fail, c.status)) break;
+                    if (!mbar_wait(full + st, par, fail, status)) break;
                     mbar_arrive_cluster(peer + st, 0);
                 }
             }
@@ -592,7 +595,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                     const float f = (float)ph * inv_T;     // in half turns, [0, 2)
                     const float an = 3.14159265358979f * (f - (f >= 1.0f ? 2.0f : 0.0f));
                     const float C = __cosf(an), S = __sinf(an);
-                    if (it >= kStagesP && !mbar_wait(empty + st, ((it / kStagesP) - 1) & 1, fail, c.status)) { live = false; break; }
+                    if (it >= kStagesP && !mbar_wait(empty + st, ((it / kStagesP) - 1) & 1, fail, status)) { live = false; break; }
                     unsigned char* a_dst = stage0 + (size_t)st * kStage;
                     uint32_t h0[4], l0[4], h1[4], l1[4];
 #pragma unroll
@@ -612,7 +615,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                 }
                 if (!live) break;
                 // ---------------- epilogue of the segment: accumulators are added to the coefficient rows ----------------
-                const bool ok = mbar_wait(acc_ready, seg & 1, fail, c.status);
+                const bool ok = mbar_wait(acc_ready, seg & 1, fail, status);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 asm volatile("griddepcontrol.wait;" ::: "memory");      // (the coefficients are cleared by a kernel before this one)
                 if (!ok) break;
@@ -622,6 +625,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                     // 32 rows x 32 columns at a time through the idle ring: then eight lanes hold a row's 128 bytes
                     float* tile = reinterpret_cast<float*>(stage0) + (warp - 2) * (32 * 36);
                     const int npc = (ncol + 31) >> 5;      // pieces of 32 columns per head
+                    const int layer = RAG ? 0 : g.b / s.B;
 #pragma unroll 1
                     for (int pc = part; pc < HP * npc; pc += 2) {
                         const int hh = pc / npc, c0 = (pc - hh * npc) * 32;
@@ -634,7 +638,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                         if (col < ncol) {
                             const bool is_k = col < s.dck;
                             const int nc = is_k ? s.dck : s.dcv;
-                            float* dst = coef_rows(is_k ? c.coef_k : c.coef_v, s, g.b, g.h0 + hh, nc) + (size_t)(m_base + rr0) * nc + (is_k ? col : col - s.dck);
+                            float* dst = coef_rows(is_k ? layers.k[layer] : layers.v[layer], s, g.b - layer * s.B, g.h0 + hh, nc) + (size_t)(m_base + rr0) * nc + (is_k ? col : col - s.dck);
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
                                 const float4 x = *reinterpret_cast<const float4*>(tile + (rr0 + 4 * i) * 36 + 4 * q);
@@ -651,7 +655,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive(epi_done);
-                    if (!mbar_wait(epi_done, seg & 1, fail, c.status)) break;
+                    if (!mbar_wait(epi_done, seg & 1, fail, status)) break;
                 }
             }
         }
@@ -659,6 +663,8 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     cluster_sync_all();
+    if (tid == 0 && *fail)                                 // (a wait that runs out tells the first layer)
+        for (int l = 1; l < layers.n; ++l) layers.status[l][0] = status[0];
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(HP * 256) : "memory");
@@ -716,7 +722,10 @@ cudaError_t launch_moments(const CUtensorMap& tmK, const CUtensorMap& tmV, const
 }
 
 template <int HP, bool RAG>
-cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev& c, const MomRows& rows, cudaStream_t stream) {
+cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int n_layers, const MomRows& rows, cudaStream_t stream) {
+    MomLayers layers = {};
+    layers.n = n_layers;
+    for (int i = 0; i < n_layers; ++i) { layers.k[i] = c[i].coef_k; layers.v[i] = c[i].coef_v; layers.status[i] = c[i].status; }
     const size_t smem = (size_t)kStagesP * (kABytesP + HP * 128 * 128) + 8 * (3 * kStagesP + 2) + 16 + 1024;
     cudaError_t err = ensure_dynamic_smem(moment_project_kernel<HP, RAG>, smem);
     if (err != cudaSuccess) return err;
@@ -801,7 +810,7 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev& c, cons
     while (!walk(lo, cuts.start)) ++lo;
     cuts.start[n_teams] = (uint32_t)total;
     cfg.gridDim = dim3(2 * n_teams * n_pairs);
-    return cudaLaunchKernelEx(&cfg, moment_project_kernel<HP, RAG>, static_cast<const bf16*>(Y), s, c, rows, cuts, npad_of(s));
+    return cudaLaunchKernelEx(&cfg, moment_project_kernel<HP, RAG>, static_cast<const bf16*>(Y), s, layers, rows, cuts, npad_of(s));
 }
 
 }  // namespace
@@ -821,6 +830,24 @@ bool compress_mom_supported(const Dims& s) {
 size_t compress_mom_row_bytes(const Dims& s, int n_mid) {
     const int R = block_tokens(s);
     return (size_t)((n_mid + R - 1) / R) * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
+}
+
+static cudaError_t launch_rows(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
+                               int64_t sh, int L, MomRows rows, char* Y, bool wait_first, cudaStream_t stream) {
+    const bool rag = rows.lens.n != 0;
+    cudaError_t err;
+    for (int i = 0; i < n_layers; ++i) {
+        CUtensorMap tmK, tmV;
+        if (!prefill_map(&tmK, K[i], s, sb, st, sh, L) || !prefill_map(&tmV, V[i], s, sb, st, sh, L)) return cudaErrorInvalidValue;
+        char* y = Y + (size_t)i * rows.total * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
+        if (s.d == 128) err = rag ? launch_moments<128, true>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream) : launch_moments<128, false>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream);
+        else err = rag ? launch_moments<64, true>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream) : launch_moments<64, false>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream);
+        if (err != cudaSuccess) return err;
+    }
+    rows.nb *= n_layers;
+    rows.total *= n_layers;
+    if (s.Hkv % 2 == 0) return rag ? launch_project<2, true>(Y, s, c, n_layers, rows, stream) : launch_project<2, false>(Y, s, c, n_layers, rows, stream);
+    return rag ? launch_project<1, true>(Y, s, c, n_layers, rows, stream) : launch_project<1, false>(Y, s, c, n_layers, rows, stream);
 }
 
 // Coefficients (the caller has zeroed them) and the kept-dim rows of the middle tokens of batch rows b0 .. b0 + nb; the windows
@@ -850,16 +877,23 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
         rows.total = rows.nblk * nb;
     }
     if (rows.total == 0) return cudaSuccess;
-    CUtensorMap tmK, tmV;
-    if (!prefill_map(&tmK, K, s, sb, st, sh, L) || !prefill_map(&tmV, V, s, sb, st, sh, L))
-        return cudaErrorInvalidValue;
-    const bool rag = rows.lens.n != 0;
-    cudaError_t err;
-    if (s.d == 128) err = rag ? launch_moments<128, true>(tmK, tmV, s, c, L, rows, Y, wait_first, stream) : launch_moments<128, false>(tmK, tmV, s, c, L, rows, Y, wait_first, stream);
-    else err = rag ? launch_moments<64, true>(tmK, tmV, s, c, L, rows, Y, wait_first, stream) : launch_moments<64, false>(tmK, tmV, s, c, L, rows, Y, wait_first, stream);
-    if (err != cudaSuccess) return err;
-    if (s.Hkv % 2 == 0) return rag ? launch_project<2, true>(Y, s, c, rows, stream) : launch_project<2, false>(Y, s, c, rows, stream);
-    return rag ? launch_project<1, true>(Y, s, c, rows, stream) : launch_project<1, false>(Y, s, c, rows, stream);
+    return launch_rows(s, &c, &K, &V, 1, sb, st, sh, L, rows, static_cast<char*>(Y), wait_first, stream);
+}
+
+// The same for all batch rows of up to kMomLayers layers of one shape: a moment kernel each, then one projection.  A projection
+// takes 31 us for a layer of 8 heads, 32K tokens and 1024 coefficients, a third of it its start and the segments that teams
+// share, which six layers together pay once: 6 x 31 -> 146 us.  Y: room for the moments of all of them.
+cudaError_t launch_compress_mom_layers(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
+                                       int64_t sh, int L, void* Y, bool wait_first, cudaStream_t stream) {
+    if (n_layers < 1 || n_layers > kMomLayers) return cudaErrorInvalidValue;
+    MomRows rows = {};
+    rows.R = block_tokens(s);
+    rows.nb = s.B;
+    rows.nblk = (mid_of(s, L) + rows.R - 1) / rows.R;
+    rows.total = rows.nblk * s.B;
+    if (rows.total == 0) return cudaSuccess;
+    if ((long long)rows.nblk * s.B * n_layers >= (1ll << 24)) return cudaErrorInvalidValue;
+    return launch_rows(s, c, K, V, n_layers, sb, st, sh, L, rows, static_cast<char*>(Y), wait_first, stream);
 }
 
 }  // namespace fa

@@ -78,7 +78,7 @@ def _row_bytes(layout, n_mid):
 
 def _workspace(layout, n_mid, rows, short=0):
     """A workspace with room for the moments of `rows` rows of n_mid middle tokens, less `short` bytes."""
-    decode = fa.fa_workspace_bytes(layout) - 2 * layout.batch * _row_bytes(layout, layout.max_mid)
+    decode = fa.fa_workspace_bytes(layout) - 8 * layout.batch * _row_bytes(layout, layout.max_mid)
     return torch.zeros(decode + rows * _row_bytes(layout, n_mid) - short, dtype=torch.uint8, device="cuda")
 
 
@@ -106,17 +106,17 @@ def test_groups_of_rows_and_the_direct_contraction_agree(ragged, strided):
         assert not ws[:4096].any()                        # the barrier counters of the decode call are left alone
 
 
-@pytest.mark.parametrize("halves", [1, 2])
-def test_layers_in_one_call_and_replayed_from_a_graph(halves):
+@pytest.mark.parametrize("room,B", [(1, 1), (2, 1), (3, 1), (4, 1), (7, 1), (4, 2)])      # layers whose moments the workspace holds
+def test_layers_in_one_call_and_replayed_from_a_graph(room, B):
     """Layers with scratch for one or two layers at a time, with inputs that change between the replays of a graph."""
-    shape = _shape(B=1, L=3000, Hkv=4, Hq=4)
+    shape = _shape(B=B, L=3000, Hkv=4, Hq=4)
     layout = layout_of(shape, max_mid=shape.T, P=16)
     n = 4
     streams = [synth.KVStream(shape, seed=20 + i, device="cuda", freq="offgrid") for i in range(n)]
     toks = [[s.tokens(t, t + shape.L, work_dtype=torch.float32) for s in streams] for t in (0, 1000)]
     K, V = ([torch.empty_like(p[0]) for p in toks[0]] for _ in range(2))
     caches = [_cache(layout, s) for s in streams]
-    ws = _workspace(layout, shape.L - 68, halves)
+    ws = _workspace(layout, shape.L - 68, room * B)
 
     def fill(which):
         for i in range(n):
