@@ -624,6 +624,11 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                                                                   char* wsp, const bf16* __restrict__ k_new,
                                                                   const bf16* __restrict__ v_new) {
     constexpr bool step = STEP;
+    // What an instance cannot meet is not in it (its code is fetched cold on every call): two CTAs to an SM are lone parts of their
+    // heads, a step is always the fused kernel.  The latter is left to run time for the long transforms, where the smaller
+    // instance was the slower one (a 2K chat's step 25.9 -> 25.3 us with it, a step at 32K 34.0 -> 34.3).
+    const bool fused = (STEP && LS <= 8) || OCC == 2 || p.fused;
+    const int n_part = OCC == 2 ? 1 : p.n_part, n_split = OCC == 2 ? 1 : p.n_split, n_wsplit = OCC == 2 ? 0 : p.n_wsplit;
     constexpr int N = GH / 2;
     constexpr int S = 1 << LS;
     // Short transforms have fewer pairs of bins than threads: up to 2^kLgPair neighbouring lanes share a pair and take a
@@ -659,7 +664,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     const int fb_floats = L.fb_floats, pbs = L.pbs;
 
     const int part = blockIdx.x;                          // partial-result index: class CTAs, then window CTAs
-    const bool is_win = part >= p.n_split;
+    const bool is_win = part >= n_split;
     const int h = idiv(blockIdx.y, p.n_pass), pass = blockIdx.y - h * p.n_pass;
     const int b = blockIdx.z;
     const int g_first = h * s.G + pass * GH;
@@ -701,7 +706,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     }
     // This part's rows of C^K start towards the transform buffers, and its rows of C^V towards L2, as soon as
     // the kernels before this one are done (the previous step's kernel writes coefficient rows).
-    const int m0 = 4 * idiv(part * (s.M >> 2), p.n_part), m1 = 4 * idiv((part + 1) * (s.M >> 2), p.n_part);
+    const int m0 = 4 * idiv(part * (s.M >> 2), n_part), m1 = 4 * idiv((part + 1) * (s.M >> 2), n_part);
     // rows of C^K staged at a time: the transform buffers and, behind them, the kept-dim score and probability
     // buffers (one contiguous area, all idle until the first batch)
     const int uch = L.uch;
@@ -740,7 +745,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
         }
     };
     // fused kernel: everything below reads what earlier kernels in the stream wrote (state, cache, coefficients, q)
-    if (p.fused) {
+    if (fused) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         SPAN(1);
         start_coef_rows();
@@ -786,12 +791,12 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             *reinterpret_cast<uint4*>(xrow_s + side * s.d + 8 * ch) =
                 *reinterpret_cast<const uint4*>((side == 0 ? k_new : v_new) + ((size_t)b * s.Hkv + h) * s.d + 8 * ch);
     }
-    const int c0 = is_win ? 0 : part * s.P / p.n_split;
-    const int c1 = is_win ? 0 : (part + 1) * s.P / p.n_split;
+    const int c0 = is_win ? 0 : part * s.P / n_split;
+    const int c1 = is_win ? 0 : (part + 1) * s.P / n_split;
     const int n_win = n_init + n_local;
     // window tokens: spread over the class CTAs, or over CTAs of their own
-    const int wi = p.n_wsplit ? part - p.n_split : part, wn = p.n_wsplit ? p.n_wsplit : p.n_split;
-    const bool has_win = p.n_wsplit ? is_win : true;
+    const int wi = n_wsplit ? part - n_split : part, wn = n_wsplit ? n_wsplit : n_split;
+    const bool has_win = n_wsplit ? is_win : true;
     const int w0 = has_win ? wi * n_win / wn : 0, w1 = has_win ? (wi + 1) * n_win / wn : 0;
     auto n_of_class = [&](int cls) { return cls < n_mid ? (n_mid - cls + s.P - 1) >> log2P : 0; };
 
@@ -911,7 +916,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     int32_t* bar = ws.bar + 4 * (((size_t)b * s.Hkv + h) * p.n_pass + pass);
     // gathered query of the compressed K dims (one element per thread and round), loaded early
     float qc_early = 0.f;
-    if (p.fused && s.dck > 0 && tid < GH * s.dck) {
+    if (fused && s.dck > 0 && tid < GH * s.dck) {
         const int g = idiv(tid, s.dck), e = tid - g * s.dck;
         if (g < ng) qc_early = __bfloat162float(qs_s[g * s.d + c.idx_comp_k[(size_t)h * s.dck + e]]);
     }
@@ -1000,7 +1005,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                     patch_mid_k(tile + (uint32_t)((astar - a0) * rowb_k), c.idx_full_k + (size_t)h * s.nfk, s.nfk, xrow_s, lane);
                 }
                 // Two groups of the warp at a time, whose loads and products are independent, where registers allow (layer
-                // step at 32 K tokens 35.6 -> 34.0 us, ragged batch 74.7 -> 73.4); one in the two-per-SM and split instances,
+                // step at 32 K tokens 35.6 -> 34.0 us, ragged batch 74.7 -> 73.0); one in the two-per-SM and split instances,
                 // which lose 1-2 % to it.
                 constexpr int U = OCC == 1 && !SPLIT ? 2 : 1;
 #pragma unroll 1
@@ -1056,9 +1061,9 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     // Exchange areas of this (b, KV head, pass): u, and of every part (m, l) per slot, o, z (window parts have no z),
     // its slice of o^c; all in slot order.  u and z as ut / z_s hold them.  A part on its own exchanges nothing.
     constexpr int EF = 2 * GH;                            // floats of an entry of ut / z_s
-    const int np = p.n_part, nz = p.n_split, job = (b * s.Hkv + h) * p.n_pass + pass;
+    const int np = n_part, nz = n_split, job = (b * s.Hkv + h) * p.n_pass + pass;
     float* ug = np > 1 ? ws.u + (size_t)job * (EF * s.k) : ut;
-    if (p.fused) {
+    if (fused) {
         // u_g[m] = scale * log2(e) * w_m * sum_e C^K[m][e] q_g[D^kc[e]] for rows [m0, m1): eight lanes per row
         if (s.dck > 0) {
             float* qc = reinterpret_cast<float*>(o_s);     // [GH][dck] gathered query, fp32 (o_s is not in use yet)
@@ -1121,7 +1126,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
                 }
             }
             TL(2);
-            part_arrive<kAll>(bar + 0, p.n_part, tid);
+            part_arrive<kAll>(bar + 0, n_part, tid);
         }
         TL(3);
     } else {
@@ -1135,9 +1140,9 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
     constexpr int kXf = SPLIT ? kConsumers : kAll, kXfBar = SPLIT ? 2 : 1;
     auto load_u = [&]() {
         if (s.dck == 0) return;
-        if (p.fused) part_wait<kXf, kXfBar>(bar + 0, p.n_part, tid, fail, c.status);
+        if (fused) part_wait<kXf, kXfBar>(bar + 0, n_part, tid, fail, c.status);
         TL(5);
-        if (p.fused) {
+        if (fused) {
             if (np > 1)
                 #pragma unroll 1
                 for (int i = 4 * (int)tid; i < EF * s.k; i += 4 * kXf) cp_async16(ut + i, ug + i);
@@ -1882,7 +1887,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), OCC) decode_fft_kernel(cons
             e[1] = e0 * e[1] + e1 * e[3];
         }
     }
-    if (!p.fused) {
+    if (!fused) {
         // for the epilogue kernel: per head and part
         #pragma unroll 1
         for (int i = tid; i < GH * s.d; i += kAll) {
@@ -2222,16 +2227,14 @@ cudaError_t launch_fft_len(const Dims& s, const CacheDev& c, const DecodePlan& p
                            const void* k_new, const void* v_new, cudaStream_t st) {
     if constexpr (LS <= 8)
         if (p.occ == 2)
-            return step ? launch_fft_t<GH, LS, 2, true>(s, c, p, q, out, ws, step, k_new, v_new, st) : launch_fft_t<GH, LS, 2, false>(s, c, p, q, out, ws, step, k_new, v_new, st);
+            return step ? cudaErrorInvalidValue : launch_fft_t<GH, LS, 2, false>(s, c, p, q, out, ws, step, k_new, v_new, st);      // (more heads than SMs: a step is two launches)
     if constexpr (LS == 10)
         if (p.split)
             return step ? launch_fft_t<GH, LS, 1, true, true>(s, c, p, q, out, ws, step, k_new, v_new, st) : launch_fft_t<GH, LS, 1, false, true>(s, c, p, q, out, ws, step, k_new, v_new, st);
     return step ? launch_fft_t<GH, LS, 1, true>(s, c, p, q, out, ws, step, k_new, v_new, st) : launch_fft_t<GH, LS, 1, false>(s, c, p, q, out, ws, step, k_new, v_new, st);
 }
 template <int GH, int LS>
-int resident_fft_len(const Dims& s, const DecodePlan& p) {
-    if constexpr (LS <= 8)
-        if (p.occ == 2) return resident_ctas_t<GH, LS, 2>(s, p);
+int resident_fft_len(const Dims& s, const DecodePlan& p) {                  // (plans whose parts wait for one another: one CTA to an SM)
     if constexpr (LS == 10)
         if (p.split) return resident_ctas_t<GH, LS, 1, true, false>(s, p);
     return resident_ctas_t<GH, LS, 1>(s, p);
