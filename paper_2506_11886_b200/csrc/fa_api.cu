@@ -538,7 +538,7 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
     bool tc_rows = tc && (tc2 || compress_tc_gathers(s));
     if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, !tc, ordered, tc_rows ? kTcMinMid : kNoTc, true, cs) != cudaSuccess)
         return FA_ERR_CUDA;
-    if (tc2 && launch_compress_tc2(s, make_cache(*cache), K, V, sbb, stride_t, stride_h, L, ordered, tc_rows, cs) != cudaSuccess) {
+    if (tc2 && launch_compress_tc2(s, make_cache(*cache), K, V, sbb, stride_t, stride_h, L, ordered, cs) != cudaSuccess) {
         // the cluster launch was refused (e.g. a partitioned device): the single-CTA kernel does the same work; if it
         // cannot write the kept-dim rows itself, the partition kernel runs once more with them
         cudaGetLastError();
@@ -655,7 +655,7 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
             behind_whole = whole;
             odd = !odd;
         } else {
-            err = launch_compress_tc2(s, make_cache(caches[i]), K[i], V[i], sbb, stride_t, stride_h, L, ordered, true, cs);
+            err = launch_compress_tc2(s, make_cache(caches[i]), K[i], V[i], sbb, stride_t, stride_h, L, ordered, cs);
         }
         if (err != cudaSuccess) {
             // the cluster launch was refused: finish this and the remaining layers one by one (each call redoes its layer in full)
@@ -758,7 +758,7 @@ fa_status fa_compress_ragged(const fa_layout* layout, fa_cache* cache, const voi
                 cudaGetLastError();                       // the cluster launch was refused: these rows and the rest one by one
                 break;
             }
-            if (tc && launch_compress_tc2(s, make_cache(rows), Kb, Vb, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, false, true, cs, &lens,
+            if (tc && launch_compress_tc2(s, make_cache(rows), Kb, Vb, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, false, cs, &lens,
                                           kTcMinMid) != cudaSuccess) {
                 cudaGetLastError();                       // the cluster launch was refused: these rows and the rest one by one
                 break;
@@ -836,7 +836,7 @@ fa_status fa_decode_attention(const fa_layout* layout, const fa_cache* cache, co
 // group takes no part in the update: eight parts or more there.  With more heads than SMs (one part each, two to an SM) one launch
 // gains 1 us at 256 rows and loses 9 at 128 (MHA, batch 8): two launches.
 static bool step_in_one_launch(const fa_layout& l, const DecodePlan& p) {
-    if (!p.fused || p.n_pass != 1) return false;
+    if (!p.fused || p.n_pass != 1 || p.occ != 1) return false;
     if (p.n_part >= 8) return true;
     const int rows = (l.n_coef / 4 + p.n_part - 1) / p.n_part * 4;
     return !p.split && rows <= 260 && (p.n_part >= 2 || l.batch * l.n_kv_heads <= sm_count());
@@ -856,7 +856,7 @@ static fa_status decode_step_impl(const fa_layout* layout, fa_cache* cache, cons
     if (st != FA_OK) return st;
     if (!ws || !aligned16(ws) || ws_bytes < p.total) return FA_ERR_WORKSPACE;
     Dims s = make_dims(*layout);
-    // The push rides on the decode launch where a head has many parts (each then updates a small slice of the
+    // The push rides on the decode launch where step_in_one_launch says so (each part then updates a slice of the
     // coefficient rows as it streams them for u and for the output product).
     // Whether the device can hold all parts at once is asked before anything is enqueued: nothing to undo.
     const bool channels = p.chan.on && ws_bytes >= p.chan.total;

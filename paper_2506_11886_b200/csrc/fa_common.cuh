@@ -145,7 +145,7 @@ bool compress_tc_gathers(const Dims& s);
 // The same path on CTA pairs (fa_compress_tc2.cu): needs an even number of 128-row tiles.
 bool compress_tc2_supported(const Dims& s);
 cudaError_t launch_compress_tc2(const Dims&, const CacheDev&, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh,
-                                int L, bool ordered, bool gather, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
+                                int L, bool ordered, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
 // The contraction by block moments (fa_compress_mom.cu): batch rows b0 .. b0 + nb, moments in Y.
 bool compress_mom_supported(const Dims& s);
 size_t compress_mom_row_bytes(const Dims& s, int n_mid);

@@ -18,7 +18,7 @@
 // What bounds it: the first kernel HBM (per box of 64 tokens of one side 740 to 840 cycles against the 700 that 16 KB take at an SM's
 // share of the measured rate; its write of the moments is 10 % of the traffic at k / T = 1 / 64 and 20 % at 1 / 32), the
 // second the tensor cores (1200 cycles a block and pair against 1152 for its products) plus 8 K cycles of reductions per segment.
-// Direct contraction against this path: six layers of 32 K tokens, 1024 rows: 701 -> 374 us; 128 K tokens, batch 4, 2048 rows:
+// Direct contraction against this path: six layers of 32 K tokens, 1024 rows: 701 -> 374 us, with one projection for all 333; 128 K tokens, batch 4, 2048 rows:
 // 3207 -> 778 us; six ragged rows of 3 to 12 K tokens, 512 rows: 123 -> 85 us; 4 K tokens of 256 heads, 256 rows (T / k = 32, blocks of
 // 192 tokens): 231 -> 221 us.  Relative error of the coefficients 4e-6 against 2.4e-4.
 #include <mutex>
@@ -882,7 +882,7 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
 
 // The same for all batch rows of up to kMomLayers layers of one shape: a moment kernel each, then one projection.  A projection
 // takes 31 us for a layer of 8 heads, 32K tokens and 1024 coefficients, a third of it its start and the segments that teams
-// share, which six layers together pay once: 6 x 31 -> 146 us.  Y: room for the moments of all of them.
+// share, which six layers together pay once: 6 x 31 -> 115 us (ncu; 76 % of the pipe's active cycles).  Y: room for the moments of all of them.
 cudaError_t launch_compress_mom_layers(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
                                        int64_t sh, int L, void* Y, bool wait_first, cudaStream_t stream) {
     if (n_layers < 1 || n_layers > kMomLayers) return cudaErrorInvalidValue;

@@ -34,8 +34,8 @@ __host__ __device__ inline int gather_rounds(int n_pairs, int hp, int nf, int pe
     while (r < 8 && ((kBK / r + n_pairs - 1) / n_pairs) * hp * (nf >> 3) > per_round) r *= 2;
     return r;
 }
-// Warps GW that write the kept-dim rows of the middle from the B boxes, and 16-byte chunks GI per thread and round: as few
-// as hold a stage's items, because the contraction runs at the power cap and idle items and waiting warps cost it clock
+// Warps GW that write the kept-dim rows of the middle from the B boxes, and 16-byte chunks GI per thread and round: the smallest
+// of the instances that holds a stage's items, because the contraction runs at the power cap and idle items and waiting warps cost it clock
 // (32 K tokens: 779 us for six layers with six warps of four items, 751 with four of four, 689 with four of two); eight
 // warps of four where there are more (few pairs per team and many kept dims: every pair writes most rows of its boxes
 // itself; 4 K tokens of the 32-head MHA layout, 48 kept dims: fa_compress 264 us with four warps, 227 with eight, and 320
@@ -67,7 +67,7 @@ template <int D, int HP, int kGatherWarps, int kItems, bool RAG>
 __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                      const __grid_constant__ CUtensorMap tmV, Dims s,
                                                                      CacheDev c, int Lall, const __grid_constant__ TeamCuts cuts,
-                                                                     const __grid_constant__ RowCuts rows, int per, int gather) {
+                                                                     const __grid_constant__ RowCuts rows, int per) {
     constexpr int N = 2 * D;
     constexpr int kABytes = kBM * kBK * 2;                 // 16 KB basis tile
     constexpr int kBoxBytes = kBK * 64 * 2;                // 8 KB per [64 tokens x 64 dims] box
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
             // the pairs of the team load the same boxes and share the tokens: this pair takes rows pair, pair + n_pairs, ...
             const int rounds = kItems == 4 ? gather_rounds(n_pairs, HP, nf_side, kItems * 32 * kGatherWarps) : 1, rpr = kBK / rounds;
             const int n_tok = pair < rpr ? (rpr - pair + n_pairs - 1) / n_pairs : 0;
-            const int n_items = gather ? n_tok * HP * cph : 0;                // per round, <= kItems per thread
+            const int n_items = n_tok * HP * cph;                // per round, <= kItems per thread
             const bool p2 = (s.P & (s.P - 1)) == 0;
             const int lgP = 31 - __clz(s.P);
             int it = 0;
@@ -246,11 +246,10 @@ __global__ void __launch_bounds__(threads_tc(kGatherWarps), 1) compress_tc2_kern
                 const Seg g = seg_at(pos);
                 // the kept dims of this side of the segment's heads (the gather warps, on their own barrier)
                 asm volatile("bar.sync 3, %0;" ::"n"(32 * kGatherWarps) : "memory");
-                if (gather)
-                    for (int i = gt; i < HP * nf_side; i += 32 * kGatherWarps) {
-                        const int hh = i / nf_side, r = i - hh * nf_side;
-                        idf_s[hh * D + r] = (side ? c.idx_full_v : c.idx_full_k)[(size_t)(g.h0 + hh) * nf_side + r];
-                    }
+                for (int i = gt; i < HP * nf_side; i += 32 * kGatherWarps) {
+                    const int hh = i / nf_side, r = i - hh * nf_side;
+                    idf_s[hh * D + r] = (side ? c.idx_full_v : c.idx_full_k)[(size_t)(g.h0 + hh) * nf_side + r];
+                }
                 asm volatile("bar.sync 3, %0;" ::"n"(32 * kGatherWarps) : "memory");
                 // An item = one 16-byte chunk (8 kept dims) of one kept-dim row.  A thread keeps the same items in every
                 // block: token row r of the boxes, head, side and LOGICAL chunk, so the eight source offsets inside a stage
@@ -500,7 +499,7 @@ bool make_map2(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int
 
 template <int D, int HP, int GW, int GI, bool RAG>
 cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, const RowCuts& rows,
-                         bool ordered, bool gather, cudaStream_t stream) {
+                         bool ordered, cudaStream_t stream) {
     constexpr size_t stage = (size_t)kBM * kBK * 2 + (size_t)HP * (D / 64) * kBK * 64 * 2;
     constexpr size_t n_stages = (200 * 1024) / stage < 6 ? (200 * 1024) / stage : 6;
     const size_t smem = n_stages * stage + 8 * (3 * n_stages + 3) + 16 + sizeof(int) * HP * D + 64 + 1024;
@@ -592,7 +591,7 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
         cuts.start[n_teams] = (uint32_t)total;
     }
     cfg.gridDim = dim3(2 * n_teams * n_pairs);
-    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW, GI, RAG>, tmK, tmV, s, c, L, cuts, rows, per, gather ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, compress_tc2_kernel<D, HP, GW, GI, RAG>, tmK, tmV, s, c, L, cuts, rows, per);
 }
 
 }  // namespace
@@ -600,11 +599,11 @@ cudaError_t launch_tc2_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const D
 // True if the pair kernel serves this layout: what the single-CTA kernel needs, and an even number of row tiles.
 bool compress_tc2_supported(const Dims& s) { return s.M % (2 * kBM) == 0; }
 
-// Coefficients (the caller has zeroed them) and, with gather, the kept-dim rows of the middle tokens; the windows
+// Coefficients (the caller has zeroed them) and the kept-dim rows of the middle tokens; the windows
 // and the counters are the caller's (the partition kernel).  lens: prompt lengths of the batch rows (at most L; rows with
 // fewer than tc_min middle tokens are left out), or none.
 cudaError_t launch_compress_tc2(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb, int64_t st,
-                                int64_t sh, int L, bool ordered, bool gather, cudaStream_t stream, const RowLens* lens, int tc_min) {
+                                int64_t sh, int L, bool ordered, cudaStream_t stream, const RowLens* lens, int tc_min) {
     RowCuts rows = {};
     if (lens && lens->n) {
         if (ordered || lens->n != s.B) return cudaErrorInvalidValue;
@@ -625,15 +624,15 @@ cudaError_t launch_compress_tc2(const Dims& s, const CacheDev& c, const void* K,
     if (!make_map2(&tmK, K, s, sb, st, sh, L) || !make_map2(&tmV, V, s, sb, st, sh, L)) return cudaErrorInvalidValue;
     const bool pair = s.Hkv % 2 == 0;                        // two heads share a CTA pair and its basis tiles
     const int nf = s.nfk > s.nfv ? s.nfk : s.nfv;
-    const int n_pairs = s.M / (2 * kBM), items = gather ? (kBK + n_pairs - 1) / n_pairs * (pair ? 2 : 1) * (nf >> 3) : 0;
+    const int n_pairs = s.M / (2 * kBM), items = (kBK + n_pairs - 1) / n_pairs * (pair ? 2 : 1) * (nf >> 3);
     auto go = [&](auto d, auto hp) {
         if (rows.lens.n)
-            return items <= 256 ? launch_tc2_t<d, hp, 4, 2, true>(tmK, tmV, s, c, L, rows, ordered, gather, stream)
-                                : launch_tc2_t<d, hp, 8, 4, true>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
-        if (items <= 64) return launch_tc2_t<d, hp, 2, 1, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
-        if (items <= 128) return launch_tc2_t<d, hp, 4, 1, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
-        if (items <= 256) return launch_tc2_t<d, hp, 4, 2, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
-        return launch_tc2_t<d, hp, 8, 4, false>(tmK, tmV, s, c, L, rows, ordered, gather, stream);
+            return items <= 256 ? launch_tc2_t<d, hp, 4, 2, true>(tmK, tmV, s, c, L, rows, ordered, stream)
+                                : launch_tc2_t<d, hp, 8, 4, true>(tmK, tmV, s, c, L, rows, ordered, stream);
+        if (items <= 64) return launch_tc2_t<d, hp, 2, 1, false>(tmK, tmV, s, c, L, rows, ordered, stream);
+        if (items <= 128) return launch_tc2_t<d, hp, 4, 1, false>(tmK, tmV, s, c, L, rows, ordered, stream);
+        if (items <= 256) return launch_tc2_t<d, hp, 4, 2, false>(tmK, tmV, s, c, L, rows, ordered, stream);
+        return launch_tc2_t<d, hp, 8, 4, false>(tmK, tmV, s, c, L, rows, ordered, stream);
     };
     using std::integral_constant;
     if (s.d == 128) return pair ? go(integral_constant<int, 128>{}, integral_constant<int, 2>{}) : go(integral_constant<int, 128>{}, integral_constant<int, 1>{});
