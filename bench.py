@@ -322,7 +322,7 @@ def bench_compress_layers(torch, fa, synth, dev, n_layers, bf16_peak):
     caches = [fa.Cache(layout, stream.idx_full_k, stream.idx_full_v, device=dev) for _ in range(n_layers)]
     for c in caches[:2]:
         fa.fa_compress(layout, c, Kp, Vp, ws)
-    layouts, Ks, Vs = [layout] * n_layers, [Kp] * n_layers, [Vp] * n_layers
+    layouts, Ks, Vs = [layout] * n_layers, [Kp.clone() for _ in range(n_layers)], [Vp.clone() for _ in range(n_layers)]      # a tensor per layer, as a prefill leaves them
     fa.fa_compress_layers(layouts, caches, Ks, Vs, ws)
     torch.cuda.synchronize()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -334,8 +334,8 @@ def bench_compress_layers(torch, fa, synth, dev, n_layers, bf16_peak):
         torch.cuda.synchronize()
         tot.append(ev0.elapsed_time(ev1))
         ev0.record()
-        for c in caches:
-            fa.fa_compress(layout, c, Kp, Vp, ws)                    # the same work as n_layers single calls
+        for c, K, V in zip(caches, Ks, Vs):
+            fa.fa_compress(layout, c, K, V, ws)                      # the same work as n_layers single calls
         ev1.record()
         torch.cuda.synchronize()
         single.append(ev0.elapsed_time(ev1))
@@ -343,13 +343,13 @@ def bench_compress_layers(torch, fa, synth, dev, n_layers, bf16_peak):
     flop = 2.0 * shape.M * n_mid0 * ((shape.d - shape.n_full_k) + (shape.d - shape.n_full_v)) * shape.Hkv * shape.B * n_layers
     tf = flop / (min(tot) * 1e-3) / 1e12
     tf1 = flop / (min(single) * 1e-3) / 1e12
-    out = {"workload": shape.name, "layers": n_layers, "call": "fa_compress_layers (one call; the layers' kernels overlap)",
+    out = {"workload": shape.name, "layers": n_layers, "call": "fa_compress_layers (one call; up to eight layers share a projection)",
            "total_ms": min(tot), "ms_per_layer": min(tot) / n_layers,
            "useful_tflops": tf, "frac_of_bf16_tflops": tf / bf16_peak if bf16_peak else None,
            "single_calls_ms_per_layer": min(single) / n_layers, "single_calls_useful_tflops": tf1,
            "single_calls_frac_of_bf16_tflops": tf1 / bf16_peak if bf16_peak else None,
-           "note": "same prefill tensor for every layer (3.1 GB of K/V per layer would not change the kernel's work)"}
-    del caches, Kp, Vp
+           "note": "useful FLOPs are those of the projection as Eq.3 states it; the block moments do about a quarter of them"}
+    del caches, Kp, Vp, Ks, Vs
     torch.cuda.empty_cache()
     return out
 
@@ -510,7 +510,7 @@ def run_ours(args):
     if args.config == 1:
         rd, wr = profile_counter("decode_cfg1", "decode", "dram read"), profile_counter("decode_cfg1", "decode", "dram write")
         traffic = int(rd + wr) if rd is not None and wr is not None else None
-    tensor_pct = profile_counter("compress_cfg1", "compress_tc", "tensor pipe % (active cycles)")
+    tensor_pct = profile_counter("compress_cfg1", "moment_project", "tensor pipe % (active cycles)")
     line = {
         "metric": METRIC if args.config == 1 else f"decode_attn_us_per_step_cfg{args.config}", "value": us_step / world, "unit": UNIT,
         "n_gpus": world, "steps": K_steps, "warmup": W,
@@ -526,7 +526,7 @@ def run_ours(args):
                       "compress_ms_per_layer": min(comp_ms), "compress_tflops": comp_flop / (min(comp_ms) * 1e-3) / 1e12,
                       "compress_frac_of_bf16_tflops": comp_flop / (min(comp_ms) * 1e-3) / 1e12 / bf16_peak,
                       "compress_tensor_pipe_pct": tensor_pct,
-                      "compress_path": "tcgen05.mma.cta_group::2 bf16 x bf16 -> f32 (TMEM), CTA pairs, basis tiles generated in registers",
+                      "compress_path": "tcgen05.mma bf16 x bf16 -> f32 (TMEM): block moments, then their projection on CTA pairs (cta_group::2)",
                       "compress_fft_ms_per_layer": min(comp_fft_ms),
                       "compress_fft_frac_of_hbm": prefill_bytes / (min(comp_fft_ms) * 1e-3) / 1e9 / _peaks()[0],
                       "compress_ordered_ms_per_layer": min(comp_ord_ms),
