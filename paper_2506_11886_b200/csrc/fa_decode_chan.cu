@@ -176,10 +176,11 @@ struct RowStream {
         mbar_wait(bar + i % n_st, (uint32_t)(i / n_st) & 1u, fail, status);
         return buf + (size_t)(i % n_st) * kStageRows * nc;
     }
-    __device__ __forceinline__ void done(int i, int tid) const {       // (all threads)
+    __device__ __forceinline__ void done(int i, int n, int tid) const {          // stages i .. i + n (all threads)
         if (i + n_st < n_chunk) {
             __syncthreads();
-            if (tid == 0) issue(i + n_st);
+            if (tid == 0)
+                for (int x = i; x < i + n && x + n_st < n_chunk; ++x) issue(x + n_st);
         }
     }
 };
@@ -277,41 +278,64 @@ __global__ void __launch_bounds__(kChanThreads) chan_in_kernel(Dims s, CacheDev 
     const float w_gen = sl2 * (s.norm == FA_NORM_PAPER ? 1.0f / (float)s.k : 2.f * inv_T), w_0 = s.norm == FA_NORM_PAPER ? w_gen : 0.5f * w_gen, w_1 = s.norm == FA_NORM_PAPER ? w_gen : 0.f;
     const uint32_t u_peer = CL > 1 ? peer_addr(smem_addr(u_s), (uint32_t)(l8 < CL ? l8 : 0)) : smem_addr(u_s);
     cluster_meet(CL);                                      // every CTA of the cluster has started: its shared memory can be written
-    for (int i = 0; i < rs.n_chunk; ++i) {
-        const float* xs = rs.wait(i, fail, c.status);
-        const int rows = min(kStageRows, rs.rows - i * kStageRows), m = m0 + i * kStageRows + rgi;
-        float a[4] = {0.f, 0.f, 0.f, 0.f};
-        if (rgi < rows) {
-            const float f = pu.j >= 0 ? f_s[m - m0] : 0.f;
-#pragma unroll 4
+    // two stages at a time: eight lanes take a row of each, so that a turn's chain (row, sums over lanes, barrier) is paid half as
+    // often and the query's columns are read once for both (a step of 8 rows of 32 heads, 4K tokens 101.8 -> 100.3 us, of 4 rows of
+    // 128K tokens 192.8 -> 190.5, with the same in the last kernel)
+    for (int i = 0; i < rs.n_chunk; i += 2) {
+        const bool both = i + 1 < rs.n_chunk;
+        const float* xs0 = rs.wait(i, fail, c.status);
+        const float* xs1 = both ? rs.wait(i + 1, fail, c.status) : xs0;
+        const int r0 = i * kStageRows + rgi;               // rows r0 and r0 + kStageRows
+        const bool on[2] = {r0 < rs.rows, r0 + kStageRows < rs.rows};
+        const float f[2] = {pu.j >= 0 && on[0] ? f_s[r0] : 0.f, pu.j >= 0 && on[1] ? f_s[r0 + kStageRows] : 0.f};
+        float a[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int g = 0; g < 4; ++g) a[u][g] = 0.f;
+        if (on[0]) {
+#pragma unroll 2
             for (int v = l8; v < nv; v += 8) {
-                float4 x = *reinterpret_cast<const float4*>(xs + rgi * s.dck + 4 * v);
+                float4 x[2], y = make_float4(0.f, 0.f, 0.f, 0.f);
+                x[0] = *reinterpret_cast<const float4*>(xs0 + rgi * s.dck + 4 * v);
+                x[1] = on[1] ? *reinterpret_cast<const float4*>(xs1 + rgi * s.dck + 4 * v) : y;
                 if (pu.j >= 0) {
-                    const float4 y = *reinterpret_cast<const float4*>(xc + 4 * v);
-                    x.x = fmaf(f, y.x, x.x); x.y = fmaf(f, y.y, x.y); x.z = fmaf(f, y.z, x.z); x.w = fmaf(f, y.w, x.w);
-                    *reinterpret_cast<float4*>(ckg + (size_t)m * s.dck + 4 * v) = x;
+                    y = *reinterpret_cast<const float4*>(xc + 4 * v);
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        x[u].x = fmaf(f[u], y.x, x[u].x); x[u].y = fmaf(f[u], y.y, x[u].y); x[u].z = fmaf(f[u], y.z, x[u].z); x[u].w = fmaf(f[u], y.w, x[u].w);
+                        if (on[u]) *reinterpret_cast<float4*>(ckg + (size_t)(m0 + r0 + u * kStageRows) * s.dck + 4 * v) = x[u];
+                    }
                 }
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
                     if (g < nh) {
-                        const float4 y = *reinterpret_cast<const float4*>(qc + g * s.dck + 4 * v);
-                        a[g] = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, a[g]))));
+                        const float4 z = *reinterpret_cast<const float4*>(qc + g * s.dck + 4 * v);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) a[u][g] = fmaf(x[u].x, z.x, fmaf(x[u].y, z.y, fmaf(x[u].z, z.z, fmaf(x[u].w, z.w, a[u][g]))));
                     }
                 }
             }
         }
 #pragma unroll
-        for (int g = 0; g < 4; ++g)
-            if (g < nh) {
+        for (int o = 1; o < 8; o <<= 1)
 #pragma unroll
-                for (int o = 1; o < 8; o <<= 1) a[g] += __shfl_xor_sync(0xffffffffu, a[g], o);
+            for (int g = 0; g < 4; ++g)
+                if (g < nh) {
+                    a[0][g] += __shfl_xor_sync(0xffffffffu, a[0][g], o);
+                    a[1][g] += __shfl_xor_sync(0xffffffffu, a[1][g], o);
+                }
+        if (l8 < CL) {                                     // lane x of a row writes to CTA x of the cluster
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int m = m0 + r0 + u * kStageRows;
+                const float w = m == 0 ? w_0 : m == 1 ? w_1 : w_gen;
+                if (on[u])
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) if (g < nh) st_peer(u_peer + 4u * (uint32_t)(g * s.M + m), w * a[u][g]);
             }
-        if (rgi < rows && l8 < CL) {                       // lane x of a row writes to CTA x of the cluster
-            const float w = m == 0 ? w_0 : m == 1 ? w_1 : w_gen;
-#pragma unroll
-            for (int g = 0; g < 4; ++g) if (g < nh) st_peer(u_peer + 4u * (uint32_t)(g * s.M + m), w * a[g]);
         }
-        rs.done(i, tid);
+        rs.done(i, 2, tid);
     }
     cluster_meet(CL);
     if (blockIdx.y == 0 && b == 0) {                       // the channels' factors, for the last kernel of the chain
@@ -1090,7 +1114,7 @@ __global__ void __launch_bounds__(kChanThreads) chan_out_kernel(Dims s, CacheDev
                 }
             }
         }
-        rs.done(i, tid);
+        if ((i & 1) || i + 1 == rs.n_chunk) rs.done(i & ~1, 2, tid);         // two stages at a time
     }
     if (rg < nrg) {
 #pragma unroll
