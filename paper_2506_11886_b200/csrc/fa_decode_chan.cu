@@ -211,7 +211,7 @@ __device__ __forceinline__ RowParts row_parts(const int32_t* state, const Dims& 
 // memory; then Z of nq channel pairs per CTA (a transform carries channels 2 q and 2 q + 1 of one head).  With k_new (a step, one
 // pass) also the push: C^K's rows are updated on their way, the leaving row's kept dims and the new token are written.
 template <int LS>
-__global__ void __launch_bounds__(kChanThreads) chan_in_kernel(Dims s, CacheDev c, ChanPlan mp, const bf16* __restrict__ q, const bf16* __restrict__ k_new,
+__global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, CacheDev c, ChanPlan mp, const bf16* __restrict__ q, const bf16* __restrict__ k_new,
                                                                const bf16* __restrict__ v_new, char* wsp) {
     constexpr int S = 1 << LS;
     extern __shared__ __align__(16) float smz[];
@@ -913,8 +913,9 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
 // Cluster per job, 256 threads: the parts' statistics and outputs merged, z of nq channel pairs per CTA, summed over the cluster
 // through distributed shared memory, a slice of the rows of C^V per CTA, its products summed likewise, the output rows.
 // After a step's push (step != 0) C^V's rows are updated on their way.
+// (128 registers at most: the plan counts on two CTAs to an SM, and the instances of 64 and 512 slots took 155, 9 to 11 % of a step)
 template <int LS>
-__global__ void __launch_bounds__(kChanThreads) chan_out_kernel(Dims s, CacheDev c, ChanPlan mp, bf16* __restrict__ out, char* wsp, int step) {
+__global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, CacheDev c, ChanPlan mp, bf16* __restrict__ out, char* wsp, int step) {
     constexpr int S = 1 << LS;
     extern __shared__ __align__(16) float smz[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
