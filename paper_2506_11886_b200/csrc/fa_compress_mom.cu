@@ -14,13 +14,16 @@
 //   2. moment_project_kernel: C += G Y on CTA pairs (tcgen05.mma.cta_group::2), G generated from exact integer phases
 //      and 32 Bessel factors per frequency; three products hi hi, lo hi, hi lo.
 // Both factors carry 2^-17, where the contraction over tokens rounds its basis to bf16 (2^-9).
+// Where the frequencies fill tiles of 256 the blocks are folded in pairs about the middle of the row, which halves the second contraction (see there).
 //
 // What bounds it: the first kernel HBM (per box of 64 tokens of one side 740 to 840 cycles against the 700 that 16 KB take at an SM's
 // share of the measured rate; its write of the moments is 10 % of the traffic at k / T = 1 / 64 and 20 % at 1 / 32), the
-// second the tensor cores (1200 cycles a block and pair against 1152 for its products) plus 8 K cycles of reductions per segment.
-// Direct contraction against this path: six layers of 32 K tokens, 1024 rows: 701 -> 374 us, with one projection for all 333; 128 K tokens, batch 4, 2048 rows:
-// 3207 -> 778 us; six ragged rows of 3 to 12 K tokens, 512 rows: 123 -> 85 us; 4 K tokens of 256 heads, 256 rows (T / k = 32, blocks of
-// 192 tokens): 231 -> 221 us.  Relative error of the coefficients 4e-6 against 2.4e-4.
+// second the tensor cores (1152 cycles of products a position and pair) plus 20 K cycles a segment, at the rate at which L2 adds vectors of
+// floats (four rows of 128 K tokens: 242 K cycles, 69 % of them on the tensor cores).
+// Direct contraction against this path: six layers of 32 K tokens, 1024 rows: 701 -> 374 us, with one projection for all 333, folded 292; 128 K
+// tokens, batch 4, 2048 rows: 3207 -> 777, folded 674 us; six ragged rows of 3 to 12 K tokens, 512 rows: 123 -> 85, folded 79 us; 4 K tokens of 256
+// heads, 256 rows (T / k = 32, blocks of 192 tokens, too few frequencies to fold): 231 -> 221 us.  The projection of the four rows of 128 K tokens alone:
+// 275 -> 162 us.  Relative error of the coefficients 4e-6 against 2.4e-4.
 #include <mutex>
 #include <type_traits>
 
@@ -47,6 +50,21 @@ __device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint3
     const __nv_bfloat162 l = __floats2bfloat162_rn(x - __uint_as_float(hi << 16), y - __uint_as_float(hi & 0xffff0000u));
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
+// two runs of 16 columns of tensor memory
+__device__ __forceinline__ void tmem_ld16_two(uint32_t a0, uint32_t a1, float (&x)[16], float (&y)[16]) {
+    uint32_t r[16], q[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]),
+          "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]),
+          "=r"(q[6]), "=r"(q[7]), "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15])
+        : "r"(a0), "r"(a1)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) { x[i] = __uint_as_float(r[i]); y[i] = __uint_as_float(q[i]); }
+}
 __device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
     uint16_t v;
     asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
@@ -55,19 +73,23 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
 
 // Blocks of a launch: batch rows b0 .. b0 + nb of the call; row b owns blocks first[b] .. first[b + 1] of the launch
 // (lens.n = 0: nblk each, and first is not used).  R tokens to a block.
+// Folded (the tiles of frequencies are whole, k a multiple of 256): a position of the launch is a PAIR of blocks of a row, p and n - 1 - p of
+// its n blocks (the middle one of an odd number by itself); nblk, first and total then count pairs.
 struct MomRows {
-    int R, nblk, b0, nb, total;
+    int R, nblk, b0, nb, total, n_blk;                     // (n_blk: blocks of a row, where all are alike)
     RowLens lens;
     uint32_t first[kMaxRagged + 1];
 };
+__host__ __device__ inline int blocks_of(int n_mid, int R) { return (n_mid + R - 1) / R; }
 
 // Item = (block, KV head[, side]): D = 128: one side's 128 dims, D = 64: K dims and V dims side by side.  A persistent CTA
 // takes items blockIdx.x, blockIdx.x + gridDim.x, ...: CTAs that run together read the same tokens' heads.
-template <int D, bool RAG>
+template <int D, bool RAG, bool FOLD>
 __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                                                                  Dims s, CacheDev c, int Lall, const __grid_constant__ MomRows rows, bf16* __restrict__ Y,
                                                                  int n_stages, int n_items, int wait_first) {
     constexpr int kSides = D == 128 ? 2 : 1;               // items per (block, head)
+    constexpr int kTypes = FOLD ? 2 : 1;                   // operands per position: real and imaginary rows want different sums of a pair
     // A: 64-dim rows of a token, MN-major; B: P, K-major; M = 128 dims, N = 64 (hi and lo rows of P)
     constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(2 * kMF >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     extern __shared__ unsigned char smem_unaligned[];
@@ -76,7 +98,7 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
     const int n_chunk = rows.R / kChunk;
     unsigned char* Hs = stage0 + (size_t)n_stages * kChunkBytes;
     unsigned char* y_s = Hs + (size_t)n_chunk * kHChunk;   // [128 columns][128 bytes] moments of an item on their way out
-    uint64_t* full = reinterpret_cast<uint64_t*>(y_s + 128 * 4 * kMF);
+    uint64_t* full = reinterpret_cast<uint64_t*>(y_s + kTypes * 128 * 4 * kMF);
     uint64_t* empty = full + n_stages;
     uint64_t* acc_full = empty + n_stages;
     uint64_t* acc_empty = acc_full + kAcc;
@@ -143,7 +165,7 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
 
     // A role's place in the CTA's items: the next item is gridDim.x further on, taken by additions with carries.
     const int n_mid_all = mid_of(s, Lall);
-    struct Walk { int i, side, h, gblk, b, blk, nblk, n_mid, n_ch; };
+    struct Walk { int i, side, h, gblk, b, blk, nblk, n_mid, n_blk; };
     const int d_side = kSides == 2 ? (int)gridDim.x & 1 : 0, d_t = kSides == 2 ? (int)gridDim.x >> 1 : (int)gridDim.x;
     const int d_blk = d_t / s.Hkv, d_h = d_t - d_blk * s.Hkv;
     auto settle = [&](Walk& w) {                           // block number -> batch row and block of the row
@@ -154,8 +176,12 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
             if (RAG) w.nblk = (int)(rows.first[w.b + 1] - rows.first[w.b]);
         }
         if (RAG) w.n_mid = mid_of(s, rows.lens.len[w.b]);
-        w.n_ch = min(n_chunk, (w.n_mid - w.blk * rows.R + kChunk - 1) / kChunk);
+        if (RAG && FOLD) w.n_blk = blocks_of(w.n_mid, rows.R);
     };
+    // the blocks of an item: one, or (folded) the pair p, n - 1 - p; a block's boxes
+    auto halves = [&](const Walk& w) { return FOLD && w.n_blk - 1 - w.blk != w.blk ? 2 : 1; };
+    auto block_of = [&](const Walk& w, int half) { return FOLD && half ? w.n_blk - 1 - w.blk : w.blk; };
+    auto boxes_of = [&](const Walk& w, int blk) { return min(n_chunk, (w.n_mid - blk * rows.R + kChunk - 1) / kChunk); };
     auto walk_begin = [&]() {
         Walk w;
         w.i = blockIdx.x;
@@ -167,7 +193,7 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
         w.b = RAG ? 0 : rows.b0;
         w.nblk = RAG ? (int)rows.first[1] : rows.nblk;
         w.n_mid = n_mid_all;
-        w.n_ch = 0;
+        w.n_blk = FOLD ? blocks_of(n_mid_all, rows.R) : 0;
         settle(w);
         return w;
     };
@@ -190,9 +216,11 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
             int st = 0, issued = 0;
             uint32_t par = 1;
             bool live = true;
-            for (Walk it = walk_begin(); live && it.i < n_items; walk_next(it)) {
-                int tok = s.l_init + it.blk * rows.R;
-                for (int q = 0; q < it.n_ch; ++q, tok += kChunk) {
+            for (Walk it = walk_begin(); live && it.i < n_items; walk_next(it))
+            for (int half = 0; live && half < halves(it); ++half) {
+                const int blk = block_of(it, half), n_ch = boxes_of(it, blk);
+                int tok = s.l_init + blk * rows.R;
+                for (int q = 0; q < n_ch; ++q, tok += kChunk) {
                     if (!mbar_wait(empty + st, par, fail, c.status)) { live = false; break; }
                     unsigned char* dst = stage0 + (size_t)st * kChunkBytes;
                     mbar_expect_tx(full + st, (uint32_t)kChunkBytes);
@@ -220,13 +248,15 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
             bool live = true;
             // descriptors with the addresses of stage 0 and box 0 of P (in units of 16 bytes; the sums stay below the field's end)
             const uint64_t xdesc0 = umma_desc(smem_u32(stage0), (kChunkBytes / 2) >> 4, 1024 >> 4), hdesc0 = umma_desc(smem_u32(Hs), 1, 1024 >> 4);
-            for (Walk it = walk_begin(); live && it.i < n_items; walk_next(it), ++a) {
+            for (Walk it = walk_begin(); live && it.i < n_items; walk_next(it))
+            for (int half = 0; live && half < halves(it); ++half, ++a) {
+                const int blk = block_of(it, half), n_ch = boxes_of(it, blk);
                 const int ab = a % kAcc;
-                if (a >= kAcc && !mbar_wait(acc_empty + ab, ((a / kAcc) - 1) & 1, fail, c.status)) break;
+                if (a >= kAcc && !mbar_wait(acc_empty + ab, ((a / kAcc) - 1) & 1, fail, c.status)) { live = false; break; }
                 const uint32_t acc = tmem_base + ab * (2 * kMF);
                 uint64_t hdesc = hdesc0;
-                int left = it.n_mid - it.blk * rows.R;
-                for (int q = 0; q < it.n_ch; ++q, left -= kChunk, hdesc += kHChunk >> 4) {
+                int left = it.n_mid - blk * rows.R;
+                for (int q = 0; q < n_ch; ++q, left -= kChunk, hdesc += kHChunk >> 4) {
                     if (!mbar_wait(full + st, par, fail, c.status)) { live = false; break; }
                     if (left < kChunk) {
                         if (!mbar_wait(masked + st, (mpar >> st) & 1u, fail, c.status)) { live = false; break; }
@@ -249,16 +279,11 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
         const int lg = warp & 3, e = lg * 32 + lane;       // tensor-memory lane: the dim, or (D = 64) K's dims then V's
         const int ncol = s.dck + s.dcv;
         int a = 0;
-        for (Walk it = walk_begin(); it.i < n_items; walk_next(it), ++a) {
-            const int ab = a % kAcc;
-            if (!mbar_wait(acc_full + ab, (a / kAcc) & 1, fail, c.status)) break;
+        for (Walk it = walk_begin(); it.i < n_items; walk_next(it)) {
+            const int n_half = halves(it);
+            // (after a time-out the walk goes on, on what is there: the four warps keep meeting)
+            for (int half = 0; half < n_half; ++half) mbar_wait(acc_full + (a + half) % kAcc, ((a + half) / kAcc) & 1, fail, c.status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float y[kMF], y2[kMF];
-            tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(ab * 2 * kMF), y);
-            tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(ab * 2 * kMF + kMF), y2);
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty + ab);
             const int side = kSides == 2 ? it.side : e >> 6, dim = kSides == 2 ? e : e & 63;
             const int pos = inv_s[(it.h * 2 + side) * D + dim];
             // The columns of the item are one contiguous run of rows of Y: they are put together in shared memory and leave with one
@@ -266,27 +291,63 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
             // permuted as the 128-byte swizzle of the products' operand wants them, so the second kernel copies rows as they are.
             if (warp == 2 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the copy before has read the buffer
             asm volatile("bar.sync 2, %0;" ::"n"(32 * kEpiWarps) : "memory");
-            if (pos != 255) {
-                const int col = (kSides == 1 && side ? s.dck : 0) + pos;
-                unsigned char* dst = y_s + col * (4 * kMF);
+            const uint32_t t0 = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)((a % kAcc) * 2 * kMF), t1 = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(((a + 1) % kAcc) * 2 * kMF);
+            const int col = (kSides == 1 && side ? s.dck : 0) + pos;
+            // 16 moments at a time (all 32 of two blocks do not fit the registers)
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    uint32_t hi[4], lo[4];
+            for (int r0 = 0; r0 < kMF; r0 += 16) {
+                auto put = [&](unsigned char* dst, const float (&v)[16]) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) split_bf16(y[8 * r + 2 * u] + y2[8 * r + 2 * u], y[8 * r + 2 * u + 1] + y2[8 * r + 2 * u + 1], hi[u], lo[u]);
-                    *reinterpret_cast<uint4*>(dst + ((r ^ (col & 7)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                    *reinterpret_cast<uint4*>(dst + (((4 + r) ^ (col & 7)) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                    for (int r = 0; r < 2; ++r) {
+                        uint32_t hi[4], lo[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) split_bf16(v[8 * r + 2 * u], v[8 * r + 2 * u + 1], hi[u], lo[u]);
+                        const int piece = r0 / 8 + r;
+                        *reinterpret_cast<uint4*>(dst + ((piece ^ (col & 7)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                        *reinterpret_cast<uint4*>(dst + (((4 + piece) ^ (col & 7)) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                    }
+                };
+                float y[16], t[16];                        // of the one block, or of block p
+                tmem_ld16_two(t0 + r0, t0 + kMF + r0, y, t);
+#pragma unroll
+                for (int r = 0; r < 16; ++r) y[r] += t[r];
+                if (FOLD) {
+                    float z[16];                           // of block n - 1 - p
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) z[r] = 0.f;
+                    if (n_half == 2) {
+                        tmem_ld16_two(t1 + r0, t1 + kMF + r0, z, t);
+#pragma unroll
+                        for (int r = 0; r < 16; ++r) z[r] += t[r];
+                    }
+                    // even orders: sum and difference, odd ones: difference and sum (the middle block by itself: itself and nothing)
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) {
+                        const float sum = z[r] + y[r], dif = n_half == 2 ? z[r] - y[r] : 0.f;
+                        y[r] = (r & 1) ? dif : sum;
+                        z[r] = (r & 1) ? sum : dif;
+                    }
+                    if (pos != 255) put(y_s + (128 + col) * (4 * kMF), z);
                 }
+                if (pos != 255) put(y_s + col * (4 * kMF), y);
             }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                for (int half = 0; half < n_half; ++half) mbar_arrive(acc_empty + (a + half) % kAcc);
+            a += n_half;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("bar.sync 2, %0;" ::"n"(32 * kEpiWarps) : "memory");
             if (warp == 2 && lane == 0) {
                 const int c0 = kSides == 2 && it.side ? s.dck : 0, nc = kSides == 1 ? ncol : it.side ? s.dcv : s.dck;
-                char* dst = reinterpret_cast<char*>(Y) + (((size_t)it.gblk * s.Hkv + it.h) * ncol + c0) * (size_t)(4 * kMF);
-                if (nc > 0)
-                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(dst)), "r"(smem_u32(y_s)),
-                                 "r"(nc * (4 * kMF))
-                                 : "memory");
+#pragma unroll
+                for (int ty = 0; ty < kTypes; ++ty) {
+                    char* dst = reinterpret_cast<char*>(Y) + ((((size_t)it.gblk * kTypes + ty) * s.Hkv + it.h) * ncol + c0) * (size_t)(4 * kMF);
+                    if (nc > 0)
+                        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(dst)),
+                                     "r"(smem_u32(y_s + ty * 128 * 4 * kMF)), "r"(nc * (4 * kMF))
+                                     : "memory");
+                }
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
         }
@@ -331,8 +392,10 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
                 const uint32_t col = (uint32_t)(16 * (v ? p - nk8 : p));
                 const int mask = v ? vmask : 0;
                 char* dst0 = reinterpret_cast<char*>(v ? c.v_mid : c.k_mid) + bh * (size_t)rowb;
-                int j0 = it.blk * rows.R + 8 * w + sub, left = it.n_mid - it.blk * rows.R;
-                for (int q = 0; q < it.n_ch; ++q, j0 += kChunk, left -= kChunk) {
+                for (int half = 0; live && half < halves(it); ++half) {
+                const int blk = block_of(it, half), n_ch = boxes_of(it, blk);
+                int j0 = blk * rows.R + 8 * w + sub, left = it.n_mid - blk * rows.R;
+                for (int q = 0; q < n_ch; ++q, j0 += kChunk, left -= kChunk) {
                     if (!mbar_wait(full + st, par, fail, c.status)) { live = false; break; }
                     const uint32_t box = smem_u32(stage0) + (uint32_t)(st * kChunkBytes + w * 1024), src = box + (uint32_t)(sub * 128);
                     uint4 val[NI];
@@ -372,6 +435,7 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
                         }
                     }
                 }
+                }
             };
             using std::integral_constant;
             if (np <= 4) gather(integral_constant<int, 2>{});
@@ -392,7 +456,7 @@ constexpr int kBMp = 128;             // coefficient rows per CTA (256 per pair)
 constexpr int kGenWarpsP = 8;
 constexpr int kThreadsP = 64 + 32 * kGenWarpsP;
 constexpr int kABytesP = kBMp * 128;  // rows of 32 hi and 32 lo values
-constexpr int kStagesP = 4;
+constexpr int kStagesP = 4;             // stages at most
 
 // Positions: the blocks of all (batch row, head group) units of the launch, laid end to end; a team of M / 256 pairs takes
 // positions start[t] .. start[t + 1] (cut on the host so that every team has the same cost, as in fa_compress_tc2.cu).
@@ -407,19 +471,23 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                  : "memory");
 }
 
-// HP heads share a pair and its basis tiles.  npad: accumulator columns per head (the compressed dims of both sides, up to a
-// multiple of 32); each CTA of a pair brings half of them.
-template <int HP, bool RAG>
+// npad: accumulator columns of a product (the compressed dims of both sides, up to a multiple of 32); each CTA of a CTA pair brings half of
+// them.  A stage feeds two products:
+//   as they are: one tile of 128 frequencies (rows Re and Im interleaved) against HP heads;
+//   folded: with t_b = m + d_b about the middle m of the row, blocks at +d and -d enter as e^{i theta n d} Y+ + e^{-i theta n d} Y- =
+//     cos E + i sin O with E, O = Y+ +- Y-.  By the parity of i^r, the real part of e^{-i theta n m} C_n takes E of even r and O of odd r only, the
+//     imaginary part the others: two tiles (256 frequencies, Re; the same, Im) against one head's two operands, each 32 long for TWO
+//     blocks.  Half the products of the plain form; the epilogue turns (Re, Im) by e^{i theta n m} in registers.
+template <int HP, bool RAG, bool FOLD>
 __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16* __restrict__ Y, Dims s, const __grid_constant__ MomLayers layers,
-                                                                      const __grid_constant__ MomRows rows, const __grid_constant__ MomCuts cuts, int npad) {
-    constexpr int kBHalf1 = 128 * 128;                     // room for this CTA's columns of one head: at most 128 rows of 128 bytes
-    constexpr int kStage = kABytesP + HP * kBHalf1;
-    const int nh = npad >> 1;
+                                                                      const __grid_constant__ MomRows rows, const __grid_constant__ MomCuts cuts, int npad, int n_stages) {
+    constexpr int kTiles = FOLD ? 2 : 1, kOps = FOLD ? 2 : HP;     // A tiles and B operands of a stage
+    const int nh = npad >> 1, b_op = nh * 128, n_stage = kTiles * kABytesP + kOps * b_op;     // rows of 128 bytes
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(npad >> 3) << 17) | ((uint32_t)((2 * kBMp) >> 4) << 24);
     extern __shared__ unsigned char smem_unaligned[];
     unsigned char* smem = smem_unaligned + ((1024u - (smem_u32(smem_unaligned) & 1023u)) & 1023u);
     unsigned char* stage0 = smem;
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStagesP * kStage);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + n_stages * n_stage);
     uint64_t* peer = full + kStagesP;                      // even CTA: the odd CTA's stage is complete
     uint64_t* empty = peer + kStagesP;
     uint64_t* acc_ready = empty + kStagesP;
@@ -429,13 +497,13 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank();
-    const int n_pairs = s.M / (2 * kBMp);
+    const int n_pairs = s.M / (kTiles * 2 * kBMp);
     const int cluster = (int)blockIdx.x >> 1, team = cluster / n_pairs, pair = cluster - team * n_pairs;
     const int mt = 2 * pair + (int)rank;
     const int n_hg = s.Hkv / HP, ncol = s.dck + s.dcv;
     const uint32_t pos_begin = cuts.start[team], pos_end = cuts.start[team + 1];
     int32_t* status = layers.status[0];
-    struct Seg { int b, h0, kb0, kb1; uint32_t g0; };      // batch row, heads, blocks, first block of the row in the launch
+    struct Seg { int b, h0, kb0, kb1, n_blk; uint32_t g0; };      // batch row, heads, positions, blocks of the row, first position of the row in the launch
     auto seg_at = [&](uint32_t pos) {
         int b, nblk = rows.nblk;
         uint32_t g0, off;
@@ -452,11 +520,12 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
             b += rows.b0;
         }
         const int hg = (int)(off / (uint32_t)nblk), kb0 = (int)off - hg * nblk;
-        return Seg{b, hg * HP, kb0, (int)min((uint32_t)nblk, (uint32_t)kb0 + (pos_end - pos)), g0};
+        const int n_blk = !FOLD ? 0 : RAG ? blocks_of(mid_of(s, rows.lens.len[b]), rows.R) : rows.n_blk;
+        return Seg{b, hg * HP, kb0, (int)min((uint32_t)nblk, (uint32_t)kb0 + (pos_end - pos)), n_blk, g0};
     };
 
     if (tid == 0) {
-        for (int i = 0; i < kStagesP; ++i) {
+        for (int i = 0; i < n_stages; ++i) {
             mbar_init(full + i, kGenWarpsP + 1);
             mbar_init(peer + i, 1);
             mbar_init(empty + i, 1);
@@ -467,7 +536,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(HP * 256) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kOps * 256) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -483,7 +552,8 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                 asm volatile("griddepcontrol.wait;" ::: "memory");       // the moments
                 // (only now: a kernel that this lets start may count the kernel before this one as finished)
                 asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-                int it = 0, seg = 0;
+                int it = 0, seg = 0, st = 0;
+                uint32_t par = 1;
                 bool live = true;
                 // (the rows past the last column are whatever the stage held: their accumulator columns are not read)
                 const uint32_t bytes = (uint32_t)min(nh, max(0, ncol - (int)rank * nh)) * (4 * kMF);
@@ -491,73 +561,76 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                     const Seg g = seg_at(pos);
                     if (seg > 0 && !mbar_wait(epi_done, (seg - 1) & 1, fail, status)) { live = false; break; }
                     for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
-                        const int st = it % kStagesP;
-                        if (it >= kStagesP && !mbar_wait(empty + st, ((it / kStagesP) - 1) & 1, fail, status)) { live = false; break; }
-                        unsigned char* bdst = stage0 + (size_t)st * kStage + kABytesP;
-                        mbar_expect_tx(full + st, HP * bytes);
+                        if (!mbar_wait(empty + st, par, fail, status)) { live = false; break; }
+                        unsigned char* bdst = stage0 + (size_t)st * n_stage + kTiles * kABytesP;
+                        mbar_expect_tx(full + st, kOps * bytes);
                         const char* src = reinterpret_cast<const char*>(Y) +
-                                          ((((size_t)g.g0 + kb) * s.Hkv + g.h0) * ncol + (size_t)rank * nh) * (size_t)(4 * kMF);
+                                          ((((size_t)g.g0 + kb) * kTiles * s.Hkv + g.h0) * ncol + (size_t)rank * nh) * (size_t)(4 * kMF);
                         if (bytes) {
 #pragma unroll
-                            for (int hh = 0; hh < HP; ++hh) bulk_load(bdst + hh * kBHalf1, src + (size_t)hh * ncol * (4 * kMF), bytes, full + st);
+                            for (int o = 0; o < kOps; ++o) bulk_load(bdst + o * b_op, src + (size_t)o * (FOLD ? s.Hkv : 1) * ncol * (4 * kMF), bytes, full + st);
                         }
+                        if (++st == n_stages) { st = 0; par ^= 1; }
                     }
                     pos += (uint32_t)(g.kb1 - g.kb0);
                 }
                 if (!live)                                 // a wait ran out: this CTA's boxes under way land, or the bound is reached, before it ends
-                    for (int q = it - kStagesP < 0 ? 0 : it - kStagesP; q < it; ++q)
-                        for (uint32_t n = 0; n < (1u << 16) && !mbar_try_wait(full + q % kStagesP, (uint32_t)(q / kStagesP) & 1u); ++n) { }
+                    for (int q = it - n_stages < 0 ? 0 : it - n_stages; q < it; ++q)
+                        for (uint32_t n = 0; n < (1u << 16) && !mbar_try_wait(full + q % n_stages, (uint32_t)(q / n_stages) & 1u); ++n) { }
             }
         } else if (warp == 1) {
             // ---------------- MMA issuer: the even CTA, for the pair ----------------
             if (lane == 0 && rank == 0) {
-                int it = 0;
+                int st = 0;
+                uint32_t par = 0;
                 bool live = true;
                 for (uint32_t pos = pos_begin; live && pos < pos_end;) {
                     const Seg g = seg_at(pos);
-                    for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
-                        const int st = it % kStagesP;
-                        const uint32_t par = (it / kStagesP) & 1;
+                    for (int kb = g.kb0; kb < g.kb1; ++kb) {
                         if (!mbar_wait(full + st, par, fail, status) || !mbar_wait(peer + st, par, fail, status)) { live = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t a_addr = smem_u32(stage0 + (size_t)st * kStage), b_addr = a_addr + kABytesP;
+                        const uint32_t a_addr = smem_u32(stage0 + (size_t)st * n_stage), b_addr = a_addr + kTiles * kABytesP;
                         // rows of 128 bytes, 32 hi and 32 lo values: hi hi, lo hi, hi lo, sixteen values at a time
 #pragma unroll
                         for (int pr = 0; pr < 3; ++pr)
 #pragma unroll
                             for (int ks = 0; ks < 2; ++ks) {
-                                const uint64_t adesc = umma_desc(a_addr + (pr == 1 ? 64 : 0) + ks * 32, 1, 1024 >> 4);
 #pragma unroll
-                                for (int hh = 0; hh < HP; ++hh)
-                                    umma_bf16_pair(tmem_base + hh * 256, adesc, umma_desc(b_addr + hh * kBHalf1 + (pr == 2 ? 64 : 0) + ks * 32, 1, 1024 >> 4),
-                                                   idesc, (kb > g.kb0 || pr > 0 || ks > 0) ? 1u : 0u);
+                                for (int o = 0; o < kOps; ++o)
+                                    umma_bf16_pair(tmem_base + o * 256, umma_desc(a_addr + (FOLD ? o * kABytesP : 0) + (pr == 1 ? 64 : 0) + ks * 32, 1, 1024 >> 4),
+                                                   umma_desc(b_addr + o * b_op + (pr == 2 ? 64 : 0) + ks * 32, 1, 1024 >> 4), idesc,
+                                                   (kb > g.kb0 || pr > 0 || ks > 0) ? 1u : 0u);
                             }
                         umma_commit_pair(empty + st);
+                        if (++st == n_stages) { st = 0; par ^= 1; }
                     }
                     if (live) umma_commit_pair(acc_ready);
                     pos += (uint32_t)(g.kb1 - g.kb0);
                 }
             } else if (lane == 0) {
                 const int n_it = (int)(pos_end - pos_begin);
+                int st = 0;
+                uint32_t par = 0;
                 for (int it = 0; it < n_it; ++it) {
-                    const int st = it % kStagesP;
-                    const uint32_t par = (it / kStagesP) & 1;
                     if (!mbar_wait(full + st, par, fail, status)) break;
                     mbar_arrive_cluster(peer + st, 0);
+                    if (++st == n_stages) { st = 0; par ^= 1; }
                 }
             }
         } else {
-            // ---------------- generators: rows 2 n (Re) and 2 n + 1 (Im) of e^{i theta n center} (2 r + 1) i^r j_r(phi_n) ----------------
+            // ---------------- generators: rows Re and Im of e^{i theta n t_b} (2 r + 1) i^r j_r(phi_n), t_b the block's middle or (folded)
+            // its distance from the row's middle; Re and Im rows of a frequency follow one another, or lie in tiles of their own ----------------
+            constexpr int LT = FOLD ? 1 : 2, NR = kMF >> LT;       // 2^LT threads to a frequency, NR moments each
             const int t = tid - 64;
-            const int fi = t >> 2, tq = t & 3;             // frequency of the tile, quarter of the 32 moments
-            const unsigned n = (unsigned)(mt * (kBMp / 2) + fi);
-            float gb[8];                                   // (2 r + 1) j_r(phi_n) for r = 8 tq .. 8 tq + 7
+            const int fi = t >> LT, tq = t & ((1 << LT) - 1);      // frequency of the tile, this thread's share of the moments
+            const unsigned n = (unsigned)(mt * (FOLD ? kBMp : kBMp / 2) + fi);
+            float gb[NR];                                  // (2 r + 1) j_r(phi_n) for r = NR tq .. NR tq + NR - 1
             {
                 // j_r by the recurrence downward from r = 10 + 2.4 phi (55 at most: far enough past phi that what is left out is
                 // below 1e-9, near enough that the values stay in range), scaled by the closed form of j_0 or j_1, whichever is larger
-                float keep[8], sn, cs, jn = 0.f, jc = 0.f, j0 = 1.f, j1 = 0.f;
+                float keep[NR], sn, cs, jn = 0.f, jc = 0.f, j0 = 1.f, j1 = 0.f;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) keep[i] = 0.f;
+                for (int i = 0; i < NR; ++i) keep[i] = 0.f;
                 const double invd = n ? (double)s.T / (3.14159265358979324 * (double)(n * (unsigned)rows.R)) : 0.0;      // 1 / phi: fp32's rounding of it adds up
                 const float x = (float)(n * (unsigned)rows.R) / (float)s.T, inv = (float)invd;
                 const int top = min(55, 10 + (int)(7.54f * x));
@@ -567,7 +640,9 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                     for (int i = 7; i >= 0; --i) {         // jc = j_r, jn = j_{r + 1}
                         const int r = r8 + i;
                         if (r == top) jc = 1e-20f;
-                        if (r8 == 8 * tq) keep[i] = (float)(2 * r + 1) * jc;
+#pragma unroll
+                        for (int u = 0; u < NR; u += 8)
+                            if (r8 == NR * tq + u) keep[u + i] = (float)(2 * r + 1) * jc;
                         if (i == 1) j1 = jc;
                         if (i == 0) j0 = jc;
                         const float jp = fmaf((float)((double)(2 * r + 1) * invd), jc, -jn);
@@ -578,40 +653,45 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                 sincospif(x, &sn, &cs);
                 const float t0 = sn * inv, t1 = (t0 - cs) * inv, sc = fabsf(t0) > fabsf(t1) ? t0 / j0 : t1 / j1;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) gb[i] = n ? keep[i] * sc : (i == 0 && tq == 0 ? 1.f : 0.f);
+                for (int i = 0; i < NR; ++i) gb[i] = n ? keep[i] * sc : (i == 0 && tq == 0 ? 1.f : 0.f);
             }
-            const int r0 = 2 * fi, r1 = 2 * fi + 1;
-            const uint32_t off0 = (uint32_t)((r0 >> 3) * 1024 + (r0 & 7) * 128), off1 = (uint32_t)((r1 >> 3) * 1024 + (r1 & 7) * 128);
+            const int r0 = FOLD ? fi : 2 * fi, r1 = FOLD ? fi : 2 * fi + 1;
+            const uint32_t off0 = (uint32_t)((r0 >> 3) * 1024 + (r0 & 7) * 128), off1 = (uint32_t)((r1 >> 3) * 1024 + (r1 & 7) * 128) + (FOLD ? kABytesP : 0);
             const unsigned T2 = 2u * (unsigned)s.T;
             const float inv_T = 1.0f / (float)s.T;
-            int it = 0, seg = 0;
+            int seg = 0, st = 0;
+            uint32_t par = 1;
             bool live = true;
             for (uint32_t pos = pos_begin; live && pos < pos_end; ++seg) {
                 const Seg g = seg_at(pos);
-                for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
-                    const int st = it % kStagesP;
-                    // phase of the block's middle: pi n (2 kb R + R - 1) / T, exact in integers
-                    const unsigned ph = (n * (unsigned)(2 * kb * rows.R + rows.R - 1)) % T2;
+                for (int kb = g.kb0; kb < g.kb1; ++kb) {
+                    // phase of the block's middle: pi n (2 kb R + R - 1) / T, or of its distance: pi n (n_blk - 1 - 2 kb) R / T; exact in integers
+                    const unsigned ph = (n * (unsigned)(FOLD ? (g.n_blk - 1 - 2 * kb) * rows.R : 2 * kb * rows.R + rows.R - 1)) % T2;
                     const float f = (float)ph * inv_T;     // in half turns, [0, 2)
                     const float an = 3.14159265358979f * (f - (f >= 1.0f ? 2.0f : 0.0f));
                     const float C = __cosf(an), S = __sinf(an);
-                    if (it >= kStagesP && !mbar_wait(empty + st, ((it / kStagesP) - 1) & 1, fail, status)) { live = false; break; }
-                    unsigned char* a_dst = stage0 + (size_t)st * kStage;
-                    uint32_t h0[4], l0[4], h1[4], l1[4];
+                    if (!mbar_wait(empty + st, par, fail, status)) { live = false; break; }
+                    unsigned char* a_dst = stage0 + (size_t)st * n_stage;
 #pragma unroll
-                    for (int i2 = 0; i2 < 4; ++i2) {       // moments 2 i2 (i^r = +-1), 2 i2 + 1 (i^r = +-i)
-                        const float sg = (i2 & 1) ? -1.f : 1.f;
-                        const float ga = sg * gb[2 * i2], go = sg * gb[2 * i2 + 1];
-                        split_bf16(ga * C, -go * S, h0[i2], l0[i2]);
-                        split_bf16(ga * S, go * C, h1[i2], l1[i2]);
+                    for (int u = 0; u < NR / 8; ++u) {
+                        const int cq = tq * (NR / 8) + u;  // 16-byte piece of a row: eight moments
+                        uint32_t h0[4], l0[4], h1[4], l1[4];
+#pragma unroll
+                        for (int i2 = 0; i2 < 4; ++i2) {   // moments 2 i2 (i^r = +-1), 2 i2 + 1 (i^r = +-i)
+                            const float sg = (i2 & 1) ? -1.f : 1.f;
+                            const float ga = sg * gb[8 * u + 2 * i2], go = sg * gb[8 * u + 2 * i2 + 1];
+                            split_bf16(ga * C, -go * S, h0[i2], l0[i2]);
+                            split_bf16(ga * S, go * C, h1[i2], l1[i2]);
+                        }
+                        *reinterpret_cast<uint4*>(a_dst + off0 + ((cq ^ (r0 & 7)) << 4)) = make_uint4(h0[0], h0[1], h0[2], h0[3]);
+                        *reinterpret_cast<uint4*>(a_dst + off0 + (((4 + cq) ^ (r0 & 7)) << 4)) = make_uint4(l0[0], l0[1], l0[2], l0[3]);
+                        *reinterpret_cast<uint4*>(a_dst + off1 + ((cq ^ (r1 & 7)) << 4)) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
+                        *reinterpret_cast<uint4*>(a_dst + off1 + (((4 + cq) ^ (r1 & 7)) << 4)) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
                     }
-                    *reinterpret_cast<uint4*>(a_dst + off0 + ((tq ^ (r0 & 7)) << 4)) = make_uint4(h0[0], h0[1], h0[2], h0[3]);
-                    *reinterpret_cast<uint4*>(a_dst + off0 + (((4 + tq) ^ (r0 & 7)) << 4)) = make_uint4(l0[0], l0[1], l0[2], l0[3]);
-                    *reinterpret_cast<uint4*>(a_dst + off1 + ((tq ^ (r1 & 7)) << 4)) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
-                    *reinterpret_cast<uint4*>(a_dst + off1 + (((4 + tq) ^ (r1 & 7)) << 4)) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive(full + st);
+                    if (++st == n_stages) { st = 0; par ^= 1; }
                 }
                 if (!live) break;
                 // ---------------- epilogue of the segment: accumulators are added to the coefficient rows ----------------
@@ -621,16 +701,30 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                 if (!ok) break;
                 {
                     const int lane_grp = warp & 3, part = (warp - 2) >> 2;
-                    const int m_base = mt * kBMp + lane_grp * 32;
-                    // 32 rows x 32 columns at a time through the idle ring: then eight lanes hold a row's 128 bytes
-                    float* tile = reinterpret_cast<float*>(stage0) + (warp - 2) * (32 * 36);
+                    // 32 accumulator rows x 32 columns at a time (folded: of both products) through the idle ring: then eight lanes hold a row's 128 bytes
+                    float* tile = reinterpret_cast<float*>(stage0) + (warp - 2) * (kTiles * 32 * 36);
                     const int npc = (ncol + 31) >> 5;      // pieces of 32 columns per head
                     const int layer = RAG ? 0 : g.b / s.B;
+                    const int row0 = FOLD ? 2 * (mt * kBMp + lane_grp * 32) : mt * kBMp + lane_grp * 32;
+                    float cm = 1.f, sm = 0.f;              // e^{i theta n m}, m the row's middle
+                    if (FOLD) sincospif((float)(((unsigned)(mt * kBMp + lane_grp * 32 + lane) * (unsigned)(g.n_blk * rows.R - 1)) % T2) * inv_T, &sm, &cm);
 #pragma unroll 1
                     for (int pc = part; pc < HP * npc; pc += 2) {
                         const int hh = pc / npc, c0 = (pc - hh * npc) * 32;
                         float v[32];
                         tmem_ld32(tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(hh * 256 + c0), v);
+                        if (FOLD) {
+                            float w[32];
+                            tmem_ld32(tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(256 + c0), w);
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) {
+                                const float re = cm * v[i] - sm * w[i];
+                                w[i] = sm * v[i] + cm * w[i];
+                                v[i] = re;
+                            }
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + (32 + lane) * 36 + 4 * i) = make_float4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                        }
 #pragma unroll
                         for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + lane * 36 + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
                         __syncwarp();
@@ -638,11 +732,13 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                         if (col < ncol) {
                             const bool is_k = col < s.dck;
                             const int nc = is_k ? s.dck : s.dcv;
-                            float* dst = coef_rows(is_k ? layers.k[layer] : layers.v[layer], s, g.b - layer * s.B, g.h0 + hh, nc) + (size_t)(m_base + rr0) * nc + (is_k ? col : col - s.dck);
+                            float* dst = coef_rows(is_k ? layers.k[layer] : layers.v[layer], s, g.b - layer * s.B, g.h0 + hh, nc) + (size_t)row0 * nc + (is_k ? col : col - s.dck);
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float4 x = *reinterpret_cast<const float4*>(tile + (rr0 + 4 * i) * 36 + 4 * q);
-                                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + (size_t)(4 * i) * nc), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w)
+                            for (int i = 0; i < 8 * kTiles; ++i) {
+                                // row of the coefficients: the tile's, or (folded) Re in rows 0 - 31 and Im in 32 - 63 of the tile, taken in turn
+                                const int m = rr0 + 4 * i, src = FOLD ? (m >> 1) + 32 * (m & 1) : m;
+                                const float4 x = *reinterpret_cast<const float4*>(tile + src * 36 + 4 * q);
+                                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + (size_t)m * nc), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w)
                                              : "memory");
                             }
                         }
@@ -667,7 +763,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
         for (int l = 1; l < layers.n; ++l) layers.status[l][0] = status[0];
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(HP * 256) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kOps * 256) : "memory");
     }
 }
 
@@ -690,8 +786,11 @@ int block_tokens(const Dims& s) {
     return (int)(r > kMaxBlockTokens ? kMaxBlockTokens : r);
 }
 
+// Whether the blocks are taken in pairs about the middle of a row: the projection then takes 256 frequencies at a time.
+bool folds(const Dims& s) { return s.k % 256 == 0; }
+
 size_t mom_smem_fixed(const Dims& s) {      // everything but the stages, the slack of the alignment among it
-    return (size_t)block_tokens(s) / kChunk * kHChunk + 128 * 4 * kMF + 8 * (3 * 16 + 2 * kAcc) + 16 + (size_t)s.Hkv * (2 * s.d + s.nfk + s.nfv) + 64 + 1024;
+    return (size_t)block_tokens(s) / kChunk * kHChunk + (folds(s) ? 2 : 1) * 128 * 4 * kMF + 8 * (3 * 16 + 2 * kAcc) + 16 + (size_t)s.Hkv * (2 * s.d + s.nfk + s.nfv) + 64 + 1024;
 }
 int mom_stages(const Dims& s) {
     const long long left = 227 * 1024 - (long long)mom_smem_fixed(s);
@@ -699,12 +798,12 @@ int mom_stages(const Dims& s) {
     return n > 16 ? 16 : n;
 }
 
-template <int D, bool RAG>
+template <int D, bool RAG, bool FOLD>
 cudaError_t launch_moments(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, const MomRows& rows, void* Y,
                            bool wait_first, cudaStream_t stream) {
     const int n_stages = mom_stages(s);
     const size_t smem = mom_smem_fixed(s) + (size_t)n_stages * kChunkBytes;
-    cudaError_t err = ensure_dynamic_smem(moments_kernel<D, RAG>, smem);
+    cudaError_t err = ensure_dynamic_smem(moments_kernel<D, RAG, FOLD>, smem);
     if (err != cudaSuccess) return err;
     const long long items = (long long)rows.total * s.Hkv * (D == 128 ? 2 : 1);
     if (items <= 0 || items >= (1ll << 31)) return cudaErrorInvalidValue;
@@ -718,16 +817,18 @@ cudaError_t launch_moments(const CUtensorMap& tmK, const CUtensorMap& tmV, const
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, moments_kernel<D, RAG>, tmK, tmV, s, c, L, rows, static_cast<bf16*>(Y), n_stages, (int)items, wait_first ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, moments_kernel<D, RAG, FOLD>, tmK, tmV, s, c, L, rows, static_cast<bf16*>(Y), n_stages, (int)items, wait_first ? 1 : 0);
 }
 
-template <int HP, bool RAG>
+template <int HP, bool RAG, bool FOLD>
 cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int n_layers, const MomRows& rows, cudaStream_t stream) {
     MomLayers layers = {};
     layers.n = n_layers;
     for (int i = 0; i < n_layers; ++i) { layers.k[i] = c[i].coef_k; layers.v[i] = c[i].coef_v; layers.status[i] = c[i].status; }
-    const size_t smem = (size_t)kStagesP * (kABytesP + HP * 128 * 128) + 8 * (3 * kStagesP + 2) + 16 + 1024;
-    cudaError_t err = ensure_dynamic_smem(moment_project_kernel<HP, RAG>, smem);
+    const size_t stage = FOLD ? 2 * kABytesP + (size_t)npad_of(s) * 128 : kABytesP + (size_t)HP * (npad_of(s) / 2) * 128, fixed = 8 * (3 * kStagesP + 2) + 16 + 1024;
+    const int fit = (int)((227 * 1024 - fixed) / stage), n_stages = fit < kStagesP ? fit : kStagesP;
+    const size_t smem = n_stages * stage + fixed;
+    cudaError_t err = ensure_dynamic_smem(moment_project_kernel<HP, RAG, FOLD>, smem);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kThreadsP);
@@ -742,7 +843,7 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const int n_pairs = s.M / (2 * kBMp), n_hg = s.Hkv / HP;
+    const int n_pairs = s.M / ((FOLD ? 4 : 2) * kBMp), n_hg = s.Hkv / HP;
     const long long total = (long long)rows.total * n_hg;
     if (total <= 0 || total >= (1ll << 31)) return cudaErrorInvalidValue;
     int n_teams;
@@ -757,7 +858,7 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
             cfg.gridDim = dim3(2 * sm_count());
             cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, moment_project_kernel<HP, RAG>, &cfg) != cudaSuccess || n < 1) {
+            if (cudaOccupancyMaxActiveClusters(&n, moment_project_kernel<HP, RAG, FOLD>, &cfg) != cudaSuccess || n < 1) {
                 cudaGetLastError();
                 n = sm_count() / 2 - 2;
             }
@@ -810,7 +911,7 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     while (!walk(lo, cuts.start)) ++lo;
     cuts.start[n_teams] = (uint32_t)total;
     cfg.gridDim = dim3(2 * n_teams * n_pairs);
-    return cudaLaunchKernelEx(&cfg, moment_project_kernel<HP, RAG>, static_cast<const bf16*>(Y), s, layers, rows, cuts, npad_of(s));
+    return cudaLaunchKernelEx(&cfg, moment_project_kernel<HP, RAG, FOLD>, static_cast<const bf16*>(Y), s, layers, rows, cuts, npad_of(s), n_stages);
 }
 
 }  // namespace
@@ -829,25 +930,29 @@ bool compress_mom_supported(const Dims& s) {
 // Bytes of moments that a batch row of n_mid middle tokens needs (of a layout that is supported).
 size_t compress_mom_row_bytes(const Dims& s, int n_mid) {
     const int R = block_tokens(s);
-    return (size_t)((n_mid + R - 1) / R) * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
+    const int n = blocks_of(n_mid, R);
+    return (size_t)(folds(s) ? (n + 1) / 2 * 2 : n) * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
 }
 
 static cudaError_t launch_rows(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
                                int64_t sh, int L, MomRows rows, char* Y, bool wait_first, cudaStream_t stream) {
-    const bool rag = rows.lens.n != 0;
+    const bool rag = rows.lens.n != 0, fold = folds(s);
     cudaError_t err;
     for (int i = 0; i < n_layers; ++i) {
         CUtensorMap tmK, tmV;
         if (!prefill_map(&tmK, K[i], s, sb, st, sh, L) || !prefill_map(&tmV, V[i], s, sb, st, sh, L)) return cudaErrorInvalidValue;
-        char* y = Y + (size_t)i * rows.total * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
-        if (s.d == 128) err = rag ? launch_moments<128, true>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream) : launch_moments<128, false>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream);
-        else err = rag ? launch_moments<64, true>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream) : launch_moments<64, false>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream);
+        char* y = Y + (size_t)i * rows.total * (fold ? 2 : 1) * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
+        auto launch = [&](auto d, auto r, auto f) { return launch_moments<decltype(d)::value, decltype(r)::value, decltype(f)::value>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream); };
+        auto by_fold = [&](auto d, auto r) { return fold ? launch(d, r, std::true_type{}) : launch(d, r, std::false_type{}); };
+        auto by_rows = [&](auto d) { return rag ? by_fold(d, std::true_type{}) : by_fold(d, std::false_type{}); };
+        err = s.d == 128 ? by_rows(std::integral_constant<int, 128>{}) : by_rows(std::integral_constant<int, 64>{});
         if (err != cudaSuccess) return err;
     }
     rows.nb *= n_layers;
     rows.total *= n_layers;
-    if (s.Hkv % 2 == 0) return rag ? launch_project<2, true>(Y, s, c, n_layers, rows, stream) : launch_project<2, false>(Y, s, c, n_layers, rows, stream);
-    return rag ? launch_project<1, true>(Y, s, c, n_layers, rows, stream) : launch_project<1, false>(Y, s, c, n_layers, rows, stream);
+    if (fold) return rag ? launch_project<1, true, true>(Y, s, c, n_layers, rows, stream) : launch_project<1, false, true>(Y, s, c, n_layers, rows, stream);
+    if (s.Hkv % 2 == 0) return rag ? launch_project<2, true, false>(Y, s, c, n_layers, rows, stream) : launch_project<2, false, false>(Y, s, c, n_layers, rows, stream);
+    return rag ? launch_project<1, true, false>(Y, s, c, n_layers, rows, stream) : launch_project<1, false, false>(Y, s, c, n_layers, rows, stream);
 }
 
 // Coefficients (the caller has zeroed them) and the kept-dim rows of the middle tokens of batch rows b0 .. b0 + nb; the windows
@@ -860,19 +965,21 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
     rows.R = block_tokens(s);
     rows.b0 = b0;
     rows.nb = nb;
+    auto positions = [&](int n_mid) { const int n = blocks_of(n_mid, rows.R); return folds(s) ? (n + 1) / 2 : n; };
     if (lens && lens->n) {
         if (lens->n != s.B) return cudaErrorInvalidValue;
         rows.lens = *lens;
         long long at = 0;
         for (int b = 0; b < s.B; ++b) {
             const int m = mid_of(s, lens->len[b]);
-            if (b >= b0 && b < b0 + nb && m >= tc_min) at += (m + rows.R - 1) / rows.R;
+            if (b >= b0 && b < b0 + nb && m >= tc_min) at += positions(m);
             if (at >= (1ll << 24)) return cudaErrorInvalidValue;
             rows.first[b + 1] = (uint32_t)at;
         }
         rows.total = (int)at;
     } else {
-        rows.nblk = (mid_of(s, L) + rows.R - 1) / rows.R;
+        rows.n_blk = blocks_of(mid_of(s, L), rows.R);
+        rows.nblk = positions(mid_of(s, L));
         if ((long long)rows.nblk * nb >= (1ll << 24)) return cudaErrorInvalidValue;
         rows.total = rows.nblk * nb;
     }
@@ -881,15 +988,16 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
 }
 
 // The same for all batch rows of up to kMomLayers layers of one shape: a moment kernel each, then one projection.  A projection
-// takes 31 us for a layer of 8 heads, 32K tokens and 1024 coefficients, a third of it its start and the segments that teams
-// share, which six layers together pay once: 6 x 31 -> 115 us (ncu; 76 % of the pipe's active cycles).  Y: room for the moments of all of them.
+// takes 31 us (plain form) for a layer of 8 heads, 32K tokens and 1024 coefficients, a third of it its start and the segments that teams
+// share, which six layers together pay once: 6 x 31 -> 115 us, folded 72.  Y: room for the moments of all of them.
 cudaError_t launch_compress_mom_layers(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
                                        int64_t sh, int L, void* Y, bool wait_first, cudaStream_t stream) {
     if (n_layers < 1 || n_layers > kMomLayers) return cudaErrorInvalidValue;
     MomRows rows = {};
     rows.R = block_tokens(s);
     rows.nb = s.B;
-    rows.nblk = (mid_of(s, L) + rows.R - 1) / rows.R;
+    rows.n_blk = blocks_of(mid_of(s, L), rows.R);
+    rows.nblk = folds(s) ? (rows.n_blk + 1) / 2 : rows.n_blk;
     rows.total = rows.nblk * s.B;
     if (rows.total == 0) return cudaSuccess;
     if ((long long)rows.nblk * s.B * n_layers >= (1ll << 24)) return cudaErrorInvalidValue;

@@ -43,6 +43,45 @@ def test_block_moments_against_oracle(kw):
     assert worst <= MOMENT_REL
 
 
+@pytest.mark.parametrize("kw", [
+    # blocks folded about the middle of a row (k a multiple of 256): T = 16384, M = 512: blocks of 384 tokens
+    dict(L=3 * 384 + 68),                                 # odd number of blocks: the middle one by itself
+    dict(L=4 * 384 + 68), dict(L=4 * 384 + 69),           # even; the last block holds one token
+    dict(L=5 * 384 + 68 + 63, B=3),
+    dict(L=16384 + 68),                                   # period full
+    dict(L=5001, Hkv=3, Hq=3, n_full_k=0, n_full_v=128),
+    dict(L=4000, n_full_k=0, n_full_v=0),                 # all 256 columns: three stages
+    dict(L=4999, d=64, n_full_k=64, n_full_v=24, Hkv=4, Hq=4),
+    dict(L=4999, d=64, n_full_k=8, n_full_v=56),
+    dict(L=2900, M=1024, T=32768, B=2),                   # two pairs of tiles
+    dict(L=3000, M=512, T=10000),                         # period not a power of two
+])
+def test_folded_blocks_against_oracle(kw):
+    shape = _shape(**{**dict(M=512, T=16384), **kw})
+    P = 1 if shape.T == 10000 else 8
+    pair, _ = make_pair(shape, seed=72, P=P, max_mid=min(shape.T, shape.L), algo=fa.FA_DECODE_DIRECT, freq="offgrid")
+    assert pair.check_state() <= MOMENT_REL
+
+
+def test_folded_rows_of_different_length():
+    """Rows of odd and even numbers of blocks, one too short for the path, in one call: each as its row alone."""
+    shape = _shape(B=5, L=6000, M=512, T=16384, n_full_k=24, n_full_v=48)
+    layout = layout_of(shape, max_mid=shape.T, P=16)
+    stream = synth.KVStream(shape, seed=10, device="cuda", freq="offgrid")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    lengths = [6000, 700, 1092 + 384, 4 * 384 + 69, 5 * 384 + 68]
+    got = _compress(layout, stream, K, V, fa.new_workspace(layout), lengths)
+    for b, n in enumerate(lengths):
+        one = layout_of(shape.with_(B=1), max_mid=shape.T, P=16)
+        c = _cache(one, stream)
+        fa.fa_compress(one, c, K[b:b + 1, :n], V[b:b + 1, :n], fa.new_workspace(one))
+        torch.cuda.synchronize()
+        for side in ("coef_k", "coef_v"):
+            x, y = getattr(got, side)[b], getattr(c, side)[0]
+            assert ((x - y).abs() <= 1e-5 * y.abs().amax(dim=(-1, -2), keepdim=True)).all(), (b, side)
+        assert torch.equal(got.state[b], c.state[0])
+
+
 def _cache(layout, stream):
     """A cache full of old values: what a call has to write is overwritten, slots past the middle stay."""
     c = fa.Cache(layout, stream.idx_full_k, stream.idx_full_v)
