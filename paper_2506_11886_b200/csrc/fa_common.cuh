@@ -154,7 +154,10 @@ cudaError_t launch_compress_mom(const Dims&, const CacheDev&, const void* K, con
 constexpr int kMomLayers = 8;        // layers of a launch_compress_mom_layers call
 cudaError_t launch_compress_mom_layers(const Dims&, const CacheDev*, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
                                        int64_t sh, int L, void* Y, bool wait_first, cudaStream_t);
-// Tensor-core reconstruction of the dimension selection (fa_select_tc.cu).
+// Reconstruction of the dimension selection by block moments (fa_select_mom.cu) and over coefficient rows (fa_select_tc.cu).
+size_t select_mom_bytes(const Dims& s, int dtype);
+cudaError_t launch_select_mom(const Dims& s, const float* coef_k, const float* coef_v, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh,
+                              int n_init, int n_mid, int L, float* sq, int32_t* status, char* scratch, cudaStream_t stream);
 bool reconstruct_tc_supported(const Dims& s, int dtype, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int n_mid);
 size_t reconstruct_tc_scratch_bytes(const Dims& s);
 cudaError_t launch_reconstruct_tc(const Dims& s, const float* coef_k, const float* coef_v, const void* K, const void* V, int64_t sb,

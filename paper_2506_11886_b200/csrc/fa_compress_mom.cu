@@ -27,29 +27,20 @@
 #include <mutex>
 #include <type_traits>
 
-#include "fa_umma.cuh"
+#include "fa_moments.cuh"
 
 namespace fa {
 namespace {
 
-using bf16 = __nv_bfloat16;
-using namespace umma;
+using namespace mom;
 
-constexpr int kMF = 32;              // moments per block
-constexpr int kChunk = 64;           // tokens per box and pipeline stage
 constexpr int kChunkBytes = 128 * kChunk * 2;      // [64 tokens x 64 dims] twice
 constexpr int kHChunk = 2 * kMF * kChunk * 2;      // P of 64 tokens, hi and lo rows
 constexpr int kAcc = 8;              // accumulators (64 columns each) in tensor memory
 constexpr int kEpiWarps = 4, kGathWarps = 8;
 constexpr int kThreadsMom = 32 * (2 + kEpiWarps + kGathWarps);
-constexpr int kMaxBlockTokens = 768;
 
-__device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-    hi = *reinterpret_cast<const uint32_t*>(&h);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(x - __uint_as_float(hi << 16), y - __uint_as_float(hi & 0xffff0000u));
-    lo = *reinterpret_cast<const uint32_t*>(&l);
-}
+
 // two runs of 16 columns of tensor memory
 __device__ __forceinline__ void tmem_ld16_two(uint32_t a0, uint32_t a1, float (&x)[16], float (&y)[16]) {
     uint32_t r[16], q[16];
@@ -80,7 +71,6 @@ struct MomRows {
     RowLens lens;
     uint32_t first[kMaxRagged + 1];
 };
-__host__ __device__ inline int blocks_of(int n_mid, int R) { return (n_mid + R - 1) / R; }
 
 // Item = (block, KV head[, side]): D = 128: one side's 128 dims, D = 64: K dims and V dims side by side.  A persistent CTA
 // takes items blockIdx.x, blockIdx.x + gridDim.x, ...: CTAs that run together read the same tokens' heads.
@@ -465,12 +455,6 @@ struct MomCuts { uint32_t start[kMaxTeamsP + 1]; };
 // Coefficients of the layers of a launch: its batch row b is row b % B of layer b / B.
 struct MomLayers { int n; float *k[kMomLayers], *v[kMomLayers]; int32_t* status[kMomLayers]; };
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
-                 "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
 // npad: accumulator columns of a product (the compressed dims of both sides, up to a multiple of 32); each CTA of a CTA pair brings half of
 // them.  A stage feeds two products:
 //   as they are: one tile of 128 frequencies (rows Re and Im interleaved) against HP heads;
@@ -625,36 +609,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
             const int fi = t >> LT, tq = t & ((1 << LT) - 1);      // frequency of the tile, this thread's share of the moments
             const unsigned n = (unsigned)(mt * (FOLD ? kBMp : kBMp / 2) + fi);
             float gb[NR];                                  // (2 r + 1) j_r(phi_n) for r = NR tq .. NR tq + NR - 1
-            {
-                // j_r by the recurrence downward from r = 10 + 2.4 phi (55 at most: far enough past phi that what is left out is
-                // below 1e-9, near enough that the values stay in range), scaled by the closed form of j_0 or j_1, whichever is larger
-                float keep[NR], sn, cs, jn = 0.f, jc = 0.f, j0 = 1.f, j1 = 0.f;
-#pragma unroll
-                for (int i = 0; i < NR; ++i) keep[i] = 0.f;
-                const double invd = n ? (double)s.T / (3.14159265358979324 * (double)(n * (unsigned)rows.R)) : 0.0;      // 1 / phi: fp32's rounding of it adds up
-                const float x = (float)(n * (unsigned)rows.R) / (float)s.T, inv = (float)invd;
-                const int top = min(55, 10 + (int)(7.54f * x));
-#pragma unroll 1
-                for (int r8 = 48; r8 >= 0 && n; r8 -= 8) {
-#pragma unroll
-                    for (int i = 7; i >= 0; --i) {         // jc = j_r, jn = j_{r + 1}
-                        const int r = r8 + i;
-                        if (r == top) jc = 1e-20f;
-#pragma unroll
-                        for (int u = 0; u < NR; u += 8)
-                            if (r8 == NR * tq + u) keep[u + i] = (float)(2 * r + 1) * jc;
-                        if (i == 1) j1 = jc;
-                        if (i == 0) j0 = jc;
-                        const float jp = fmaf((float)((double)(2 * r + 1) * invd), jc, -jn);
-                        jn = jc;
-                        jc = jp;
-                    }
-                }
-                sincospif(x, &sn, &cs);
-                const float t0 = sn * inv, t1 = (t0 - cs) * inv, sc = fabsf(t0) > fabsf(t1) ? t0 / j0 : t1 / j1;
-#pragma unroll
-                for (int i = 0; i < NR; ++i) gb[i] = n ? keep[i] * sc : (i == 0 && tq == 0 ? 1.f : 0.f);
-            }
+            legendre_factors<NR>(n, rows.R, s.T, tq, gb);
             const int r0 = FOLD ? fi : 2 * fi, r1 = FOLD ? fi : 2 * fi + 1;
             const uint32_t off0 = (uint32_t)((r0 >> 3) * 1024 + (r0 & 7) * 128), off1 = (uint32_t)((r1 >> 3) * 1024 + (r1 & 7) * 128) + (FOLD ? kABytesP : 0);
             const unsigned T2 = 2u * (unsigned)s.T;
@@ -767,24 +722,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
     }
 }
 
-// 4-D view (dim, head, token, batch) of a prefilled K or V with element strides (1, sh, st, sb); box = 64 dims x 64 tokens.
-bool prefill_map(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int64_t st, int64_t sh, int L) {
-    EncodeTiledFn fn = encode_tiled_fn();
-    if (!fn) return false;
-    cuuint64_t dims[4] = {(cuuint64_t)s.d, (cuuint64_t)s.Hkv, (cuuint64_t)L, (cuuint64_t)s.B};
-    cuuint64_t strides[3] = {(cuuint64_t)sh * 2, (cuuint64_t)st * 2, (cuuint64_t)(s.B > 1 ? sb : st * (int64_t)L) * 2};
-    cuuint32_t box[4] = {64, 1, (cuuint32_t)kChunk, 1};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 int npad_of(const Dims& s) { return (s.dck + s.dcv + 31) / 32 * 32; }
-
-// The longest block of a layout: a whole number of boxes, k R <= 6 T.
-int block_tokens(const Dims& s) {
-    const long long r = 6LL * s.T / s.k / kChunk * kChunk;
-    return (int)(r > kMaxBlockTokens ? kMaxBlockTokens : r);
-}
 
 // Whether the blocks are taken in pairs about the middle of a row: the projection then takes 256 frequencies at a time.
 bool folds(const Dims& s) { return s.k % 256 == 0; }
@@ -873,7 +811,7 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     // Equal cost per team: a segment costs its blocks plus kEpi (epilogue and refill, in blocks); the smallest budget with
     // which the walk covers all positions in n_teams teams, by bisection.
     MomCuts cuts = {};
-    constexpr long long kEpi = 6, kMinSeg = 2;
+    constexpr long long kEpi = FOLD ? 16 : 6, kMinSeg = 2;
     auto unit_end_of = [&](long long pos) {
         long long first = 0, nblk = rows.nblk;
         if (RAG) {

@@ -4,7 +4,8 @@
 //   1. coefficients of all d dims: fa_compress on a scratch cache whose layout compresses everything
 //      (the tensor-core kernel already multiplies all dims), carved from the workspace;
 //   2. the middle tokens rebuilt, x~[j][e] = sum_m w_m F[m][j] C[m][e], and the squared error summed per dim:
-//      for bf16 tensors on the tensor cores (reconstruct_tc_kernel, fa_select_tc.cu), otherwise mse_kernel
+//      for bf16 tensors on the tensor cores, over block moments (fa_select_mom.cu) or coefficient rows
+//      (reconstruct_tc_kernel, fa_select_tc.cu), otherwise mse_kernel
 //      (fp32, 64 middle tokens per CTA, basis by rotation recurrence re-seeded exactly every 16 frequencies);
 //   3. select_kernel: mean over the batch rows, rank by (error, index), write the sorted index sets.
 #include <cstring>
@@ -14,10 +15,12 @@
 namespace fa {
 
 fa_status check_layout(const fa_layout* l);
+fa_status decode_scratch_bytes(const fa_layout* layout, size_t* out);
 
 namespace {
 
 constexpr int kMseTokens = 64;      // middle tokens per CTA
+constexpr int kSelectMomMid = 1024; // middle tokens from which the reconstruction goes by block moments
 constexpr int kMseRows = 32;        // coefficient rows staged per round (16 frequencies)
 
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -132,7 +135,9 @@ struct Scratch {
     char* wc16;                 // weighted coefficients in bf16, the B operand of the tensor-core reconstruction
     char* ws_compress;
     size_t ws_compress_bytes;
-    size_t total;
+    char* mom;                  // scratch of the reconstruction by block moments, behind everything else
+    size_t mom_bytes;
+    size_t least, total;        // what the call cannot do without (direct contractions), what it takes
 };
 
 // Lays the scratch cache (everything compressed) and the error sums out in a workspace.
@@ -162,8 +167,14 @@ fa_status plan_scratch(const fa_layout& l, char* base, Scratch* out) {
     size_t wsb = 0;
     st = fa_workspace_bytes(&sc.layout, &wsb);
     if (st != FA_OK) return st;
+    size_t decode = 0;
+    st = decode_scratch_bytes(&sc.layout, &decode);
+    if (st != FA_OK) return st;
+    sc.least = off + align_up(decode, 256);
     sc.ws_compress = take(wsb);
     sc.ws_compress_bytes = wsb;
+    sc.mom_bytes = select_mom_bytes(make_dims(sc.layout), l.kv_dtype);
+    sc.mom = take(sc.mom_bytes);
     sc.total = off;
     *out = sc;
     return FA_OK;
@@ -216,7 +227,12 @@ fa_status fa_select_dims(const fa_layout* layout, const void* K, const void* V, 
     Scratch sc;
     st = plan_scratch(*layout, static_cast<char*>(ws), &sc);
     if (st != FA_OK) return st;
-    if (ws_bytes < sc.total) return FA_ERR_WORKSPACE;
+    if (ws_bytes < sc.least) return FA_ERR_WORKSPACE;
+    if (ws_bytes < sc.total) {                             // a size from before the moments' scratch was asked for: the compression takes what there is
+        const size_t left = ws_bytes - (size_t)(sc.ws_compress - static_cast<char*>(ws));
+        if (left < sc.ws_compress_bytes) sc.ws_compress_bytes = left;
+        sc.mom_bytes = 0;
+    }
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const Dims s = make_dims(*layout);
     const int n_sq = s.B * s.Hkv * 2 * s.d, n_counters = (int)(sc.ws_compress_bytes < 4096 ? sc.ws_compress_bytes : 4096) / 4;
@@ -230,11 +246,18 @@ fa_status fa_select_dims(const fa_layout* layout, const void* K, const void* V, 
     const int n_init = L < s.l_init ? L : s.l_init;
     const int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;
     const int n_mid = L - n_init - n_local;
-    if (n_mid > 0 && reconstruct_tc_supported(s, layout->kv_dtype, K, V, stride_b, stride_t, stride_h, n_mid)) {
+    bool done = n_mid == 0;
+    if (n_mid >= kSelectMomMid && sc.mom_bytes) {
+        done = launch_select_mom(make_dims(sc.layout), sc.cache.coef_k, sc.cache.coef_v, K, V, stride_b, stride_t, stride_h, n_init, n_mid, L, sc.sq,
+                                 sc.cache.status, sc.mom, cs) == cudaSuccess;
+        if (!done) cudaGetLastError();                     // (the last of its kernels alone adds to the sums)
+    }
+    if (done) {
+    } else if (reconstruct_tc_supported(s, layout->kv_dtype, K, V, stride_b, stride_t, stride_h, n_mid)) {
         if (launch_reconstruct_tc(s, sc.cache.coef_k, sc.cache.coef_v, K, V, stride_b, stride_t, stride_h, n_init, n_mid, sc.sq,
                                   sc.cache.status, sc.wc16, cs) != cudaSuccess)
             return FA_ERR_CUDA;
-    } else if (n_mid > 0) {
+    } else {
         cudaError_t err = layout->kv_dtype == FA_BF16
                               ? launch_mse<__nv_bfloat16>(s, sc.cache, K, V, stride_b, stride_t, stride_h, n_init, n_mid, sc.sq, cs)
                               : launch_mse<float>(s, sc.cache, K, V, stride_b, stride_t, stride_h, n_init, n_mid, sc.sq, cs);

@@ -79,6 +79,68 @@ def test_tensor_core_reconstruction_against_oracle_and_fp32_path(Hkv, d, M, L):
     np.testing.assert_allclose(to64(got[4])[big], to64(got32[4])[big], rtol=5e-3)
 
 
+@pytest.mark.parametrize("kw", [
+    dict(L=1024 + 36, M=256, T=4096),                     # shortest middle of this path: five blocks of 192 tokens and one of 64
+    dict(L=1152 + 36, M=256, T=4096), dict(L=1153 + 36, M=256, T=4096),      # whole blocks, and one token more (odd number: the middle one by itself)
+    dict(L=9 * 192 + 36 + 65, M=256, T=4096, B=1, Hkv=3),                    # ten blocks: two tiles of pairs
+    dict(L=4096 + 36, M=256, T=4096, Hkv=1),              # period full
+    dict(L=2500, M=512, T=16384, d=64),                   # K and V in one item
+    dict(L=2222, M=256, T=65536, L_init=0, L_local=1),    # the longest blocks
+    dict(L=1500, M=256, T=5000),                          # period not a power of two
+    dict(L=1500, M=256, T=4096, norm=1),                  # the paper's weights
+])
+def test_reconstruction_by_block_moments(kw):
+    """Against the same quantity in 64 bits: x~ from its definition (coefficients, weights, basis by phases
+    reduced in integers).  Factors carry 2^-17 and coefficients 4e-6: relative to a dim's mean square and to its error (cross term
+    2 sqrt(error * mean square) * 2e-5)."""
+    kw = dict(kw)
+    norm = kw.pop("norm", 0)
+    shape = synth.Shape("selm", **{**dict(B=2, layers=1, Hq=2, Hkv=2, d=128, dtype="bf16", n_full_k=32, n_full_v=24, L_init=4, L_local=32), **kw,
+                                   "Hq": kw.get("Hkv", 2)})
+    layout = layout_of(shape, max_mid=shape.T, P=1 if shape.T == 5000 else 16)
+    layout.norm = norm
+    stream = synth.KVStream(shape, seed=29, device="cuda", freq="offgrid")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    got = fa.fa_select_dims(layout, K, V)[4].double()
+    n0 = min(shape.L, shape.L_init)
+    X = torch.stack([K, V], 3)[:, n0:shape.L - min(shape.L - n0, shape.L_local)].double()            # [B][mid][H][2][d]
+    n = X.shape[1]
+    ph = (torch.arange(n, device="cuda")[None] * torch.arange(shape.M // 2, device="cuda")[:, None]) % shape.T
+    ang = ph.double() * (2 * np.pi / shape.T)
+    F = torch.stack([ang.cos(), ang.sin()], 1).reshape(shape.M, n)
+    w = torch.full((shape.M,), 2.0 / shape.T, dtype=torch.float64, device="cuda")
+    w[:2] = torch.tensor([1.0 / shape.T, 0.0])
+    if norm:
+        w[:] = 1.0 / (shape.M // 2)
+    C = torch.einsum("mj,bjhse->bhsme", F, X)
+    want = (torch.einsum("mj,bhsme->bjhse", F * w[:, None], C) - X).square().mean(1)
+    power = torch.einsum("mj,bhsme->bjhse", F * w[:, None], C).square().mean(1) + X.square().mean(1)
+    assert ((got - want).abs() <= 4e-5 * (want * power).sqrt() + 1e-8 * power).all()
+
+
+def test_select_workspace_of_an_older_size():
+    """A workspace without room for the moments is taken as before, by the direct contractions."""
+    import ctypes as C
+    shape = synth.Shape("selw", B=1, layers=1, Hq=2, Hkv=2, d=128, L=2000, dtype="bf16", n_full_k=32, n_full_v=32, M=256, T=4096, L_init=4, L_local=32)
+    layout = layout_of(shape, max_mid=4096, P=16)
+    K, V = (x.cuda().contiguous() for x in synth.KVStream(shape, seed=3).tokens(0, 2000))
+    want = fa.fa_select_dims(layout, K, V)
+    mom_row = -(-4096 // 192) * 2 * 256 * 128
+    full = C.c_size_t(0)
+    assert fa.lib().fa_select_workspace_bytes(C.byref(layout.c()), C.byref(full)) == fa.FA_OK
+    for drop in (256, 2 * 128 * 4 * 256 * 2 + 32 * 128 * 4 + mom_row + 8 * mom_row):          # the last bytes; all moments, of both directions
+        ws = torch.zeros(full.value - drop, dtype=torch.uint8, device="cuda")
+        idx = [torch.zeros_like(t) for t in want[:4]]
+        mse = torch.zeros_like(want[4])
+        st = fa.lib().fa_select_dims(C.byref(layout.c()), K.data_ptr(), V.data_ptr(), K.stride(0), K.stride(1), K.stride(2), 2000,
+                                     *[t.data_ptr() for t in idx], mse.data_ptr(), ws.data_ptr(), ws.numel(), None)
+        torch.cuda.synchronize()
+        assert st == fa.FA_OK
+        for a, b in zip(idx, want[:4]):
+            assert torch.equal(a, b)
+        torch.testing.assert_close(mse, want[4], rtol=2e-2, atol=4e-6)          # (basis and coefficients in bf16: 1e-6 of the mean square)
+
+
 def test_select_dims_empty_middle_and_workspace_check():
     shape = synth.Shape("sel0", B=1, layers=1, Hq=2, Hkv=2, d=64, L=20, dtype="bf16", n_full_k=16, n_full_v=8, M=16,
                         T=256, L_init=4, L_local=32)
