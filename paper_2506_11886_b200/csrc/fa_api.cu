@@ -406,7 +406,7 @@ static cudaError_t compress_by_moments(const Dims& s, const CacheDev& c, const v
     for (int b0 = 0, i = 0; b0 < s.B; b0 += group, ++i) {
         const int nb = s.B - b0 < group ? s.B - b0 : group;
         char* Y = room.at + (fit >= 2 && (i & 1) ? (size_t)group * row : 0);
-        const cudaError_t err = launch_compress_mom(s, c, K, V, sb, st, sh, L, b0, nb, Y, fit < 2 && i > 0, stream, lens, tc_min);
+        const cudaError_t err = launch_compress_mom(s, c, K, V, sb, st, sh, L, b0, nb, Y, fit < 2 && i > 0, i > 0, stream, lens, tc_min);
         if (err != cudaSuccess) return err;
     }
     return cudaSuccess;
@@ -527,10 +527,10 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
     // block moments where the workspace has room for them; the order-fixed mode keeps the direct contraction
     const MomentRoom room = tc && !ordered ? moment_room(*layout, ws, ws_bytes) : MomentRoom{nullptr, 0};
     if (room.at && room.bytes >= compress_mom_row_bytes(s, n_mid_host)) {
-        if (launch_compress(s, make_cache(*cache), layout->kv_dtype, K, V, stride_b, stride_t, stride_h, L, false, false, kTcMinMid, true, cs) != cudaSuccess)
-            return FA_ERR_CUDA;
-        if (compress_by_moments(s, make_cache(*cache), K, V, sbb, stride_t, stride_h, L, room, cs) == cudaSuccess) return FA_OK;
-        cudaGetLastError();                                 // the cluster launch was refused: everything below once more
+        const CacheDev c = make_cache(*cache);
+        if (compress_by_moments(s, c, K, V, sbb, stride_t, stride_h, L, room, cs) == cudaSuccess)
+            return launch_windows(s, &c, &K, &V, 1, sbb, stride_t, stride_h, L, cs) == cudaSuccess ? FA_OK : FA_ERR_CUDA;
+        cudaGetLastError();                                 // the cluster launch was refused: everything below, from the start
     }
     // tensor-core path: its kernel also writes the kept-dim rows of the middle from the boxes it loads; the partition
     // kernel is left with the windows and the counters
@@ -625,10 +625,10 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
         most = need > most ? need : most;
     }
     moments = moments && room.bytes >= most;
-    for (int i = 0; i < n_layers; ++i) {
+    for (int i = 0; i < n_layers && !moments; ++i) {
         const Dims s = make_dims(layouts[i]);
-        if (launch_compress(s, make_cache(caches[i]), layouts[i].kv_dtype, K[i], V[i], stride_b, stride_t, stride_h, L, false, ordered, kTcMinMid,
-                            true, cs, i > 0) != cudaSuccess)
+        if (launch_compress(s, make_cache(caches[i]), layouts[i].kv_dtype, K[i], V[i], stride_b, stride_t, stride_h, L, false, ordered, kTcMinMid, 1, cs,
+                            i > 0) != cudaSuccess)
             return FA_ERR_CUDA;
     }
     // Groups of layers take the two halves of the room in turn where they fit them, so that a group's moments are formed while
@@ -651,7 +651,7 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
             for (int j = 0; j < n; ++j) c[j] = make_cache(caches[i + j]);
             const bool whole = n * need > half;
             err = launch_compress_mom_layers(s, c, K + i, V + i, n, sbb, stride_t, stride_h, L, room.at + (!whole && odd ? half : 0),
-                                             i > 0 && (whole || behind_whole), cs);
+                                             i > 0 && (whole || behind_whole), i > 0, cs);
             behind_whole = whole;
             odd = !odd;
         } else {
@@ -660,12 +660,20 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
         if (err != cudaSuccess) {
             // the cluster launch was refused: finish this and the remaining layers one by one (each call redoes its layer in full)
             cudaGetLastError();
-            for (int j = i; j < n_layers; ++j) {
+            for (int j = moments ? 0 : i; j < n_layers; ++j) {
                 const fa_status st = fa_compress_ex(&layouts[j], &caches[j], K[j], V[j], stride_b, stride_t, stride_h, L, flags, ws, ws_bytes, stream);
                 if (st != FA_OK) return st;
             }
             return FA_OK;
         }
+    }
+    // (with the moments, whose kernels clear the coefficients, the windows at the end, beside the last projection)
+    for (int i = 0, n; i < n_layers && moments; i += n) {
+        for (n = 1; n < kMomLayers && i + n < n_layers && std::memcmp(&layouts[i + n], &layouts[i], sizeof(fa_layout)) == 0;) ++n;
+        CacheDev c[kMomLayers];
+        for (int j = 0; j < n; ++j) c[j] = make_cache(caches[i + j]);
+        const Dims s = make_dims(layouts[i]);
+        if (launch_windows(s, c, K + i, V + i, n, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, cs) != cudaSuccess) return FA_ERR_CUDA;
     }
     return FA_OK;
 }
@@ -745,19 +753,25 @@ fa_status fa_compress_ragged(const fa_layout* layout, fa_cache* cache, const voi
             if (L == 0) { L = Lmax; }                     // (the kernels go by the rows' lengths)
             const void *Kb = prefill(K, b0), *Vb = prefill(V, b0);
             const bool tc = pairs && shortest < part.batch;
-            if (launch_compress(s, make_cache(rows), layout->kv_dtype, Kb, Vb, stride_b, stride_t, stride_h, L, true, false,
-                                tc ? kTcMinMid : kNoTc, true, cs, false, &lens) != cudaSuccess)
-                return FA_ERR_CUDA;
+            auto partition = [&](bool behind) {            // behind the moments, whose kernels clear the coefficients of the long rows
+                return launch_compress(s, make_cache(rows), layout->kv_dtype, Kb, Vb, stride_b, stride_t, stride_h, L, true, false, tc ? kTcMinMid : kNoTc,
+                                       behind ? 2 : 1, cs, behind, &lens);
+            };
             int n_mid = 0;
             for (int i = 0; i < part.batch; ++i) n_mid = mid_of(s, lens.len[i]) > n_mid ? mid_of(s, lens.len[i]) : n_mid;
             const MomentRoom room = tc ? moment_room(*layout, ws, ws_bytes) : MomentRoom{nullptr, 0};
             if (room.at && room.bytes >= compress_mom_row_bytes(s, n_mid)) {
                 if (compress_by_moments(s, make_cache(rows), Kb, Vb, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, room, cs, &lens,
-                                        kTcMinMid) == cudaSuccess)
+                                        kTcMinMid) == cudaSuccess) {
+                    const CacheDev c = make_cache(rows);
+                    if ((shortest ? partition(true) : launch_windows(s, &c, &Kb, &Vb, 1, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, cs, &lens)) != cudaSuccess)
+                        return FA_ERR_CUDA;
                     continue;
+                }
                 cudaGetLastError();                       // the cluster launch was refused: these rows and the rest one by one
                 break;
             }
+            if (partition(false) != cudaSuccess) return FA_ERR_CUDA;
             if (tc && launch_compress_tc2(s, make_cache(rows), Kb, Vb, s.B > 1 ? stride_b : 0, stride_t, stride_h, L, false, cs, &lens,
                                           kTcMinMid) != cudaSuccess) {
                 cudaGetLastError();                       // the cluster launch was refused: these rows and the rest one by one

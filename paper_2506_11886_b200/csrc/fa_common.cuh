@@ -139,7 +139,7 @@ constexpr int kNoTc = 0x7fffffff;
 // Kernel launchers (defined next to their kernels).  All return the launch error, if any.
 cudaError_t launch_validate(const Dims&, const CacheDev&, cudaStream_t);
 cudaError_t launch_compress(const Dims&, const CacheDev&, int dtype, const void* K, const void* V, int64_t sb,
-                            int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, bool zero_coef, cudaStream_t,
+                            int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, int zero_coef, cudaStream_t,
                             bool chained = false, const RowLens* lens = nullptr);
 bool compress_tc_gathers(const Dims& s);
 // The same path on CTA pairs (fa_compress_tc2.cu): needs an even number of 128-row tiles.
@@ -150,10 +150,12 @@ cudaError_t launch_compress_tc2(const Dims&, const CacheDev&, const void* K, con
 bool compress_mom_supported(const Dims& s);
 size_t compress_mom_row_bytes(const Dims& s, int n_mid);
 cudaError_t launch_compress_mom(const Dims&, const CacheDev&, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int L, int b0,
-                                int nb, void* Y, bool wait_first, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
+                                int nb, void* Y, bool wait_first, bool chained, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
 constexpr int kMomLayers = 8;        // layers of a launch_compress_mom_layers call
 cudaError_t launch_compress_mom_layers(const Dims&, const CacheDev*, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
-                                       int64_t sh, int L, void* Y, bool wait_first, cudaStream_t);
+                                       int64_t sh, int L, void* Y, bool wait_first, bool chained, cudaStream_t);
+cudaError_t launch_windows(const Dims&, const CacheDev*, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st, int64_t sh, int L,
+                           cudaStream_t, const RowLens* lens = nullptr);
 // Reconstruction of the dimension selection by block moments (fa_select_mom.cu) and over coefficient rows (fa_select_tc.cu).
 size_t select_mom_bytes(const Dims& s, int dtype);
 cudaError_t launch_select_mom(const Dims& s, const float* coef_k, const float* coef_v, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh,

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
         c.state[kStateStride * b + 4] = 0;          // append ticket
     }
     const int nfull = side == 0 ? s.nfk : s.nfv;
-    if (zero_coef && s.d > nfull) {
+    if ((zero_coef == 1 || (zero_coef == 2 && n_mid < tc_min)) && s.d > nfull) {
         // the contraction kernels behind this one ADD their partial sums: the CTAs of a (b, head, side) clear its coefficients
         float4* cz = reinterpret_cast<float4*>(coef_rows(side == 0 ? c.coef_k : c.coef_v, s, b, h, s.d - nfull));
         const int n4 = s.M * (s.d - nfull) / 4;
@@ -116,8 +116,11 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
         if (dst) reinterpret_cast<uint4*>(dst)[ch] = reinterpret_cast<const uint4*>(rows_s)[i];
     }
     // kept-dim rows of the middle
+    // (one CTA waits for the kernel in front, so that the end of this grid implies that one's; if all did, they would keep theirs from
+    // taking turns beside a projection)
+    const bool waits = blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
     if (!mid_rows) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (waits) asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }
     const int cpo = nfull / EPC;                          // chunks per output row
@@ -138,6 +141,7 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
     // programmatically behind the one before), the end of this grid then implies the end of all before it.  Launched
     // the plain way this returns at once.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (waits) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---- Eq.3-4: C[m][e] += sum_j F[m][j] X[n_init + j][D^c[e]] ------------------
@@ -240,7 +244,7 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
 
 template <typename KV>
 static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb,
-                                     int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, bool zero_coef, bool chained,
+                                     int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, int zero_coef, bool chained,
                                      const RowLens* lens, cudaStream_t stream) {
     RowLens rl = {};
     if (lens) rl = *lens;
@@ -276,7 +280,7 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
         cfg.attrs = attr;
         cfg.numAttrs = chained ? 1 : 0;
         err = cudaLaunchKernelEx(&cfg, partition_gather_kernel<KV>, s, c, static_cast<const KV*>(K), static_cast<const KV*>(V), sb, st, sh, L,
-                                 rl, tc_min, zero_coef ? 1 : 0);
+                                 rl, tc_min, zero_coef);
     }
     if (err != cudaSuccess) return err;
     int max_comp = s.dck > s.dcv ? s.dck : s.dcv;
@@ -321,9 +325,10 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
 // with_coef = false runs only the partition / gather kernel (the tensor-core or the transform path computes the
 // coefficients); rows with at least tc_min middle tokens get no kept-dim rows and no coefficients here (windows and
 // counters only: the tensor-core kernel writes the rest); lens: prompt lengths of the batch rows (at most L), or none;
-// zero_coef clears the coefficients in the same launch (for the contraction kernels, which add to them).
+// zero_coef: 1 clears the coefficients in the same launch (for the contraction kernels, which add to them), 2 those of the rows with fewer than
+// tc_min middle tokens; chained: may run beside the kernel of the same call in front of it.
 cudaError_t launch_compress(const Dims& s, const CacheDev& c, int dtype, const void* K, const void* V, int64_t sb,
-                            int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, bool zero_coef,
+                            int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, int zero_coef,
                             cudaStream_t stream, bool chained, const RowLens* lens) {
     if (dtype == FA_BF16) return launch_compress_t<__nv_bfloat16>(s, c, K, V, sb, st, sh, L, with_coef, ordered, tc_min, zero_coef, chained, lens, stream);
     return launch_compress_t<float>(s, c, K, V, sb, st, sh, L, with_coef, ordered, tc_min, zero_coef, chained, lens, stream);

@@ -20,10 +20,11 @@
 // share of the measured rate; its write of the moments is 10 % of the traffic at k / T = 1 / 64 and 20 % at 1 / 32), the
 // second the tensor cores (1152 cycles of products a position and pair) plus 20 K cycles a segment, at the rate at which L2 adds vectors of
 // floats (four rows of 128 K tokens: 242 K cycles, 69 % of them on the tensor cores).
-// Direct contraction against this path: six layers of 32 K tokens, 1024 rows: 701 -> 374 us, with one projection for all 333, folded 292; 128 K
-// tokens, batch 4, 2048 rows: 3207 -> 777, folded 674 us; six ragged rows of 3 to 12 K tokens, 512 rows: 123 -> 85, folded 79 us; 4 K tokens of 256
-// heads, 256 rows (T / k = 32, blocks of 192 tokens, too few frequencies to fold): 231 -> 221 us.  The projection of the four rows of 128 K tokens alone:
-// 275 -> 162 us.  Relative error of the coefficients 4e-6 against 2.4e-4.
+// Direct contraction against this path, in us: six layers of 32 K tokens, 1024 rows: 701 -> 374, with one projection for all 333, folded 292, the
+// moments of all layers in one launch and the windows beside the projection 277; 128 K tokens, batch 4, 2048 rows: 3207 -> 777, folded 674; six ragged
+// rows of 3 to 12 K tokens, 512 rows: 123 -> 85, folded 79, windows beside it 73; 4 K tokens of 256 heads, 256 rows (T / k = 32, blocks of 192
+// tokens, too few frequencies to fold): 231 -> 221, windows beside it 199.  The projection of the four rows of 128 K tokens alone:
+// 275 -> 162.  Relative error of the coefficients 4e-6 against 2.4e-4.
 #include <mutex>
 #include <type_traits>
 
@@ -72,12 +73,18 @@ struct MomRows {
     uint32_t first[kMaxRagged + 1];
 };
 
+// Layers of a launch: its batch row b is row b % B of layer b / B (several layers, all of their rows; one, some of them).
+struct MomIn {
+    CUtensorMap k[kMomLayers], v[kMomLayers];
+    CacheDev c[kMomLayers];
+    int n;
+};
+
 // Item = (block, KV head[, side]): D = 128: one side's 128 dims, D = 64: K dims and V dims side by side.  A persistent CTA
 // takes items blockIdx.x, blockIdx.x + gridDim.x, ...: CTAs that run together read the same tokens' heads.
 template <int D, bool RAG, bool FOLD>
-__global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                                                                 Dims s, CacheDev c, int Lall, const __grid_constant__ MomRows rows, bf16* __restrict__ Y,
-                                                                 int n_stages, int n_items, int wait_first) {
+__global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_constant__ MomIn in, Dims s, int Lall, const __grid_constant__ MomRows rows,
+                                                                 bf16* __restrict__ Y, int n_stages, int n_items, int wait_first) {
     constexpr int kSides = D == 128 ? 2 : 1;               // items per (block, head)
     constexpr int kTypes = FOLD ? 2 : 1;                   // operands per position: real and imaginary rows want different sums of a pair
     // A: 64-dim rows of a token, MN-major; B: P, K-major; M = 128 dims, N = 64 (hi and lo rows of P)
@@ -95,8 +102,9 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
     uint64_t* masked = acc_empty + kAcc;                   // per stage: rows past the end of a batch row's last box are zero
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(masked + n_stages);
     volatile int* fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    uint8_t* inv_s = reinterpret_cast<uint8_t*>(tmem_slot + 2);      // [Hkv][2][D] position of a dim among the compressed ones, 255: kept
-    uint8_t* idf_s = inv_s + s.Hkv * 2 * D;                          // [Hkv][nfk + nfv] the kept dims
+    uint8_t* inv_s = reinterpret_cast<uint8_t*>(tmem_slot + 2);      // [layer][Hkv][2][D] position of a dim among the compressed ones, 255: kept
+    uint8_t* idf_s = inv_s + in.n * s.Hkv * 2 * D;                   // [layer][Hkv][nfk + nfv] the kept dims
+    int32_t* status = in.c[0].status;
     const int nf = s.nfk + s.nfv;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -118,8 +126,9 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
         constexpr int kW = kThreadsMom / 32 - 1;
         const int u = tid - 32, wu = warp - 1;
         // where a dim is: a warp takes whole rows (head, side)
-        for (int r = wu; r < 2 * s.Hkv; r += kW) {
-            const int h = r >> 1, sd = r & 1, nfr = sd ? s.nfv : s.nfk, ncr = D - nfr;
+        for (int r = wu; r < 2 * in.n * s.Hkv; r += kW) {
+            const int lh = r >> 1, sd = r & 1, nfr = sd ? s.nfv : s.nfk, ncr = D - nfr, layer = lh / s.Hkv, h = lh - layer * s.Hkv;
+            const CacheDev& c = in.c[layer];
             const int32_t* idf = (sd ? c.idx_full_v : c.idx_full_k) + h * nfr;
             const int32_t* idc = (sd ? c.idx_comp_v : c.idx_comp_k) + h * ncr;
             uint8_t* inv = inv_s + r * D;
@@ -127,7 +136,7 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
             for (int e0 = 0; e0 < D; e0 += 32) {
                 const int e = e0 + lane;
                 const int d = e < nfr ? idf[e] : idc[e - nfr];
-                if (e < nfr) idf_s[h * nf + (sd ? s.nfk : 0) + e] = (uint8_t)d;
+                if (e < nfr) idf_s[lh * nf + (sd ? s.nfk : 0) + e] = (uint8_t)d;
                 inv[d] = e < nfr ? 255 : (uint8_t)(e - nfr);
             }
         }
@@ -155,14 +164,14 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
 
     // A role's place in the CTA's items: the next item is gridDim.x further on, taken by additions with carries.
     const int n_mid_all = mid_of(s, Lall);
-    struct Walk { int i, side, h, gblk, b, blk, nblk, n_mid, n_blk; };
+    struct Walk { int i, side, h, gblk, b, blk, nblk, n_mid, n_blk, layer; };      // (b: row of the layer)
     const int d_side = kSides == 2 ? (int)gridDim.x & 1 : 0, d_t = kSides == 2 ? (int)gridDim.x >> 1 : (int)gridDim.x;
     const int d_blk = d_t / s.Hkv, d_h = d_t - d_blk * s.Hkv;
     auto settle = [&](Walk& w) {                           // block number -> batch row and block of the row
         if (w.i >= n_items) return;
         while (w.blk >= w.nblk) {
             w.blk -= w.nblk;
-            ++w.b;
+            if (++w.b == s.B && w.layer + 1 < in.n) { w.b = 0; ++w.layer; }
             if (RAG) w.nblk = (int)(rows.first[w.b + 1] - rows.first[w.b]);
         }
         if (RAG) w.n_mid = mid_of(s, rows.lens.len[w.b]);
@@ -181,6 +190,7 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
         w.h = t - w.gblk * s.Hkv;
         w.blk = w.gblk;
         w.b = RAG ? 0 : rows.b0;
+        w.layer = 0;
         w.nblk = RAG ? (int)rows.first[1] : rows.nblk;
         w.n_mid = n_mid_all;
         w.n_blk = FOLD ? blocks_of(n_mid_all, rows.R) : 0;
@@ -211,16 +221,16 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
                 const int blk = block_of(it, half), n_ch = boxes_of(it, blk);
                 int tok = s.l_init + blk * rows.R;
                 for (int q = 0; q < n_ch; ++q, tok += kChunk) {
-                    if (!mbar_wait(empty + st, par, fail, c.status)) { live = false; break; }
+                    if (!mbar_wait(empty + st, par, fail, status)) { live = false; break; }
                     unsigned char* dst = stage0 + (size_t)st * kChunkBytes;
                     mbar_expect_tx(full + st, (uint32_t)kChunkBytes);
                     if (kSides == 2) {
-                        const CUtensorMap* tm = it.side ? &tmV : &tmK;
+                        const CUtensorMap* tm = it.side ? &in.v[it.layer] : &in.k[it.layer];
                         tma_load_4d(dst, tm, 0, it.h, tok, it.b, full + st);
                         tma_load_4d(dst + kChunkBytes / 2, tm, 64, it.h, tok, it.b, full + st);
                     } else {
-                        tma_load_4d(dst, &tmK, 0, it.h, tok, it.b, full + st);
-                        tma_load_4d(dst + kChunkBytes / 2, &tmV, 0, it.h, tok, it.b, full + st);
+                        tma_load_4d(dst, &in.k[it.layer], 0, it.h, tok, it.b, full + st);
+                        tma_load_4d(dst + kChunkBytes / 2, &in.v[it.layer], 0, it.h, tok, it.b, full + st);
                     }
                     ++issued;
                     if (++st == n_stages) { st = 0; par ^= 1; }
@@ -242,14 +252,14 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
             for (int half = 0; live && half < halves(it); ++half, ++a) {
                 const int blk = block_of(it, half), n_ch = boxes_of(it, blk);
                 const int ab = a % kAcc;
-                if (a >= kAcc && !mbar_wait(acc_empty + ab, ((a / kAcc) - 1) & 1, fail, c.status)) { live = false; break; }
+                if (a >= kAcc && !mbar_wait(acc_empty + ab, ((a / kAcc) - 1) & 1, fail, status)) { live = false; break; }
                 const uint32_t acc = tmem_base + ab * (2 * kMF);
                 uint64_t hdesc = hdesc0;
                 int left = it.n_mid - blk * rows.R;
                 for (int q = 0; q < n_ch; ++q, left -= kChunk, hdesc += kHChunk >> 4) {
-                    if (!mbar_wait(full + st, par, fail, c.status)) { live = false; break; }
+                    if (!mbar_wait(full + st, par, fail, status)) { live = false; break; }
                     if (left < kChunk) {
-                        if (!mbar_wait(masked + st, (mpar >> st) & 1u, fail, c.status)) { live = false; break; }
+                        if (!mbar_wait(masked + st, (mpar >> st) & 1u, fail, status)) { live = false; break; }
                         mpar ^= 1u << st;
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -268,14 +278,24 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
         if (wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");   // Y may still be read by the kernel before this one
         const int lg = warp & 3, e = lg * 32 + lane;       // tensor-memory lane: the dim, or (D = 64) K's dims then V's
         const int ncol = s.dck + s.dcv;
+        // the projection adds to the coefficients: they are cleared here
+        for (int lb = 0; lb < rows.nb; ++lb) {
+            const int layer = lb / s.B, b = rows.b0 + lb - layer * s.B;
+            if (RAG && rows.first[b] == rows.first[b + 1]) continue;       // (a short row: the direct contraction's)
+            for (int sd = 0; sd < 2; ++sd) {
+                const int nc = sd ? s.dcv : s.dck, n4 = s.Hkv * (s.M >> 2) * nc;
+                float4* z = reinterpret_cast<float4*>(coef_rows(sd ? in.c[layer].coef_v : in.c[layer].coef_k, s, b, 0, nc));
+                for (int i = blockIdx.x * (32 * kEpiWarps) + tid - 64; i < n4; i += gridDim.x * (32 * kEpiWarps)) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
         int a = 0;
         for (Walk it = walk_begin(); it.i < n_items; walk_next(it)) {
             const int n_half = halves(it);
             // (after a time-out the walk goes on, on what is there: the four warps keep meeting)
-            for (int half = 0; half < n_half; ++half) mbar_wait(acc_full + (a + half) % kAcc, ((a + half) / kAcc) & 1, fail, c.status);
+            for (int half = 0; half < n_half; ++half) mbar_wait(acc_full + (a + half) % kAcc, ((a + half) / kAcc) & 1, fail, status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int side = kSides == 2 ? it.side : e >> 6, dim = kSides == 2 ? e : e & 63;
-            const int pos = inv_s[(it.h * 2 + side) * D + dim];
+            const int pos = inv_s[((it.layer * s.Hkv + it.h) * 2 + side) * D + dim];
             // The columns of the item are one contiguous run of rows of Y: they are put together in shared memory and leave with one
             // bulk copy (stored by the lanes, every 16 bytes went to a line of its own).  The 16-byte pieces of a row are
             // permuted as the 128-byte swizzle of the products' operand wants them, so the second kernel copies rows as they are.
@@ -370,7 +390,7 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
 #pragma unroll
                 for (int u = 0; u < 4; ++u) o[u] = 0;
                 if (on) {
-                    const uint8_t* id = idf_s + it.h * nf + (v ? s.nfk : 0) + 8 * (v ? p - nk8 : p);
+                    const uint8_t* id = idf_s + (it.layer * s.Hkv + it.h) * nf + (v ? s.nfk : 0) + 8 * (v ? p - nk8 : p);
                     const int bx = kSides == 1 && v ? kChunkBytes / 2 : 0;
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
@@ -381,12 +401,12 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
                 }
                 const uint32_t col = (uint32_t)(16 * (v ? p - nk8 : p));
                 const int mask = v ? vmask : 0;
-                char* dst0 = reinterpret_cast<char*>(v ? c.v_mid : c.k_mid) + bh * (size_t)rowb;
+                char* dst0 = reinterpret_cast<char*>(v ? in.c[it.layer].v_mid : in.c[it.layer].k_mid) + bh * (size_t)rowb;
                 for (int half = 0; live && half < halves(it); ++half) {
                 const int blk = block_of(it, half), n_ch = boxes_of(it, blk);
                 int j0 = blk * rows.R + 8 * w + sub, left = it.n_mid - blk * rows.R;
                 for (int q = 0; q < n_ch; ++q, j0 += kChunk, left -= kChunk) {
-                    if (!mbar_wait(full + st, par, fail, c.status)) { live = false; break; }
+                    if (!mbar_wait(full + st, par, fail, status)) { live = false; break; }
                     const uint32_t box = smem_u32(stage0) + (uint32_t)(st * kChunkBytes + w * 1024), src = box + (uint32_t)(sub * 128);
                     uint4 val[NI];
 #pragma unroll
@@ -435,6 +455,8 @@ __global__ void __launch_bounds__(kThreadsMom, 1) moments_kernel(const __grid_co
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (tid == 0 && *fail)                                 // (a wait that runs out tells the first layer)
+        for (int l = 1; l < in.n; ++l) in.c[l].status[0] = status[0];
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
@@ -462,8 +484,9 @@ struct MomLayers { int n; float *k[kMomLayers], *v[kMomLayers]; int32_t* status[
 //     cos E + i sin O with E, O = Y+ +- Y-.  By the parity of i^r, the real part of e^{-i theta n m} C_n takes E of even r and O of odd r only, the
 //     imaginary part the others: two tiles (256 frequencies, Re; the same, Im) against one head's two operands, each 32 long for TWO
 //     blocks.  Half the products of the plain form; the epilogue turns (Re, Im) by e^{i theta n m} in registers.
+// (128 registers at most: three warps on one scheduler then leave room for those of the windows kernel's, or the partition kernel's, CTAs)
 template <int HP, bool RAG, bool FOLD>
-__global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16* __restrict__ Y, Dims s, const __grid_constant__ MomLayers layers,
+__global__ void __maxnreg__(128) moment_project_kernel(const bf16* __restrict__ Y, Dims s, const __grid_constant__ MomLayers layers,
                                                                       const __grid_constant__ MomRows rows, const __grid_constant__ MomCuts cuts, int npad, int n_stages) {
     constexpr int kTiles = FOLD ? 2 : 1, kOps = FOLD ? 2 : HP;     // A tiles and B operands of a stage
     const int nh = npad >> 1, b_op = nh * 128, n_stage = kTiles * kABytesP + kOps * b_op;     // rows of 128 bytes
@@ -487,7 +510,8 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
     const int n_hg = s.Hkv / HP, ncol = s.dck + s.dcv;
     const uint32_t pos_begin = cuts.start[team], pos_end = cuts.start[team + 1];
     int32_t* status = layers.status[0];
-    struct Seg { int b, h0, kb0, kb1, n_blk; uint32_t g0; };      // batch row, heads, positions, blocks of the row, first position of the row in the launch
+    // batch row, heads, positions, blocks of the row, whether these are all positions of the unit; first position of the row in the launch
+    struct Seg { int b, h0, kb0, kb1, n_blk; bool whole; uint32_t g0; };
     auto seg_at = [&](uint32_t pos) {
         int b, nblk = rows.nblk;
         uint32_t g0, off;
@@ -505,7 +529,8 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
         }
         const int hg = (int)(off / (uint32_t)nblk), kb0 = (int)off - hg * nblk;
         const int n_blk = !FOLD ? 0 : RAG ? blocks_of(mid_of(s, rows.lens.len[b]), rows.R) : rows.n_blk;
-        return Seg{b, hg * HP, kb0, (int)min((uint32_t)nblk, (uint32_t)kb0 + (pos_end - pos)), n_blk, g0};
+        const int kb1 = (int)min((uint32_t)nblk, (uint32_t)kb0 + (pos_end - pos));
+        return Seg{b, hg * HP, kb0, kb1, n_blk, kb0 == 0 && kb1 == nblk, g0};
     };
 
     if (tid == 0) {
@@ -666,22 +691,30 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
 #pragma unroll 1
                     for (int pc = part; pc < HP * npc; pc += 2) {
                         const int hh = pc / npc, c0 = (pc - hh * npc) * 32;
-                        float v[32];
-                        tmem_ld32(tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(hh * 256 + c0), v);
-                        if (FOLD) {
-                            float w[32];
-                            tmem_ld32(tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(256 + c0), w);
+                        const uint32_t at = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(hh * 256 + c0);
+                        if (FOLD) {                        // (16 columns at a time: registers, see below)
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) {
-                                const float re = cm * v[i] - sm * w[i];
-                                w[i] = sm * v[i] + cm * w[i];
-                                v[i] = re;
+                            for (int x = 0; x < 32; x += 16) {
+                                float v[16], w[16];
+                                tmem_ld16_two(at + x, at + 256 + x, v, w);
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) {
+                                    const float re = cm * v[i] - sm * w[i];
+                                    w[i] = sm * v[i] + cm * w[i];
+                                    v[i] = re;
+                                }
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    *reinterpret_cast<float4*>(tile + lane * 36 + x + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                                    *reinterpret_cast<float4*>(tile + (32 + lane) * 36 + x + 4 * i) = make_float4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                                }
                             }
+                        } else {
+                            float v[32];
+                            tmem_ld32(at, v);
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + (32 + lane) * 36 + 4 * i) = make_float4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                            for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + lane * 36 + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
                         }
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + lane * 36 + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
                         __syncwarp();
                         const int q = lane & 7, rr0 = lane >> 3, col = c0 + 4 * q;
                         if (col < ncol) {
@@ -693,8 +726,10 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
                                 // row of the coefficients: the tile's, or (folded) Re in rows 0 - 31 and Im in 32 - 63 of the tile, taken in turn
                                 const int m = rr0 + 4 * i, src = FOLD ? (m >> 1) + 32 * (m & 1) : m;
                                 const float4 x = *reinterpret_cast<const float4*>(tile + src * 36 + 4 * q);
-                                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + (size_t)m * nc), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w)
-                                             : "memory");
+                                if (g.whole) *reinterpret_cast<float4*>(dst + (size_t)m * nc) = x;       // nobody else adds to these
+                                else
+                                    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + (size_t)m * nc), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w)
+                                                 : "memory");
                             }
                         }
                         __syncwarp();
@@ -722,25 +757,111 @@ __global__ void __launch_bounds__(kThreadsP, 1) moment_project_kernel(const bf16
     }
 }
 
+// ---- windows and counters -------------------------------------------------------------------------------------------
+// Behind the projection and beside it: that one leaves the memory idle, this one needs a warp and 49 KB.  A CTA takes a few boxes of 64 tokens of one head and
+// side, which one lane moves: in by TMA, out by bulk copies (the window rows of a head are contiguous), two boxes on their way in all the time.
+// 270 MB of 256 heads and a projection of 43 us: one after the other 101 us, the partition kernel (16-byte loads and stores, 24 warps of it beside the
+// projection) 77 us, this one 63.
+constexpr int kWinStages = 3, kWinBytes = 64 * 256;
+struct WinIn {
+    CUtensorMap k[kMomLayers], v[kMomLayers];
+    CacheDev c[kMomLayers];
+    int n;
+};
+__global__ void __launch_bounds__(32) windows_kernel(const __grid_constant__ WinIn in, Dims s, int Lall, const __grid_constant__ RowLens lens, int n_init_ch,
+                                                     int n_ch, int per_cta, int n_items) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kWinStages * kWinBytes);
+    volatile int* fail = reinterpret_cast<volatile int*>(full + kWinStages);
+    const int lane = threadIdx.x;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (blockIdx.x == 0)
+        for (int i = lane; i < in.n * s.B; i += 32) {
+            const int layer = i / s.B, b = i - layer * s.B, L = row_len(lens, Lall, b), n_init = min(L, s.l_init), n_local = min(L - n_init, s.l_local);
+            int32_t* st = in.c[layer].state + kStateStride * b;
+            st[0] = n_init;
+            st[1] = n_local;
+            st[2] = L - n_init - n_local;
+            st[3] = 0;                                     // ring starts at physical row 0
+            st[4] = 0;                                     // append ticket
+        }
+    if (lane == 0) {
+        for (int i = 0; i < kWinStages; ++i) mbar_init(full + i, 1);
+        *fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // box i: head fastest, then the chunk of the windows, side, batch row, layer
+        struct Box { int layer, b, h, side, tok, rows; bf16* dst; };
+        auto box = [&](int i) {
+            Box x;
+            int r = i / s.Hkv, ch;
+            x.h = i - r * s.Hkv;
+            ch = r % n_ch; r /= n_ch;
+            x.side = r & 1; r >>= 1;
+            x.layer = r / s.B;
+            x.b = r - x.layer * s.B;
+            const int L = row_len(lens, Lall, x.b), n_init = min(L, s.l_init), n_local = min(L - n_init, s.l_local);
+            const CacheDev& c = in.c[x.layer];
+            const int row = (ch < n_init_ch ? ch : ch - n_init_ch) * 64, n = ch < n_init_ch ? n_init : n_local;
+            x.rows = min(64, n - row);
+            x.tok = (ch < n_init_ch ? 0 : L - n_local) + row;
+            x.dst = x.rows <= 0 ? nullptr : ch < n_init_ch ? win_row<bf16>(x.side ? c.v_init : c.k_init, s, x.b, x.h, s.l_init, row)
+                                                           : win_row<bf16>(x.side ? c.v_local : c.k_local, s, x.b, x.h, s.l_local, row);
+            return x;
+        };
+        const int i0 = blockIdx.x * per_cta, i1 = min(n_items, i0 + per_cta);
+        const uint32_t bytes = (uint32_t)(64 * s.d * 2);
+        auto load = [&](int i) {
+            const Box x = box(i);
+            const int st = (i - i0) % kWinStages;
+            if (x.rows <= 0) { mbar_arrive(full + st); return; }
+            mbar_expect_tx(full + st, bytes);
+            tma_load_4d(smem + st * kWinBytes, x.side ? &in.v[x.layer] : &in.k[x.layer], 0, x.h, x.tok, x.b, full + st);
+        };
+        for (int i = i0; i < i1 && i < i0 + kWinStages - 1; ++i) load(i);
+        int i = i0;
+        for (; i < i1; ++i) {
+            const int st = (i - i0) % kWinStages;
+            if (!mbar_wait(full + st, ((i - i0) / kWinStages) & 1, fail, in.c[0].status)) break;
+            const Box x = box(i);
+            if (x.rows > 0)
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(x.dst)), "r"(smem_u32(smem + st * kWinBytes)),
+                             "r"(x.rows * s.d * 2)
+                             : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");       // the copy before has read its stage
+            if (i + kWinStages - 1 < i1) load(i + kWinStages - 1);
+        }
+        if (i < i1)                                        // a wait ran out: the boxes under way land, or the bound is reached, first
+            for (int q = i; q < i1 && q < i + kWinStages - 1; ++q)
+                for (uint32_t n = 0; n < (1u << 16) && !mbar_try_wait(full + (q - i0) % kWinStages, ((q - i0) / kWinStages) & 1); ++n) { }
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        if (*fail)
+            for (int l = 1; l < in.n; ++l) in.c[l].status[0] = in.c[0].status[0];
+        // (one CTA waits for the kernel in front, so that the end of this grid implies that one's)
+        if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
+}
+
 int npad_of(const Dims& s) { return (s.dck + s.dcv + 31) / 32 * 32; }
 
 // Whether the blocks are taken in pairs about the middle of a row: the projection then takes 256 frequencies at a time.
 bool folds(const Dims& s) { return s.k % 256 == 0; }
 
-size_t mom_smem_fixed(const Dims& s) {      // everything but the stages, the slack of the alignment among it
-    return (size_t)block_tokens(s) / kChunk * kHChunk + (folds(s) ? 2 : 1) * 128 * 4 * kMF + 8 * (3 * 16 + 2 * kAcc) + 16 + (size_t)s.Hkv * (2 * s.d + s.nfk + s.nfv) + 64 + 1024;
+size_t mom_tables(const Dims& s) { return (size_t)s.Hkv * (2 * s.d + s.nfk + s.nfv); }
+size_t mom_smem_fixed(const Dims& s, int n_layers = 1) {      // everything but the stages, the slack of the alignment among it
+    return (size_t)block_tokens(s) / kChunk * kHChunk + (folds(s) ? 2 : 1) * 128 * 4 * kMF + 8 * (3 * 16 + 2 * kAcc) + 16 + (size_t)n_layers * mom_tables(s) + 64 + 1024;
 }
-int mom_stages(const Dims& s) {
-    const long long left = 227 * 1024 - (long long)mom_smem_fixed(s);
+int mom_stages(const Dims& s, int n_layers = 1) {
+    const long long left = 227 * 1024 - (long long)mom_smem_fixed(s, n_layers);
     const int n = (int)(left / kChunkBytes);
     return n > 16 ? 16 : n;
 }
 
+// chained: behind a kernel of the same call (else all work in front of it on the stream has ended when it starts, so that it may write anything)
 template <int D, bool RAG, bool FOLD>
-cudaError_t launch_moments(const CUtensorMap& tmK, const CUtensorMap& tmV, const Dims& s, const CacheDev& c, int L, const MomRows& rows, void* Y,
-                           bool wait_first, cudaStream_t stream) {
-    const int n_stages = mom_stages(s);
-    const size_t smem = mom_smem_fixed(s) + (size_t)n_stages * kChunkBytes;
+cudaError_t launch_moments(const MomIn& in, const Dims& s, int L, const MomRows& rows, void* Y, bool wait_first, bool chained, cudaStream_t stream) {
+    const int n_stages = mom_stages(s, in.n);
+    const size_t smem = mom_smem_fixed(s, in.n) + (size_t)n_stages * kChunkBytes;
     cudaError_t err = ensure_dynamic_smem(moments_kernel<D, RAG, FOLD>, smem);
     if (err != cudaSuccess) return err;
     const long long items = (long long)rows.total * s.Hkv * (D == 128 ? 2 : 1);
@@ -754,8 +875,8 @@ cudaError_t launch_moments(const CUtensorMap& tmK, const CUtensorMap& tmV, const
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, moments_kernel<D, RAG, FOLD>, tmK, tmV, s, c, L, rows, static_cast<bf16*>(Y), n_stages, (int)items, wait_first ? 1 : 0);
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, moments_kernel<D, RAG, FOLD>, in, s, L, rows, static_cast<bf16*>(Y), n_stages, (int)items, wait_first ? 1 : 0);
 }
 
 template <int HP, bool RAG, bool FOLD>
@@ -764,7 +885,8 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     layers.n = n_layers;
     for (int i = 0; i < n_layers; ++i) { layers.k[i] = c[i].coef_k; layers.v[i] = c[i].coef_v; layers.status[i] = c[i].status; }
     const size_t stage = FOLD ? 2 * kABytesP + (size_t)npad_of(s) * 128 : kABytesP + (size_t)HP * (npad_of(s) / 2) * 128, fixed = 8 * (3 * kStagesP + 2) + 16 + 1024;
-    const int fit = (int)((227 * 1024 - fixed) / stage), n_stages = fit < kStagesP ? fit : kStagesP;
+    // (room for a CTA of the windows kernel beside it)
+    const int fit = (int)((227 * 1024 - (kWinStages * kWinBytes + 2048) - fixed) / stage), n_stages = fit < kStagesP ? fit : kStagesP;
     const size_t smem = n_stages * stage + fixed;
     cudaError_t err = ensure_dynamic_smem(moment_project_kernel<HP, RAG, FOLD>, smem);
     if (err != cudaSuccess) return err;
@@ -772,15 +894,18 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     cfg.blockDim = dim3(kThreadsP);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
+    // all of the SM's memory as shared memory, whatever this kernel takes of it: CTAs of the windows kernel start beside it
+    attr[2].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[2].val.sharedMemCarveout = 100;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 3;
     const int n_pairs = s.M / ((FOLD ? 4 : 2) * kBMp), n_hg = s.Hkv / HP;
     const long long total = (long long)rows.total * n_hg;
     if (total <= 0 || total >= (1ll << 31)) return cudaErrorInvalidValue;
@@ -800,7 +925,7 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
                 cudaGetLastError();
                 n = sm_count() / 2 - 2;
             }
-            cfg.numAttrs = 2;
+            cfg.numAttrs = 3;
             resident[dev] = n;
         }
         n_teams = resident[dev] / n_pairs;
@@ -873,14 +998,26 @@ size_t compress_mom_row_bytes(const Dims& s, int n_mid) {
 }
 
 static cudaError_t launch_rows(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
-                               int64_t sh, int L, MomRows rows, char* Y, bool wait_first, cudaStream_t stream) {
+                               int64_t sh, int L, MomRows rows, char* Y, bool wait_first, bool chained, cudaStream_t stream) {
     const bool rag = rows.lens.n != 0, fold = folds(s);
     cudaError_t err;
-    for (int i = 0; i < n_layers; ++i) {
-        CUtensorMap tmK, tmV;
-        if (!prefill_map(&tmK, K[i], s, sb, st, sh, L) || !prefill_map(&tmV, V[i], s, sb, st, sh, L)) return cudaErrorInvalidValue;
+    // Layers to a launch: as many as a sixth of the ring's room holds the tables of.  A launch of its own for each pays its start, its first loads
+    // and its last items every time.
+    int per = (int)(32 * 1024 / (mom_tables(s) + 1));
+    if (per < 1) per = 1;
+    per = (n_layers + (n_layers + per - 1) / per - 1) / ((n_layers + per - 1) / per);
+    for (int i = 0; i < n_layers; i += per) {
+        MomIn in = {};
+        in.n = n_layers - i < per ? n_layers - i : per;
+        for (int l = 0; l < in.n; ++l) {
+            in.c[l] = c[i + l];
+            if (!prefill_map(&in.k[l], K[i + l], s, sb, st, sh, L) || !prefill_map(&in.v[l], V[i + l], s, sb, st, sh, L)) return cudaErrorInvalidValue;
+        }
+        MomRows part = rows;
+        part.nb *= in.n;
+        part.total *= in.n;
         char* y = Y + (size_t)i * rows.total * (fold ? 2 : 1) * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
-        auto launch = [&](auto d, auto r, auto f) { return launch_moments<decltype(d)::value, decltype(r)::value, decltype(f)::value>(tmK, tmV, s, c[i], L, rows, y, wait_first, stream); };
+        auto launch = [&](auto d, auto r, auto f) { return launch_moments<decltype(d)::value, decltype(r)::value, decltype(f)::value>(in, s, L, part, y, wait_first, chained || i > 0, stream); };
         auto by_fold = [&](auto d, auto r) { return fold ? launch(d, r, std::true_type{}) : launch(d, r, std::false_type{}); };
         auto by_rows = [&](auto d) { return rag ? by_fold(d, std::true_type{}) : by_fold(d, std::false_type{}); };
         err = s.d == 128 ? by_rows(std::integral_constant<int, 128>{}) : by_rows(std::integral_constant<int, 64>{});
@@ -893,12 +1030,12 @@ static cudaError_t launch_rows(const Dims& s, const CacheDev* c, const void* con
     return rag ? launch_project<1, true, false>(Y, s, c, n_layers, rows, stream) : launch_project<1, false, false>(Y, s, c, n_layers, rows, stream);
 }
 
-// Coefficients (the caller has zeroed them) and the kept-dim rows of the middle tokens of batch rows b0 .. b0 + nb; the windows
-// and the counters are the caller's (the partition kernel).  lens: prompt lengths of all batch rows (at most L; rows
+// Coefficients and the kept-dim rows of the middle tokens of batch rows b0 .. b0 + nb; the windows and the counters are left to launch_windows
+// or the partition kernel, launched behind.  lens: prompt lengths of all batch rows (at most L; rows
 // with fewer than tc_min middle tokens are left out), or none.  Y: room for these rows' moments, 128-byte aligned;
-// wait_first: a kernel of this stream that may still run reads Y.
+// wait_first: a kernel of this call that may still run reads Y; chained: there is a kernel of this call in front.
 cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int L, int b0,
-                                int nb, void* Y, bool wait_first, cudaStream_t stream, const RowLens* lens, int tc_min) {
+                                int nb, void* Y, bool wait_first, bool chained, cudaStream_t stream, const RowLens* lens, int tc_min) {
     MomRows rows = {};
     rows.R = block_tokens(s);
     rows.b0 = b0;
@@ -922,14 +1059,14 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
         rows.total = rows.nblk * nb;
     }
     if (rows.total == 0) return cudaSuccess;
-    return launch_rows(s, &c, &K, &V, 1, sb, st, sh, L, rows, static_cast<char*>(Y), wait_first, stream);
+    return launch_rows(s, &c, &K, &V, 1, sb, st, sh, L, rows, static_cast<char*>(Y), wait_first, chained, stream);
 }
 
 // The same for all batch rows of up to kMomLayers layers of one shape: a moment kernel each, then one projection.  A projection
 // takes 31 us (plain form) for a layer of 8 heads, 32K tokens and 1024 coefficients, a third of it its start and the segments that teams
 // share, which six layers together pay once: 6 x 31 -> 115 us, folded 72.  Y: room for the moments of all of them.
 cudaError_t launch_compress_mom_layers(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
-                                       int64_t sh, int L, void* Y, bool wait_first, cudaStream_t stream) {
+                                       int64_t sh, int L, void* Y, bool wait_first, bool chained, cudaStream_t stream) {
     if (n_layers < 1 || n_layers > kMomLayers) return cudaErrorInvalidValue;
     MomRows rows = {};
     rows.R = block_tokens(s);
@@ -939,7 +1076,47 @@ cudaError_t launch_compress_mom_layers(const Dims& s, const CacheDev* c, const v
     rows.total = rows.nblk * s.B;
     if (rows.total == 0) return cudaSuccess;
     if ((long long)rows.nblk * s.B * n_layers >= (1ll << 24)) return cudaErrorInvalidValue;
-    return launch_rows(s, c, K, V, n_layers, sb, st, sh, L, rows, static_cast<char*>(Y), wait_first, stream);
+    return launch_rows(s, c, K, V, n_layers, sb, st, sh, L, rows, static_cast<char*>(Y), wait_first, chained, stream);
+}
+
+// The windows and counters of layers whose middles launch_compress_mom(_layers) has enqueued in front, on the same stream.
+cudaError_t launch_windows(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st, int64_t sh, int L,
+                           cudaStream_t stream, const RowLens* lens) {
+    RowLens rl = {};
+    if (lens) rl = *lens;
+    // chunks of the longest windows of any row (a row's own may be fewer)
+    const int n_init = L < s.l_init ? L : s.l_init, n_local = L - n_init < s.l_local ? L - n_init : s.l_local;
+    const int n_init_ch = (n_init + 63) / 64, n_ch = n_init_ch + (n_local + 63) / 64;
+    const size_t smem = kWinStages * kWinBytes + 8 * kWinStages + 16;
+    cudaError_t err = ensure_dynamic_smem(windows_kernel, smem);
+    if (err != cudaSuccess) return err;
+    for (int i = 0; i < n_layers; i += kMomLayers) {
+        WinIn in = {};
+        in.n = n_layers - i < kMomLayers ? n_layers - i : kMomLayers;
+        for (int l = 0; l < in.n; ++l) {
+            in.c[l] = c[i + l];
+            if (!prefill_map(&in.k[l], K[i + l], s, sb, st, sh, L, s.d, CU_TENSOR_MAP_SWIZZLE_NONE) || !prefill_map(&in.v[l], V[i + l], s, sb, st, sh, L, s.d, CU_TENSOR_MAP_SWIZZLE_NONE))
+                return cudaErrorInvalidValue;
+        }
+        const long long items = (long long)in.n * s.B * 2 * n_ch * s.Hkv;
+        if (items >= (1ll << 30)) return cudaErrorInvalidValue;
+        // (a few boxes to a CTA: short enough for an even end, long enough for the ring to pay)
+        long long per = items / (2 * sm_count());
+        per = per < 3 ? 3 : per > 8 ? 8 : per;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(items > 0 ? (items + per - 1) / per : 1));
+        cfg.blockDim = dim3(32);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        err = cudaLaunchKernelEx(&cfg, windows_kernel, in, s, L, rl, n_init_ch, n_ch > 0 ? n_ch : 1, (int)per, (int)items);
+        if (err != cudaSuccess) return err;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace fa

@@ -65,16 +65,17 @@ __device__ __forceinline__ void legendre_factors(unsigned n, int R, int T, int t
     for (int i = 0; i < NR; ++i) gb[i] = n ? keep[i] * sc : (i == 0 && tq == 0 ? 1.f : 0.f);
 }
 
-// 4-D view (dim, head, token, batch) of a prefilled K or V with element strides (1, sh, st, sb); box = 64 dims x 64 tokens.
-inline bool prefill_map(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int64_t st, int64_t sh, int L) {
+// 4-D view (dim, head, token, batch) of a prefilled K or V with element strides (1, sh, st, sb); box = box_dims dims x 64 tokens.
+inline bool prefill_map(CUtensorMap* tm, const void* base, const Dims& s, int64_t sb, int64_t st, int64_t sh, int L, int box_dims = 64,
+                        CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     cuuint64_t dims[4] = {(cuuint64_t)s.d, (cuuint64_t)s.Hkv, (cuuint64_t)L, (cuuint64_t)s.B};
     cuuint64_t strides[3] = {(cuuint64_t)sh * 2, (cuuint64_t)st * 2, (cuuint64_t)(s.B > 1 ? sb : st * (int64_t)L) * 2};
-    cuuint32_t box[4] = {64, 1, (cuuint32_t)kChunk, 1};
+    cuuint32_t box[4] = {(cuuint32_t)box_dims, 1, (cuuint32_t)kChunk, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+              swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace mom

@@ -82,6 +82,30 @@ def test_folded_rows_of_different_length():
         assert torch.equal(got.state[b], c.state[0])
 
 
+@pytest.mark.parametrize("l_init,l_local,d", [(0, 0, 128), (4, 63, 128), (64, 64, 64), (70, 65, 128), (1, 700, 64)])
+def test_windows_behind_the_projection(l_init, l_local, d):
+    """Window rows are the prompt's, slots past them stay, rows of one length (several boxes to a CTA) and of different ones."""
+    shape = _shape(B=3, Hkv=4, Hq=4, L=2000 + l_init + l_local, d=d, n_full_k=16, n_full_v=16, L_init=l_init, L_local=l_local)
+    layout = layout_of(shape, max_mid=shape.T, P=16)
+    stream = synth.KVStream(shape, seed=5, device="cuda", freq="offgrid")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    for lengths in (None, [shape.L, l_init + l_local + 1100, shape.L - 1]):
+        c = _cache(layout, stream)
+        for n in ("k_init", "v_init", "k_local", "v_local"):
+            getattr(c, n).fill_(3.0)
+        ws = fa.new_workspace(layout)
+        if lengths:
+            fa.fa_compress_ragged(layout, c, K, V, lengths, ws)
+        else:
+            fa.fa_compress(layout, c, K, V, ws)
+        torch.cuda.synchronize()
+        assert fa.fa_poll_status(c) == fa.FA_OK
+        for b, n in enumerate(lengths or [shape.L] * 3):
+            assert c.state[b, :5].tolist() == [l_init, l_local, n - l_init - l_local, 0, 0]
+            for X, init, local in ((K, c.k_init, c.k_local), (V, c.v_init, c.v_local)):
+                assert torch.equal(init[b], X[b, :l_init].transpose(0, 1)) and torch.equal(local[b], X[b, n - l_local:n].transpose(0, 1))
+
+
 def _cache(layout, stream):
     """A cache full of old values: what a call has to write is overwritten, slots past the middle stay."""
     c = fa.Cache(layout, stream.idx_full_k, stream.idx_full_v)
