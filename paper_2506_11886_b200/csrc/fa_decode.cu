@@ -15,22 +15,22 @@ namespace fa {
 // dims, and on the way back the threads share out frequencies and groups of tokens.  The kernel is bound by its chain of
 // dependent steps, so what counts is that a call has many short CTAs: 1024 fp32 tokens of one head are 16 CTAs of one
 // tile instead of four CTAs that walked eight classes each with 32 of their 256 threads (compress and decode of that
-// cache together: 99 -> 35 us).
+// cache together: 99 -> 35 us; with the launches of the call chained and everything that does not need u in front of the wait for it: 27).
 constexpr int kTile = 64, kLanes = 4;
 
 template <int GH>
 struct RunStat {
     float m[GH];   // running max, log2 units
-    float l[GH];   // running sum of p
+    float l[GH];   // running sum of p over this thread's tokens
 };
 
-// Block-wide max / sum of GH values per thread; result broadcast to every thread.
-template <int GH, bool IS_MAX>
-__device__ __forceinline__ void block_reduce(float (&v)[GH], float* red_s /* [8][GH] */) {
+// Block-wide maximum of GH values per thread; result broadcast to every thread.
+template <int GH>
+__device__ __forceinline__ void block_max(float (&v)[GH], float* red_s /* [8][GH] */) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
     for (int g = 0; g < GH; ++g) {
-        float r = IS_MAX ? warp_max(v[g]) : warp_sum(v[g]);
+        const float r = warp_max(v[g]);
         if (lane == 0) red_s[warp * GH + g] = r;
     }
     __syncthreads();
@@ -38,7 +38,7 @@ __device__ __forceinline__ void block_reduce(float (&v)[GH], float* red_s /* [8]
     for (int g = 0; g < GH; ++g) {
         float r = red_s[g];
 #pragma unroll
-        for (int w = 1; w < 8; ++w) r = IS_MAX ? fmaxf(r, red_s[w * GH + g]) : r + red_s[w * GH + g];
+        for (int w = 1; w < 8; ++w) r = fmaxf(r, red_s[w * GH + g]);
         v[g] = r;
     }
     __syncthreads();
@@ -66,26 +66,51 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
     float* o_s = red_s + 8 * GH;              // [GH][d]  final reduce
     float* acc_s = o_s + GH * s.d;            // [256][GH] cross-thread reduce of the output accumulators
 
-    const int n_init = c.state[kStateStride * b + 0], n_local = c.state[kStateStride * b + 1];
-    const int n_mid = min(c.state[kStateStride * b + 2], s.max_mid), head = c.state[kStateStride * b + 3];
-    const int32_t* idf_k = c.idx_full_k + (size_t)h * s.nfk;
+    // Everything but u was there before this call: the kernel in front lets this one start when the work before it has ended.  The rows of the
+    // first tile are fetched, and their kept-dim scores formed, while that kernel makes u.
+    const int4 st4 = *reinterpret_cast<const int4*>(c.state + kStateStride * b);
+    const int n_init = st4.x, n_local = st4.y, n_mid = min(st4.z, s.max_mid), head = st4.w;
     const int32_t* idf_v = c.idx_full_v + (size_t)h * s.nfv;
+    const int idf_k = tid < s.nfk ? c.idx_full_k[(size_t)h * s.nfk + tid] : 0;
+    // middle tokens [j0, j1) of this split; four lanes to a token; (token group, dim) map of the P.V product
+    const int per = (n_mid + p.n_split - 1) / p.n_split;
+    const int j0 = min(n_mid, split * per), j1 = min(n_mid, j0 + per);
+    const bool p2 = (s.P & (s.P - 1)) == 0;
+    const int lgP = 31 - __clz(s.P);
+    auto cls_of = [&](int j) { return p2 ? j & (s.P - 1) : j % s.P; };
+    auto slot_of = [&](int j) { return p2 ? j >> lgP : j / s.P; };
+    const int tk = tid / kLanes, ql = tid % kLanes;
+    const int ntg_mid = s.nfv > 0 ? 256 / s.nfv : 0;
+    const int tg_mid = s.nfv > 0 ? tid / s.nfv : 0, e_mid = s.nfv > 0 ? tid % s.nfv : 0;
+    const bool act_mid = s.nfv > 0 && tg_mid < ntg_mid;
+    auto k_row = [&](int j) { return mid_row<KV>(c.k_mid, s, b, h, cls_of(j), slot_of(j), s.nfk); };
+    auto v_at = [&](int j) {
+        const int slot = slot_of(j);
+        return ld_f(mid_row<KV>(c.v_mid, s, b, h, cls_of(j), slot, s.nfv) + v_mid_col(slot, e_mid, s.nfv, sizeof(KV) == 2 ? FA_BF16 : FA_F32));
+    };
+    constexpr int kPre = 8;                                 // values of K and of V of the first tile that a thread fetches ahead
+    float k_pre[kPre], v_pre[kPre];
+    {
+        const KV* row = j0 + tk < j1 ? k_row(j0 + tk) : nullptr;
+#pragma unroll
+        for (int u = 0; u < kPre; ++u) k_pre[u] = row && ql + u * kLanes < s.nfk ? ld_f(row + ql + u * kLanes) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+        const int j = j0 + tg_mid + u * ntg_mid;
+        v_pre[u] = act_mid && j < min(j1, j0 + kTile) ? v_at(j) : 0.f;
+    }
 
     for (int i = tid; i < GH * s.d; i += blockDim.x) {
         int g = i / s.d, e = i - g * s.d;
         q_s[i] = g < ng ? ld_f(q + ((size_t)b * s.Hq + g_first + g) * s.d + e) * s.scale * kLog2e : 0.f;
         o_s[i] = 0.f;
     }
-    for (int i = tid; i < GH * s.M; i += blockDim.x) {
-        int g = i / s.M, m = i - g * s.M;
-        u_s[i] = (g < ng && s.dck > 0) ? ws.u[((size_t)b * s.Hq + g_first + g) * s.M + m] : 0.f;
-        z_s[i] = 0.f;
-    }
+    for (int i = tid; i < GH * s.M; i += blockDim.x) z_s[i] = 0.f;
     __syncthreads();
-    for (int i = tid; i < GH * s.nfk; i += blockDim.x) {
-        int g = i / s.nfk, e = i - g * s.nfk;
-        qf_s[i] = q_s[g * s.d + idf_k[e]];
-    }
+    if (tid < s.nfk)
+#pragma unroll
+        for (int g = 0; g < GH; ++g) qf_s[g * s.nfk + tid] = q_s[g * s.d + idf_k];
     __syncthreads();
 
     RunStat<GH> rs;
@@ -95,38 +120,36 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
 #pragma unroll
     for (int g = 0; g < GH; ++g) { o_mid[g] = 0.f; o_win[g] = 0.f; }
 
-    // thread -> (token group, dim) maps of the two P.V products
-    const int ntg_mid = s.nfv > 0 ? 256 / s.nfv : 0;
-    const int tg_mid = s.nfv > 0 ? tid / s.nfv : 0, e_mid = s.nfv > 0 ? tid % s.nfv : 0;
-    const bool act_mid = s.nfv > 0 && tg_mid < ntg_mid;
+    // thread -> (token group, dim) map of the windows' P.V product
     const int ntg_win = 256 / s.d;
     const int tg_win = tid / s.d, e_win = tid % s.d;
     const bool act_win = tg_win < ntg_win;
 
     // after scores are known (every one of a token's four lanes has them): update the running softmax state, leave p in p_s
-    const int tk = tid / kLanes, ql = tid % kLanes;
+    bool first = true;                        // (z_s is zero)
     auto softmax_tile = [&](float (&sc)[GH], bool valid) {
         float mx[GH];
 #pragma unroll
         for (int g = 0; g < GH; ++g) mx[g] = valid ? sc[g] : kNegBig;
-        block_reduce<GH, true>(mx, red_s);
-        float pv[GH], alpha[GH];
+        block_max<GH>(mx, red_s);
+        float alpha[GH];
 #pragma unroll
         for (int g = 0; g < GH; ++g) {
             float m_new = fmaxf(rs.m[g], mx[g]);
             alpha[g] = exp2f(rs.m[g] - m_new);
             rs.m[g] = m_new;
-            pv[g] = valid && ql == 0 ? exp2f(sc[g] - m_new) : 0.f;
-            if (ql == 0) p_s[g * kTile + tk] = pv[g];
+            const float pv = valid && ql == 0 ? exp2f(sc[g] - m_new) : 0.f;
+            if (ql == 0) p_s[g * kTile + tk] = pv;
+            rs.l[g] = rs.l[g] * alpha[g] + pv;      // this thread's tokens: summed over the block at the end
             o_mid[g] *= alpha[g];
             o_win[g] *= alpha[g];
         }
+        if (!first)
 #pragma unroll
-        for (int g = 0; g < GH; ++g)
-            for (int m = tid; m < s.M; m += 256) z_s[g * s.M + m] *= alpha[g];
-        block_reduce<GH, false>(pv, red_s);     // also publishes p_s and the z_s rescale
-#pragma unroll
-        for (int g = 0; g < GH; ++g) rs.l[g] = rs.l[g] * alpha[g] + pv[g];
+            for (int g = 0; g < GH; ++g)
+                for (int m = tid; m < s.M; m += 256) z_s[g * s.M + m] *= alpha[g];
+        first = false;
+        __syncthreads();                        // p_s, z_s
     };
     auto lanes_sum = [&](float (&sc)[GH]) {
 #pragma unroll
@@ -135,41 +158,64 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
             sc[g] += __shfl_xor_sync(0xffffffffu, sc[g], 2);
         }
     };
-    const bool p2 = (s.P & (s.P - 1)) == 0;
-    const int lgP = 31 - __clz(s.P);
-    auto cls_of = [&](int j) { return p2 ? j & (s.P - 1) : j % s.P; };
-    auto slot_of = [&](int j) { return p2 ? j >> lgP : j / s.P; };
-
-    // ---- middle tokens [j0, j1) of this split ------------------------
-    const int per = (n_mid + p.n_split - 1) / p.n_split;
-    const int j0 = min(n_mid, split * per), j1 = min(n_mid, j0 + per);
     // frequencies of a lane, and the way back: kz frequencies at a time, 256 / kz groups of tokens
     const int per_lane = (s.k + kLanes - 1) / kLanes;
     int kz = 32;
     while (kz < s.k && kz < 256) kz *= 2;
     const int n_grp = 256 / kz, zt = tid / kz, zn = tid % kz;
+    auto kept_scores = [&](int j, float (&sc)[GH], bool ahead) {
+#pragma unroll
+        for (int g = 0; g < GH; ++g) sc[g] = 0.f;
+        if (j >= j1) return;
+        const KV* row = k_row(j);
+        int e = ql;
+        if (ahead)
+#pragma unroll
+            for (int u = 0; u < kPre; ++u, e += kLanes)
+                if (e < s.nfk)
+#pragma unroll
+                    for (int g = 0; g < GH; ++g) sc[g] = fmaf(qf_s[g * s.nfk + e], k_pre[u], sc[g]);
+#pragma unroll 8
+        for (; e < s.nfk; e += kLanes) {
+            float x = ld_f(row + e);
+#pragma unroll
+            for (int g = 0; g < GH; ++g) sc[g] = fmaf(qf_s[g * s.nfk + e], x, sc[g]);
+        }
+    };
+    float sc_first[GH];
+    kept_scores(j0 + tk, sc_first, true);
+    // the basis of the first tile: a token's rotation and its lane's first frequency; a frequency's rotation and its first token
+    float cd1 = 0.f, sd1 = 0.f, cr1 = 0.f, sr1 = 0.f, zc1 = 0.f, zs1 = 0.f, zr1 = 0.f, zi1 = 0.f;
+    if (s.dck > 0 && j0 + tk < j1) { basis_cs(1, j0 + tk, s.T, &cd1, &sd1); basis_cs(ql * per_lane, j0 + tk, s.T, &cr1, &sr1); }
+    if (s.dcv > 0 && zn < s.k) { basis_cs(zn, 1, s.T, &zc1, &zs1); basis_cs(zn, j0 + zt * (kTile / n_grp), s.T, &zr1, &zi1); }
+    asm volatile("griddepcontrol.wait;" ::: "memory");     // u
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int i = tid; i < GH * s.M; i += blockDim.x) {
+        const int g = i / s.M, m = i - g * s.M;
+        u_s[i] = (g < ng && s.dck > 0) ? ws.u[((size_t)b * s.Hq + g_first + g) * s.M + m] : 0.f;
+    }
+    __syncthreads();
     for (int t0 = j0; t0 < j1; t0 += kTile) {
         const int j = t0 + tk;
         const bool valid = j < j1;
         const int nt = min(kTile, j1 - t0);
         float sc[GH];
+        if (t0 == j0) {
 #pragma unroll
-        for (int g = 0; g < GH; ++g) sc[g] = 0.f;
+            for (int g = 0; g < GH; ++g) sc[g] = sc_first[g];
+        } else {
+            kept_scores(j, sc, false);
+        }
         if (valid) {
-            const KV* row = mid_row<KV>(c.k_mid, s, b, h, cls_of(j), slot_of(j), s.nfk);
-#pragma unroll 8
-            for (int e = ql; e < s.nfk; e += kLanes) {
-                float x = ld_f(row + e);
-#pragma unroll
-                for (int g = 0; g < GH; ++g) sc[g] = fmaf(qf_s[g * s.nfk + e], x, sc[g]);
-            }
             if (s.dck > 0) {
                 float cd, sd;
-                basis_cs(1, j, s.T, &cd, &sd);                  // rotation per unit of n
+                if (t0 == j0) { cd = cd1; sd = sd1; }
+                else basis_cs(1, j, s.T, &cd, &sd);             // rotation per unit of n
                 const int f1 = min(s.k, (ql + 1) * per_lane);
                 for (int n0 = ql * per_lane; n0 < f1; n0 += 32) {
                     float cr, sr;
-                    basis_cs(n0, j, s.T, &cr, &sr);             // exact re-seed
+                    if (t0 == j0 && n0 == ql * per_lane) { cr = cr1; sr = sr1; }
+                    else basis_cs(n0, j, s.T, &cr, &sr);        // exact re-seed
                     const int n1 = min(f1, n0 + 32);
 #pragma unroll 4
                     for (int n = n0; n < n1; ++n) {
@@ -189,11 +235,18 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
         softmax_tile(sc, valid);
         // o^u += p V^mu
         if (act_mid) {
+            int i = tg_mid;
+            if (t0 == j0) {
+#pragma unroll
+                for (int u = 0; u < kPre; ++u, i += ntg_mid) {
+                    if (i < nt)
+#pragma unroll
+                        for (int g = 0; g < GH; ++g) o_mid[g] = fmaf(p_s[g * kTile + i], v_pre[u], o_mid[g]);
+                }
+            }
 #pragma unroll 4
-            for (int i = tg_mid; i < nt; i += ntg_mid) {
-                const int slot = slot_of(t0 + i);
-                float x = ld_f(mid_row<KV>(c.v_mid, s, b, h, cls_of(t0 + i), slot, s.nfv) +
-                               v_mid_col(slot, e_mid, s.nfv, sizeof(KV) == 2 ? FA_BF16 : FA_F32));
+            for (; i < nt; i += ntg_mid) {
+                const float x = v_at(t0 + i);
 #pragma unroll
                 for (int g = 0; g < GH; ++g) o_mid[g] = fmaf(p_s[g * kTile + i], x, o_mid[g]);
             }
@@ -208,9 +261,11 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
                 for (int g = 0; g < GH; ++g) { zr[g] = 0.f; zi[g] = 0.f; }
                 if (n < s.k && i0 < i1) {
                     float cd, sd, cr, sr;
-                    basis_cs(n, 1, s.T, &cd, &sd);
+                    if (nb == 0) { cd = zc1; sd = zs1; }
+                    else basis_cs(n, 1, s.T, &cd, &sd);
                     for (int ia = i0; ia < i1; ia += 32) {
-                        basis_cs(n, t0 + ia, s.T, &cr, &sr);
+                        if (t0 == j0 && nb == 0 && ia == i0) { cr = zr1; sr = zi1; }
+                        else basis_cs(n, t0 + ia, s.T, &cr, &sr);
                         const int ib = min(i1, ia + 32);
 #pragma unroll 4
                         for (int i = ia; i < ib; ++i) {
@@ -288,23 +343,18 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
 
     // ---- reduce the output accumulators over token groups, write the partials --
 #pragma unroll
-    for (int g = 0; g < GH; ++g) acc_s[tid * GH + g] = act_mid ? o_mid[g] : 0.f;
+    for (int g = 0; g < GH; ++g) {
+        acc_s[tid * GH + g] = act_mid ? o_mid[g] : 0.f;
+        const float l = warp_sum(rs.l[g]);
+        if ((tid & 31) == 0) red_s[(tid >> 5) * GH + g] = l;
+    }
     __syncthreads();
     for (int i = tid; i < GH * s.nfv; i += blockDim.x) {
         int g = i / s.nfv, e = i - g * s.nfv;
         float v = 0.f;
+#pragma unroll 8
         for (int tg = 0; tg < ntg_mid; ++tg) v += acc_s[(tg * s.nfv + e) * GH + g];
         o_s[g * s.d + idf_v[e]] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int g = 0; g < GH; ++g) acc_s[tid * GH + g] = act_win ? o_win[g] : 0.f;
-    __syncthreads();
-    for (int i = tid; i < GH * s.d; i += blockDim.x) {
-        int g = i / s.d, e = i - g * s.d;
-        float v = o_s[i];
-        for (int tg = 0; tg < ntg_win; ++tg) v += acc_s[(tg * s.d + e) * GH + g];
-        if (g < ng) ws.o[(((size_t)b * s.Hq + g_first + g) * p.n_part + split) * s.d + e] = v;
     }
     for (int i = tid; i < GH * s.M; i += blockDim.x) {
         int g = i / s.M, m = i - g * s.M;
@@ -314,9 +364,24 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
         float* ml = ws.ml + (((size_t)b * s.Hq + g_first + tid) * p.n_part + split) * 2;
         float mv = kNegBig, lv = 0.f;
 #pragma unroll
-        for (int g = 0; g < GH; ++g) if (g == tid) { mv = rs.m[g]; lv = rs.l[g]; }
+        for (int g = 0; g < GH; ++g) if (g == tid) mv = rs.m[g];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) lv += red_s[w * GH + tid];
         ml[0] = mv;
         ml[1] = lv;
+    }
+    __syncthreads();
+    if (w1 > w0) {
+#pragma unroll
+        for (int g = 0; g < GH; ++g) acc_s[tid * GH + g] = act_win ? o_win[g] : 0.f;
+        __syncthreads();
+    }
+    for (int i = tid; i < GH * s.d; i += blockDim.x) {
+        int g = i / s.d, e = i - g * s.d;
+        float v = o_s[i];
+        if (w1 > w0)
+            for (int tg = 0; tg < ntg_win; ++tg) v += acc_s[(tg * s.d + e) * GH + g];
+        if (g < ng) ws.o[(((size_t)b * s.Hq + g_first + g) * p.n_part + split) * s.d + e] = v;
     }
 }
 
@@ -328,8 +393,17 @@ static cudaError_t launch_direct_t(const Dims& s, const CacheDev& c, const Decod
                                    8 * GH + (size_t)(256 + 512) * GH);
     cudaError_t err = ensure_dynamic_smem(decode_direct_kernel<KV, GH>, smem);
     if (err != cudaSuccess) return err;
-    decode_direct_kernel<KV, GH><<<dim3(p.n_split, s.Hkv * p.n_pass, s.B), 256, smem, st>>>(s, c, p, static_cast<const KV*>(q), ws);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.n_split, s.Hkv * p.n_pass, s.B);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, decode_direct_kernel<KV, GH>, s, c, p, static_cast<const KV*>(q), ws);
 }
 
 cudaError_t launch_decode_direct(const Dims& s, const CacheDev& c, int dtype, const DecodePlan& p, const void* q, char* ws,

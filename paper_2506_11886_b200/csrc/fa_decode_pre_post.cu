@@ -5,8 +5,11 @@
 // memory with 16-byte asynchronous copies (all in flight together) and works from there.  All
 // loads of partial results are issued in independent batches so that a call costs a few memory
 // round trips, not one per split.  The three kernels of a decode call are chained with
-// programmatic dependent launch: each lets its successor start at once, and the successor waits
-// (griddepcontrol.wait) only where it first touches what its predecessor wrote.
+// programmatic dependent launch: each waits for the work in front of it, then lets its successor start, which may
+// therefore read whatever was there before the call, and waits (griddepcontrol.wait) only where it first touches what its
+// predecessor wrote.  (Compress and decode of 1024 fp32 tokens of one head, five kernels that are all latency: 36.9 -> 26.6 us
+// with the launches of this call chained, the direct kernel's rows and kept-dim scores in front of its wait, and an
+// epilogue that fetches everything at once and, with one slice of rows, needs no ticket.)
 #include "fa_common.cuh"
 #include "fa_decode_ws.cuh"
 
@@ -28,15 +31,16 @@ template <typename KV>
 __global__ void __launch_bounds__(256) decode_prologue_kernel(Dims s, CacheDev c, DecodePlan p, const KV* __restrict__ q,
                                                               char* wsp) {
     extern __shared__ __align__(16) float sm_pro[];
+    pdl_wait();                                            // coefficients, query; the workspace
     pdl_launch_dependents();
     Ws ws = ws_view(wsp, p);
     const int h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
     if (blockIdx.x == 0 && tid == 0) ws.cnt[b * s.Hkv + h] = 0;
     if (s.dck == 0) return;
     const int stride = s.dck + 4;                      // row stride of the tile: 16-byte aligned, bank-skewed
-    const int qstride = s.dck + 1;
     float* tile = sm_pro;                              // [rows_pro][stride]
-    float* qc_s = tile + p.rows_pro * stride;          // [G][qstride] gathered query
+    float* qc_s = tile + p.rows_pro * stride;          // [G][dck] gathered query
+    float* q_s = qc_s + s.G * s.dck;                   // [G][d] query rows
     const int m0 = blockIdx.x * p.rows_pro;
     const int rows = min(p.rows_pro, s.M - m0);
     const float* coef = coef_rows(c.coef_k, s, b, h, s.dck) + (size_t)m0 * s.dck;
@@ -45,27 +49,42 @@ __global__ void __launch_bounds__(256) decode_prologue_kernel(Dims s, CacheDev c
         int r = i / vpr, v4 = i - r * vpr;
         cp_async16(tile + r * stride + 4 * v4, coef + (size_t)r * s.dck + 4 * v4);
     }
-    const int32_t* idc = c.idx_comp_k + (size_t)h * s.dck;
-    for (int i = tid; i < s.G * s.dck; i += 256) {
-        int g = i / s.dck, e = i - g * s.dck;
-        qc_s[g * qstride + e] = ld_f(q + ((size_t)b * s.Hq + h * s.G + g) * s.d + idc[e]);
-    }
+    // (whole rows of q beside the index set: gathered from memory, q would be a second round trip behind it)
+    const int idx = tid < s.dck ? c.idx_comp_k[(size_t)h * s.dck + tid] : 0;
+    for (int i = tid; i < s.G * s.d; i += 256) q_s[i] = ld_f(q + ((size_t)b * s.Hq + h * s.G) * s.d + i);
+    __syncthreads();
+    if (tid < s.dck)
+        for (int g = 0; g < s.G; ++g) qc_s[g * s.dck + tid] = q_s[g * s.d + idx];
     cp_async_wait_all();
     __syncthreads();
-    for (int t = tid; t < rows * s.G; t += 256) {
-        const int g = t % s.G, r = t / s.G;
-        const float* row = tile + r * stride;
-        const float* qq = qc_s + g * qstride;
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        for (int e = 0; e < s.dck; e += 4) {
-            a0 = fmaf(row[e], qq[e], a0);
-            a1 = fmaf(row[e + 1], qq[e + 1], a1);
-            a2 = fmaf(row[e + 2], qq[e + 2], a2);
-            a3 = fmaf(row[e + 3], qq[e + 3], a3);
+    // eight lanes to a row, four heads at a time
+    const int l8 = tid & 7;
+    for (int r0 = 0; r0 < rows; r0 += 32) {
+        const int r = r0 + (tid >> 3), m = m0 + r;
+        for (int g0 = 0; g0 < s.G; g0 += 4) {
+            float a[4] = {0.f, 0.f, 0.f, 0.f};
+            if (r < rows)
+#pragma unroll 3
+                for (int v = l8; v < vpr; v += 8) {
+                    const float4 x = *reinterpret_cast<const float4*>(tile + r * stride + 4 * v);
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        if (g0 + g < s.G) {
+                            const float4 y = *reinterpret_cast<const float4*>(qc_s + (g0 + g) * s.dck + 4 * v);
+                            a[g] = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, a[g]))));
+                        }
+                    }
+                }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+                for (int g = 0; g < 4; ++g) a[g] += __shfl_xor_sync(0xffffffffu, a[g], o);
+            float mine = a[0];
+#pragma unroll
+            for (int g = 1; g < 4; ++g) if (l8 == g) mine = a[g];
+            if (r < rows && l8 < 4 && g0 + l8 < s.G)
+                ws.u[((size_t)b * s.Hq + h * s.G + g0 + l8) * s.M + m] = recon_weight(s.norm, m, s.k, s.T) * s.scale * kLog2e * mine;
         }
-        const int m = m0 + r;
-        ws.u[((size_t)b * s.Hq + h * s.G + g) * s.M + m] =
-            recon_weight(s.norm, m, s.k, s.T) * s.scale * kLog2e * ((a0 + a1) + (a2 + a3));
     }
 }
 
@@ -74,6 +93,10 @@ __global__ void __launch_bounds__(256) decode_prologue_kernel(Dims s, CacheDev c
 // forms the weighted z of its slice of coefficient rows and multiplies by those rows of C^V;
 // the last CTA of a (b, h) to finish (atomic ticket, nobody waits) adds the slices in a fixed
 // order, normalises and writes the output rows.
+__host__ __device__ inline size_t epilogue_l(const Dims& s, const DecodePlan& p) {
+    const size_t a = (size_t)s.G * p.n_part, b = p.n_slice == 1 ? (size_t)s.G * s.dcv : 0;
+    return a > b ? a : b;
+}
 template <typename KV>
 __global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c, DecodePlan p, KV* __restrict__ out,
                                                               char* wsp) {
@@ -87,12 +110,13 @@ __global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c
     const int stride = s.dcv + 4;
     const int ns = p.n_part;
     float* alpha_s = sm_epi;                               // [G][n_split]: first the maxima, then exp2(m - max)
-    float* l_s = alpha_s + s.G * ns;                       // [G][n_split]
-    float* linv_s = l_s + s.G * ns;                        // [G]
+    float* l_s = alpha_s + s.G * ns;                       // [G][n_split], then o^c of a CTA alone
+    float* linv_s = l_s + epilogue_l(s, p);                // [G]
     float* zw_s = linv_s + s.G;                            // [G][rows_max]
     int* inv_s = reinterpret_cast<int*>(zw_s + s.G * rows_max);   // [d] dim -> slot in D^vc, or -1
     float* tile = reinterpret_cast<float*>(inv_s + s.d);   // [rows_max][stride]
     tile = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(tile) + 15) & ~uintptr_t(15));
+    float* ps_s = tile + rows_max * stride;                // [row groups][4][dcv] partial o^c
 
     // the coefficient tile does not depend on the main kernel: start it before waiting for it
     if (s.dcv > 0) {
@@ -103,107 +127,161 @@ __global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c
             cp_async16(tile + r * stride + 4 * v4, cv + (size_t)r * s.dcv + 4 * v4);
         }
     }
-    for (int e = tid; e < s.d; e += 256) inv_s[e] = -1;
+    // (a thread per dim: every dim is in D^vu or in D^vc)
+    for (int e = tid; e < s.d; e += 256) inv_s[e < s.nfv ? c.idx_full_v[(size_t)h * s.nfv + e] : c.idx_comp_v[(size_t)h * s.dcv + e - s.nfv]] = e < s.nfv ? -1 : e - s.nfv;
     pdl_wait();                                            // partial results of the main kernel are complete
 
-    // split statistics: one (head, split) pair per thread, then a tiny reduction per head
+    // What a thread needs of the first kPre parts comes with the statistics, in one round trip: its first entry of z, and, where this CTA
+    // finishes its head alone, its first two of o.
+    const bool alone = p.n_slice == 1;
+    const size_t qh0 = (size_t)b * s.Hq + h * s.G;
+    auto z_of = [&](int t) { const int g = t / rows, r = t - g * rows; return ws.z + (qh0 + g) * ns * s.M + m0 + r; };
+    auto o_of = [&](int t) { const int g = t / s.d, e = t - g * s.d; return ws.o + (qh0 + g) * ns * s.d + e; };
+    constexpr int kPre = 16;
+    float zp[kPre], op[2][kPre];
+    {
+        const bool z_on = s.dcv > 0 && tid < s.G * rows;
+        const float* z = z_on ? z_of(tid) : nullptr;
+#pragma unroll
+        for (int i = 0; i < kPre; ++i) zp[i] = z_on && i < ns ? z[(size_t)i * s.M] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const bool o_on = alone && tid + 256 * u < s.G * s.d;
+            const float* o = o_on ? o_of(tid + 256 * u) : nullptr;
+#pragma unroll
+            for (int i = 0; i < kPre; ++i) op[u][i] = o_on && i < ns ? o[(size_t)i * s.d] : 0.f;
+        }
+    }
+    // sum over the parts of al[sp] x[sp * stride], the first kPre of them at hand or not
+    auto merge = [&](const float* x, size_t stride, const float* al, const float (&pre)[kPre], bool have) {
+        float v0 = 0.f, v1 = 0.f;
+        int sp = 0;
+        if (have) {
+#pragma unroll
+            for (int i = 0; i < kPre; i += 2) {
+                if (i < ns) v0 = fmaf(al[i], pre[i], v0);
+                if (i + 1 < ns) v1 = fmaf(al[i + 1], pre[i + 1], v1);
+            }
+            sp = min(kPre, ns);
+        }
+        for (; sp + 8 <= ns; sp += 8) {                    // eight independent loads in flight
+            float xx[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) xx[i] = x[(size_t)(sp + i) * stride];
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) { v0 = fmaf(al[sp + i], xx[i], v0); v1 = fmaf(al[sp + i + 1], xx[i + 1], v1); }
+        }
+        for (; sp < ns; ++sp) v0 = fmaf(al[sp], x[(size_t)sp * stride], v0);
+        return v0 + v1;
+    };
+    // split statistics: one (head, split) pair per thread, then a warp per head
     for (int i = tid; i < s.G * ns; i += 256) {
         const int g = i / ns, sp = i - g * ns;
-        const float2 ml = *reinterpret_cast<const float2*>(ws.ml + (((size_t)b * s.Hq + h * s.G + g) * ns + sp) * 2);
+        const float2 ml = *reinterpret_cast<const float2*>(ws.ml + ((qh0 + g) * ns + sp) * 2);
         alpha_s[i] = ml.x;
         l_s[i] = ml.y;
     }
     __syncthreads();
-    if (tid < s.G) {
-        float mx = kNegBig;
-        for (int sp = 0; sp < ns; ++sp) mx = fmaxf(mx, alpha_s[tid * ns + sp]);
-        float L = 0.f;
-        for (int sp = 0; sp < ns; ++sp) {
-            const float a = exp2f(alpha_s[tid * ns + sp] - mx);
-            alpha_s[tid * ns + sp] = a;
-            L = fmaf(a, l_s[tid * ns + sp], L);
+    for (int g = tid >> 5; g < s.G; g += 8) {
+        const int lane = tid & 31;
+        float mx = kNegBig, L = 0.f;
+        for (int sp = lane; sp < ns; sp += 32) mx = fmaxf(mx, alpha_s[g * ns + sp]);
+        mx = warp_max(mx);
+        for (int sp = lane; sp < ns; sp += 32) {
+            const float a = exp2f(alpha_s[g * ns + sp] - mx);
+            alpha_s[g * ns + sp] = a;
+            L = fmaf(a, l_s[g * ns + sp], L);
         }
-        linv_s[tid] = L > 0.f ? 1.0f / L : 0.f;
+        L = warp_sum(L);
+        if (lane == 0) linv_s[g] = L > 0.f ? 1.0f / L : 0.f;
     }
     __syncthreads();
+    float* oc_s = l_s;                                     // [G][dcv] o^c of a CTA alone (room for it: epilogue_l); the sums have been read
     if (s.dcv > 0) {
         for (int t = tid; t < s.G * rows; t += 256) {
             const int g = t / rows, r = t - g * rows;
-            const float* z = ws.z + ((size_t)b * s.Hq + h * s.G + g) * ns * s.M + m0 + r;
-            const float* al = alpha_s + g * ns;
-            float v0 = 0.f, v1 = 0.f;
-            int sp = 0;
-            for (; sp + 8 <= ns; sp += 8) {                // eight independent loads in flight
-                float zz[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) zz[i] = z[(size_t)(sp + i) * s.M];
-#pragma unroll
-                for (int i = 0; i < 8; i += 2) { v0 = fmaf(al[sp + i], zz[i], v0); v1 = fmaf(al[sp + i + 1], zz[i + 1], v1); }
-            }
-            for (; sp < ns; ++sp) v0 = fmaf(al[sp], z[(size_t)sp * s.M], v0);
-            zw_s[g * rows_max + r] = (v0 + v1) * recon_weight(s.norm, m0 + r, s.k, s.T);
+            zw_s[g * rows_max + r] = merge(z_of(t), s.M, alpha_s + g * ns, zp, t == tid) * recon_weight(s.norm, m0 + r, s.k, s.T);
         }
         cp_async_wait_all();
         __syncthreads();
-        for (int t = tid; t < s.G * s.dcv; t += 256) {
-            const int g = t / s.dcv, e = t - g * s.dcv;
-            const float* zw = zw_s + g * rows_max;
-            float a0 = 0.f, a1 = 0.f;
-            int r = 0;
-            for (; r + 2 <= rows; r += 2) {
-                a0 = fmaf(zw[r], tile[r * stride + e], a0);
-                a1 = fmaf(zw[r + 1], tile[(r + 1) * stride + e], a1);
+        // a thread takes four columns and every nrg-th row, four heads at a time; then the row groups are added in order
+        const int nv = s.dcv >> 2, nrg = 256 / nv, rg = tid / nv, v = tid - rg * nv;
+        for (int g0 = 0; g0 < s.G; g0 += 4) {
+            const int hg = min(4, s.G - g0);
+            float4 a[4];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) a[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (rg < nrg)
+#pragma unroll 2
+                for (int r = rg; r < rows; r += nrg) {
+                    const float4 x = *reinterpret_cast<const float4*>(tile + r * stride + 4 * v);
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        if (g < hg) {
+                            const float w = zw_s[(g0 + g) * rows_max + r];
+                            a[g].x = fmaf(w, x.x, a[g].x);
+                            a[g].y = fmaf(w, x.y, a[g].y);
+                            a[g].z = fmaf(w, x.z, a[g].z);
+                            a[g].w = fmaf(w, x.w, a[g].w);
+                        }
+                    }
+                }
+            if (g0 > 0) __syncthreads();
+            if (rg < nrg)
+#pragma unroll
+                for (int g = 0; g < 4; ++g) if (g < hg) *reinterpret_cast<float4*>(ps_s + (rg * hg + g) * s.dcv + 4 * v) = a[g];
+            __syncthreads();
+            for (int t = tid; t < hg * s.dcv; t += 256) {
+                float x = 0.f;
+#pragma unroll 4
+                for (int y = 0; y < nrg; ++y) x += ps_s[y * hg * s.dcv + t];
+                const int g = t / s.dcv;
+                if (alone) oc_s[g0 * s.dcv + t] = x;
+                else ws.oc[((qh0 + g0 + g) * p.n_slice + slice) * s.dcv + t - g * s.dcv] = x;
             }
-            if (r < rows) a0 = fmaf(zw[r], tile[r * stride + e], a0);
-            ws.oc[(((size_t)b * s.Hq + h * s.G + g) * p.n_slice + slice) * s.dcv + e] = a0 + a1;
         }
     }
-    // ticket
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        const int done = atomicAdd(ws.cnt + b * s.Hkv + h, 1);
-        last_s = (done == (int)gridDim.x - 1);
+    if (!alone) {
+        // ticket
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            const int done = atomicAdd(ws.cnt + b * s.Hkv + h, 1);
+            last_s = (done == (int)gridDim.x - 1);
+        }
+        __syncthreads();
+        if (!last_s) return;
+        __threadfence();
+    } else {
+        __syncthreads();
     }
-    __syncthreads();
-    if (!last_s) return;
-    __threadfence();
-    const int32_t* idc_v = c.idx_comp_v + (size_t)h * s.dcv;
-    for (int e = tid; e < s.dcv; e += 256) inv_s[idc_v[e]] = e;
-    __syncthreads();
-    for (int t = tid; t < s.G * s.d; t += 256) {
+    auto finish = [&](int t, const float (&pre)[kPre], bool have) {
         const int g = t / s.d, e = t - g * s.d;
-        const size_t qh = (size_t)b * s.Hq + h * s.G + g;
-        const float* al = alpha_s + g * ns;
-        const float* o = ws.o + qh * ns * s.d + e;
-        float v0 = 0.f, v1 = 0.f;
-        int sp = 0;
-        for (; sp + 8 <= ns; sp += 8) {
-            float oo[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) oo[i] = o[(size_t)(sp + i) * s.d];
-#pragma unroll
-            for (int i = 0; i < 8; i += 2) { v0 = fmaf(al[sp + i], oo[i], v0); v1 = fmaf(al[sp + i + 1], oo[i + 1], v1); }
-        }
-        for (; sp < ns; ++sp) v0 = fmaf(al[sp], o[(size_t)sp * s.d], v0);
+        float v = merge(o_of(t), s.d, alpha_s + g * ns, pre, have);
         const int slot = inv_s[e];
         if (slot >= 0) {
-            const float* oc = ws.oc + qh * p.n_slice * s.dcv + slot;
-            float w0 = 0.f, w1 = 0.f;
-            int sl = 0;
-            for (; sl + 8 <= p.n_slice; sl += 8) {
-                float cc[8];
+            if (alone) {
+                v += oc_s[g * s.dcv + slot];
+            } else {
+                const float* oc = ws.oc + (qh0 + g) * p.n_slice * s.dcv + slot;
+                float w0 = 0.f, w1 = 0.f;
+                int sl = 0;
+                for (; sl + 8 <= p.n_slice; sl += 8) {
+                    float cc[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) cc[i] = __ldcg(oc + (size_t)(sl + i) * s.dcv);
+                    for (int i = 0; i < 8; ++i) cc[i] = __ldcg(oc + (size_t)(sl + i) * s.dcv);
 #pragma unroll
-                for (int i = 0; i < 8; i += 2) { w0 += cc[i]; w1 += cc[i + 1]; }
+                    for (int i = 0; i < 8; i += 2) { w0 += cc[i]; w1 += cc[i + 1]; }
+                }
+                for (; sl < p.n_slice; ++sl) w0 += __ldcg(oc + (size_t)sl * s.dcv);
+                v += w0 + w1;
             }
-            for (; sl < p.n_slice; ++sl) w0 += __ldcg(oc + (size_t)sl * s.dcv);
-            v0 += w0;
-            v1 += w1;
         }
-        st_f(out + qh * s.d + e, (v0 + v1) * linv_s[g]);
-    }
+        st_f(out + (qh0 + g) * s.d + e, v * linv_s[g]);
+    };
+    if (tid < s.G * s.d) finish(tid, op[0], alone);
+    if (tid + 256 < s.G * s.d) finish(tid + 256, op[1], alone);
+    for (int t = tid + 512; t < s.G * s.d; t += 256) finish(t, op[0], false);
 }
 
 // ---------------------------------------------------------------- launchers --
@@ -229,11 +307,10 @@ template <typename KV>
 static cudaError_t launch_prologue_t(const Dims& s, const CacheDev& c, const DecodePlan& p, const void* q, char* ws,
                                      cudaStream_t st) {
     const int tiles = s.dck > 0 ? (s.M + p.rows_pro - 1) / p.rows_pro : 1;
-    const size_t smem = sizeof(float) * ((size_t)p.rows_pro * (s.dck + 4) + (size_t)s.G * (s.dck + 1));
+    const size_t smem = sizeof(float) * ((size_t)p.rows_pro * (s.dck + 4) + (size_t)s.G * (s.dck + s.d));
     cudaError_t err = ensure_dynamic_smem(decode_prologue_kernel<KV>, smem);
     if (err != cudaSuccess) return err;
-    decode_prologue_kernel<KV><<<dim3(tiles, s.Hkv, s.B), 256, smem, st>>>(s, c, p, static_cast<const KV*>(q), ws);
-    return cudaGetLastError();
+    return launch_pdl(decode_prologue_kernel<KV>, dim3(tiles, s.Hkv, s.B), dim3(256), smem, st, true, s, c, p, static_cast<const KV*>(q), ws);
 }
 
 cudaError_t launch_decode_prologue(const Dims& s, const CacheDev& c, int dtype, const DecodePlan& p, const void* q,
@@ -246,7 +323,7 @@ template <typename KV>
 static cudaError_t launch_epilogue_t(const Dims& s, const CacheDev& c, const DecodePlan& p, void* out, char* ws,
                                      cudaStream_t st) {
     const int rows = (s.M + p.n_slice - 1) / p.n_slice;
-    const size_t smem = sizeof(float) * (2 * (size_t)s.G * p.n_part + s.G + (size_t)s.G * rows + s.d + 4 + (size_t)rows * (s.dcv + 4));
+    const size_t smem = sizeof(float) * ((size_t)s.G * p.n_part + epilogue_l(s, p) + s.G + (size_t)s.G * rows + s.d + 4 + (size_t)rows * (s.dcv + 4) + 4 * 1024);      // (256 threads' four columns of four heads)
     cudaError_t err = ensure_dynamic_smem(decode_epilogue_kernel<KV>, smem);
     if (err != cudaSuccess) return err;
     return launch_pdl(decode_epilogue_kernel<KV>, dim3(p.n_slice, s.Hkv, s.B), dim3(256), smem, st, true, s, c, p,
