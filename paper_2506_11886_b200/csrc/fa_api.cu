@@ -308,7 +308,9 @@ static fa_status make_plan(const fa_layout& l, CallPlan* p) {
     if (p->algo == FA_DECODE_FFT && l.decode_algo == FA_DECODE_AUTO && channels_pay(s) &&
         plan_channels(s, log2S, kNumSms, &p->chan)) {
         // the channel form has its areas behind the barrier counters
-        p->chan.total = place_channels(s, log2S, align_up(sizeof(int32_t) * 4 * (size_t)kBarSlots, 256), &p->chan);
+        p->chan.base = align_up(sizeof(int32_t) * 4 * (size_t)kBarSlots, 256);
+        p->chan.per_layer = place_channels(s, log2S, &p->chan);
+        p->chan.total = p->chan.base + p->chan.per_layer;
         p->chan.on = 1;
     }
     return FA_OK;
@@ -387,13 +389,18 @@ static size_t compress_scratch_bytes(const fa_layout& l) {
     if (rows > (size_t)kMomLayers * s.B) rows = (size_t)kMomLayers * s.B;
     return rows * row;
 }
+// Areas of the layers behind the first that share the launches of the channel form, behind the moments' room (so that a workspace of a smaller size
+// serves what it served; with the compression's layers, what is there counts).
+static size_t chan_layers_at(const fa_layout& l, size_t decode) { return align_up(decode_room_bytes(l, decode) + compress_scratch_bytes(l), 256); }
+static size_t chan_layers_bytes(const CallPlan& p) { return p.chan.on && p.chan.n_pass == 1 ? (kChanLayers - 1) * p.chan.per_layer : 0; }
 // Where the moments of a call go and how many bytes there are (0: the direct contraction).
 struct MomentRoom { char* at; size_t bytes; };
 static MomentRoom moment_room(const fa_layout& l, void* ws, size_t ws_bytes) {
     size_t decode = 0;
     if (!ws || !aligned16(ws) || !compress_mom_supported(make_dims(l)) || decode_scratch_bytes(&l, &decode) != FA_OK) return {nullptr, 0};
     decode = decode_room_bytes(l, decode);
-    return ws_bytes > decode ? MomentRoom{static_cast<char*>(ws) + decode, ws_bytes - decode} : MomentRoom{nullptr, 0};
+    const size_t most = compress_scratch_bytes(l), left = ws_bytes > decode ? ws_bytes - decode : 0;
+    return left ? MomentRoom{static_cast<char*>(ws) + decode, left < most ? left : most} : MomentRoom{nullptr, 0};
 }
 // The two kernels of the block-moment path over all batch rows: all at once, or in groups that take half of the room in turn
 // (one row at least fits).
@@ -443,7 +450,12 @@ fa_status fa_cache_sizes_of(const fa_layout* layout, fa_cache_sizes* out) {
 fa_status fa_workspace_bytes(const fa_layout* layout, size_t* out) {
     fa_status st = decode_scratch_bytes(layout, out);
     if (st != FA_OK) return st;
-    *out = decode_room_bytes(*layout, *out) + compress_scratch_bytes(*layout);
+    const size_t decode = *out;
+    CallPlan p;
+    st = plan_decode(*layout, &p);
+    if (st != FA_OK) return st;
+    const size_t more = chan_layers_bytes(p);
+    *out = more ? chan_layers_at(*layout, decode) + more : decode_room_bytes(*layout, decode) + compress_scratch_bytes(*layout);
     return FA_OK;
 }
 
@@ -817,7 +829,8 @@ fa_status fa_decode_attention(const fa_layout* layout, const fa_cache* cache, co
     char* w = static_cast<char*>(ws);
     if (p.chan.on && ws_bytes >= p.chan.total) {
         bool begun = false;
-        if (launch_decode_channels(s, c, p.chan, p.fft_log2, q, out, nullptr, nullptr, w, cs, &begun) == cudaSuccess) return FA_OK;
+        const ChanArgs a = {c, q, nullptr, nullptr, out, w + p.chan.base};
+        if (launch_decode_channels(s, &a, 1, p.chan, p.fft_log2, cs, &begun) == cudaSuccess) return FA_OK;
         if (begun) return FA_ERR_CUDA;
         cudaGetLastError();                                  // refused before anything ran: the transform kernel
     }
@@ -876,8 +889,8 @@ static fa_status decode_step_impl(const fa_layout* layout, fa_cache* cache, cons
     const bool channels = p.chan.on && ws_bytes >= p.chan.total;
     if (channels && p.chan.n_pass == 1) {
         bool begun = false;
-        if (launch_decode_channels(s, make_cache(*cache), p.chan, p.fft_log2, q, out, k_new, v_new, static_cast<char*>(ws), static_cast<cudaStream_t>(stream), &begun) == cudaSuccess)
-            return FA_OK;
+        const ChanArgs a = {make_cache(*cache), q, k_new, v_new, out, static_cast<char*>(ws) + p.chan.base};
+        if (launch_decode_channels(s, &a, 1, p.chan, p.fft_log2, static_cast<cudaStream_t>(stream), &begun) == cudaSuccess) return FA_OK;
         if (begun) return FA_ERR_CUDA;
         cudaGetLastError();                                  // refused before anything ran
     }
@@ -891,6 +904,60 @@ static fa_status decode_step_impl(const fa_layout* layout, fa_cache* cache, cons
     st = fa_append(layout, cache, k_new, v_new, stream);
     if (st != FA_OK) return st;
     return fa_decode_attention(layout, cache, q, out, ws, ws_bytes, stream);
+}
+
+// Whether two layers of a step may run side by side: neither writes what the other reads or writes.
+static bool layers_apart(const fa_layout& l, const fa_cache_sizes& z, const fa_cache& a, const void* const (&in_a)[3], const void* out_a, const fa_cache& b,
+                         const void* const (&in_b)[3], const void* out_b) {
+    const size_t eb = elt_bytes(l.kv_dtype), qb = (size_t)l.batch * l.n_q_heads * l.head_dim * eb, kb = (size_t)l.batch * l.n_kv_heads * l.head_dim * eb;
+    struct Range { const void* p; size_t n; };
+    constexpr int kWritten = 10, kAll = 13;
+    auto ranges = [&](const fa_cache& c, const void* const (&in)[3], const void* out, Range (&r)[kAll]) {
+        const Range x[kAll] = {{out, qb},           {c.k_init, z.k_init}, {c.v_init, z.v_init}, {c.k_local, z.k_local}, {c.v_local, z.v_local}, {c.k_mid, z.k_mid}, {c.v_mid, z.v_mid},
+                               {c.coef_k, z.coef_k}, {c.coef_v, z.coef_v}, {c.state, z.state}, {in[0], qb},               {in[1], kb},               {in[2], kb}};
+        for (int i = 0; i < kAll; ++i) r[i] = x[i];
+    };
+    Range x[kAll], y[kAll];
+    ranges(a, in_a, out_a, x);
+    ranges(b, in_b, out_b, y);
+    for (int i = 0; i < kAll; ++i)
+        for (int j = 0; j < kAll; ++j)
+            if ((i < kWritten || j < kWritten) && x[i].n && y[j].n) {
+                const char *p = static_cast<const char*>(x[i].p), *q = static_cast<const char*>(y[j].p);
+                if (p < q + y[j].n && q < p + x[i].n) return false;
+            }
+    return true;
+}
+
+// The first layers of a step over several, in the channel form and side by side: how many (0: none, the caller goes on one by one; -1: an
+// error after the first launch).  Layers of one layout, as many as the workspace has areas for; the same plan as for one, so the same bits.
+static int step_channel_layers(int n_layers, const fa_layout* layouts, fa_cache* caches, const void* const* q, const void* const* k_new, const void* const* v_new,
+                               void* const* out, char* ws, size_t ws_bytes, cudaStream_t stream) {
+    CallPlan p;
+    if (n_layers < 2 || plan_decode(layouts[0], &p) != FA_OK || !p.chan.on || p.chan.n_pass != 1) return 0;
+    size_t decode = 0;
+    fa_cache_sizes z;
+    if (decode_scratch_bytes(&layouts[0], &decode) != FA_OK || fa_cache_sizes_of(&layouts[0], &z) != FA_OK) return 0;
+    const size_t at = chan_layers_at(layouts[0], decode);
+    ChanArgs a[kChanLayers];
+    int n = 0;
+    for (; n < n_layers && n < kChanLayers; ++n) {
+        if (n > 0 && (std::memcmp(&layouts[n], &layouts[0], sizeof(fa_layout)) != 0 || ws_bytes < at + n * p.chan.per_layer)) break;
+        const void* const in_n[3] = {q[n], k_new[n], v_new[n]};
+        bool apart = true;
+        for (int i = 0; i < n && apart; ++i) {
+            const void* const in_i[3] = {q[i], k_new[i], v_new[i]};
+            apart = layers_apart(layouts[0], z, caches[i], in_i, out[i], caches[n], in_n, out[n]);
+        }
+        if (!apart) break;
+        a[n] = ChanArgs{make_cache(caches[n]), q[n], k_new[n], v_new[n], out[n], n == 0 ? ws + p.chan.base : ws + at + (n - 1) * p.chan.per_layer};
+    }
+    if (n < 2) return 0;
+    bool begun = false;
+    if (launch_decode_channels(make_dims(layouts[0]), a, n, p.chan, p.fft_log2, stream, &begun) == cudaSuccess) return n;
+    if (begun) return -1;
+    cudaGetLastError();                                      // refused before anything ran
+    return 0;
 }
 
 extern "C" {
@@ -917,7 +984,11 @@ fa_status fa_decode_step_layers(int32_t n_layers, const fa_layout* layouts, fa_c
         if (st != FA_OK) return st;
         if (!ws || !aligned16(ws) || ws_bytes < p.total) return FA_ERR_WORKSPACE;
     }
-    for (int i = 0; i < n_layers; ++i) {
+    for (int i = 0, n = 1; i < n_layers; i += n) {
+        n = step_channel_layers(n_layers - i, layouts + i, caches + i, q + i, k_new + i, v_new + i, out + i, static_cast<char*>(ws), ws_bytes, static_cast<cudaStream_t>(stream));
+        if (n < 0) return FA_ERR_CUDA;
+        if (n > 0) continue;
+        n = 1;
         const fa_status st = decode_step_impl(&layouts[i], &caches[i], q[i], k_new[i], v_new[i], out[i], ws, ws_bytes, stream);
         if (st != FA_OK) return st;
     }

@@ -69,7 +69,16 @@ struct ChanPlan {
     int n_cx, n_wpart;       // CTAs per (KV head, pass): class parts of all batch rows, window parts of one
     int nq, nz;              // channel pairs per CTA of the kernels in front and behind, and CTAs of their clusters
     int st_in, st_out;       // stages of their streams of coefficient rows
-    size_t off_z, off_w, off_mw, off_ml, off_o, off_g, off_x, off_j, off_p, total;
+    size_t off_z, off_w, off_mw, off_ml, off_o, off_g, off_x, off_j, off_p;      // from the start of a layer's areas
+    size_t base, per_layer, total;       // one layer's areas in the workspace: their start, size and end
+};
+constexpr int kChanLayers = 4;           // layers that share the launches of the channel form
+// A layer of a launch of the channel form; ws: its areas.
+struct ChanArgs {
+    CacheDev c;
+    const void *q, *k_new, *v_new;
+    void* out;
+    char* ws;
 };
 
 // Plan of one fa_decode_attention call; a pure function of the layout so that
@@ -181,9 +190,8 @@ cudaError_t launch_decode_fft(const Dims&, const CacheDev&, int dtype, const Dec
                               const void* k_new, const void* v_new, cudaStream_t);
 // The channel form (fa_decode_chan.cu): its plan, its areas of the workspace, its launches (k_new / v_new: behind a push).
 bool plan_channels(const Dims&, int log2S, int sms, ChanPlan*);
-size_t place_channels(const Dims&, int log2S, size_t off, ChanPlan*);
-cudaError_t launch_decode_channels(const Dims&, const CacheDev&, const ChanPlan&, int log2S, const void* q, void* out, const void* k_new, const void* v_new, char* ws,
-                                   cudaStream_t, bool* begun);
+size_t place_channels(const Dims&, int log2S, ChanPlan*);
+cudaError_t launch_decode_channels(const Dims&, const ChanArgs* layers, int n, const ChanPlan&, int log2S, cudaStream_t, bool* begun);
 size_t decode_fft_smem_bytes(const Dims&, int log2S, int gh, int nb, int occ = 1, int split = 0);
 bool decode_fft_fused_fits(const Dims&, int log2S, int gh, int nb, int n_part, int occ = 1, int split = 0);
 bool decode_fft_launchable(const Dims&, const DecodePlan&);
