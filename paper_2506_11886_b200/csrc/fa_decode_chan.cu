@@ -207,15 +207,34 @@ __device__ __forceinline__ RowParts row_parts(const int32_t* state, const Dims& 
     return r;
 }
 
+// The layers of a call (each a fa_decode_step or fa_decode_attention of its own; k_new null: the latter).  Layers of one layout that do not touch
+// one another's memory share the three launches: the kernels in front and behind are chains of short phases, which CTAs at different places in theirs fill
+// for one another, and a launch's start and end are paid once.
+struct ChanLayer {
+    CacheDev c;
+    const bf16 *q, *k_new, *v_new;
+    bf16* out;
+    char* ws;
+};
+struct ChanCall {
+    int n;
+    ChanLayer l[kChanLayers];
+};
+struct LayerMaps { CUtensorMap km, vm, ki, vi, kl, vl; };
+struct ChanMaps { LayerMaps l[kChanLayers]; };
+
 // Cluster per job, 256 threads.  u = scale log2(e) W C^K q, a slice of the rows per CTA, exchanged through distributed shared
 // memory; then Z of nq channel pairs per CTA (a transform carries channels 2 q and 2 q + 1 of one head).  With k_new (a step, one
 // pass) also the push: C^K's rows are updated on their way, the leaving row's kept dims and the new token are written.
 template <int LS>
-__global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, CacheDev c, ChanPlan mp, const bf16* __restrict__ q, const bf16* __restrict__ k_new,
-                                                               const bf16* __restrict__ v_new, char* wsp) {
+__global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
     constexpr int S = 1 << LS;
     extern __shared__ __align__(16) float smz[];
-    const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass, b = blockIdx.z;
+    const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass;
+    const int layer = blockIdx.z / s.B, b = blockIdx.z - layer * s.B;
+    const CacheDev& c = call.l[layer].c;
+    const bf16 *q = call.l[layer].q, *k_new = call.l[layer].k_new, *v_new = call.l[layer].v_new;
+    char* wsp = call.l[layer].ws;
     const int g_first = h * s.G + pass * mp.nh, ng = min(mp.nh, s.G - pass * mp.nh), nh = mp.nh, nq = mp.nq, q0 = rank * nq;
     constexpr int fb = pf_size(S * 2);
     const int m0 = 2 * ((rank * s.k) / CL), m1 = 2 * (((rank + 1) * s.k) / CL), nv = s.dck >> 2;
@@ -449,16 +468,21 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, CacheD
 // each for four heads, all four slots in one for two).  The maximum is only worked out when some score is above the running one.
 // Window parts: a stage holds 16 rows of K or V.
 template <int HP>
-__global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(const __grid_constant__ CUtensorMap tm_km, const __grid_constant__ CUtensorMap tm_vm,
-                                                                       const __grid_constant__ CUtensorMap tm_ki, const __grid_constant__ CUtensorMap tm_vi,
-                                                                       const __grid_constant__ CUtensorMap tm_kl, const __grid_constant__ CUtensorMap tm_vl,
-                                                                       Dims s, CacheDev c, ChanPlan mp, const bf16* __restrict__ q, char* wsp) {
+__global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(const __grid_constant__ ChanMaps maps, Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
     extern __shared__ __align__(128) unsigned char smem_unaligned[];
     unsigned char* smem = smem_unaligned + ((1024u - (smem_addr(smem_unaligned) & 1023u)) & 1023u);
     constexpr int NT = HP / 2, SL = 8 / HP;                // products per 16 classes, slots of a product
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
     const int h = blockIdx.x / mp.n_pass, pass = blockIdx.x - h * mp.n_pass;
-    const bool is_win = (int)blockIdx.y >= mp.n_cx;
+    // part `part` of layer `layer`: the class parts of all layers, then their window parts
+    const int n_win_y = s.B * mp.n_wpart, n_class_y = call.n * mp.n_cx;
+    const bool is_win = (int)blockIdx.y >= n_class_y;
+    const int layer = is_win ? ((int)blockIdx.y - n_class_y) / n_win_y : (int)blockIdx.y / mp.n_cx;
+    const int part = is_win ? mp.n_cx + (int)blockIdx.y - n_class_y - layer * n_win_y : (int)blockIdx.y - layer * mp.n_cx;
+    const CacheDev& c = call.l[layer].c;
+    const LayerMaps& tm_l = maps.l[layer];
+    const bf16* q = call.l[layer].q;
+    char* wsp = call.l[layer].ws;
     const int g_first = h * s.G + pass * mp.nh, ng = min(mp.nh, s.G - pass * mp.nh);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem) + 8 * warp;           // this warp's stages (at most 8)
     volatile int* fail = reinterpret_cast<volatile int*>(smem + 256);
@@ -500,11 +524,11 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
     // batch row and share: class parts by the rows' lengths, window parts alike
     int b = 0, x0 = 0, cnt = mp.n_cx;
     if (is_win) {
-        b = ((int)blockIdx.y - mp.n_cx) / mp.n_wpart;
+        b = (part - mp.n_cx) / mp.n_wpart;
     } else {
-        const RowParts r = row_parts(c.state, s, mp.n_cx, (int)blockIdx.y, 0);
+        const RowParts r = row_parts(c.state, s, mp.n_cx, part, 0);
         if (r.b == s.B) return;
-        if ((int)blockIdx.y == r.x0 && blockIdx.x == 0 && tid == 0) reinterpret_cast<int2*>(wsp + mp.off_p)[r.b] = make_int2(r.x0, r.cnt);      // for the last kernel
+        if (part == r.x0 && blockIdx.x == 0 && tid == 0) reinterpret_cast<int2*>(wsp + mp.off_p)[r.b] = make_int2(r.x0, r.cnt);      // for the last kernel
         b = r.b;
         x0 = r.x0;
         cnt = r.cnt;
@@ -514,9 +538,9 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
     const int n_mid = min(c.state[kStateStride * b + 2], s.max_mid), head = c.state[kStateStride * b + 3];
     const int nhalf = (s.d + 63) >> 6, rowb_k = 2 * s.nfk, rowb_v = 2 * s.nfv, n_ch = s.P >> 4;
     // class parts: supersteps [st0, st1), n_ch stages each; window parts: tokens [w0, w1) in runs of at most 16 rows
-    const int steps = (n_mid + 4 * s.P - 1) / (4 * s.P), wq = kMainWarps * ((int)blockIdx.y - x0) + warp;
+    const int steps = (n_mid + 4 * s.P - 1) / (4 * s.P), wq = kMainWarps * (part - x0) + warp;
     const int st0 = is_win ? 0 : (int)((long long)wq * steps / (kMainWarps * cnt)), st1 = is_win ? 0 : (int)((long long)(wq + 1) * steps / (kMainWarps * cnt));
-    const int n_win = n_init + n_local, wi = kMainWarps * ((int)blockIdx.y - mp.n_cx - b * mp.n_wpart) + warp;
+    const int n_win = n_init + n_local, wi = kMainWarps * (part - mp.n_cx - b * mp.n_wpart) + warp;
     const int w0 = is_win ? (int)((long long)wi * n_win / (kMainWarps * mp.n_wpart)) : 0, w1 = is_win ? (int)((long long)(wi + 1) * n_win / (kMainWarps * mp.n_wpart)) : 0;
     // place of the next stage to load: superstep and chunk of 16 classes, or window token
     int ld_step = is_win ? w0 : st0, ld_ch = 0, ld_v = 0, ld_st = 0, issued = 0;
@@ -537,13 +561,13 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
             if (bytes)
                 asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-                             "l"(reinterpret_cast<uint64_t>(ld_v ? &tm_vm : &tm_km)), "r"(0), "r"(ld_ch * 16), "r"(4 * ld_step), "r"(b * s.Hkv + h), "r"(bar) : "memory");
+                             "l"(reinterpret_cast<uint64_t>(ld_v ? &tm_l.vm : &tm_l.km)), "r"(0), "r"(ld_ch * 16), "r"(4 * ld_step), "r"(b * s.Hkv + h), "r"(bar) : "memory");
             if (ld_v && ++ld_ch == n_ch) { ld_ch = 0; ++ld_step; }
         } else {
             if (ld_step >= w1) return;
             int buf, row;
             const int n = win_run(ld_step, buf, row);
-            const CUtensorMap* tm = ld_v ? (buf == 0 ? &tm_vi : &tm_vl) : (buf == 0 ? &tm_ki : &tm_kl);
+            const CUtensorMap* tm = ld_v ? (buf == 0 ? &tm_l.vi : &tm_l.vl) : (buf == 0 ? &tm_l.ki : &tm_l.kl);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(nhalf * 2048) : "memory");
             for (int hf = 0; hf < nhalf; ++hf)
                 asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
@@ -888,7 +912,7 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
     if (!is_win)
         for (int e = tid; e < s.nfv; e += 32 * kMainWarps) inv[c.idx_full_v[h * s.nfv + e]] = (int16_t)e;
     __syncthreads();
-    const size_t slot = (size_t)blockIdx.x * gridDim.y + blockIdx.y;
+    const size_t slot = (size_t)blockIdx.x * (mp.n_cx + n_win_y) + part;
     float2* mlg = reinterpret_cast<float2*>(wsp + mp.off_ml) + slot * 4;
     float* og = reinterpret_cast<float*>(wsp + mp.off_o) + slot * 4 * s.d;
     for (int i = tid; i < 4 * s.d; i += 32 * kMainWarps) {
@@ -915,11 +939,15 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
 // After a step's push (step != 0) C^V's rows are updated on their way.
 // (128 registers at most: the plan counts on two CTAs to an SM, and the instances of 64 and 512 slots took 155, 9 to 11 % of a step)
 template <int LS>
-__global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, CacheDev c, ChanPlan mp, bf16* __restrict__ out, char* wsp, int step) {
+__global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
     constexpr int S = 1 << LS;
     extern __shared__ __align__(16) float smz[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass, b = blockIdx.z;
+    const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass;
+    const int layer = blockIdx.z / s.B, b = blockIdx.z - layer * s.B, step = call.l[layer].k_new != nullptr;
+    const CacheDev& c = call.l[layer].c;
+    bf16* out = call.l[layer].out;
+    char* wsp = call.l[layer].ws;
     const int g_first = h * s.G + pass * mp.nh, ng = min(mp.nh, s.G - pass * mp.nh), nh = mp.nh, nq = mp.nq, q0 = rank * nq;
     constexpr int fb = pf_size(S * 2);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smz);     // [8]
@@ -1271,8 +1299,9 @@ bool plan_channels(const Dims& s, int log2S, int sms, ChanPlan* m) {
     return true;
 }
 
-// Offsets of the channel form's areas, from `off` on; returns the end.
-size_t place_channels(const Dims& s, int log2S, size_t off, ChanPlan* m) {
+// Offsets of the channel form's areas of one layer, and their bytes.
+size_t place_channels(const Dims& s, int log2S, ChanPlan* m) {
+    size_t off = 0;
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t jobs = (size_t)s.B * s.Hkv * m->n_pass, slots = (size_t)1 << log2S, parts = (size_t)s.Hkv * m->n_pass * (m->n_cx + s.B * m->n_wpart);
     m->off_z = off;  off = up(off + jobs * slots * (kMR / 2) * m->hp * 8);
@@ -1288,38 +1317,43 @@ size_t place_channels(const Dims& s, int log2S, size_t off, ChanPlan* m) {
 }
 
 template <int LS>
-static cudaError_t launch_channels_t(const Dims& s, const CacheDev& c, const ChanPlan& m, const void* q, void* out, const void* k_new, const void* v_new,
-                                     char* ws, cudaStream_t st, bool* begun) {
+static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, const ChanPlan& m, cudaStream_t st, bool* begun) {
     *begun = false;
-    const dim3 cg(m.nz, s.Hkv * m.n_pass, s.B), mg(s.Hkv * m.n_pass, m.n_cx + s.B * m.n_wpart);
-    CUtensorMap km, vm, ki, vi, kl, vl;
-    const int n_bh = s.B * s.Hkv, step = k_new != nullptr;
-    const bool ok_i = window_map(&ki, c.k_init, s.l_init, s.d, n_bh, 16) & window_map(&vi, c.v_init, s.l_init, s.d, n_bh, 16);
-    const bool ok_l = window_map(&kl, c.k_local, s.l_local, s.d, n_bh, 16) & window_map(&vl, c.v_local, s.l_local, s.d, n_bh, 16);
-    if ((s.l_init > 0 && !ok_i) || (s.l_local > 0 && !ok_l)) return cudaErrorInvalidValue;
-    if (!mid_map(&km, c.k_mid, s, s.nfk) || !mid_map(&vm, c.v_mid, s, s.nfv)) return cudaErrorInvalidValue;
-    const bf16* qb = static_cast<const bf16*>(q);
-    cudaError_t err = launch_chained(chan_in_kernel<LS>, cg, dim3(kChanThreads), in_smem(s, LS, m), m.nz, st, s, c, m, qb, static_cast<const bf16*>(k_new),
-                                     static_cast<const bf16*>(v_new), ws);
+    if (n < 1 || n > kChanLayers) return cudaErrorInvalidValue;
+    const dim3 cg(m.nz, s.Hkv * m.n_pass, s.B * n), mg(s.Hkv * m.n_pass, n * (m.n_cx + s.B * m.n_wpart));
+    ChanCall call = {};
+    ChanMaps maps;
+    call.n = n;
+    const int n_bh = s.B * s.Hkv;
+    for (int i = 0; i < n; ++i) {
+        const CacheDev& c = a[i].c;
+        call.l[i] = ChanLayer{c, static_cast<const bf16*>(a[i].q), static_cast<const bf16*>(a[i].k_new), static_cast<const bf16*>(a[i].v_new), static_cast<bf16*>(a[i].out), a[i].ws};
+        LayerMaps& t = maps.l[i];
+        const bool ok_i = window_map(&t.ki, c.k_init, s.l_init, s.d, n_bh, 16) & window_map(&t.vi, c.v_init, s.l_init, s.d, n_bh, 16);
+        const bool ok_l = window_map(&t.kl, c.k_local, s.l_local, s.d, n_bh, 16) & window_map(&t.vl, c.v_local, s.l_local, s.d, n_bh, 16);
+        if ((s.l_init > 0 && !ok_i) || (s.l_local > 0 && !ok_l)) return cudaErrorInvalidValue;
+        if (!mid_map(&t.km, c.k_mid, s, s.nfk) || !mid_map(&t.vm, c.v_mid, s, s.nfv)) return cudaErrorInvalidValue;
+    }
+    cudaError_t err = launch_chained(chan_in_kernel<LS>, cg, dim3(kChanThreads), in_smem(s, LS, m), m.nz, st, s, m, call);
     if (err != cudaSuccess) return err;
     *begun = true;
-    err = m.hp == 2 ? launch_chained(chan_main_kernel<2>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, km, vm, ki, vi, kl, vl, s, c, m, qb, ws)
-                    : launch_chained(chan_main_kernel<4>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, km, vm, ki, vi, kl, vl, s, c, m, qb, ws);
+    err = m.hp == 2 ? launch_chained(chan_main_kernel<2>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, maps, s, m, call)
+                    : launch_chained(chan_main_kernel<4>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, maps, s, m, call);
     if (err != cudaSuccess) return err;
-    return launch_chained(chan_out_kernel<LS>, cg, dim3(kChanThreads), out_smem(s, LS, m), m.nz, st, s, c, m, static_cast<bf16*>(out), ws, step);
+    return launch_chained(chan_out_kernel<LS>, cg, dim3(kChanThreads), out_smem(s, LS, m), m.nz, st, s, m, call);
 }
 
-// The decode call, with k_new / v_new (not null; one pass only) behind the push of Eq.5.  *begun: an error came after the
-// first launch (before it nothing has been enqueued: the device refused the cluster, say).
-cudaError_t launch_decode_channels(const Dims& s, const CacheDev& c, const ChanPlan& m, int log2S, const void* q, void* out, const void* k_new, const void* v_new,
-                                   char* ws, cudaStream_t st, bool* begun) {
+// The decode calls of n layers of one layout, with k_new / v_new (not null; one pass only) each behind the push of Eq.5.  Several layers do not touch
+// one another's memory.  *begun: an error came after the first launch (before it nothing has been enqueued: the device refused the
+// cluster, say).
+cudaError_t launch_decode_channels(const Dims& s, const ChanArgs* a, int n, const ChanPlan& m, int log2S, cudaStream_t st, bool* begun) {
     switch (log2S) {
-        case 5: return launch_channels_t<5>(s, c, m, q, out, k_new, v_new, ws, st, begun);
-        case 6: return launch_channels_t<6>(s, c, m, q, out, k_new, v_new, ws, st, begun);
-        case 7: return launch_channels_t<7>(s, c, m, q, out, k_new, v_new, ws, st, begun);
-        case 8: return launch_channels_t<8>(s, c, m, q, out, k_new, v_new, ws, st, begun);
-        case 9: return launch_channels_t<9>(s, c, m, q, out, k_new, v_new, ws, st, begun);
-        case 10: return launch_channels_t<10>(s, c, m, q, out, k_new, v_new, ws, st, begun);
+        case 5: return launch_channels_t<5>(s, a, n, m, st, begun);
+        case 6: return launch_channels_t<6>(s, a, n, m, st, begun);
+        case 7: return launch_channels_t<7>(s, a, n, m, st, begun);
+        case 8: return launch_channels_t<8>(s, a, n, m, st, begun);
+        case 9: return launch_channels_t<9>(s, a, n, m, st, begun);
+        case 10: return launch_channels_t<10>(s, a, n, m, st, begun);
         default: return cudaErrorInvalidValue;
     }
 }
