@@ -31,6 +31,9 @@ constexpr int kChanThreads = 256;    // (as many as the transform passes are wri
 constexpr int kMainWarps = 4;
 constexpr int kMainCtas = 3;         // CTAs of the main kernel to an SM
 constexpr int kWinStage = 4096;      // window parts of the main kernel: 16 rows of K or of V
+// CTAs of the outer kernels to an SM: three where 80 registers do without spills, which several layers in a launch fill (the instances of 64 and 512
+// slots, whose last pass is of eight points, spill 400 bytes there).
+constexpr int outer_ctas(int ls) { return ls == 5 || ls == 7 || ls == 8 ? 3 : 2; }
 constexpr double kPartCost = 64 * 1024;          // what a part of the main kernel costs beside its bytes, in bytes
 
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
@@ -82,6 +85,12 @@ __device__ __forceinline__ void channel_factors(float* g_s, int q0, int nq, int 
     }
 }
 
+// Over how many threads (as a power of two) the nq channel pairs (a power of two) of a bin are split so that `items` bins fill the CTA.
+__device__ __forceinline__ int split_pairs(int items, int nq) {
+    int lg = 0;
+    while ((items << lg) < kChanThreads && (2 << lg) <= nq) ++lg;
+    return lg;
+}
 template <int LS>
 __device__ __forceinline__ void pass_twiddles(float* twf, int tid) {
     for (int l = LS; l > 0;) {
@@ -117,6 +126,14 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t a, uint32_t rank) {
     return r;
 }
 __device__ __forceinline__ void st_peer(uint32_t a, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void st_peer4(uint32_t a, float4 v) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ float2 ld_peer2(uint32_t a) {
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
 __device__ __forceinline__ float ld_peer(uint32_t a) {
     float v;
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
@@ -129,6 +146,15 @@ __device__ __forceinline__ float sum_peers(uint32_t a, int n) {
     for (int w = 0; w < 8; ++w) y[w] = w < n ? ld_peer(peer_addr(a, (uint32_t)w)) : 0.f;
 #pragma unroll
     for (int w = 0; w < 8; ++w) v += y[w];
+    return v;
+}
+
+__device__ __forceinline__ float2 sum_peers2(uint32_t a, int n) {
+    float2 y[8], v = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < 8; ++w) y[w] = w < n ? ld_peer2(peer_addr(a, (uint32_t)w)) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < 8; ++w) { v.x += y[w].x; v.y += y[w].y; }
     return v;
 }
 
@@ -152,31 +178,37 @@ __device__ __forceinline__ const bf16* leaving_row(const CacheDev& c, const Dims
 }
 
 // Rows of coefficients of a CTA come in by bulk copies, kStageRows rows to a stage; as many as the stages hold set off at once, the
-// rest is asked for in L2.  All threads use a stage (wait), then one refills it (done).
+// rest is asked for in L2.  All threads use a stage (wait), then one refills it (done).  Stages and their phases are carried along: as remainders and
+// quotients of the stage's number they were a third of the time of the loops over the rows.
 constexpr int kStageRows = 32, kMaxRowStages = 8;
 struct RowStream {
     uint64_t* bar;                                         // [stages]
     float* buf;
     const float* src;
     int rows, nc, n_st, n_chunk;
-    __device__ __forceinline__ void issue(int i) const {   // (one thread)
-        const uint32_t bytes = (uint32_t)(min(kStageRows, rows - i * kStageRows) * nc * 4), bb = smem_addr(bar + i % n_st);
+    int st = 0, ist = 0;                                   // next stage to use; to refill (one thread)
+    uint32_t ph = 0;
+    __device__ __forceinline__ void issue(int i) {         // (one thread) chunk i into the stage after the one before
+        const uint32_t bytes = (uint32_t)(min(kStageRows, rows - i * kStageRows) * nc * 4), bb = smem_addr(bar + ist);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb), "r"(bytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(buf + (size_t)(i % n_st) * kStageRows * nc)),
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(buf + ist * kStageRows * nc)),
                      "l"(__cvta_generic_to_global(src + (size_t)i * kStageRows * nc)), "r"(bytes), "r"(bb)
                      : "memory");
+        if (++ist == n_st) ist = 0;
     }
-    __device__ __forceinline__ void begin() const {        // (one thread; the barriers are initialised)
+    __device__ __forceinline__ void begin() {              // (one thread; the barriers are initialised)
         for (int i = 0; i < n_st && i < n_chunk; ++i) issue(i);
         const int left = rows - n_st * kStageRows;
         if (left > 0)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(src + (size_t)n_st * kStageRows * nc)), "r"(left * nc * 4) : "memory");
     }
-    __device__ __forceinline__ const float* wait(int i, volatile int* fail, int32_t* status) const {
-        mbar_wait(bar + i % n_st, (uint32_t)(i / n_st) & 1u, fail, status);
-        return buf + (size_t)(i % n_st) * kStageRows * nc;
+    __device__ __forceinline__ const float* wait(volatile int* fail, int32_t* status) {      // the next stage
+        const float* x = buf + st * kStageRows * nc;
+        mbar_wait(bar + st, ph, fail, status);
+        if (++st == n_st) { st = 0; ph ^= 1; }
+        return x;
     }
-    __device__ __forceinline__ void done(int i, int n, int tid) const {          // stages i .. i + n (all threads)
+    __device__ __forceinline__ void done(int i, int n, int tid) {                // chunks i .. i + n (all threads)
         if (i + n_st < n_chunk) {
             __syncthreads();
             if (tid == 0)
@@ -226,8 +258,8 @@ struct ChanMaps { LayerMaps l[kChanLayers]; };
 // Cluster per job, 256 threads.  u = scale log2(e) W C^K q, a slice of the rows per CTA, exchanged through distributed shared
 // memory; then Z of nq channel pairs per CTA (a transform carries channels 2 q and 2 q + 1 of one head).  With k_new (a step, one
 // pass) also the push: C^K's rows are updated on their way, the leaving row's kept dims and the new token are written.
-template <int LS>
-__global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
+template <int LS, int NH>
+__global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) chan_in_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
     constexpr int S = 1 << LS;
     extern __shared__ __align__(16) float smz[];
     const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass;
@@ -246,13 +278,14 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, ChanPl
     float* qc = g_s + ((2 * nq * s.k + 3) & ~3);           // [4][dck]
     float* xc = qc + 4 * s.dck;                            // [dck] compressed dims of the leaving row
     float* f_s = xc + s.dck;                               // [rows] basis column of the push
-    bf16* qs = reinterpret_cast<bf16*>(f_s + (((s.M + CL - 1) / CL + 5) & ~3));      // [4][d] query rows, [2][d] the leaving row, [2][d] the new one
+    float2* ph_s = reinterpret_cast<float2*>(f_s + (((s.M + CL - 1) / CL + 5) & ~3));          // [k] e^{i theta n c0}
+    bf16* qs = reinterpret_cast<bf16*>(ph_s + ((s.k + 1) & ~1));       // [4][d] query rows, [2][d] the leaving row, [2][d] the new one
     bf16* xr = qs + 4 * s.d;
     bf16* nr = xr + 2 * s.d;
     float* fbuf = reinterpret_cast<float*>(nr + 2 * s.d);  // [nq nh][fb]; before the transforms: staged rows of C^K
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float* ckg = coef_rows(c.coef_k, s, b, h, s.dck);
-    const RowStream rs = {bars, fbuf, ckg + (size_t)m0 * s.dck, m1 - m0, s.dck, mp.st_in, (m1 - m0 + kStageRows - 1) / kStageRows};
+    RowStream rs = {bars, fbuf, ckg + (size_t)m0 * s.dck, m1 - m0, s.dck, mp.st_in, (m1 - m0 + kStageRows - 1) / kStageRows};
     if (tid == 0) {
         for (int i = 0; i < mp.st_in; ++i) mbar_init(bars + i, 1);
         *fail = 0;
@@ -260,6 +293,7 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, ChanPl
     }
     pass_twiddles<LS>(twf, tid);
     channel_factors(g_s, q0, nq, s.k, S, tid);
+    for (int n = tid; n < s.k; n += kChanThreads) ph_s[n] = mid_phase(n, s);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (tid == 0) rs.begin();
     // everything that a CTA needs of memory, each read once and all at the same time as far as addresses are known
@@ -295,31 +329,41 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, ChanPl
     const int l8 = tid & 7, rgi = tid >> 3;
     const float sl2 = s.scale * kLog2e, inv_T = __int_as_float((127 << 23) - ((31 - __clz(s.T)) << 23));      // T is a power of two
     const float w_gen = sl2 * (s.norm == FA_NORM_PAPER ? 1.0f / (float)s.k : 2.f * inv_T), w_0 = s.norm == FA_NORM_PAPER ? w_gen : 0.5f * w_gen, w_1 = s.norm == FA_NORM_PAPER ? w_gen : 0.f;
-    const uint32_t u_peer = CL > 1 ? peer_addr(smem_addr(u_s), (uint32_t)(l8 < CL ? l8 : 0)) : smem_addr(u_s);
-    cluster_meet(CL);                                      // every CTA of the cluster has started: its shared memory can be written
+    // A thread has the same columns of every row, up to four vectors: the query's and the leaving row's are in registers.  (Read for every row
+    // they were most of what kept the shared-memory pipe busy, and that, not memory, set this loop's pace: 2.6 K cycles per 64 rows of four heads; sums sent to every
+    // CTA of the cluster one by one were the rest.)
+    float4 qr[NH][4], xr4[4];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool on = l8 + 8 * i < nv;
+#pragma unroll
+        for (int g = 0; g < NH; ++g) qr[g][i] = on && g < nh ? *reinterpret_cast<const float4*>(qc + g * s.dck + 4 * (l8 + 8 * i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        xr4[i] = on && pu.j >= 0 ? *reinterpret_cast<const float4*>(xc + 4 * (l8 + 8 * i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     // two stages at a time: eight lanes take a row of each, so that a turn's chain (row, sums over lanes, barrier) is paid half as
-    // often and the query's columns are read once for both (a step of 8 rows of 32 heads, 4K tokens 101.8 -> 100.3 us, of 4 rows of
-    // 128K tokens 192.8 -> 190.5, with the same in the last kernel)
+    // often (a step of 8 rows of 32 heads, 4K tokens 101.8 -> 100.3 us, of 4 rows of 128K tokens 192.8 -> 190.5, with the same in the last kernel)
     for (int i = 0; i < rs.n_chunk; i += 2) {
         const bool both = i + 1 < rs.n_chunk;
-        const float* xs0 = rs.wait(i, fail, c.status);
-        const float* xs1 = both ? rs.wait(i + 1, fail, c.status) : xs0;
+        const float* xs0 = rs.wait(fail, c.status);
+        const float* xs1 = both ? rs.wait(fail, c.status) : xs0;
         const int r0 = i * kStageRows + rgi;               // rows r0 and r0 + kStageRows
         const bool on[2] = {r0 < rs.rows, r0 + kStageRows < rs.rows};
         const float f[2] = {pu.j >= 0 && on[0] ? f_s[r0] : 0.f, pu.j >= 0 && on[1] ? f_s[r0 + kStageRows] : 0.f};
-        float a[2][4];
+        float a[2][NH];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
-            for (int g = 0; g < 4; ++g) a[u][g] = 0.f;
-        if (on[0]) {
-#pragma unroll 2
-            for (int v = l8; v < nv; v += 8) {
-                float4 x[2], y = make_float4(0.f, 0.f, 0.f, 0.f);
-                x[0] = *reinterpret_cast<const float4*>(xs0 + rgi * s.dck + 4 * v);
-                x[1] = on[1] ? *reinterpret_cast<const float4*>(xs1 + rgi * s.dck + 4 * v) : y;
+            for (int g = 0; g < NH; ++g) a[u][g] = 0.f;
+#pragma unroll
+        for (int x4 = 0; x4 < 4; ++x4) {
+            const int v = l8 + 8 * x4;
+            if (v < nv) {
+                float4 x[2];
+                x[0] = on[0] ? *reinterpret_cast<const float4*>(xs0 + rgi * s.dck + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+                x[1] = on[1] ? *reinterpret_cast<const float4*>(xs1 + rgi * s.dck + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
                 if (pu.j >= 0) {
-                    y = *reinterpret_cast<const float4*>(xc + 4 * v);
+                    const float4 y = xr4[x4];
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         x[u].x = fmaf(f[u], y.x, x[u].x); x[u].y = fmaf(f[u], y.y, x[u].y); x[u].z = fmaf(f[u], y.z, x[u].z); x[u].w = fmaf(f[u], y.w, x[u].w);
@@ -327,34 +371,49 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, ChanPl
                     }
                 }
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    if (g < nh) {
-                        const float4 z = *reinterpret_cast<const float4*>(qc + g * s.dck + 4 * v);
+                for (int g = 0; g < NH; ++g) {
+                    const float4 z = qr[g][x4];
 #pragma unroll
-                        for (int u = 0; u < 2; ++u) a[u][g] = fmaf(x[u].x, z.x, fmaf(x[u].y, z.y, fmaf(x[u].z, z.z, fmaf(x[u].w, z.w, a[u][g]))));
-                    }
+                    for (int u = 0; u < 2; ++u) a[u][g] = fmaf(x[u].x, z.x, fmaf(x[u].y, z.y, fmaf(x[u].z, z.z, fmaf(x[u].w, z.w, a[u][g]))));
                 }
             }
         }
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1)
 #pragma unroll
-            for (int g = 0; g < 4; ++g)
-                if (g < nh) {
-                    a[0][g] += __shfl_xor_sync(0xffffffffu, a[0][g], o);
-                    a[1][g] += __shfl_xor_sync(0xffffffffu, a[1][g], o);
-                }
-        if (l8 < CL) {                                     // lane x of a row writes to CTA x of the cluster
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int m = m0 + r0 + u * kStageRows;
-                const float w = m == 0 ? w_0 : m == 1 ? w_1 : w_gen;
-                if (on[u])
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) if (g < nh) st_peer(u_peer + 4u * (uint32_t)(g * s.M + m), w * a[u][g]);
+            for (int g = 0; g < NH; ++g) {
+                a[0][g] += __shfl_xor_sync(0xffffffffu, a[0][g], o);
+                a[1][g] += __shfl_xor_sync(0xffffffffu, a[1][g], o);
             }
+        // lane x of a row keeps head x's
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int m = m0 + r0 + u * kStageRows;
+            float mine = a[u][0];
+#pragma unroll
+            for (int g = 1; g < NH; ++g) if (l8 == g) mine = a[u][g];
+            if (on[u] && l8 < nh) u_s[l8 * s.M + m] = (m == 0 ? w_0 : m == 1 ? w_1 : w_gen) * mine;
         }
         rs.done(i, 2, tid);
+    }
+    if (CL > 1) {                                          // this CTA's rows to the others
+        cluster_meet(CL);                                  // every CTA of the cluster has started: its shared memory can be written; all rows are there
+        const int n = m1 - m0;
+        if (((m0 | n) & 3) == 0) {
+            for (int i = tid; i < nh * (n >> 2); i += kChanThreads) {
+                const int g = i / (n >> 2), at = g * s.M + m0 + 4 * (i - g * (n >> 2));
+                const float4 v = *reinterpret_cast<const float4*>(u_s + at);
+                for (int w = 0; w < CL; ++w)
+                    if (w != rank) st_peer4(peer_addr(smem_addr(u_s + at), (uint32_t)w), v);
+            }
+        } else {
+            for (int i = tid; i < nh * n; i += kChanThreads) {
+                const int g = i / n, at = g * s.M + m0 + i - g * n;
+                const float v = u_s[at];
+                for (int w = 0; w < CL; ++w)
+                    if (w != rank) st_peer(peer_addr(smem_addr(u_s + at), (uint32_t)w), v);
+            }
+        }
     }
     cluster_meet(CL);
     if (blockIdx.y == 0 && b == 0) {                       // the channels' factors, for the last kernel of the chain
@@ -362,14 +421,16 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_in_kernel(Dims s, ChanPl
         for (int i = tid; i < 2 * nq * s.k; i += kChanThreads) gg[i] = g_s[i];
     }
     // packed Hermitian spectra: X_m = V^A_m + i V^B_m, V_m = v_m + conj(v_{S-m}), v_n = (1/2) (2 r + 1) i^r j_r u~_n e^{i theta n c0}
-    for (int i = tid; i < (S / 2) * nh; i += kChanThreads) {
-        const int g = i >> (LS - 1), pr = i & (S / 2 - 1), m = pr, mc = pr == 0 ? S / 2 : S - pr;
+    // (with few bins the channel pairs of a bin go to neighbouring runs of threads)
+    const int lg_q = split_pairs(S / 2 * nh, nq), nq_t = nq >> lg_q;
+    for (int i = tid; i < ((S / 2) * nh) << lg_q; i += kChanThreads) {
+        const int pr = i & (S / 2 - 1), gq = i >> (LS - 1), qs0 = (gq & ((1 << lg_q) - 1)) * nq_t, g = gq >> lg_q, m = pr, mc = pr == 0 ? S / 2 : S - pr;
         float2 bm = make_float2(0.f, 0.f), bc = bm;
         const float* ug = u_s + g * s.M;
-        if (m < s.k) { const float2 x = *reinterpret_cast<const float2*>(ug + 2 * m); bm = cmulf(make_float2(0.5f * x.x, -0.5f * x.y), mid_phase(m, s)); }
-        if (mc < s.k) { const float2 x = *reinterpret_cast<const float2*>(ug + 2 * mc); bc = cmulf(make_float2(0.5f * x.x, -0.5f * x.y), mid_phase(mc, s)); }
+        if (m < s.k) { const float2 x = *reinterpret_cast<const float2*>(ug + 2 * m); bm = cmulf(make_float2(0.5f * x.x, -0.5f * x.y), ph_s[m]); }
+        if (mc < s.k) { const float2 x = *reinterpret_cast<const float2*>(ug + 2 * mc); bc = cmulf(make_float2(0.5f * x.x, -0.5f * x.y), ph_s[mc]); }
 #pragma unroll 2
-        for (int qi = 0; qi < nq; ++qi) {
+        for (int qi = qs0; qi < qs0 + nq_t; ++qi) {
             const float sg = ((q0 + qi) & 1) ? -1.f : 1.f;
             const float am = m < s.k ? sg * g_s[2 * qi * s.k + m] : 0.f, om = m < s.k ? sg * g_s[(2 * qi + 1) * s.k + m] : 0.f;
             const float ac = mc < s.k ? sg * g_s[2 * qi * s.k + mc] : 0.f, oc = mc < s.k ? sg * g_s[(2 * qi + 1) * s.k + mc] : 0.f;
@@ -939,7 +1000,7 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
 // After a step's push (step != 0) C^V's rows are updated on their way.
 // (128 registers at most: the plan counts on two CTAs to an SM, and the instances of 64 and 512 slots took 155, 9 to 11 % of a step)
 template <int LS>
-__global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
+__global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
     constexpr int S = 1 << LS;
     extern __shared__ __align__(16) float smz[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -961,12 +1022,13 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, ChanP
     float* xc = zw_s + 4 * (((s.M + CL - 1) / CL + 5) & ~3);           // [dcv]
     float* f_s = xc + s.dcv;                               // [rows] basis column of the push
     int16_t* inv = reinterpret_cast<int16_t*>(f_s + (((s.M + CL - 1) / CL + 5) & ~3));      // dim -> position in D^vc, or -1
-    float* cv_s = reinterpret_cast<float*>(inv + ((s.d + 7) & ~7));    // stages of rows of C^V
+    float2* ph_s = reinterpret_cast<float2*>(inv + ((s.d + 7) & ~7));  // [k] e^{i theta n c0}
+    float* cv_s = reinterpret_cast<float*>(ph_s + ((s.k + 1) & ~1));   // stages of rows of C^V
     float* fbuf = cv_s + (size_t)mp.st_out * kStageRows * s.dcv;       // [nq nh][fb]
     float* ps_s = fbuf;                                    // [row groups][4][dcv], when the transforms are over
     const int m0 = 2 * ((rank * s.k) / CL), m1 = 2 * (((rank + 1) * s.k) / CL), nv = s.dcv >> 2, nrg = kChanThreads / nv;
     float* cvg = coef_rows(c.coef_v, s, b, h, s.dcv);
-    const RowStream rs = {bars, cv_s, cvg + (size_t)m0 * s.dcv, m1 - m0, s.dcv, mp.st_out, (m1 - m0 + kStageRows - 1) / kStageRows};
+    RowStream rs = {bars, cv_s, cvg + (size_t)m0 * s.dcv, m1 - m0, s.dcv, mp.st_out, (m1 - m0 + kStageRows - 1) / kStageRows};
     if (tid == 0) {
         for (int i = 0; i < mp.st_out; ++i) mbar_init(bars + i, 1);
         *fail = 0;
@@ -975,6 +1037,7 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, ChanP
         rs.begin();
     }
     pass_twiddles<LS>(twf, tid);
+    for (int n = tid; n < s.k; n += kChanThreads) ph_s[n] = mid_phase(n, s);
     asm volatile("griddepcontrol.wait;" ::: "memory");    // the parts
     const int job = (b * s.Hkv + h) * mp.n_pass + pass, X = mp.n_cx + s.B * mp.n_wpart;
     const float2* ml = reinterpret_cast<const float2*>(wsp + mp.off_ml) + (size_t)blockIdx.y * X * 4;       // [part][4]
@@ -1069,12 +1132,14 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, ChanP
     }
     consumer_sync();
     fft_run<2, LS, LS, true>(fbuf, fb, nq * nh, twf, tid);
-    for (int i = tid; i < (S / 2) * nh; i += kChanThreads) {
-        const int g = i >> (LS - 1), pr = i & (S / 2 - 1), m = pr, mc = pr == 0 ? S / 2 : S - pr;
-        if (m >= s.k && mc >= s.k) continue;
+    // (with few bins the channel pairs of a bin go to neighbouring lanes, whose sums are added in a fixed order)
+    const int lg_q = split_pairs(S / 2 * nh, nq), nq_t = nq >> lg_q;
+    for (int i = tid; i < ((S / 2) * nh) << lg_q; i += kChanThreads) {      // (whole warps: S is a multiple of 32 bins and pairs of them)
+        const int bi = i >> lg_q, qs0 = (i & ((1 << lg_q) - 1)) * nq_t, g = bi >> (LS - 1), pr = bi & (S / 2 - 1), m = pr, mc = pr == 0 ? S / 2 : S - pr;
         float2 zm = make_float2(0.f, 0.f), zc = zm;
+        if (m < s.k || mc < s.k)
 #pragma unroll 2
-        for (int qi = 0; qi < nq; ++qi) {
+        for (int qi = qs0; qi < qs0 + nq_t; ++qi) {
             const float* base = fbuf + (qi * nh + g) * fb;
             const float2 ya = *reinterpret_cast<const float2*>(base + pf(m * 2)), yb = *reinterpret_cast<const float2*>(base + pf(mc * 2));
             float2 am, bm, ac, bc;                         // spectra of the two channels at bins m and mc
@@ -1099,34 +1164,42 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, ChanP
                 zc.y += ga * ac.y + go * bc.x;
             }
         }
-        if (m < s.k) *reinterpret_cast<float2*>(z_s + g * s.M + 2 * m) = cmulf(zm, mid_phase(m, s));
-        if (mc < s.k) *reinterpret_cast<float2*>(z_s + g * s.M + 2 * mc) = cmulf(zc, mid_phase(mc, s));
+        for (int o = 1; o < (1 << lg_q); o <<= 1) {
+            zm.x += __shfl_xor_sync(0xffffffffu, zm.x, o);
+            zm.y += __shfl_xor_sync(0xffffffffu, zm.y, o);
+            zc.x += __shfl_xor_sync(0xffffffffu, zc.x, o);
+            zc.y += __shfl_xor_sync(0xffffffffu, zc.y, o);
+        }
+        if (qs0 == 0 && m < s.k) *reinterpret_cast<float2*>(z_s + g * s.M + 2 * m) = cmulf(zm, ph_s[m]);
+        if (qs0 == 0 && mc < s.k) *reinterpret_cast<float2*>(z_s + g * s.M + 2 * mc) = cmulf(zc, ph_s[mc]);
     }
     cluster_meet(CL);                                      // all shares of z are there
     // rows of C^V against the sum of the shares
     const float inv_T = __int_as_float((127 << 23) - ((31 - __clz(s.T)) << 23));      // T is a power of two
     const float w_gen = s.norm == FA_NORM_PAPER ? 1.0f / (float)s.k : 2.f * inv_T, w_0 = s.norm == FA_NORM_PAPER ? w_gen : inv_T, w_1 = s.norm == FA_NORM_PAPER ? w_gen : 0.f;
     const int n_rows = m1 - m0;
-    for (int x = tid; x < n_rows * nh; x += kChanThreads) {
-        const int g = x / n_rows, r = x - g * n_rows, m = m0 + r;
-        const float v = CL == 1 ? z_s[g * s.M + m] : sum_peers(smem_addr(z_s + g * s.M + m), CL);
-        zw_s[r * 4 + g] = v * (m == 0 ? w_0 : m == 1 ? w_1 : w_gen);
+    for (int x = tid; x < (n_rows >> 1) * nh; x += kChanThreads) {          // (rows in pairs, cos and sin of a frequency)
+        const int g = x / (n_rows >> 1), r = 2 * (x - g * (n_rows >> 1)), m = m0 + r;
+        const float2 v = CL == 1 ? *reinterpret_cast<const float2*>(z_s + g * s.M + m) : sum_peers2(smem_addr(z_s + g * s.M + m), CL);
+        zw_s[r * 4 + g] = v.x * (m == 0 ? w_0 : w_gen);
+        zw_s[(r + 1) * 4 + g] = v.y * (m == 0 ? w_1 : w_gen);
     }
     __syncthreads();
     float4 acc4[4];
 #pragma unroll
     for (int g = 0; g < 4; ++g) acc4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int rg = tid / nv, vcol = tid - rg * nv;
-    for (int i = 0; i < rs.n_chunk; ++i) {
-        const int rows = min(kStageRows, rs.rows - i * kStageRows), first = i * kStageRows;
-        const float* xs = rs.wait(i, fail, c.status);
+    const float4 y = j_push >= 0 ? *reinterpret_cast<const float4*>(xc + 4 * vcol) : make_float4(0.f, 0.f, 0.f, 0.f);      // (the thread's columns are the same in every row)
+    for (int i = 0; i < rs.n_chunk; i += 2) {              // two stages at a time
+        const float* xs0 = rs.wait(fail, c.status);
+        const float* xs1 = i + 1 < rs.n_chunk ? rs.wait(fail, c.status) : xs0;
+        const int first = i * kStageRows, rows = min(2 * kStageRows, rs.rows - first);
         if (rg < nrg) {
-#pragma unroll 2
+#pragma unroll 4
             for (int r = rg; r < rows; r += nrg) {
-                float4 x = *reinterpret_cast<const float4*>(xs + r * s.dcv + 4 * vcol);
+                float4 x = *reinterpret_cast<const float4*>((r < kStageRows ? xs0 + r * s.dcv : xs1 + (r - kStageRows) * s.dcv) + 4 * vcol);
                 if (j_push >= 0) {
                     const float f = f_s[first + r];
-                    const float4 y = *reinterpret_cast<const float4*>(xc + 4 * vcol);
                     x.x = fmaf(f, y.x, x.x); x.y = fmaf(f, y.y, x.y); x.z = fmaf(f, y.z, x.z); x.w = fmaf(f, y.w, x.w);
                     *reinterpret_cast<float4*>(cvg + (size_t)(m0 + first + r) * s.dcv + 4 * vcol) = x;
                 }
@@ -1143,7 +1216,7 @@ __global__ void __launch_bounds__(kChanThreads, 2) chan_out_kernel(Dims s, ChanP
                 }
             }
         }
-        if ((i & 1) || i + 1 == rs.n_chunk) rs.done(i & ~1, 2, tid);         // two stages at a time
+        rs.done(i, 2, tid);
     }
     if (rg < nrg) {
 #pragma unroll
@@ -1191,12 +1264,12 @@ bool mid_map(CUtensorMap* tm, const void* base, const Dims& s, int nf) {
 size_t in_smem(const Dims& s, int ls, const ChanPlan& m) {
     const size_t fft = (size_t)m.nq * m.nh * pf_size(2 << ls), stage = (size_t)m.st_in * kStageRows * s.dck;
     return sizeof(float) * (20 + ((2 * (tw_total(ls) + 1) + 3) & ~3) + (size_t)m.nh * s.M + ((2 * m.nq * s.k + 3) & ~3) + 5 * s.dck +
-                            (((s.M + m.nz - 1) / m.nz + 5) & ~3) + 4 * s.d + (fft > stage ? fft : stage)) + 64;
+                            (((s.M + m.nz - 1) / m.nz + 5) & ~3) + 2 * ((s.k + 1) & ~1) + 4 * s.d + (fft > stage ? fft : stage)) + 64;
 }
 size_t out_smem(const Dims& s, int ls, const ChanPlan& m) {
     const size_t fft = (size_t)m.nq * m.nh * pf_size(2 << ls), ps = (size_t)kChanThreads * 4 * m.nh;
     return sizeof(float) * (20 + ((2 * (tw_total(ls) + 1) + 3) & ~3) + (size_t)m.nh * s.M + ((2 * m.nq * s.k + 3) & ~3) + 8 + 5 * s.dcv +
-                            5 * (size_t)(((s.M + m.nz - 1) / m.nz + 5) & ~3) + ((s.d + 7) & ~7) / 2 + (size_t)m.st_out * kStageRows * s.dcv + (fft > ps ? fft : ps)) + 64;
+                            5 * (size_t)(((s.M + m.nz - 1) / m.nz + 5) & ~3) + ((s.d + 7) & ~7) / 2 + 2 * ((s.k + 1) & ~1) + (size_t)m.st_out * kStageRows * s.dcv + (fft > ps ? fft : ps)) + 64;
 }
 
 template <typename... Params, typename... Args>
@@ -1221,6 +1294,15 @@ cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, siz
 }
 
 }  // namespace
+
+// As many stages of the outer kernels' rows as a CTA's rows take and the limit of shared memory holds, two at least.
+static void fit_stages(const Dims& s, int log2S, size_t limit, ChanPlan* m) {
+    auto fits = [&]() { return in_smem(s, log2S, *m) <= limit && out_smem(s, log2S, *m) <= limit; };
+    const int chunks = (s.M / m->nz + 2 + kStageRows - 1) / kStageRows, most = chunks < kMaxRowStages ? chunks : kMaxRowStages;
+    m->st_in = m->st_out = 2;
+    for (; m->st_in < most; ++m->st_in) { ++m->st_in; const bool ok = fits(); --m->st_in; if (!ok) break; }
+    for (; m->st_out < most; ++m->st_out) { ++m->st_out; const bool ok = fits(); --m->st_out; if (!ok) break; }
+}
 
 // When the last of n1 parts of cost a, then n2 of cost b, ends on so many slots.
 static double makespan(long long n1, double a, long long n2, double b, int slots) {
@@ -1291,11 +1373,7 @@ bool plan_channels(const Dims& s, int log2S, int sms, ChanPlan* m) {
     if (!best_nz) return false;
     m->nz = best_nz;
     m->nq = kMR / 2 / m->nz;
-    // then as many stages as a CTA's rows take
-    const size_t limit = occ == 2 && jobs * m->nz > sms ? kHalf : kAll;
-    const int chunks = (s.M / m->nz + 2 + kStageRows - 1) / kStageRows, most = chunks < kMaxRowStages ? chunks : kMaxRowStages;
-    for (; m->st_in < most; ++m->st_in) { ++m->st_in; const bool ok = fits(limit); --m->st_in; if (!ok) break; }
-    for (; m->st_out < most; ++m->st_out) { ++m->st_out; const bool ok = fits(limit); --m->st_out; if (!ok) break; }
+    fit_stages(s, log2S, occ == 2 && jobs * m->nz > sms ? kHalf : kAll, m);
     return true;
 }
 
@@ -1317,9 +1395,17 @@ size_t place_channels(const Dims& s, int log2S, ChanPlan* m) {
 }
 
 template <int LS>
-static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, const ChanPlan& m, cudaStream_t st, bool* begun) {
+static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, const ChanPlan& one, cudaStream_t st, bool* begun) {
     *begun = false;
     if (n < 1 || n > kChanLayers) return cudaErrorInvalidValue;
+    ChanPlan m = one;
+    // several layers, more CTAs than two to an SM: fewer stages each, so that three fit (the sums do not depend on the number of stages)
+    constexpr size_t kThird = 74 * 1024;
+    if (outer_ctas(LS) == 3 && (long long)n * s.B * s.Hkv * m.n_pass * m.nz > 2 * sm_count()) {
+        m.st_in = m.st_out = 2;
+        if (in_smem(s, LS, m) <= kThird && out_smem(s, LS, m) <= kThird) fit_stages(s, LS, kThird, &m);
+        else m = one;
+    }
     const dim3 cg(m.nz, s.Hkv * m.n_pass, s.B * n), mg(s.Hkv * m.n_pass, n * (m.n_cx + s.B * m.n_wpart));
     ChanCall call = {};
     ChanMaps maps;
@@ -1334,7 +1420,8 @@ static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, co
         if ((s.l_init > 0 && !ok_i) || (s.l_local > 0 && !ok_l)) return cudaErrorInvalidValue;
         if (!mid_map(&t.km, c.k_mid, s, s.nfk) || !mid_map(&t.vm, c.v_mid, s, s.nfv)) return cudaErrorInvalidValue;
     }
-    cudaError_t err = launch_chained(chan_in_kernel<LS>, cg, dim3(kChanThreads), in_smem(s, LS, m), m.nz, st, s, m, call);
+    cudaError_t err = m.hp == 2 ? launch_chained(chan_in_kernel<LS, 2>, cg, dim3(kChanThreads), in_smem(s, LS, m), m.nz, st, s, m, call)
+                                : launch_chained(chan_in_kernel<LS, 4>, cg, dim3(kChanThreads), in_smem(s, LS, m), m.nz, st, s, m, call);
     if (err != cudaSuccess) return err;
     *begun = true;
     err = m.hp == 2 ? launch_chained(chan_main_kernel<2>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, maps, s, m, call)

@@ -127,3 +127,58 @@ def test_channels_ragged_small_workspace_and_graph(ragged_one_short):
     assert all(fa.fa_poll_status(x) == status for x in a + b + c + d)
     del g
 
+
+
+def test_layers_share_launches_and_depend_on_one_another():
+    """Five layers in one call (four side by side, one more) give the bits of single calls; layers that touch one another's memory (a layer's
+    result is the next one's query; one cache twice) run one after the other; with a workspace for one layer's areas they do too."""
+    shape = _shape(Hq=32, L=900, M=64)
+    pair, stream = make_pair(shape, seed=11, P=128, max_mid=shape.T, freq="offgrid")
+    layout, n = pair.layout, 5
+    assert fa.fa_launch_count(layout, 7) == 3
+    kn, vn = (x.cuda() for x in stream.tokens(shape.L, shape.L + n))
+    ks, vs = ([x[:, i].contiguous() for i in range(n)] for x in (kn, vn))
+    qs = [synth.queries(shape, seed=3, layer=i).cuda() for i in range(n)]
+
+    def caches():
+        out = [fa.Cache(layout, stream.idx_full_k, stream.idx_full_v) for _ in range(n)]
+        for c in out:
+            for name in BUFFERS:
+                getattr(c, name).copy_(getattr(pair.gpu, name))
+        return out
+
+    def call(cs, q, out, ws=None):
+        fa.fa_decode_step_layers(fa.LayerStep([layout] * n, cs, q, ks, vs, out), pair.ws if ws is None else ws)
+        torch.cuda.synchronize()
+
+    def one_by_one(cs, q, out):
+        for i in range(n):
+            fa.fa_decode_step(layout, cs[i], q[i], ks[i], vs[i], out[i], pair.ws)
+        torch.cuda.synchronize()
+
+    def same(a, b, ca, cb):
+        for x, y in zip(a, b):
+            assert torch.equal(x.view(torch.int16), y.view(torch.int16))
+        for x, y in zip(ca, cb):
+            assert all(torch.equal(getattr(x, m), getattr(y, m)) for m in BUFFERS)
+            assert fa.fa_poll_status(x) == fa.FA_OK
+
+    new = lambda: [torch.full_like(q, float("nan")) for q in qs]
+    ca, cb, a, b = caches(), caches(), new(), new()
+    call(ca, qs, a)
+    one_by_one(cb, qs, b)
+    same(a, b, ca, cb)
+    cc, c = caches(), new()
+    call(cc, qs, c, torch.zeros(fa.fa_workspace_bytes(layout) // 3, dtype=torch.uint8, device="cuda"))
+    same(c, b, cc, cb)
+    # a chain: layer i + 1 asks with layer i's result
+    ca, cb, a, b = caches(), caches(), new(), new()
+    call(ca, [qs[0]] + a[:-1], a)
+    one_by_one(cb, [qs[0]] + b[:-1], b)
+    same(a, b, ca, cb)
+    # one cache for all: n pushes, each asked after it
+    ca, cb, a, b = caches(), caches(), new(), new()
+    call([ca[0]] * n, qs, a)
+    one_by_one([cb[0]] * n, qs, b)
+    same(a, b, ca[:1], cb[:1])
+    assert ca[0].state[:, 2].tolist() == [shape.L - 68 + n] * shape.B
