@@ -27,13 +27,14 @@ namespace fa {
 namespace {
 
 constexpr int kMR = 16;              // channels
-constexpr int kChanThreads = 256;    // (as many as the transform passes are written for)
 constexpr int kMainWarps = 4;
 constexpr int kMainCtas = 3;         // CTAs of the main kernel to an SM
 constexpr int kWinStage = 4096;      // window parts of the main kernel: 16 rows of K or of V
 // CTAs of the outer kernels to an SM: three where 80 registers do without spills, which several layers in a launch fill (the instances of 64 and 512
 // slots, whose last pass is of eight points, spill 400 bytes there).
-constexpr int outer_ctas(int ls) { return ls == 5 || ls == 7 || ls == 8 ? 3 : 2; }
+// Threads of an outer kernel's CTA.  The longest transforms leave room for one CTA to an SM: sixteen warps of it instead of eight.
+__host__ __device__ constexpr int outer_threads(int ls) { return ls == 10 ? 512 : 256; }
+__host__ __device__ constexpr int outer_ctas(int ls) { return ls == 10 ? 1 : ls == 5 || ls == 7 || ls == 8 ? 3 : 2; }
 constexpr double kPartCost = 64 * 1024;          // what a part of the main kernel costs beside its bytes, in bytes
 
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
@@ -52,8 +53,9 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t&
 }
 
 // (2 r + 1) j_r(pi n / S) of channels 2 q0 .. 2 q0 + 2 nq for n < k, into g_s[2 nq][k].
+template <int NT>
 __device__ __forceinline__ void channel_factors(float* g_s, int q0, int nq, int k, int S, int tid) {
-    for (int n = tid; n < k; n += kChanThreads) {
+    for (int n = tid; n < k; n += NT) {
         float keep[kMR];
 #pragma unroll
         for (int r = 0; r < kMR; ++r) keep[r] = 0.f;
@@ -86,9 +88,9 @@ __device__ __forceinline__ void channel_factors(float* g_s, int q0, int nq, int 
 }
 
 // Over how many threads (as a power of two) the nq channel pairs (a power of two) of a bin are split so that `items` bins fill the CTA.
-__device__ __forceinline__ int split_pairs(int items, int nq) {
+__device__ __forceinline__ int split_pairs(int items, int nq, int threads) {
     int lg = 0;
-    while ((items << lg) < kChanThreads && (2 << lg) <= nq) ++lg;
+    while ((items << lg) < threads && (2 << lg) <= nq) ++lg;
     return lg;
 }
 template <int LS>
@@ -97,7 +99,7 @@ __device__ __forceinline__ void pass_twiddles(float* twf, int tid) {
         const int rl = radix_log2(l), R = 1 << rl, st = 1 << (l - rl);
         if (l > rl) {
             const int off = tw_offset(LS, l);
-            for (int i = tid; i < (R - 1) * st; i += kChanThreads) {
+            for (int i = tid; i < (R - 1) * st; i += outer_threads(LS)) {
                 const int qm1 = i >> (l - rl), j = i & (st - 1);
                 reinterpret_cast<float2*>(twf)[off + i] = cis_frac((float)(((qm1 + 1) * j) & ((1 << l) - 1)) * (1.0f / (float)(1 << l)));
             }
@@ -202,11 +204,16 @@ struct RowStream {
         if (left > 0)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(src + (size_t)n_st * kStageRows * nc)), "r"(left * nc * 4) : "memory");
     }
-    __device__ __forceinline__ const float* wait(volatile int* fail, int32_t* status) {      // the next stage
-        const float* x = buf + st * kStageRows * nc;
-        mbar_wait(bar + st, ph, fail, status);
-        if (++st == n_st) { st = 0; ph ^= 1; }
-        return x;
+    __device__ __forceinline__ const float* wait(int k, volatile int* fail, int32_t* status) const {      // the k-th stage from the next one on
+        int x = st + k;
+        uint32_t p = ph;
+        if (x >= n_st) { x -= n_st; p ^= 1; }
+        mbar_wait(bar + x, p, fail, status);
+        return buf + x * kStageRows * nc;
+    }
+    __device__ __forceinline__ void next(int n) {          // past n stages (at most as many as there are)
+        st += n;
+        if (st >= n_st) { st -= n_st; ph ^= 1; }
     }
     __device__ __forceinline__ void done(int i, int n, int tid) {                // chunks i .. i + n (all threads)
         if (i + n_st < n_chunk) {
@@ -259,8 +266,8 @@ struct ChanMaps { LayerMaps l[kChanLayers]; };
 // memory; then Z of nq channel pairs per CTA (a transform carries channels 2 q and 2 q + 1 of one head).  With k_new (a step, one
 // pass) also the push: C^K's rows are updated on their way, the leaving row's kept dims and the new token are written.
 template <int LS, int NH>
-__global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) chan_in_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
-    constexpr int S = 1 << LS;
+__global__ void __launch_bounds__(outer_threads(LS), NH == 4 && outer_ctas(LS) == 3 ? 2 : outer_ctas(LS)) chan_in_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
+    constexpr int S = 1 << LS, NT = outer_threads(LS);
     extern __shared__ __align__(16) float smz[];
     const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass;
     const int layer = blockIdx.z / s.B, b = blockIdx.z - layer * s.B;
@@ -292,8 +299,8 @@ __global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) ch
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     pass_twiddles<LS>(twf, tid);
-    channel_factors(g_s, q0, nq, s.k, S, tid);
-    for (int n = tid; n < s.k; n += kChanThreads) ph_s[n] = mid_phase(n, s);
+    channel_factors<NT>(g_s, q0, nq, s.k, S, tid);
+    for (int n = tid; n < s.k; n += NT) ph_s[n] = mid_phase(n, s);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (tid == 0) rs.begin();
     // everything that a CTA needs of memory, each read once and all at the same time as far as addresses are known
@@ -318,7 +325,7 @@ __global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) ch
             *reinterpret_cast<uint4*>(xr + side * s.d + 8 * ch) =
                 *reinterpret_cast<const uint4*>(leaving_row(c, s, b, h, side, pu.head, side == 0 ? k_new : v_new) + 8 * ch);
         }
-        for (int r = tid; r < m1 - m0; r += kChanThreads) f_s[r] = basis_value(m0 + r, pu.j, s.T);
+        for (int r = tid; r < m1 - m0; r += NT) f_s[r] = basis_value(m0 + r, pu.j, s.T);
     }
     __syncthreads();
     if (tid < s.dck) {
@@ -343,13 +350,14 @@ __global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) ch
     }
     // two stages at a time: eight lanes take a row of each, so that a turn's chain (row, sums over lanes, barrier) is paid half as
     // often (a step of 8 rows of 32 heads, 4K tokens 101.8 -> 100.3 us, of 4 rows of 128K tokens 192.8 -> 190.5, with the same in the last kernel)
-    for (int i = 0; i < rs.n_chunk; i += 2) {
-        const bool both = i + 1 < rs.n_chunk;
-        const float* xs0 = rs.wait(fail, c.status);
-        const float* xs1 = both ? rs.wait(fail, c.status) : xs0;
-        const int r0 = i * kStageRows + rgi;               // rows r0 and r0 + kStageRows
-        const bool on[2] = {r0 < rs.rows, r0 + kStageRows < rs.rows};
-        const float f[2] = {pu.j >= 0 && on[0] ? f_s[r0] : 0.f, pu.j >= 0 && on[1] ? f_s[r0 + kStageRows] : 0.f};
+    constexpr int RP = NT / 8, SP = RP / kStageRows;       // rows at a time, their stages; two of these to a turn
+    for (int i = 0; i < rs.n_chunk; i += 2 * SP) {
+        const int r0 = i * kStageRows + rgi;               // rows r0 and r0 + RP (a warp's are in one stage each)
+        const bool on[2] = {r0 < rs.rows, r0 + RP < rs.rows};
+        const float* xs[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) xs[u] = on[u] ? rs.wait(u * SP + rgi / kStageRows, fail, c.status) + (rgi % kStageRows) * s.dck : nullptr;
+        const float f[2] = {pu.j >= 0 && on[0] ? f_s[r0] : 0.f, pu.j >= 0 && on[1] ? f_s[r0 + RP] : 0.f};
         float a[2][NH];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
@@ -360,14 +368,14 @@ __global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) ch
             const int v = l8 + 8 * x4;
             if (v < nv) {
                 float4 x[2];
-                x[0] = on[0] ? *reinterpret_cast<const float4*>(xs0 + rgi * s.dck + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
-                x[1] = on[1] ? *reinterpret_cast<const float4*>(xs1 + rgi * s.dck + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) x[u] = on[u] ? *reinterpret_cast<const float4*>(xs[u] + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
                 if (pu.j >= 0) {
                     const float4 y = xr4[x4];
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         x[u].x = fmaf(f[u], y.x, x[u].x); x[u].y = fmaf(f[u], y.y, x[u].y); x[u].z = fmaf(f[u], y.z, x[u].z); x[u].w = fmaf(f[u], y.w, x[u].w);
-                        if (on[u]) *reinterpret_cast<float4*>(ckg + (size_t)(m0 + r0 + u * kStageRows) * s.dck + 4 * v) = x[u];
+                        if (on[u]) *reinterpret_cast<float4*>(ckg + (size_t)(m0 + r0 + u * RP) * s.dck + 4 * v) = x[u];
                     }
                 }
 #pragma unroll
@@ -388,26 +396,27 @@ __global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) ch
         // lane x of a row keeps head x's
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int m = m0 + r0 + u * kStageRows;
+            const int m = m0 + r0 + u * RP;
             float mine = a[u][0];
 #pragma unroll
             for (int g = 1; g < NH; ++g) if (l8 == g) mine = a[u][g];
             if (on[u] && l8 < nh) u_s[l8 * s.M + m] = (m == 0 ? w_0 : m == 1 ? w_1 : w_gen) * mine;
         }
-        rs.done(i, 2, tid);
+        rs.next(2 * SP);
+        rs.done(i, 2 * SP, tid);
     }
     if (CL > 1) {                                          // this CTA's rows to the others
         cluster_meet(CL);                                  // every CTA of the cluster has started: its shared memory can be written; all rows are there
         const int n = m1 - m0;
         if (((m0 | n) & 3) == 0) {
-            for (int i = tid; i < nh * (n >> 2); i += kChanThreads) {
+            for (int i = tid; i < nh * (n >> 2); i += NT) {
                 const int g = i / (n >> 2), at = g * s.M + m0 + 4 * (i - g * (n >> 2));
                 const float4 v = *reinterpret_cast<const float4*>(u_s + at);
                 for (int w = 0; w < CL; ++w)
                     if (w != rank) st_peer4(peer_addr(smem_addr(u_s + at), (uint32_t)w), v);
             }
         } else {
-            for (int i = tid; i < nh * n; i += kChanThreads) {
+            for (int i = tid; i < nh * n; i += NT) {
                 const int g = i / n, at = g * s.M + m0 + i - g * n;
                 const float v = u_s[at];
                 for (int w = 0; w < CL; ++w)
@@ -418,12 +427,12 @@ __global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) ch
     cluster_meet(CL);
     if (blockIdx.y == 0 && b == 0) {                       // the channels' factors, for the last kernel of the chain
         float* gg = reinterpret_cast<float*>(wsp + mp.off_g) + (size_t)2 * q0 * s.k;
-        for (int i = tid; i < 2 * nq * s.k; i += kChanThreads) gg[i] = g_s[i];
+        for (int i = tid; i < 2 * nq * s.k; i += NT) gg[i] = g_s[i];
     }
     // packed Hermitian spectra: X_m = V^A_m + i V^B_m, V_m = v_m + conj(v_{S-m}), v_n = (1/2) (2 r + 1) i^r j_r u~_n e^{i theta n c0}
     // (with few bins the channel pairs of a bin go to neighbouring runs of threads)
-    const int lg_q = split_pairs(S / 2 * nh, nq), nq_t = nq >> lg_q;
-    for (int i = tid; i < ((S / 2) * nh) << lg_q; i += kChanThreads) {
+    const int lg_q = split_pairs(S / 2 * nh, nq, NT), nq_t = nq >> lg_q;
+    for (int i = tid; i < ((S / 2) * nh) << lg_q; i += NT) {
         const int pr = i & (S / 2 - 1), gq = i >> (LS - 1), qs0 = (gq & ((1 << lg_q) - 1)) * nq_t, g = gq >> lg_q, m = pr, mc = pr == 0 ? S / 2 : S - pr;
         float2 bm = make_float2(0.f, 0.f), bc = bm;
         const float* ug = u_s + g * s.M;
@@ -447,34 +456,35 @@ __global__ void __launch_bounds__(kChanThreads, NH == 2 ? outer_ctas(LS) : 2) ch
             }
         }
     }
-    consumer_sync();
-    fft_run<2, LS, LS, false>(fbuf, fb, nq * nh, twf, tid);
+    __syncthreads();
+    fft_run<2, LS, LS, false, 1, NT>(fbuf, fb, nq * nh, twf, tid);
     // last pass, and Z as [channel pair][slot][HP heads][hi, lo]: a thread has all heads of its slots
     constexpr int RL = last_radix_log2(LS), R = 1 << RL, JL = LS - RL;
     const int job = (b * s.Hkv + h) * mp.n_pass + pass;
     uint32_t* Z = reinterpret_cast<uint32_t*>(wsp + mp.off_z) + ((size_t)job * (kMR / 2) + q0) * S * 2 * mp.hp;
-    for (int i = tid; i < nq << JL; i += kChanThreads) {
-        const int qi = i >> JL, j = i & ((1 << JL) - 1);
-        uint32_t hl[R][4][2];
+    const int lg_h = mp.hp == 4 && (nq << JL) < NT ? 1 : 0;            // a slot's two pairs of heads by two neighbouring threads where there are threads for it
+    for (int i = tid; i < (nq << JL) << lg_h; i += NT) {
+        const int it = i >> lg_h, qi = it >> JL, j = it & ((1 << JL) - 1);
+        for (int hv = i & lg_h; hv < (mp.hp >> 1); hv += 1 + lg_h) {
+            uint32_t hl[R][2][2];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            PC<1> v[R];
+            for (int g2 = 0; g2 < 2; ++g2) {
+                const int g = 2 * hv + g2;
+                PC<1> v[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = PC<1>{PR<1>{0.f}, PR<1>{0.f}};
-            if (g < nh) {
-                const float* base = fbuf + (qi * nh + g) * fb + pf(dif_pos<LS>(j) * 2);
+                for (int r = 0; r < R; ++r) v[r] = PC<1>{PR<1>{0.f}, PR<1>{0.f}};
+                if (g < nh) {
+                    const float* base = fbuf + (qi * nh + g) * fb + pf(dif_pos<LS>(j) * 2);
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[r] = ld_pt<1>(base + pf(r * 2));
-                dft<R, 1>(v);
+                    for (int r = 0; r < R; ++r) v[r] = ld_pt<1>(base + pf(r * 2));
+                    dft<R, 1>(v);
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) split2(v[r].re.v, v[r].im.v, hl[r][g2][0], hl[r][g2][1]);
             }
 #pragma unroll
-            for (int r = 0; r < R; ++r) split2(v[r].re.v, v[r].im.v, hl[r][g][0], hl[r][g][1]);
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            uint4* dst = reinterpret_cast<uint4*>(Z + ((size_t)qi * S + j + (r << JL)) * 2 * mp.hp);
-            dst[0] = make_uint4(hl[r][0][0], hl[r][0][1], hl[r][1][0], hl[r][1][1]);
-            if (mp.hp == 4) dst[1] = make_uint4(hl[r][2][0], hl[r][2][1], hl[r][3][0], hl[r][3][1]);
+            for (int r = 0; r < R; ++r)
+                reinterpret_cast<uint4*>(Z + ((size_t)qi * S + j + (r << JL)) * 2 * mp.hp)[hv] = make_uint4(hl[r][0][0], hl[r][0][1], hl[r][1][0], hl[r][1][1]);
         }
     }
     // The push's rows and counters.  What the cluster reads of the old ones it has read before its meeting (one cluster per KV
@@ -1000,8 +1010,8 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
 // After a step's push (step != 0) C^V's rows are updated on their way.
 // (128 registers at most: the plan counts on two CTAs to an SM, and the instances of 64 and 512 slots took 155, 9 to 11 % of a step)
 template <int LS>
-__global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
-    constexpr int S = 1 << LS;
+__global__ void __launch_bounds__(outer_threads(LS), outer_ctas(LS)) chan_out_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
+    constexpr int S = 1 << LS, NT = outer_threads(LS);
     extern __shared__ __align__(16) float smz[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass;
@@ -1026,7 +1036,7 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
     float* cv_s = reinterpret_cast<float*>(ph_s + ((s.k + 1) & ~1));   // stages of rows of C^V
     float* fbuf = cv_s + (size_t)mp.st_out * kStageRows * s.dcv;       // [nq nh][fb]
     float* ps_s = fbuf;                                    // [row groups][4][dcv], when the transforms are over
-    const int m0 = 2 * ((rank * s.k) / CL), m1 = 2 * (((rank + 1) * s.k) / CL), nv = s.dcv >> 2, nrg = kChanThreads / nv;
+    const int m0 = 2 * ((rank * s.k) / CL), m1 = 2 * (((rank + 1) * s.k) / CL), nv = s.dcv >> 2, nrg = NT / nv;
     float* cvg = coef_rows(c.coef_v, s, b, h, s.dcv);
     RowStream rs = {bars, cv_s, cvg + (size_t)m0 * s.dcv, m1 - m0, s.dcv, mp.st_out, (m1 - m0 + kStageRows - 1) / kStageRows};
     if (tid == 0) {
@@ -1037,7 +1047,7 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
         rs.begin();
     }
     pass_twiddles<LS>(twf, tid);
-    for (int n = tid; n < s.k; n += kChanThreads) ph_s[n] = mid_phase(n, s);
+    for (int n = tid; n < s.k; n += NT) ph_s[n] = mid_phase(n, s);
     asm volatile("griddepcontrol.wait;" ::: "memory");    // the parts
     const int job = (b * s.Hkv + h) * mp.n_pass + pass, X = mp.n_cx + s.B * mp.n_wpart;
     const float2* ml = reinterpret_cast<const float2*>(wsp + mp.off_ml) + (size_t)blockIdx.y * X * 4;       // [part][4]
@@ -1047,7 +1057,7 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
     const int2 rp = reinterpret_cast<const int2*>(wsp + mp.off_p)[b];      // this row's class parts: first, number
     const int n_mid = min(c.state[kStateStride * b + 2], s.max_mid), a_end = (n_mid + s.P - 1) / s.P;
     const int j_push = step ? reinterpret_cast<const int32_t*>(wsp + mp.off_j)[b] : -1;
-    for (int i = tid; i < 2 * nq * s.k / 4; i += kChanThreads)
+    for (int i = tid; i < 2 * nq * s.k / 4; i += NT)
         cp_async16(g_s + 4 * i, reinterpret_cast<const float*>(wsp + mp.off_g) + (size_t)2 * q0 * s.k + 4 * i);
     const int np = rp.y + mp.n_wpart, wshift = mp.n_cx + b * mp.n_wpart - rp.y;
     auto part_at = [&](int i) { return i < rp.y ? rp.x + i : wshift + i; };
@@ -1069,41 +1079,43 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
         }
     }
     if (j_push >= 0)
-        for (int r = tid; r < m1 - m0; r += kChanThreads) f_s[r] = basis_value(m0 + r, j_push, s.T);
+        for (int r = tid; r < m1 - m0; r += NT) f_s[r] = basis_value(m0 + r, j_push, s.T);
     cp_async_wait_all();
     __syncthreads();
     constexpr int RL = last_radix_log2(LS), R = 1 << RL, JL = LS - RL;
-    for (int i = tid; i < nq << JL; i += kChanThreads) {
-        const int qi = i >> JL, j = i & ((1 << JL) - 1);
-        float4 x[R][2], mw[R];                             // the heads' two channels at this thread's slots, what they refer to
+    const int lg_h = mp.hp == 4 && (nq << JL) < NT ? 1 : 0;
+    for (int i = tid; i < (nq << JL) << lg_h; i += NT) {
+        const int it = i >> lg_h, qi = it >> JL, j = it & ((1 << JL) - 1);
+        for (int hv = i & lg_h; hv < (mp.hp >> 1); hv += 1 + lg_h) {
+            float4 x[R];                                   // two heads' two channels at this thread's slots
+            float2 mw[R];                                  // what they refer to
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int a = j + (r << JL);
-            x[r][0] = x[r][1] = mw[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (a < a_end) {
-                const float4* src = reinterpret_cast<const float4*>(W + ((size_t)qi * S + a) * mp.hp);
-                x[r][0] = src[0];
-                if (mp.hp == 4) x[r][1] = src[1];
-                mw[r] = *reinterpret_cast<const float4*>(mW + (a >> 2) * 4);
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            if (g < nh) {
-                PC<1> v[R];
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float mv = g == 0 ? mw[r].x : g == 1 ? mw[r].y : g == 2 ? mw[r].z : mw[r].w;
-                    const float2 y = g == 0 ? make_float2(x[r][0].x, x[r][0].y) : g == 1 ? make_float2(x[r][0].z, x[r][0].w)
-                                   : g == 2 ? make_float2(x[r][1].x, x[r][1].y) : make_float2(x[r][1].z, x[r][1].w);
-                    const float sc = ex2(mv - mfin[g]);
-                    const bool on = j + (r << JL) < a_end && g < ng;
-                    v[r] = on ? PC<1>{PR<1>{y.x * sc}, PR<1>{y.y * sc}} : PC<1>{PR<1>{0.f}, PR<1>{0.f}};
+            for (int r = 0; r < R; ++r) {
+                const int a = j + (r << JL);
+                x[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+                mw[r] = make_float2(0.f, 0.f);
+                if (a < a_end) {
+                    x[r] = reinterpret_cast<const float4*>(W + ((size_t)qi * S + a) * mp.hp)[hv];
+                    mw[r] = reinterpret_cast<const float2*>(mW + (a >> 2) * 4)[hv];
                 }
-                dft<R, 1>(v);
-                float* base = fbuf + (qi * nh + g) * fb + pf(dif_pos<LS>(j) * 2);
+            }
 #pragma unroll
-                for (int r = 0; r < R; ++r) st_pt(base + pf(r * 2), v[r]);
+            for (int g2 = 0; g2 < 2; ++g2) {
+                const int g = 2 * hv + g2;
+                if (g < nh) {
+                    PC<1> v[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float2 y = g2 == 0 ? make_float2(x[r].x, x[r].y) : make_float2(x[r].z, x[r].w);
+                        const float sc = ex2((g2 == 0 ? mw[r].x : mw[r].y) - mfin[g]);
+                        const bool on = j + (r << JL) < a_end && g < ng;
+                        v[r] = on ? PC<1>{PR<1>{y.x * sc}, PR<1>{y.y * sc}} : PC<1>{PR<1>{0.f}, PR<1>{0.f}};
+                    }
+                    dft<R, 1>(v);
+                    float* base = fbuf + (qi * nh + g) * fb + pf(dif_pos<LS>(j) * 2);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) st_pt(base + pf(r * 2), v[r]);
+                }
             }
         }
     }
@@ -1112,7 +1124,7 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
     float o_acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const int i = el0 + ((tid + u * kChanThreads) >> lgTP), sub = tid & (TP - 1);
+        const int i = el0 + ((tid + u * NT) >> lgTP), sub = tid & (TP - 1);
         if (i < el1) {
             const int g = i / s.d;
             const float mg = mfin[g];
@@ -1130,11 +1142,11 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
             o_acc[u] = v;
         }
     }
-    consumer_sync();
-    fft_run<2, LS, LS, true>(fbuf, fb, nq * nh, twf, tid);
+    __syncthreads();
+    fft_run<2, LS, LS, true, 1, NT>(fbuf, fb, nq * nh, twf, tid);
     // (with few bins the channel pairs of a bin go to neighbouring lanes, whose sums are added in a fixed order)
-    const int lg_q = split_pairs(S / 2 * nh, nq), nq_t = nq >> lg_q;
-    for (int i = tid; i < ((S / 2) * nh) << lg_q; i += kChanThreads) {      // (whole warps: S is a multiple of 32 bins and pairs of them)
+    const int lg_q = split_pairs(S / 2 * nh, nq, NT), nq_t = nq >> lg_q;
+    for (int i = tid; i < ((S / 2) * nh) << lg_q; i += NT) {      // (whole warps: S is a multiple of 32 bins and pairs of them)
         const int bi = i >> lg_q, qs0 = (i & ((1 << lg_q) - 1)) * nq_t, g = bi >> (LS - 1), pr = bi & (S / 2 - 1), m = pr, mc = pr == 0 ? S / 2 : S - pr;
         float2 zm = make_float2(0.f, 0.f), zc = zm;
         if (m < s.k || mc < s.k)
@@ -1178,7 +1190,7 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
     const float inv_T = __int_as_float((127 << 23) - ((31 - __clz(s.T)) << 23));      // T is a power of two
     const float w_gen = s.norm == FA_NORM_PAPER ? 1.0f / (float)s.k : 2.f * inv_T, w_0 = s.norm == FA_NORM_PAPER ? w_gen : inv_T, w_1 = s.norm == FA_NORM_PAPER ? w_gen : 0.f;
     const int n_rows = m1 - m0;
-    for (int x = tid; x < (n_rows >> 1) * nh; x += kChanThreads) {          // (rows in pairs, cos and sin of a frequency)
+    for (int x = tid; x < (n_rows >> 1) * nh; x += NT) {          // (rows in pairs, cos and sin of a frequency)
         const int g = x / (n_rows >> 1), r = 2 * (x - g * (n_rows >> 1)), m = m0 + r;
         const float2 v = CL == 1 ? *reinterpret_cast<const float2*>(z_s + g * s.M + m) : sum_peers2(smem_addr(z_s + g * s.M + m), CL);
         zw_s[r * 4 + g] = v.x * (m == 0 ? w_0 : w_gen);
@@ -1190,14 +1202,19 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
     for (int g = 0; g < 4; ++g) acc4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int rg = tid / nv, vcol = tid - rg * nv;
     const float4 y = j_push >= 0 ? *reinterpret_cast<const float4*>(xc + 4 * vcol) : make_float4(0.f, 0.f, 0.f, 0.f);      // (the thread's columns are the same in every row)
-    for (int i = 0; i < rs.n_chunk; i += 2) {              // two stages at a time
-        const float* xs0 = rs.wait(fail, c.status);
-        const float* xs1 = i + 1 < rs.n_chunk ? rs.wait(fail, c.status) : xs0;
-        const int first = i * kStageRows, rows = min(2 * kStageRows, rs.rows - first);
+    constexpr int SP = NT / 128;                           // stages at a time: the thread's chain through them is paid once
+    for (int i = 0; i < rs.n_chunk; i += SP) {
+        const float* xs[SP];
+#pragma unroll
+        for (int u = 0; u < SP; ++u) xs[u] = i + u < rs.n_chunk ? rs.wait(u, fail, c.status) - u * kStageRows * s.dcv : nullptr;
+        const int first = i * kStageRows, rows = min(SP * kStageRows, rs.rows - first);
         if (rg < nrg) {
 #pragma unroll 4
             for (int r = rg; r < rows; r += nrg) {
-                float4 x = *reinterpret_cast<const float4*>((r < kStageRows ? xs0 + r * s.dcv : xs1 + (r - kStageRows) * s.dcv) + 4 * vcol);
+                const float* xr = xs[0];
+#pragma unroll
+                for (int u = 1; u < SP; ++u) if (r >= u * kStageRows) xr = xs[u];
+                float4 x = *reinterpret_cast<const float4*>(xr + r * s.dcv + 4 * vcol);
                 if (j_push >= 0) {
                     const float f = f_s[first + r];
                     x.x = fmaf(f, y.x, x.x); x.y = fmaf(f, y.y, x.y); x.z = fmaf(f, y.z, x.z); x.w = fmaf(f, y.w, x.w);
@@ -1216,14 +1233,15 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
                 }
             }
         }
-        rs.done(i, 2, tid);
+        rs.next(SP);
+        rs.done(i, SP, tid);
     }
     if (rg < nrg) {
 #pragma unroll
         for (int g = 0; g < 4; ++g) if (g < nh) *reinterpret_cast<float4*>(ps_s + (rg * nh + g) * s.dcv + 4 * vcol) = acc4[g];
     }
     __syncthreads();
-    for (int i = tid; i < nh * s.dcv; i += kChanThreads) {
+    for (int i = tid; i < nh * s.dcv; i += NT) {
         float v = 0.f;
 #pragma unroll 8
         for (int x = 0; x < nrg; ++x) v += ps_s[x * nh * s.dcv + i];
@@ -1232,7 +1250,7 @@ __global__ void __launch_bounds__(kChanThreads, outer_ctas(LS)) chan_out_kernel(
     cluster_meet(CL);                                      // all shares of o^c are there
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const int i = el0 + ((tid + u * kChanThreads) >> lgTP);
+        const int i = el0 + ((tid + u * NT) >> lgTP);
         float v = o_acc[u];
         for (int o = 1; o < TP; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (i < el1 && (tid & (TP - 1)) == 0) {
@@ -1267,7 +1285,7 @@ size_t in_smem(const Dims& s, int ls, const ChanPlan& m) {
                             (((s.M + m.nz - 1) / m.nz + 5) & ~3) + 2 * ((s.k + 1) & ~1) + 4 * s.d + (fft > stage ? fft : stage)) + 64;
 }
 size_t out_smem(const Dims& s, int ls, const ChanPlan& m) {
-    const size_t fft = (size_t)m.nq * m.nh * pf_size(2 << ls), ps = (size_t)kChanThreads * 4 * m.nh;
+    const size_t fft = (size_t)m.nq * m.nh * pf_size(2 << ls), ps = (size_t)outer_threads(ls) * 4 * m.nh;
     return sizeof(float) * (20 + ((2 * (tw_total(ls) + 1) + 3) & ~3) + (size_t)m.nh * s.M + ((2 * m.nq * s.k + 3) & ~3) + 8 + 5 * s.dcv +
                             5 * (size_t)(((s.M + m.nz - 1) / m.nz + 5) & ~3) + ((s.d + 7) & ~7) / 2 + 2 * ((s.k + 1) & ~1) + (size_t)m.st_out * kStageRows * s.dcv + (fft > ps ? fft : ps)) + 64;
 }
@@ -1295,11 +1313,13 @@ cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, siz
 
 }  // namespace
 
-// As many stages of the outer kernels' rows as a CTA's rows take and the limit of shared memory holds, two at least.
+// (as many as the threads of a CTA take at a time)
+static int least_stages(int log2S) { return outer_threads(log2S) / 128; }
+// As many stages of the outer kernels' rows as a CTA's rows take and the limit of shared memory holds.
 static void fit_stages(const Dims& s, int log2S, size_t limit, ChanPlan* m) {
     auto fits = [&]() { return in_smem(s, log2S, *m) <= limit && out_smem(s, log2S, *m) <= limit; };
     const int chunks = (s.M / m->nz + 2 + kStageRows - 1) / kStageRows, most = chunks < kMaxRowStages ? chunks : kMaxRowStages;
-    m->st_in = m->st_out = 2;
+    m->st_in = m->st_out = least_stages(log2S);
     for (; m->st_in < most; ++m->st_in) { ++m->st_in; const bool ok = fits(); --m->st_in; if (!ok) break; }
     for (; m->st_out < most; ++m->st_out) { ++m->st_out; const bool ok = fits(); --m->st_out; if (!ok) break; }
 }
@@ -1359,12 +1379,12 @@ bool plan_channels(const Dims& s, int log2S, int sms, ChanPlan* m) {
     // times that for a job in one CTA (32 jobs of 2048 coefficients: 35 us a kernel in one wave of clusters of four, 55 in two of eight)
     auto fits = [&](size_t limit) { return in_smem(s, log2S, *m) <= limit && out_smem(s, log2S, *m) <= limit; };
     constexpr size_t kHalf = 112 * 1024, kAll = 226 * 1024;
-    m->st_in = m->st_out = 2;
+    m->st_in = m->st_out = least_stages(log2S);
     int best_nz = 0, occ = 0;
     double least = 0;
     for (m->nz = 8; m->nz >= 1; m->nz /= 2) {
         m->nq = kMR / 2 / m->nz;
-        const int fit = fits(kHalf) ? 2 : fits(kAll) ? 1 : 0;
+        const int fit = fits(kHalf) && outer_ctas(log2S) > 1 ? 2 : fits(kAll) ? 1 : 0;
         if (!fit) continue;
         const long long held = (long long)(m->nz == 8 ? 15 : m->nz == 4 ? 33 : m->nz == 2 ? 74 : 148) * sms / 148 * fit;
         const double cost = (double)((jobs + held - 1) / held) * (1.0 + 4.0 / m->nz);
@@ -1402,7 +1422,7 @@ static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, co
     // several layers, more CTAs than two to an SM: fewer stages each, so that three fit (the sums do not depend on the number of stages)
     constexpr size_t kThird = 74 * 1024;
     if (outer_ctas(LS) == 3 && (long long)n * s.B * s.Hkv * m.n_pass * m.nz > 2 * sm_count()) {
-        m.st_in = m.st_out = 2;
+        m.st_in = m.st_out = least_stages(LS);
         if (in_smem(s, LS, m) <= kThird && out_smem(s, LS, m) <= kThird) fit_stages(s, LS, kThird, &m);
         else m = one;
     }
@@ -1420,14 +1440,14 @@ static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, co
         if ((s.l_init > 0 && !ok_i) || (s.l_local > 0 && !ok_l)) return cudaErrorInvalidValue;
         if (!mid_map(&t.km, c.k_mid, s, s.nfk) || !mid_map(&t.vm, c.v_mid, s, s.nfv)) return cudaErrorInvalidValue;
     }
-    cudaError_t err = m.hp == 2 ? launch_chained(chan_in_kernel<LS, 2>, cg, dim3(kChanThreads), in_smem(s, LS, m), m.nz, st, s, m, call)
-                                : launch_chained(chan_in_kernel<LS, 4>, cg, dim3(kChanThreads), in_smem(s, LS, m), m.nz, st, s, m, call);
+    auto launch_in = [&](auto nh) { return launch_chained(chan_in_kernel<LS, decltype(nh)::value>, cg, dim3(outer_threads(LS)), in_smem(s, LS, m), m.nz, st, s, m, call); };
+    cudaError_t err = m.nh == 1 ? launch_in(std::integral_constant<int, 1>{}) : m.nh == 2 ? launch_in(std::integral_constant<int, 2>{}) : launch_in(std::integral_constant<int, 4>{});
     if (err != cudaSuccess) return err;
     *begun = true;
     err = m.hp == 2 ? launch_chained(chan_main_kernel<2>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, maps, s, m, call)
                     : launch_chained(chan_main_kernel<4>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, maps, s, m, call);
     if (err != cudaSuccess) return err;
-    return launch_chained(chan_out_kernel<LS>, cg, dim3(kChanThreads), out_smem(s, LS, m), m.nz, st, s, m, call);
+    return launch_chained(chan_out_kernel<LS>, cg, dim3(outer_threads(LS)), out_smem(s, LS, m), m.nz, st, s, m, call);
 }
 
 // The decode calls of n layers of one layout, with k_new / v_new (not null; one pass only) each behind the push of Eq.5.  Several layers do not touch

@@ -354,14 +354,14 @@ __host__ __device__ constexpr int tw_total(int LS) { return tw_offset(LS, 0); }
 // One in-place pass of radix R = 2^RL over sub-transforms of length 2^LL, for nb transforms of
 // length 2^LS held in consecutive buffers.  DIF: butterfly, then twiddle the outputs; DIT:
 // twiddle the inputs, then butterfly.  Twiddles are stored [q - 1][j] as splat pairs (wr, wi).
-template <int GH, int LS, int LL, bool DIT>
+template <int GH, int LS, int LL, bool DIT, int NT = kConsumers>
 __device__ __forceinline__ void fft_pass(float* fbuf, int fb_floats, int nb, const float* twf, int tid) {
     constexpr int N = GH / 2;
     constexpr int RL = radix_log2(LL), R = 1 << RL;
     constexpr int STL = LL - RL, PERL = LS - RL;          // log2 butterflies per sub-transform / per transform
     constexpr bool kTw = LL > RL;
     constexpr int kTwOff = tw_offset(LS, LL);
-    for (int item = tid; item < (nb << PERL); item += kConsumers) {
+    for (int item = tid; item < (nb << PERL); item += NT) {
         const int ci = item >> PERL, rest = item & ((1 << PERL) - 1);
         const int blk = rest >> STL, j = rest & ((1 << STL) - 1);
         float* base = fbuf + ci * fb_floats;
@@ -394,19 +394,19 @@ __device__ __forceinline__ void fft_pass(float* fbuf, int fb_floats, int nb, con
 
 // The passes of the transform except the one over the shortest sub-transforms (the last of the score transform, the first
 // of the probability transform), which is done together with the softmax below; each ends with a barrier.
-// (kConsumers threads take part: all consumer warps, or the transform group of the split kernel with its barrier BID)
-template <int GH, int LS, int LL, bool DIT, int BID = 1>
+// (NT threads take part: all consumer warps, or the transform group of the split kernel with its barrier BID)
+template <int GH, int LS, int LL, bool DIT, int BID = 1, int NT = kConsumers>
 __device__ __forceinline__ void fft_run(float* fbuf, int fb_floats, int nb, const float* twf, int tid) {
     constexpr int RL = radix_log2(LL);
     if constexpr (LL - RL > 0) {
         if constexpr (!DIT) {
-            fft_pass<GH, LS, LL, false>(fbuf, fb_floats, nb, twf, tid);
-            consumer_sync<kConsumers, BID>();
-            fft_run<GH, LS, LL - RL, false, BID>(fbuf, fb_floats, nb, twf, tid);
+            fft_pass<GH, LS, LL, false, NT>(fbuf, fb_floats, nb, twf, tid);
+            consumer_sync<NT, BID>();
+            fft_run<GH, LS, LL - RL, false, BID, NT>(fbuf, fb_floats, nb, twf, tid);
         } else {
-            fft_run<GH, LS, LL - RL, true, BID>(fbuf, fb_floats, nb, twf, tid);
-            fft_pass<GH, LS, LL, true>(fbuf, fb_floats, nb, twf, tid);
-            consumer_sync<kConsumers, BID>();
+            fft_run<GH, LS, LL - RL, true, BID, NT>(fbuf, fb_floats, nb, twf, tid);
+            fft_pass<GH, LS, LL, true, NT>(fbuf, fb_floats, nb, twf, tid);
+            consumer_sync<NT, BID>();
         }
     }
 }
