@@ -11,9 +11,9 @@
 //      the prefill come in by TMA beside it and a lane sums the squares of its dim's differences.
 // All factors carry 2^-17 (two bf16 numbers, three products), where the direct reconstruction (fa_select_tc.cu) rounds basis and coefficients
 // to bf16: the floor under the reported errors falls from 1e-6 to 1e-9 of a dimension's mean square.
-// What bounds it: the third kernel HBM and the shared-memory reads of its differences (34 us for the 134 MB of 8 heads, 32 K tokens, ncu, cold),
-// the second its loads of 64 KB a stage against 1536 cycles of products (34 us for sixteen stages on 88 SMs, cold).  The whole selection of that
-// prompt, 1024 coefficients: 246 us with the reconstruction over coefficient rows (166 of them), 133 us here.
+// What bounds it: the third kernel HBM and the shared-memory reads of its differences (31 us for the 134 MB of 8 heads, 32 K tokens), the second its
+// loads (every tile of four pairs reads all of a head's a and b: 92 MB through L2) beside 24.6 K cycles of products on 88 SMs (30 us).  The whole
+// selection of that prompt, 1024 coefficients: 246 us with the reconstruction over coefficient rows (166 of them), 131 us here.
 #include "fa_moments.cuh"
 
 namespace fa {
@@ -22,12 +22,13 @@ namespace {
 using namespace mom;
 
 constexpr int kPairs = 4;              // pairs of blocks to a tile of the second kernel
-constexpr int kKn = 32;                // frequencies per stage
-constexpr int kBoxB = kKn * 128;       // [32 frequencies x 64 dims]
-constexpr int kTileA = 128 * 128;      // [128 rows x (32 hi, 32 lo)]
+constexpr int kKn = 16;                // frequencies per stage
+constexpr int kBoxB = kKn * 128;       // [16 frequencies x 64 dims]
+constexpr int kTileA = 128 * 128;      // [128 rows x (Re hi, Re lo, Im hi, Im lo of the 16)]
+constexpr int kBoxY = 32 * 128;        // [32 moments x 64 dims]
 constexpr int kGenWarpsE = 8;
 constexpr int kThreadsE = 64 + 32 * kGenWarpsE;
-constexpr int kStagesE = 2;
+constexpr int kStagesE = 4;
 constexpr int kBoxX = 128 * kChunk * 2;        // [64 tokens x 64 dims] twice
 constexpr int kTileP = kChunk * 128;           // [64 tokens x (32 hi, 32 lo)]
 constexpr int kTileY = 16384;                  // hi, lo x two halves of 64 dims x [32 moments x 64 dims]
@@ -39,7 +40,7 @@ struct SelPlan {
     int R, n_blk, n_pair, nbx;         // tokens to a block, blocks of a row and pairs of them, 64-dim boxes of a head's K and V
     const float* coef_k;
     const float* coef_v;
-    char* ab;                          // [B][Hkv][k / 32][a hi, a lo, b hi, b lo][nbx][32][128 bytes, 128-byte swizzle]
+    char* ab;                          // [B][Hkv][k / 16][a hi, a lo, b hi, b lo][nbx][16][128 bytes, 128-byte swizzle]
     float* g;                          // [32][k]
     char* y;                           // [B][n_blk][Hkv][nbx / 2][hi, lo][2][32][128 bytes, 128-byte swizzle]
 };
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(256) rotate_kernel(Dims s, SelPlan p, int n_fa
 // grid (tiles of four pairs, Hkv, B).
 template <int D>
 __global__ void __launch_bounds__(kThreadsE, 1) expand_kernel(Dims s, SelPlan p, int32_t* status) {
-    constexpr int N = 2 * D, kNbx = N / 64, kB = 4 * kNbx * kBoxB, kStage = 2 * kTileA + kB;
+    constexpr int N = 2 * D, kNbx = N / 64, kB = 4 * kNbx * kBoxB, kStage = kTileA + kB;
     // A K-major, B MN-major
     constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     extern __shared__ unsigned char smem_unaligned[];
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(kThreadsE, 1) expand_kernel(Dims s, SelPlan p,
     const int p0 = blockIdx.x * kPairs, h = blockIdx.y, b = blockIdx.z, n_k = s.k / kKn;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
-        for (int i = 0; i < kStagesE; ++i) { mbar_init(full + i, kGenWarpsE + 1); mbar_init(empty + i, 1); }
+        for (int i = 0; i < kStagesE; ++i) { mbar_init(full + i, kGenWarpsE / kStagesE + 1); mbar_init(empty + i, 1); }
         mbar_init(acc_ready, 1);
         *fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(kThreadsE, 1) expand_kernel(Dims s, SelPlan p,
                 const int st = it % kStagesE;
                 if (!mbar_wait(empty + st, ((it / kStagesE) & 1) ^ 1, fail, status)) { live = false; break; }
                 mbar_expect_tx(full + st, (uint32_t)kB);
-                bulk_load(stage0 + (size_t)st * kStage + 2 * kTileA, src + (size_t)it * kB, (uint32_t)kB, full + st);
+                bulk_load(stage0 + (size_t)st * kStage + kTileA, src + (size_t)it * kB, (uint32_t)kB, full + st);
             }
             if (!live)                                     // a wait ran out: the copies under way land, or the bound is reached, first
                 for (int q = it < kStagesE ? 0 : it - kStagesE; q < it; ++q)
@@ -149,90 +150,97 @@ __global__ void __launch_bounds__(kThreadsE, 1) expand_kernel(Dims s, SelPlan p,
                 const int st = it % kStagesE;
                 if (!mbar_wait(full + st, (it / kStagesE) & 1, fail, status)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t a_addr = smem_u32(stage0 + (size_t)st * kStage), b_addr = a_addr + 2 * kTileA;
+                const uint32_t a_addr = smem_u32(stage0 + (size_t)st * kStage), b_addr = a_addr + kTileA;
 #pragma unroll
                 for (int ty = 0; ty < 2; ++ty)             // Re against a, Im against b
 #pragma unroll
                     for (int pr = 0; pr < 3; ++pr)         // hi hi, lo hi, hi lo
-#pragma unroll
-                        for (int ks = 0; ks < kKn / 16; ++ks)
-                            umma_bf16(tmem_base + ty * N, umma_desc(a_addr + ty * kTileA + (pr == 1 ? 64 : 0) + ks * 32, 1, 1024 >> 4),
-                                      umma_desc(b_addr + (2 * ty + (pr == 2 ? 1 : 0)) * kNbx * kBoxB + ks * 2048, kBoxB >> 4, 1024 >> 4), kIdesc,
-                                      (it > 0 || pr > 0 || ks > 0) ? 1u : 0u);
+                        umma_bf16(tmem_base + ty * N, umma_desc(a_addr + 64 * ty + (pr == 1 ? 32 : 0), 1, 1024 >> 4),
+                                  umma_desc(b_addr + (2 * ty + (pr == 2 ? 1 : 0)) * kNbx * kBoxB, kBoxB >> 4, 1024 >> 4), kIdesc, (it > 0 || pr > 0) ? 1u : 0u);
                 umma_commit(empty + st);
             }
             umma_commit(acc_ready);
         }
     } else {
-        // ---------------- generators: a warp has one pair and half of the moments, a lane two frequencies and eight moments ----------------
-        const int gw = warp - 2, q = gw & 3, np2 = lane & 15, sub = lane >> 4, r0 = 16 * (gw >> 2) + 4 * sub;      // moments r0 + i, r0 + 8 + i
-        const unsigned dist = (unsigned)(max(0, p.n_blk - 1 - 2 * (p0 + q)) * p.R), T2 = 2u * (unsigned)s.T;
+        // ---------------- generators: two warps to a stage, four stages in the making: a stage's chain (phases, products, the fence) is longer
+        // than its products take on the tensor cores.  A warp has two pairs, a lane two frequencies and eight moments ----------------
+        const int gw = warp - 2, np2 = lane & 7, sub = lane >> 3, q0 = 2 * (gw & 1);       // pairs q0, q0 + 1; moments 16 j + 4 sub + i
+        const unsigned T2 = 2u * (unsigned)s.T;
         const float inv_T = 1.0f / (float)s.T;
-        const uint32_t row0 = (uint32_t)((q * 32 + r0) >> 3) * 1024, word = (uint32_t)(np2 & 3) * 4;
-        const float* g0 = p.g + 2 * np2;
+        const uint32_t word = (uint32_t)(np2 & 3) * 4;
+        const float* g0 = p.g + 2 * np2 + (size_t)(4 * sub) * s.k;
         float2 g[2][4];
         auto fetch = [&](int it) {
 #pragma unroll
             for (int j = 0; j < 2; ++j)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) g[j][i] = *reinterpret_cast<const float2*>(g0 + (size_t)(r0 + 8 * j + i) * s.k + it * kKn);
+                for (int i = 0; i < 4; ++i) g[j][i] = *reinterpret_cast<const float2*>(g0 + (size_t)(16 * j + i) * s.k + it * kKn);
         };
-        fetch(0);
-        for (int it = 0; it < n_k; ++it) {
-            const int st = it % kStagesE;
-            float C[2], S[2];
+        const int st = gw >> 1;
+        uint32_t par = 1;
+        if (st < n_k) fetch(st);
+        for (int it = st; it < n_k; it += kStagesE, par ^= 1) {
+            float C[2][2], S[2][2];                        // [pair][frequency]
 #pragma unroll
-            for (int v = 0; v < 2; ++v) {                  // pi n dist / T, exact in integers
-                const float f = (float)(((unsigned)(it * kKn + 2 * np2 + v) * dist) % T2) * inv_T;
-                const float an = 3.14159265358979f * (f - (f >= 1.0f ? 2.0f : 0.0f));
-                C[v] = __cosf(an);
-                S[v] = __sinf(an);
+            for (int q = 0; q < 2; ++q) {
+                const unsigned dist = (unsigned)(max(0, p.n_blk - 1 - 2 * (p0 + q0 + q)) * p.R);
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {              // pi n dist / T, exact in integers
+                    const float f = (float)(((unsigned)(it * kKn + 2 * np2 + v) * dist) % T2) * inv_T;
+                    const float an = 3.14159265358979f * (f - (f >= 1.0f ? 2.0f : 0.0f));
+                    C[q][v] = __cosf(an);
+                    S[q][v] = __sinf(an);
+                }
             }
-            if (!mbar_wait(empty + st, ((it / kStagesE) & 1) ^ 1, fail, status)) break;
-            unsigned char* at = stage0 + (size_t)st * kStage + row0 + word;
+            if (!mbar_wait(empty + st, par, fail, status)) break;
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
+            for (int q = 0; q < 2; ++q)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {              // (r & 3) = i: i^r = 1, i, -1, -i
-                    const float x = (i & 2) ? -g[j][i].x : g[j][i].x, z = (i & 2) ? -g[j][i].y : g[j][i].y;
-                    uint32_t hr, lr, hm, lm;
-                    if (i & 1) {
-                        split_bf16(-x * S[0], -z * S[1], hr, lr);
-                        split_bf16(x * C[0], z * C[1], hm, lm);
-                    } else {
-                        split_bf16(x * C[0], z * C[1], hr, lr);
-                        split_bf16(x * S[0], z * S[1], hm, lm);
+                for (int j = 0; j < 2; ++j) {
+                    unsigned char* at = stage0 + (size_t)st * kStage + (((q0 + q) * 32 + 16 * j + 4 * sub) >> 3) * 1024 + word;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {          // (r & 3) = i: i^r = 1, i, -1, -i
+                        const float x = (i & 2) ? -g[j][i].x : g[j][i].x, z = (i & 2) ? -g[j][i].y : g[j][i].y;
+                        uint32_t w[4];                     // Re hi, Re lo, Im hi, Im lo
+                        if (i & 1) {
+                            split_bf16(-x * S[q][0], -z * S[q][1], w[0], w[1]);
+                            split_bf16(x * C[q][0], z * C[q][1], w[2], w[3]);
+                        } else {
+                            split_bf16(x * C[q][0], z * C[q][1], w[0], w[1]);
+                            split_bf16(x * S[q][0], z * S[q][1], w[2], w[3]);
+                        }
+                        const int r7 = (4 * sub + i) & 7;  // row & 7
+                        unsigned char* row = at + r7 * 128;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) *reinterpret_cast<uint32_t*>(row + (((2 * u + (np2 >> 2)) ^ r7) << 4)) = w[u];
                     }
-                    const int r7 = 4 * sub + i;            // row & 7
-                    unsigned char* row = at + j * 1024 + r7 * 128;
-                    const uint32_t ph = (uint32_t)(((np2 >> 2) ^ r7) << 4), pl = (uint32_t)((((np2 >> 2) + 4) ^ r7) << 4);
-                    *reinterpret_cast<uint32_t*>(row + ph) = hr;
-                    *reinterpret_cast<uint32_t*>(row + pl) = lr;
-                    *reinterpret_cast<uint32_t*>(row + kTileA + ph) = hm;
-                    *reinterpret_cast<uint32_t*>(row + kTileA + pl) = lm;
                 }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(full + st);
-            if (it + 1 < n_k) fetch(it + 1);
+            if (it + kStagesE < n_k) fetch(it + kStagesE);
         }
-        // ---------------- epilogue: a warp has a pair (lanes its moments) and half of the columns ----------------
+        // ---------------- epilogue: a warp has a pair (lanes its moments) and half of the columns.  A block's moments are put together in the idle
+        // ring and leave with bulk copies (stored by the lanes, every 16 bytes went to a line of its own: 16 K cycles) ----------------
         const bool ok = mbar_wait(acc_ready, 0, fail, status);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int lg = warp & 3, pp = p0 + lg, half = gw >> 2;
+        const int lg = warp & 3, pp = p0 + lg, half = (warp - 2) >> 2;
         if (ok && pp < p.n_pair) {
+            constexpr int kHalfBoxes = D / 64, kPart = kHalfBoxes * kBoxY;       // a half's 64-dim boxes; its hi or lo values
+            unsigned char* buf = stage0 + (warp - 2) * (2 * kPart);
             const int b_hi = p.n_blk - 1 - pp;
-            const size_t per_blk = (size_t)s.Hkv * (kNbx / 2) * kTileY;
-            char* y_hi = p.y + ((size_t)b * p.n_blk + b_hi) * per_blk + (size_t)h * (kNbx / 2) * kTileY;
-            char* y_lo = p.y + ((size_t)b * p.n_blk + pp) * per_blk + (size_t)h * (kNbx / 2) * kTileY;
+            for (int w = 0; w < (b_hi != pp ? 2 : 1); ++w) {                    // the block at +d, the one at -d
+                const float sa = w && (lane & 1) ? -1.f : 1.f, sb = w ? 1.f : -1.f;
+                if (w) {
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    __syncwarp();
+                }
 #pragma unroll 1
-            for (int c0 = half * D; c0 < (half + 1) * D; c0 += 32) {
-                float u[32], v[32];
-                tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)c0, u);
-                tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(N + c0), v);
-                const int bx = c0 >> 6;
-                const size_t off = (size_t)((bx >> 1) * 4 + (bx & 1)) * kBoxB + lane * 128;
-                auto put = [&](char* to, float sa, float sb) {       // sa (u + sb v)
+                for (int c0 = 0; c0 < D; c0 += 32) {
+                    float u[32], v[32];
+                    tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(half * D + c0), u);
+                    tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(N + half * D + c0), v);
+                    unsigned char* row = buf + (c0 >> 6) * kBoxY + lane * 128;
 #pragma unroll
                     for (int q4 = 0; q4 < 4; ++q4) {
                         uint32_t hi[4], lo[4];
@@ -241,15 +249,26 @@ __global__ void __launch_bounds__(kThreadsE, 1) expand_kernel(Dims s, SelPlan p,
                             const int e = 8 * q4 + 2 * x;
                             split_bf16(sa * (u[e] + sb * v[e]), sa * (u[e + 1] + sb * v[e + 1]), hi[x], lo[x]);
                         }
-                        const int piece = ((c0 & 63) >> 3) + q4;
-                        char* dst = to + off + ((piece ^ (lane & 7)) << 4);
-                        *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                        *reinterpret_cast<uint4*>(dst + 2 * kBoxB) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                        const int at = ((((c0 & 63) >> 3) + q4) ^ (lane & 7)) << 4;
+                        *reinterpret_cast<uint4*>(row + at) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                        *reinterpret_cast<uint4*>(row + kPart + at) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                     }
-                };
-                put(y_hi, 1.f, -1.f);
-                if (b_hi != pp) put(y_lo, (lane & 1) ? -1.f : 1.f, 1.f);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    char* y = p.y + (((size_t)b * p.n_blk + (w ? pp : b_hi)) * s.Hkv + h) * (size_t)(kNbx / 2) * kTileY;
+#pragma unroll
+                    for (int hl = 0; hl < 2; ++hl) {
+                        char* dst = D == 128 ? y + half * kTileY + hl * kPart : y + (2 * hl + half) * kPart;
+                        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(dst)), "r"(smem_u32(buf + hl * kPart)),
+                                     "r"(kPart)
+                                     : "memory");
+                    }
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
             }
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -384,7 +403,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) residual_kernel(const __grid_con
                     for (int pr = 0; pr < 3; ++pr)         // hi hi, lo hi, hi lo
 #pragma unroll
                         for (int ks = 0; ks < kMF / 16; ++ks)
-                            umma_bf16(tmem_base + (uint32_t)(a % kAccR) * kChunk, umma_desc(y_addr + (pr == 1 ? 2 * kBoxB : 0) + ks * 2048, kBoxB >> 4, 1024 >> 4),
+                            umma_bf16(tmem_base + (uint32_t)(a % kAccR) * kChunk, umma_desc(y_addr + (pr == 1 ? 2 * kBoxY : 0) + ks * 2048, kBoxY >> 4, 1024 >> 4),
                                       umma_desc(p_addr + (pr == 2 ? 64 : 0) + ks * 32, 1, 1024 >> 4), kIdesc, (pr > 0 || ks > 0) ? 1u : 0u);
                     umma_commit(acc_full + a % kAccR);
                 }
@@ -485,7 +504,7 @@ cudaError_t launch_select_mom_t(const Dims& s, const SelPlan& p, const void* K, 
     if (n_rot >= (1ll << 30) || items >= (1ll << 30)) return cudaErrorInvalidValue;
     cudaError_t err = launch_behind(rotate_kernel, dim3((unsigned)(n_rot + s.k / 32)), 256, 0, stream, s, p, s.k / 32);
     if (err != cudaSuccess) return err;
-    constexpr size_t smem_e = (size_t)kStagesE * (2 * kTileA + 4 * (2 * D / 64) * kBoxB) + 8 * (2 * kStagesE + 1) + 16 + 1024;
+    constexpr size_t smem_e = (size_t)kStagesE * (kTileA + 4 * (2 * D / 64) * kBoxB) + 8 * (2 * kStagesE + 1) + 16 + 1024;
     err = launch_behind(expand_kernel<D>, dim3((p.n_pair + kPairs - 1) / kPairs, s.Hkv, s.B), kThreadsE, smem_e, stream, s, p, status);
     if (err != cudaSuccess) return err;
     const int n_stages = residual_stages(s);
