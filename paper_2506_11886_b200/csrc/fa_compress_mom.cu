@@ -933,11 +933,11 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     if (n_teams < 1) n_teams = 1;
     if (n_teams > kMaxTeamsP) n_teams = kMaxTeamsP;
     if (n_teams > total) n_teams = (int)total;
-    // Equal cost per team: a segment costs its blocks plus kEpi (epilogue and refill, in blocks); the smallest budget with
-    // which the walk covers all positions in n_teams teams, by bisection.
+    // Equal cost per team: a segment costs its positions plus its epilogue and refill, kEpi where its sums are added to others', kWhole where a unit is
+    // taken whole and they are stored; the smallest budget with which the walk covers all positions in n_teams teams, by bisection.
     MomCuts cuts = {};
-    constexpr long long kEpi = FOLD ? 16 : 6, kMinSeg = 2;
-    auto unit_end_of = [&](long long pos) {
+    constexpr long long kEpi = FOLD ? 16 : 6, kWhole = FOLD ? 9 : 4, kMinSeg = 2;
+    auto unit_of = [&](long long pos, long long* begin) {  // returns its end
         long long first = 0, nblk = rows.nblk;
         if (RAG) {
             int b = 0;
@@ -945,7 +945,8 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
             first = (long long)rows.first[b] * n_hg;
             nblk = (long long)rows.first[b + 1] - rows.first[b];
         }
-        return first + ((pos - first) / nblk + 1) * nblk;
+        *begin = first + (pos - first) / nblk * nblk;
+        return *begin + nblk;
     };
     auto walk = [&](long long budget, uint32_t* start) {
         long long pos = 0;
@@ -953,8 +954,15 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
         for (; t < n_teams && pos < total; ++t) {
             if (start) start[t] = (uint32_t)pos;
             long long left = budget;
-            while (pos < total && left >= kEpi + kMinSeg) {
-                const long long unit_end = unit_end_of(pos);
+            while (pos < total && left >= kWhole + kMinSeg) {
+                long long unit_begin;
+                const long long unit_end = unit_of(pos, &unit_begin);
+                if (pos == unit_begin && unit_end - pos + kWhole <= left) {
+                    pos = unit_end;
+                    left -= unit_end - unit_begin + kWhole;
+                    continue;
+                }
+                if (left < kEpi + kMinSeg) break;
                 long long take = unit_end - pos < left - kEpi ? unit_end - pos : left - kEpi;
                 if (unit_end - pos - take > 0 && unit_end - pos - take < kMinSeg) take = unit_end - pos - kMinSeg;
                 if (take <= 0) break;
