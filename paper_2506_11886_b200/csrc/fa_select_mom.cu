@@ -32,7 +32,7 @@ constexpr int kStagesE = 4;
 constexpr int kBoxX = 128 * kChunk * 2;        // [64 tokens x 64 dims] twice
 constexpr int kTileP = kChunk * 128;           // [64 tokens x (32 hi, 32 lo)]
 constexpr int kTileY = 16384;                  // hi, lo x two halves of 64 dims x [32 moments x 64 dims]
-constexpr int kYStages = 2, kAccR = 8, kErrSets = 4, kErrWarps = 4 * kErrSets;
+constexpr int kYStages = 2, kAccR = 8 /* (a multiple of the sets) */, kErrSets = 4, kErrWarps = 4 * kErrSets;
 constexpr int kThreadsR = 64 + 32 * kErrWarps;
 
 // Sizes of one call.
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) residual_kernel(const __grid_con
                                       umma_desc(p_addr + (pr == 2 ? 64 : 0) + ks * 32, 1, 1024 >> 4), kIdesc, (pr > 0 || ks > 0) ? 1u : 0u);
                     umma_commit(acc_full + a % kAccR);
                 }
-                if (live) umma_commit(y_empty + ys);
+                if (live && i + kYStages * (int)gridDim.x < n_items) umma_commit(y_empty + ys);      // (else nobody would wait for it: the CTA could end first)
             }
         }
     } else {
@@ -471,10 +471,13 @@ __global__ void __launch_bounds__(kThreadsR, 1) residual_kernel(const __grid_con
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 size_t ab_bytes(const Dims& s) { return up256((size_t)s.B * s.Hkv * s.k * 4 * 2 * s.d * 2); }
 size_t g_bytes(const Dims& s) { return up256((size_t)kMF * s.k * 4); }
-size_t residual_fixed(const Dims& s) { return (size_t)block_tokens(s) / kChunk * kTileP + kYStages * kTileY + 8 * (2 * 8 + 2 * kYStages + 2 * kAccR) + 64 + 1024; }
+size_t residual_fixed(const Dims& s) { return (size_t)block_tokens(s) / kChunk * kTileP + kYStages * kTileY + 8 * (2 * 2 * kErrSets + 2 * kYStages + 2 * kAccR) + 64 + 1024; }
+// Stages of the prefill's ring: a multiple of the sets of warps that take them in turn, so that a stage always falls to the same set.  (A set
+// waits for the boxes that it takes only.  Were a stage's box before the one that it waits for another set's and late, the barrier's
+// parity would still be that of two boxes ago and the wait would fall through.)
 int residual_stages(const Dims& s) {
     const int n = (int)((227 * 1024 - residual_fixed(s)) / kBoxX);
-    return n > 8 ? 8 : n;
+    return n >= 2 * kErrSets ? 2 * kErrSets : n >= kErrSets ? kErrSets : 0;
 }
 
 template <typename... Params, typename... Args>
@@ -516,7 +519,7 @@ cudaError_t launch_select_mom_t(const Dims& s, const SelPlan& p, const void* K, 
 
 // Bytes of scratch of the reconstruction by block moments (0: it does not serve this layout).
 size_t select_mom_bytes(const Dims& s, int dtype) {
-    if (dtype != FA_BF16 || (s.d != 64 && s.d != 128) || !compress_mom_supported(s) || residual_stages(s) < 4) return 0;
+    if (dtype != FA_BF16 || (s.d != 64 && s.d != 128) || !compress_mom_supported(s) || residual_stages(s) == 0) return 0;
     const size_t n_blk = (size_t)blocks_of(s.max_mid, block_tokens(s));
     return ab_bytes(s) + g_bytes(s) + n_blk * s.B * s.Hkv * (2 * s.d / 128) * kTileY;
 }

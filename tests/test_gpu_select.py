@@ -86,6 +86,8 @@ def test_tensor_core_reconstruction_against_oracle_and_fp32_path(Hkv, d, M, L):
     dict(L=4096 + 36, M=256, T=4096, Hkv=1),              # period full
     dict(L=2500, M=512, T=16384, d=64),                   # K and V in one item
     dict(L=2222, M=256, T=65536, L_init=0, L_local=1),    # the longest blocks
+    dict(L=16000, M=256, T=16384, B=1, Hkv=32),           # and many of them to a CTA: a ring of four stages, the sets of warps apart
+    dict(L=9000, M=512, T=16384, B=1, Hkv=16),            # a ring of eight
     dict(L=1500, M=256, T=5000),                          # period not a power of two
     dict(L=1500, M=256, T=4096, norm=1),                  # the paper's weights
 ])
