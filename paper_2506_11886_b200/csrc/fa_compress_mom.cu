@@ -21,10 +21,11 @@
 // second the tensor cores (1152 cycles of products a position and pair) plus 20 K cycles a segment, at the rate at which L2 adds vectors of
 // floats (four rows of 128 K tokens: 242 K cycles, 69 % of them on the tensor cores).
 // Direct contraction against this path, in us: six layers of 32 K tokens, 1024 rows: 701 -> 374, with one projection for all 333, folded 292, the
-// moments of all layers in one launch and the windows beside the projection 277; 128 K tokens, batch 4, 2048 rows: 3207 -> 777, folded 674; six ragged
+// moments of all layers in one launch and the windows beside the projection 277; 128 K tokens, batch 4, 2048 rows: 3207 -> 777, folded 664; six ragged
 // rows of 3 to 12 K tokens, 512 rows: 123 -> 85, folded 79, windows beside it 73; 4 K tokens of 256 heads, 256 rows (T / k = 32, blocks of 192
 // tokens, too few frequencies to fold): 231 -> 221, windows beside it 199.  The projection of the four rows of 128 K tokens alone:
 // 275 -> 162.  Relative error of the coefficients 4e-6 against 2.4e-4.
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -769,10 +770,10 @@ struct WinIn {
     int n;
 };
 __global__ void __launch_bounds__(32) windows_kernel(const __grid_constant__ WinIn in, Dims s, int Lall, const __grid_constant__ RowLens lens, int n_init_ch,
-                                                     int n_ch, int per_cta, int n_items) {
+                                                     int n_ch, int per_cta, int n_items, int n_stages) {
     extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kWinStages * kWinBytes);
-    volatile int* fail = reinterpret_cast<volatile int*>(full + kWinStages);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + n_stages * kWinBytes);
+    volatile int* fail = reinterpret_cast<volatile int*>(full + n_stages);
     const int lane = threadIdx.x;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (blockIdx.x == 0)
@@ -786,7 +787,7 @@ __global__ void __launch_bounds__(32) windows_kernel(const __grid_constant__ Win
             st[4] = 0;                                     // append ticket
         }
     if (lane == 0) {
-        for (int i = 0; i < kWinStages; ++i) mbar_init(full + i, 1);
+        for (int i = 0; i < n_stages; ++i) mbar_init(full + i, 1);
         *fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // box i: head fastest, then the chunk of the windows, side, batch row, layer
@@ -812,16 +813,16 @@ __global__ void __launch_bounds__(32) windows_kernel(const __grid_constant__ Win
         const uint32_t bytes = (uint32_t)(64 * s.d * 2);
         auto load = [&](int i) {
             const Box x = box(i);
-            const int st = (i - i0) % kWinStages;
+            const int st = (i - i0) % n_stages;
             if (x.rows <= 0) { mbar_arrive(full + st); return; }
             mbar_expect_tx(full + st, bytes);
             tma_load_4d(smem + st * kWinBytes, x.side ? &in.v[x.layer] : &in.k[x.layer], 0, x.h, x.tok, x.b, full + st);
         };
-        for (int i = i0; i < i1 && i < i0 + kWinStages - 1; ++i) load(i);
+        for (int i = i0; i < i1 && i < i0 + n_stages - 1; ++i) load(i);
         int i = i0;
         for (; i < i1; ++i) {
-            const int st = (i - i0) % kWinStages;
-            if (!mbar_wait(full + st, ((i - i0) / kWinStages) & 1, fail, in.c[0].status)) break;
+            const int st = (i - i0) % n_stages;
+            if (!mbar_wait(full + st, ((i - i0) / n_stages) & 1, fail, in.c[0].status)) break;
             const Box x = box(i);
             if (x.rows > 0)
                 asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(x.dst)), "r"(smem_u32(smem + st * kWinBytes)),
@@ -829,11 +830,11 @@ __global__ void __launch_bounds__(32) windows_kernel(const __grid_constant__ Win
                              : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");       // the copy before has read its stage
-            if (i + kWinStages - 1 < i1) load(i + kWinStages - 1);
+            if (i + n_stages - 1 < i1) load(i + n_stages - 1);
         }
         if (i < i1)                                        // a wait ran out: the boxes under way land, or the bound is reached, first
-            for (int q = i; q < i1 && q < i + kWinStages - 1; ++q)
-                for (uint32_t n = 0; n < (1u << 16) && !mbar_try_wait(full + (q - i0) % kWinStages, ((q - i0) / kWinStages) & 1); ++n) { }
+            for (int q = i; q < i1 && q < i + n_stages - 1; ++q)
+                for (uint32_t n = 0; n < (1u << 16) && !mbar_try_wait(full + (q - i0) % n_stages, ((q - i0) / n_stages) & 1); ++n) { }
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         if (*fail)
             for (int l = 1; l < in.n; ++l) in.c[l].status[0] = in.c[0].status[0];
@@ -844,15 +845,35 @@ __global__ void __launch_bounds__(32) windows_kernel(const __grid_constant__ Win
 
 int npad_of(const Dims& s) { return (s.dck + s.dcv + 31) / 32 * 32; }
 
-// Whether the blocks are taken in pairs about the middle of a row: the projection then takes 256 frequencies at a time.
-bool folds(const Dims& s) { return s.k % 256 == 0; }
+// Whether the blocks may be taken in pairs about the middle of a row: the projection then takes 256 frequencies at a time.
+bool can_fold(const Dims& s) { return s.k % 256 == 0; }
+// Whether a launch does so: n_pairs of blocks of all rows and layers.  Pairs are coarser work: SMs without one while the last of the moments are
+// formed, 256 frequencies to a segment.  That costs 2 to 4 us, which the halved products regain from some five and a half positions to a CTA pair on (between
+// 400 and 430 it goes either way).  us, plain / folded: 512 coefficients, 8 heads: 320 positions 59/60, 336 34/37, 416 72/76, 456 57/56, 520 89/85, 608
+// 69/66, six ragged rows 424 79/77;  32 heads: 320 50/55, 352 67/69, 416 75/80, 512 85/83, 608 71/67;  1024 coefficients, 8 heads: 336 42/42, 400 46/44,
+// 480 50/47, 656 69/66, 1312 115/101.
+constexpr long long kFoldPositions = 400;
+bool folds(const Dims& s, long long n_pairs) { return can_fold(s) && n_pairs * s.Hkv * (s.k / 256) >= kFoldPositions; }
+
+// The projection's stages leave room for a CTA of the windows kernel beside it: one of three stages, or of two where the projection would otherwise
+// have two itself (more than 192 columns, folded: 22 us instead of 16 for a head group of 256 columns, 512 coefficients and 3600 tokens).
+constexpr size_t kProjectFixed = 8 * (3 * kStagesP + 2) + 16 + 1024;
+size_t project_stage_bytes(const Dims& s, bool fold) {
+    return fold ? 2 * kABytesP + (size_t)npad_of(s) * 128 : kABytesP + (size_t)(s.Hkv % 2 == 0 ? 2 : 1) * (npad_of(s) / 2) * 128;
+}
+int project_fit(const Dims& s, bool fold, int win_stages) {
+    const int n = (int)((227 * 1024 - (win_stages * kWinBytes + 1280) - kProjectFixed) / project_stage_bytes(s, fold));
+    return n < kStagesP ? n : kStagesP;
+}
+int windows_stages(const Dims& s) { return project_fit(s, can_fold(s), kWinStages) >= 3 ? kWinStages : kWinStages - 1; }
+int project_stages(const Dims& s, bool fold) { return project_fit(s, fold, windows_stages(s)); }
 
 size_t mom_tables(const Dims& s) { return (size_t)s.Hkv * (2 * s.d + s.nfk + s.nfv); }
-size_t mom_smem_fixed(const Dims& s, int n_layers = 1) {      // everything but the stages, the slack of the alignment among it
-    return (size_t)block_tokens(s) / kChunk * kHChunk + (folds(s) ? 2 : 1) * 128 * 4 * kMF + 8 * (3 * 16 + 2 * kAcc) + 16 + (size_t)n_layers * mom_tables(s) + 64 + 1024;
+size_t mom_smem_fixed(const Dims& s, bool fold, int n_layers) {      // everything but the stages, the slack of the alignment among it
+    return (size_t)block_tokens(s) / kChunk * kHChunk + (fold ? 2 : 1) * 128 * 4 * kMF + 8 * (3 * 16 + 2 * kAcc) + 16 + (size_t)n_layers * mom_tables(s) + 64 + 1024;
 }
-int mom_stages(const Dims& s, int n_layers = 1) {
-    const long long left = 227 * 1024 - (long long)mom_smem_fixed(s, n_layers);
+int mom_stages(const Dims& s, bool fold, int n_layers) {
+    const long long left = 227 * 1024 - (long long)mom_smem_fixed(s, fold, n_layers);
     const int n = (int)(left / kChunkBytes);
     return n > 16 ? 16 : n;
 }
@@ -860,8 +881,8 @@ int mom_stages(const Dims& s, int n_layers = 1) {
 // chained: behind a kernel of the same call (else all work in front of it on the stream has ended when it starts, so that it may write anything)
 template <int D, bool RAG, bool FOLD>
 cudaError_t launch_moments(const MomIn& in, const Dims& s, int L, const MomRows& rows, void* Y, bool wait_first, bool chained, cudaStream_t stream) {
-    const int n_stages = mom_stages(s, in.n);
-    const size_t smem = mom_smem_fixed(s, in.n) + (size_t)n_stages * kChunkBytes;
+    const int n_stages = mom_stages(s, FOLD, in.n);
+    const size_t smem = mom_smem_fixed(s, FOLD, in.n) + (size_t)n_stages * kChunkBytes;
     cudaError_t err = ensure_dynamic_smem(moments_kernel<D, RAG, FOLD>, smem);
     if (err != cudaSuccess) return err;
     const long long items = (long long)rows.total * s.Hkv * (D == 128 ? 2 : 1);
@@ -884,10 +905,9 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     MomLayers layers = {};
     layers.n = n_layers;
     for (int i = 0; i < n_layers; ++i) { layers.k[i] = c[i].coef_k; layers.v[i] = c[i].coef_v; layers.status[i] = c[i].status; }
-    const size_t stage = FOLD ? 2 * kABytesP + (size_t)npad_of(s) * 128 : kABytesP + (size_t)HP * (npad_of(s) / 2) * 128, fixed = 8 * (3 * kStagesP + 2) + 16 + 1024;
-    // (room for a CTA of the windows kernel beside it)
-    const int fit = (int)((227 * 1024 - (kWinStages * kWinBytes + 2048) - fixed) / stage), n_stages = fit < kStagesP ? fit : kStagesP;
-    const size_t smem = n_stages * stage + fixed;
+    const int n_stages = project_stages(s, FOLD);
+    // (more than half of an SM's: each CTA takes all of its tensor memory, a second one could only wait for that)
+    const size_t smem = std::max(n_stages * project_stage_bytes(s, FOLD) + kProjectFixed, (size_t)116 * 1024);
     cudaError_t err = ensure_dynamic_smem(moment_project_kernel<HP, RAG, FOLD>, smem);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
@@ -993,7 +1013,7 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
 bool compress_mom_supported(const Dims& s) {
     if (s.M % (2 * kBMp) != 0 || s.d > 128 || s.dck + s.dcv == 0) return false;
     if (block_tokens(s) < 3 * kChunk) return false;
-    if (mom_stages(s) < 5) return false;
+    if (mom_stages(s, can_fold(s), 1) < 5) return false;
     // phases n (2 j + R - 1) stay in 32 bits
     return (unsigned long long)(s.M / 2) * (2ull * (unsigned long long)s.T + 2ull * kMaxBlockTokens) < (1ull << 32);
 }
@@ -1002,12 +1022,12 @@ bool compress_mom_supported(const Dims& s) {
 size_t compress_mom_row_bytes(const Dims& s, int n_mid) {
     const int R = block_tokens(s);
     const int n = blocks_of(n_mid, R);
-    return (size_t)(folds(s) ? (n + 1) / 2 * 2 : n) * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
+    return (size_t)(can_fold(s) ? (n + 1) / 2 * 2 : n) * s.Hkv * (s.dck + s.dcv) * (4 * kMF);
 }
 
 static cudaError_t launch_rows(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
-                               int64_t sh, int L, MomRows rows, char* Y, bool wait_first, bool chained, cudaStream_t stream) {
-    const bool rag = rows.lens.n != 0, fold = folds(s);
+                               int64_t sh, int L, MomRows rows, bool fold, char* Y, bool wait_first, bool chained, cudaStream_t stream) {
+    const bool rag = rows.lens.n != 0;
     cudaError_t err;
     // Layers to a launch: as many as a sixth of the ring's room holds the tables of.  A launch of its own for each pays its start, its first loads
     // and its last items every time.
@@ -1048,7 +1068,14 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
     rows.R = block_tokens(s);
     rows.b0 = b0;
     rows.nb = nb;
-    auto positions = [&](int n_mid) { const int n = blocks_of(n_mid, rows.R); return folds(s) ? (n + 1) / 2 : n; };
+    auto pairs = [&](int n_mid) { return (blocks_of(n_mid, rows.R) + 1) / 2; };
+    long long n_pairs = 0;
+    for (int b = b0; b < b0 + nb; ++b) {
+        const int m = lens && lens->n == s.B ? mid_of(s, lens->len[b]) : mid_of(s, L);
+        if (!lens || !lens->n || m >= tc_min) n_pairs += pairs(m);
+    }
+    const bool fold = folds(s, n_pairs);
+    auto positions = [&](int n_mid) { return fold ? pairs(n_mid) : blocks_of(n_mid, rows.R); };
     if (lens && lens->n) {
         if (lens->n != s.B) return cudaErrorInvalidValue;
         rows.lens = *lens;
@@ -1067,7 +1094,7 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
         rows.total = rows.nblk * nb;
     }
     if (rows.total == 0) return cudaSuccess;
-    return launch_rows(s, &c, &K, &V, 1, sb, st, sh, L, rows, static_cast<char*>(Y), wait_first, chained, stream);
+    return launch_rows(s, &c, &K, &V, 1, sb, st, sh, L, rows, fold, static_cast<char*>(Y), wait_first, chained, stream);
 }
 
 // The same for all batch rows of up to kMomLayers layers of one shape: a moment kernel each, then one projection.  A projection
@@ -1080,11 +1107,12 @@ cudaError_t launch_compress_mom_layers(const Dims& s, const CacheDev* c, const v
     rows.R = block_tokens(s);
     rows.nb = s.B;
     rows.n_blk = blocks_of(mid_of(s, L), rows.R);
-    rows.nblk = folds(s) ? (rows.n_blk + 1) / 2 : rows.n_blk;
+    const bool fold = folds(s, (long long)(rows.n_blk + 1) / 2 * s.B * n_layers);
+    rows.nblk = fold ? (rows.n_blk + 1) / 2 : rows.n_blk;
     rows.total = rows.nblk * s.B;
     if (rows.total == 0) return cudaSuccess;
     if ((long long)rows.nblk * s.B * n_layers >= (1ll << 24)) return cudaErrorInvalidValue;
-    return launch_rows(s, c, K, V, n_layers, sb, st, sh, L, rows, static_cast<char*>(Y), wait_first, chained, stream);
+    return launch_rows(s, c, K, V, n_layers, sb, st, sh, L, rows, fold, static_cast<char*>(Y), wait_first, chained, stream);
 }
 
 // The windows and counters of layers whose middles launch_compress_mom(_layers) has enqueued in front, on the same stream.
@@ -1095,7 +1123,8 @@ cudaError_t launch_windows(const Dims& s, const CacheDev* c, const void* const* 
     // chunks of the longest windows of any row (a row's own may be fewer)
     const int n_init = L < s.l_init ? L : s.l_init, n_local = L - n_init < s.l_local ? L - n_init : s.l_local;
     const int n_init_ch = (n_init + 63) / 64, n_ch = n_init_ch + (n_local + 63) / 64;
-    const size_t smem = kWinStages * kWinBytes + 8 * kWinStages + 16;
+    const int n_stages = windows_stages(s);
+    const size_t smem = n_stages * kWinBytes + 8 * n_stages + 16;
     cudaError_t err = ensure_dynamic_smem(windows_kernel, smem);
     if (err != cudaSuccess) return err;
     for (int i = 0; i < n_layers; i += kMomLayers) {
@@ -1121,7 +1150,7 @@ cudaError_t launch_windows(const Dims& s, const CacheDev* c, const void* const* 
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        err = cudaLaunchKernelEx(&cfg, windows_kernel, in, s, L, rl, n_init_ch, n_ch > 0 ? n_ch : 1, (int)per, (int)items);
+        err = cudaLaunchKernelEx(&cfg, windows_kernel, in, s, L, rl, n_init_ch, n_ch > 0 ? n_ch : 1, (int)per, (int)items, n_stages);
         if (err != cudaSuccess) return err;
     }
     return cudaSuccess;

@@ -5,6 +5,8 @@ Bounds.  Both factors of the two products are held as two bf16 numbers: 2^-17 re
 truncated expansion (1.5e-5 at the edge of the band, 6e-7 rms) are below that; relative to the largest coefficient of a
 head 3e-5 covers four times their sum.  The direct contraction rounds its basis to bf16: 2^-9 a term, averaged over at
 least 1024 tokens, within the 1e-3 that the parity suite allows it."""
+import math
+
 import pytest
 import torch
 
@@ -56,16 +58,35 @@ def test_block_moments_against_oracle(kw):
     dict(L=2900, M=1024, T=32768, B=2),                   # two pairs of tiles
     dict(L=3000, M=512, T=10000),                         # period not a power of two
 ])
-def test_folded_blocks_against_oracle(kw):
-    shape = _shape(**{**dict(M=512, T=16384), **kw})
-    P = 1 if shape.T == 10000 else 8
-    pair, _ = make_pair(shape, seed=72, P=P, max_mid=min(shape.T, shape.L), algo=fa.FA_DECODE_DIRECT, freq="offgrid")
-    assert pair.check_state() <= MOMENT_REL
+def test_folded_blocks(kw):
+    """As many rows as it takes for blocks to be folded, against the definition in 64 bits; one row (blocks as they are) likewise; the
+    kept dims and windows exactly as by the order-fixed mode."""
+    one = _shape(**{**dict(M=512, T=16384), **kw})
+    P = 1 if one.T == 10000 else 8
+    n0, n_mid = one.L_init, one.L - one.L_init - one.L_local
+    pairs = -(-n_mid // (6 * one.T // (one.M // 2) // 64 * 64)) + 1 >> 1
+    folded = one.with_(B=-(-400 * 512 // (pairs * one.Hkv * one.M)))
+    ang = ((torch.arange(n_mid, device="cuda")[None] * torch.arange(one.M // 2, device="cuda")[:, None]) % one.T).double() * (2 * math.pi / one.T)
+    F = torch.stack([ang.cos(), ang.sin()], 1).reshape(one.M, n_mid)
+    for shape in (folded, folded.with_(B=1)):
+        layout = layout_of(shape, max_mid=shape.T, P=P)
+        stream = synth.KVStream(shape, seed=72, device="cuda", freq="offgrid")
+        K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+        ws = fa.new_workspace(layout)
+        got, want = _compress(layout, stream, K, V, ws), _cache(layout, stream)
+        fa.fa_compress(layout, want, K, V, ws, flags=fa.FA_COMPRESS_ORDERED)
+        torch.cuda.synchronize()
+        for n in EXACT_KEYS:
+            assert torch.equal(getattr(got, n), getattr(want, n)), n
+        for X, coef, idx in ((K, got.coef_k, got.idx_comp_k), (V, got.coef_v, got.idx_comp_v)):
+            for h in range(shape.Hkv if coef.numel() else 0):
+                y = torch.einsum("mj,bje->bme", F, X[:, n0:n0 + n_mid, h][..., idx[h].long()].double())
+                assert ((coef[:, h] - y).abs() <= MOMENT_REL * y.abs().amax(dim=(-1, -2), keepdim=True)).all(), h
 
 
 def test_folded_rows_of_different_length():
-    """Rows of odd and even numbers of blocks, one too short for the path, in one call: each as its row alone."""
-    shape = _shape(B=5, L=6000, M=512, T=16384, n_full_k=24, n_full_v=48)
+    """Rows of odd and even numbers of blocks, one too short for the path, in one call: each as its row alone (too little work to be folded)."""
+    shape = _shape(B=5, Hkv=28, Hq=28, L=6000, M=512, T=16384, n_full_k=24, n_full_v=48)
     layout = layout_of(shape, max_mid=shape.T, P=16)
     stream = synth.KVStream(shape, seed=10, device="cuda", freq="offgrid")
     K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
@@ -78,7 +99,7 @@ def test_folded_rows_of_different_length():
         torch.cuda.synchronize()
         for side in ("coef_k", "coef_v"):
             x, y = getattr(got, side)[b], getattr(c, side)[0]
-            assert ((x - y).abs() <= 1e-5 * y.abs().amax(dim=(-1, -2), keepdim=True)).all(), (b, side)
+            assert ((x - y).abs() <= MOMENT_REL * y.abs().amax(dim=(-1, -2), keepdim=True)).all(), (b, side)
         assert torch.equal(got.state[b], c.state[0])
 
 
