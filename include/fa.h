@@ -241,6 +241,8 @@ fa_status fa_decode_step(const fa_layout* layout, fa_cache* cache, const void* q
  * and caches are HOST arrays of n_layers entries; q, k_new, v_new, out are HOST arrays of n_layers
  * DEVICE pointers ([B][H_q][d] / [B][H_kv][d] of that layer).  One workspace serves all layers (the
  * calls are ordered by the stream): ws_bytes must cover the largest fa_workspace_bytes of the layouts.
+ * Neighbouring layers of one layout may run side by side in shared launches where none writes what another one
+ * reads or writes (their arguments tell) and the workspace has room for all of them; the result is the same.
  * All layers are checked on the host before the first launch; after that the call only enqueues
  * kernels, so a whole token step can be captured in one CUDA graph (after one eager call).  Stops at,
  * and returns, the first error. */
@@ -276,8 +278,8 @@ size_t fa_step_staging_bytes(const fa_layout* layout);
  *   ws / ws_bytes: scratch of fa_select_workspace_bytes(layout) bytes, 256-byte aligned (it holds the
  *     coefficients of all dimensions).  head_dim must be 64, 128 or 256.
  * For bf16 tensors (head_dim 64 or 128, 16-byte aligned bases and strides) the reconstruction runs on the tensor cores: with
- * n_coef a multiple of 256, a period of at least 16 n_coef and 1024 middle tokens by block moments, whose factors carry 2^-17 (a dimension
- * that its coefficients rebuild exactly reports about 1e-9 of its mean square); else, n_coef a multiple of 64, with the basis and the
+ * n_coef a multiple of 256, a period of at least 16 n_coef, 1024 middle tokens and 6 M values of the middle of K (all rows and heads) by block
+ * moments, whose factors carry 2^-17 (a dimension that its coefficients rebuild exactly reports about 1e-9 of its mean square); else, n_coef a multiple of 64, with the basis and the
  * weighted coefficients rounded to bf16 (about 1e-6).
  * Asynchronous on `stream`.  An empty middle gives zero errors (the lowest indices are compressed). */
 fa_status fa_select_workspace_bytes(const fa_layout* layout, size_t* out);

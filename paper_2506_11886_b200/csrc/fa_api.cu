@@ -501,8 +501,12 @@ fa_status fa_validate(const fa_layout* layout, const fa_cache* cache, void* stre
     return fa_poll_status(cache, stream);
 }
 
-fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K, const void* V, int64_t stride_b,
-                         int64_t stride_t, int64_t stride_h, int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream) {
+}  // extern "C"
+
+// fa_compress_ex; without windows, the caller has no use for them, nor for the counters, and the path by block moments leaves them out.
+namespace fa {
+fa_status compress_call(const fa_layout* layout, fa_cache* cache, const void* K, const void* V, int64_t stride_b, int64_t stride_t, int64_t stride_h,
+                        int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream, bool windows) {
     fa_status st = check_layout(layout);
     if (st != FA_OK) return st;
     st = check_cache(layout, cache);
@@ -541,7 +545,7 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
     if (room.at && room.bytes >= compress_mom_row_bytes(s, n_mid_host)) {
         const CacheDev c = make_cache(*cache);
         if (compress_by_moments(s, c, K, V, sbb, stride_t, stride_h, L, room, cs) == cudaSuccess)
-            return launch_windows(s, &c, &K, &V, 1, sbb, stride_t, stride_h, L, cs) == cudaSuccess ? FA_OK : FA_ERR_CUDA;
+            return !windows || launch_windows(s, &c, &K, &V, 1, sbb, stride_t, stride_h, L, cs) == cudaSuccess ? FA_OK : FA_ERR_CUDA;
         cudaGetLastError();                                 // the cluster launch was refused: everything below, from the start
     }
     // tensor-core path: its kernel also writes the kept-dim rows of the middle from the boxes it loads; the partition
@@ -563,6 +567,14 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
     }
     if (tc && !tc2 && launch_compress_tc(s, make_cache(*cache), K, V, sbb, stride_t, stride_h, L, ordered, tc_rows, cs) != cudaSuccess) return FA_ERR_CUDA;
     return FA_OK;
+}
+}  // namespace fa
+
+extern "C" {
+
+fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K, const void* V, int64_t stride_b,
+                         int64_t stride_t, int64_t stride_h, int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream) {
+    return compress_call(layout, cache, K, V, stride_b, stride_t, stride_h, L, flags, ws, ws_bytes, stream, true);
 }
 
 namespace {

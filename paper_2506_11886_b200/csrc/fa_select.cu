@@ -16,11 +16,14 @@ namespace fa {
 
 fa_status check_layout(const fa_layout* l);
 fa_status decode_scratch_bytes(const fa_layout* layout, size_t* out);
+fa_status compress_call(const fa_layout* layout, fa_cache* cache, const void* K, const void* V, int64_t stride_b, int64_t stride_t, int64_t stride_h,
+                        int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream, bool windows);
 
 namespace {
 
 constexpr int kMseTokens = 64;      // middle tokens per CTA
-constexpr int kSelectMomMid = 1024; // middle tokens from which the reconstruction goes by block moments
+constexpr int kSelectMomMid = 1024; // middle tokens of a row and
+constexpr long long kSelectMomDims = 48ll * 1024 * 128;               // dimensions of all middle tokens from which the reconstruction goes by block moments
 constexpr int kMseRows = 32;        // coefficient rows staged per round (16 frequencies)
 
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -241,13 +244,18 @@ fa_status fa_select_dims(const fa_layout* layout, const void* K, const void* V, 
                                                                s.Hkv, s.d, sc.cache.status, reinterpret_cast<int32_t*>(sc.ws_compress), n_counters,
                                                                sc.sq, n_sq);
     if (cudaGetLastError() != cudaSuccess) return FA_ERR_CUDA;
-    st = fa_compress(&sc.layout, &sc.cache, K, V, stride_b, stride_t, stride_h, L, sc.ws_compress, sc.ws_compress_bytes, stream);
+    st = compress_call(&sc.layout, &sc.cache, K, V, stride_b, stride_t, stride_h, L, 0, sc.ws_compress, sc.ws_compress_bytes, stream, false);      // (coefficients only)
     if (st != FA_OK) return st;
     const int n_init = L < s.l_init ? L : s.l_init;
     const int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;
     const int n_mid = L - n_init - n_local;
     bool done = n_mid == 0;
-    if (n_mid >= kSelectMomMid && sc.mom_bytes) {
+    // By block moments it is three launches, chained: 8 to 10 us more than the one over coefficient rows before either has done anything.  What
+    // they save grows with the prefill, whatever the number of coefficients.  The whole call, us, over coefficient rows / by moments (128 dims unless
+    // stated, k coefficients; in M: dimensions of the middle tokens):  2.9 M 60/69 (k = 256); 3.7 M 66/77 (512); 64 dims, 4.1 M 101/97 (2048), 71/73
+    // (1024), 60/63 (512);  7.1 M 75/73 (256), 87/83 (512);  8.2 M 79/79 (256), 87/85 (512), 112/98 (1024); 64 dims, 8.1 M 85/73 (512), 163/116
+    // (2048);  12 M 105/93 (256);  15 M 110/91 (256), 169/120 (1024);  32 M 257/140 (1024), 398/233 (2048).
+    if (n_mid >= kSelectMomMid && (long long)s.B * n_mid * s.Hkv * s.d >= kSelectMomDims && sc.mom_bytes) {
         done = launch_select_mom(make_dims(sc.layout), sc.cache.coef_k, sc.cache.coef_v, K, V, stride_b, stride_t, stride_h, n_init, n_mid, L, sc.sq,
                                  sc.cache.status, sc.mom, cs) == cudaSuccess;
         if (!done) cudaGetLastError();                     // (the last of its kernels alone adds to the sums)
