@@ -304,7 +304,7 @@ def bench_layers(torch, fa, synth, timer, dev, cfg_id, n_layers, tok_steps, warm
            "decode_gbs": dec_gbs, "frac": dec_gbs / peak,
            "step_gbs": (by["decode"] + by["append"]) * n_layers / (tok["median"] * 1e-6) / 1e9,
            "tokens_per_s": shape.B * 1e6 / tok["median"],
-           "launches_per_token_step": n_layers * step_launches(fa, layout),
+           "launches_per_layer_step": step_launches(fa, layout),      # (in the channel form the layers of a call share them, up to four)
            "compress_ms_per_layer": min(comp), "compress_tflops": comp_flop / (min(comp) * 1e-3) / 1e12}
     del caches, args
     torch.cuda.empty_cache()

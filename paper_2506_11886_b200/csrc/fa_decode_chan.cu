@@ -17,8 +17,9 @@
 // No CTA waits for another one outside its cluster; the kernels are chained with programmatic dependent launch.  P and Z, and the
 // probabilities of the way back, are held as two bf16 numbers each (2^-17), three products; the kept dims as everywhere
 // (q . K exact, p rounded to bf16 for p . V).
-// A step, transform kernel -> here: 8 rows of 32 KV heads, 4K tokens 118 -> 100 us (17 + 65 + 18 by kernel; 56 us of bytes), 4 rows of
-// 8 KV heads, 128K tokens 242 -> 193 us (35 + 116 + 37; 101 us of bytes).
+// A launch takes up to four layers whose memory is apart: the outer kernels are chains of round trips that leave the SMs half idle, and the middle
+// one's parts end evenly.  A step, transform kernel -> a layer by itself -> layers together: 8 rows of 32 KV heads, 4K tokens 118 -> 100 -> 78 us (14 + 50 + 14
+// by kernel, four layers; 56 us of bytes), 4 rows of 8 KV heads, 128K tokens 242 -> 190 -> 162 us (28 + 103 + 30, two layers; 101 us of bytes).
 #include <type_traits>
 
 #include "fa_decode_fft.cuh"
@@ -531,7 +532,7 @@ __global__ void __launch_bounds__(outer_threads(LS), NH == 4 && outer_ctas(LS) =
 // stages that its first lane refills, running maxima, sums and outputs; the four meet once, at the end.  Bound by the latency of
 // its chain of shared-memory reads and mma per 64 tokens (a warp issues in one cycle of seven), so warps count: 8 rows of 32 KV
 // heads, 4K tokens, 48 + 48 kept dims (281 MB) in 73 us with two CTAs to an SM and K and V in one stage, in 65 us with three and a
-// stage for K or V; 562 MB of four rows of 128K tokens in 116 us.  (Warps that shared the classes of a step met twice per step
+// stage for K or V, four such layers in one launch in 199 (5.7 TB/s); 562 MB of four rows of 128K tokens in 116 us, two layers in 206 (5.5 TB/s).  (Warps that shared the classes of a step met twice per step
 // for its maximum and for W: 217 us there.)
 // The class parts of all heads come first in the grid, the shorter window parts fill the gaps behind them.
 // Class parts: a superstep is four neighbouring slots of all P classes, a stage the K rows or V rows of 16 classes as
