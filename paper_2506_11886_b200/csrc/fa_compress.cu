@@ -141,7 +141,6 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
     // programmatically behind the one before), the end of this grid then implies the end of all before it.  Launched
     // the plain way this returns at once.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (waits) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---- Eq.3-4: C[m][e] += sum_j F[m][j] X[n_init + j][D^c[e]] ------------------
