@@ -149,7 +149,10 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
 // tile in shared memory; thread (rg, lane) accumulates rows 4 rg..4 rg + 3 of
 // the tile for columns lane, lane + 32, ...  Partial sums of the token splits
 // are added to the zeroed coefficients with atomics.
-// R rows per thread: eight where that leaves CTAs enough (half the shared-memory reads per product), else four.
+// R rows per thread: eight where tiles of 64 rows and chunks of 64 tokens make two CTAs to an SM (half the shared-memory reads per product), else
+// four.  us, four / eight rows:  tiles x chunks 80 11.3/13.3, 112 17.4/17.4, 136 29.7/31.7 (a selection), 160 46.1/46.1, 480 64/59 and, four layers, 159/134,
+// 896 70/62 (8 rows of 8 KV heads, 700 tokens, 64 coefficients).  Bound by the FMA and shared-memory pipes beside a chain of index, load and
+// barrier per chunk.
 constexpr int kTJ = 64;
 
 // NC: columns per lane (32 NC >= the compressed dims of either side; the products of lanes without a column are not issued).
@@ -208,8 +211,7 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
             int n = m0 / 2 + nn;
             float cs = 0.f, sn = 0.f;
             if (jj < nj && n < s.k) basis_cs(n, j0 + jj, s.T, &cs, &sn);
-            F_s[jj * kTM + 2 * nn] = cs;
-            F_s[jj * kTM + 2 * nn + 1] = sn;
+            *reinterpret_cast<float2*>(F_s + jj * kTM + 2 * nn) = make_float2(cs, sn);
         }
         __syncthreads();
 #pragma unroll 4
@@ -285,9 +287,9 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     int max_comp = s.dck > s.dcv ? s.dck : s.dcv;
     if (n_mid == 0 || max_comp == 0 || !with_coef) return cudaSuccess;
     const int live_rows = rl.n ? n_short : s.B;
-    const int rpt = (long long)((s.M + 63) / 64) * live_rows * s.Hkv * 2 >= 2 * sm_count() ? 8 : 4;
-    const int row_tiles = (s.M + 8 * rpt - 1) / (8 * rpt);
     int chunks = (n_mid + kTJ - 1) / kTJ;
+    const int rpt = (long long)((s.M + 63) / 64) * live_rows * s.Hkv * 2 * chunks >= 2 * sm_count() ? 8 : 4;
+    const int row_tiles = (s.M + 8 * rpt - 1) / (8 * rpt);
     int ctas_fixed = row_tiles * live_rows * s.Hkv * 2;
     int n_tsplit = (4 * sm_count() + ctas_fixed - 1) / ctas_fixed;
     if (n_tsplit > chunks) n_tsplit = chunks;
