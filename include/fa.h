@@ -70,7 +70,7 @@ typedef enum { FA_NORM_ORTHO = 0, FA_NORM_PAPER = 1 } fa_norm;
  * FFT_SPLIT always takes the three-kernel form.  AUTO also takes it when there
  * are more (batch, KV head) pairs than SMs and the last wave of the one-kernel
  * form would be nearly empty.  For bf16 caches with many (batch, KV head) pairs
- * and classes (see fa_launch_count, 7) AUTO evaluates the classes by 16 Legendre
+ * and classes (see fa_launch_count, 7) and n_coef a multiple of four AUTO evaluates the classes by 16 Legendre
  * channels instead of one transform per class (left out: below 1e-9 relative), as a
  * chain of three kernels, when ws_bytes has the room that fa_workspace_bytes asks
  * for; with less it is FFT. */

@@ -1340,13 +1340,16 @@ static double makespan(long long n1, double a, long long n2, double b, int slots
 }
 
 // Whether the channel form serves a layout that the transform kernel serves (period a power of two, S >= k, at most 64 kept dims
-// a side, head_dim at most 128), and its plan.
+// a side, head_dim at most 128) with a multiple of four coefficients, and its plan.
 bool plan_channels(const Dims& s, int log2S, int sms, ChanPlan* m) {
     memset(m, 0, sizeof(*m));
     const int S = 1 << log2S;
     m->slots = S;
     if (s.dck == 0 || s.dcv == 0 || s.nfk > 64 || s.nfv > 64 || s.nfk + s.nfv == 0 || s.d > 128) return false;
     if (s.P % 16 || s.P > 512 || s.k > S || s.P * S != s.T || s.S_cap > S || s.B > 256) return false;
+    // A head's coefficients, and a pair of channels' factors, follow one another in shared memory and are read and exchanged 16 bytes at a time: whole
+    // groups of four of them.  (n_coef = 2 mod 4 is left to the transform kernel, whose rows may end anywhere.)
+    if (s.M % 4) return false;
     m->n_pass = (s.G + 3) / 4;
     m->nh = (s.G + m->n_pass - 1) / m->n_pass;
     m->hp = m->nh > 2 ? 4 : 2;

@@ -111,6 +111,12 @@ def test_launch_plan_is_host_logic():
     assert launches(2, **dict(mha, batch=5)) == 1                                  # 160 heads, all resident at once: stays fused
     long_ctx = dict(batch=4, n_coef=2048, period=131072, max_mid=131072, mid_classes=128, l_local=2048)
     assert launches(4, **long_ctx) == 1 and launches(5, **long_ctx) == 2           # longest transforms: split build, two classes per batch
+    # the channel form works on groups of four coefficients: heads' rows that end inside a group of 16 bytes are the transform kernel's
+    chan = dict(batch=8, n_q_heads=16, period=4096, max_mid=4096, mid_classes=128, l_local=64)
+    for m in range(2, 66, 2):
+        for hq in (8, 16, 24, 32):
+            assert launches(7, **dict(chan, n_coef=m, n_q_heads=hq)) == (3 if m % 4 == 0 else 0), (m, hq)
+    assert launches(2, **dict(chan, n_coef=50)) == 3 and launches(3, **dict(chan, n_coef=50)) == 4
     # the workspace grows with the number of partial results but stays far below the static limit's order
     small, big = fa.fa_workspace_bytes(_layout()), fa.fa_workspace_bytes(_layout(batch=8))
     assert 0 < small < big

@@ -63,6 +63,20 @@ def test_channels_against_oracle(P, kw):
     pair.check_state()
 
 
+@pytest.mark.parametrize("M", [50, 62])
+@pytest.mark.parametrize("Hq,kw", [(16, dict()), (24, dict(n_full_k=48)), (32, dict(B=4, Hkv=16, Hq=64)), (8, dict(n_full_v=16))])
+def test_coefficients_not_in_groups_of_four(M, Hq, kw):
+    """Heads' rows of coefficients that end inside 16 bytes, two, three, four heads and one to a pass: not the channel form, and right."""
+    shape = _shape(**{**dict(Hq=Hq, M=M, L=700), **kw})
+    pair, stream = make_pair(shape, seed=6, P=128, max_mid=shape.T, freq="offgrid")
+    assert fa.fa_launch_count(pair.layout, 7) == 0 and fa.fa_launch_count(dataclasses.replace(pair.layout, n_coef=M + 2), 7) == 3
+    K, V = stream.tokens(shape.L, shape.L + 2)
+    pair.check_decode(synth.queries(shape, seed=1))
+    for t in range(2):
+        pair.check_step(synth.queries(shape, seed=1, step=t + 1), K[:, t], V[:, t])
+    pair.check_state()
+
+
 @pytest.mark.parametrize("ragged_one_short", [False, True])
 def test_channels_ragged_small_workspace_and_graph(ragged_one_short):
     """Rows of different length (empty, inside the windows, long, one that is full after a step and says so at the next); a
