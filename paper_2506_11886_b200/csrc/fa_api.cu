@@ -5,6 +5,7 @@
 #include <mutex>
 
 #include "fa_common.cuh"
+#include "fa_row_groups.h"
 
 namespace fa {
 
@@ -406,17 +407,15 @@ static MomentRoom moment_room(const fa_layout& l, void* ws, size_t ws_bytes) {
 // (one row at least fits).
 static cudaError_t compress_by_moments(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int L,
                                        MomentRoom room, cudaStream_t stream, const RowLens* lens = nullptr, int tc_min = 1) {
-    int n_mid = lens ? 0 : mid_of(s, L);
-    for (int b = 0; lens && b < s.B; ++b) n_mid = mid_of(s, lens->len[b]) > n_mid ? mid_of(s, lens->len[b]) : n_mid;
+    auto mid = [&](int b) { return mid_of(s, lens ? lens->len[b] : L); };
+    int n_mid = 0;
+    for (int b = 0; b < (lens ? s.B : 1); ++b) n_mid = mid(b) > n_mid ? mid(b) : n_mid;
     const size_t row = compress_mom_row_bytes(s, n_mid), fit = room.bytes / row;
-    const int group = fit >= (size_t)s.B ? s.B : fit >= 2 ? (int)(fit / 2) : 1;
-    for (int b0 = 0, i = 0; b0 < s.B; b0 += group, ++i) {
-        const int nb = s.B - b0 < group ? s.B - b0 : group;
-        char* Y = room.at + (fit >= 2 && (i & 1) ? (size_t)group * row : 0);
-        const cudaError_t err = launch_compress_mom(s, c, K, V, sb, st, sh, L, b0, nb, Y, fit < 2 && i > 0, i > 0, stream, lens, tc_min);
-        if (err != cudaSuccess) return err;
-    }
-    return cudaSuccess;
+    return (cudaError_t)for_row_groups(
+        s.B, fit, [&](int b) { return !lens || mid(b) >= tc_min; },
+        [&](const RowGroup& g) {
+            return (int)launch_compress_mom(s, c, K, V, sb, st, sh, L, g.b0, g.nb, room.at + (g.second ? fit / 2 * row : 0), g.wait_first, g.chained, stream, lens, tc_min);
+        });
 }
 
 }  // namespace fa
