@@ -190,6 +190,37 @@ def test_groups_of_rows_and_the_direct_contraction_agree(ragged, strided):
         assert not ws[:4096].any()                        # the barrier counters of the decode call are left alone
 
 
+@pytest.mark.parametrize("lengths", [
+    [300, 700, 2900, 1500, 1092, 2400],                   # the first group short throughout (rooms of four: groups of two)
+    [2900, 1500, 300, 700, 2400, 1092],                   # one in the middle
+    [2900, 1500, 2400, 1092, 0, 700],                     # the last
+    [100, 2900, 50, 2800, 60, 2700],                      # every other row: groups of one
+])
+def test_groups_without_a_long_row(lengths):
+    """Rows too short for the path make up whole groups: two layers' calls back to back in one stream on one workspace, each row as by itself."""
+    shape = _shape(B=6, L=2900, Hkv=4, Hq=4, n_full_k=24, n_full_v=48)
+    layout, one = layout_of(shape, max_mid=shape.T, P=16), layout_of(shape.with_(B=1), max_mid=shape.T, P=16)
+    streams = [synth.KVStream(shape, seed=30 + i, device="cuda", freq="offgrid") for i in range(2)]
+    toks = [s.tokens(0, shape.L, work_dtype=torch.float32) for s in streams]
+    want = [[_compress(one, s, K[b:b + 1, :n], V[b:b + 1, :n], fa.new_workspace(one)) for b, n in enumerate(lengths)] for s, (K, V) in zip(streams, toks)]
+    for rows in (1, 2, 3, 4, 5):
+        ws = _workspace(layout, shape.L - 68, rows)
+        got = [_cache(layout, s) for s in streams]
+        for c, (K, V) in zip(got, toks):
+            fa.fa_compress_ragged(layout, c, K, V, lengths, ws)
+        torch.cuda.synchronize()
+        for c, singles in zip(got, want):
+            assert fa.fa_poll_status(c) == fa.FA_OK
+            for b, y in enumerate(singles):
+                for name in ("k_init", "v_init", "k_local", "v_local", "k_mid", "v_mid", "state"):
+                    assert torch.equal(getattr(c, name)[b], getattr(y, name)[0]), (rows, b, name)
+                for name in ("coef_k", "coef_v"):
+                    a, r = getattr(c, name)[b], getattr(y, name)[0]
+                    den = r.abs().amax(dim=(-1, -2), keepdim=True)
+                    # (the same products in another order; short rows fp32 sums in another order)
+                    assert ((a - r).abs() <= 2e-6 * den).all(), (rows, b, name)
+
+
 @pytest.mark.parametrize("room,B", [(1, 1), (2, 1), (3, 1), (4, 1), (7, 1), (4, 2)])      # layers whose moments the workspace holds
 def test_layers_in_one_call_and_replayed_from_a_graph(room, B):
     """Layers with scratch for one or two layers at a time, with inputs that change between the replays of a graph."""

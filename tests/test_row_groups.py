@@ -39,3 +39,11 @@ def test_every_row_with_moments_once_and_chained_behind_a_launch_of_the_call(gro
         assert [g[4] for g in gs] == [0] + [1] * (len(gs) - 1), (B, fit, live, gs)
         assert all(any(live >> b & 1 for b in range(g[0], g[0] + g[1])) for g in gs)
         assert all(g[1] <= (fit if len(gs) == 1 and fit >= B else max(1, fit // 2)) for g in gs), (B, fit, live, gs)
+
+
+def test_no_launch_writes_where_the_one_in_front_reads(groups):
+    """Neighbours among the launches of a call take different halves, or the later one waits."""
+    for (B, fit, live), gs in groups:
+        for (*_, second, _, _), (*_, second_next, wait, _) in zip(gs, gs[1:]):
+            assert second != second_next or wait, (B, fit, live, gs)
+        assert fit >= 2 or not any(g[2] for g in gs)
