@@ -390,18 +390,32 @@ static size_t compress_scratch_bytes(const fa_layout& l) {
     if (rows > (size_t)kMomLayers * s.B) rows = (size_t)kMomLayers * s.B;
     return rows * row;
 }
-// Areas of the layers behind the first that share the launches of the channel form, behind the moments' room (so that a workspace of a smaller size
-// serves what it served; with the compression's layers, what is there counts).
-static size_t chan_layers_at(const fa_layout& l, size_t decode) { return align_up(decode_room_bytes(l, decode) + compress_scratch_bytes(l), 256); }
-static size_t chan_layers_bytes(const CallPlan& p) { return p.chan.on && p.chan.n_pass == 1 ? (kChanLayers - 1) * p.chan.per_layer : 0; }
+// What lies where in a workspace of ws_bytes: a decode call's areas, those of the layers behind the first that share the launches of the channel form
+// (as many as there is room for in front of the share that fa_workspace_bytes asks for the moments), and from there to the end the moments of a compression.
+struct WsAreas {
+    size_t layers, moments;  // where they begin
+    int more;                // layers behind the first
+};
+static bool workspace_areas(const fa_layout& l, size_t ws_bytes, WsAreas* a) {
+    size_t decode = 0;
+    CallPlan p;
+    if (decode_scratch_bytes(&l, &decode) != FA_OK || plan_decode(l, &p) != FA_OK) return false;
+    a->layers = decode_room_bytes(l, decode);
+    a->more = 0;
+    const size_t least = a->layers + compress_scratch_bytes(l);
+    if (p.chan.on && p.chan.n_pass == 1 && ws_bytes > least) {
+        const size_t n = (ws_bytes - least) / p.chan.per_layer;
+        a->more = n < (size_t)(kChanLayers - 1) ? (int)n : kChanLayers - 1;
+    }
+    a->moments = a->layers + a->more * p.chan.per_layer;
+    return true;
+}
 // Where the moments of a call go and how many bytes there are (0: the direct contraction).
 struct MomentRoom { char* at; size_t bytes; };
 static MomentRoom moment_room(const fa_layout& l, void* ws, size_t ws_bytes) {
-    size_t decode = 0;
-    if (!ws || !aligned16(ws) || !compress_mom_supported(make_dims(l)) || decode_scratch_bytes(&l, &decode) != FA_OK) return {nullptr, 0};
-    decode = decode_room_bytes(l, decode);
-    const size_t most = compress_scratch_bytes(l), left = ws_bytes > decode ? ws_bytes - decode : 0;
-    return left ? MomentRoom{static_cast<char*>(ws) + decode, left < most ? left : most} : MomentRoom{nullptr, 0};
+    WsAreas a;
+    if (!ws || !aligned16(ws) || !compress_mom_supported(make_dims(l)) || !workspace_areas(l, ws_bytes, &a) || ws_bytes <= a.moments) return {nullptr, 0};
+    return MomentRoom{static_cast<char*>(ws) + a.moments, ws_bytes - a.moments};
 }
 // The two kernels of the block-moment path over all batch rows: all at once, or in groups that take half of the room in turn
 // (one row at least fits).
@@ -453,8 +467,8 @@ fa_status fa_workspace_bytes(const fa_layout* layout, size_t* out) {
     CallPlan p;
     st = plan_decode(*layout, &p);
     if (st != FA_OK) return st;
-    const size_t more = chan_layers_bytes(p);
-    *out = more ? chan_layers_at(*layout, decode) + more : decode_room_bytes(*layout, decode) + compress_scratch_bytes(*layout);
+    *out = decode_room_bytes(*layout, decode) + compress_scratch_bytes(*layout);
+    if (p.chan.on && p.chan.n_pass == 1) *out += (kChanLayers - 1) * p.chan.per_layer;
     return FA_OK;
 }
 
@@ -946,14 +960,13 @@ static int step_channel_layers(int n_layers, const fa_layout* layouts, fa_cache*
                                void* const* out, char* ws, size_t ws_bytes, cudaStream_t stream) {
     CallPlan p;
     if (n_layers < 2 || plan_decode(layouts[0], &p) != FA_OK || !p.chan.on || p.chan.n_pass != 1) return 0;
-    size_t decode = 0;
+    WsAreas areas;
     fa_cache_sizes z;
-    if (decode_scratch_bytes(&layouts[0], &decode) != FA_OK || fa_cache_sizes_of(&layouts[0], &z) != FA_OK) return 0;
-    const size_t at = chan_layers_at(layouts[0], decode);
+    if (!workspace_areas(layouts[0], ws_bytes, &areas) || fa_cache_sizes_of(&layouts[0], &z) != FA_OK) return 0;
     ChanArgs a[kChanLayers];
     int n = 0;
-    for (; n < n_layers && n < kChanLayers; ++n) {
-        if (n > 0 && (std::memcmp(&layouts[n], &layouts[0], sizeof(fa_layout)) != 0 || ws_bytes < at + n * p.chan.per_layer)) break;
+    for (; n < n_layers && n <= areas.more; ++n) {
+        if (n > 0 && std::memcmp(&layouts[n], &layouts[0], sizeof(fa_layout)) != 0) break;
         const void* const in_n[3] = {q[n], k_new[n], v_new[n]};
         bool apart = true;
         for (int i = 0; i < n && apart; ++i) {
@@ -961,7 +974,7 @@ static int step_channel_layers(int n_layers, const fa_layout* layouts, fa_cache*
             apart = layers_apart(layouts[0], z, caches[i], in_i, out[i], caches[n], in_n, out[n]);
         }
         if (!apart) break;
-        a[n] = ChanArgs{make_cache(caches[n]), q[n], k_new[n], v_new[n], out[n], n == 0 ? ws + p.chan.base : ws + at + (n - 1) * p.chan.per_layer};
+        a[n] = ChanArgs{make_cache(caches[n]), q[n], k_new[n], v_new[n], out[n], ws + (n == 0 ? p.chan.base : areas.layers + (n - 1) * p.chan.per_layer)};
     }
     if (n < 2) return 0;
     bool begun = false;

@@ -254,6 +254,59 @@ def test_layers_in_one_call_and_replayed_from_a_graph(room, B):
     assert all(fa.fa_poll_status(c) == fa.FA_OK for c in caches)
 
 
+def _touched(ws, call):
+    """First and last byte of a workspace (past the barrier counters) that a call writes."""
+    lo, hi = ws.numel(), 0
+    for fill in (0x5A, 0xA5):
+        ws[4096:] = fill
+        call()
+        torch.cuda.synchronize()
+        at = (ws[4096:] != fill).nonzero()
+        if at.numel():
+            lo, hi = min(lo, 4096 + int(at[0])), max(hi, 4096 + int(at[-1]))
+    return lo, hi
+
+
+def test_steps_in_front_of_moments():
+    """In one workspace a step over layers stays in front of what the compression of the same layout uses, with areas for four layers as for two."""
+    shape = _shape(B=8, Hq=32, Hkv=32, L=1500)
+    layout = layout_of(shape, max_mid=shape.T, P=32)
+    assert fa.fa_launch_count(layout, 7) == 3
+    stream = synth.KVStream(shape, seed=6, device="cuda", freq="offgrid")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    kn, vn = (x[:, 0].contiguous() for x in stream.tokens(shape.L, shape.L + 1, work_dtype=torch.float32))
+    caches = [_compress(layout, stream, K, V, fa.new_workspace(layout)) for _ in range(4)]
+    qs = [synth.queries(shape, seed=i, device="cuda") for i in range(4)]
+    outs = [torch.zeros_like(q) for q in qs]
+    args = fa.LayerStep([layout] * 4, caches, qs, [kn] * 4, [vn] * 4, outs)
+    target = _cache(layout, stream)
+    ends = []
+    for less in (0, 16 << 20):                             # (a layer's areas are some 10 MiB)
+        ws = torch.zeros(fa.fa_workspace_bytes(layout) - less, dtype=torch.uint8, device="cuda")
+        _, end = _touched(ws, lambda: fa.fa_decode_step_layers(args, ws))
+        begin, _ = _touched(ws, lambda: fa.fa_compress(layout, target, K, V, ws))
+        assert 0 < end < begin < ws.numel()
+        ends.append(end)
+    assert ends[1] < ends[0]
+
+
+def test_a_larger_workspace_holds_all_rows_at_once():
+    """What a workspace has beyond the size that is asked for serves the moments: eight rows whose moments exceed the 192 MiB of that size."""
+    shape = _shape(B=8, Hq=32, Hkv=32, L=16384, M=512, T=16384)
+    layout = layout_of(shape, max_mid=shape.T, P=1)
+    stream = synth.KVStream(shape, seed=7, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(7)
+    K, V = (torch.randn(shape.B, shape.L, shape.Hkv, shape.d, device="cuda", dtype=torch.bfloat16, generator=g) for _ in range(2))
+    rows = shape.B * 44 * shape.Hkv * 192 * 128            # (blocks of 384 tokens, an even number of them)
+    want = _compress(layout, stream, K, V, fa.new_workspace(layout))
+    ws = torch.zeros(fa.fa_workspace_bytes(layout) + (100 << 20), dtype=torch.uint8, device="cuda")
+    got = _cache(layout, stream)
+    begin, end = _touched(ws, lambda: fa.fa_compress(layout, got, K, V, ws))
+    assert end - begin > 0.95 * rows > 192 << 20
+    # (segments are cut at other places: 22 pairs of blocks x six additions in the accumulators, each to 2^-23 of what is there)
+    _same(got, want, 22 * 6 * 2.0 ** -23)
+
+
 def test_not_finite_dims_stay_alone():
     """A NaN or an infinity in one dim of one token spoils that dim's coefficients only."""
     shape = _shape(L=2500)
