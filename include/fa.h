@@ -132,7 +132,8 @@ fa_status fa_cache_sizes_of(const fa_layout* layout, fa_cache_sizes* out);
 /* Host only.  Bytes of workspace fa_decode_attention needs and, behind them, fa_compress makes use of for this layout
  * (the latter's share is at most 192 MiB, or what one batch row takes; what a workspace has beyond this size serves
  * it too).  Calls of one kind that may overlap on the GPU
- * need workspaces of their own; a decode call or step and a compression may overlap in one.  The workspace is scratch whose contents need not survive
+ * need workspaces of their own; a decode call or step and a compression of the same layout may overlap in one (what lies where in it goes by the layout and by ws_bytes: pass the
+ * same size to both; calls of different layouts that may overlap need workspaces of their own).  The workspace is scratch whose contents need not survive
  * between calls, with one rule: its first 4 KiB hold barrier counters that must be zero
  * when a call starts.  Zero-fill a new workspace once (cudaMemset); every call that ends
  * without FA_ERR_TIMEOUT leaves the counters at zero again.  After FA_ERR_TIMEOUT
