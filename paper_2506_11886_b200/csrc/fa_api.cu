@@ -517,9 +517,10 @@ fa_status fa_validate(const fa_layout* layout, const fa_cache* cache, void* stre
 }  // extern "C"
 
 // fa_compress_ex; without windows, the caller has no use for them, nor for the counters, and the path by block moments leaves them out.
+// ws_of: the layout whose workspace it is, where the cache is a row of another one's.
 namespace fa {
 fa_status compress_call(const fa_layout* layout, fa_cache* cache, const void* K, const void* V, int64_t stride_b, int64_t stride_t, int64_t stride_h,
-                        int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream, bool windows) {
+                        int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream, bool windows, const fa_layout* ws_of) {
     fa_status st = check_layout(layout);
     if (st != FA_OK) return st;
     st = check_cache(layout, cache);
@@ -554,7 +555,7 @@ fa_status compress_call(const fa_layout* layout, fa_cache* cache, const void* K,
     const int n_mid_host = L - n_init - n_local;
     const bool tc = L > 0 && n_mid_host >= kTcMinMid && compress_tc_supported(s, layout->kv_dtype, sbb, stride_t, stride_h);
     // block moments where the workspace has room for them; the order-fixed mode keeps the direct contraction
-    const MomentRoom room = tc && !ordered ? moment_room(*layout, ws, ws_bytes) : MomentRoom{nullptr, 0};
+    const MomentRoom room = tc && !ordered ? moment_room(*ws_of, ws, ws_bytes) : MomentRoom{nullptr, 0};
     if (room.at && room.bytes >= compress_mom_row_bytes(s, n_mid_host)) {
         const CacheDev c = make_cache(*cache);
         if (compress_by_moments(s, c, K, V, sbb, stride_t, stride_h, L, room, cs) == cudaSuccess)
@@ -587,7 +588,7 @@ extern "C" {
 
 fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K, const void* V, int64_t stride_b,
                          int64_t stride_t, int64_t stride_h, int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream) {
-    return compress_call(layout, cache, K, V, stride_b, stride_t, stride_h, L, flags, ws, ws_bytes, stream, true);
+    return compress_call(layout, cache, K, V, stride_b, stride_t, stride_h, L, flags, ws, ws_bytes, stream, true, layout);
 }
 
 namespace {
@@ -819,7 +820,7 @@ fa_status fa_compress_ragged(const fa_layout* layout, fa_cache* cache, const voi
     part.batch = 1;
     for (int b = b0; b < layout->batch; ++b) {
         fa_cache row = slice(b);
-        st = fa_compress(&part, &row, prefill(K, b), prefill(V, b), stride_b, stride_t, stride_h, lengths[b], ws, ws_bytes, stream);
+        st = compress_call(&part, &row, prefill(K, b), prefill(V, b), stride_b, stride_t, stride_h, lengths[b], 0u, ws, ws_bytes, stream, true, layout);
         if (st != FA_OK) return st;
     }
     return FA_OK;

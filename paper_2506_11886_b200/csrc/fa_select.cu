@@ -17,7 +17,7 @@ namespace fa {
 fa_status check_layout(const fa_layout* l);
 fa_status decode_scratch_bytes(const fa_layout* layout, size_t* out);
 fa_status compress_call(const fa_layout* layout, fa_cache* cache, const void* K, const void* V, int64_t stride_b, int64_t stride_t, int64_t stride_h,
-                        int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream, bool windows);
+                        int32_t L, uint32_t flags, void* ws, size_t ws_bytes, void* stream, bool windows, const fa_layout* ws_of);
 
 namespace {
 
@@ -244,7 +244,7 @@ fa_status fa_select_dims(const fa_layout* layout, const void* K, const void* V, 
                                                                s.Hkv, s.d, sc.cache.status, reinterpret_cast<int32_t*>(sc.ws_compress), n_counters,
                                                                sc.sq, n_sq);
     if (cudaGetLastError() != cudaSuccess) return FA_ERR_CUDA;
-    st = compress_call(&sc.layout, &sc.cache, K, V, stride_b, stride_t, stride_h, L, 0, sc.ws_compress, sc.ws_compress_bytes, stream, false);      // (coefficients only)
+    st = compress_call(&sc.layout, &sc.cache, K, V, stride_b, stride_t, stride_h, L, 0, sc.ws_compress, sc.ws_compress_bytes, stream, false, &sc.layout);      // (coefficients only)
     if (st != FA_OK) return st;
     const int n_init = L < s.l_init ? L : s.l_init;
     const int n_local = (L - n_init) < s.l_local ? (L - n_init) : s.l_local;

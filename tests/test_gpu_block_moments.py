@@ -290,6 +290,21 @@ def test_steps_in_front_of_moments():
     assert ends[1] < ends[0]
 
 
+def test_rows_one_by_one_keep_off_the_decode_areas():
+    """Rows that are compressed one at a time (a local window shorter than a box) use the workspace as the whole batch's layout has it."""
+    shape = _shape(B=8, Hq=8, Hkv=8, L=2000, L_local=32)
+    layout = layout_of(shape, max_mid=shape.T, P=16)
+    stream = synth.KVStream(shape, seed=6, device="cuda", freq="offgrid")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    lengths, ws = [2000, 1999, 1500, 300, 2000, 1200, 1800, 0], fa.new_workspace(layout)
+    c = _compress(layout, stream, K, V, ws, lengths)
+    q = synth.queries(shape, seed=1, device="cuda")
+    out = torch.zeros_like(q)
+    _, end = _touched(ws, lambda: fa.fa_decode_attention(layout, c, q, out, ws))
+    begin, _ = _touched(ws, lambda: fa.fa_compress_ragged(layout, c, K, V, lengths, ws))
+    assert 0 < end < begin < ws.numel()
+
+
 def test_a_larger_workspace_holds_all_rows_at_once():
     """What a workspace has beyond the size that is asked for serves the moments: eight rows whose moments exceed the 192 MiB of that size."""
     shape = _shape(B=8, Hq=32, Hkv=32, L=16384, M=512, T=16384)
