@@ -955,8 +955,11 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     if (n_teams > total) n_teams = (int)total;
     // Equal cost per team: a segment costs its positions plus its epilogue and refill, kEpi where its sums are added to others', kWhole where a unit is
     // taken whole and they are stored; the smallest budget with which the walk covers all positions in n_teams teams, by bisection.
+    // (Folded units of fewer than 16 positions were taken whole at a kWhole of 9, by as many teams as there are units, where the others had nothing to
+    // do.  us at 9 / 12, the same at 16: 32 heads of 512 coefficients, 13 positions each 69.3/64.1, 15 each 75.6/70.2; 8 heads of 2048, 14 each 52.2/49.4; six
+    // ragged rows 65.8/64.3, 80.8/78.7; four rows of 86 positions and 2048 coefficients 690/673; six layers of 32 K tokens 273/273 (277 at 16).)
     MomCuts cuts = {};
-    constexpr long long kEpi = FOLD ? 16 : 6, kWhole = FOLD ? 9 : 4, kMinSeg = 2;
+    constexpr long long kEpi = FOLD ? 16 : 6, kWhole = FOLD ? 12 : 4, kMinSeg = 2;
     auto unit_of = [&](long long pos, long long* begin) {  // returns its end
         long long first = 0, nblk = rows.nblk;
         if (RAG) {
