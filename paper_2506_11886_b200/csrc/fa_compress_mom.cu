@@ -956,10 +956,12 @@ cudaError_t launch_project(const void* Y, const Dims& s, const CacheDev* c, int 
     // Equal cost per team: a segment costs its positions plus its epilogue and refill, kEpi where its sums are added to others', kWhole where a unit is
     // taken whole and they are stored; the smallest budget with which the walk covers all positions in n_teams teams, by bisection.
     // (Folded units of fewer than 16 positions were taken whole at a kWhole of 9, by as many teams as there are units, where the others had nothing to
-    // do.  us at 9 / 12, the same at 16: 32 heads of 512 coefficients, 13 positions each 69.3/64.1, 15 each 75.6/70.2; 8 heads of 2048, 14 each 52.2/49.4; six
-    // ragged rows 65.8/64.3, 80.8/78.7; four rows of 86 positions and 2048 coefficients 690/673; six layers of 32 K tokens 273/273 (277 at 16).)
+    // do.  us at 9 / 12, the same at 16: 32 heads of 512 coefficients, 13 positions each 69.3/64.1, 15 each 75.6/70.2; 8 heads of 2048, 14 each 52.2/49.4;
+    // four rows of 86 positions and 2048 coefficients 690/673; six layers of 32 K tokens 273/273 (277 at 16).  Rows of different length, whose longest
+    // units alone are shared, at 9 / 10 / 12: six rows of 2 to 15 positions and 8 heads, 104 and 88 columns, windows of 1024 tokens 72.0/72.0/72.9;
+    // 96 columns 69.6/68.0/68.1, windows of 64 tokens 66.2/65.1/62.8; five rows of 4 to 13 120.7/115.4/121.9.)
     MomCuts cuts = {};
-    constexpr long long kEpi = FOLD ? 16 : 6, kWhole = FOLD ? 12 : 4, kMinSeg = 2;
+    constexpr long long kEpi = FOLD ? 16 : 6, kWhole = FOLD ? (RAG ? 10 : 12) : 4, kMinSeg = 2;
     auto unit_of = [&](long long pos, long long* begin) {  // returns its end
         long long first = 0, nblk = rows.nblk;
         if (RAG) {
