@@ -847,13 +847,25 @@ int npad_of(const Dims& s) { return (s.dck + s.dcv + 31) / 32 * 32; }
 
 // Whether the blocks may be taken in pairs about the middle of a row: the projection then takes 256 frequencies at a time.
 bool can_fold(const Dims& s) { return s.k % 256 == 0; }
-// Whether a launch does so: n_pairs of blocks of all rows and layers.  Pairs are coarser work: SMs without one while the last of the moments are
-// formed, 256 frequencies to a segment.  That costs 2 to 4 us, which the halved products regain from some five and a half positions to a CTA pair on (between
-// 400 and 430 it goes either way).  us, plain / folded: 512 coefficients, 8 heads: 320 positions 59/60, 336 34/37, 416 72/76, 456 57/56, 520 89/85, 608
-// 69/66, six ragged rows 424 79/77;  32 heads: 320 50/55, 352 67/69, 416 75/80, 512 85/83, 608 71/67;  1024 coefficients, 8 heads: 336 42/42, 400 46/44,
-// 480 50/47, 656 69/66, 1312 115/101.
-constexpr long long kFoldPositions = 400;
-bool folds(const Dims& s, long long n_pairs) { return can_fold(s) && n_pairs * s.Hkv * (s.k / 256) >= kFoldPositions; }
+// Whether a launch does so: n_pairs pairs, n_blocks blocks of all rows and layers.  In us: 3 for coarser work (256 frequencies to a segment, SMs without a pair while the
+// last of the moments are formed), less a 110th of the projection's positions for its halved products; what is longer at the moments' end, where the busiest
+// CTA has two blocks more instead of one (a 320th of a us per token); a 190th per pair and head of blocks past 384 tokens, whose tables leave the
+// moments' ring a stage less.  Fitted to 270 launches of 4 to 32 heads, 512 to 2048 coefficients, rows of one length and of several: 0.25 % behind the better form on average,
+// 5 % at worst (2048 coefficients, 448 positions: 47.5/49.4).  us, plain / folded:
+//   512 coefficients, 32 heads, blocks of 384: 352 positions 58.2/58.3, 384 61.9/63.0 (two blocks more), 416 64.8/64.1, 512 73.5/72.4, 1024 135/128
+//   the same, blocks of 768: 416 positions 98.1/99.0, 448 103.9/109.3, 480 108.1/111.9 (both two blocks more), 576 129.6/130.1, 1088 216/213
+//   1024 coefficients, 8 heads, blocks of 384: 368 positions 43.4/43.4, 400 46.1/44.5, 432 47.5/45.3, 688 62.1/58.3
+//   2048 coefficients, 8 heads, blocks of 768: 416 positions 45.5/47.8 (two blocks more), 480 51.8/50.6, 1024 84.4/80.4, 11008 765/673
+//   512 coefficients, 8 heads, six ragged rows: 424 positions 70.2/68.7, 544 82.6/80.8
+bool folds(const Dims& s, long long n_pairs, long long n_blocks) {
+    if (!can_fold(s)) return false;
+    const long long items = s.Hkv * (s.d == 128 ? 2 : 1), sms = sm_count();
+    auto turns = [&](long long n) { return (n * items + sms - 1) / sms; };
+    const int R = block_tokens(s);
+    const double more = 3.0 - (double)(n_pairs * s.Hkv * (s.k / 256)) / 110.0 + (double)(2 * turns(n_pairs) - turns(n_blocks)) * R / 320.0 +
+                        (R > 384 ? (double)(n_pairs * s.Hkv) / 190.0 : 0.0);
+    return more < 0.0;
+}
 
 // The projection's stages leave room for a CTA of the windows kernel beside it: one of three stages, or of two where the projection would otherwise
 // have two itself (more than 192 columns, folded: 22 us instead of 16 for a head group of 256 columns, 512 coefficients and 3600 tokens).
@@ -1074,12 +1086,12 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
     rows.b0 = b0;
     rows.nb = nb;
     auto pairs = [&](int n_mid) { return (blocks_of(n_mid, rows.R) + 1) / 2; };
-    long long n_pairs = 0;
+    long long n_pairs = 0, n_blocks = 0;
     for (int b = b0; b < b0 + nb; ++b) {
         const int m = lens && lens->n == s.B ? mid_of(s, lens->len[b]) : mid_of(s, L);
-        if (!lens || !lens->n || m >= tc_min) n_pairs += pairs(m);
+        if (!lens || !lens->n || m >= tc_min) { n_pairs += pairs(m); n_blocks += blocks_of(m, rows.R); }
     }
-    const bool fold = folds(s, n_pairs);
+    const bool fold = folds(s, n_pairs, n_blocks);
     auto positions = [&](int n_mid) { return fold ? pairs(n_mid) : blocks_of(n_mid, rows.R); };
     if (lens && lens->n) {
         if (lens->n != s.B) return cudaErrorInvalidValue;
@@ -1112,7 +1124,8 @@ cudaError_t launch_compress_mom_layers(const Dims& s, const CacheDev* c, const v
     rows.R = block_tokens(s);
     rows.nb = s.B;
     rows.n_blk = blocks_of(mid_of(s, L), rows.R);
-    const bool fold = folds(s, (long long)(rows.n_blk + 1) / 2 * s.B * n_layers);
+    const long long n_rows = (long long)s.B * n_layers;
+    const bool fold = folds(s, (long long)(rows.n_blk + 1) / 2 * n_rows, rows.n_blk * n_rows);
     rows.nblk = fold ? (rows.n_blk + 1) / 2 : rows.n_blk;
     rows.total = rows.nblk * s.B;
     if (rows.total == 0) return cudaSuccess;

@@ -65,7 +65,7 @@ def test_folded_blocks(kw):
     P = 1 if one.T == 10000 else 8
     n0, n_mid = one.L_init, one.L - one.L_init - one.L_local
     pairs = -(-n_mid // (6 * one.T // (one.M // 2) // 64 * 64)) + 1 >> 1
-    folded = one.with_(B=-(-400 * 512 // (pairs * one.Hkv * one.M)))
+    folded = one.with_(B=-(-700 * 512 // (pairs * one.Hkv * one.M)))       # (700 positions: folded however the moments' items come out)
     ang = ((torch.arange(n_mid, device="cuda")[None] * torch.arange(one.M // 2, device="cuda")[:, None]) % one.T).double() * (2 * math.pi / one.T)
     F = torch.stack([ang.cos(), ang.sin()], 1).reshape(one.M, n_mid)
     for shape in (folded, folded.with_(B=1)):
@@ -86,7 +86,7 @@ def test_folded_blocks(kw):
 
 def test_folded_rows_of_different_length():
     """Rows of odd and even numbers of blocks, one too short for the path, in one call: each as its row alone (too little work to be folded)."""
-    shape = _shape(B=5, Hkv=28, Hq=28, L=6000, M=512, T=16384, n_full_k=24, n_full_v=48)
+    shape = _shape(B=5, Hkv=48, Hq=48, L=6000, M=512, T=16384, n_full_k=24, n_full_v=48)       # 768 positions: folded
     layout = layout_of(shape, max_mid=shape.T, P=16)
     stream = synth.KVStream(shape, seed=10, device="cuda", freq="offgrid")
     K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
