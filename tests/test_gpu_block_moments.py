@@ -340,3 +340,27 @@ def test_not_finite_dims_stay_alone():
     assert not torch.isfinite(got.coef_k[0, 1, :, 5]).all()
     den = want.coef_k.abs().max()
     assert ((got.coef_k - want.coef_k).abs()[rest] <= 2e-6 * den).all()
+
+
+def test_not_finite_dims_stay_alone_in_pairs_of_blocks():
+    """The same where blocks are folded (30 rows of three pairs and eight heads), whose sums and differences meet in an operand: a dim with a NaN and an infinity in
+    the two blocks of a pair, one with a NaN in the block by itself; windows full of NaN do not reach the middle."""
+    shape = _shape(B=30, Hkv=8, Hq=8, M=512, T=16384, L=68 + 4 * 384 + 100)
+    layout = layout_of(shape, max_mid=shape.T, P=16)
+    stream = synth.KVStream(shape, seed=4, device="cuda", freq="offgrid")
+    K, V = stream.tokens(0, shape.L, work_dtype=torch.float32)
+    ws = fa.new_workspace(layout)
+    want = _compress(layout, stream, K, V, ws)
+    for X in (K, V):
+        X[:, :4], X[:, -64:] = float("nan"), float("nan")
+    K[3, 4 + 10, 1, int(want.idx_comp_k[1, 5])] = float("inf")              # blocks 0 and 4 are a pair, 2 the one in the middle
+    K[3, 4 + 4 * 384 + 50, 1, int(want.idx_comp_k[1, 5])] = float("nan")
+    V[29, 4 + 2 * 384 + 7, 6, int(want.idx_comp_v[6, 95])] = float("nan")
+    K[0, 900, 0, int(want.idx_full_k[0, 3])] = float("nan")
+    got = _compress(layout, stream, K, V, ws)
+    for side, bad in (("coef_k", (3, 1, 5)), ("coef_v", (29, 6, 95))):
+        x, y = getattr(got, side), getattr(want, side)
+        rest = torch.ones_like(x, dtype=torch.bool)
+        rest[bad[0], bad[1], :, bad[2]] = False
+        assert not torch.isfinite(x[bad[0], bad[1], :, bad[2]]).any()
+        assert ((x - y).abs()[rest] <= 2e-6 * y.abs().max()).all()          # (comparison with a NaN is false)

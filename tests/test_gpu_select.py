@@ -125,6 +125,24 @@ def test_reconstruction_by_block_moments(kw):
     assert ok.all()
 
 
+def test_not_finite_dims_stay_alone():
+    """By block moments, a NaN or an infinity in the middle spoils the error of its dim only (row 1's here), and what the windows hold does not reach the
+    errors.  Bound: two runs of the test above, with mean squares of at most 4 for a dim and for what is rebuilt of it."""
+    shape = synth.Shape("seln", B=2, layers=1, Hq=24, Hkv=24, d=128, L=1153 + 36, dtype="bf16", n_full_k=32, n_full_v=24, M=256, T=4096, L_init=4, L_local=32)
+    layout = layout_of(shape, max_mid=shape.T, P=16)
+    K, V = synth.KVStream(shape, seed=29, device="cuda", freq="offgrid").tokens(0, shape.L, work_dtype=torch.float32)
+    want = fa.fa_select_dims(layout, K, V)[4]
+    for X in (K, V):
+        X[:, :4], X[:, -32:] = float("nan"), float("-inf")
+    K[1, 4 + 1152, 5, 17], V[1, 4 + 300, 23, 127], V[1, 4, 0, 64] = float("nan"), float("inf"), float("nan")
+    got = fa.fa_select_dims(layout, K, V)[4]
+    bad = torch.zeros_like(got, dtype=torch.bool)
+    for h, side, e in ((5, 0, 17), (23, 1, 127), (0, 1, 64)):
+        bad[1, h, side, e] = True
+    assert not torch.isfinite(got[bad]).any()
+    assert ((got - want).abs() <= 2 * (4e-5 * (want * 8).sqrt() + 1e-8 * 8))[~bad].all()
+
+
 def test_select_workspace_of_an_older_size():
     """A workspace without room for the moments is taken as before, by the direct contractions."""
     import ctypes as C
