@@ -3,6 +3,8 @@
 //   z[m] += p_j F[m][j];  window tokens: ordinary attention in the same softmax.
 // The M basis terms of every token are summed one by one (any period, any class count):
 // the reference of the GPU side and the fallback of the transform kernel.
+#include <type_traits>
+
 #include "fa_common.cuh"
 #include "fa_decode_ws.cuh"
 
@@ -44,9 +46,12 @@ __device__ __forceinline__ void block_max(float (&v)[GH], float* red_s /* [8][GH
     __syncthreads();
 }
 
-template <typename KV, int GH>
-__global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, DecodePlan p, const KV* __restrict__ q,
+// OCC: CTAs to an SM, by registers.  The first two (three with fewer than four heads) leave room to fetch the rows of the first tile, and form its kept-dim scores and
+// basis, in front of the wait for u.
+template <typename KV, int GH, int OCC>
+__global__ void __launch_bounds__(256, OCC) decode_direct_kernel(Dims s, CacheDev c, DecodePlan p, const KV* __restrict__ q,
                                                             char* wsp) {
+    constexpr bool AHEAD = OCC == 2 || (OCC == 3 && GH < 4);
     extern __shared__ float sm[];
     Ws ws = ws_view(wsp, p);
     const int split = blockIdx.x;
@@ -67,7 +72,7 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
     float* acc_s = o_s + GH * s.d;            // [256][GH] cross-thread reduce of the output accumulators
 
     // Everything but u was there before this call: the kernel in front lets this one start when the work before it has ended.  The rows of the
-    // first tile are fetched, and their kept-dim scores formed, while that kernel makes u.
+    // first tile are fetched, and their kept-dim scores formed, while that kernel makes u (AHEAD).
     const int4 st4 = *reinterpret_cast<const int4*>(c.state + kStateStride * b);
     const int n_init = st4.x, n_local = st4.y, n_mid = min(st4.z, s.max_mid), head = st4.w;
     const int32_t* idf_v = c.idx_full_v + (size_t)h * s.nfv;
@@ -88,17 +93,17 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
         const int slot = slot_of(j);
         return ld_f(mid_row<KV>(c.v_mid, s, b, h, cls_of(j), slot, s.nfv) + v_mid_col(slot, e_mid, s.nfv, sizeof(KV) == 2 ? FA_BF16 : FA_F32));
     };
-    constexpr int kPre = 8;                                 // values of K and of V of the first tile that a thread fetches ahead
+    constexpr int kPre = AHEAD ? 8 : 1;                     // values of K and of V of the first tile that a thread fetches ahead
     float k_pre[kPre], v_pre[kPre];
-    {
+    if (AHEAD) {
         const KV* row = j0 + tk < j1 ? k_row(j0 + tk) : nullptr;
 #pragma unroll
         for (int u = 0; u < kPre; ++u) k_pre[u] = row && ql + u * kLanes < s.nfk ? ld_f(row + ql + u * kLanes) : 0.f;
-    }
 #pragma unroll
-    for (int u = 0; u < kPre; ++u) {
-        const int j = j0 + tg_mid + u * ntg_mid;
-        v_pre[u] = act_mid && j < min(j1, j0 + kTile) ? v_at(j) : 0.f;
+        for (int u = 0; u < kPre; ++u) {
+            const int j = j0 + tg_mid + u * ntg_mid;
+            v_pre[u] = act_mid && j < min(j1, j0 + kTile) ? v_at(j) : 0.f;
+        }
     }
 
     for (int i = tid; i < GH * s.d; i += blockDim.x) {
@@ -169,7 +174,7 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
         if (j >= j1) return;
         const KV* row = k_row(j);
         int e = ql;
-        if (ahead)
+        if (AHEAD && ahead)
 #pragma unroll
             for (int u = 0; u < kPre; ++u, e += kLanes)
                 if (e < s.nfk)
@@ -183,11 +188,13 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
         }
     };
     float sc_first[GH];
-    kept_scores(j0 + tk, sc_first, true);
     // the basis of the first tile: a token's rotation and its lane's first frequency; a frequency's rotation and its first token
     float cd1 = 0.f, sd1 = 0.f, cr1 = 0.f, sr1 = 0.f, zc1 = 0.f, zs1 = 0.f, zr1 = 0.f, zi1 = 0.f;
-    if (s.dck > 0 && j0 + tk < j1) { basis_cs(1, j0 + tk, s.T, &cd1, &sd1); basis_cs(ql * per_lane, j0 + tk, s.T, &cr1, &sr1); }
-    if (s.dcv > 0 && zn < s.k) { basis_cs(zn, 1, s.T, &zc1, &zs1); basis_cs(zn, j0 + zt * (kTile / n_grp), s.T, &zr1, &zi1); }
+    if (AHEAD) {
+        kept_scores(j0 + tk, sc_first, true);
+        if (s.dck > 0 && j0 + tk < j1) { basis_cs(1, j0 + tk, s.T, &cd1, &sd1); basis_cs(ql * per_lane, j0 + tk, s.T, &cr1, &sr1); }
+        if (s.dcv > 0 && zn < s.k) { basis_cs(zn, 1, s.T, &zc1, &zs1); basis_cs(zn, j0 + zt * (kTile / n_grp), s.T, &zr1, &zi1); }
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");     // u
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (int i = tid; i < GH * s.M; i += blockDim.x) {
@@ -200,7 +207,8 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
         const bool valid = j < j1;
         const int nt = min(kTile, j1 - t0);
         float sc[GH];
-        if (t0 == j0) {
+        const bool first_tile = AHEAD && t0 == j0;
+        if (first_tile) {
 #pragma unroll
             for (int g = 0; g < GH; ++g) sc[g] = sc_first[g];
         } else {
@@ -209,12 +217,12 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
         if (valid) {
             if (s.dck > 0) {
                 float cd, sd;
-                if (t0 == j0) { cd = cd1; sd = sd1; }
+                if (first_tile) { cd = cd1; sd = sd1; }
                 else basis_cs(1, j, s.T, &cd, &sd);             // rotation per unit of n
                 const int f1 = min(s.k, (ql + 1) * per_lane);
                 for (int n0 = ql * per_lane; n0 < f1; n0 += 32) {
                     float cr, sr;
-                    if (t0 == j0 && n0 == ql * per_lane) { cr = cr1; sr = sr1; }
+                    if (first_tile && n0 == ql * per_lane) { cr = cr1; sr = sr1; }
                     else basis_cs(n0, j, s.T, &cr, &sr);        // exact re-seed
                     const int n1 = min(f1, n0 + 32);
 #pragma unroll 4
@@ -236,7 +244,7 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
         // o^u += p V^mu
         if (act_mid) {
             int i = tg_mid;
-            if (t0 == j0) {
+            if (first_tile) {
 #pragma unroll
                 for (int u = 0; u < kPre; ++u, i += ntg_mid) {
                     if (i < nt)
@@ -261,10 +269,10 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
                 for (int g = 0; g < GH; ++g) { zr[g] = 0.f; zi[g] = 0.f; }
                 if (n < s.k && i0 < i1) {
                     float cd, sd, cr, sr;
-                    if (nb == 0) { cd = zc1; sd = zs1; }
+                    if (AHEAD && nb == 0) { cd = zc1; sd = zs1; }
                     else basis_cs(n, 1, s.T, &cd, &sd);
                     for (int ia = i0; ia < i1; ia += 32) {
-                        if (t0 == j0 && nb == 0 && ia == i0) { cr = zr1; sr = zi1; }
+                        if (first_tile && nb == 0 && ia == i0) { cr = zr1; sr = zi1; }
                         else basis_cs(n, t0 + ia, s.T, &cr, &sr);
                         const int ib = min(i1, ia + 32);
 #pragma unroll 4
@@ -386,12 +394,14 @@ __global__ void __launch_bounds__(256) decode_direct_kernel(Dims s, CacheDev c, 
 }
 
 
-template <typename KV, int GH>
+static size_t direct_smem(const Dims& s, int gh) {
+    return sizeof(float) * ((size_t)gh * s.d * 2 + (size_t)gh * s.nfk + 2 * (size_t)gh * s.M + (size_t)gh * kTile + 8 * gh + (size_t)(256 + 512) * gh);
+}
+template <typename KV, int GH, int OCC>
 static cudaError_t launch_direct_t(const Dims& s, const CacheDev& c, const DecodePlan& p, const void* q, char* ws,
                                    cudaStream_t st) {
-    size_t smem = sizeof(float) * ((size_t)GH * s.d * 2 + (size_t)GH * s.nfk + 2 * (size_t)GH * s.M + (size_t)GH * kTile +
-                                   8 * GH + (size_t)(256 + 512) * GH);
-    cudaError_t err = ensure_dynamic_smem(decode_direct_kernel<KV, GH>, smem);
+    const size_t smem = direct_smem(s, GH);
+    cudaError_t err = ensure_dynamic_smem(decode_direct_kernel<KV, GH, OCC>, smem);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.n_split, s.Hkv * p.n_pass, s.B);
@@ -403,19 +413,38 @@ static cudaError_t launch_direct_t(const Dims& s, const CacheDev& c, const Decod
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, decode_direct_kernel<KV, GH>, s, c, p, static_cast<const KV*>(q), ws);
+    return cudaLaunchKernelEx(&cfg, decode_direct_kernel<KV, GH, OCC>, s, c, p, static_cast<const KV*>(q), ws);
+}
+
+// As many CTAs to an SM as the grid needs to run at once, or as many as there can be.  Registers that a wave does not need fetch ahead; and CTAs that start while the
+// kernel in front ends crowd on the SMs that it leaves first, up to this number.  The call, us, two CTAs to an SM / three (four heads): 16 CTAs (1 K tokens) 18.1/20.0,
+// 72 27.4/28.6, 296 (2 K) 39.3/45.2; 304 (8 K) 146/111, 320 (a prompt of 5.8 K) 332/242, 384 (23 K) 2577/1554.  One head: 296 CTAs (10 K tokens) 177 with
+// as many as three to an SM, 133 with two.
+static int direct_occ(const Dims& s, const DecodePlan& p) {
+    const int most = p.gh == 4 ? 3 : 4, held = (int)(227 * 1024 / (direct_smem(s, p.gh) + 1024));
+    const long long ctas = (long long)p.n_split * s.Hkv * p.n_pass * s.B;
+    int occ = 2;
+    while (occ < most && occ < held && ctas > (long long)occ * sm_count()) ++occ;
+    return occ;
 }
 
 cudaError_t launch_decode_direct(const Dims& s, const CacheDev& c, int dtype, const DecodePlan& p, const void* q, char* ws,
                                  cudaStream_t st) {
-    if (dtype == FA_BF16) {
-        if (p.gh == 4) return launch_direct_t<__nv_bfloat16, 4>(s, c, p, q, ws, st);
-        if (p.gh == 2) return launch_direct_t<__nv_bfloat16, 2>(s, c, p, q, ws, st);
-        return launch_direct_t<__nv_bfloat16, 1>(s, c, p, q, ws, st);
-    }
-    if (p.gh == 4) return launch_direct_t<float, 4>(s, c, p, q, ws, st);
-    if (p.gh == 2) return launch_direct_t<float, 2>(s, c, p, q, ws, st);
-    return launch_direct_t<float, 1>(s, c, p, q, ws, st);
+    using std::integral_constant;
+    const int occ = direct_occ(s, p);
+    auto by_occ = [&](auto kv, auto heads) {
+        using KV = decltype(kv);
+        constexpr int GH = decltype(heads)::value;
+        if (occ == 2) return launch_direct_t<KV, GH, 2>(s, c, p, q, ws, st);
+        if (occ == 3) return launch_direct_t<KV, GH, 3>(s, c, p, q, ws, st);
+        return launch_direct_t<KV, GH, GH == 4 ? 3 : 4>(s, c, p, q, ws, st);
+    };
+    auto by_heads = [&](auto kv) {
+        if (p.gh == 4) return by_occ(kv, integral_constant<int, 4>{});
+        if (p.gh == 2) return by_occ(kv, integral_constant<int, 2>{});
+        return by_occ(kv, integral_constant<int, 1>{});
+    };
+    return dtype == FA_BF16 ? by_heads(__nv_bfloat16{}) : by_heads(float{});
 }
 
 }  // namespace fa
