@@ -26,9 +26,10 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---------------------------------------------------------------- prologue --
-// grid (ceil(M / rows_pro), Hkv, B), 256 threads.
-template <typename KV>
-__global__ void __launch_bounds__(256) decode_prologue_kernel(Dims s, CacheDev c, DecodePlan p, const KV* __restrict__ q,
+// grid (ceil(M / rows_pro), Hkv, B), 256 threads.  SHORT: fewest round trips and shortest chains, for a grid that is one wave; else fewest instructions and
+// registers, eight CTAs to an SM.  The call, us, SHORT / else: 64 CTAs 25.6/26.4, 256 27.0/27.8, 512 29.3/29.5, 1024 38.8/38.7, 4096 84.4/78.3, 8192 107/95, 12288 200/179.
+template <typename KV, bool SHORT>
+__global__ void __launch_bounds__(256, SHORT ? 4 : 8) decode_prologue_kernel(Dims s, CacheDev c, DecodePlan p, const KV* __restrict__ q,
                                                               char* wsp) {
     extern __shared__ __align__(16) float sm_pro[];
     pdl_wait();                                            // coefficients, query; the workspace
@@ -40,7 +41,7 @@ __global__ void __launch_bounds__(256) decode_prologue_kernel(Dims s, CacheDev c
     const int stride = s.dck + 4;                      // row stride of the tile: 16-byte aligned, bank-skewed
     float* tile = sm_pro;                              // [rows_pro][stride]
     float* qc_s = tile + p.rows_pro * stride;          // [G][dck] gathered query
-    float* q_s = qc_s + s.G * s.dck;                   // [G][d] query rows
+    float* q_s = qc_s + (SHORT ? s.G * s.dck : 0);     // [G][d] query rows; else [G][dck + 1] gathered query
     const int m0 = blockIdx.x * p.rows_pro;
     const int rows = min(p.rows_pro, s.M - m0);
     const float* coef = coef_rows(c.coef_k, s, b, h, s.dck) + (size_t)m0 * s.dck;
@@ -48,6 +49,28 @@ __global__ void __launch_bounds__(256) decode_prologue_kernel(Dims s, CacheDev c
     for (int i = tid; i < rows * vpr; i += 256) {
         int r = i / vpr, v4 = i - r * vpr;
         cp_async16(tile + r * stride + 4 * v4, coef + (size_t)r * s.dck + 4 * v4);
+    }
+    if constexpr (!SHORT) {                            // a thread per row and head
+        const int32_t* idc = c.idx_comp_k + (size_t)h * s.dck;
+        for (int i = tid; i < s.G * s.dck; i += 256) {
+            const int g = i / s.dck, e = i - g * s.dck;
+            q_s[g * (s.dck + 1) + e] = ld_f(q + ((size_t)b * s.Hq + h * s.G + g) * s.d + idc[e]);
+        }
+        cp_async_wait_all();
+        __syncthreads();
+        for (int t = tid; t < rows * s.G; t += 256) {
+            const int g = t % s.G, r = t / s.G, m = m0 + r;
+            const float *row = tile + r * stride, *qq = q_s + g * (s.dck + 1);
+            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+            for (int e = 0; e < s.dck; e += 4) {
+                a0 = fmaf(row[e], qq[e], a0);
+                a1 = fmaf(row[e + 1], qq[e + 1], a1);
+                a2 = fmaf(row[e + 2], qq[e + 2], a2);
+                a3 = fmaf(row[e + 3], qq[e + 3], a3);
+            }
+            ws.u[((size_t)b * s.Hq + h * s.G + g) * s.M + m] = recon_weight(s.norm, m, s.k, s.T) * s.scale * kLog2e * ((a0 + a1) + (a2 + a3));
+        }
+        return;
     }
     // (whole rows of q beside the index set: gathered from memory, q would be a second round trip behind it)
     const int idx = tid < s.dck ? c.idx_comp_k[(size_t)h * s.dck + tid] : 0;
@@ -97,8 +120,10 @@ __host__ __device__ inline size_t epilogue_l(const Dims& s, const DecodePlan& p)
     const size_t a = (size_t)s.G * p.n_part, b = p.n_slice == 1 ? (size_t)s.G * s.dcv : 0;
     return a > b ? a : b;
 }
-template <typename KV>
-__global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c, DecodePlan p, KV* __restrict__ out,
+// SHORT: the first parts' z and o with the statistics, the product shared out over all threads, in 125 registers (two CTAs to an SM); for grids
+// that fill no more.  The call, us, SHORT / else: 16 CTAs 30.9/38.0, 32 39.1/43.5, 192 83/93, 256 34.7/38.0; 384 29.5/22.0, 384 54.1/51.4, 1024 95.5/82.9, 4096 139/94.
+template <typename KV, bool SHORT>
+__global__ void __launch_bounds__(256, SHORT ? 2 : 5) decode_epilogue_kernel(Dims s, CacheDev c, DecodePlan p, KV* __restrict__ out,
                                                               char* wsp) {
     extern __shared__ __align__(16) float sm_epi[];
     __shared__ int last_s;
@@ -132,14 +157,14 @@ __global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c
     pdl_wait();                                            // partial results of the main kernel are complete
 
     // What a thread needs of the first kPre parts comes with the statistics, in one round trip: its first entry of z, and, where this CTA
-    // finishes its head alone, its first two of o.
+    // finishes its head alone, its first two of o (SHORT).
     const bool alone = p.n_slice == 1;
     const size_t qh0 = (size_t)b * s.Hq + h * s.G;
     auto z_of = [&](int t) { const int g = t / rows, r = t - g * rows; return ws.z + (qh0 + g) * ns * s.M + m0 + r; };
     auto o_of = [&](int t) { const int g = t / s.d, e = t - g * s.d; return ws.o + (qh0 + g) * ns * s.d + e; };
-    constexpr int kPre = 16;
+    constexpr int kPre = SHORT ? 16 : 2;
     float zp[kPre], op[2][kPre];
-    {
+    if (SHORT) {
         const bool z_on = s.dcv > 0 && tid < s.G * rows;
         const float* z = z_on ? z_of(tid) : nullptr;
 #pragma unroll
@@ -156,7 +181,7 @@ __global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c
     auto merge = [&](const float* x, size_t stride, const float* al, const float (&pre)[kPre], bool have) {
         float v0 = 0.f, v1 = 0.f;
         int sp = 0;
-        if (have) {
+        if (SHORT && have) {
 #pragma unroll
             for (int i = 0; i < kPre; i += 2) {
                 if (i < ns) v0 = fmaf(al[i], pre[i], v0);
@@ -204,6 +229,21 @@ __global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c
         }
         cp_async_wait_all();
         __syncthreads();
+        if constexpr (!SHORT) {                            // a thread per column and head
+            for (int t = tid; t < s.G * s.dcv; t += 256) {
+                const int g = t / s.dcv, e = t - g * s.dcv;
+                const float* zw = zw_s + g * rows_max;
+                float a0 = 0.f, a1 = 0.f;
+                int r = 0;
+                for (; r + 2 <= rows; r += 2) {
+                    a0 = fmaf(zw[r], tile[r * stride + e], a0);
+                    a1 = fmaf(zw[r + 1], tile[(r + 1) * stride + e], a1);
+                }
+                if (r < rows) a0 = fmaf(zw[r], tile[r * stride + e], a0);
+                if (alone) oc_s[t] = a0 + a1;
+                else ws.oc[((qh0 + g) * p.n_slice + slice) * s.dcv + e] = a0 + a1;
+            }
+        } else {
         // a thread takes four columns and every nrg-th row, four heads at a time; then the row groups are added in order
         const int nv = s.dcv >> 2, nrg = 256 / nv, rg = tid / nv, v = tid - rg * nv;
         for (int g0 = 0; g0 < s.G; g0 += 4) {
@@ -239,6 +279,7 @@ __global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c
                 if (alone) oc_s[g0 * s.dcv + t] = x;
                 else ws.oc[((qh0 + g0 + g) * p.n_slice + slice) * s.dcv + t - g * s.dcv] = x;
             }
+        }
         }
     }
     if (!alone) {
@@ -279,9 +320,11 @@ __global__ void __launch_bounds__(256) decode_epilogue_kernel(Dims s, CacheDev c
         }
         st_f(out + (qh0 + g) * s.d + e, v * linv_s[g]);
     };
-    if (tid < s.G * s.d) finish(tid, op[0], alone);
-    if (tid + 256 < s.G * s.d) finish(tid + 256, op[1], alone);
-    for (int t = tid + 512; t < s.G * s.d; t += 256) finish(t, op[0], false);
+    if (SHORT) {
+        if (tid < s.G * s.d) finish(tid, op[0], alone);
+        if (tid + 256 < s.G * s.d) finish(tid + 256, op[1], alone);
+    }
+    for (int t = tid + (SHORT ? 512 : 0); t < s.G * s.d; t += 256) finish(t, op[0], false);
 }
 
 // ---------------------------------------------------------------- launchers --
@@ -307,10 +350,14 @@ template <typename KV>
 static cudaError_t launch_prologue_t(const Dims& s, const CacheDev& c, const DecodePlan& p, const void* q, char* ws,
                                      cudaStream_t st) {
     const int tiles = s.dck > 0 ? (s.M + p.rows_pro - 1) / p.rows_pro : 1;
-    const size_t smem = sizeof(float) * ((size_t)p.rows_pro * (s.dck + 4) + (size_t)s.G * (s.dck + s.d));
-    cudaError_t err = ensure_dynamic_smem(decode_prologue_kernel<KV>, smem);
-    if (err != cudaSuccess) return err;
-    return launch_pdl(decode_prologue_kernel<KV>, dim3(tiles, s.Hkv, s.B), dim3(256), smem, st, true, s, c, p, static_cast<const KV*>(q), ws);
+    const bool one_wave = (long long)tiles * s.Hkv * s.B <= 4ll * sm_count();
+    const size_t smem = sizeof(float) * ((size_t)p.rows_pro * (s.dck + 4) + (size_t)s.G * (one_wave ? s.dck + s.d : s.dck + 1));
+    auto go = [&](auto kernel) {
+        cudaError_t err = ensure_dynamic_smem(kernel, smem);
+        if (err != cudaSuccess) return err;
+        return launch_pdl(kernel, dim3(tiles, s.Hkv, s.B), dim3(256), smem, st, true, s, c, p, static_cast<const KV*>(q), ws);
+    };
+    return one_wave ? go(decode_prologue_kernel<KV, true>) : go(decode_prologue_kernel<KV, false>);
 }
 
 cudaError_t launch_decode_prologue(const Dims& s, const CacheDev& c, int dtype, const DecodePlan& p, const void* q,
@@ -323,11 +370,15 @@ template <typename KV>
 static cudaError_t launch_epilogue_t(const Dims& s, const CacheDev& c, const DecodePlan& p, void* out, char* ws,
                                      cudaStream_t st) {
     const int rows = (s.M + p.n_slice - 1) / p.n_slice;
-    const size_t smem = sizeof(float) * ((size_t)s.G * p.n_part + epilogue_l(s, p) + s.G + (size_t)s.G * rows + s.d + 4 + (size_t)rows * (s.dcv + 4) + 4 * 1024);      // (256 threads' four columns of four heads)
-    cudaError_t err = ensure_dynamic_smem(decode_epilogue_kernel<KV>, smem);
-    if (err != cudaSuccess) return err;
-    return launch_pdl(decode_epilogue_kernel<KV>, dim3(p.n_slice, s.Hkv, s.B), dim3(256), smem, st, true, s, c, p,
-                      static_cast<KV*>(out), ws);
+    const bool one_wave = (long long)p.n_slice * s.Hkv * s.B <= 2ll * sm_count();
+    const size_t smem = sizeof(float) * ((size_t)s.G * p.n_part + epilogue_l(s, p) + s.G + (size_t)s.G * rows + s.d + 4 + (size_t)rows * (s.dcv + 4) +
+                                         (one_wave ? 4 * 1024 : 0));      // (256 threads' four columns of four heads)
+    auto go = [&](auto kernel) {
+        cudaError_t err = ensure_dynamic_smem(kernel, smem);
+        if (err != cudaSuccess) return err;
+        return launch_pdl(kernel, dim3(p.n_slice, s.Hkv, s.B), dim3(256), smem, st, true, s, c, p, static_cast<KV*>(out), ws);
+    };
+    return one_wave ? go(decode_epilogue_kernel<KV, true>) : go(decode_epilogue_kernel<KV, false>);
 }
 
 cudaError_t launch_decode_epilogue(const Dims& s, const CacheDev& c, int dtype, const DecodePlan& p, void* out, char* ws,
