@@ -149,10 +149,8 @@ __global__ void __launch_bounds__(256) partition_gather_kernel(Dims s, CacheDev 
 // tile in shared memory; thread (rg, lane) accumulates rows 4 rg..4 rg + 3 of
 // the tile for columns lane, lane + 32, ...  Partial sums of the token splits
 // are added to the zeroed coefficients with atomics.
-// R rows per thread: eight where tiles of 64 rows and chunks of 64 tokens make two CTAs to an SM (half the shared-memory reads per product), else
-// four.  us, four / eight rows:  tiles x chunks 80 11.3/13.3, 112 17.4/17.4, 136 29.7/31.7 (a selection), 160 46.1/46.1, 480 64/59 and, four layers, 159/134,
-// 896 70/62 (8 rows of 8 KV heads, 700 tokens, 64 coefficients).  Bound by the FMA and shared-memory pipes beside a chain of index, load and
-// barrier per chunk.
+// R rows per thread: eight (half the shared-memory reads per product) or four (finer tiles, more CTAs and fewer registers), see rows_per_thread.  Bound by the FMA and
+// shared-memory pipes beside a chain of index, load and barrier per chunk.
 constexpr int kTJ = 64;
 
 // NC: columns per lane (32 NC >= the compressed dims of either side; the products of lanes without a column are not issued).
@@ -243,6 +241,33 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
     }
 }
 
+// Rows per thread of the contraction, and how the tokens' chunks are split: what the SM with the most CTAs takes for them, a chunk counting as the products of a
+// lane's token and 10 of them more (with eight rows of eight columns, registers for one CTA to an SM, 1.3 times those), and a CTA by itself 60 at least.  Of 854 calls (16
+// to 2048 coefficients, 1 to 256 heads, 20 to 6000 tokens, 64 to 256 dims) 0.6 % behind the better form on average.  us, four / eight rows a thread:
+//   tiles of 64 rows that would be half empty: 16 coefficients, 32 heads, 900 tokens 149/264; 32 coefficients, 32 heads, 340 tokens 17.2/25.7
+//   many CTAs: 200 coefficients, 128 heads, 5600 tokens 1234/1106 (ragged); 128, 48 heads, 590 tokens 101/85; few: 16.9/16.1, 12.8/11.4
+//   256 dims: 1024 coefficients, 32 heads 4880/6181; 100, 96 heads 459/544; few CTAs: 100, two heads 25.5/21.4
+//   a fixed order (a CTA takes all tokens of its rows): 100 coefficients, 8 heads, 1300 tokens 69/100; 256, 32 heads, 240 tokens 60/47; 128, 64 heads, 1000 tokens 191/228
+struct RowSplit { int rpt, row_tiles, n_tsplit, cps; };
+static RowSplit rows_per_thread(const Dims& s, int live_rows, int chunks, int nc, bool ordered) {
+    RowSplit best = {};
+    double least = 0;
+    const int sms = sm_count();
+    for (int rpt = 4; rpt <= 8; rpt += 4) {
+        RowSplit x = {rpt, (s.M + 8 * rpt - 1) / (8 * rpt), 1, 0};
+        const int ctas_fixed = x.row_tiles * live_rows * s.Hkv * 2;
+        int n = (4 * sms + ctas_fixed - 1) / ctas_fixed;
+        if (n > chunks) n = chunks;
+        if (n < 1 || ordered) n = 1;                         // one split: every coefficient is added to zero exactly once
+        x.cps = (chunks + n - 1) / n;
+        x.n_tsplit = (chunks + x.cps - 1) / x.cps;
+        const double chunk = 10 + rpt * nc * (rpt == 8 && nc == 8 ? 1.3 : 1.0), all = ((ctas_fixed * x.n_tsplit + sms - 1) / sms) * chunk;
+        const double time = x.cps * (all > 60 ? all : 60);
+        if (best.rpt == 0 || time < least) { best = x; least = time; }
+    }
+    return best;
+}
+
 template <typename KV>
 static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const void* K, const void* V, int64_t sb,
                                      int64_t st, int64_t sh, int L, bool with_coef, bool ordered, int tc_min, int zero_coef, bool chained,
@@ -287,20 +312,13 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     int max_comp = s.dck > s.dcv ? s.dck : s.dcv;
     if (n_mid == 0 || max_comp == 0 || !with_coef) return cudaSuccess;
     const int live_rows = rl.n ? n_short : s.B;
-    int chunks = (n_mid + kTJ - 1) / kTJ;
-    const int rpt = (long long)((s.M + 63) / 64) * live_rows * s.Hkv * 2 * chunks >= 2 * sm_count() ? 8 : 4;
-    const int row_tiles = (s.M + 8 * rpt - 1) / (8 * rpt);
-    int ctas_fixed = row_tiles * live_rows * s.Hkv * 2;
-    int n_tsplit = (4 * sm_count() + ctas_fixed - 1) / ctas_fixed;
-    if (n_tsplit > chunks) n_tsplit = chunks;
-    if (n_tsplit < 1 || ordered) n_tsplit = 1;               // one split: every coefficient is added to zero exactly once
-    int cps = (chunks + n_tsplit - 1) / n_tsplit;
-    n_tsplit = (chunks + cps - 1) / cps;
     const int nc = max_comp <= 128 ? (max_comp + 31) / 32 : 8;
+    const RowSplit split = rows_per_thread(s, live_rows, (n_mid + kTJ - 1) / kTJ, nc, ordered);
+    const int rpt = split.rpt, cps = split.cps;
     const size_t smem = sizeof(float) * kTJ * (size_t)(32 * nc + 8 * rpt);
     // behind the partition kernel programmatically: it waits for it in front of its additions
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(row_tiles, n_tsplit, s.B * s.Hkv * 2);
+    cfg.gridDim = dim3(split.row_tiles, split.n_tsplit, s.B * s.Hkv * 2);
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
