@@ -416,15 +416,17 @@ static cudaError_t launch_direct_t(const Dims& s, const CacheDev& c, const Decod
     return cudaLaunchKernelEx(&cfg, decode_direct_kernel<KV, GH, OCC>, s, c, p, static_cast<const KV*>(q), ws);
 }
 
-// As many CTAs to an SM as the grid needs to run at once, or as many as there can be.  Registers that a wave does not need fetch ahead; and CTAs that start while the
-// kernel in front ends crowd on the SMs that it leaves first, up to this number.  The call, us, two CTAs to an SM / three (four heads): 16 CTAs (1 K tokens) 18.1/20.0,
-// 72 27.4/28.6, 296 (2 K) 39.3/45.2; 304 (8 K) 146/111, 320 (a prompt of 5.8 K) 332/242, 384 (23 K) 2577/1554.  One head: 296 CTAs (10 K tokens) 177 with
-// as many as three to an SM, 133 with two.
+// The fewest CTAs to an SM with which the grid takes no more waves.  Registers that a wave does not need fetch ahead; and CTAs that start while the kernel in front
+// ends crowd on the SMs that it leaves first, up to this number.  The call, us, two CTAs to an SM / three (four heads): 16 CTAs (1 K tokens) 18.1/20.0,
+// 72 27.4/28.6, 296 (2 K) 39.3/45.2; 304 (8 K) 146/111, 320 (a prompt of 5.8 K) 332/242, 384 (23 K) 2577/1554; of 512 53 calls 2 % faster with two, of 768 17 % slower.  One head:
+// 296 CTAs (10 K tokens) 177 with as many as three to an SM, 133 with two.
 static int direct_occ(const Dims& s, const DecodePlan& p) {
-    const int most = p.gh == 4 ? 3 : 4, held = (int)(227 * 1024 / (direct_smem(s, p.gh) + 1024));
+    const int most = p.gh == 4 ? 3 : 4, held = (int)(227 * 1024 / (direct_smem(s, p.gh) + 1024)), sms = sm_count();
     const long long ctas = (long long)p.n_split * s.Hkv * p.n_pass * s.B;
+    auto waves = [&](int occ) { return (ctas + (long long)occ * sms - 1) / ((long long)occ * sms); };
     int occ = 2;
-    while (occ < most && occ < held && ctas > (long long)occ * sm_count()) ++occ;
+    for (int more = 3; more <= most && more <= held; ++more)
+        if (waves(more) < waves(occ)) occ = more;
     return occ;
 }
 
