@@ -47,9 +47,10 @@ __device__ __forceinline__ void block_max(float (&v)[GH], float* red_s /* [8][GH
 }
 
 // OCC: CTAs to an SM, by registers.  The first two (three with fewer than four heads) leave room to fetch the rows of the first tile, and form its kept-dim scores and
-// basis, in front of the wait for u.
+// basis, in front of the wait for u.  (Three with four heads come out at 80 registers by themselves; told so, the compiler's order of the loops over frequencies is up
+// to 8 % slower: 320 CTAs of 1.3 K fp32 tokens 831 and 778 us.)
 template <typename KV, int GH, int OCC>
-__global__ void __launch_bounds__(256, OCC) decode_direct_kernel(Dims s, CacheDev c, DecodePlan p, const KV* __restrict__ q,
+__global__ void __launch_bounds__(256, OCC == 3 && GH == 4 ? 0 : OCC) decode_direct_kernel(Dims s, CacheDev c, DecodePlan p, const KV* __restrict__ q,
                                                             char* wsp) {
     constexpr bool AHEAD = OCC == 2 || (OCC == 3 && GH < 4);
     extern __shared__ float sm[];
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(256, OCC) decode_direct_kernel(Dims s, CacheDe
             o_mid[g] *= alpha[g];
             o_win[g] *= alpha[g];
         }
-        if (!first)
+        if (!AHEAD || !first)
 #pragma unroll
             for (int g = 0; g < GH; ++g)
                 for (int m = tid; m < s.M; m += 256) z_s[g * s.M + m] *= alpha[g];
