@@ -68,6 +68,7 @@ struct ChanPlan {
     int k_sh, k_mask, v_sh, v_mask;      // swizzle of the K / V rows in a stage: chunk ^ ((row >> sh) & mask)
     int n_cx, n_wpart;       // CTAs per (KV head, pass): class parts of all batch rows, window parts of one
     int nq, nz;              // channel pairs per CTA of the kernels in front and behind, and CTAs of their clusters
+    int wide;                // their CTAs have sixteen warps
     int st_in, st_out;       // stages of their streams of coefficient rows
     size_t off_z, off_w, off_mw, off_ml, off_o, off_g, off_x, off_j, off_p;      // from the start of a layer's areas
     size_t base, per_layer, total;       // one layer's areas in the workspace: their start, size and end

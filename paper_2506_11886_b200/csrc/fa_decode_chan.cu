@@ -33,9 +33,13 @@ constexpr int kMainCtas = 3;         // CTAs of the main kernel to an SM
 constexpr int kWinStage = 4096;      // window parts of the main kernel: 16 rows of K or of V
 // CTAs of the outer kernels to an SM: three where 80 registers do without spills, which several layers in a launch fill (the instances of 64 and 512
 // slots, whose last pass is of eight points, spill 400 bytes there).
-// Threads of an outer kernel's CTA.  The longest transforms leave room for one CTA to an SM: sixteen warps of it instead of eight.
-__host__ __device__ constexpr int outer_threads(int ls) { return ls == 10 ? 512 : 256; }
-__host__ __device__ constexpr int outer_ctas(int ls) { return ls == 10 ? 1 : ls == 5 || ls == 7 || ls == 8 ? 3 : 2; }
+// Threads of an outer kernel's CTA.  Where the longest transforms leave room for one CTA to an SM, it has sixteen warps instead of eight (wide, see plan_channels).
+__host__ __device__ constexpr int outer_threads(bool wide) { return wide ? 512 : 256; }
+__host__ __device__ constexpr int outer_ctas(int ls, bool wide) { return wide ? 1 : ls == 5 || ls == 7 || ls == 8 ? 3 : 2; }
+// Stages of rows that a turn of an outer kernel's loops takes: two of the kernel in front's (eight lanes to a row), and the threads' share; one with the longest transforms
+// in eight warps, whose CTAs have few rows or little room for stages.
+__host__ __device__ constexpr int in_turn(int ls, bool wide) { return ls == 10 && !wide ? 1 : 2; }
+__host__ __device__ constexpr int out_stages(int ls, bool wide) { return ls == 10 && !wide ? 1 : outer_threads(wide) / 128; }
 constexpr double kPartCost = 64 * 1024;          // what a part of the main kernel costs beside its bytes, in bytes
 
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
@@ -94,13 +98,13 @@ __device__ __forceinline__ int split_pairs(int items, int nq, int threads) {
     while ((items << lg) < threads && (2 << lg) <= nq) ++lg;
     return lg;
 }
-template <int LS>
+template <int LS, int NT>
 __device__ __forceinline__ void pass_twiddles(float* twf, int tid) {
     for (int l = LS; l > 0;) {
         const int rl = radix_log2(l), R = 1 << rl, st = 1 << (l - rl);
         if (l > rl) {
             const int off = tw_offset(LS, l);
-            for (int i = tid; i < (R - 1) * st; i += outer_threads(LS)) {
+            for (int i = tid; i < (R - 1) * st; i += NT) {
                 const int qm1 = i >> (l - rl), j = i & (st - 1);
                 reinterpret_cast<float2*>(twf)[off + i] = cis_frac((float)(((qm1 + 1) * j) & ((1 << l) - 1)) * (1.0f / (float)(1 << l)));
             }
@@ -263,12 +267,12 @@ struct ChanCall {
 struct LayerMaps { CUtensorMap km, vm, ki, vi, kl, vl; };
 struct ChanMaps { LayerMaps l[kChanLayers]; };
 
-// Cluster per job, 256 threads.  u = scale log2(e) W C^K q, a slice of the rows per CTA, exchanged through distributed shared
+// Cluster per job.  u = scale log2(e) W C^K q, a slice of the rows per CTA, exchanged through distributed shared
 // memory; then Z of nq channel pairs per CTA (a transform carries channels 2 q and 2 q + 1 of one head).  With k_new (a step, one
 // pass) also the push: C^K's rows are updated on their way, the leaving row's kept dims and the new token are written.
-template <int LS, int NH>
-__global__ void __launch_bounds__(outer_threads(LS), NH == 4 && outer_ctas(LS) == 3 ? 2 : outer_ctas(LS)) chan_in_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
-    constexpr int S = 1 << LS, NT = outer_threads(LS);
+template <int LS, int NH, bool WIDE>
+__global__ void __launch_bounds__(outer_threads(WIDE), NH == 4 && outer_ctas(LS, WIDE) == 3 ? 2 : outer_ctas(LS, WIDE)) chan_in_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
+    constexpr int S = 1 << LS, NT = outer_threads(WIDE);
     extern __shared__ __align__(16) float smz[];
     const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass;
     const int layer = blockIdx.z / s.B, b = blockIdx.z - layer * s.B;
@@ -299,7 +303,7 @@ __global__ void __launch_bounds__(outer_threads(LS), NH == 4 && outer_ctas(LS) =
         *fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    pass_twiddles<LS>(twf, tid);
+    pass_twiddles<LS, NT>(twf, tid);
     channel_factors<NT>(g_s, q0, nq, s.k, S, tid);
     for (int n = tid; n < s.k; n += NT) ph_s[n] = mid_phase(n, s);
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -351,30 +355,33 @@ __global__ void __launch_bounds__(outer_threads(LS), NH == 4 && outer_ctas(LS) =
     }
     // two stages at a time: eight lanes take a row of each, so that a turn's chain (row, sums over lanes, barrier) is paid half as
     // often (a step of 8 rows of 32 heads, 4K tokens 101.8 -> 100.3 us, of 4 rows of 128K tokens 192.8 -> 190.5, with the same in the last kernel)
-    constexpr int RP = NT / 8, SP = RP / kStageRows;       // rows at a time, their stages; two of these to a turn
-    for (int i = 0; i < rs.n_chunk; i += 2 * SP) {
+    constexpr int RP = NT / 8, SP = RP / kStageRows, U = in_turn(LS, WIDE);       // rows at a time, their stages; U of these to a turn
+    for (int i = 0; i < rs.n_chunk; i += U * SP) {
         const int r0 = i * kStageRows + rgi;               // rows r0 and r0 + RP (a warp's are in one stage each)
-        const bool on[2] = {r0 < rs.rows, r0 + RP < rs.rows};
-        const float* xs[2];
+        bool on[U];
+        const float* xs[U];
+        float f[U], a[U][NH];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) xs[u] = on[u] ? rs.wait(u * SP + rgi / kStageRows, fail, c.status) + (rgi % kStageRows) * s.dck : nullptr;
-        const float f[2] = {pu.j >= 0 && on[0] ? f_s[r0] : 0.f, pu.j >= 0 && on[1] ? f_s[r0 + RP] : 0.f};
-        float a[2][NH];
+        for (int u = 0; u < U; ++u) {
+            on[u] = r0 + u * RP < rs.rows;
+            xs[u] = on[u] ? rs.wait(u * SP + rgi / kStageRows, fail, c.status) + (rgi % kStageRows) * s.dck : nullptr;
+            f[u] = pu.j >= 0 && on[u] ? f_s[r0 + u * RP] : 0.f;
+        }
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+        for (int u = 0; u < U; ++u)
 #pragma unroll
             for (int g = 0; g < NH; ++g) a[u][g] = 0.f;
 #pragma unroll
         for (int x4 = 0; x4 < 4; ++x4) {
             const int v = l8 + 8 * x4;
             if (v < nv) {
-                float4 x[2];
+                float4 x[U];
 #pragma unroll
-                for (int u = 0; u < 2; ++u) x[u] = on[u] ? *reinterpret_cast<const float4*>(xs[u] + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int u = 0; u < U; ++u) x[u] = on[u] ? *reinterpret_cast<const float4*>(xs[u] + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
                 if (pu.j >= 0) {
                     const float4 y = xr4[x4];
 #pragma unroll
-                    for (int u = 0; u < 2; ++u) {
+                    for (int u = 0; u < U; ++u) {
                         x[u].x = fmaf(f[u], y.x, x[u].x); x[u].y = fmaf(f[u], y.y, x[u].y); x[u].z = fmaf(f[u], y.z, x[u].z); x[u].w = fmaf(f[u], y.w, x[u].w);
                         if (on[u]) *reinterpret_cast<float4*>(ckg + (size_t)(m0 + r0 + u * RP) * s.dck + 4 * v) = x[u];
                     }
@@ -383,28 +390,27 @@ __global__ void __launch_bounds__(outer_threads(LS), NH == 4 && outer_ctas(LS) =
                 for (int g = 0; g < NH; ++g) {
                     const float4 z = qr[g][x4];
 #pragma unroll
-                    for (int u = 0; u < 2; ++u) a[u][g] = fmaf(x[u].x, z.x, fmaf(x[u].y, z.y, fmaf(x[u].z, z.z, fmaf(x[u].w, z.w, a[u][g]))));
+                    for (int u = 0; u < U; ++u) a[u][g] = fmaf(x[u].x, z.x, fmaf(x[u].y, z.y, fmaf(x[u].z, z.z, fmaf(x[u].w, z.w, a[u][g]))));
                 }
             }
         }
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1)
 #pragma unroll
-            for (int g = 0; g < NH; ++g) {
-                a[0][g] += __shfl_xor_sync(0xffffffffu, a[0][g], o);
-                a[1][g] += __shfl_xor_sync(0xffffffffu, a[1][g], o);
-            }
+            for (int g = 0; g < NH; ++g)
+#pragma unroll
+                for (int u = 0; u < U; ++u) a[u][g] += __shfl_xor_sync(0xffffffffu, a[u][g], o);
         // lane x of a row keeps head x's
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < U; ++u) {
             const int m = m0 + r0 + u * RP;
             float mine = a[u][0];
 #pragma unroll
             for (int g = 1; g < NH; ++g) if (l8 == g) mine = a[u][g];
             if (on[u] && l8 < nh) u_s[l8 * s.M + m] = (m == 0 ? w_0 : m == 1 ? w_1 : w_gen) * mine;
         }
-        rs.next(2 * SP);
-        rs.done(i, 2 * SP, tid);
+        rs.next(U * SP);
+        rs.done(i, U * SP, tid);
     }
     if (CL > 1) {                                          // this CTA's rows to the others
         cluster_meet(CL);                                  // every CTA of the cluster has started: its shared memory can be written; all rows are there
@@ -1006,13 +1012,13 @@ __global__ void __launch_bounds__(32 * kMainWarps, kMainCtas) chan_main_kernel(c
     }
 }
 
-// Cluster per job, 256 threads: the parts' statistics and outputs merged, z of nq channel pairs per CTA, summed over the cluster
+// Cluster per job: the parts' statistics and outputs merged, z of nq channel pairs per CTA, summed over the cluster
 // through distributed shared memory, a slice of the rows of C^V per CTA, its products summed likewise, the output rows.
 // After a step's push (step != 0) C^V's rows are updated on their way.
-// (128 registers at most: the plan counts on two CTAs to an SM, and the instances of 64 and 512 slots took 155, 9 to 11 % of a step)
-template <int LS>
-__global__ void __launch_bounds__(outer_threads(LS), outer_ctas(LS)) chan_out_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
-    constexpr int S = 1 << LS, NT = outer_threads(LS);
+// (unbounded, the instances of 64 and 512 slots took 155 registers and one CTA to an SM: 9 to 11 % of a step)
+template <int LS, bool WIDE>
+__global__ void __launch_bounds__(outer_threads(WIDE), outer_ctas(LS, WIDE)) chan_out_kernel(Dims s, ChanPlan mp, const __grid_constant__ ChanCall call) {
+    constexpr int S = 1 << LS, NT = outer_threads(WIDE);
     extern __shared__ __align__(16) float smz[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, CL = mp.nz, rank = CL > 1 ? (int)cluster_rank() : 0, h = blockIdx.y / mp.n_pass, pass = blockIdx.y - h * mp.n_pass;
@@ -1047,7 +1053,7 @@ __global__ void __launch_bounds__(outer_threads(LS), outer_ctas(LS)) chan_out_ke
         // rows of C^V: last written by a kernel that had ended before the main kernel let this one start
         rs.begin();
     }
-    pass_twiddles<LS>(twf, tid);
+    pass_twiddles<LS, NT>(twf, tid);
     for (int n = tid; n < s.k; n += NT) ph_s[n] = mid_phase(n, s);
     asm volatile("griddepcontrol.wait;" ::: "memory");    // the parts
     const int job = (b * s.Hkv + h) * mp.n_pass + pass, X = mp.n_cx + s.B * mp.n_wpart;
@@ -1203,7 +1209,7 @@ __global__ void __launch_bounds__(outer_threads(LS), outer_ctas(LS)) chan_out_ke
     for (int g = 0; g < 4; ++g) acc4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int rg = tid / nv, vcol = tid - rg * nv;
     const float4 y = j_push >= 0 ? *reinterpret_cast<const float4*>(xc + 4 * vcol) : make_float4(0.f, 0.f, 0.f, 0.f);      // (the thread's columns are the same in every row)
-    constexpr int SP = NT / 128;                           // stages at a time: the thread's chain through them is paid once
+    constexpr int SP = out_stages(LS, WIDE);               // stages at a time: the thread's chain through them is paid once
     for (int i = 0; i < rs.n_chunk; i += SP) {
         const float* xs[SP];
 #pragma unroll
@@ -1286,7 +1292,7 @@ size_t in_smem(const Dims& s, int ls, const ChanPlan& m) {
                             (((s.M + m.nz - 1) / m.nz + 5) & ~3) + 2 * ((s.k + 1) & ~1) + 4 * s.d + (fft > stage ? fft : stage)) + 64;
 }
 size_t out_smem(const Dims& s, int ls, const ChanPlan& m) {
-    const size_t fft = (size_t)m.nq * m.nh * pf_size(2 << ls), ps = (size_t)outer_threads(ls) * 4 * m.nh;
+    const size_t fft = (size_t)m.nq * m.nh * pf_size(2 << ls), ps = (size_t)outer_threads(m.wide) * 4 * m.nh;
     return sizeof(float) * (20 + ((2 * (tw_total(ls) + 1) + 3) & ~3) + (size_t)m.nh * s.M + ((2 * m.nq * s.k + 3) & ~3) + 8 + 5 * s.dcv +
                             5 * (size_t)(((s.M + m.nz - 1) / m.nz + 5) & ~3) + ((s.d + 7) & ~7) / 2 + 2 * ((s.k + 1) & ~1) + (size_t)m.st_out * kStageRows * s.dcv + (fft > ps ? fft : ps)) + 64;
 }
@@ -1315,12 +1321,12 @@ cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, siz
 }  // namespace
 
 // (as many as the threads of a CTA take at a time)
-static int least_stages(int log2S) { return outer_threads(log2S) / 128; }
+static int least_stages(bool wide) { return outer_threads(wide) / 128; }
 // As many stages of the outer kernels' rows as a CTA's rows take and the limit of shared memory holds.
 static void fit_stages(const Dims& s, int log2S, size_t limit, ChanPlan* m) {
     auto fits = [&]() { return in_smem(s, log2S, *m) <= limit && out_smem(s, log2S, *m) <= limit; };
     const int chunks = (s.M / m->nz + 2 + kStageRows - 1) / kStageRows, most = chunks < kMaxRowStages ? chunks : kMaxRowStages;
-    m->st_in = m->st_out = least_stages(log2S);
+    m->st_in = m->st_out = least_stages(m->wide);
     for (; m->st_in < most; ++m->st_in) { ++m->st_in; const bool ok = fits(); --m->st_in; if (!ok) break; }
     for (; m->st_out < most; ++m->st_out) { ++m->st_out; const bool ok = fits(); --m->st_out; if (!ok) break; }
 }
@@ -1381,23 +1387,38 @@ bool plan_channels(const Dims& s, int log2S, int sms, ChanPlan* m) {
     // CTAs per cluster of the kernels in front and behind.  The device holds 15 clusters of eight CTAs of one to an SM, 33 of four,
     // 74 of two, twice that with two to an SM; a wave costs what does not depend on the split and the split's share, about four
     // times that for a job in one CTA (32 jobs of 2048 coefficients: 35 us a kernel in one wave of clusters of four, 55 in two of eight)
+    // The longest transforms in CTAs of sixteen warps, one to an SM (wide), or of eight: those where two of them fit and that makes it less than three quarters of the cost (as
+    // much where only the larger clusters of the wide form do not fit).  us a step of one layer / four layers, wide and not, 128 classes, cost ratio: 48 heads of three, 2048
+    // coefficients 129, 124 / 363, 366 (0.75); 48 of four 137, 162 / 388, 472 (1); 48 of two 102, 108 / 281, 325 (1), 1536 88, 84 / 250, 242 (0.67); 64 of one 105, 103 / 351, 345
+    // (0.67); 64 of four, 512 coefficients 112, 102 / 392, 358 (0.75, clusters of two); 32 of four, 40 coefficients 65, 71 / 190, 144 (1); 64 classes: 192 of one, 40
+    // coefficients 155, 123 / 555, 405 (0.56); 96 of two, 40 76, 88 / 214, 253 (0.8), 512 118, 107 / 409, 304 (0.67).
     auto fits = [&](size_t limit) { return in_smem(s, log2S, *m) <= limit && out_smem(s, log2S, *m) <= limit; };
     constexpr size_t kHalf = 112 * 1024, kAll = 226 * 1024;
-    m->st_in = m->st_out = least_stages(log2S);
-    int best_nz = 0, occ = 0;
-    double least = 0;
-    for (m->nz = 8; m->nz >= 1; m->nz /= 2) {
-        m->nq = kMR / 2 / m->nz;
-        const int fit = fits(kHalf) && outer_ctas(log2S) > 1 ? 2 : fits(kAll) ? 1 : 0;
-        if (!fit) continue;
-        const long long held = (long long)(m->nz == 8 ? 15 : m->nz == 4 ? 33 : m->nz == 2 ? 74 : 148) * sms / 148 * fit;
-        const double cost = (double)((jobs + held - 1) / held) * (1.0 + 4.0 / m->nz);
-        if (!best_nz || cost < least) { least = cost; best_nz = m->nz; occ = fit; }
+    struct Outer { int nz, occ; double cost; };
+    auto outer = [&](int wide) {
+        Outer best = {};
+        m->wide = wide;
+        m->st_in = m->st_out = least_stages(wide);
+        for (m->nz = 8; m->nz >= 1; m->nz /= 2) {
+            m->nq = kMR / 2 / m->nz;
+            const int fit = fits(kHalf) && outer_ctas(log2S, wide) > 1 ? 2 : fits(kAll) ? 1 : 0;
+            if (!fit) continue;
+            const long long held = (long long)(m->nz == 8 ? 15 : m->nz == 4 ? 33 : m->nz == 2 ? 74 : 148) * sms / 148 * fit;
+            const double cost = (double)((jobs + held - 1) / held) * (1.0 + 4.0 / m->nz);
+            if (!best.nz || cost < best.cost) best = Outer{m->nz, fit, cost};
+        }
+        return best;
+    };
+    Outer use = outer(0);
+    if (log2S == 10) {
+        const Outer w = outer(1);
+        if (w.nz && !(use.nz && (use.occ == 2 ? use.cost < 0.75 * w.cost : use.cost <= 0.75 * w.cost))) use = w;
+        else m->wide = 0;
     }
-    if (!best_nz) return false;
-    m->nz = best_nz;
+    if (!use.nz) return false;
+    m->nz = use.nz;
     m->nq = kMR / 2 / m->nz;
-    fit_stages(s, log2S, occ == 2 && jobs * m->nz > sms ? kHalf : kAll, m);
+    fit_stages(s, log2S, use.occ == 2 && jobs * m->nz > sms ? kHalf : kAll, m);
     return true;
 }
 
@@ -1418,15 +1439,15 @@ size_t place_channels(const Dims& s, int log2S, ChanPlan* m) {
     return off;
 }
 
-template <int LS>
+template <int LS, bool WIDE>
 static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, const ChanPlan& one, cudaStream_t st, bool* begun) {
     *begun = false;
     if (n < 1 || n > kChanLayers) return cudaErrorInvalidValue;
     ChanPlan m = one;
     // several layers, more CTAs than two to an SM: fewer stages each, so that three fit (the sums do not depend on the number of stages)
     constexpr size_t kThird = 74 * 1024;
-    if (outer_ctas(LS) == 3 && (long long)n * s.B * s.Hkv * m.n_pass * m.nz > 2 * sm_count()) {
-        m.st_in = m.st_out = least_stages(LS);
+    if (outer_ctas(LS, WIDE) == 3 && (long long)n * s.B * s.Hkv * m.n_pass * m.nz > 2 * sm_count()) {
+        m.st_in = m.st_out = least_stages(WIDE);
         if (in_smem(s, LS, m) <= kThird && out_smem(s, LS, m) <= kThird) fit_stages(s, LS, kThird, &m);
         else m = one;
     }
@@ -1444,14 +1465,14 @@ static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, co
         if ((s.l_init > 0 && !ok_i) || (s.l_local > 0 && !ok_l)) return cudaErrorInvalidValue;
         if (!mid_map(&t.km, c.k_mid, s, s.nfk) || !mid_map(&t.vm, c.v_mid, s, s.nfv)) return cudaErrorInvalidValue;
     }
-    auto launch_in = [&](auto nh) { return launch_chained(chan_in_kernel<LS, decltype(nh)::value>, cg, dim3(outer_threads(LS)), in_smem(s, LS, m), m.nz, st, s, m, call); };
+    auto launch_in = [&](auto nh) { return launch_chained(chan_in_kernel<LS, decltype(nh)::value, WIDE>, cg, dim3(outer_threads(WIDE)), in_smem(s, LS, m), m.nz, st, s, m, call); };
     cudaError_t err = m.nh == 1 ? launch_in(std::integral_constant<int, 1>{}) : m.nh == 2 ? launch_in(std::integral_constant<int, 2>{}) : launch_in(std::integral_constant<int, 4>{});
     if (err != cudaSuccess) return err;
     *begun = true;
     err = m.hp == 2 ? launch_chained(chan_main_kernel<2>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, maps, s, m, call)
                     : launch_chained(chan_main_kernel<4>, mg, dim3(32 * kMainWarps), (size_t)m.smem, 1, st, maps, s, m, call);
     if (err != cudaSuccess) return err;
-    return launch_chained(chan_out_kernel<LS>, cg, dim3(outer_threads(LS)), out_smem(s, LS, m), m.nz, st, s, m, call);
+    return launch_chained(chan_out_kernel<LS, WIDE>, cg, dim3(outer_threads(WIDE)), out_smem(s, LS, m), m.nz, st, s, m, call);
 }
 
 // The decode calls of n layers of one layout, with k_new / v_new (not null; one pass only) each behind the push of Eq.5.  Several layers do not touch
@@ -1459,12 +1480,12 @@ static cudaError_t launch_channels_t(const Dims& s, const ChanArgs* a, int n, co
 // cluster, say).
 cudaError_t launch_decode_channels(const Dims& s, const ChanArgs* a, int n, const ChanPlan& m, int log2S, cudaStream_t st, bool* begun) {
     switch (log2S) {
-        case 5: return launch_channels_t<5>(s, a, n, m, st, begun);
-        case 6: return launch_channels_t<6>(s, a, n, m, st, begun);
-        case 7: return launch_channels_t<7>(s, a, n, m, st, begun);
-        case 8: return launch_channels_t<8>(s, a, n, m, st, begun);
-        case 9: return launch_channels_t<9>(s, a, n, m, st, begun);
-        case 10: return launch_channels_t<10>(s, a, n, m, st, begun);
+        case 5: return launch_channels_t<5, false>(s, a, n, m, st, begun);
+        case 6: return launch_channels_t<6, false>(s, a, n, m, st, begun);
+        case 7: return launch_channels_t<7, false>(s, a, n, m, st, begun);
+        case 8: return launch_channels_t<8, false>(s, a, n, m, st, begun);
+        case 9: return launch_channels_t<9, false>(s, a, n, m, st, begun);
+        case 10: return m.wide ? launch_channels_t<10, true>(s, a, n, m, st, begun) : launch_channels_t<10, false>(s, a, n, m, st, begun);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -41,6 +41,9 @@ def _like(layout, algo):
     (64, dict(B=8, Hkv=16, Hq=64, T=4096, M=128, L=2100, n_full_k=64, n_full_v=64)),       # most kept dims: two stages a warp
     (128, dict(B=4, Hq=32, T=131072, M=2048, L=3000)),    # longest transforms, clusters of four
     (64, dict(B=8, Hq=32, T=65536, M=2048, L=1000, n_full_k=24, n_full_v=24)),     # and in two waves of clusters
+    (128, dict(B=6, Hq=24, T=131072, M=40, L=700)),       # eight warps to a CTA, two to an SM: fewer rows than a stage holds
+    (128, dict(B=8, Hq=8, T=131072, M=2048, L=900)),      # one head, many rows
+    (64, dict(B=8, Hkv=16, Hq=64, T=65536, M=512, L=800)),         # clusters of two that the sixteen warps' sums leave no room for
 ])
 def test_channels_against_oracle(P, kw):
     shape = _shape(**kw)
