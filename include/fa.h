@@ -186,10 +186,12 @@ fa_status fa_compress_ex(const fa_layout* layout, fa_cache* cache, const void* K
  * kept-dim rows and counters bit for bit; coefficients within the same tolerance: floating-point atomics).  layouts
  * and caches are HOST arrays of n_layers entries; K and V are HOST arrays of n_layers DEVICE pointers to the layers'
  * prefilled tensors, which share strides and length L.  The caches of different layers must not share memory.
- * Where every layer takes the tensor-core path on CTA pairs, the call enqueues all partition kernels and then all
- * contractions, each launched programmatically behind the one before: kernels of neighbouring layers overlap (the
+ * Where every layer takes the tensor-core path on CTA pairs, layers overlap.  By block moments (see fa_compress; groups of layers of one layout
+ * take turns where the workspace does not hold the moments of all) up to eight layers share their launches, and the windows and
+ * counters of all layers come last, beside the last group's coefficients.  Else the call enqueues all partition kernels and then all
+ * contractions, each launched programmatically behind the one before (the
  * small partition kernels run side by side, a contraction starts on the SMs that its predecessor's first CTAs to
- * finish leave) and every kernel waits for its predecessor before it ends, so that work enqueued behind the call
+ * finish leave).  Every kernel waits for its predecessor before it ends, so that work enqueued behind the call
  * sees all layers complete.  Otherwise the layers are compressed one after the other.  All layers are checked on the
  * host before the first launch; returns the first error. */
 fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cache* caches, const void* const* K,
@@ -198,7 +200,7 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
 
 /* fa_compress for a batch whose rows have different prompt lengths: row b is compressed from its
  * first lengths[b] tokens (HOST array of B entries, each 0 <= lengths[b] and within the capacity rule
- * of fa_compress; K / V rows beyond a row's length are not read).  Every row becomes what a one-row
+ * of fa_compress; what K / V hold beyond a row's length has no effect, though up to 63 tokens of it may be loaded).  Every row becomes what a one-row
  * fa_compress would make of it (coefficients within the same tolerance), in one set of launches for up to 64 rows; fa_append, fa_decode_attention and fa_decode_step then work on the
  * ragged batch as on any other (the token counters are per batch row). */
 fa_status fa_compress_ragged(const fa_layout* layout, fa_cache* cache, const void* K, const void* V,
@@ -278,7 +280,8 @@ size_t fa_step_staging_bytes(const fa_layout* layout);
  *     outputs, ascending, ready to be a cache's index sets.
  *   mse: optional DEVICE output [B][H_kv][2][d] (side 0 = K, 1 = V), the per-row mean squared errors.
  *   ws / ws_bytes: scratch of fa_select_workspace_bytes(layout) bytes, 256-byte aligned (it holds the
- *     coefficients of all dimensions).  head_dim must be 64, 128 or 256.
+ *     coefficients of all dimensions).  head_dim must be 64, 128 or 256.  A smaller workspace is refused only where the coefficients and
+ *     the scratch of a decode call do not fit: without room for block moments the direct contractions serve, which are slower.
  * For bf16 tensors (head_dim 64 or 128, 16-byte aligned bases and strides) the reconstruction runs on the tensor cores: with
  * n_coef a multiple of 256, a period of at least 16 n_coef, 1024 middle tokens and 6 M values of the middle of K (all rows and heads) by block
  * moments, whose factors carry 2^-17 (a dimension that its coefficients rebuild exactly reports about 1e-9 of its mean square); else, n_coef a multiple of 64, with the basis and the
@@ -313,7 +316,8 @@ size_t fa_static_workspace_limit(void);
 fa_status fa_poll_status(const fa_cache* cache, void* stream);
 
 /* Number of kernels one call launches for this layout (what = 0 compress, 1 append,
- * 2 decode, 3 decode step); for launch accounting by callers.  what >= 4 asks about the decode plan instead:
+ * 2 decode, 3 decode step); for launch accounting by callers.  0 is the direct contraction's; by block moments (see fa_compress) a call
+ * launches three kernels, two more for every further group of batch rows, one for rows too short for it.  what >= 4 asks about the decode plan instead:
  * 4: 1 if fa_decode_attention runs the split build of the fused kernel for this layout, else 0;
  * 5: residue classes per batch of the transform kernel (0 for the direct kernel);
  * 6: CTAs per (batch, KV head, pass of query heads); 7: kernels of a decode call in the channel form, 0 where AUTO does not

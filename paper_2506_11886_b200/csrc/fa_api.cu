@@ -125,14 +125,15 @@ static fa_status make_plan(const fa_layout& l, CallPlan* p);
 
 // Whether the channel form is ahead of the transform kernel: it makes 16 transforms per (batch row, KV head) where the other makes
 // one per residue class, but as a chain of three kernels whose first and last cost 10 to 35 us whatever the batch.  So it goes by
-// the class transforms that there are, heads * classes.  A step, transform kernel -> channel form in us (GQA 4 and 3, MHA, kept
-// dims 24 to 48 a side, 131 layouts each way):
-//   from 8192 class transforms (all periods): 64 heads of 128 classes, 4K tokens 66.5 -> 43.7, 12K 99 -> 72, 64K 314 -> 228;
-//     256 heads of 32 classes, 1K 64.5 -> 47.5, 4K 117.7 -> 100; 128 heads of 64 classes, 4K 70.9 -> 67.7, ragged 70 -> 73.5
-//   from 4096 where rows are long: 64 heads of 64 classes, 12K 101.5 -> 83, 32K 189 -> 169; 32 heads of 128, 128K 243 -> 228 to 298 -> 201;
-//     but at 4K tokens 52 -> 57
-//   below: 32 heads of 64 classes, 32K 90 -> 97, 12K 53 -> 64; 64 heads of 32 classes, 4K 50 -> 51, 32K 197 -> 207; 16 heads of
-//     128 classes, 128K 122 -> 159; one row of 8 heads, 32K 38 -> 52
+// the class transforms that there are, heads * classes, at a step of ONE layer: layers of a call share the launches and are to give the bits of single
+// calls, so they take the same form (four layers of a call are ahead in it at every size below, see the second pairs).  us, transform kernel -> channel
+// form, one layer; four layers of a call:
+//   from 8192 class transforms (all periods): 64 heads of 128 classes, 4K tokens 63 -> 47; 259 -> 127, 12K 98 -> 73; 390 -> 197, 64K 223 -> 165; 894 -> 527;
+//     256 heads of 32 classes, 1K 53 -> 42; 226 -> 134, 4K 103 -> 90; 418 -> 294; 128 heads of 64 classes, 4K 70 -> 58; 281 -> 188
+//   from 4096 where rows are long: 64 heads of 64 classes, 12K 86 -> 80; 346 -> 226, 32K 148 -> 129; 597 -> 413; 32 heads of 128, 12K 57 -> 48; 231 -> 120, 60K
+//     129 -> 116; 517 -> 358, 128K 235 -> 176; 945 -> 596; but at 4K tokens 42 -> 44; 165 -> 77, 64 heads of 64 classes 50 -> 49; 206 -> 139, 128 of 32 62 -> 62; 252 -> 196
+//   below: 48 heads of 64 classes, 12K 67 -> 67; 265 -> 177; 32 of 64, 32K 83 -> 93; 336 -> 281, 12K 51 -> 54; 211 -> 140; 64 heads of 32 classes, 4K 46 -> 49;
+//     196 -> 148, 32K 186 -> 191; 754 -> 651; 16 heads of 128 classes, 128K 125 -> 124; 501 -> 324; one row of 8 heads, 32K 32 -> 46; 133 -> 98
 static bool channels_pay(const Dims& s) {
     const long long heads = (long long)s.B * s.Hkv, transforms = heads * s.P;
     return heads >= 32 && (transforms >= 8192 || (transforms >= 4096 && s.T >= 16384));
@@ -643,7 +644,8 @@ fa_status fa_compress_layers(int32_t n_layers, const fa_layout* layouts, fa_cach
         }
         return FA_OK;
     }
-    // All partition kernels first, each launched programmatically behind the one before (they touch different caches and
+    // By block moments: the moment kernels and projections of groups of layers, then all windows.  Else all partition kernels first, each launched
+    // programmatically behind the one before (they touch different caches and
     // run side by side; each ends by waiting for its predecessor, so the end of the last implies the end of all); then
     // the contractions, likewise: the CTAs of layer i + 1 take the SMs that the first CTAs of layer i to finish
     // leave, and wait for layer i (hence for everything before it) only in front of their reductions.
@@ -1086,7 +1088,7 @@ fa_status fa_decode_step_host(const fa_layout* layout, fa_cache* cache, const vo
 int fa_launch_count(const fa_layout* layout, int what) {
     if (check_layout(layout) != FA_OK) return 0;
     switch (what) {
-        case 0: return 2;   // partition/gather + coefficient kernel (memsets not counted)
+        case 0: return 2;   // partition/gather + coefficient kernel, the direct contraction's (by block moments it is three and more, see fa.h)
         case 1: return 1;
         case 2: {           // one fused kernel, or prologue + main + epilogue
             CallPlan p;

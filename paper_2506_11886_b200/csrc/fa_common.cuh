@@ -73,7 +73,8 @@ struct ChanPlan {
     size_t off_z, off_w, off_mw, off_ml, off_o, off_g, off_x, off_j, off_p;      // from the start of a layer's areas
     size_t base, per_layer, total;       // one layer's areas in the workspace: their start, size and end
 };
-constexpr int kChanLayers = 4;           // layers that share the launches of the channel form
+constexpr int kChanLayers = 4;           // layers that share the launches of the channel form (eight layers a call, us, at most 1 / 2 / 4 / 8: 256 heads of 4 K tokens 805/728/635/579, 32 of
+                                         // 40 K 1065/835/762/706, 64 of 4 K 391/308/253/222; each takes areas in the workspace, 10 to 50 MB for those)
 // A layer of a launch of the channel form; ws: its areas.
 struct ChanArgs {
     CacheDev c;
@@ -161,7 +162,8 @@ bool compress_mom_supported(const Dims& s);
 size_t compress_mom_row_bytes(const Dims& s, int n_mid);
 cudaError_t launch_compress_mom(const Dims&, const CacheDev&, const void* K, const void* V, int64_t sb, int64_t st, int64_t sh, int L, int b0,
                                 int nb, void* Y, bool wait_first, bool chained, cudaStream_t, const RowLens* lens = nullptr, int tc_min = 1);
-constexpr int kMomLayers = 8;        // layers of a launch_compress_mom_layers call
+constexpr int kMomLayers = 8;        // layers of a launch_compress_mom_layers call (sixteen layers of 8 heads, us, at most 2 / 4 / 8 / 16: 32 K tokens 786/703/681/680, 8 K
+                                     // 260/215/190/173, 4 K 203/174/125/115)
 cudaError_t launch_compress_mom_layers(const Dims&, const CacheDev*, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
                                        int64_t sh, int L, void* Y, bool wait_first, bool chained, cudaStream_t);
 cudaError_t launch_windows(const Dims&, const CacheDev*, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st, int64_t sh, int L,

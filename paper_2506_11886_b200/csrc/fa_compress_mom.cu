@@ -1114,7 +1114,7 @@ cudaError_t launch_compress_mom(const Dims& s, const CacheDev& c, const void* K,
     return launch_rows(s, &c, &K, &V, 1, sb, st, sh, L, rows, fold, static_cast<char*>(Y), wait_first, chained, stream);
 }
 
-// The same for all batch rows of up to kMomLayers layers of one shape: a moment kernel each, then one projection.  A projection
+// The same for all batch rows of up to kMomLayers layers of one shape: moment kernels of several layers each, then one projection.  A projection
 // takes 31 us (plain form) for a layer of 8 heads, 32K tokens and 1024 coefficients, a third of it its start and the segments that teams
 // share, which six layers together pay once: 6 x 31 -> 115 us, folded 72.  Y: room for the moments of all of them.
 cudaError_t launch_compress_mom_layers(const Dims& s, const CacheDev* c, const void* const* K, const void* const* V, int n_layers, int64_t sb, int64_t st,
