@@ -242,14 +242,14 @@ __global__ void __launch_bounds__(256) compress_coef_kernel(Dims s, CacheDev c, 
 }
 
 // Rows per thread of the contraction, and how the tokens' chunks are split: what the SM with the most CTAs takes for them, a chunk counting as the products of a
-// lane's token and 10 of them more (with eight rows of eight columns, registers for one CTA to an SM, 1.3 times those), and a CTA by itself 60 at least.  Of 854 calls (16
-// to 2048 coefficients, 1 to 256 heads, 20 to 6000 tokens, 64 to 256 dims) 0.6 % behind the better form on average.  us, four / eight rows a thread:
+// lane's token and 10 of them more (with eight rows of eight columns, registers for one CTA to an SM, 1.3 times those), and a CTA by itself 60 at least.  Rows of
+// several lengths even the SMs out: what an average one has.  Of 1184 calls (16 to 2048 coefficients, 1 to 256 heads, 20 to 6000 tokens, 64 to 256 dims) 0.5 % behind the better form on average.  us, four / eight rows a thread:
 //   tiles of 64 rows that would be half empty: 16 coefficients, 32 heads, 900 tokens 149/264; 32 coefficients, 32 heads, 340 tokens 17.2/25.7
-//   many CTAs: 200 coefficients, 128 heads, 5600 tokens 1234/1106 (ragged); 128, 48 heads, 590 tokens 101/85; few: 16.9/16.1, 12.8/11.4
+//   many CTAs: 200 coefficients, 128 heads, 5600 tokens 1234/1106, 128, 64 heads, rows of 1013 and 570 tokens 154/142 (both ragged); 128, 48 heads, 590 tokens 101/85; few: 16.9/16.1, 12.8/11.4
 //   256 dims: 1024 coefficients, 32 heads 4880/6181; 100, 96 heads 459/544; few CTAs: 100, two heads 25.5/21.4
 //   a fixed order (a CTA takes all tokens of its rows): 100 coefficients, 8 heads, 1300 tokens 69/100; 256, 32 heads, 240 tokens 60/47; 128, 64 heads, 1000 tokens 191/228
 struct RowSplit { int rpt, row_tiles, n_tsplit, cps; };
-static RowSplit rows_per_thread(const Dims& s, int live_rows, int chunks, int nc, bool ordered) {
+static RowSplit rows_per_thread(const Dims& s, int live_rows, int chunks, int nc, bool ordered, bool ragged) {
     RowSplit best = {};
     double least = 0;
     const int sms = sm_count();
@@ -261,7 +261,7 @@ static RowSplit rows_per_thread(const Dims& s, int live_rows, int chunks, int nc
         if (n < 1 || ordered) n = 1;                         // one split: every coefficient is added to zero exactly once
         x.cps = (chunks + n - 1) / n;
         x.n_tsplit = (chunks + x.cps - 1) / x.cps;
-        const double chunk = 10 + rpt * nc * (rpt == 8 && nc == 8 ? 1.3 : 1.0), all = ((ctas_fixed * x.n_tsplit + sms - 1) / sms) * chunk;
+        const double chunk = 10 + rpt * nc * (rpt == 8 && nc == 8 ? 1.3 : 1.0), ctas = (double)ctas_fixed * x.n_tsplit / sms, all = (ragged ? ctas : ceil(ctas)) * chunk;
         const double time = x.cps * (all > 60 ? all : 60);
         if (best.rpt == 0 || time < least) { best = x; least = time; }
     }
@@ -313,7 +313,7 @@ static cudaError_t launch_compress_t(const Dims& s, const CacheDev& c, const voi
     if (n_mid == 0 || max_comp == 0 || !with_coef) return cudaSuccess;
     const int live_rows = rl.n ? n_short : s.B;
     const int nc = max_comp <= 128 ? (max_comp + 31) / 32 : 8;
-    const RowSplit split = rows_per_thread(s, live_rows, (n_mid + kTJ - 1) / kTJ, nc, ordered);
+    const RowSplit split = rows_per_thread(s, live_rows, (n_mid + kTJ - 1) / kTJ, nc, ordered, rl.n > 1);
     const int rpt = split.rpt, cps = split.cps;
     const size_t smem = sizeof(float) * kTJ * (size_t)(32 * nc + 8 * rpt);
     // behind the partition kernel programmatically: it waits for it in front of its additions
